@@ -314,3 +314,121 @@ def tolerance(case):
     if kind == "train":                                                  # gradients: 3.3e-3, single values 3.1e-2
         return {"rel": 1.2e-2, "max": 0.12}
     return {"rel": 1e-2, "max": 7e-2}                                    # outputs: 2.5e-3, 1.8e-2
+
+
+def _softmax_parts(s, b, h, i0, i1, gate, K, V, ctx):
+    """Gated scores of query rows [i0, i1) of one head in 64 bits: per level (first key, scores + log gate, keys, values)."""
+    c = s["case"]
+    T, d, W = c["T"], c["d"], c["W"]
+    q = s["Q"][b, h, i0:i1].double() * d ** -0.5
+    p = torch.arange(ctx + i0, ctx + i1, device=_DEV)[:, None]
+    out = []
+    for l in range(3):
+        lo = max(0, ctx + i0 - W + 1) if l == 0 else 0
+        hi = min(K[l].shape[0], ctx + i1) if l < 2 else K[l].shape[0]
+        k, v = K[l][lo:hi], V[l][lo:hi]
+        x = q @ k.T + torch.log(gate[b, i0:i1, l:l + 1])
+        if l < 2:
+            j = torch.arange(lo, hi, device=_DEV)[None]
+            x.masked_fill_((j > p) | (j <= p - W) if l == 0 else j > p, float("-inf"))
+        out.append((lo, x, k, v))
+    return out
+
+
+def _attention64(s, gate, head_kv, ctx=0, dO=None, full=False, rows=1024):
+    """Forward (and, with dO, backward) in 64 bits, one head and some query rows at a time."""
+    c = s["case"]
+    B, H, T, d = c["B"], c["H"], c["T"], c["d"]
+    new = lambda *n: torch.zeros(*n, dtype=torch.float64, device=_DEV)  # noqa: E731
+    O, LSE, F = new(B, H, T, d), new(B, H, T), new(B, H, T, d) if full else None
+    if dO is not None:
+        dQ, dG = new(B, H, T, d), new(B, T, 3)
+        dK, dV = ([new(*k.shape) for k in s["K"]] for _ in range(2))
+    for b in range(B):
+        for h in range(H):
+            g = h // (H // c.get("Hkv", H))
+            K, V = head_kv(b, g)
+            for i0 in range(0, T, rows):
+                i1 = min(T, i0 + rows)
+                parts = _softmax_parts(s, b, h, i0, i1, gate, K, V, ctx)
+                if full:
+                    F[b, h, i0:i1] = sum(gate[b, i0:i1, l:l + 1] * (torch.softmax(x, 1) @ v) for l, (_, x, _, v) in enumerate(parts))
+                lse = torch.logsumexp(torch.stack([torch.logsumexp(x, 1) for _, x, _, _ in parts]), 0)
+                P = [x.sub_(lse[:, None]).exp_() for _, x, _, _ in parts]
+                o = sum(pl @ v for pl, (_, _, _, v) in zip(P, parts))
+                O[b, h, i0:i1], LSE[b, h, i0:i1] = o, lse
+                if dO is None:
+                    continue
+                do, q = dO[b, h, i0:i1].double(), s["Q"][b, h, i0:i1].double()
+                for l, (pl, (lo, _, k, v)) in enumerate(zip(P, parts)):
+                    at = slice(lo, lo + k.shape[0])
+                    dV[l][b, g, at] += pl.T @ do
+                    ds = pl.mul_(do @ v.T - (do * o).sum(1, keepdim=True))
+                    dG[b, i0:i1, l] += ds.sum(1)
+                    dQ[b, h, i0:i1] += (ds @ k) * d ** -0.5
+                    dK[l][b, g, at] += (ds.T @ q) * d ** -0.5
+    if dO is not None:
+        x = s["X"].double().reshape(-1, H * d)
+        return O, LSE, F, dQ, dK, dV, dG, x.T @ dG.view(-1, 3), dG.view(-1, 3).sum(0)
+    return O, LSE
+
+
+def exact(case, seed):
+    """The outputs of ``run`` in 64 bits, from torch alone (``prepare`` gives the inputs)."""
+    if case["kind"] == "index":                                          # code bits, not numbers
+        return None
+    s = prepare(case, seed)
+    c = s["case"]
+    kind = c["kind"]
+    if kind == "summary":
+        X, M2, step = s["X"], torch.empty(s["X"].shape, dtype=torch.float64, device=_DEV), 256
+        m = s["state"].double() if c["carry"] else X[:, 0].double() if c["ema"] else torch.zeros_like(s["state"], dtype=torch.float64)
+        i = torch.arange(step, device=_DEV, dtype=torch.float64)
+        keep = float(torch.tensor(0.9, dtype=_F32))                      # the call takes its decay in 32 bits
+        decay = torch.where(i[:, None] >= i[None], keep ** (i[:, None] - i[None]).clamp_min(0), 0.0) * (1.0 - keep if c["ema"] else 0.0)
+        for t in range(0, X.shape[1], step):
+            x = X[:, t:t + step].double()
+            n = x.shape[1]
+            if c["ema"]:
+                y = decay[:n, :n] @ x + keep ** (i[:n, None] + 1) * m[:, None]
+                M2[:, t:t + n] = y
+            else:
+                y = x.cumsum(1) + m[:, None]
+                M2[:, t:t + n] = y / (t + 1 + i[:n, None])
+            m = y[:, -1]
+        return [M2, m]
+    gate = torch.softmax(s["X"].double() @ s["W_r"].double() + s["b_r"].double(), -1)
+    if kind in ("train", "fp32", "prefill"):
+        kv = lambda b, g: ([x[b, g].double() for x in s["K"]], [x[b, g].double() for x in s["V"]])  # noqa: E731
+        if kind == "prefill":
+            return [gate, *_attention64(s, gate, kv)]
+        O, LSE, F, dQ, dK, dV, dG, dW, db = _attention64(s, gate, kv, dO=s["dO"], full=kind == "fp32")
+        return [gate, O, LSE, dQ, dK, dV, dG, dW, db] + ([F] if kind == "fp32" else [])
+    if kind == "decode":
+        O, LSE = torch.empty(s["q"].shape, dtype=torch.float64, device=_DEV), torch.empty(c["B"], c["H"], dtype=torch.float64, device=_DEV)
+        for b in range(c["B"]):
+            q = s["q"][b].double().view(c["Hkv"], -1, c["d"]) * c["d"] ** -0.5
+            x = torch.cat([q @ k[b].double().transpose(1, 2) + torch.log(gate[b, l]) for l, k in enumerate(s["K"])], 2)
+            LSE[b] = torch.logsumexp(x, 2).view(-1)
+            O[b] = (torch.softmax(x, 2) @ torch.cat([v[b].double() for v in s["V"]], 1)).view(c["H"], c["d"])
+        return [gate, O, LSE]
+    # chunk and serve: the fused rows in the session pool
+    pools = []
+    at = s["at"].long() if kind == "serve" else torch.full((c["B"],), c["ctx"], device=_DEV)
+    tab = (s["t2"] if kind == "serve" else s["tab"][1]).long()
+    for pool, new in ((s["pk"][1], s["newK"]), (s["pv"][1], s["newV"])):
+        pool = pool.double()
+        for b in range(c["B"]):
+            r = at[b] + torch.arange(new[0].shape[2], device=_DEV)
+            pool[tab[b, r // c["page"]], :, r % c["page"]] = sum(gate[b, :, l, None] * x[b].double() for l, x in enumerate(new)).transpose(0, 1)
+        pools.append(pool)
+    if kind == "serve":                                                  # what is recalled hangs on single code bits
+        return [gate, *pools, None, None, None, None, None]
+
+    def paged(b, g):
+        out = []
+        for src, fused in ((s["pk"], pools[0]), (s["pv"], pools[1])):
+            out.append([(fused.to(_BF16) if l == 1 else src[l])[s["tab"][l][b].long(), g].reshape(-1, c["d"])[:s["n"][l]].double() for l in range(3)])
+        return out
+
+    return [gate, *_attention64(s, gate, paged, ctx=c["ctx"]), *pools]
