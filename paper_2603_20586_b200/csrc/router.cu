@@ -10,6 +10,7 @@ namespace {
 
 constexpr int kRowsPerWarp = 4;
 constexpr int kWarps = 8;
+constexpr int kMaxThreads = 256;
 
 __device__ __forceinline__ void finish_row(float g0, float g1, float g2, int route, long long row, float* gate,
                                            float* log2_gate, int8_t* idx) {
@@ -53,9 +54,10 @@ __device__ __forceinline__ void finish_row(float g0, float g1, float g2, int rou
 
 template <typename T> struct Vec8;  // eight consecutive elements as floats
 template <> struct Vec8<__nv_bfloat16> {
-    static __device__ __forceinline__ void load(const __nv_bfloat16* p, float (&x)[8]) {
-        uint4 u = __ldg(reinterpret_cast<const uint4*>(p));
-        uint32_t w[4] = {u.x, u.y, u.z, u.w};
+    using Raw = uint4;
+    static __device__ __forceinline__ Raw fetch(const __nv_bfloat16* p) { return __ldg(reinterpret_cast<const uint4*>(p)); }
+    static __device__ __forceinline__ void widen(const Raw& u, float (&x)[8]) {
+        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             x[2 * i] = __uint_as_float(w[i] << 16);
@@ -64,18 +66,94 @@ template <> struct Vec8<__nv_bfloat16> {
     }
 };
 template <> struct Vec8<float> {
-    static __device__ __forceinline__ void load(const float* p, float (&x)[8]) {
-        float4 a = __ldg(reinterpret_cast<const float4*>(p));
-        float4 b = __ldg(reinterpret_cast<const float4*>(p) + 1);
-        x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+    struct Raw { float4 a, b; };
+    static __device__ __forceinline__ Raw fetch(const float* p) {
+        return {__ldg(reinterpret_cast<const float4*>(p)), __ldg(reinterpret_cast<const float4*>(p) + 1)};
+    }
+    static __device__ __forceinline__ void widen(const Raw& u, float (&x)[8]) {
+        x[0] = u.a.x; x[1] = u.a.y; x[2] = u.a.z; x[3] = u.a.w; x[4] = u.b.x; x[5] = u.b.y; x[6] = u.b.z; x[7] = u.b.w;
     }
 };
 
-template <typename T, bool VEC>
-__global__ void __launch_bounds__(kWarps * 32)
+// One CTA takes ROWS rows and spreads D over its threads (eight columns each per pass), so the loads of a row are 16 bytes
+// a thread and independent of each other: ROWS of them are in flight, whatever the number of rows.  The kernel is bound by
+// HBM for many rows and by one load's latency for few: a warp that walks a row by itself (the former layout, four rows to
+// a warp) took 11 us for ONE row of D = 4096 and read [32768, 2048] bf16 at 4.8 TB/s.  An eight-row CTA reads W_r (from L1)
+// once for eight rows; measured times stand at launch_router.
+template <typename T, int ROWS>
+__global__ void __launch_bounds__(kMaxThreads)
 router_kernel(const T* __restrict__ R, const float* __restrict__ W_r, const float* __restrict__ b_r,
               long long rows, int D, int route, float* __restrict__ gate, float* __restrict__ log2_gate,
               int8_t* __restrict__ idx) {
+    __shared__ float part[kMaxThreads / 32][ROWS * 3];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long row0 = (long long)blockIdx.x * ROWS;
+    const long long last = rows - 1 - row0;                       // a row past the end reads the last one again
+    float acc[ROWS * 3];
+#pragma unroll
+    for (int i = 0; i < ROWS * 3; ++i) acc[i] = 0.f;
+    const T* base = R + row0 * (long long)D;
+    for (int c = threadIdx.x * 8; c < D; c += blockDim.x * 8) {
+        typename Vec8<T>::Raw x[ROWS];
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) x[r] = Vec8<T>::fetch(base + (r <= last ? r : last) * D + c);
+        float w[24];
+        const float4* wp = reinterpret_cast<const float4*>(W_r + (long long)c * 3);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            const float4 v = __ldg(wp + i);
+            w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
+        }
+#pragma unroll
+        for (int r = 0; r < ROWS; ++r) {
+            float f[8];
+            Vec8<T>::widen(x[r], f);
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int l = 0; l < 3; ++l) acc[r * 3 + l] = fmaf(f[i], w[3 * i + l], acc[r * 3 + l]);
+        }
+    }
+    // Sum over the warp: while a lane holds several rows it hands half of them to its partner and adds the partner's
+    // other half, so that eight rows cost 27 shuffles instead of 120; lane group g then holds row g.
+    int held = ROWS, off = 16, row = 0;
+#pragma unroll
+    for (int n = ROWS; n > 1; n >>= 1) {
+        const bool up = (lane & off) != 0;
+#pragma unroll
+        for (int i = 0; i < n / 2 * 3; ++i) {
+            const float give = up ? acc[i] : acc[i + n / 2 * 3];
+            const float got = __shfl_xor_sync(0xffffffffu, give, off);
+            acc[i] = (up ? acc[i + n / 2 * 3] : acc[i]) + got;
+        }
+        held >>= 1;
+        row += up ? held : 0;
+        off >>= 1;
+    }
+    for (; off > 0; off >>= 1)
+#pragma unroll
+        for (int l = 0; l < 3; ++l) acc[l] += __shfl_xor_sync(0xffffffffu, acc[l], off);
+    if ((lane & (32 / ROWS - 1)) == 0) {
+#pragma unroll
+        for (int l = 0; l < 3; ++l) part[warp][row * 3 + l] = acc[l];
+    }
+    __syncthreads();
+    if (threadIdx.x < ROWS && row0 + threadIdx.x < rows) {
+        float g[3] = {0.f, 0.f, 0.f};
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
+#pragma unroll
+            for (int l = 0; l < 3; ++l) g[l] += part[w][threadIdx.x * 3 + l];
+        if (b_r) { g[0] += b_r[0]; g[1] += b_r[1]; g[2] += b_r[2]; }
+        finish_row(g[0], g[1], g[2], route, row0 + threadIdx.x, gate, log2_gate, idx);
+    }
+}
+
+// Any D and alignment: a warp walks four rows, one element a lane.
+template <typename T>
+__global__ void __launch_bounds__(kWarps * 32)
+router_any_kernel(const T* __restrict__ R, const float* __restrict__ W_r, const float* __restrict__ b_r,
+                  long long rows, int D, int route, float* __restrict__ gate, float* __restrict__ log2_gate,
+                  int8_t* __restrict__ idx) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long row0 = ((long long)blockIdx.x * kWarps + warp) * kRowsPerWarp;
     if (row0 >= rows) return;
@@ -88,37 +166,14 @@ router_kernel(const T* __restrict__ R, const float* __restrict__ W_r, const floa
         long long rr = row0 + r < rows ? row0 + r : rows - 1;   // clamp: tail rows recompute the last row
         rp[r] = R + rr * (long long)D;
     }
-    if (VEC) {
-        for (int c = lane * 8; c < D; c += 32 * 8) {
-            float w[24];
-            const float4* wp = reinterpret_cast<const float4*>(W_r + (long long)c * 3);
+    for (int c = lane; c < D; c += 32) {
+        float w0 = W_r[c * 3], w1 = W_r[c * 3 + 1], w2 = W_r[c * 3 + 2];
 #pragma unroll
-            for (int i = 0; i < 6; ++i) {
-                float4 v = __ldg(wp + i);
-                w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
-            }
-#pragma unroll
-            for (int r = 0; r < kRowsPerWarp; ++r) {
-                float x[8];
-                Vec8<T>::load(rp[r] + c, x);
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    acc[r][0] = fmaf(x[i], w[3 * i], acc[r][0]);
-                    acc[r][1] = fmaf(x[i], w[3 * i + 1], acc[r][1]);
-                    acc[r][2] = fmaf(x[i], w[3 * i + 2], acc[r][2]);
-                }
-            }
-        }
-    } else {
-        for (int c = lane; c < D; c += 32) {
-            float w0 = W_r[c * 3], w1 = W_r[c * 3 + 1], w2 = W_r[c * 3 + 2];
-#pragma unroll
-            for (int r = 0; r < kRowsPerWarp; ++r) {
-                float x = Elem<T>::ld(rp[r] + c);
-                acc[r][0] = fmaf(x, w0, acc[r][0]);
-                acc[r][1] = fmaf(x, w1, acc[r][1]);
-                acc[r][2] = fmaf(x, w2, acc[r][2]);
-            }
+        for (int r = 0; r < kRowsPerWarp; ++r) {
+            float x = Elem<T>::ld(rp[r] + c);
+            acc[r][0] = fmaf(x, w0, acc[r][0]);
+            acc[r][1] = fmaf(x, w1, acc[r][1]);
+            acc[r][2] = fmaf(x, w2, acc[r][2]);
         }
     }
 #pragma unroll
@@ -260,21 +315,32 @@ __global__ void __launch_bounds__(256) router_bias_grad_kernel(const float* __re
 
 }  // namespace
 
+namespace {
+template <typename T>
+void router_t(const T* R, const float* W_r, const float* b_r, long long rows, int D, int route, float* gate, float* log2_gate,
+              int8_t* idx, cudaStream_t st) {
+    if (D % 8 || (uintptr_t)R % 16 || (uintptr_t)W_r % 16) {
+        const long long rows_per_cta = kWarps * kRowsPerWarp;
+        router_any_kernel<T><<<(unsigned)((rows + rows_per_cta - 1) / rows_per_cta), kWarps * 32, 0, st>>>(
+            R, W_r, b_r, rows, D, route, gate, log2_gate, idx);
+        return;
+    }
+    // Eight rows to a CTA once that gives every SM one; two rows from 296 on; else one row, for the shortest chain.
+    const int threads = D >= 8 * kMaxThreads ? kMaxThreads : (D / 8 + 31) / 32 * 32;
+    if (rows >= 8 * 148)
+        router_kernel<T, 8><<<(unsigned)((rows + 7) / 8), threads, 0, st>>>(R, W_r, b_r, rows, D, route, gate, log2_gate, idx);
+    else if (rows >= 2 * 148)
+        router_kernel<T, 2><<<(unsigned)((rows + 1) / 2), threads, 0, st>>>(R, W_r, b_r, rows, D, route, gate, log2_gate, idx);
+    else
+        router_kernel<T, 1><<<(unsigned)rows, threads, 0, st>>>(R, W_r, b_r, rows, D, route, gate, log2_gate, idx);
+}
+}  // namespace
+
 cudaError_t launch_router(const void* R, const float* W_r, const float* b_r, long long rows, int D, int r_dtype,
                           int route, float* gate, float* log2_gate, int8_t* idx, cudaStream_t st) {
     if (rows == 0) return cudaSuccess;
-    const long long rows_per_cta = kWarps * kRowsPerWarp;
-    dim3 grid((unsigned)((rows + rows_per_cta - 1) / rows_per_cta)), block(kWarps * 32);
-    const bool vec = (D % 8 == 0) && ((uintptr_t)R % 16 == 0) && ((uintptr_t)W_r % 16 == 0);
-    if (r_dtype == MKA_BF16) {
-        auto* p = static_cast<const __nv_bfloat16*>(R);
-        if (vec) router_kernel<__nv_bfloat16, true><<<grid, block, 0, st>>>(p, W_r, b_r, rows, D, route, gate, log2_gate, idx);
-        else router_kernel<__nv_bfloat16, false><<<grid, block, 0, st>>>(p, W_r, b_r, rows, D, route, gate, log2_gate, idx);
-    } else {
-        auto* p = static_cast<const float*>(R);
-        if (vec) router_kernel<float, true><<<grid, block, 0, st>>>(p, W_r, b_r, rows, D, route, gate, log2_gate, idx);
-        else router_kernel<float, false><<<grid, block, 0, st>>>(p, W_r, b_r, rows, D, route, gate, log2_gate, idx);
-    }
+    if (r_dtype == MKA_BF16) router_t(static_cast<const __nv_bfloat16*>(R), W_r, b_r, rows, D, route, gate, log2_gate, idx, st);
+    else router_t(static_cast<const float*>(R), W_r, b_r, rows, D, route, gate, log2_gate, idx, st);
     return cudaGetLastError();
 }
 
