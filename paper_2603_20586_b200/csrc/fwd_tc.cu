@@ -7,30 +7,36 @@
 //     p = 2^(s * tau * log2(e) + log2(lambda_l) - m)  =  lambda_l * exp(s*tau - m')
 // which is exactly the gated, un-normalised weight of Eq. 5.  One normalisation at the end.
 //
-// Warp roles (d = 128: 320 threads, d = 64: 384 threads):
+// Warp roles (384 threads):
 //   softmax warps    thread = one query row (TMEM lane) x 128 key columns at d = 128 (four warps per query tile), x 64
 //                    columns at d = 64 (eight warps: warp = (column half, lane quarter); the two threads of a row agree
 //                    on the row maximum through shared memory and a 256-thread barrier).  Reads S from TMEM, applies
 //                    bias and masks, running max, exp2, packs the weights to bf16 and writes them to TMEM in parts of
 //                    32 keys (at d = 128 over the columns S occupied), rescales the O accumulator when the running
 //                    maximum grows by more than 2^8 (lazy rescale), and does the epilogue.
-//   next warp        producer: one lane issues the TMA loads of Q and of the K / V tile list into 128-byte-swizzled
-//                    shared-memory rings (one mbarrier pair per stage); with paged levels the whole warp produces.
+//   next warp        producer: the warp waits converged, one lane issues the TMA loads of Q and of the K / V tile list
+//                    into 128-byte-swizzled shared-memory rings (one mbarrier pair per stage); with paged levels every
+//                    lane issues its own box.
 //   next warp        issues every tcgen05.mma (the warp runs its loop converged, one elected lane issues):
 //                    S_q = Q_q K^T (both operands from shared memory) and O_q += P_q V (P from TMEM, V from shared
 //                    memory, N-major) in pieces that follow the parts of P, so that most of the product runs under the
 //                    remaining exponentials.  At d = 128 the order is  S0(e)  O1(e-1)  S1(e)  O0(e):  each tile's
 //                    softmax overlaps the other tile's products.
-//   d = 64 only      two idle warps complete the last warpgroup, so that registers can be moved from it to the softmax
-//                    warpgroups (setmaxnreg): two CTAs per SM leave 80 registers per thread at launch.
+//   last two warps   idle: they complete the last warpgroup, so that registers can be moved from it to the softmax
+//                    warpgroups (setmaxnreg): a launch leaves 168 (d = 64, two CTAs per SM: 80) registers per thread.
 // TMEM: S tiles first (128 columns each), then the O accumulators (d columns each); at d = 64 a P region of 64 columns
 // per query tile follows, and S_q(e+1) is multiplied while the softmax of S_q(e) runs (the hand-off is "S is in
 // registers", not "P has been consumed").  d = 128 uses all 512 columns, d = 64 256.
 // What bounds the d = 128 kernel is the chain  softmax_q(e) -> O_q += P V -> S_q(e+1) -> softmax_q(e+1):  a key tile
 // costs the tensor pipe 2048 cycles and the special-function unit 2048 cycles for the two query tiles, but S_q(e+1)
 // cannot be written before P_q(e), which lies over S_q(e), has been consumed, and TMEM has no room for a second S.
+// A key tile of 256 query rows takes 1.5 us at 1.8 GHz.  Whatever lengthens the softmax lengthens the chain: with the
+// scores held in 168 registers a thread spilled, and the level loop indexed its ranges in local memory: 1.63 us, and
+// [1, 32, 8192, 128] (window 2048, 2048 slots) took 1024 us against 946.
 // Every mbarrier wait is bounded by a wall-clock limit; on expiry the CTA raises a flag in shared
 // memory, writes the device status word, lets every role drain, frees TMEM and returns.
+#include <atomic>
+
 #include "tc_ptx.cuh"
 
 namespace mka {
@@ -69,7 +75,7 @@ struct TcParams {
 template <int DH>
 struct Cfg {
     // d = 128: one CTA per SM with two query tiles (all 512 TMEM columns); a softmax thread owns a whole query row
-    // (128 key columns, 168 registers per thread).
+    // (128 key columns).
     // d = 64: the scores of one key tile cost the special-function unit as much as at d = 128 but only half the
     // tensor work, and the tile lists of the training shapes are short; there a CTA takes ONE query tile (256 TMEM
     // columns) and two CTAs share the SM, so that one CTA's start-up, waits and epilogue run under the other's steady
@@ -79,18 +85,19 @@ struct Cfg {
     static constexpr int kCtasPerSm = DH == 128 ? 1 : 2;
     static constexpr int kSplit = DH == 128 ? 1 : 2;           // threads per query row
     static constexpr int kCols = kTileN / kSplit;             // key columns of one softmax thread
+    static constexpr int kMergeCols = DH == 128 ? 16 : 8;      // columns of a row that a thread merges at a time (kSplitKeys)
     static constexpr int kParts = kCols / 32;                 // the weights of a tile are handed over in parts of 32 keys per thread
     static constexpr int kRowWarps = 4 * kSplit;              // softmax warps per query tile
     static constexpr int kSoftmaxWarps = kRowWarps * kNumQ;
-    static constexpr bool kMoveRegs = kSplit == 2;            // re-divide the registers between the warpgroups (setmaxnreg)
-    // with kMoveRegs the last warpgroup is completed by two idle warps: setmaxnreg is a warpgroup-wide instruction
-    static constexpr int kThreads = (kSoftmaxWarps + (kMoveRegs ? 4 : 2)) * 32;
+    // The registers are re-divided between the warpgroups (setmaxnreg, a warpgroup-wide instruction: two idle warps
+    // complete the last one).  At d = 128 a thread's 128 scores need more than the 168 registers that a launch gives.
+    static constexpr int kThreads = (kSoftmaxWarps + 4) * 32;
     static constexpr int kProducerWarp = kSoftmaxWarps, kMmaWarp = kSoftmaxWarps + 1;
     // What the warpgroups hold after the move must not exceed what the launch gave the CTA, or the increase would
-    // wait forever:  384 threads x 80 registers at launch = 256 x 104 + 128 x 32.
-    static constexpr int kRegsLaunch = 80, kRegsSoftmax = 104, kRegsOther = 32;
-    static_assert(!kMoveRegs || kSoftmaxWarps * 32 * kRegsSoftmax + 4 * 32 * kRegsOther <= kThreads * kRegsLaunch, "register pool of the CTA exceeded");
-    static_assert(!kMoveRegs || kThreads * kCtasPerSm * (kRegsLaunch + 8) > 65536, "the launch would get more than kRegsLaunch registers per thread");
+    // wait forever:  d = 128: 384 threads x 168 registers at launch = 256 x 216 + 128 x 72;  d = 64: 384 x 80 = 256 x 104 + 128 x 32.
+    static constexpr int kRegsLaunch = DH == 128 ? 168 : 80, kRegsSoftmax = DH == 128 ? 216 : 104, kRegsOther = DH == 128 ? 72 : 32;
+    static_assert(kSoftmaxWarps * 32 * kRegsSoftmax + 4 * 32 * kRegsOther <= kThreads * kRegsLaunch, "register pool of the CTA exceeded");
+    static_assert(kThreads * kCtasPerSm * (kRegsLaunch + 8) > 65536, "the launch would get more than kRegsLaunch registers per thread");
     static constexpr int kPanels = DH / 64;
     static constexpr uint32_t kTileBytes = kPanels * kPanelBytes;
     static constexpr int kStages = 2;
@@ -107,6 +114,33 @@ struct Cfg {
 };
 
 constexpr int kMaxQ = 2;
+constexpr int kMaxSplit = 8;              // CTAs of a cluster (the portable limit)
+
+// Value at shared-memory address `addr` (of this CTA's layout) in CTA `rank` of the cluster.
+__device__ __forceinline__ float ld_cluster(uint32_t addr, int rank) {
+    uint32_t remote;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(remote) : "memory");
+    return v;
+}
+// x[l] with l known only at run time, without giving the array an address (it would live in local memory).
+template <typename T> __device__ __forceinline__ T pick3(const T (&x)[3], int l) { return l == 0 ? x[0] : (l == 1 ? x[1] : x[2]); }
+// The n lowest bits, 0 <= n <= 32 after clamping.
+__device__ __forceinline__ uint32_t low_bits(int n) {
+    n = max(0, min(n, 32));
+    return (uint32_t)((1ull << n) - 1ull);
+}
+__device__ __forceinline__ float4 ld_cluster4(uint32_t addr, int rank) {
+    uint32_t remote;
+    float4 v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(remote) : "memory");
+    return v;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
 
 struct Barriers {
     uint64_t q_full;
@@ -116,7 +150,7 @@ struct Barriers {
 };
 
 // Key-tile range [first, end) of a block of query rows [r0, r1] (inclusive) on one level.
-__device__ __forceinline__ void tile_range(int level, long long r0, long long r1, int q_offset, int window, long long n,
+__host__ __device__ __forceinline__ void tile_range(int level, long long r0, long long r1, int q_offset, int window, long long n,
                                            int& first, int& end) {
     long long lo_f, hi_f, lo_l, hi_l;
     visible_range(level, r0 + q_offset, window, n, 0, lo_f, hi_f);
@@ -127,7 +161,10 @@ __device__ __forceinline__ void tile_range(int level, long long r0, long long r1
     end = (int)((hi + kTileN - 1) / kTileN);
 }
 
-template <int DH, bool kPaged>
+// kSplitKeys: the CTAs of a cluster share one block of query rows and split its key-tile list between them (see split_rule).
+// Each ends with its own un-normalised O and (max, sum); they meet in distributed shared memory, so no scratch memory
+// and no second launch is needed.
+template <int DH, bool kPaged, bool kSplitKeys>
 __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
     using C = Cfg<DH>;
     extern __shared__ uint8_t smem_raw[];
@@ -140,19 +177,26 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
     __shared__ WaitCtl wait_ctl;
     __shared__ float xmax[2][C::kNumQ][C::kSplit][kTileM];           // row maxima of the two column halves, double-buffered by tile parity
     __shared__ float lsum[C::kNumQ][C::kSplit][kTileM];              // row sums of the two column halves (epilogue)
+    __shared__ float cl_max[kSplitKeys ? C::kNumQ : 1][kTileM], cl_sum[kSplitKeys ? C::kNumQ : 1][kTileM];   // this CTA's (max, sum) of every row, for its cluster
 
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // tid >> 5, but provably warp-uniform for the compiler
     // Blocks start in the order of their linear index.  Within a group of p.deal (batch, head) pairs the blocks are
     // dealt by query block, heaviest (latest rows) first for every pair of the group, then the next lighter one: the
     // launch then ends with the group's lightest blocks instead of the last head's heaviest.
-    const int lin = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);      // fewer than 2^31 blocks
-    const int per_group = p.deal * (int)gridDim.x;
+    int crank = 0, csize = 1;                                 // this CTA's place in its cluster
+    if constexpr (kSplitKeys) {
+        asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
+        asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(csize));
+    }
+    const int grid_x = (int)gridDim.x / csize;                // blocks of query rows
+    const int lin = (int)blockIdx.x / csize + grid_x * (blockIdx.y + gridDim.y * blockIdx.z);      // fewer than 2^31 blocks
+    const int per_group = p.deal * grid_x;
     const int grp = lin / per_group, in_grp = lin - grp * per_group;
     const int pairs_here = min(p.deal, (int)(gridDim.y * gridDim.z) - grp * p.deal);
     const int hb = grp * p.deal + in_grp % pairs_here;
     const int b = hb / (int)gridDim.y, h = hb - b * (int)gridDim.y;
-    const int qpair = gridDim.x - 1 - in_grp / pairs_here;
+    const int qpair = grid_x - 1 - in_grp / pairs_here;
     const long long m0 = (long long)qpair * (C::kNumQ * kTileM);
     const long long m_last = (m0 + C::kNumQ * kTileM - 1 < p.T - 1) ? m0 + C::kNumQ * kTileM - 1 : p.T - 1;
 
@@ -198,10 +242,23 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
         if (nl[l] > 0) tile_range(l, m0, m_last, p.q_offset, p.window, nl[l], first[l], end[l]);
         else first[l] = end[l] = 0;
     }
+    if constexpr (kSplitKeys) {                               // this CTA's share of the list: tiles [g0, g1)
+        const int total = (end[0] - first[0]) + (end[1] - first[1]) + (end[2] - first[2]);
+        const int g0 = (int)((long long)total * crank / csize), g1 = (int)((long long)total * (crank + 1) / csize);
+        int base = 0;
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+            const int cnt = end[l] - first[l];
+            const int a = min(max(g0 - base, 0), cnt), z = min(max(g1 - base, 0), cnt);
+            end[l] = first[l] + z;
+            first[l] += a;
+            base += cnt;
+        }
+    }
     const int E = (end[0] - first[0]) + (end[1] - first[1]) + (end[2] - first[2]);
 
     if (warp >= C::kSoftmaxWarps) {
-    if constexpr (C::kMoveRegs) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegsOther));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegsOther));
     if (warp == C::kProducerWarp && kPaged) {
         // Paged levels: the whole warp produces.  Lane i owns box i of every key tile (a box = the rows of one page
         // that fall into the tile): it looks its page up while the warp waits for the stage to drain and issues its
@@ -217,20 +274,23 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
         int issued = 0;
         bool ok = true;
         const int kvh = h / p.kv_group;
+#pragma unroll 1
         for (int l = 0; l < 3 && ok; ++l) {
-            if (first[l] >= end[l]) continue;
+            const int kt_first = pick3(first, l), kt_end = pick3(end, l);
+            if (kt_first >= kt_end) continue;
+            const long long n_here = pick3(nl, l);
             const int* tab = p.table[l] + (long long)b * p.table_stride[l] + (long long)kvh * p.table_head_stride[l];
             const int rpb = p.box_rows[l];
             const bool mine = lane < kTileN / rpb;
             const int in_mask = (1 << p.page_shift[l]) - 1;
-            for (int kt = first[l]; kt < end[l]; ++kt) {
+            for (int kt = kt_first; kt < kt_end; ++kt) {
                 const int s = issued % C::kStages;
                 const uint32_t ph = (uint32_t)(issued / C::kStages) & 1u;
                 // a box past the level's last row is aimed past the pool, where the copy engine fills zeros as it does
                 // past a dense level's end
                 const long long row = (long long)kt * kTileN + lane * rpb;
                 int page = p.pool_pages[l];
-                if (mine && row < nl[l]) page = tab[row >> p.page_shift[l]];
+                if (mine && row < n_here) page = tab[row >> p.page_shift[l]];
                 const int in_row = (int)(row & in_mask);
                 if (!mbar_wait_warp(&bar.k_empty[s], ph ^ 1u, abortp)) { ok = false; break; }
                 if (lane == 0) mbar_expect_tx(&bar.k_full[s], C::kTileBytes);
@@ -265,6 +325,8 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
             mbar_wait_warp(&bar.v_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
         }
     } else if (warp == C::kProducerWarp) {
+        // Dense levels: the warp waits converged and one lane issues (inside an `if (lane == 0)` around the whole loop the
+        // kernel keeps its loop state in local memory: 1.63 us per key tile instead of 1.49 at d = 128).
         if (lane == 0) {
             mbar_expect_tx(&bar.q_full, C::kNumQ * C::kTileBytes);
 #pragma unroll
@@ -272,36 +334,46 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
 #pragma unroll
                 for (int pn = 0; pn < C::kPanels; ++pn)
                     tma_load_4d(sQ + q * C::kTileBytes + pn * kPanelBytes, &maps.q, pn * 64, (int)(m0 + q * kTileM), h, b, &bar.q_full);
-            int issued_k = 0, issued_v = 0;
-            bool ok = true;
-            const int kvh = h / p.kv_group;
-            for (int l = 0; l < 3 && ok; ++l) {
-                for (int kt = first[l]; kt < end[l]; ++kt) {
-                    if (p.test_stall && issued_k == E - 1) break;      // test hook: the last tile never arrives
-                    const int e = issued_k;
-                    const int s = e % C::kStages;
-                    const uint32_t ph = (uint32_t)(e / C::kStages) & 1u;
-                    if (!mbar_wait(&bar.k_empty[s], ph ^ 1u, abortp)) { ok = false; break; }
+        }
+        int issued = 0;
+        bool ok = true;
+        const int kvh = h / p.kv_group;
+#pragma unroll 1
+        for (int l = 0; l < 3 && ok; ++l) {
+            const int kt_end = pick3(end, l);
+            for (int kt = pick3(first, l); kt < kt_end; ++kt) {
+                if (p.test_stall && issued == E - 1) break;        // test hook: the last tile never arrives
+                const int s = issued % C::kStages;
+                const uint32_t ph = (uint32_t)(issued / C::kStages) & 1u;
+                if (!mbar_wait_warp(&bar.k_empty[s], ph ^ 1u, abortp)) { ok = false; break; }
+                if (lane == 0) {
                     mbar_expect_tx(&bar.k_full[s], C::kTileBytes);
 #pragma unroll
                     for (int pn = 0; pn < C::kPanels; ++pn)
                         tma_load_4d(sK + s * C::kTileBytes + pn * kPanelBytes, &maps.k[l], pn * 64, kt * kTileN, kvh, b, &bar.k_full[s]);
-                    ++issued_k;
-                    if (!mbar_wait(&bar.v_empty[s], ph ^ 1u, abortp)) { ok = false; break; }
+                }
+                __syncwarp();
+                if (!mbar_wait_warp(&bar.v_empty[s], ph ^ 1u, abortp)) {           // gave up with this stage's K copies in flight
+                    mbar_wait_warp(&bar.k_full[s], ph, abortp);
+                    ok = false;
+                    break;
+                }
+                if (lane == 0) {
                     mbar_expect_tx(&bar.v_full[s], C::kTileBytes);
 #pragma unroll
                     for (int pn = 0; pn < C::kPanels; ++pn)
                         tma_load_4d(sV + s * C::kTileBytes + pn * kPanelBytes, &maps.v[l], pn * 64, kt * kTileN, kvh, b, &bar.v_full[s]);
-                    ++issued_v;
                 }
+                __syncwarp();
+                ++issued;
             }
-            // Before leaving, make sure every copy this lane issued has landed (bounded): the shared
-            // memory must not be handed to another CTA with a bulk copy still in flight.
-            mbar_wait(&bar.q_full, 0, abortp);
-            for (int i = issued_k > C::kStages ? issued_k - C::kStages : 0; i < issued_k; ++i)
-                mbar_wait(&bar.k_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
-            for (int i = issued_v > C::kStages ? issued_v - C::kStages : 0; i < issued_v; ++i)
-                mbar_wait(&bar.v_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
+        }
+        // Before leaving, make sure every copy issued has landed (bounded): the shared memory must not be handed to
+        // another CTA with a bulk copy still in flight.  (A stage whose wait failed got no copies.)
+        mbar_wait_warp(&bar.q_full, 0, abortp);
+        for (int i = issued > C::kStages ? issued - C::kStages : 0; i < issued; ++i) {
+            mbar_wait_warp(&bar.k_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
+            mbar_wait_warp(&bar.v_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
         }
     } else if (warp == C::kMmaWarp) {
         {   // every lane runs the issue loop (converged); elect.sync inside the wrappers picks the issuing lane
@@ -432,7 +504,7 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
         }
     }
     } else {
-        if constexpr (C::kMoveRegs) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(C::kRegsSoftmax));
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(C::kRegsSoftmax));
         // ------------------------------------------------------------ softmax warps
         // warp = (query tile, column part, lane quarter); thread = one query row (TMEM lane) x kCols key columns.
         // With two threads per row (d = 64) they agree on the row maximum through shared memory at a 256-thread barrier
@@ -459,28 +531,34 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
         float m_run = -INFINITY, l_run = 0.f;                                    // l_run: this thread's columns only
         bool ok = true, all_ok = true;                                           // ok is warp-uniform
         int e = 0;
+#pragma unroll 1
         for (int l = 0; l < 3 && all_ok; ++l) {
-            if (first[l] == end[l]) continue;
+            const int kt_first = pick3(first, l), kt_end = pick3(end, l);
+            if (kt_first == kt_end) continue;
+            const long long n_here = pick3(nl, l);
             float bias = -INFINITY;
             int lo = 0, hi = 0;                              // visible rows of this level (levels hold fewer than 2^31 rows)
+            // A row past T has a bias of -inf, so its weights are 0 whatever it sees: it takes the last row's range and
+            // costs its warp no mask of its own.
             if (row_valid) {
                 const float g = p.gate[((long long)b * p.T + t) * 3 + l];
                 bias = g > 0.f ? log2f(g) : -INFINITY;
-                long long lo64, hi64;
-                visible_range(l, (long long)t + p.q_offset, p.window, nl[l], 0, lo64, hi64);
-                lo = (int)lo64; hi = (int)hi64;
             }
             // key tiles visible to every row of THIS query tile need no element mask
-            int full_first = 0, full_end = 0;
+            int full_first = 0, full_end = 0x7fffffff;                     // (a tile without a row inside T masks nothing)
             if (tq0 <= tq1) {
+                {
+                    long long lo64, hi64;
+                    visible_range(l, (row_valid ? (long long)t : tq1) + p.q_offset, p.window, n_here, 0, lo64, hi64);
+                    lo = (int)lo64; hi = (int)hi64;
+                }
                 long long lo_f, hi_f, lo_l, hi_l;
-                visible_range(l, tq0 + p.q_offset, p.window, nl[l], 0, lo_f, hi_f);
-                visible_range(l, tq1 + p.q_offset, p.window, nl[l], 0, lo_l, hi_l);
+                visible_range(l, tq0 + p.q_offset, p.window, n_here, 0, lo_f, hi_f);
+                visible_range(l, tq1 + p.q_offset, p.window, n_here, 0, lo_l, hi_l);
                 full_first = (int)((lo_l + kTileN - 1) / kTileN);
                 full_end = (int)(hi_f / kTileN);
-                if (tq1 - tq0 + 1 < kTileM) full_end = full_first;         // ragged query tile: always mask
             }
-            for (int kt = first[l]; kt < end[l]; ++kt, ++e) {
+            for (int kt = kt_first; kt < kt_end; ++kt, ++e) {
                 if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&bar.s_full[q], (uint32_t)e & 1u, abortp));
                 float s[C::kCols];
                 float mx = -INFINITY;
@@ -497,11 +575,17 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
                     const bool need_mask = !(kt >= full_first && kt < full_end);
                     if (need_mask) {
                         const long long col0 = (long long)kt * kTileN + half * C::kCols;
-                        const int c_lo = (int)max(-1LL, min((long long)lo - col0, (long long)C::kCols));
-                        const int c_hi = (int)max(-1LL, min((long long)hi - col0, (long long)C::kCols));
+                        const int c_lo = (int)max(0LL, min((long long)lo - col0, (long long)C::kCols));
+                        const int c_hi = (int)max(0LL, min((long long)hi - col0, (long long)C::kCols));
+                        // One bit per column: the bits of 32 columns come from two shifts and each costs a test and a select.
+                        // Two comparisons per column made a masked tile take 3.6 us against 1.6 (now 2.1).
 #pragma unroll
-                        for (int c = 0; c < C::kCols; ++c)
-                            if (c < c_lo || c >= c_hi) s[c] = -INFINITY;
+                        for (int c0 = 0; c0 < C::kCols; c0 += 32) {      // 32 columns that no row of the warp masks are passed over
+                            const uint32_t vis = low_bits(c_hi - c0) & ~low_bits(c_lo - c0);
+                            if (__all_sync(0xffffffffu, vis == 0xffffffffu)) continue;
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) s[c0 + i] = (vis >> i) & 1u ? s[c0 + i] : -INFINITY;
+                        }
                     }
                     float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
@@ -594,7 +678,37 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
             if constexpr (C::kSplit == 2) lsum[q][half][row_in_tile] = l_run;   // the row's sum is the sum of its two halves
             all_ok = row_all(ok);
         }
-        if (all_ok) {
+        if constexpr (kSplitKeys) {
+            // Every operand tile has been read when all softmax warps have seen their last product (and no copy is in
+            // flight then), so O may lie over the K and V rings: four columns of all 128 rows, then the next four.
+            if (half == 0) {
+                const bool any = all_ok && E > 0;
+                cl_max[q][row_in_tile] = any ? m_run : -INFINITY;
+                float l_row = l_run;
+                if constexpr (C::kSplit == 2) l_row += lsum[q][1][row_in_tile];
+                cl_sum[q][row_in_tile] = any ? l_row : 0.f;
+            }
+            asm volatile("bar.sync 4, %0;" ::"n"(C::kSoftmaxWarps * 32) : "memory");
+            if (all_ok && !abortp->abort) {
+                tc_fence_after();
+                float4* so = reinterpret_cast<float4*>(sK) + (q * DH + half * (DH / C::kSplit)) / 4 * kTileM + row_in_tile;
+#pragma unroll 1
+                for (int c0 = 0; c0 < DH / C::kSplit; c0 += 32) {
+                    uint32_t o[32];
+                    if (E > 0) {
+                        tmem_ld32(o_addr + c0, o);
+                        tmem_ld_wait();
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) o[i] = 0u;
+                    }
+#pragma unroll
+                    for (int i = 0; i < 32; i += 4)
+                        so[(c0 + i) / 4 * kTileM] = make_float4(__uint_as_float(o[i]), __uint_as_float(o[i + 1]), __uint_as_float(o[i + 2]), __uint_as_float(o[i + 3]));
+                }
+            }
+        }
+        if (!kSplitKeys && all_ok) {
             tc_fence_after();
             float l_row = l_run;
             if constexpr (C::kSplit == 2) l_row += lsum[q][half ^ 1][row_in_tile];
@@ -628,6 +742,76 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
         }
     }
 
+    if constexpr (kSplitKeys) {
+        // Merge: every CTA takes its share of the block's columns, a few at a time, and adds the cluster's parts with the
+        // weights 2^(max_i - max) / sum.  The second barrier keeps a CTA's shared memory alive until all have read it.
+        __syncwarp();
+        cluster_sync();
+        if (warp < C::kSoftmaxWarps) {
+            const int row_in_tile = (warp & 3) * 32 + lane;
+            const uint32_t so = smem_u32(sK) + row_in_tile * 16;
+            float w[kMaxSplit];
+            int have_q = -1;
+            for (int u = crank * (C::kSoftmaxWarps / 4) + (warp >> 2); u < C::kNumQ * DH / C::kMergeCols; u += csize * (C::kSoftmaxWarps / 4)) {
+                const int q = u / (DH / C::kMergeCols), c0 = (u % (DH / C::kMergeCols)) * C::kMergeCols;
+                const int t = (int)m0 + q * kTileM + row_in_tile;
+                if (t >= p.T) continue;
+                if (q != have_q || c0 == 0) {
+                    float mi[kMaxSplit], mx = -INFINITY, sum = 0.f;
+#pragma unroll
+                    for (int i = 0; i < kMaxSplit; ++i) {
+                        mi[i] = i < csize ? ld_cluster(smem_u32(&cl_max[q][row_in_tile]), i) : -INFINITY;
+                        mx = fmaxf(mx, mi[i]);
+                    }
+#pragma unroll
+                    for (int i = 0; i < kMaxSplit; ++i) {
+                        w[i] = mi[i] == -INFINITY ? 0.f : ex2(mi[i] - mx);
+                        if (i < csize) sum = fmaf(w[i], ld_cluster(smem_u32(&cl_sum[q][row_in_tile]), i), sum);
+                    }
+                    const float inv = sum > 0.f ? 1.f / sum : 0.f;       // rows with nothing visible: exact zeros
+#pragma unroll
+                    for (int i = 0; i < kMaxSplit; ++i) w[i] = inv > 0.f ? w[i] * inv : 0.f;
+                    have_q = inv > 0.f ? q : kMaxQ + q;
+                    if (c0 == 0 && p.LSE) p.LSE[((long long)b * p.H + h) * p.T + t] = sum > 0.f ? (mx + log2f(sum)) * kLn2 : -INFINITY;
+                }
+                float acc[C::kMergeCols];
+#pragma unroll
+                for (int c = 0; c < C::kMergeCols; ++c) acc[c] = 0.f;
+                if (have_q == q) {
+#pragma unroll
+                    for (int i0 = 0; i0 < kMaxSplit; i0 += 2) {          // the loads of two parts are in flight together
+                        if (i0 >= csize) break;
+                        const int i1 = i0 + 1 < csize ? i0 + 1 : i0;      // (an odd last part is read twice and added once)
+                        float4 o[2][C::kMergeCols / 4];
+#pragma unroll
+                        for (int c = 0; c < C::kMergeCols; c += 4) {
+                            o[0][c / 4] = ld_cluster4(so + (q * DH + c0 + c) / 4 * (kTileM * 16), i0);
+                            o[1][c / 4] = ld_cluster4(so + (q * DH + c0 + c) / 4 * (kTileM * 16), i1);
+                        }
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            if (i0 + i >= csize) continue;
+#pragma unroll
+                            for (int c = 0; c < C::kMergeCols; c += 4) {
+                                acc[c] = fmaf(w[i0 + i], o[i][c / 4].x, acc[c]); acc[c + 1] = fmaf(w[i0 + i], o[i][c / 4].y, acc[c + 1]);
+                                acc[c + 2] = fmaf(w[i0 + i], o[i][c / 4].z, acc[c + 2]); acc[c + 3] = fmaf(w[i0 + i], o[i][c / 4].w, acc[c + 3]);
+                            }
+                        }
+                    }
+                }
+                __nv_bfloat16* out = p.O + (((long long)b * p.H + h) * p.T + t) * DH + c0;
+#pragma unroll
+                for (int c = 0; c < C::kMergeCols; c += 8) {
+                    uint4 v;
+                    v.x = pack_bf16(acc[c], acc[c + 1]); v.y = pack_bf16(acc[c + 2], acc[c + 3]);
+                    v.z = pack_bf16(acc[c + 4], acc[c + 5]); v.w = pack_bf16(acc[c + 6], acc[c + 7]);
+                    *reinterpret_cast<uint4*>(out + c) = v;
+                }
+            }
+        }
+        __syncwarp();
+        cluster_sync();
+    }
     tc_fence_before();
     __syncthreads();
     if (tid == 0 && wait_ctl.abort) atomicExch(p.status, (unsigned int)MKA_ERR_TIMEOUT);
@@ -636,6 +820,81 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
 
 inline bool make_map(CUtensorMap* map, const void* base, int d, long long rows, int H, int B, long long sn, long long sh, long long sb) {
     return make_bf16_map(map, base, d, rows, H, B, sn, sh, sb, 128);
+}
+
+template <int DH>
+cudaLaunchConfig_t cluster_config(int split, dim3 grid, cudaStream_t st, cudaLaunchAttribute* at) {
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = split; at->val.clusterDim.y = 1; at->val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = grid; cfg.blockDim = dim3(Cfg<DH>::kThreads); cfg.dynamicSmemBytes = Cfg<DH>::kSmemBytes; cfg.stream = st;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    return cfg;
+}
+
+// Clusters of `split` CTAs that the device keeps resident at a time (a cluster stays within one GPC, so this is less than
+// the number of CTAs / split); asked once per device and size.
+template <int DH>
+int resident_clusters(int split) {
+    static std::atomic<int> known[64][kMaxSplit + 1];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    int n = known[dev][split].load(std::memory_order_relaxed);
+    if (n) return n - 1;
+    auto kern = fwd_tc_kernel<DH, false, true>;
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t cfg = cluster_config<DH>(split, dim3(split), nullptr, &at);
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<DH>::kSmemBytes) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        n = 0;
+    }
+    known[dev][split].store(n + 1, std::memory_order_relaxed);
+    return n;
+}
+
+// Key tiles of one block of query rows (device row counts of paged levels are not known here: n bounds them).
+template <int DH>
+int block_tiles(const FwdParams& fp, long long q_block) {
+    const long long r0 = q_block * Cfg<DH>::kNumQ * kTileM;
+    const long long r1 = r0 + Cfg<DH>::kNumQ * kTileM - 1 < fp.T - 1 ? r0 + Cfg<DH>::kNumQ * kTileM - 1 : fp.T - 1;
+    int tiles = 0;
+    for (int l = 0; l < 3; ++l) {
+        int first = 0, end = 0;
+        if (fp.L[l].n > 0) tile_range(l, r0, r1, fp.q_offset, fp.window, fp.L[l].n, first, end);
+        tiles += end - first;
+    }
+    return tiles;
+}
+
+// CTAs that share a block of query rows.  A launch with fewer blocks than the chip holds CTAs (a chunk of a prompt, short
+// sequences) leaves SMs idle while every block walks its whole tile list; splitting the list between the CTAs of a cluster
+// costs each of them its start-up and the merge.  Counted in key tiles (1.5 us at d = 128): 3 for start-up and epilogue,
+// 7 with the merge; blocks start heaviest first, so round r of the resident clusters lasts as long as its first block, and
+// two CTAs on one SM (d = 64) take 1.3 times as long each.  A split has to promise 15 % (below that the model is no better
+// than a coin).  Measured, forward alone, unsplit / split by 2 / 3 / 4 / 5 / 8, chosen in brackets:
+//   d = 128, 28 heads, 512 rows at 15,000 rows of context    263 / [144] / 199 / 160 / 197 / 197 us  (56 blocks, 160 tiles)
+//   d = 128, 12 heads, 700 rows at 6000 rows                 121 / 72 / [56] / 86 / 77 / 91 us       (36 blocks, 71 tiles)
+//   d = 128, 32 heads, 100 rows at 1500 rows                 50 / 34 / 28 / [25] / 43 / 53 us        (32 blocks, 24 tiles)
+//   d = 128, 16 heads, 1500 rows                             [96] / 102 / 109 / 103 / 121 / 167 us   (96 blocks, 36 to 54 tiles)
+//   d = 64, 28 heads, 1500 rows                              [57] / 61 / 75 / 80 / 95 / 138 us       (336 blocks)
+template <int DH>
+int split_rule(const FwdParams& fp, int q_blocks) {
+    const long long pairs = (long long)fp.B * fp.H, blocks = pairs * q_blocks;
+    const int slots = 148 * Cfg<DH>::kCtasPerSm;
+    if (blocks > slots) return 1;
+    int best = 1;
+    double best_cost = 0.85 * (block_tiles<DH>(fp, q_blocks - 1) + 3) * (blocks > 148 ? 1.3 : 1.0);
+    for (int split = 2; split <= kMaxSplit; ++split) {
+        const int fit = resident_clusters<DH>(split);
+        if (fit < 1) continue;
+        double cost = 0.0;
+        for (long long blk = 0; blk < blocks && cost < best_cost; blk += fit)
+            cost += ((double)block_tiles<DH>(fp, q_blocks - 1 - blk / pairs) / split + 7) * (blocks * split > 148 ? (DH == 64 ? 1.3 : 1.0) : 1.0);
+        if (cost < best_cost) { best = split; best_cost = cost; }
+    }
+    return best;
 }
 
 template <int DH>
@@ -683,10 +942,18 @@ cudaError_t launch_t(const FwdParams& fp, unsigned int* status_word, cudaStream_
         const double fit = pair_bytes > 0.0 ? 48.0 * 1024 * 1024 / pair_bytes : pairs;
         p.deal = fit < 1.0 ? 1 : (fit > pairs ? (int)pairs : (int)fit);
     }
-    auto kern = fp.paged ? fwd_tc_kernel<DH, true> : fwd_tc_kernel<DH, false>;
+    const int q_blocks = (fp.T + Cfg<DH>::kNumQ * kTileM - 1) / (Cfg<DH>::kNumQ * kTileM);
+    const int split = split_rule<DH>(fp, q_blocks);
+    auto kern = fp.paged ? (split > 1 ? fwd_tc_kernel<DH, true, true> : fwd_tc_kernel<DH, true, false>)
+                         : (split > 1 ? fwd_tc_kernel<DH, false, true> : fwd_tc_kernel<DH, false, false>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<DH>::kSmemBytes);
     if (e != cudaSuccess) return e;
-    dim3 grid((fp.T + Cfg<DH>::kNumQ * kTileM - 1) / (Cfg<DH>::kNumQ * kTileM), fp.H, fp.B);
+    if (split > 1) {
+        cudaLaunchAttribute at;
+        const cudaLaunchConfig_t cfg = cluster_config<DH>(split, dim3(q_blocks * split, fp.H, fp.B), st, &at);
+        return cudaLaunchKernelEx(&cfg, kern, maps, p);
+    }
+    dim3 grid(q_blocks, fp.H, fp.B);
     kern<<<grid, Cfg<DH>::kThreads, Cfg<DH>::kSmemBytes, st>>>(maps, p);
     return cudaGetLastError();
 }

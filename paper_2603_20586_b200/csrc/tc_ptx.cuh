@@ -79,18 +79,19 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 // The same descriptors split into their two 32-bit words.  The high word is one constant for every operand of
-// these kernels; the low word is the start-address field (address >> 4: shared-memory addresses are
-// below 256 KB, so the 14-bit field cannot overflow and byte offsets are simply added as offset >> 4)
+// these kernels; the low word is the start-address field (address >> 4: shared memory is smaller than 256 KB,
+// so the 14-bit field cannot overflow and byte offsets are simply added as offset >> 4; in a cluster the
+// address of a CTA's own shared memory carries its rank in higher bits, which are masked off)
 // plus the leading-dimension field.  The issuing warp then spends one add per operand and matrix product.
 constexpr uint32_t kDescHi = 64u | (1u << 14) | (2u << 29);
-__device__ __forceinline__ uint32_t desc_lo_kmajor(uint32_t addr) { return (addr >> 4) | (1u << 16); }
+__device__ __forceinline__ uint32_t desc_lo_kmajor(uint32_t addr) { return ((addr >> 4) & 0x3FFF) | (1u << 16); }
 __device__ __forceinline__ uint32_t desc_lo_mnmajor(uint32_t addr, uint32_t panel_stride_bytes) {
-    return (addr >> 4) | ((panel_stride_bytes >> 4) << 16);
+    return ((addr >> 4) & 0x3FFF) | ((panel_stride_bytes >> 4) << 16);
 }
 // Descriptor words of a K-major operand slab WITHOUT swizzle, 16 columns (one K-step) wide: core matrices of 8 rows x 16
 // bytes; the two core matrices of a row group lie 128 bytes apart (leading-dimension field), row groups 256 bytes apart.
 constexpr uint32_t kDescHiFlat = (256u >> 4) | (1u << 14);
-__device__ __forceinline__ uint32_t desc_lo_flat(uint32_t addr) { return (addr >> 4) | ((128u >> 4) << 16); }
+__device__ __forceinline__ uint32_t desc_lo_flat(uint32_t addr) { return ((addr >> 4) & 0x3FFF) | ((128u >> 4) << 16); }
 __device__ __forceinline__ uint64_t make_desc_flat(uint32_t lo) {
     uint64_t d;
     asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(kDescHiFlat));

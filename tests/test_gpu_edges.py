@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 import torch
 
-from gpu_helpers import err, np64, problem
+from gpu_helpers import check, err, np64, problem
 
 pytestmark = pytest.mark.gpu
 
@@ -33,3 +33,32 @@ def test_router_rows_per_cta(mka, orc, dtype, rows, D):
     # the same rows one at a time: the row count moves the sums to another split, not to another row
     one = torch.cat([mka.mka_router(X[r:r + 1], W, b) for r in (0, rows // 2, rows - 1)])
     assert np.abs(np64(one) - ref[[0, rows // 2, rows - 1]]).max() <= 2e-6
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("B,H,Hkv,T,W,q_off,N", [
+    (1, 2, 2, 130, 700, 1870, (2000, 2000, 300)),        # a few blocks, long lists: the widest cluster
+    (1, 4, 1, 257, 129, 1000, (1257, 1257, 0)),          # a block with one row, no long-term level, window edges inside
+    (1, 1, 1, 1, 1, 900, (901, 901, 1)),                 # one row; the window is its own tile
+    (2, 20, 4, 300, 64, 0, (300, 300, 2100)),            # the first rows see little of a list that the long-term level fills
+    (1, 3, 3, 64, 5000, 4000, (4064, 100, 17)),          # window wider than the level, short session level
+])
+def test_fwd_key_tiles_split_between_ctas(mka, orc, d, B, H, Hkv, T, W, q_off, N):
+    """Few blocks of query rows: the key-tile list is split over a cluster and merged (also in its ragged and masked parts)."""
+    P = problem(31, B, H, T, d, N, 64, torch.bfloat16, router_std=0.5)
+    K, V = ([x[:, :Hkv].contiguous() for x in P[k]] for k in ("K", "V"))
+    shape = mka.make_shape(B, H, T, d, 64, W, q_off, kv_heads=Hkv)
+    assert mka.mka_fwd_kernel_kind(shape, K, V) == 1
+    for route in (mka.binding.MKA_ROUTE_SOFT, mka.binding.MKA_ROUTE_TOP1):      # TOP1: whole levels weigh 0 for a row
+        gate = mka.mka_router(P["X"], P["W_r"], None, route=route)
+        ws = mka.alloc_workspace(shape, N, mka.binding.MKA_WS_FWD, "cuda")
+        O, LSE = mka.mka_fwd(shape, P["Q"], K, V, gate, ws=ws)
+        assert mka.mka_device_status(ws) == 0
+        rep = [[x.repeat_interleave(H // Hkv, 1) for x in t] for t in (K, V)]
+        Or, Lr = orc.fwd(P["Q"], rep[0], rep[1], np64(gate), W, q_off)
+        check(O, Or, torch.bfloat16, "O")
+        finite = np.isfinite(Lr)
+        assert np.array_equal(np.isfinite(np64(LSE)), finite)
+        assert np.abs(np64(LSE)[finite] - Lr[finite]).max() <= 2e-3
+        again, _ = mka.mka_fwd(shape, P["Q"], K, V, gate, ws=ws)
+        assert torch.equal(O, again)
