@@ -188,6 +188,18 @@ __global__ void __launch_bounds__(256) bwd_prep_kernel(const __nv_bfloat16* __re
     }
 }
 
+// Scores outside columns [c_lo, c_hi) of the thread's 64 become -inf: one bit per column, so a column costs a test and a
+// select; 32 columns that no row of the warp masks are passed over.
+__device__ __forceinline__ void mask_cols(float (&x)[64], int c_lo, int c_hi) {
+#pragma unroll
+    for (int c0 = 0; c0 < 64; c0 += 32) {
+        const uint32_t vis = low_bits(c_hi - c0) & ~low_bits(c_lo - c0);
+        if (__all_sync(0xffffffffu, vis == 0xffffffffu)) continue;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) x[c0 + i] = (vis >> i) & 1u ? x[c0 + i] : -INFINITY;
+    }
+}
+
 // Key tile range [first, end) (128-row units) of query rows [r0, r1] on one level.
 __device__ __forceinline__ void key_tile_range(int level, long long r0, long long r1, int q_offset, int window, long long n,
                                                int& first, int& end) {
@@ -380,7 +392,8 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
         for (int l = 0; l < 3; ++l) {
             if (!ok || first[l] == end[l]) continue;
             long long lo = 0, hi = 0;
-            if (row_valid) visible_range(l, t + p.q_offset, p.window, p.n[l], 0, lo, hi);
+            // a row past T has a bias of -inf, so its weights are 0 whatever it sees: it takes the last row's range
+            visible_range(l, (row_valid ? t : m_last) + p.q_offset, p.window, p.n[l], 0, lo, hi);
             int full_first = 0, full_end = 0;
             {
                 long long lo_f, hi_f, lo_l, hi_l;
@@ -388,7 +401,6 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
                 visible_range(l, m_last + p.q_offset, p.window, p.n[l], 0, lo_l, hi_l);
                 full_first = (int)((lo_l + kBlk - 1) / kBlk);
                 full_end = (int)(hi_f / kBlk);
-                if (m_last - m0 + 1 < kBlk) full_end = full_first;          // ragged query tile: always mask
             }
             // sums over this thread's columns as packed pairs (even, odd column)
             uint64_t a2 = pack2(0.f, 0.f), z2 = a2;
@@ -409,11 +421,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
                 }
                 if (!(kt >= full_first && kt < full_end)) {
                     const long long j0 = (long long)kt * kBlk + w * 64;
-                    const int c_lo = (int)max(-1LL, min(lo - j0, 64LL));
-                    const int c_hi = (int)max(-1LL, min(hi - j0, 64LL));
-#pragma unroll
-                    for (int c = 0; c < 64; ++c)
-                        if (c < c_lo || c >= c_hi) pr[c] = -INFINITY;
+                    mask_cols(pr, (int)max(0LL, min(lo - j0, 64LL)), (int)max(0LL, min(hi - j0, 64LL)));
                 }
 #pragma unroll
                 for (int c = 0; c < 64; c += 2) {
@@ -760,12 +768,10 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
         const uint32_t s_addr = tmem + lane_base + kColS + w * 64;
         const uint32_t dp_addr = tmem + lane_base + kColDP + w * 64;
         // queries [q_lo, q_hi) that see key j (the bound t < T is carried by the padded biases)
-        long long q_lo = 0, q_hi = 0;
-        if (row_valid) {
-            q_lo = lvl == 2 ? 0 : j - p.q_offset;
-            q_hi = lvl == 0 ? j + p.window - p.q_offset : (long long)p.Tpad;
-        }
-        const bool rows_full = j0 + kBlk - 1 < n;
+        // a key past n has its own row of dK and dV, which nobody stores: it takes the last key's range and needs no mask
+        const long long j_see = row_valid ? j : j_last;
+        const long long q_lo = lvl == 2 ? 0 : j_see - p.q_offset;
+        const long long q_hi = lvl == 0 ? j_see + p.window - p.q_offset : (long long)p.Tpad;
         bool ok = true;
         int eq = 0;                                                    // tile within the current query head
         for (int e = 0; e < E; ++e) {
@@ -782,16 +788,12 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
             tmem_ld32(s_addr + 32, reinterpret_cast<uint32_t*>(pr) + 32);
             tmem_ld_wait();
             // tiles whose every (key, query) pair is visible need no mask
-            bool full = rows_full;
+            bool full = true;
             if (lvl != 2) full = full && (j_last - p.q_offset <= tt);
             if (lvl == 0) full = full && (j0 + p.window - p.q_offset >= tt + kBlk);
             if (!full) {
                 const long long c0 = tt + w * 64;
-                const int c_lo = (int)max(-1LL, min(q_lo - c0, 64LL));
-                const int c_hi = (int)max(-1LL, min(q_hi - c0, 64LL));
-#pragma unroll
-                for (int c = 0; c < 64; ++c)
-                    if (c < c_lo || c >= c_hi) pr[c] = -INFINITY;
+                mask_cols(pr, (int)max(0LL, min(q_lo - c0, 64LL)), (int)max(0LL, min(q_hi - c0, 64LL)));
             }
             uint32_t pk[32];        // P^T rounded to bf16; phase 2 uses these same rounded values
             const uint64_t scale2 = pack2(p.scale_log2, p.scale_log2);

@@ -124,13 +124,6 @@ __device__ __forceinline__ float ld_cluster(uint32_t addr, int rank) {
     asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(remote) : "memory");
     return v;
 }
-// x[l] with l known only at run time, without giving the array an address (it would live in local memory).
-template <typename T> __device__ __forceinline__ T pick3(const T (&x)[3], int l) { return l == 0 ? x[0] : (l == 1 ? x[1] : x[2]); }
-// The n lowest bits, 0 <= n <= 32 after clamping.
-__device__ __forceinline__ uint32_t low_bits(int n) {
-    n = max(0, min(n, 32));
-    return (uint32_t)((1ull << n) - 1ull);
-}
 __device__ __forceinline__ float4 ld_cluster4(uint32_t addr, int rank) {
     uint32_t remote;
     float4 v;

@@ -183,6 +183,13 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
     return d;
 }
+// The n lowest bits, 0 <= n <= 32 after clamping.
+__device__ __forceinline__ uint32_t low_bits(int n) {
+    n = max(0, min(n, 32));
+    return (uint32_t)((1ull << n) - 1ull);
+}
+// x[l] with l known only at run time, without giving the array an address (it would live in local memory).
+template <typename T> __device__ __forceinline__ T pick3(const T (&x)[3], int l) { return l == 0 ? x[0] : (l == 1 ? x[1] : x[2]); }
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     uint32_t r;
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
