@@ -512,7 +512,9 @@ mka_status mka_bwd(const mka_shape* s, const void* Q, const mka_level L[3], cons
     if (e == cudaErrorNotSupported) return MKA_ERR_UNSUPPORTED;
     if (e != cudaSuccess) return MKA_ERR_CUDA;
     if (dW_r || db_r) {
-        e = launch_router_bwd(R, r_dtype, dG, (long long)s->B * s->T, s->D, dW_r, db_r, rpart, kRouterBwdChunks, cs);
+        // the statistics have had their last reader: their room takes the chunks' sums of dG
+        double* db_part = bwd_stats_bytes(s) >= kRouterBwdChunks * 3 * sizeof(double) ? reinterpret_cast<double*>(p.stats) : nullptr;
+        e = launch_router_bwd(R, r_dtype, dG, (long long)s->B * s->T, s->D, dW_r, db_r, rpart, db_part, kRouterBwdChunks, cs);
         if (e != cudaSuccess) return MKA_ERR_CUDA;
     }
     return MKA_OK;

@@ -130,32 +130,38 @@ __device__ __forceinline__ void softmax_group_sync() { asm volatile("bar.sync 1,
 // ------------------------------------------------------------------------------------------ prep
 // D = dO . O and the three exponent biases of every padded row.  DH / 8 lanes share a row (one 16-byte load of O and
 // one of dO each), a warp covers 2 or 4 rows per pass and a thread works on four passes at once, so eight loads are
-// in flight per thread.  Padding rows (t >= T) get a bias of -inf so that a streamed sub-tile may run past the last
-// query without a mask.
+// in flight per thread; the row's LSE and gate are fetched with them.  blockIdx.y is the (batch, head): with the row split
+// by 64-bit divisions the arithmetic took most of the time (2.5 TB/s).  Padding rows (t >= T) get a bias of -inf so
+// that a streamed sub-tile may run past the last query without a mask.
 template <int DH>
 __global__ void __launch_bounds__(256) bwd_prep_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfloat16* __restrict__ dO,
                                                        const float* __restrict__ LSE, const float* __restrict__ gate, int H,
-                                                       int T, int Tpad, long long rows_pad, float* __restrict__ sD,
+                                                       int T, int Tpad, float* __restrict__ sD,
                                                        float* __restrict__ b0, float* __restrict__ b1, float* __restrict__ b2) {
     constexpr int LPR = DH / 8;                            // lanes per row: 16 or 8
     constexpr int RPW = 32 / LPR;                          // rows per warp and pass
     constexpr int kPasses = 4;
     const int lane = threadIdx.x & 31, sub = lane % LPR, grp = lane / LPR;
-    const long long warp_row0 = ((long long)blockIdx.x * 8 + (threadIdx.x >> 5)) * (RPW * kPasses);
+    const long long bh = (long long)blockIdx.z * H + blockIdx.y;
+    const int row0 = (blockIdx.x * 8 + (threadIdx.x >> 5)) * (RPW * kPasses) + grp;
+    const __nv_bfloat16* Ob = O + bh * T * DH + sub * 8;
+    const __nv_bfloat16* dOb = dO + bh * T * DH + sub * 8;
     uint4 a[kPasses], g[kPasses];
-    long long rr[kPasses];
-    bool in[kPasses];
+    float lse[kPasses], gt[kPasses][3];
 #pragma unroll
     for (int u = 0; u < kPasses; ++u) {
-        rr[u] = warp_row0 + u * RPW + grp;
-        const long long bh = rr[u] / Tpad;
-        const int t = (int)(rr[u] % Tpad);
-        in[u] = rr[u] < rows_pad && t < T;
+        const int t = row0 + u * RPW;
         a[u] = g[u] = make_uint4(0u, 0u, 0u, 0u);
-        if (in[u]) {
-            const long long off = (bh * T + t) * DH + sub * 8;
-            a[u] = __ldg(reinterpret_cast<const uint4*>(O + off));
-            g[u] = __ldg(reinterpret_cast<const uint4*>(dO + off));
+        lse[u] = -INFINITY;
+        gt[u][0] = gt[u][1] = gt[u][2] = 0.f;
+        if (t < T) {
+            a[u] = __ldg(reinterpret_cast<const uint4*>(Ob + (long long)t * DH));
+            g[u] = __ldg(reinterpret_cast<const uint4*>(dOb + (long long)t * DH));
+            if (sub == 0) {
+                lse[u] = LSE[bh * T + t];
+                const float* gr = gate + ((long long)blockIdx.z * T + t) * 3;
+                gt[u][0] = gr[0]; gt[u][1] = gr[1]; gt[u][2] = gr[2];
+            }
         }
     }
 #pragma unroll
@@ -169,21 +175,15 @@ __global__ void __launch_bounds__(256) bwd_prep_kernel(const __nv_bfloat16* __re
         }
 #pragma unroll
         for (int o = LPR / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (sub == 0 && rr[u] < rows_pad) {
-            float o0 = -INFINITY, o1 = -INFINITY, o2 = -INFINITY;
-            if (in[u]) {
-                const long long bh = rr[u] / Tpad;
-                const int t = (int)(rr[u] % Tpad);
-                const float lse = LSE[bh * T + t];
-                const float* gt = gate + ((bh / H) * T + t) * 3;
-                const bool live = lse > -INFINITY;
-                const float l2 = lse * kLog2e;
-                o0 = (live && gt[0] > 0.f) ? log2f(gt[0]) - l2 : -INFINITY;
-                o1 = (live && gt[1] > 0.f) ? log2f(gt[1]) - l2 : -INFINITY;
-                o2 = (live && gt[2] > 0.f) ? log2f(gt[2]) - l2 : -INFINITY;
-            }
-            sD[rr[u]] = in[u] ? s : 0.f;
-            b0[rr[u]] = o0; b1[rr[u]] = o1; b2[rr[u]] = o2;
+        const int t = row0 + u * RPW;
+        if (sub == 0 && t < Tpad) {
+            const bool live = lse[u] > -INFINITY;
+            const float l2 = lse[u] * kLog2e;
+            const long long at = bh * Tpad + t;
+            sD[at] = s;
+            b0[at] = (live && gt[u][0] > 0.f) ? log2f(gt[u][0]) - l2 : -INFINITY;
+            b1[at] = (live && gt[u][1] > 0.f) ? log2f(gt[u][1]) - l2 : -INFINITY;
+            b2[at] = (live && gt[u][2] > 0.f) ? log2f(gt[u][2]) - l2 : -INFINITY;
         }
     }
 }
@@ -892,9 +892,9 @@ cudaError_t launch_t(const BwdParams& bp, unsigned int* status_word, cudaStream_
     const long long sq_n = DH, sq_h = (long long)bp.T * DH, sq_b = (long long)bp.H * bp.T * DH;
 
     constexpr int kPrepRowsPerBlock = 8 * (32 / (DH / 8)) * 4;          // 8 warps x rows per pass x passes
-    bwd_prep_kernel<DH><<<(unsigned)((rows_pad + kPrepRowsPerBlock - 1) / kPrepRowsPerBlock), 256, 0, st>>>(
+    bwd_prep_kernel<DH><<<dim3((Tpad + kPrepRowsPerBlock - 1) / kPrepRowsPerBlock, bp.H, bp.B), 256, 0, st>>>(
         static_cast<const __nv_bfloat16*>(bp.O), static_cast<const __nv_bfloat16*>(bp.dO), bp.LSE, bp.gate, bp.H, bp.T, Tpad,
-        rows_pad, statD, statB[0], statB[1], statB[2]);
+        statD, statB[0], statB[1], statB[2]);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
 

@@ -154,7 +154,7 @@ struct BwdParams {
 };
 cudaError_t launch_bwd_simt(const BwdParams& p, int dtype, cudaStream_t st);
 cudaError_t launch_router_bwd(const void* R, int r_dtype, const float* dG, long long rows, int D, float* dW_r,
-                              float* db_r, float* partial, int n_row_chunks, cudaStream_t st);
+                              float* db_r, float* partial, double* db_partial, int n_row_chunks, cudaStream_t st);
 
 cudaError_t launch_fuse_kv(const LevelDev L[3], const LevelGradDev& out, const float* gate, int B, int H, long long n, int d,
                            long long dst_offset, int dtype, cudaStream_t st, const int* dst_table = nullptr,

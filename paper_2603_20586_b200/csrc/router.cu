@@ -1,7 +1,6 @@
 // Router gate kernel: lambda = softmax over three levels of (R W_r + b_r), one gate per token
 // (Alg. 1 step 12 / Alg. 2 step 5), plus the hard top-1 / top-2 and uniform routing variants
-// (Table 10).  HBM-bound: every row of R is read exactly once with 16-byte loads; each warp owns
-// four rows at a time so that one read of W_r serves four rows.
+// (Table 10).  HBM-bound for many rows, latency-bound for few: every row of R is read exactly once with 16-byte loads.
 // Also the router's backward: dW_r = R^T dG, db_r = sum dG (two deterministic passes).
 #include "common.cuh"
 
@@ -75,11 +74,35 @@ template <> struct Vec8<float> {
     }
 };
 
+// Sums of ROWS rows x 3 logits over a warp: while a lane holds several rows it hands half of them to its partner and adds
+// the partner's other half, so that eight rows cost 27 shuffles instead of 120.  The lanes of group `row` (32 / ROWS of
+// them) end with that row's sums in acc[0..2].
+template <int ROWS>
+__device__ __forceinline__ void sum_rows(float (&acc)[ROWS * 3], int lane, int& row) {
+    int held = ROWS, off = 16;
+    row = 0;
+#pragma unroll
+    for (int n = ROWS; n > 1; n >>= 1) {
+        const bool up = (lane & off) != 0;
+#pragma unroll
+        for (int i = 0; i < n / 2 * 3; ++i) {
+            const float give = up ? acc[i] : acc[i + n / 2 * 3];
+            const float got = __shfl_xor_sync(0xffffffffu, give, off);
+            acc[i] = (up ? acc[i + n / 2 * 3] : acc[i]) + got;
+        }
+        held >>= 1;
+        row += up ? held : 0;
+        off >>= 1;
+    }
+    for (; off > 0; off >>= 1)
+#pragma unroll
+        for (int l = 0; l < 3; ++l) acc[l] += __shfl_xor_sync(0xffffffffu, acc[l], off);
+}
+
 // One CTA takes ROWS rows and spreads D over its threads (eight columns each per pass), so the loads of a row are 16 bytes
 // a thread and independent of each other: ROWS of them are in flight, whatever the number of rows.  The kernel is bound by
-// HBM for many rows and by one load's latency for few: a warp that walks a row by itself (the former layout, four rows to
-// a warp) took 11 us for ONE row of D = 4096 and read [32768, 2048] bf16 at 4.8 TB/s.  An eight-row CTA reads W_r (from L1)
-// once for eight rows; measured times stand at launch_router.
+// one load's latency: a warp that walks four rows by itself took 11 us for ONE row of D = 4096.  With thousands of rows
+// the order turns round (see router_rows_kernel).
 template <typename T, int ROWS>
 __global__ void __launch_bounds__(kMaxThreads)
 router_kernel(const T* __restrict__ R, const float* __restrict__ W_r, const float* __restrict__ b_r,
@@ -114,25 +137,8 @@ router_kernel(const T* __restrict__ R, const float* __restrict__ W_r, const floa
                 for (int l = 0; l < 3; ++l) acc[r * 3 + l] = fmaf(f[i], w[3 * i + l], acc[r * 3 + l]);
         }
     }
-    // Sum over the warp: while a lane holds several rows it hands half of them to its partner and adds the partner's
-    // other half, so that eight rows cost 27 shuffles instead of 120; lane group g then holds row g.
-    int held = ROWS, off = 16, row = 0;
-#pragma unroll
-    for (int n = ROWS; n > 1; n >>= 1) {
-        const bool up = (lane & off) != 0;
-#pragma unroll
-        for (int i = 0; i < n / 2 * 3; ++i) {
-            const float give = up ? acc[i] : acc[i + n / 2 * 3];
-            const float got = __shfl_xor_sync(0xffffffffu, give, off);
-            acc[i] = (up ? acc[i + n / 2 * 3] : acc[i]) + got;
-        }
-        held >>= 1;
-        row += up ? held : 0;
-        off >>= 1;
-    }
-    for (; off > 0; off >>= 1)
-#pragma unroll
-        for (int l = 0; l < 3; ++l) acc[l] += __shfl_xor_sync(0xffffffffu, acc[l], off);
+    int row = 0;
+    sum_rows<ROWS>(acc, lane, row);
     if ((lane & (32 / ROWS - 1)) == 0) {
 #pragma unroll
         for (int l = 0; l < 3; ++l) part[warp][row * 3 + l] = acc[l];
@@ -145,6 +151,48 @@ router_kernel(const T* __restrict__ R, const float* __restrict__ W_r, const floa
             for (int l = 0; l < 3; ++l) g[l] += part[w][threadIdx.x * 3 + l];
         if (b_r) { g[0] += b_r[0]; g[1] += b_r[1]; g[2] += b_r[2]; }
         finish_row(g[0], g[1], g[2], route, row0 + threadIdx.x, gate, log2_gate, idx);
+    }
+}
+
+// Many rows: a warp owns four of them and walks D by itself; one read of W_r serves the four, nothing waits for a CTA's
+// slowest warp and no barrier follows.
+template <typename T>
+__global__ void __launch_bounds__(kWarps * 32)
+router_rows_kernel(const T* __restrict__ R, const float* __restrict__ W_r, const float* __restrict__ b_r,
+                   long long rows, int D, int route, float* __restrict__ gate, float* __restrict__ log2_gate,
+                   int8_t* __restrict__ idx) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long row0 = ((long long)blockIdx.x * kWarps + warp) * kRowsPerWarp;
+    if (row0 >= rows) return;
+    float acc[kRowsPerWarp * 3];
+#pragma unroll
+    for (int i = 0; i < kRowsPerWarp * 3; ++i) acc[i] = 0.f;
+    const T* rp[kRowsPerWarp];
+#pragma unroll
+    for (int r = 0; r < kRowsPerWarp; ++r) rp[r] = R + (row0 + r < rows ? row0 + r : rows - 1) * (long long)D;   // a row past the end reads the last one again
+    for (int c = lane * 8; c < D; c += 32 * 8) {
+        float w[24];
+        const float4* wp = reinterpret_cast<const float4*>(W_r + (long long)c * 3);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            const float4 v = __ldg(wp + i);
+            w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
+        }
+#pragma unroll
+        for (int r = 0; r < kRowsPerWarp; ++r) {
+            float f[8];
+            Vec8<T>::widen(Vec8<T>::fetch(rp[r] + c), f);
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+#pragma unroll
+                for (int l = 0; l < 3; ++l) acc[r * 3 + l] = fmaf(f[i], w[3 * i + l], acc[r * 3 + l]);
+        }
+    }
+    int row = 0;
+    sum_rows<kRowsPerWarp>(acc, lane, row);
+    if ((lane & (32 / kRowsPerWarp - 1)) == 0 && row0 + row < rows) {
+        if (b_r) { acc[0] += b_r[0]; acc[1] += b_r[1]; acc[2] += b_r[2]; }
+        finish_row(acc[0], acc[1], acc[2], route, row0 + row, gate, log2_gate, idx);
     }
 }
 
@@ -222,95 +270,127 @@ router_bwd_partial_kernel(const T* __restrict__ R, const float* __restrict__ dG,
     }
 }
 
-// The same with four consecutive columns per thread (one 8- or 16-byte load per row), rows taken four at a time so that
-// four loads are in flight; used when D is a multiple of 4 and R is 16-byte aligned.  Per column the rows are added in
-// the same order as above.
-template <typename T>
-__global__ void __launch_bounds__(256)
-router_bwd_partial4_kernel(const T* __restrict__ R, const float* __restrict__ dG, long long rows, int D,
-                           int n_row_chunks, float* __restrict__ partial) {
-    const int c = (blockIdx.x * 256 + threadIdx.x) * 4;
-    const int chunk = blockIdx.y;
-    const long long per = (rows + n_row_chunks - 1) / n_row_chunks;
-    const long long r0 = chunk * per, r1 = r0 + per < rows ? r0 + per : rows;
-    __shared__ float g[64][3];
-    float a[4][3];
+// Sum of rows [r0, r1) of a [rows, 3] array by the 256 threads of a CTA, valid in thread 0.
+template <typename V>
+__device__ __forceinline__ void sum_dG(const V* __restrict__ x, long long r0, long long r1, double (&sm)[256][3], double (&a)[3]) {
+    a[0] = a[1] = a[2] = 0.0;
+    for (long long r = r0 + threadIdx.x; r < r1; r += 256)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) a[j][0] = a[j][1] = a[j][2] = 0.f;
-    auto load4 = [&](long long r, float (&x)[4]) {
-        if (sizeof(T) == 2) {
-            const uint2 w = __ldg(reinterpret_cast<const uint2*>(R + r * (long long)D + c));
-            x[0] = __uint_as_float(w.x << 16); x[1] = __uint_as_float(w.x & 0xffff0000u);
-            x[2] = __uint_as_float(w.y << 16); x[3] = __uint_as_float(w.y & 0xffff0000u);
-        } else {
-            const float4 w = __ldg(reinterpret_cast<const float4*>(R + r * (long long)D + c));
-            x[0] = w.x; x[1] = w.y; x[2] = w.z; x[3] = w.w;
-        }
-    };
-    for (long long rb = r0; rb < r1; rb += 64) {
-        __syncthreads();
-        if (threadIdx.x < 64 * 3) {
-            long long rr = rb + threadIdx.x / 3;
-            g[threadIdx.x / 3][threadIdx.x % 3] = rr < r1 ? dG[rr * 3 + threadIdx.x % 3] : 0.f;
-        }
-        __syncthreads();
-        if (c < D) {
-            const int lim = (int)((r1 - rb) < 64 ? (r1 - rb) : 64);
-            int i = 0;
-            for (; i + 4 <= lim; i += 4) {
-                float x[4][4];
+        for (int l = 0; l < 3; ++l) a[l] += (double)x[r * 3 + l];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) load4(rb + i + u, x[u]);
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        a[j][0] = fmaf(x[u][j], g[i + u][0], a[j][0]);
-                        a[j][1] = fmaf(x[u][j], g[i + u][1], a[j][1]);
-                        a[j][2] = fmaf(x[u][j], g[i + u][2], a[j][2]);
-                    }
-            }
-            for (; i < lim; ++i) {
-                float x[4];
-                load4(rb + i, x);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    a[j][0] = fmaf(x[j], g[i][0], a[j][0]); a[j][1] = fmaf(x[j], g[i][1], a[j][1]); a[j][2] = fmaf(x[j], g[i][2], a[j][2]);
-                }
-            }
-        }
-    }
-    if (c < D) {
-        float* o = partial + ((long long)chunk * D + c) * 3;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) { o[3 * j] = a[j][0]; o[3 * j + 1] = a[j][1]; o[3 * j + 2] = a[j][2]; }
-    }
-}
-
-__global__ void router_bwd_reduce_kernel(const float* __restrict__ partial, int D, int n_row_chunks,
-                                         float* __restrict__ dW_r) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;   // over D*3
-    if (i >= D * 3) return;
-    float s = 0.f;
-    for (int k = 0; k < n_row_chunks; ++k) s += partial[(long long)k * D * 3 + i];
-    dW_r[i] = s;
-}
-
-// db_r = sum over rows of dG: one CTA, fixed-order tree.
-__global__ void __launch_bounds__(256) router_bias_grad_kernel(const float* __restrict__ dG, long long rows,
-                                                               float* __restrict__ db_r) {
-    __shared__ float sm[256][3];
-    float a[3] = {0.f, 0.f, 0.f};
-    for (long long r = threadIdx.x; r < rows; r += 256)
-        for (int l = 0; l < 3; ++l) a[l] += dG[r * 3 + l];
     for (int l = 0; l < 3; ++l) sm[threadIdx.x][l] = a[l];
     __syncthreads();
     for (int s = 128; s > 0; s >>= 1) {
         if (threadIdx.x < s)
+#pragma unroll
             for (int l = 0; l < 3; ++l) sm[threadIdx.x][l] += sm[threadIdx.x + s][l];
         __syncthreads();
     }
-    if (threadIdx.x < 3) db_r[threadIdx.x] = sm[0][threadIdx.x];
+#pragma unroll
+    for (int l = 0; l < 3; ++l) a[l] = sm[0][l];
+}
+
+// The same with eight consecutive columns per lane (16-byte loads of bf16): a warp takes every eighth row of the chunk, and
+// the next eight rows' loads are in flight while the current eight are added (without that the kernel waits for
+// loads most of the time: 2 TB/s); the eight warps' sums meet in shared memory.  Used when D is a multiple of 8 and R is
+// 16-byte aligned.  The CTAs of the first column block also add up the chunk's rows of dG for db_r, in 64 bits because the
+// rows' terms cancel (one CTA over all rows took 22 us at 32768 rows).
+template <typename T>
+__global__ void __launch_bounds__(256, 2)
+router_bwd_partial8_kernel(const T* __restrict__ R, const float* __restrict__ dG, long long rows, int D,
+                           int n_row_chunks, float* __restrict__ partial, double* __restrict__ db_partial) {
+    constexpr int kBatch = sizeof(T) == 2 ? 8 : 4;             // rows of a batch: 16-byte loads in flight a lane = 8
+    __shared__ float sum[8][24][33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c = blockIdx.x * 256 + lane * 8;
+    const int chunk = blockIdx.y;
+    const long long per = (rows + n_row_chunks - 1) / n_row_chunks;
+    const long long r0 = chunk * per, r1 = r0 + per < rows ? r0 + per : rows;
+    float a[24];
+#pragma unroll
+    for (int j = 0; j < 24; ++j) a[j] = 0.f;
+    typename Vec8<T>::Raw x[2][kBatch];
+    float g[2];
+    // rows rb, rb + 8, ..; a row past the chunk's end reads row rb again and weighs 0.  Lane 3u + l fetches dG[row u][l].
+    auto fetch = [&](long long rb, typename Vec8<T>::Raw (&to)[kBatch], float& gv) {
+        if (rb >= r1) return;
+        if (c < D)
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) to[u] = Vec8<T>::fetch(R + (rb + 8 * u < r1 ? rb + 8 * u : rb) * (long long)D + c);
+        const long long gr = rb + 8 * (lane / 3);
+        gv = lane < 3 * kBatch && gr < r1 ? __ldg(dG + gr * 3 + lane % 3) : 0.f;
+    };
+    auto add = [&](long long rb, const typename Vec8<T>::Raw (&from)[kBatch], float gv) {
+        if (rb >= r1) return;
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            const bool in = rb + 8 * u < r1;                   // (a repeated row weighs 0, but 0 x inf would not be 0)
+            float f[8];
+            Vec8<T>::widen(from[u], f);
+#pragma unroll
+            for (int l = 0; l < 3; ++l) {
+                const float gl = __shfl_sync(0xffffffffu, gv, 3 * u + l);
+                if (in)
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) a[j * 3 + l] = fmaf(f[j], gl, a[j * 3 + l]);
+            }
+        }
+    };
+    fetch(r0 + warp, x[0], g[0]);
+    for (long long rb = r0 + warp; rb < r1; rb += 16 * kBatch) {
+        fetch(rb + 8 * kBatch, x[1], g[1]);
+        add(rb, x[0], g[0]);
+        fetch(rb + 16 * kBatch, x[0], g[0]);
+        add(rb + 8 * kBatch, x[1], g[1]);
+    }
+#pragma unroll
+    for (int j = 0; j < 24; ++j) sum[warp][j][lane] = a[j];
+    __syncthreads();
+    const int cols = min(256, D - (int)blockIdx.x * 256) * 3;
+    for (int i = threadIdx.x; i < cols; i += 256) {
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) s += sum[w][i % 24][i / 24];
+        partial[((long long)chunk * D + blockIdx.x * 256) * 3 + i] = s;
+    }
+    if (blockIdx.x == 0 && db_partial) {
+        __shared__ double sm[256][3];
+        double b[3];
+        sum_dG(dG, r0, r1, sm, b);
+        if (threadIdx.x == 0)
+#pragma unroll
+            for (int l = 0; l < 3; ++l) db_partial[chunk * 3 + l] = b[l];
+    }
+}
+
+// dW_r = sum of the chunks' partials (32 outputs to a CTA, eight threads to an output: the loads of one output are eight
+// short chains, not one of 128); the last CTA instead gives db_r, from the chunks' sums or (db_partial null) from dG.
+__global__ void __launch_bounds__(256) router_bwd_reduce_kernel(const float* __restrict__ partial, const float* __restrict__ dG, long long rows,
+                                                                int D, int n_row_chunks, const double* __restrict__ db_partial,
+                                                                float* __restrict__ dW_r, float* __restrict__ db_r) {
+    if (db_r && blockIdx.x == gridDim.x - 1) {
+        __shared__ double sm[256][3];
+        double b[3];
+        if (db_partial) sum_dG(db_partial, 0, n_row_chunks, sm, b);
+        else sum_dG(dG, 0, rows, sm, b);
+        if (threadIdx.x == 0)
+#pragma unroll
+            for (int l = 0; l < 3; ++l) db_r[l] = (float)b[l];
+        return;
+    }
+    __shared__ float sm[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane;
+    float s = 0.f;
+    if (i < D * 3)
+        for (int k = warp; k < n_row_chunks; k += 8) s += partial[(long long)k * D * 3 + i];
+    sm[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0 && i < D * 3) {
+#pragma unroll
+        for (int w = 1; w < 8; ++w) s += sm[w][lane];
+        dW_r[i] = s;
+    }
 }
 
 }  // namespace
@@ -325,7 +405,15 @@ void router_t(const T* R, const float* W_r, const float* b_r, long long rows, in
             R, W_r, b_r, rows, D, route, gate, log2_gate, idx);
         return;
     }
-    // Eight rows to a CTA once that gives every SM one; two rows from 296 on; else one row, for the shortest chain.
+    // Up to two rows per SM: one row to a CTA, for the shortest chain; to eight per SM: two; below 32 a row is still better
+    // split over a CTA (2000 rows of 2048 bf16: 5.2 us against 8.4), above it the warps have enough to do on their own
+    // (32768 rows: 28 us against 51; loads ahead of the sums and W_r in shared memory were slower too, 35 and 44 us).
+    if (rows >= 32 * 148) {
+        const long long rows_per_cta = kWarps * kRowsPerWarp;
+        router_rows_kernel<T><<<(unsigned)((rows + rows_per_cta - 1) / rows_per_cta), kWarps * 32, 0, st>>>(
+            R, W_r, b_r, rows, D, route, gate, log2_gate, idx);
+        return;
+    }
     const int threads = D >= 8 * kMaxThreads ? kMaxThreads : (D / 8 + 31) / 32 * 32;
     if (rows >= 8 * 148)
         router_kernel<T, 8><<<(unsigned)((rows + 7) / 8), threads, 0, st>>>(R, W_r, b_r, rows, D, route, gate, log2_gate, idx);
@@ -345,23 +433,26 @@ cudaError_t launch_router(const void* R, const float* W_r, const float* b_r, lon
 }
 
 cudaError_t launch_router_bwd(const void* R, int r_dtype, const float* dG, long long rows, int D, float* dW_r,
-                              float* db_r, float* partial, int n_row_chunks, cudaStream_t st) {
-    if (dW_r && D % 4 == 0 && (reinterpret_cast<uintptr_t>(R) & 15) == 0) {
-        dim3 grid((D / 4 + 255) / 256, n_row_chunks), block(256);
-        if (r_dtype == MKA_BF16)
-            router_bwd_partial4_kernel<__nv_bfloat16><<<grid, block, 0, st>>>(static_cast<const __nv_bfloat16*>(R), dG, rows, D, n_row_chunks, partial);
-        else
-            router_bwd_partial4_kernel<float><<<grid, block, 0, st>>>(static_cast<const float*>(R), dG, rows, D, n_row_chunks, partial);
-        router_bwd_reduce_kernel<<<(D * 3 + 255) / 256, 256, 0, st>>>(partial, D, n_row_chunks, dW_r);
-    } else if (dW_r) {
-        dim3 grid((D + 255) / 256, n_row_chunks), block(256);
-        if (r_dtype == MKA_BF16)
-            router_bwd_partial_kernel<__nv_bfloat16><<<grid, block, 0, st>>>(static_cast<const __nv_bfloat16*>(R), dG, rows, D, n_row_chunks, partial);
-        else
-            router_bwd_partial_kernel<float><<<grid, block, 0, st>>>(static_cast<const float*>(R), dG, rows, D, n_row_chunks, partial);
-        router_bwd_reduce_kernel<<<(D * 3 + 255) / 256, 256, 0, st>>>(partial, D, n_row_chunks, dW_r);
+                              float* db_r, float* partial, double* db_partial, int n_row_chunks, cudaStream_t st) {
+    // as many row chunks as fill the chip's CTA slots once (two to an SM), at most the caller's
+    const int col_blocks = (D + 255) / 256;
+    if (n_row_chunks > 296 / col_blocks) n_row_chunks = 296 / col_blocks > 0 ? 296 / col_blocks : 1;
+    const bool vec = dW_r && D % 8 == 0 && (reinterpret_cast<uintptr_t>(R) & 15) == 0;
+    double* db_part = vec && db_r ? db_partial : nullptr;
+    if (dW_r) {
+        const dim3 grid(col_blocks, n_row_chunks);
+        if (r_dtype == MKA_BF16) {
+            auto* r = static_cast<const __nv_bfloat16*>(R);
+            if (vec) router_bwd_partial8_kernel<<<grid, 256, 0, st>>>(r, dG, rows, D, n_row_chunks, partial, db_part);
+            else router_bwd_partial_kernel<<<grid, 256, 0, st>>>(r, dG, rows, D, n_row_chunks, partial);
+        } else {
+            auto* r = static_cast<const float*>(R);
+            if (vec) router_bwd_partial8_kernel<<<grid, 256, 0, st>>>(r, dG, rows, D, n_row_chunks, partial, db_part);
+            else router_bwd_partial_kernel<<<grid, 256, 0, st>>>(r, dG, rows, D, n_row_chunks, partial);
+        }
     }
-    if (db_r) router_bias_grad_kernel<<<1, 256, 0, st>>>(dG, rows, db_r);
+    const int blocks = (dW_r ? (D * 3 + 31) / 32 : 0) + (db_r ? 1 : 0);
+    if (blocks) router_bwd_reduce_kernel<<<blocks, 256, 0, st>>>(partial, dG, rows, D, n_row_chunks, db_part, dW_r, db_r);
     return cudaGetLastError();
 }
 

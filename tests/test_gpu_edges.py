@@ -21,7 +21,7 @@ def orc():
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
-@pytest.mark.parametrize("rows,D", [(1, 4096), (295, 8), (296, 264), (297, 2056), (1183, 2048), (1184, 256), (1191, 3584)])
+@pytest.mark.parametrize("rows,D", [(1, 4096), (295, 8), (296, 264), (297, 2056), (1183, 2048), (1184, 256), (1191, 3584), (4735, 64), (4739, 520)])
 def test_router_rows_per_cta(mka, orc, dtype, rows, D):
     """One, two and eight rows to a CTA, with a last CTA that is not full and widths that leave threads idle."""
     X = problem(15, 1, 1, rows, 32, (1, 1, 1), D, dtype)["X"].view(rows, D)
@@ -62,3 +62,21 @@ def test_fwd_key_tiles_split_between_ctas(mka, orc, d, B, H, Hkv, T, W, q_off, N
         assert np.abs(np64(LSE)[finite] - Lr[finite]).max() <= 2e-3
         again, _ = mka.mka_fwd(shape, P["Q"], K, V, gate, ws=ws)
         assert torch.equal(O, again)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("B,T,D", [(1, 1, 64), (1, 127, 264), (2, 300, 2048), (3, 1111, 1000), (1, 5000, 256), (2, 70, 100)])
+def test_router_gradient_splits(mka, orc, dtype, B, T, D):
+    """dW_r and db_r: row chunks without a row, batches that end inside a chunk, column blocks that are not full."""
+    H, d, N = 1, 64, (T, T, 40)
+    P = problem(17, B, H, T, d, N, D, dtype, router_std=0.3, with_dO=True)
+    gate = mka.mka_router(P["X"], P["W_r"], None)
+    shape = mka.make_shape(B, H, T, d, D, 32, dtype=mka.binding.MKA_BF16 if dtype == torch.bfloat16 else mka.binding.MKA_F32)
+    O, LSE = mka.mka_fwd(shape, P["Q"], P["K"], P["V"], gate)
+    g = mka.mka_bwd(shape, P["Q"], P["K"], P["V"], gate, O, LSE, P["dO"], R=P["X"])
+    dG = np64(g["dG"])
+    dW, db = orc.router_bwd(np64(P["X"]), dG)
+    # fp32 sums of B T products: the bound is their number times the unit roundoff times the sum of magnitudes
+    mag = np.abs(np64(P["X"]).reshape(-1, D)).T @ np.abs(dG.reshape(-1, 3))
+    assert (np.abs(np64(g["dW_r"]) - dW) <= (B * T + 130) * 6e-8 * mag + 1e-30).all()
+    assert (np.abs(np64(g["db_r"]) - db) <= 6e-8 * np.abs(db) + 1e-15 * np.abs(dG).sum() * B * T).all()
