@@ -64,6 +64,10 @@ struct BwdTcParams {
     int window, q_offset;
     float scale, scale_log2;
     int kv_tiles[3];          // 128-row key tiles per level
+    int H_kv;
+    long long dkv_items;      // key tiles of all levels, KV heads and batches
+    long long dq_items;       // query tiles of all heads and batches
+    unsigned int *dkv_ticket, *dq_ticket;   // zero at launch
     unsigned int* status;
     unsigned long long wait_limit_ns;
     int test_stall;           // test hook: the dK/dV kernel's loader leaves out the last query tile of every CTA
@@ -122,10 +126,38 @@ struct BwdBarriers {
     uint64_t dp_full;                                     // dP landed in TMEM
     uint64_t p_part[2];                                   // phase 1 (dK/dV kernel): the first / second 32 columns of every thread's P^T are written
     uint64_t ds_part[2];                                  // phase 2: the same for dS
-    uint64_t acc_done;
+    uint64_t acc_done;                                    // per item: its accumulators are complete
+    uint64_t fixed_free;                                  // per item: its own tiles have had their last reader
+    uint64_t item_full[2], item_free[2];                  // the item numbers, two slots
 };
 
+// Items (output tiles) are dealt from a ticket counter: a CTA takes the next one when it is free, in the order in which
+// blocks of a plain grid would start.  The producing warp posts the number of item `it` to the other roles; a number past
+// the last item ends them all.
+__device__ __forceinline__ bool post_item(BwdBarriers& bar, int (&items)[2], int it, int item, int lane, volatile WaitCtl* ctl) {
+    if (it >= 2 && !mbar_wait_warp(&bar.item_free[it & 1], (uint32_t)((it >> 1) - 1) & 1u, ctl)) return false;
+    if (lane == 0) {
+        *reinterpret_cast<volatile int*>(&items[it & 1]) = item;
+        mbar_arrive(&bar.item_full[it & 1]);
+    }
+    __syncwarp();
+    return true;
+}
+__device__ __forceinline__ bool take_item(BwdBarriers& bar, int (&items)[2], int it, int& item, int lane, volatile WaitCtl* ctl) {
+    if (!mbar_wait_warp(&bar.item_full[it & 1], (uint32_t)(it >> 1) & 1u, ctl)) return false;
+    item = *reinterpret_cast<volatile int*>(&items[it & 1]);
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&bar.item_free[it & 1]);
+    return true;
+}
+
 __device__ __forceinline__ void softmax_group_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+__device__ __forceinline__ bool softmax_group_all(bool flag) {        // the same barrier; true when it is for all 256 threads
+    uint32_t out;
+    asm volatile("{\n.reg .pred pi, po;\nsetp.ne.u32 pi, %1, 0;\nbar.red.and.pred po, 1, 256, pi;\nselp.u32 %0, 1, 0, po;\n}"
+                 : "=r"(out) : "r"((uint32_t)flag) : "memory");
+    return out != 0;
+}
 
 // ------------------------------------------------------------------------------------------ prep
 // D = dO . O and the three exponent biases of every padded row.  DH / 8 lanes share a row (one 16-byte load of O and
@@ -229,6 +261,26 @@ __device__ __forceinline__ void store_row_bf16(__nv_bfloat16* dst, const uint32_
 __device__ __forceinline__ uint32_t packed_half_col(int k) { return (uint32_t)((k >> 2) * 64 + (k & 3) * 8); }
 
 // ------------------------------------------------------------------------------------------ dQ
+// One item of the dQ kernel: 128 query rows of one head, with the key tiles of the three levels that they see.
+struct DqItem {
+    int b, h, E;
+    int first[3], end[3];
+    long long m0, m_last;
+    __device__ __forceinline__ DqItem(const BwdTcParams& p, int item) {
+        const int tiles = p.Tpad / kBlk, bh = item / tiles;
+        b = bh / p.H; h = bh - b * p.H;
+        m0 = (long long)(tiles - 1 - (item - bh * tiles)) * kBlk;          // latest (heaviest) rows of a head first
+        m_last = (m0 + kBlk - 1 < p.T - 1) ? m0 + kBlk - 1 : p.T - 1;
+        E = 0;
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+            if (p.n[l] > 0) key_tile_range(l, m0, m_last, p.q_offset, p.window, p.n[l], first[l], end[l]);
+            else first[l] = end[l] = 0;
+            E += end[l] - first[l];
+        }
+    }
+};
+
 template <int DH>
 __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_constant__ BwdMaps maps, const BwdTcParams p) {
     using C = BCfg<DH>;
@@ -239,18 +291,15 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
     uint8_t* sdO = sQ + C::kTile;
     uint8_t* sK = sdO + C::kTile;                         // kStagesK tiles
     uint8_t* sV = sK + C::kStagesK * C::kTile;            // kStages tiles
-    float (*gsm)[6] = reinterpret_cast<float (*)[6]>(sQ); // epilogue scratch; Q is dead once the last S product has completed
     __shared__ BwdBarriers bar;
     __shared__ uint32_t tmem_base_slot;
     __shared__ WaitCtl wait_ctl;
+    __shared__ int items[2];
+    __shared__ float gsm[3][kBlk];                        // the second warpgroup's sums of a row, on their way to the first
 
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // tid >> 5, but provably warp-uniform for the compiler
-    const int b = blockIdx.z, h = blockIdx.y;
-    const long long bh = (long long)b * p.H + h;
-    const int qtile = gridDim.x - 1 - blockIdx.x;          // latest (heaviest) rows first
-    const long long m0 = (long long)qtile * kBlk;
-    const long long m_last = (m0 + kBlk - 1 < p.T - 1) ? m0 + kBlk - 1 : p.T - 1;
+    const int total = (int)p.dq_items;
 
     if (tid == 0) {
         wait_ctl.abort = 0;
@@ -264,6 +313,8 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
         mbar_init(&bar.dp_full, 1);
         for (int i = 0; i < 2; ++i) { mbar_init(&bar.p_part[i], 8); mbar_init(&bar.ds_part[i], 8); }   // 8 = one arrival per element-wise warp
         mbar_init(&bar.acc_done, 1);
+        mbar_init(&bar.fixed_free, 1);
+        for (int i = 0; i < 2; ++i) { mbar_init(&bar.item_full[i], 1); mbar_init(&bar.item_free[i], 9); }   // 9: the issuing warp and the element-wise warps
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
@@ -276,107 +327,146 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
     const uint32_t tmem = tmem_base_slot;
     volatile WaitCtl* abortp = &wait_ctl;
 
-    int first[3], end[3];
-#pragma unroll
-    for (int l = 0; l < 3; ++l) {
-        if (p.n[l] > 0) key_tile_range(l, m0, m_last, p.q_offset, p.window, p.n[l], first[l], end[l]);
-        else first[l] = end[l] = 0;
-    }
-    const int E = (end[0] - first[0]) + (end[1] - first[1]) + (end[2] - first[2]);
-
     if (warp == kProducerWarp) {
-        if (lane == 0) {
-            mbar_expect_tx(&bar.fixed_full, 2 * C::kTile);
+        int issued_k = 0, issued_v = 0, filled = 0;          // key tiles requested (per ring), items
+        bool ok = true;
+        int item = blockIdx.x;
+        for (int it = 0; ok; ++it) {
+            if (!(ok = post_item(bar, items, it, item, lane, abortp)) || item >= total) break;
+            const DqItem I(p, item);
+            const int kvh = I.h / p.kv_group;
+            if (I.E > 0) {
+                // the previous item's Q and dO have had their last reader when its last dP is complete
+                if (filled > 0 && !mbar_wait_warp(&bar.fixed_free, (uint32_t)(filled - 1) & 1u, abortp)) { ok = false; break; }
+                if (lane == 0) {
+                    mbar_expect_tx(&bar.fixed_full, 2 * C::kTile);
 #pragma unroll
-            for (int pn = 0; pn < C::kPanels; ++pn) {
-                tma_load_4d(sQ + pn * kPanel, &maps.q, pn * 64, (int)m0, h, b, &bar.fixed_full);
-                tma_load_4d(sdO + pn * kPanel, &maps.dO, pn * 64, (int)m0, h, b, &bar.fixed_full);
+                    for (int pn = 0; pn < C::kPanels; ++pn) {
+                        tma_load_4d(sQ + pn * kPanel, &maps.q, pn * 64, (int)I.m0, I.h, I.b, &bar.fixed_full);
+                        tma_load_4d(sdO + pn * kPanel, &maps.dO, pn * 64, (int)I.m0, I.h, I.b, &bar.fixed_full);
+                    }
+                }
+                __syncwarp();
+                ++filled;
             }
-            int issued_k = 0, issued_v = 0;
-            bool ok = true;
+#pragma unroll 1
             for (int l = 0; l < 3 && ok; ++l) {
-                for (int kt = first[l]; kt < end[l]; ++kt) {
+                const int kt_end = pick3(I.end, l);
+                for (int kt = pick3(I.first, l); kt < kt_end; ++kt) {
                     const int s = issued_k % C::kStagesK, sv = issued_k % C::kStages;
                     const uint32_t ph = (uint32_t)(issued_k / C::kStagesK) & 1u, phv = (uint32_t)(issued_k / C::kStages) & 1u;
-                    if (!mbar_wait(&bar.a_empty[s], ph ^ 1u, abortp)) { ok = false; break; }
-                    mbar_expect_tx(&bar.a_full[s], C::kTile);
+                    if (!mbar_wait_warp(&bar.a_empty[s], ph ^ 1u, abortp)) { ok = false; break; }
+                    if (lane == 0) {
+                        mbar_expect_tx(&bar.a_full[s], C::kTile);
 #pragma unroll
-                    for (int pn = 0; pn < C::kPanels; ++pn)
-                        tma_load_4d(sK + s * C::kTile + pn * kPanel, &maps.k[l], pn * 64, kt * kBlk, h / p.kv_group, b, &bar.a_full[s]);
+                        for (int pn = 0; pn < C::kPanels; ++pn)
+                            tma_load_4d(sK + s * C::kTile + pn * kPanel, &maps.k[l], pn * 64, kt * kBlk, kvh, I.b, &bar.a_full[s]);
+                    }
+                    __syncwarp();
                     ++issued_k;
-                    if (!mbar_wait(&bar.b_empty[sv], phv ^ 1u, abortp)) { ok = false; break; }
-                    mbar_expect_tx(&bar.b_full[sv], C::kTile);
+                    if (!mbar_wait_warp(&bar.b_empty[sv], phv ^ 1u, abortp)) { ok = false; break; }
+                    if (lane == 0) {
+                        mbar_expect_tx(&bar.b_full[sv], C::kTile);
 #pragma unroll
-                    for (int pn = 0; pn < C::kPanels; ++pn)
-                        tma_load_4d(sV + sv * C::kTile + pn * kPanel, &maps.v[l], pn * 64, kt * kBlk, h / p.kv_group, b, &bar.b_full[sv]);
+                        for (int pn = 0; pn < C::kPanels; ++pn)
+                            tma_load_4d(sV + sv * C::kTile + pn * kPanel, &maps.v[l], pn * 64, kt * kBlk, kvh, I.b, &bar.b_full[sv]);
+                    }
+                    __syncwarp();
                     ++issued_v;
                 }
             }
-            // every copy issued above must have landed before the shared memory can be given up
-            mbar_wait(&bar.fixed_full, 0, abortp);
-            for (int i = issued_k > C::kStagesK ? issued_k - C::kStagesK : 0; i < issued_k; ++i)
-                mbar_wait(&bar.a_full[i % C::kStagesK], (uint32_t)(i / C::kStagesK) & 1u, abortp);
-            for (int i = issued_v > C::kStages ? issued_v - C::kStages : 0; i < issued_v; ++i)
-                mbar_wait(&bar.b_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
+            // The next item is taken only now, with this one's last tiles still in the rings: taken earlier, the items left
+            // for a second round would go to whichever CTAs started first, the ones with the longest items among them.
+            if (lane == 0) item = (int)gridDim.x + (int)atomicAdd(p.dq_ticket, 1u);
+            item = __shfl_sync(0xffffffffu, item, 0);
         }
+        // every copy issued above must have landed before the shared memory can be given up
+        if (filled > 0) mbar_wait_warp(&bar.fixed_full, (uint32_t)(filled - 1) & 1u, abortp);
+        for (int i = issued_k > C::kStagesK ? issued_k - C::kStagesK : 0; i < issued_k; ++i)
+            mbar_wait_warp(&bar.a_full[i % C::kStagesK], (uint32_t)(i / C::kStagesK) & 1u, abortp);
+        for (int i = issued_v > C::kStages ? issued_v - C::kStages : 0; i < issued_v; ++i)
+            mbar_wait_warp(&bar.b_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
     } else if (warp == kMmaWarp) {
-        if (E > 0) {   // every lane runs the issue loop (converged); elect.sync inside the wrappers picks the issuing lane
-            bool ok = mbar_wait_warp(&bar.fixed_full, 0, abortp);
-            tc_fence_after();
+        {   // every lane runs the issue loop (converged); elect.sync inside the wrappers picks the issuing lane
             // low descriptor words of the operands (see make_desc): K-major views for S and dP, MN-major view of K for dQ
             const uint32_t q_lo = desc_lo_kmajor(smem_u32(sQ)), g_lo = desc_lo_kmajor(smem_u32(sdO));
             const uint32_t k_lo = desc_lo_kmajor(smem_u32(sK)), v_lo = desc_lo_kmajor(smem_u32(sV));
             const uint32_t kt_lo = desc_lo_mnmajor(smem_u32(sK), kPanel);
-            auto issue_s = [&](int e) -> bool {             // S(e) = Q K(e)^T into the ping/pong buffer e & 1
-                const int s = e % C::kStagesK;
-                if (!mbar_wait_warp(&bar.a_full[s], (uint32_t)(e / C::kStagesK) & 1u, abortp)) return false;
+            // g numbers the CTA's key tiles across its items
+            auto issue_s = [&](int g) -> bool {             // S(g) = Q K(g)^T into the ping/pong buffer g & 1
+                const int s = g % C::kStagesK;
+                if (!mbar_wait_warp(&bar.a_full[s], (uint32_t)(g / C::kStagesK) & 1u, abortp)) return false;
                 tc_fence_after();
                 const uint32_t ka = k_lo + s * (C::kTile >> 4);
 #pragma unroll
                 for (int k = 0; k < DH / 16; ++k)
-                    mma_ss_elect(tmem + kColS + (e & 1) * 128, make_desc(q_lo + kstep_off(k, kPanel)), make_desc(ka + kstep_off(k, kPanel)),
+                    mma_ss_elect(tmem + kColS + (g & 1) * 128, make_desc(q_lo + kstep_off(k, kPanel)), make_desc(ka + kstep_off(k, kPanel)),
                            C::kIdescS, k > 0);
-                mma_commit_elect(&bar.s_full[e & 1]);
+                mma_commit_elect(&bar.s_full[g & 1]);
                 return true;
             };
-            if (ok) ok = issue_s(0);
-            for (int e = 0; e < E && ok; ++e) {
-                const int s = e % C::kStagesK, sv = e % C::kStages;
-                if (!mbar_wait_warp(&bar.b_full[sv], (uint32_t)(e / C::kStages) & 1u, abortp)) { ok = false; break; }
+            int g = 0, filled = 0;
+            bool ok = true;
+            for (int it = 0; ok; ++it) {
+                int item;
+                if (!(ok = take_item(bar, items, it, item, lane, abortp)) || item >= total) break;
+                const int E = DqItem(p, item).E;
+                if (E == 0) continue;
+                // S(0) and dP(0) of this item run while the element-wise threads still store the previous one's dQ: the
+                // accumulator is not touched before those threads hand over the first dS.
+                if (!mbar_wait_warp(&bar.fixed_full, (uint32_t)filled & 1u, abortp)) { ok = false; break; }
+                ++filled;
                 tc_fence_after();
-                const uint32_t va = v_lo + sv * (C::kTile >> 4), kta = kt_lo + s * (C::kTile >> 4);
-#pragma unroll
-                for (int k = 0; k < DH / 16; ++k)          // dP(e) = dO V(e)^T  (dS(e-1), which shares the columns, was consumed by dQ(e-1) issued before)
-                    mma_ss_elect(tmem + kColDP, make_desc(g_lo + kstep_off(k, kPanel)), make_desc(va + kstep_off(k, kPanel)), C::kIdescS, k > 0);
-                mma_commit_elect(&bar.dp_full);
-                mma_commit_elect(&bar.b_empty[sv]);
-                if (e + 1 < E && !issue_s(e + 1)) { ok = false; break; }
-                // dQ += dS(e) K(e), in the two parts in which the element-wise threads hand dS over (32 of each thread's
-                // 64 columns: K-steps {0, 1, 4, 5}, then {2, 3, 6, 7}), so that the first half runs under the second
-#pragma unroll
-                for (int part = 0; part < 2; ++part) {
-                    if (!mbar_wait_warp(&bar.ds_part[part], (uint32_t)e & 1u, abortp)) { ok = false; break; }
+                if (!issue_s(g)) { ok = false; break; }
+                for (int e = 0; e < E && ok; ++e, ++g) {
+                    const int s = g % C::kStagesK, sv = g % C::kStages;
+                    if (!mbar_wait_warp(&bar.b_full[sv], (uint32_t)(g / C::kStages) & 1u, abortp)) { ok = false; break; }
                     tc_fence_after();
+                    const uint32_t va = v_lo + sv * (C::kTile >> 4), kta = kt_lo + s * (C::kTile >> 4);
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int k = (i >> 1) * 4 + part * 2 + (i & 1);
-                        mma_ts_elect(tmem + kColAcc, tmem + kColDP + packed_half_col(k), make_desc(kta + k * (2048 >> 4)), C::kIdescAcc,
-                               (e > 0 || part > 0 || i > 0) ? 1u : 0u);
+                    for (int k = 0; k < DH / 16; ++k)          // dP(e) = dO V(e)^T  (dS(e-1), which shares the columns, was consumed by dQ(e-1) issued before)
+                        mma_ss_elect(tmem + kColDP, make_desc(g_lo + kstep_off(k, kPanel)), make_desc(va + kstep_off(k, kPanel)), C::kIdescS, k > 0);
+                    mma_commit_elect(&bar.dp_full);
+                    mma_commit_elect(&bar.b_empty[sv]);
+                    if (e + 1 == E) mma_commit_elect(&bar.fixed_free);
+                    if (e + 1 < E && !issue_s(g + 1)) { ok = false; break; }
+                    // dQ += dS(e) K(e), in the two parts in which the element-wise threads hand dS over (32 of each thread's
+                    // 64 columns: K-steps {0, 1, 4, 5}, then {2, 3, 6, 7}), so that the first half runs under the second
+#pragma unroll
+                    for (int part = 0; part < 2; ++part) {
+                        if (!mbar_wait_warp(&bar.ds_part[part], (uint32_t)g & 1u, abortp)) { ok = false; break; }
+                        tc_fence_after();
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const int k = (i >> 1) * 4 + part * 2 + (i & 1);
+                            mma_ts_elect(tmem + kColAcc, tmem + kColDP + packed_half_col(k), make_desc(kta + k * (2048 >> 4)), C::kIdescAcc,
+                                   (e > 0 || part > 0 || i > 0) ? 1u : 0u);
+                        }
                     }
+                    if (!ok) break;
+                    mma_commit_elect(&bar.a_empty[s]);
                 }
-                if (!ok) break;
-                mma_commit_elect(&bar.a_empty[s]);
+                if (ok) mma_commit_elect(&bar.acc_done);
             }
-            if (ok) mma_commit_elect(&bar.acc_done);
         }
     } else {
         // ------------------------------------------------------------ element-wise warpgroups (thread = query row, 64 of the 128 columns)
         const int w = warp >> 2;
         const int r = tid & 127;
-        const long long t = m0 + r;
-        const bool row_valid = t < p.T;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t dp_addr = tmem + lane_base + kColDP + w * 64;
+        bool ok = true;
+        int g = 0, filled = 0;
+#pragma unroll 1
+        for (int it = 0;; ++it) {
+        // The warps leave together: those that took an item meet at barriers in its epilogue, so none may be missing there.
+        int item = total;
+        if (ok) ok = take_item(bar, items, it, item, lane, abortp);
+        if (!softmax_group_all(ok && item < total)) break;
+        const DqItem I(p, item);
+        const int E = I.E;
+        const long long bh = (long long)I.b * p.H + I.h, m0 = I.m0, m_last = I.m_last, t = m0 + r;
+        const bool row_valid = t < p.T;
         float Dt = 0.f, bias[3] = {-INFINITY, -INFINITY, -INFINITY};
         if (row_valid) {
             Dt = p.statD[bh * p.Tpad + t];
@@ -386,11 +476,9 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
             }
         }
         float Al[3] = {0.f, 0.f, 0.f}, Sl[3] = {0.f, 0.f, 0.f};   // per level: sum p dP and sum p over this thread's columns
-        bool ok = true;
-        int e = 0;
 #pragma unroll
         for (int l = 0; l < 3; ++l) {
-            if (!ok || first[l] == end[l]) continue;
+            if (!ok || I.first[l] == I.end[l]) continue;
             long long lo = 0, hi = 0;
             // a row past T has a bias of -inf, so its weights are 0 whatever it sees: it takes the last row's range
             visible_range(l, (row_valid ? t : m_last) + p.q_offset, p.window, p.n[l], 0, lo, hi);
@@ -406,15 +494,15 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
             uint64_t a2 = pack2(0.f, 0.f), z2 = a2;
             const float bl = bias[l];
             const uint64_t scale2 = pack2(p.scale_log2, p.scale_log2), bl2 = pack2(bl, bl), negD2 = pack2(-Dt, -Dt);
-            for (int kt = first[l]; kt < end[l]; ++kt, ++e) {
+            for (int kt = I.first[l]; kt < I.end[l]; ++kt, ++g) {
                 // phase 1: p = 2^(s * scale + bias) for this thread's 64 columns (needs S only)
-                ok = mbar_wait(&bar.s_full[e & 1], (uint32_t)(e >> 1) & 1u, abortp);
+                ok = mbar_wait(&bar.s_full[g & 1], (uint32_t)(g >> 1) & 1u, abortp);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
                 float pr[64];
                 {
-                    const uint32_t s_addr = tmem + lane_base + kColS + (e & 1) * 128 + w * 64;
+                    const uint32_t s_addr = tmem + lane_base + kColS + (g & 1) * 128 + w * 64;
                     tmem_ld32(s_addr, reinterpret_cast<uint32_t*>(pr));
                     tmem_ld32(s_addr + 32, reinterpret_cast<uint32_t*>(pr) + 32);
                     tmem_ld_wait();
@@ -432,7 +520,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
                     z2 = add2(z2, pack2(pr[c], pr[c + 1]));
                 }
                 // phase 2: dS = p (dP - D), written (bf16) over the dP columns just read
-                ok = mbar_wait(&bar.dp_full, (uint32_t)e & 1u, abortp);
+                ok = mbar_wait(&bar.dp_full, (uint32_t)g & 1u, abortp);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
@@ -475,7 +563,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
         }
         // ------------------------------------------------------------ epilogue
         if (ok && E > 0) {
-            ok = mbar_wait(&bar.acc_done, 0, abortp);
+            ok = mbar_wait(&bar.acc_done, (uint32_t)filled++ & 1u, abortp);
             ok = __all_sync(0xffffffffu, ok);
         }
         if (ok) {
@@ -497,21 +585,27 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
         // Gate-logit gradient of this head: G_l = sum_{j in l} p (dP - D').  D' = sum p dP / sum p equals
         // dO . O in exact arithmetic but does not inherit the rounding of O to bf16, so sum_l G_l = 0 holds
         // to fp32 accuracy.  The two warpgroups hold disjoint columns: add their partial sums first.
-        if (w == 1) {
+        // (A warp that gave up joins these barriers too.)
+        float asum[3], zsum[3];
 #pragma unroll
-            for (int l = 0; l < 3; ++l) { gsm[r][l] = Al[l]; gsm[r][3 + l] = Sl[l]; }
+        for (int half = 0; half < 2; ++half) {
+            if (half) softmax_group_sync();
+            if (w == 1)
+#pragma unroll
+                for (int l = 0; l < 3; ++l) gsm[l][r] = half ? Sl[l] : Al[l];
+            softmax_group_sync();
+            if (w == 0)
+#pragma unroll
+                for (int l = 0; l < 3; ++l) (half ? zsum : asum)[l] = (half ? Sl[l] : Al[l]) + gsm[l][r];
         }
-        softmax_group_sync();
         if (w == 0 && ok && row_valid) {
-            float a[3], z[3];
+            const float ztot = zsum[0] + zsum[1] + zsum[2];
+            const float dd = ztot > 0.f ? (asum[0] + asum[1] + asum[2]) / ztot : 0.f;
+            float* gp = p.Gpart + (bh * p.T + t) * 3;
 #pragma unroll
-            for (int l = 0; l < 3; ++l) { a[l] = Al[l] + gsm[r][l]; z[l] = Sl[l] + gsm[r][3 + l]; }
-            const float ztot = z[0] + z[1] + z[2];
-            const float dd = ztot > 0.f ? (a[0] + a[1] + a[2]) / ztot : 0.f;
-            float* g = p.Gpart + (bh * p.T + t) * 3;
-#pragma unroll
-            for (int l = 0; l < 3; ++l) g[l] = a[l] - z[l] * dd;
+            for (int l = 0; l < 3; ++l) gp[l] = asum[l] - zsum[l] * dd;
         }
+        }   // items
     }
 
     tc_fence_before();
@@ -521,6 +615,32 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
 }
 
 // ------------------------------------------------------------------------------------------ dK, dV
+// One item of the dK/dV kernel: a key tile of one level and KV head, with the query tiles that see it.
+struct DkvItem {
+    int b, h, lvl, first, Eq, E;          // h: KV head; its query heads are h * G .. h * G + G - 1
+    long long n, j0, j_last;
+    __device__ __forceinline__ DkvItem(const BwdTcParams& p, int item) {
+        const int tiles = p.kv_tiles[0] + p.kv_tiles[1] + p.kv_tiles[2], bh = item / tiles;
+        int kt = item - bh * tiles;
+        b = bh / p.H_kv; h = bh - b * p.H_kv;
+        // key tiles of a head in decreasing order of work: L3 (seen by every query), L2 from the oldest key on, L1
+        lvl = 2;
+        if (kt >= p.kv_tiles[2]) { kt -= p.kv_tiles[2]; lvl = 1; if (kt >= p.kv_tiles[1]) { kt -= p.kv_tiles[1]; lvl = 0; } }
+        n = pick3(p.n, lvl);
+        j0 = (long long)kt * kBlk;
+        j_last = (j0 + kBlk - 1 < n - 1) ? j0 + kBlk - 1 : n - 1;
+        // queries t (position t + q_offset) that can see a key of this tile
+        long long t_lo = 0, t_hi = p.T;
+        if (lvl == 0) { t_lo = j0 - p.q_offset; t_hi = j_last + p.window - p.q_offset; }
+        else if (lvl == 1) { t_lo = j0 - p.q_offset; }
+        if (t_lo < 0) t_lo = 0;
+        if (t_hi > p.T) t_hi = p.T;
+        first = t_hi > t_lo ? (int)(t_lo / kBlk) : 0;
+        Eq = t_hi > t_lo ? (int)((t_hi + kBlk - 1) / kBlk) - first : 0;    // query tiles of ONE head that see this key tile
+        E = Eq * p.kv_group;                                                // the stream: head by head, each head's tiles in order
+    }
+};
+
 template <int DH>
 __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_constant__ BwdMaps maps, const BwdTcParams p) {
     using C = BCfg<DH>;
@@ -541,33 +661,11 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
     __shared__ BwdBarriers bar;
     __shared__ uint32_t tmem_base_slot;
     __shared__ WaitCtl wait_ctl;
+    __shared__ int items[2];
 
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // tid >> 5, but provably warp-uniform for the compiler
-    const int b = blockIdx.z, h = blockIdx.y;               // h: KV head; its query heads are h * G .. h * G + G - 1
-    // key tiles in decreasing order of work: L3 (seen by every query), L2 from the oldest key on, L1
-    int lvl, kt;
-    {
-        int x = blockIdx.x;
-        if (x < p.kv_tiles[2]) { lvl = 2; kt = x; }
-        else if (x < p.kv_tiles[2] + p.kv_tiles[1]) { lvl = 1; kt = x - p.kv_tiles[2]; }
-        else { lvl = 0; kt = x - p.kv_tiles[2] - p.kv_tiles[1]; }
-    }
-    const long long n = p.n[lvl];
-    const long long j0 = (long long)kt * kBlk;
-    const long long j_last = (j0 + kBlk - 1 < n - 1) ? j0 + kBlk - 1 : n - 1;
-    // queries t (position t + q_offset) that can see a key of this tile
-    long long t_lo = 0, t_hi = p.T;
-    if (lvl == 0) { t_lo = j0 - p.q_offset; t_hi = j_last + p.window - p.q_offset; }
-    else if (lvl == 1) { t_lo = j0 - p.q_offset; }
-    if (t_lo < 0) t_lo = 0;
-    if (t_hi > p.T) t_hi = p.T;
-    const int first = t_hi > t_lo ? (int)(t_lo / kBlk) : 0;
-    const int Eq = t_hi > t_lo ? (int)((t_hi + kBlk - 1) / kBlk) - first : 0;    // query tiles of ONE head that see this key tile
-    const int E = Eq * p.kv_group;                          // the stream: head by head, each head's tiles in order
-
-    // The thread that issues the copies sets the barriers up itself and requests the CTA's own K and V tiles at once,
-    // before the CTA-wide start-up (slabs, TMEM allocation) that the copies' latency can run under.
+    const int total = (int)p.dkv_items;
     if (warp == kProducerWarp && lane == 0) {
         wait_ctl.abort = 0;
         wait_ctl.limit_ns = p.wait_limit_ns;
@@ -580,15 +678,9 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
         mbar_init(&bar.dp_full, 1);
         for (int i = 0; i < 2; ++i) { mbar_init(&bar.p_part[i], 8); mbar_init(&bar.ds_part[i], 8); }   // 8 = one arrival per element-wise warp
         mbar_init(&bar.acc_done, 1);
+        mbar_init(&bar.fixed_free, 1);
+        for (int i = 0; i < 2; ++i) { mbar_init(&bar.item_full[i], 1); mbar_init(&bar.item_free[i], 9); }   // 9: the issuing warp and the element-wise warps
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        if (E > 0) {
-            mbar_expect_tx(&bar.fixed_full, 2 * C::kTile);
-#pragma unroll
-            for (int pn = 0; pn < C::kPanels; ++pn) {
-                tma_load_4d(sK + pn * kPanel, &maps.k[lvl], pn * 64, (int)j0, h, b, &bar.fixed_full);
-                tma_load_4d(sV + pn * kPanel, &maps.v[lvl], pn * 64, (int)j0, h, b, &bar.fixed_full);
-            }
-        }
     }
     // every slab zero (columns 3..15 stay zero), ones for the keys: all threads share the 36 KB
     for (int i = tid; i < (int)((C::kStages * 2 + 1) * C::kAugBytes / 16); i += kThreads)
@@ -607,78 +699,102 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
     volatile WaitCtl* abortp = &wait_ctl;
 
     if (warp == kProducerWarp) {
-        if (E > 0) {   // the whole warp runs the loop (converged): lane 0 issues the copies, every lane writes its share of the slabs
-            int issued = 0, issued_b = 0;
-            const float inv_scale = 1.f / p.scale_log2;
-            int hq = h * p.kv_group, eq = 0;                // query head and tile-within-head of stage e
-            // this lane's four queries of a tile: their biases and D_t, fetched one tile ahead of the stage they go into
-            auto fetch = [&](float4& bq, float4& dq) {
-                const long long at = ((long long)b * p.H + hq) * p.Tpad + (long long)(first + eq) * kBlk + 4 * lane;
-                bq = *reinterpret_cast<const float4*>(p.statB[lvl] + at);
-                dq = *reinterpret_cast<const float4*>(p.statD + at);
-            };
-            float4 bq, dq;
-            fetch(bq, dq);
-            // Two rings: a stage's dO tile is free again after dV of its tile, its Q tile only after dK, one product later;
-            // and the next tile's Q is what the issuing warp waits for first.  Each is re-filled as soon as it is free.
-            for (int e = 0; e < E; ++e) {
-                const int s = e % C::kStages;
-                const uint32_t ph = (uint32_t)(e / C::kStages) & 1u;
-                if (p.test_stall && e == E - 1) break;                 // test hook: the last tile never arrives
-                const int tt = (first + eq) * kBlk;
-                const float bv[4] = {bq.x, bq.y, bq.z, bq.w}, dv[4] = {dq.x, dq.y, dq.z, dq.w};
-                if (!mbar_wait_warp(&bar.b_empty[s], ph ^ 1u, abortp)) break;
+        // the whole warp runs the loop (converged): lane 0 issues the copies, every lane writes its share of the slabs
+        const float inv_scale = 1.f / p.scale_log2;
+        int issued = 0, issued_b = 0, filled = 0;            // query tiles requested (per ring), items with tiles
+        bool ok = true;
+        int item = blockIdx.x;
+        for (int it = 0; ok; ++it) {
+            if (!(ok = post_item(bar, items, it, item, lane, abortp)) || item >= total) break;
+            const DkvItem I(p, item);
+            if (I.E > 0) {
+                // the previous item's K and V have had their last reader when its last dP^T is complete
+                if (filled > 0 && !mbar_wait_warp(&bar.fixed_free, (uint32_t)(filled - 1) & 1u, abortp)) { ok = false; break; }
                 if (lane == 0) {
-                    mbar_expect_tx(&bar.b_full[s], C::kTile);
+                    mbar_expect_tx(&bar.fixed_full, 2 * C::kTile);
 #pragma unroll
-                    for (int pn = 0; pn < C::kPanels; ++pn)
-                        tma_load_4d(sdO + s * C::kTile + pn * kPanel, &maps.dO, pn * 64, tt, hq, b, &bar.b_full[s]);
+                    for (int pn = 0; pn < C::kPanels; ++pn) {
+                        tma_load_4d(sK + pn * kPanel, &maps.k[I.lvl], pn * 64, (int)I.j0, I.h, I.b, &bar.fixed_full);
+                        tma_load_4d(sV + pn * kPanel, &maps.v[I.lvl], pn * 64, (int)I.j0, I.h, I.b, &bar.fixed_full);
+                    }
                 }
-                ++issued_b;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {                          // -D as three bf16 terms
-                    const int r = 4 * lane + i;
-                    *reinterpret_cast<uint4*>(sAugQ + (s * 2 + 1) * C::kAugBytes + (r & 7) * 16 + (r >> 3) * 256) = split3_bf16(-dv[i]);
-                }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&bar.b_full[s]);
-                if (!mbar_wait_warp(&bar.a_empty[s], ph ^ 1u, abortp)) break;
-                if (lane == 0) {
-                    mbar_expect_tx(&bar.a_full[s], C::kTile);
+                ++filled;
+                const float* statB = pick3(p.statB, I.lvl);
+                int hq = I.h * p.kv_group, eq = 0;           // query head and tile-within-head of tile e
+                // this lane's four queries of a tile: their biases and D_t, fetched one tile ahead of the stage they go into
+                auto fetch = [&](float4& bq, float4& dq) {
+                    const long long at = ((long long)I.b * p.H + hq) * p.Tpad + (long long)(I.first + eq) * kBlk + 4 * lane;
+                    bq = *reinterpret_cast<const float4*>(statB + at);
+                    dq = *reinterpret_cast<const float4*>(p.statD + at);
+                };
+                float4 bq, dq;
+                fetch(bq, dq);
+                // Two rings: a stage's dO tile is free again after dV of its tile, its Q tile only after dK, one product later;
+                // and the next tile's Q is what the issuing warp waits for first.  Each is re-filled as soon as it is free.
+                for (int e = 0; e < I.E; ++e) {
+                    const int s = issued % C::kStages;
+                    const uint32_t ph = (uint32_t)(issued / C::kStages) & 1u;
+                    if (p.test_stall && e == I.E - 1) { ok = false; break; }       // test hook: the last tile never arrives
+                    const int tt = (I.first + eq) * kBlk;
+                    const float bv[4] = {bq.x, bq.y, bq.z, bq.w}, dv[4] = {dq.x, dq.y, dq.z, dq.w};
+                    if (!mbar_wait_warp(&bar.b_empty[s], ph ^ 1u, abortp)) { ok = false; break; }
+                    if (lane == 0) {
+                        mbar_expect_tx(&bar.b_full[s], C::kTile);
 #pragma unroll
-                    for (int pn = 0; pn < C::kPanels; ++pn)
-                        tma_load_4d(sQ + s * C::kTile + pn * kPanel, &maps.q, pn * 64, tt, hq, b, &bar.a_full[s]);
-                }
-                ++issued;
+                        for (int pn = 0; pn < C::kPanels; ++pn)
+                            tma_load_4d(sdO + s * C::kTile + pn * kPanel, &maps.dO, pn * 64, tt, hq, I.b, &bar.b_full[s]);
+                    }
+                    ++issued_b;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {                          // bias / scale as three bf16 terms
-                    const int r = 4 * lane + i;
-                    *reinterpret_cast<uint4*>(sAugQ + (s * 2) * C::kAugBytes + (r & 7) * 16 + (r >> 3) * 256) = split3_bf16(bv[i] * inv_scale);
+                    for (int i = 0; i < 4; ++i) {                          // -D as three bf16 terms
+                        const int r = 4 * lane + i;
+                        *reinterpret_cast<uint4*>(sAugQ + (s * 2 + 1) * C::kAugBytes + (r & 7) * 16 + (r >> 3) * 256) = split3_bf16(-dv[i]);
+                    }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&bar.b_full[s]);
+                    if (!mbar_wait_warp(&bar.a_empty[s], ph ^ 1u, abortp)) { ok = false; break; }
+                    if (lane == 0) {
+                        mbar_expect_tx(&bar.a_full[s], C::kTile);
+#pragma unroll
+                        for (int pn = 0; pn < C::kPanels; ++pn)
+                            tma_load_4d(sQ + s * C::kTile + pn * kPanel, &maps.q, pn * 64, tt, hq, I.b, &bar.a_full[s]);
+                    }
+                    ++issued;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {                          // bias / scale as three bf16 terms
+                        const int r = 4 * lane + i;
+                        *reinterpret_cast<uint4*>(sAugQ + (s * 2) * C::kAugBytes + (r & 7) * 16 + (r >> 3) * 256) = split3_bf16(bv[i] * inv_scale);
+                    }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&bar.a_full[s]);
+                    if (++eq == I.Eq) { eq = 0; ++hq; }
+                    if (e + 1 < I.E) fetch(bq, dq);
                 }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&bar.a_full[s]);
-                if (++eq == Eq) { eq = 0; ++hq; }
-                if (e + 1 < E) fetch(bq, dq);
             }
-            mbar_wait_warp(&bar.fixed_full, 0, abortp);
-            for (int i = issued > C::kStages ? issued - C::kStages : 0; i < issued; ++i)
-                mbar_wait_warp(&bar.a_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
-            for (int i = issued_b > C::kStages ? issued_b - C::kStages : 0; i < issued_b; ++i)
-                mbar_wait_warp(&bar.b_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
+            // The next item is taken only now, with this one's last tiles still in the rings: taken earlier, the items left
+            // for a second round would go to whichever CTAs started first, the ones with the longest items among them.
+            if (lane == 0) item = (int)gridDim.x + (int)atomicAdd(p.dkv_ticket, 1u);
+            item = __shfl_sync(0xffffffffu, item, 0);
         }
+        // every copy issued above must have landed before the shared memory can be given up
+        if (filled > 0) mbar_wait_warp(&bar.fixed_full, (uint32_t)(filled - 1) & 1u, abortp);
+        for (int i = issued > C::kStages ? issued - C::kStages : 0; i < issued; ++i)
+            mbar_wait_warp(&bar.a_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
+        for (int i = issued_b > C::kStages ? issued_b - C::kStages : 0; i < issued_b; ++i)
+            mbar_wait_warp(&bar.b_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
     } else if (warp == kMmaWarp) {
-        if (E > 0) {   // every lane runs the issue loop (converged); elect.sync inside the wrappers picks the issuing lane
-            bool ok = mbar_wait_warp(&bar.fixed_full, 0, abortp);
-            tc_fence_after();
+        {   // every lane runs the issue loop (converged); elect.sync inside the wrappers picks the issuing lane
             // low descriptor words (see make_desc): K-major views for S^T and dP^T, MN-major views of Q and dO for dK and dV
             const uint32_t k_lo = desc_lo_kmajor(smem_u32(sK)), v_lo = desc_lo_kmajor(smem_u32(sV));
             const uint32_t q_lo = desc_lo_kmajor(smem_u32(sQ)), g_lo = desc_lo_kmajor(smem_u32(sdO));
             const uint32_t qt_lo = desc_lo_mnmajor(smem_u32(sQ), kPanel), gt_lo = desc_lo_mnmajor(smem_u32(sdO), kPanel);
             const uint32_t augk_lo = desc_lo_flat(smem_u32(sAugK)), augq_lo = desc_lo_flat(smem_u32(sAugQ));
-            auto issue_s = [&](int e) {                     // S^T(e) = K Q(e)^T   (P^T(e-1), which shares the columns, was consumed by dV(e-1) issued before; Q(e) has landed)
-                const int s = e % C::kStages;
+            // g numbers the CTA's query tiles across its items
+            auto issue_s = [&](int g) {                     // S^T(g) = K Q(g)^T   (P^T(g-1), which shares the columns, was consumed by dV(g-1) issued before; Q(g) has landed)
+                const int s = g % C::kStages;
                 tc_fence_after();
                 const uint32_t qa = q_lo + s * (C::kTile >> 4);
 #pragma unroll
@@ -687,99 +803,121 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
                 mma_ss_elect(tmem + kColS, make_desc_flat(augk_lo), make_desc_flat(augq_lo + s * (2 * C::kAugBytes >> 4)), C::kIdescS, 1u);   // + bias_t / scale
                 mma_commit_elect(&bar.s_full[0]);
             };
-            auto issue_dp = [&](int e) -> bool {            // dP^T(e) = V dO(e)^T
-                if (!mbar_wait_warp(&bar.b_full[e % C::kStages], (uint32_t)(e / C::kStages) & 1u, abortp)) return false;
+            auto issue_dp = [&](int g) -> bool {            // dP^T(g) = V dO(g)^T
+                if (!mbar_wait_warp(&bar.b_full[g % C::kStages], (uint32_t)(g / C::kStages) & 1u, abortp)) return false;
                 tc_fence_after();
-                const uint32_t ga = g_lo + (e % C::kStages) * (C::kTile >> 4);
+                const uint32_t ga = g_lo + (g % C::kStages) * (C::kTile >> 4);
 #pragma unroll
                 for (int k = 0; k < DH / 16; ++k)
                     mma_ss_elect(tmem + kColDP, make_desc(v_lo + kstep_off(k, kPanel)), make_desc(ga + kstep_off(k, kPanel)), C::kIdescS, k > 0);
-                mma_ss_elect(tmem + kColDP, make_desc_flat(augk_lo), make_desc_flat(augq_lo + ((e % C::kStages) * 2 + 1) * (C::kAugBytes >> 4)), C::kIdescS, 1u);   // - D_t
+                mma_ss_elect(tmem + kColDP, make_desc_flat(augk_lo), make_desc_flat(augq_lo + ((g % C::kStages) * 2 + 1) * (C::kAugBytes >> 4)), C::kIdescS, 1u);   // - D_t
                 mma_commit_elect(&bar.dp_full);
                 return true;
             };
-            if (ok) ok = mbar_wait_warp(&bar.a_full[0], 0, abortp);
-            if (ok) issue_s(0);
-            if (ok) ok = issue_dp(0);
-            for (int e = 0; e < E && ok; ++e) {
-                const int s = e % C::kStages;
-                const uint32_t qta = qt_lo + s * (C::kTile >> 4), gta = gt_lo + s * (C::kTile >> 4);
-                // dV += P^T(e) dO(e) and dK += dS^T(e) Q(e), each in the two parts in which the element-wise threads
-                // hand their 64 columns over (K-steps {0, 1, 4, 5}, then {2, 3, 6, 7})
+            int g = 0, filled = 0;
+            bool ok = true;
+            for (int it = 0; ok; ++it) {
+                int item;
+                if (!(ok = take_item(bar, items, it, item, lane, abortp)) || item >= total) break;
+                const int E = DkvItem(p, item).E;
+                if (E == 0) continue;
+                // S^T(0) and dP^T(0) of this item run while the element-wise threads still store the previous one's dK and
+                // dV: the accumulators are not touched before those threads hand over the first P^T.
+                if (!mbar_wait_warp(&bar.fixed_full, (uint32_t)filled & 1u, abortp) ||
+                    !mbar_wait_warp(&bar.a_full[g % C::kStages], (uint32_t)(g / C::kStages) & 1u, abortp)) { ok = false; break; }
+                ++filled;
+                issue_s(g);
+                if (!issue_dp(g)) { ok = false; break; }
+                if (E == 1) mma_commit_elect(&bar.fixed_free);
+                for (int e = 0; e < E && ok; ++e, ++g) {
+                    const int s = g % C::kStages;
+                    const uint32_t qta = qt_lo + s * (C::kTile >> 4), gta = gt_lo + s * (C::kTile >> 4);
+                    // dV += P^T(e) dO(e) and dK += dS^T(e) Q(e), each in the two parts in which the element-wise threads
+                    // hand their 64 columns over (K-steps {0, 1, 4, 5}, then {2, 3, 6, 7})
 #pragma unroll
-                for (int part = 0; part < 2; ++part) {
-                    if (!mbar_wait_warp(&bar.p_part[part], (uint32_t)e & 1u, abortp)) { ok = false; break; }
-                    tc_fence_after();
+                    for (int part = 0; part < 2; ++part) {
+                        if (!mbar_wait_warp(&bar.p_part[part], (uint32_t)g & 1u, abortp)) { ok = false; break; }
+                        tc_fence_after();
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int k = (i >> 1) * 4 + part * 2 + (i & 1);
-                        mma_ts_elect(tmem + kColDV, tmem + kColS + packed_half_col(k), make_desc(gta + k * (2048 >> 4)), C::kIdescAcc,
-                               (e > 0 || part > 0 || i > 0) ? 1u : 0u);
-                    }
-                }
-                if (!ok) break;
-                mma_commit_elect(&bar.b_empty[s]);                     // dO(e) has had its last reader
-                // S^T(e+1) needs Q(e+1), which can only be requested once dK(e-1) has released its stage; dK(e) needs dS^T(e)
-                // from the element-wise threads.  Either may be ready first, and neither may wait for the other (a late
-                // dK delays the release, the release the copy, the copy the next S^T): poll both.
-                {
-                    const int sn = (e + 1) % C::kStages;
-                    const uint32_t phn = (uint32_t)((e + 1) / C::kStages) & 1u;
-                    bool s_out = e + 1 >= E;
-                    int dk_part = 0;
-                    const unsigned long long t0 = gtimer();
-                    while (!s_out || dk_part < 2) {
-                        bool moved = false;
-                        if (!s_out && __all_sync(0xffffffffu, mbar_try(&bar.a_full[sn], phn))) {
-                            issue_s(e + 1);
-                            s_out = moved = true;
+                        for (int i = 0; i < 4; ++i) {
+                            const int k = (i >> 1) * 4 + part * 2 + (i & 1);
+                            mma_ts_elect(tmem + kColDV, tmem + kColS + packed_half_col(k), make_desc(gta + k * (2048 >> 4)), C::kIdescAcc,
+                                   (e > 0 || part > 0 || i > 0) ? 1u : 0u);
                         }
-                        if (dk_part < 2 && __all_sync(0xffffffffu, mbar_try(&bar.ds_part[dk_part], (uint32_t)e & 1u))) {
-                            tc_fence_after();
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                const int k = (i >> 1) * 4 + dk_part * 2 + (i & 1);
-                                mma_ts_elect(tmem + kColDK, tmem + kColDP + packed_half_col(k), make_desc(qta + k * (2048 >> 4)), C::kIdescAcc,
-                                       (e > 0 || dk_part > 0 || i > 0) ? 1u : 0u);
+                    }
+                    if (!ok) break;
+                    mma_commit_elect(&bar.b_empty[s]);                     // dO(e) has had its last reader
+                    // S^T(e+1) needs Q(e+1), which can only be requested once dK(e-1) has released its stage; dK(e) needs dS^T(e)
+                    // from the element-wise threads.  Either may be ready first, and neither may wait for the other (a late
+                    // dK delays the release, the release the copy, the copy the next S^T): poll both.
+                    {
+                        const int sn = (g + 1) % C::kStages;
+                        const uint32_t phn = (uint32_t)((g + 1) / C::kStages) & 1u;
+                        bool s_out = e + 1 >= E;
+                        int dk_part = 0;
+                        const unsigned long long t0 = gtimer();
+                        while (!s_out || dk_part < 2) {
+                            bool moved = false;
+                            if (!s_out && __all_sync(0xffffffffu, mbar_try(&bar.a_full[sn], phn))) {
+                                issue_s(g + 1);
+                                s_out = moved = true;
                             }
-                            ++dk_part;
-                            moved = true;
-                        }
-                        if (!moved) {                            // bounded like every other wait of the kernel
-                            bool give_up = abortp->abort != 0;
-                            if (!give_up && gtimer() - t0 > abortp->limit_ns) { abortp->abort = 1; give_up = true; }
-                            if (__any_sync(0xffffffffu, give_up)) { ok = false; break; }
+                            if (dk_part < 2 && __all_sync(0xffffffffu, mbar_try(&bar.ds_part[dk_part], (uint32_t)g & 1u))) {
+                                tc_fence_after();
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) {
+                                    const int k = (i >> 1) * 4 + dk_part * 2 + (i & 1);
+                                    mma_ts_elect(tmem + kColDK, tmem + kColDP + packed_half_col(k), make_desc(qta + k * (2048 >> 4)), C::kIdescAcc,
+                                           (e > 0 || dk_part > 0 || i > 0) ? 1u : 0u);
+                                }
+                                ++dk_part;
+                                moved = true;
+                            }
+                            if (!moved) {                            // bounded like every other wait of the kernel
+                                bool give_up = abortp->abort != 0;
+                                if (!give_up && gtimer() - t0 > abortp->limit_ns) { abortp->abort = 1; give_up = true; }
+                                if (__any_sync(0xffffffffu, give_up)) { ok = false; break; }
+                            }
                         }
                     }
+                    if (!ok) break;
+                    mma_commit_elect(&bar.a_empty[s]);
+                    if (e + 1 < E) {
+                        if (!issue_dp(g + 1)) { ok = false; break; }
+                        if (e + 2 == E) mma_commit_elect(&bar.fixed_free);
+                    }
                 }
-                if (!ok) break;
-                mma_commit_elect(&bar.a_empty[s]);
-                if (e + 1 < E && !issue_dp(e + 1)) { ok = false; break; }
+                if (ok) mma_commit_elect(&bar.acc_done);
             }
-            if (ok) mma_commit_elect(&bar.acc_done);
         }
     } else {
         // ------------------------------------------------------------ element-wise warpgroups (thread = key row, 64 of the 128 query columns)
         const int w = warp >> 2;
         const int r = tid & 127;
-        const long long j = j0 + r;
-        const bool row_valid = j < n;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t s_addr = tmem + lane_base + kColS + w * 64;
         const uint32_t dp_addr = tmem + lane_base + kColDP + w * 64;
+        bool ok = true;
+        int g = 0, filled = 0;
+#pragma unroll 1
+        for (int it = 0; ok; ++it) {
+        int item;
+        if (!(ok = take_item(bar, items, it, item, lane, abortp)) || item >= total) break;
+        const DkvItem I(p, item);
+        const int lvl = I.lvl, E = I.E, Eq = I.Eq, first = I.first;
+        const long long j0 = I.j0, j_last = I.j_last, j = j0 + r;
+        const bool row_valid = j < I.n;
         // queries [q_lo, q_hi) that see key j (the bound t < T is carried by the padded biases)
         // a key past n has its own row of dK and dV, which nobody stores: it takes the last key's range and needs no mask
         const long long j_see = row_valid ? j : j_last;
         const long long q_lo = lvl == 2 ? 0 : j_see - p.q_offset;
         const long long q_hi = lvl == 0 ? j_see + p.window - p.q_offset : (long long)p.Tpad;
-        bool ok = true;
         int eq = 0;                                                    // tile within the current query head
-        for (int e = 0; e < E; ++e) {
-            const int s = e % C::kStages;
+        for (int e = 0; e < E; ++e, ++g) {
             const long long tt = (long long)(first + eq) * kBlk;       // first query of the tile
             if (++eq == Eq) eq = 0;
             // phase 1: P^T = 2^(scale * (s + bias_t / scale)) for this thread's 64 query columns; the sum comes from the tensor pipe
-            ok = mbar_wait(&bar.s_full[0], (uint32_t)e & 1u, abortp);
+            ok = mbar_wait(&bar.s_full[0], (uint32_t)g & 1u, abortp);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
@@ -826,7 +964,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
             tmem_st16(s_addr + 16, pk + 16);
             hand_over(&bar.p_part[1]);
             // phase 2: dS^T = P^T (dP^T - D_t), written over the columns just read; the difference comes from the tensor pipe
-            ok = mbar_wait(&bar.dp_full, (uint32_t)e & 1u, abortp);
+            ok = mbar_wait(&bar.dp_full, (uint32_t)g & 1u, abortp);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
@@ -852,13 +990,13 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
         }
         // ------------------------------------------------------------ epilogue: warpgroup 0 writes dK, 1 writes dV
         if (ok && E > 0) {
-            ok = mbar_wait(&bar.acc_done, 0, abortp);
+            ok = mbar_wait(&bar.acc_done, (uint32_t)filled++ & 1u, abortp);
             ok = __all_sync(0xffffffffu, ok);
         }
         if (ok) {
             tc_fence_after();
             const LevelGradDev dL = p.dL[lvl];
-            __nv_bfloat16* out = static_cast<__nv_bfloat16*>(w == 0 ? dL.dk : dL.dv) + b * dL.sb + h * dL.sh + j * dL.sn;
+            __nv_bfloat16* out = static_cast<__nv_bfloat16*>(w == 0 ? dL.dk : dL.dv) + I.b * dL.sb + I.h * dL.sh + j * dL.sn;
             const float mul = w == 0 ? p.scale : 1.f;
 #pragma unroll
             for (int c0 = 0; c0 < DH; c0 += 32) {
@@ -873,6 +1011,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
                 if (row_valid) store_row_bf16(out + c0, o, mul);
             }
         }
+        }   // items
     }
 
     tc_fence_before();
@@ -909,7 +1048,7 @@ cudaError_t launch_t(const BwdParams& bp, unsigned int* status_word, cudaStream_
         p.kv_tiles[l] = (int)((bp.L[l].n + 127) / 128);
     }
     p.B = bp.B; p.H = bp.H; p.T = bp.T; p.Tpad = Tpad; p.kv_group = bp.kv_group > 0 ? bp.kv_group : 1;
-    const int H_kv = bp.H / p.kv_group;
+    const int H_kv = p.H_kv = bp.H / p.kv_group;
     p.window = bp.window; p.q_offset = bp.q_offset;
     p.scale = bp.scale; p.scale_log2 = bp.scale * kLog2e;
     p.status = status_word;
@@ -930,8 +1069,9 @@ cudaError_t launch_t(const BwdParams& bp, unsigned int* status_word, cudaStream_
         }
         e = cudaFuncSetAttribute(bwd_dq_tc_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmemDq);
         if (e != cudaSuccess) return e;
-        dim3 grid((bp.T + 127) / 128, bp.H, bp.B);
-        bwd_dq_tc_kernel<DH><<<grid, kThreads, C::kSmemDq, st>>>(m, p);
+        p.dq_items = (long long)(Tpad / kBlk) * bp.H * bp.B;
+        p.dq_ticket = status_word + 2;
+        bwd_dq_tc_kernel<DH><<<(unsigned)(p.dq_items < 148 ? p.dq_items : 148), kThreads, C::kSmemDq, st>>>(m, p);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     const int tiles = p.kv_tiles[0] + p.kv_tiles[1] + p.kv_tiles[2];
@@ -948,8 +1088,9 @@ cudaError_t launch_t(const BwdParams& bp, unsigned int* status_word, cudaStream_
         }
         e = cudaFuncSetAttribute(bwd_dkv_tc_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmemDkv);
         if (e != cudaSuccess) return e;
-        dim3 grid(tiles, H_kv, bp.B);
-        bwd_dkv_tc_kernel<DH><<<grid, kThreads, C::kSmemDkv, st>>>(m, p);
+        p.dkv_items = (long long)tiles * H_kv * bp.B;
+        p.dkv_ticket = status_word + 1;
+        bwd_dkv_tc_kernel<DH><<<(unsigned)(p.dkv_items < 148 ? p.dkv_items : 148), kThreads, C::kSmemDkv, st>>>(m, p);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return launch_bwd_dgate(bp.Gpart, bp.B, bp.H, bp.T, bp.dG, st);
