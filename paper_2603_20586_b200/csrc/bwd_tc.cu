@@ -41,8 +41,6 @@
 namespace mka {
 namespace {
 
-constexpr int kThreads = 320;
-constexpr int kProducerWarp = 8, kMmaWarp = 9;
 constexpr int kBlk = 128;                             // rows of every tile
 constexpr uint32_t kPanel = 128 * 128;                // bytes of a [128 rows][64 bf16] panel
 constexpr int kMaxStages = 4;
@@ -105,6 +103,18 @@ __device__ __forceinline__ void exp2_pair_fma(float x0, float x1, float& p0, flo
 
 template <int DH>
 struct BCfg {
+    static constexpr int kEw = DH == 128 ? 8 : 16;                    // element-wise warps
+    static constexpr int kGroups = kEw / 4;                   // threads per row: warpgroup w owns columns [w * kCols, (w + 1) * kCols) of a tile
+    static constexpr int kCols = kBlk / kGroups;
+    static constexpr int kProducerWarp = kEw, kMmaWarp = kEw + 1;
+    static constexpr int kSlabWarp = kEw + 2;                 // dK/dV kernel: this one and the next write the operand slabs
+    static constexpr int kThreads = (kEw + 2) * 32, kThreadsDkv = (kEw + 4) * 32;
+    // A-operand column (32-bit TMEM columns) of K-step k of a 128-wide bf16 row: every warpgroup packs its kCols columns into
+    // the first kCols / 2 of the TMEM columns it has read them from.  The weights are handed over in two parts, the first and
+    // the second half of every thread's columns: K-step kstep(part, i), i = 0..3.
+    static __host__ __device__ constexpr uint32_t packed_col(int k) { return (uint32_t)((k * 16 / kCols) * kCols + (k * 16 % kCols) / 2); }
+    static __host__ __device__ constexpr int kstep(int part, int i) { return kGroups == 2 ? (i >> 1) * 4 + part * 2 + (i & 1) : 2 * i + part; }
+    static constexpr int kGsm = DH == 128 ? 1 : kGroups - 1;  // warpgroups whose row sums meet in shared memory at a time (dQ kernel)
     static constexpr int kPanels = DH / 64;
     static constexpr uint32_t kTile = kPanels * kPanel;       // a 128-row tile
     static constexpr int kStages = DH == 128 ? 2 : 4;         // also keeps the CTA above half of shared memory
@@ -131,6 +141,25 @@ struct BwdBarriers {
     uint64_t item_full[2], item_free[2];                  // the item numbers, two slots
 };
 
+// Which of two barriers completes first (0 or 1; the first one when both have), -1 when the wait was given up.  Executed by a
+// converged warp; bounded like every other wait.
+__device__ __forceinline__ int poll_two(uint64_t* b0, uint32_t ph0, uint64_t* b1, uint32_t ph1, volatile WaitCtl* ctl) {
+    int got = -2;
+    if (__all_sync(0xffffffffu, mbar_try(b0, ph0))) return 0;
+    if (__all_sync(0xffffffffu, mbar_try(b1, ph1))) return 1;
+    const unsigned long long t0 = gtimer();
+    while (got == -2) {
+        if (__all_sync(0xffffffffu, mbar_try(b0, ph0))) got = 0;
+        else if (__all_sync(0xffffffffu, mbar_try(b1, ph1))) got = 1;
+        else {
+            bool give_up = ctl->abort != 0;
+            if (!give_up && gtimer() - t0 > ctl->limit_ns) { ctl->abort = 1; give_up = true; }
+            if (__any_sync(0xffffffffu, give_up)) got = -1;
+        }
+    }
+    return __shfl_sync(0xffffffffu, got, 0);
+}
+
 // Items (output tiles) are dealt from a ticket counter: a CTA takes the next one when it is free, in the order in which
 // blocks of a plain grid would start.  The producing warp posts the number of item `it` to the other roles; a number past
 // the last item ends them all.
@@ -145,17 +174,16 @@ __device__ __forceinline__ bool post_item(BwdBarriers& bar, int (&items)[2], int
 }
 __device__ __forceinline__ bool take_item(BwdBarriers& bar, int (&items)[2], int it, int& item, int lane, volatile WaitCtl* ctl) {
     if (!mbar_wait_warp(&bar.item_full[it & 1], (uint32_t)(it >> 1) & 1u, ctl)) return false;
-    item = *reinterpret_cast<volatile int*>(&items[it & 1]);
-    __syncwarp();
+    item = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&items[it & 1]), 0);   // warp-uniform for the compiler too
     if (lane == 0) mbar_arrive(&bar.item_free[it & 1]);
     return true;
 }
 
-__device__ __forceinline__ void softmax_group_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
-__device__ __forceinline__ bool softmax_group_all(bool flag) {        // the same barrier; true when it is for all 256 threads
+template <int kWarps> __device__ __forceinline__ void softmax_group_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kWarps * 32) : "memory"); }
+template <int kWarps> __device__ __forceinline__ bool softmax_group_all(bool flag) {        // the same barrier; true when it is for all of its threads
     uint32_t out;
-    asm volatile("{\n.reg .pred pi, po;\nsetp.ne.u32 pi, %1, 0;\nbar.red.and.pred po, 1, 256, pi;\nselp.u32 %0, 1, 0, po;\n}"
-                 : "=r"(out) : "r"((uint32_t)flag) : "memory");
+    asm volatile("{\n.reg .pred pi, po;\nsetp.ne.u32 pi, %1, 0;\nbar.red.and.pred po, 1, %2, pi;\nselp.u32 %0, 1, 0, po;\n}"
+                 : "=r"(out) : "r"((uint32_t)flag), "n"(kWarps * 32) : "memory");
     return out != 0;
 }
 
@@ -220,11 +248,12 @@ __global__ void __launch_bounds__(256) bwd_prep_kernel(const __nv_bfloat16* __re
     }
 }
 
-// Scores outside columns [c_lo, c_hi) of the thread's 64 become -inf: one bit per column, so a column costs a test and a
+// Scores outside columns [c_lo, c_hi) of the thread's become -inf: one bit per column, so a column costs a test and a
 // select; 32 columns that no row of the warp masks are passed over.
-__device__ __forceinline__ void mask_cols(float (&x)[64], int c_lo, int c_hi) {
+template <int N>
+__device__ __forceinline__ void mask_cols(float (&x)[N], int c_lo, int c_hi) {
 #pragma unroll
-    for (int c0 = 0; c0 < 64; c0 += 32) {
+    for (int c0 = 0; c0 < N; c0 += 32) {
         const uint32_t vis = low_bits(c_hi - c0) & ~low_bits(c_lo - c0);
         if (__all_sync(0xffffffffu, vis == 0xffffffffu)) continue;
 #pragma unroll
@@ -244,9 +273,26 @@ __device__ __forceinline__ void key_tile_range(int level, long long r0, long lon
     end = (int)((hi + kBlk - 1) / kBlk);
 }
 
-__device__ __forceinline__ void store_row_bf16(__nv_bfloat16* dst, const uint32_t (&o)[32], float mul) {
+// N 32-bit TMEM columns of this thread's lane, N = 16 or a multiple of 32.
+template <int N>
+__device__ __forceinline__ void tmem_load(uint32_t addr, uint32_t* r) {
+    if constexpr (N == 16) tmem_ld16(addr, r);
+    else {
 #pragma unroll
-    for (int i = 0; i < 32; i += 8) {
+        for (int c = 0; c < N; c += 32) tmem_ld32(addr + c, r + c);
+    }
+}
+// The packed halves (N / 2 values) of N columns.
+template <int N>
+__device__ __forceinline__ void tmem_store_part(uint32_t addr, const uint32_t* r) {
+    if constexpr (N == 32) tmem_st16(addr, r);
+    else tmem_st8(addr, r);
+}
+
+template <int N>
+__device__ __forceinline__ void store_row_bf16(__nv_bfloat16* dst, const uint32_t (&o)[N], float mul) {
+#pragma unroll
+    for (int i = 0; i < N; i += 8) {
         uint4 v;
         v.x = pack_bf16(__uint_as_float(o[i]) * mul, __uint_as_float(o[i + 1]) * mul);
         v.y = pack_bf16(__uint_as_float(o[i + 2]) * mul, __uint_as_float(o[i + 3]) * mul);
@@ -255,10 +301,6 @@ __device__ __forceinline__ void store_row_bf16(__nv_bfloat16* dst, const uint32_
         *reinterpret_cast<uint4*>(dst + i) = v;
     }
 }
-
-// A-operand column (32-bit TMEM columns) of K-step k of a 128-wide bf16 row that the two warpgroups wrote
-// as two packed halves: keys 0-63 at columns [0,32), keys 64-127 at columns [64,96) of the region.
-__device__ __forceinline__ uint32_t packed_half_col(int k) { return (uint32_t)((k >> 2) * 64 + (k & 3) * 8); }
 
 // ------------------------------------------------------------------------------------------ dQ
 // One item of the dQ kernel: 128 query rows of one head, with the key tiles of the three levels that they see.
@@ -282,7 +324,7 @@ struct DqItem {
 };
 
 template <int DH>
-__global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_constant__ BwdMaps maps, const BwdTcParams p) {
+__global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const __grid_constant__ BwdMaps maps, const BwdTcParams p) {
     using C = BCfg<DH>;
     constexpr uint32_t kColS = 0, kColDP = 256, kColAcc = 384;
     extern __shared__ uint8_t smem_raw[];
@@ -295,7 +337,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
     __shared__ uint32_t tmem_base_slot;
     __shared__ WaitCtl wait_ctl;
     __shared__ int items[2];
-    __shared__ float gsm[3][kBlk];                        // the second warpgroup's sums of a row, on their way to the first
+    __shared__ float gsm[C::kGsm][3][kBlk];               // the other warpgroups' sums of a row, on their way to the first
 
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // tid >> 5, but provably warp-uniform for the compiler
@@ -311,10 +353,10 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
         }
         mbar_init(&bar.s_full[0], 1); mbar_init(&bar.s_full[1], 1);
         mbar_init(&bar.dp_full, 1);
-        for (int i = 0; i < 2; ++i) { mbar_init(&bar.p_part[i], 8); mbar_init(&bar.ds_part[i], 8); }   // 8 = one arrival per element-wise warp
+        for (int i = 0; i < 2; ++i) { mbar_init(&bar.p_part[i], C::kEw); mbar_init(&bar.ds_part[i], C::kEw); }   // one arrival per element-wise warp
         mbar_init(&bar.acc_done, 1);
         mbar_init(&bar.fixed_free, 1);
-        for (int i = 0; i < 2; ++i) { mbar_init(&bar.item_full[i], 1); mbar_init(&bar.item_free[i], 9); }   // 9: the issuing warp and the element-wise warps
+        for (int i = 0; i < 2; ++i) { mbar_init(&bar.item_full[i], 1); mbar_init(&bar.item_free[i], 1 + C::kEw); }   // the issuing warp and the element-wise warps
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
@@ -327,7 +369,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
     const uint32_t tmem = tmem_base_slot;
     volatile WaitCtl* abortp = &wait_ctl;
 
-    if (warp == kProducerWarp) {
+    if (warp == C::kProducerWarp) {
         int issued_k = 0, issued_v = 0, filled = 0;          // key tiles requested (per ring), items
         bool ok = true;
         int item = blockIdx.x;
@@ -386,7 +428,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
             mbar_wait_warp(&bar.a_full[i % C::kStagesK], (uint32_t)(i / C::kStagesK) & 1u, abortp);
         for (int i = issued_v > C::kStages ? issued_v - C::kStages : 0; i < issued_v; ++i)
             mbar_wait_warp(&bar.b_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
-    } else if (warp == kMmaWarp) {
+    } else if (warp == C::kMmaWarp) {
         {   // every lane runs the issue loop (converged); elect.sync inside the wrappers picks the issuing lane
             // low descriptor words of the operands (see make_desc): K-major views for S and dP, MN-major view of K for dQ
             const uint32_t q_lo = desc_lo_kmajor(smem_u32(sQ)), g_lo = desc_lo_kmajor(smem_u32(sdO));
@@ -438,8 +480,8 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
                         tc_fence_after();
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            const int k = (i >> 1) * 4 + part * 2 + (i & 1);
-                            mma_ts_elect(tmem + kColAcc, tmem + kColDP + packed_half_col(k), make_desc(kta + k * (2048 >> 4)), C::kIdescAcc,
+                            const int k = C::kstep(part, i);
+                            mma_ts_elect(tmem + kColAcc, tmem + kColDP + C::packed_col(k), make_desc(kta + k * (2048 >> 4)), C::kIdescAcc,
                                    (e > 0 || part > 0 || i > 0) ? 1u : 0u);
                         }
                     }
@@ -454,7 +496,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
         const int w = warp >> 2;
         const int r = tid & 127;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        const uint32_t dp_addr = tmem + lane_base + kColDP + w * 64;
+        const uint32_t dp_addr = tmem + lane_base + kColDP + w * C::kCols;
         bool ok = true;
         int g = 0, filled = 0;
 #pragma unroll 1
@@ -462,7 +504,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
         // The warps leave together: those that took an item meet at barriers in its epilogue, so none may be missing there.
         int item = total;
         if (ok) ok = take_item(bar, items, it, item, lane, abortp);
-        if (!softmax_group_all(ok && item < total)) break;
+        if (!softmax_group_all<C::kEw>(ok && item < total)) break;
         const DqItem I(p, item);
         const int E = I.E;
         const long long bh = (long long)I.b * p.H + I.h, m0 = I.m0, m_last = I.m_last, t = m0 + r;
@@ -500,19 +542,15 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
-                float pr[64];
-                {
-                    const uint32_t s_addr = tmem + lane_base + kColS + (g & 1) * 128 + w * 64;
-                    tmem_ld32(s_addr, reinterpret_cast<uint32_t*>(pr));
-                    tmem_ld32(s_addr + 32, reinterpret_cast<uint32_t*>(pr) + 32);
-                    tmem_ld_wait();
-                }
+                float pr[C::kCols];
+                tmem_load<C::kCols>(tmem + lane_base + kColS + (g & 1) * 128 + w * C::kCols, reinterpret_cast<uint32_t*>(pr));
+                tmem_ld_wait();
                 if (!(kt >= full_first && kt < full_end)) {
-                    const long long j0 = (long long)kt * kBlk + w * 64;
-                    mask_cols(pr, (int)max(0LL, min(lo - j0, 64LL)), (int)max(0LL, min(hi - j0, 64LL)));
+                    const long long j0 = (long long)kt * kBlk + w * C::kCols;
+                    mask_cols(pr, (int)max(0LL, min(lo - j0, (long long)C::kCols)), (int)max(0LL, min(hi - j0, (long long)C::kCols)));
                 }
 #pragma unroll
-                for (int c = 0; c < 64; c += 2) {
+                for (int c = 0; c < C::kCols; c += 2) {
                     float x0, x1;
                     unpack2(fma2(pack2(pr[c], pr[c + 1]), scale2, bl2), x0, x1);
                     pr[c] = ex2(x0);
@@ -524,11 +562,11 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
-                float dp[64];
-                tmem_ld32(dp_addr, reinterpret_cast<uint32_t*>(dp));
-                tmem_ld32(dp_addr + 32, reinterpret_cast<uint32_t*>(dp) + 32);
+                float dp[C::kCols];
+                tmem_load<C::kCols>(dp_addr, reinterpret_cast<uint32_t*>(dp));
                 tmem_ld_wait();
-                uint32_t pk[16];
+                constexpr int kHalf = C::kCols / 2;
+                uint32_t pk[kHalf / 2];
                 auto ds_cols = [&](int c_from, int c_to, int c_base) {
 #pragma unroll
                     for (int c = c_from; c < c_to; c += 2) {
@@ -545,12 +583,12 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&bar.ds_part[part]);
                 };
-                ds_cols(0, 32, 0);
-                tmem_st16(dp_addr, pk);
-                ds_cols(32, 48, 32);
+                ds_cols(0, kHalf, 0);
+                tmem_store_part<kHalf>(dp_addr, pk);
+                ds_cols(kHalf, kHalf + kHalf / 2, kHalf);
                 hand_over(0);                                // the first part's store has completed by now
-                ds_cols(48, 64, 32);
-                tmem_st16(dp_addr + 16, pk);
+                ds_cols(kHalf + kHalf / 2, C::kCols, kHalf);
+                tmem_store_part<kHalf>(dp_addr + kHalf / 2, pk);
                 hand_over(1);
             }
             {
@@ -569,15 +607,16 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
         if (ok) {
             tc_fence_after();
             __nv_bfloat16* out = p.dQ + (bh * p.T + t) * DH;
+            constexpr int kOut = DH / C::kGroups, kStep = kOut < 32 ? kOut : 32;     // columns of a warpgroup
 #pragma unroll
-            for (int c0 = w * (DH / 2); c0 < (w + 1) * (DH / 2); c0 += 32) {
-                uint32_t o[32];
+            for (int c0 = w * kOut; c0 < (w + 1) * kOut; c0 += kStep) {
+                uint32_t o[kStep];
                 if (E > 0) {
-                    tmem_ld32(tmem + lane_base + kColAcc + c0, o);
+                    tmem_load<kStep>(tmem + lane_base + kColAcc + c0, o);
                     tmem_ld_wait();
                 } else {
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) o[i] = 0u;
+                    for (int i = 0; i < kStep; ++i) o[i] = 0u;
                 }
                 if (row_valid) store_row_bf16(out + c0, o, p.scale);
             }
@@ -588,16 +627,23 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dq_tc_kernel(const __grid_con
         // (A warp that gave up joins these barriers too.)
         float asum[3], zsum[3];
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            if (half) softmax_group_sync();
-            if (w == 1)
+        for (int half = 0; half < 2; ++half)
 #pragma unroll
-                for (int l = 0; l < 3; ++l) gsm[l][r] = half ? Sl[l] : Al[l];
-            softmax_group_sync();
-            if (w == 0)
+            for (int w0 = 1; w0 < C::kGroups; w0 += C::kGsm) {
+                if (half || w0 > 1) softmax_group_sync<C::kEw>();
+                if (w >= w0 && w < w0 + C::kGsm)
 #pragma unroll
-                for (int l = 0; l < 3; ++l) (half ? zsum : asum)[l] = (half ? Sl[l] : Al[l]) + gsm[l][r];
-        }
+                    for (int l = 0; l < 3; ++l) gsm[w - w0][l][r] = half ? Sl[l] : Al[l];
+                softmax_group_sync<C::kEw>();
+                if (w == 0)
+#pragma unroll
+                    for (int l = 0; l < 3; ++l) {
+                        float v = w0 == 1 ? (half ? Sl[l] : Al[l]) : (half ? zsum[l] : asum[l]);
+#pragma unroll
+                        for (int i = 0; i < C::kGsm; ++i) v += gsm[i][l][r];
+                        (half ? zsum : asum)[l] = v;
+                    }
+            }
         if (w == 0 && ok && row_valid) {
             const float ztot = zsum[0] + zsum[1] + zsum[2];
             const float dd = ztot > 0.f ? (asum[0] + asum[1] + asum[2]) / ztot : 0.f;
@@ -642,9 +688,13 @@ struct DkvItem {
 };
 
 template <int DH>
-__global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_constant__ BwdMaps maps, const BwdTcParams p) {
+__global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(const __grid_constant__ BwdMaps maps, const BwdTcParams p) {
     using C = BCfg<DH>;
     constexpr uint32_t kColS = 0, kColDP = 128, kColDK = 256, kColDV = 256 + DH;
+    // d = 64 leaves room for a second S^T: S^T(g+1) is multiplied while the element-wise threads still work on S^T(g).
+    constexpr bool kTwoS = DH == 64;
+    constexpr uint32_t kColS1 = kTwoS ? 384 : kColS;
+    static_assert(!kTwoS || kColDV + DH <= kColS1, "TMEM columns exceeded");
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     uint8_t* sK = smem;
@@ -666,7 +716,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // tid >> 5, but provably warp-uniform for the compiler
     const int total = (int)p.dkv_items;
-    if (warp == kProducerWarp && lane == 0) {
+    if (warp == C::kProducerWarp && lane == 0) {
         wait_ctl.abort = 0;
         wait_ctl.limit_ns = p.wait_limit_ns;
         mbar_init(&bar.fixed_full, 1);
@@ -674,16 +724,16 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
             mbar_init(&bar.a_full[s], 2); mbar_init(&bar.a_empty[s], 1);
             mbar_init(&bar.b_full[s], 2); mbar_init(&bar.b_empty[s], 1);
         }
-        mbar_init(&bar.s_full[0], 1);
+        mbar_init(&bar.s_full[0], 1); mbar_init(&bar.s_full[1], 1);
         mbar_init(&bar.dp_full, 1);
-        for (int i = 0; i < 2; ++i) { mbar_init(&bar.p_part[i], 8); mbar_init(&bar.ds_part[i], 8); }   // 8 = one arrival per element-wise warp
+        for (int i = 0; i < 2; ++i) { mbar_init(&bar.p_part[i], C::kEw); mbar_init(&bar.ds_part[i], C::kEw); }   // one arrival per element-wise warp
         mbar_init(&bar.acc_done, 1);
         mbar_init(&bar.fixed_free, 1);
-        for (int i = 0; i < 2; ++i) { mbar_init(&bar.item_full[i], 1); mbar_init(&bar.item_free[i], 9); }   // 9: the issuing warp and the element-wise warps
+        for (int i = 0; i < 2; ++i) { mbar_init(&bar.item_full[i], 1); mbar_init(&bar.item_free[i], 3 + C::kEw); }   // the issuing, the slab and the element-wise warps
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // every slab zero (columns 3..15 stay zero), ones for the keys: all threads share the 36 KB
-    for (int i = tid; i < (int)((C::kStages * 2 + 1) * C::kAugBytes / 16); i += kThreads)
+    for (int i = tid; i < (int)((C::kStages * 2 + 1) * C::kAugBytes / 16); i += C::kThreadsDkv)
         reinterpret_cast<uint4*>(sAugQ)[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
     if (tid < kBlk) *reinterpret_cast<uint4*>(sAugK + (tid & 7) * 16 + (tid >> 3) * 256) = make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u);
@@ -698,9 +748,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
     const uint32_t tmem = tmem_base_slot;
     volatile WaitCtl* abortp = &wait_ctl;
 
-    if (warp == kProducerWarp) {
-        // the whole warp runs the loop (converged): lane 0 issues the copies, every lane writes its share of the slabs
-        const float inv_scale = 1.f / p.scale_log2;
+    if (warp == C::kProducerWarp) {
         int issued = 0, issued_b = 0, filled = 0;            // query tiles requested (per ring), items with tiles
         bool ok = true;
         int item = blockIdx.x;
@@ -720,16 +768,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
                 }
                 __syncwarp();
                 ++filled;
-                const float* statB = pick3(p.statB, I.lvl);
                 int hq = I.h * p.kv_group, eq = 0;           // query head and tile-within-head of tile e
-                // this lane's four queries of a tile: their biases and D_t, fetched one tile ahead of the stage they go into
-                auto fetch = [&](float4& bq, float4& dq) {
-                    const long long at = ((long long)I.b * p.H + hq) * p.Tpad + (long long)(I.first + eq) * kBlk + 4 * lane;
-                    bq = *reinterpret_cast<const float4*>(statB + at);
-                    dq = *reinterpret_cast<const float4*>(p.statD + at);
-                };
-                float4 bq, dq;
-                fetch(bq, dq);
                 // Two rings: a stage's dO tile is free again after dV of its tile, its Q tile only after dK, one product later;
                 // and the next tile's Q is what the issuing warp waits for first.  Each is re-filled as soon as it is free.
                 for (int e = 0; e < I.E; ++e) {
@@ -737,7 +776,6 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
                     const uint32_t ph = (uint32_t)(issued / C::kStages) & 1u;
                     if (p.test_stall && e == I.E - 1) { ok = false; break; }       // test hook: the last tile never arrives
                     const int tt = (I.first + eq) * kBlk;
-                    const float bv[4] = {bq.x, bq.y, bq.z, bq.w}, dv[4] = {dq.x, dq.y, dq.z, dq.w};
                     if (!mbar_wait_warp(&bar.b_empty[s], ph ^ 1u, abortp)) { ok = false; break; }
                     if (lane == 0) {
                         mbar_expect_tx(&bar.b_full[s], C::kTile);
@@ -745,15 +783,8 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
                         for (int pn = 0; pn < C::kPanels; ++pn)
                             tma_load_4d(sdO + s * C::kTile + pn * kPanel, &maps.dO, pn * 64, tt, hq, I.b, &bar.b_full[s]);
                     }
-                    ++issued_b;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {                          // -D as three bf16 terms
-                        const int r = 4 * lane + i;
-                        *reinterpret_cast<uint4*>(sAugQ + (s * 2 + 1) * C::kAugBytes + (r & 7) * 16 + (r >> 3) * 256) = split3_bf16(-dv[i]);
-                    }
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(&bar.b_full[s]);
+                    ++issued_b;
                     if (!mbar_wait_warp(&bar.a_empty[s], ph ^ 1u, abortp)) { ok = false; break; }
                     if (lane == 0) {
                         mbar_expect_tx(&bar.a_full[s], C::kTile);
@@ -761,17 +792,9 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
                         for (int pn = 0; pn < C::kPanels; ++pn)
                             tma_load_4d(sQ + s * C::kTile + pn * kPanel, &maps.q, pn * 64, tt, hq, I.b, &bar.a_full[s]);
                     }
-                    ++issued;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {                          // bias / scale as three bf16 terms
-                        const int r = 4 * lane + i;
-                        *reinterpret_cast<uint4*>(sAugQ + (s * 2) * C::kAugBytes + (r & 7) * 16 + (r >> 3) * 256) = split3_bf16(bv[i] * inv_scale);
-                    }
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(&bar.a_full[s]);
+                    ++issued;
                     if (++eq == I.Eq) { eq = 0; ++hq; }
-                    if (e + 1 < I.E) fetch(bq, dq);
                 }
             }
             // The next item is taken only now, with this one's last tiles still in the rings: taken earlier, the items left
@@ -785,7 +808,45 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
             mbar_wait_warp(&bar.a_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
         for (int i = issued_b > C::kStages ? issued_b - C::kStages : 0; i < issued_b; ++i)
             mbar_wait_warp(&bar.b_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
-    } else if (warp == kMmaWarp) {
+    } else if (warp == C::kSlabWarp || warp == C::kSlabWarp + 1) {
+        // The operand slabs of the ninth K-step: the first of these warps writes the bias slabs (ring of the Q tiles), the second
+        // the D slabs (ring of the dO tiles), four queries a lane, fetched one tile ahead.  Warps of their own: when the
+        // warp that issues the copies wrote them too, its loop took 2400 cycles a tile and everything waited for it.
+        const bool is_d = warp != C::kSlabWarp;
+        uint64_t *const full = is_d ? bar.b_full : bar.a_full, *const empty = is_d ? bar.b_empty : bar.a_empty;
+        uint8_t* const slab = sAugQ + (is_d ? C::kAugBytes : 0);
+        const float mul = is_d ? -1.f : 1.f / p.scale_log2;
+        int n_out = 0;
+        bool ok = true;
+        for (int it = 0; ok; ++it) {
+            int item;
+            if (!(ok = take_item(bar, items, it, item, lane, abortp)) || item >= total) break;
+            const DkvItem I(p, item);
+            const float* src = (is_d ? p.statD : pick3(p.statB, I.lvl)) + ((long long)I.b * p.H + (long long)I.h * p.kv_group) * p.Tpad +
+                               (long long)I.first * kBlk + 4 * lane;
+            int eq = 0;
+            float4 next = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (I.E > 0) next = *reinterpret_cast<const float4*>(src);
+            for (int e = 0; e < I.E; ++e, ++n_out) {
+                const int s = n_out % C::kStages;
+                const float v[4] = {next.x * mul, next.y * mul, next.z * mul, next.w * mul};
+                if (++eq == I.Eq) { eq = 0; src += p.Tpad; }
+                if (e + 1 < I.E) next = *reinterpret_cast<const float4*>(src + (long long)eq * kBlk);
+                uint4 row[4];                                        // each value as three bf16 terms
+#pragma unroll
+                for (int i = 0; i < 4; ++i) row[i] = split3_bf16(v[i]);
+                if (!mbar_wait_warp(&empty[s], ((uint32_t)(n_out / C::kStages) & 1u) ^ 1u, abortp)) { ok = false; break; }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = 4 * lane + i;
+                    *reinterpret_cast<uint4*>(slab + s * 2 * C::kAugBytes + (r & 7) * 16 + (r >> 3) * 256) = row[i];
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&full[s]);
+            }
+        }
+    } else if (warp == C::kMmaWarp) {
         {   // every lane runs the issue loop (converged); elect.sync inside the wrappers picks the issuing lane
             // low descriptor words (see make_desc): K-major views for S^T and dP^T, MN-major views of Q and dO for dK and dV
             const uint32_t k_lo = desc_lo_kmajor(smem_u32(sK)), v_lo = desc_lo_kmajor(smem_u32(sV));
@@ -797,11 +858,12 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
                 const int s = g % C::kStages;
                 tc_fence_after();
                 const uint32_t qa = q_lo + s * (C::kTile >> 4);
+                const uint32_t s_col = (g & 1) ? kColS1 : kColS;
 #pragma unroll
                 for (int k = 0; k < DH / 16; ++k)
-                    mma_ss_elect(tmem + kColS, make_desc(k_lo + kstep_off(k, kPanel)), make_desc(qa + kstep_off(k, kPanel)), C::kIdescS, k > 0);
-                mma_ss_elect(tmem + kColS, make_desc_flat(augk_lo), make_desc_flat(augq_lo + s * (2 * C::kAugBytes >> 4)), C::kIdescS, 1u);   // + bias_t / scale
-                mma_commit_elect(&bar.s_full[0]);
+                    mma_ss_elect(tmem + s_col, make_desc(k_lo + kstep_off(k, kPanel)), make_desc(qa + kstep_off(k, kPanel)), C::kIdescS, k > 0);
+                mma_ss_elect(tmem + s_col, make_desc_flat(augk_lo), make_desc_flat(augq_lo + s * (2 * C::kAugBytes >> 4)), C::kIdescS, 1u);   // + bias_t / scale
+                mma_commit_elect(&bar.s_full[kTwoS ? g & 1 : 0]);
             };
             auto issue_dp = [&](int g) -> bool {            // dP^T(g) = V dO(g)^T
                 if (!mbar_wait_warp(&bar.b_full[g % C::kStages], (uint32_t)(g / C::kStages) & 1u, abortp)) return false;
@@ -830,6 +892,11 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
                 if (!issue_dp(g)) { ok = false; break; }
                 if (E == 1) mma_commit_elect(&bar.fixed_free);
                 for (int e = 0; e < E && ok; ++e, ++g) {
+                    const uint32_t s_col = (g & 1) ? kColS1 : kColS;
+                    if (kTwoS && e + 1 < E) {              // its columns: P^T(g-1) was consumed by dV(g-1), issued before
+                        if (!mbar_wait_warp(&bar.a_full[(g + 1) % C::kStages], (uint32_t)((g + 1) / C::kStages) & 1u, abortp)) { ok = false; break; }
+                        issue_s(g + 1);
+                    }
                     const int s = g % C::kStages;
                     const uint32_t qta = qt_lo + s * (C::kTile >> 4), gta = gt_lo + s * (C::kTile >> 4);
                     // dV += P^T(e) dO(e) and dK += dS^T(e) Q(e), each in the two parts in which the element-wise threads
@@ -840,47 +907,60 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
                         tc_fence_after();
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            const int k = (i >> 1) * 4 + part * 2 + (i & 1);
-                            mma_ts_elect(tmem + kColDV, tmem + kColS + packed_half_col(k), make_desc(gta + k * (2048 >> 4)), C::kIdescAcc,
+                            const int k = C::kstep(part, i);
+                            mma_ts_elect(tmem + kColDV, tmem + s_col + C::packed_col(k), make_desc(gta + k * (2048 >> 4)), C::kIdescAcc,
                                    (e > 0 || part > 0 || i > 0) ? 1u : 0u);
                         }
                     }
                     if (!ok) break;
                     mma_commit_elect(&bar.b_empty[s]);                     // dO(e) has had its last reader
-                    // S^T(e+1) needs Q(e+1), which can only be requested once dK(e-1) has released its stage; dK(e) needs dS^T(e)
+                    // S^T(g+1) needs Q(g+1), which can only be requested once dK(g-1) has released its stage; dK(g) needs dS^T(g)
                     // from the element-wise threads.  Either may be ready first, and neither may wait for the other (a late
-                    // dK delays the release, the release the copy, the copy the next S^T): poll both.
-                    {
-                        const int sn = (g + 1) % C::kStages;
-                        const uint32_t phn = (uint32_t)((g + 1) / C::kStages) & 1u;
-                        bool s_out = e + 1 >= E;
-                        int dk_part = 0;
-                        const unsigned long long t0 = gtimer();
-                        while (!s_out || dk_part < 2) {
-                            bool moved = false;
-                            if (!s_out && __all_sync(0xffffffffu, mbar_try(&bar.a_full[sn], phn))) {
-                                issue_s(g + 1);
-                                s_out = moved = true;
-                            }
-                            if (dk_part < 2 && __all_sync(0xffffffffu, mbar_try(&bar.ds_part[dk_part], (uint32_t)g & 1u))) {
-                                tc_fence_after();
+                    // dK delays the release, the release the copy, the copy the next S^T): whichever comes first goes out first.
+                    // The polls stand apart from the products: inside a polling loop the operands of a product are moved
+                    // to uniform registers one by one, and the four products of a part took 390 cycles to issue
+                    // instead of 36.
+                    const uint32_t phg = (uint32_t)g & 1u;
+                    uint64_t* const q_bar = &bar.a_full[(g + 1) % C::kStages];
+                    const uint32_t q_ph = (uint32_t)((g + 1) / C::kStages) & 1u;
+                    auto issue_dk = [&](int part) {
+                        tc_fence_after();
 #pragma unroll
-                                for (int i = 0; i < 4; ++i) {
-                                    const int k = (i >> 1) * 4 + dk_part * 2 + (i & 1);
-                                    mma_ts_elect(tmem + kColDK, tmem + kColDP + packed_half_col(k), make_desc(qta + k * (2048 >> 4)), C::kIdescAcc,
-                                           (e > 0 || dk_part > 0 || i > 0) ? 1u : 0u);
-                                }
-                                ++dk_part;
-                                moved = true;
-                            }
-                            if (!moved) {                            // bounded like every other wait of the kernel
-                                bool give_up = abortp->abort != 0;
-                                if (!give_up && gtimer() - t0 > abortp->limit_ns) { abortp->abort = 1; give_up = true; }
-                                if (__any_sync(0xffffffffu, give_up)) { ok = false; break; }
+                        for (int i = 0; i < 4; ++i) {
+                            const int k = C::kstep(part, i);
+                            mma_ts_elect(tmem + kColDK, tmem + kColDP + C::packed_col(k), make_desc(qta + k * (2048 >> 4)), C::kIdescAcc,
+                                         (e > 0 || part > 0 || i > 0) ? 1u : 0u);
+                        }
+                    };
+                    if (!kTwoS && e + 1 < E) {
+                        const int first = poll_two(q_bar, q_ph, &bar.ds_part[0], phg, abortp);
+                        if (first < 0) { ok = false; break; }
+                        if (first == 0) {
+                            issue_s(g + 1);
+                            if (!mbar_wait_warp(&bar.ds_part[0], phg, abortp)) { ok = false; break; }
+                            issue_dk(0);
+                            if (!mbar_wait_warp(&bar.ds_part[1], phg, abortp)) { ok = false; break; }
+                            issue_dk(1);
+                        } else {
+                            issue_dk(0);
+                            const int second = poll_two(q_bar, q_ph, &bar.ds_part[1], phg, abortp);
+                            if (second < 0) { ok = false; break; }
+                            if (second == 0) {
+                                issue_s(g + 1);
+                                if (!mbar_wait_warp(&bar.ds_part[1], phg, abortp)) { ok = false; break; }
+                                issue_dk(1);
+                            } else {
+                                issue_dk(1);
+                                if (!mbar_wait_warp(q_bar, q_ph, abortp)) { ok = false; break; }
+                                issue_s(g + 1);
                             }
                         }
+                    } else {
+                        if (!mbar_wait_warp(&bar.ds_part[0], phg, abortp)) { ok = false; break; }
+                        issue_dk(0);
+                        if (!mbar_wait_warp(&bar.ds_part[1], phg, abortp)) { ok = false; break; }
+                        issue_dk(1);
                     }
-                    if (!ok) break;
                     mma_commit_elect(&bar.a_empty[s]);
                     if (e + 1 < E) {
                         if (!issue_dp(g + 1)) { ok = false; break; }
@@ -895,8 +975,7 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
         const int w = warp >> 2;
         const int r = tid & 127;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        const uint32_t s_addr = tmem + lane_base + kColS + w * 64;
-        const uint32_t dp_addr = tmem + lane_base + kColDP + w * 64;
+        const uint32_t dp_addr = tmem + lane_base + kColDP + w * C::kCols;
         bool ok = true;
         int g = 0, filled = 0;
 #pragma unroll 1
@@ -917,23 +996,24 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
             const long long tt = (long long)(first + eq) * kBlk;       // first query of the tile
             if (++eq == Eq) eq = 0;
             // phase 1: P^T = 2^(scale * (s + bias_t / scale)) for this thread's 64 query columns; the sum comes from the tensor pipe
-            ok = mbar_wait(&bar.s_full[0], (uint32_t)g & 1u, abortp);
+            ok = kTwoS ? mbar_wait(&bar.s_full[g & 1], (uint32_t)(g >> 1) & 1u, abortp) : mbar_wait(&bar.s_full[0], (uint32_t)g & 1u, abortp);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
-            float pr[64];
-            tmem_ld32(s_addr, reinterpret_cast<uint32_t*>(pr));
-            tmem_ld32(s_addr + 32, reinterpret_cast<uint32_t*>(pr) + 32);
+            const uint32_t s_addr = tmem + lane_base + ((g & 1) ? kColS1 : kColS) + w * C::kCols;
+            float pr[C::kCols];
+            tmem_load<C::kCols>(s_addr, reinterpret_cast<uint32_t*>(pr));
             tmem_ld_wait();
             // tiles whose every (key, query) pair is visible need no mask
             bool full = true;
             if (lvl != 2) full = full && (j_last - p.q_offset <= tt);
             if (lvl == 0) full = full && (j0 + p.window - p.q_offset >= tt + kBlk);
             if (!full) {
-                const long long c0 = tt + w * 64;
-                mask_cols(pr, (int)max(0LL, min(q_lo - c0, 64LL)), (int)max(0LL, min(q_hi - c0, 64LL)));
+                const long long c0 = tt + w * C::kCols;
+                mask_cols(pr, (int)max(0LL, min(q_lo - c0, (long long)C::kCols)), (int)max(0LL, min(q_hi - c0, (long long)C::kCols)));
             }
-            uint32_t pk[32];        // P^T rounded to bf16; phase 2 uses these same rounded values
+            constexpr int kHalf = C::kCols / 2;
+            uint32_t pk[kHalf];     // P^T rounded to bf16; phase 2 uses these same rounded values
             const uint64_t scale2 = pack2(p.scale_log2, p.scale_log2);
             auto p_cols = [&](int c_from, int c_to) {
 #pragma unroll
@@ -954,22 +1034,21 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar_part);
             };
-            // each half of the thread's 64 columns goes out as soon as it is ready; the first half is handed over in
+            // each half of the thread's columns goes out as soon as it is ready; the first half is handed over in
             // the middle of the second half's exponentials, when its store has long completed
-            p_cols(0, 32);
-            tmem_st16(s_addr, pk);
-            p_cols(32, 48);
+            p_cols(0, kHalf);
+            tmem_store_part<kHalf>(s_addr, pk);
+            p_cols(kHalf, kHalf + kHalf / 2);
             hand_over(&bar.p_part[0]);
-            p_cols(48, 64);
-            tmem_st16(s_addr + 16, pk + 16);
+            p_cols(kHalf + kHalf / 2, C::kCols);
+            tmem_store_part<kHalf>(s_addr + kHalf / 2, pk + kHalf / 2);
             hand_over(&bar.p_part[1]);
             // phase 2: dS^T = P^T (dP^T - D_t), written over the columns just read; the difference comes from the tensor pipe
             ok = mbar_wait(&bar.dp_full, (uint32_t)g & 1u, abortp);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
-            tmem_ld32(dp_addr, reinterpret_cast<uint32_t*>(pr));
-            tmem_ld32(dp_addr + 32, reinterpret_cast<uint32_t*>(pr) + 32);
+            tmem_load<C::kCols>(dp_addr, reinterpret_cast<uint32_t*>(pr));
             tmem_ld_wait();
             auto ds_cols = [&](int c_from, int c_to) {
 #pragma unroll
@@ -980,29 +1059,33 @@ __global__ void __launch_bounds__(kThreads, 1) bwd_dkv_tc_kernel(const __grid_co
                     pk[c / 2] = pack_bf16(s0, s1);
                 }
             };
-            ds_cols(0, 32);
-            tmem_st16(dp_addr, pk);
-            ds_cols(32, 48);
+            ds_cols(0, kHalf);
+            tmem_store_part<kHalf>(dp_addr, pk);
+            ds_cols(kHalf, kHalf + kHalf / 2);
             hand_over(&bar.ds_part[0]);
-            ds_cols(48, 64);
-            tmem_st16(dp_addr + 16, pk + 16);
+            ds_cols(kHalf + kHalf / 2, C::kCols);
+            tmem_store_part<kHalf>(dp_addr + kHalf / 2, pk + kHalf / 2);
             hand_over(&bar.ds_part[1]);
         }
-        // ------------------------------------------------------------ epilogue: warpgroup 0 writes dK, 1 writes dV
+        // ------------------------------------------------------------ epilogue
         if (ok && E > 0) {
             ok = mbar_wait(&bar.acc_done, (uint32_t)filled++ & 1u, abortp);
             ok = __all_sync(0xffffffffu, ok);
         }
         if (ok) {
             tc_fence_after();
+            // half of the warpgroups write dK, the others dV, each its share of the columns
+            const bool is_k = w < C::kGroups / 2;
+            constexpr int kOut = 2 * DH / C::kGroups;
+            const int c_first = (is_k ? w : w - C::kGroups / 2) * kOut;
             const LevelGradDev dL = p.dL[lvl];
-            __nv_bfloat16* out = static_cast<__nv_bfloat16*>(w == 0 ? dL.dk : dL.dv) + I.b * dL.sb + I.h * dL.sh + j * dL.sn;
-            const float mul = w == 0 ? p.scale : 1.f;
+            __nv_bfloat16* out = static_cast<__nv_bfloat16*>(is_k ? dL.dk : dL.dv) + I.b * dL.sb + I.h * dL.sh + j * dL.sn;
+            const float mul = is_k ? p.scale : 1.f;
 #pragma unroll
-            for (int c0 = 0; c0 < DH; c0 += 32) {
+            for (int c0 = c_first; c0 < c_first + kOut; c0 += 32) {
                 uint32_t o[32];
                 if (E > 0) {
-                    tmem_ld32(tmem + lane_base + (w == 0 ? kColDK : kColDV) + c0, o);
+                    tmem_ld32(tmem + lane_base + (is_k ? kColDK : kColDV) + c0, o);
                     tmem_ld_wait();
                 } else {
 #pragma unroll
@@ -1071,7 +1154,7 @@ cudaError_t launch_t(const BwdParams& bp, unsigned int* status_word, cudaStream_
         if (e != cudaSuccess) return e;
         p.dq_items = (long long)(Tpad / kBlk) * bp.H * bp.B;
         p.dq_ticket = status_word + 2;
-        bwd_dq_tc_kernel<DH><<<(unsigned)(p.dq_items < 148 ? p.dq_items : 148), kThreads, C::kSmemDq, st>>>(m, p);
+        bwd_dq_tc_kernel<DH><<<(unsigned)(p.dq_items < 148 ? p.dq_items : 148), C::kThreads, C::kSmemDq, st>>>(m, p);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     const int tiles = p.kv_tiles[0] + p.kv_tiles[1] + p.kv_tiles[2];
@@ -1090,7 +1173,7 @@ cudaError_t launch_t(const BwdParams& bp, unsigned int* status_word, cudaStream_
         if (e != cudaSuccess) return e;
         p.dkv_items = (long long)tiles * H_kv * bp.B;
         p.dkv_ticket = status_word + 1;
-        bwd_dkv_tc_kernel<DH><<<(unsigned)(p.dkv_items < 148 ? p.dkv_items : 148), kThreads, C::kSmemDkv, st>>>(m, p);
+        bwd_dkv_tc_kernel<DH><<<(unsigned)(p.dkv_items < 148 ? p.dkv_items : 148), C::kThreadsDkv, C::kSmemDkv, st>>>(m, p);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return launch_bwd_dgate(bp.Gpart, bp.B, bp.H, bp.T, bp.dG, st);
