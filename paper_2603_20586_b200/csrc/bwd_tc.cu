@@ -163,18 +163,26 @@ __device__ __forceinline__ int poll_two(uint64_t* b0, uint32_t ph0, uint64_t* b1
 // Items (output tiles) are dealt from a ticket counter: a CTA takes the next one when it is free, in the order in which
 // blocks of a plain grid would start.  The producing warp posts the number of item `it` to the other roles; a number past
 // the last item ends them all.
-__device__ __forceinline__ bool post_item(BwdBarriers& bar, int (&items)[2], int it, int item, int lane, volatile WaitCtl* ctl) {
+// The posted item is the whole description (Item: ints only), so that its divisions are made once and early.
+template <typename Item>
+__device__ __forceinline__ bool post_item(BwdBarriers& bar, Item (&items)[2], int it, const Item& item, int lane, volatile WaitCtl* ctl) {
     if (it >= 2 && !mbar_wait_warp(&bar.item_free[it & 1], (uint32_t)((it >> 1) - 1) & 1u, ctl)) return false;
     if (lane == 0) {
-        *reinterpret_cast<volatile int*>(&items[it & 1]) = item;
+        items[it & 1] = item;
         mbar_arrive(&bar.item_full[it & 1]);
     }
     __syncwarp();
     return true;
 }
-__device__ __forceinline__ bool take_item(BwdBarriers& bar, int (&items)[2], int it, int& item, int lane, volatile WaitCtl* ctl) {
+template <typename Item>
+__device__ __forceinline__ bool take_item(BwdBarriers& bar, Item (&items)[2], int it, Item& item, int lane, volatile WaitCtl* ctl) {
     if (!mbar_wait_warp(&bar.item_full[it & 1], (uint32_t)(it >> 1) & 1u, ctl)) return false;
-    item = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&items[it & 1]), 0);   // warp-uniform for the compiler too
+    const int* src = reinterpret_cast<const int*>(&items[it & 1]);
+    int v[sizeof(Item) / 4];
+#pragma unroll
+    for (int i = 0; i < (int)(sizeof(Item) / 4); ++i) v[i] = __shfl_sync(0xffffffffu, src[i], 0);      // warp-uniform for the compiler too
+    memcpy(&item, v, sizeof(Item));
+    __syncwarp();
     if (lane == 0) mbar_arrive(&bar.item_free[it & 1]);
     return true;
 }
@@ -289,30 +297,20 @@ __device__ __forceinline__ void tmem_store_part(uint32_t addr, const uint32_t* r
     else tmem_st8(addr, r);
 }
 
-template <int N>
-__device__ __forceinline__ void store_row_bf16(__nv_bfloat16* dst, const uint32_t (&o)[N], float mul) {
-#pragma unroll
-    for (int i = 0; i < N; i += 8) {
-        uint4 v;
-        v.x = pack_bf16(__uint_as_float(o[i]) * mul, __uint_as_float(o[i + 1]) * mul);
-        v.y = pack_bf16(__uint_as_float(o[i + 2]) * mul, __uint_as_float(o[i + 3]) * mul);
-        v.z = pack_bf16(__uint_as_float(o[i + 4]) * mul, __uint_as_float(o[i + 5]) * mul);
-        v.w = pack_bf16(__uint_as_float(o[i + 6]) * mul, __uint_as_float(o[i + 7]) * mul);
-        *reinterpret_cast<uint4*>(dst + i) = v;
-    }
-}
-
 // ------------------------------------------------------------------------------------------ dQ
 // One item of the dQ kernel: 128 query rows of one head, with the key tiles of the three levels that they see.
 struct DqItem {
-    int b, h, E;
+    int b, h, E;                          // E < 0: there is no further item
     int first[3], end[3];
-    long long m0, m_last;
+    int m0, m_last;
+    DqItem() = default;
     __device__ __forceinline__ DqItem(const BwdTcParams& p, int item) {
+        E = -1;
+        if (item >= (int)p.dq_items) return;
         const int tiles = p.Tpad / kBlk, bh = item / tiles;
         b = bh / p.H; h = bh - b * p.H;
-        m0 = (long long)(tiles - 1 - (item - bh * tiles)) * kBlk;          // latest (heaviest) rows of a head first
-        m_last = (m0 + kBlk - 1 < p.T - 1) ? m0 + kBlk - 1 : p.T - 1;
+        m0 = (tiles - 1 - (item - bh * tiles)) * kBlk;          // latest (heaviest) rows of a head first
+        m_last = min(m0 + kBlk - 1, p.T - 1);
         E = 0;
 #pragma unroll
         for (int l = 0; l < 3; ++l) {
@@ -336,13 +334,11 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const 
     __shared__ BwdBarriers bar;
     __shared__ uint32_t tmem_base_slot;
     __shared__ WaitCtl wait_ctl;
-    __shared__ int items[2];
+    __shared__ DqItem items[2];
     __shared__ float gsm[C::kGsm][3][kBlk];               // the other warpgroups' sums of a row, on their way to the first
 
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // tid >> 5, but provably warp-uniform for the compiler
-    const int total = (int)p.dq_items;
-
     if (tid == 0) {
         wait_ctl.abort = 0;
         wait_ctl.limit_ns = p.wait_limit_ns;
@@ -374,8 +370,8 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const 
         bool ok = true;
         int item = blockIdx.x;
         for (int it = 0; ok; ++it) {
-            if (!(ok = post_item(bar, items, it, item, lane, abortp)) || item >= total) break;
             const DqItem I(p, item);
+            if (!(ok = post_item(bar, items, it, I, lane, abortp)) || I.E < 0) break;
             const int kvh = I.h / p.kv_group;
             if (I.E > 0) {
                 // the previous item's Q and dO have had their last reader when its last dP is complete
@@ -450,9 +446,9 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const 
             int g = 0, filled = 0;
             bool ok = true;
             for (int it = 0; ok; ++it) {
-                int item;
-                if (!(ok = take_item(bar, items, it, item, lane, abortp)) || item >= total) break;
-                const int E = DqItem(p, item).E;
+                DqItem I;
+                if (!(ok = take_item(bar, items, it, I, lane, abortp)) || I.E < 0) break;
+                const int E = I.E;
                 if (E == 0) continue;
                 // S(0) and dP(0) of this item run while the element-wise threads still store the previous one's dQ: the
                 // accumulator is not touched before those threads hand over the first dS.
@@ -502,10 +498,10 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const 
 #pragma unroll 1
         for (int it = 0;; ++it) {
         // The warps leave together: those that took an item meet at barriers in its epilogue, so none may be missing there.
-        int item = total;
-        if (ok) ok = take_item(bar, items, it, item, lane, abortp);
-        if (!softmax_group_all<C::kEw>(ok && item < total)) break;
-        const DqItem I(p, item);
+        DqItem I;
+        I.E = -1;
+        if (ok) ok = take_item(bar, items, it, I, lane, abortp);
+        if (!softmax_group_all<C::kEw>(ok && I.E >= 0)) break;
         const int E = I.E;
         const long long bh = (long long)I.b * p.H + I.h, m0 = I.m0, m_last = I.m_last, t = m0 + r;
         const bool row_valid = t < p.T;
@@ -606,7 +602,8 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const 
         }
         if (ok) {
             tc_fence_after();
-            __nv_bfloat16* out = p.dQ + (bh * p.T + t) * DH;
+            const int first_row = (warp & 3) * 32;                     // of this warp, within the tile
+            __nv_bfloat16* out = p.dQ + (bh * p.T + m0 + first_row) * DH;
             constexpr int kOut = DH / C::kGroups, kStep = kOut < 32 ? kOut : 32;     // columns of a warpgroup
 #pragma unroll
             for (int c0 = w * kOut; c0 < (w + 1) * kOut; c0 += kStep) {
@@ -618,7 +615,7 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const 
 #pragma unroll
                     for (int i = 0; i < kStep; ++i) o[i] = 0u;
                 }
-                if (row_valid) store_row_bf16(out + c0, o, p.scale);
+                store_rows_bf16<kStep>(out + c0, DH, (int)min(32LL, p.T - m0 - first_row), o, p.scale, lane);
             }
         }
         // Gate-logit gradient of this head: G_l = sum_{j in l} p (dP - D').  D' = sum p dP / sum p equals
@@ -663,22 +660,25 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const 
 // ------------------------------------------------------------------------------------------ dK, dV
 // One item of the dK/dV kernel: a key tile of one level and KV head, with the query tiles that see it.
 struct DkvItem {
-    int b, h, lvl, first, Eq, E;          // h: KV head; its query heads are h * G .. h * G + G - 1
-    long long n, j0, j_last;
+    int b, h, lvl, first, Eq, E;          // h: KV head; its query heads are h * G .. h * G + G - 1;  E < 0: there is no further item
+    int n, j0, j_last;                    // (levels of this path hold fewer than 2^31 - 256 rows)
+    DkvItem() = default;
     __device__ __forceinline__ DkvItem(const BwdTcParams& p, int item) {
+        E = -1;
+        if (item >= (int)p.dkv_items) return;
         const int tiles = p.kv_tiles[0] + p.kv_tiles[1] + p.kv_tiles[2], bh = item / tiles;
         int kt = item - bh * tiles;
         b = bh / p.H_kv; h = bh - b * p.H_kv;
         // key tiles of a head in decreasing order of work: L3 (seen by every query), L2 from the oldest key on, L1
         lvl = 2;
         if (kt >= p.kv_tiles[2]) { kt -= p.kv_tiles[2]; lvl = 1; if (kt >= p.kv_tiles[1]) { kt -= p.kv_tiles[1]; lvl = 0; } }
-        n = pick3(p.n, lvl);
-        j0 = (long long)kt * kBlk;
-        j_last = (j0 + kBlk - 1 < n - 1) ? j0 + kBlk - 1 : n - 1;
+        n = (int)pick3(p.n, lvl);
+        j0 = kt * kBlk;
+        j_last = min(j0 + kBlk - 1, n - 1);
         // queries t (position t + q_offset) that can see a key of this tile
         long long t_lo = 0, t_hi = p.T;
-        if (lvl == 0) { t_lo = j0 - p.q_offset; t_hi = j_last + p.window - p.q_offset; }
-        else if (lvl == 1) { t_lo = j0 - p.q_offset; }
+        if (lvl == 0) { t_lo = (long long)j0 - p.q_offset; t_hi = (long long)j_last + p.window - p.q_offset; }
+        else if (lvl == 1) { t_lo = (long long)j0 - p.q_offset; }
         if (t_lo < 0) t_lo = 0;
         if (t_hi > p.T) t_hi = p.T;
         first = t_hi > t_lo ? (int)(t_lo / kBlk) : 0;
@@ -711,11 +711,10 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
     __shared__ BwdBarriers bar;
     __shared__ uint32_t tmem_base_slot;
     __shared__ WaitCtl wait_ctl;
-    __shared__ int items[2];
+    __shared__ DkvItem items[2];
 
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // tid >> 5, but provably warp-uniform for the compiler
-    const int total = (int)p.dkv_items;
     if (warp == C::kProducerWarp && lane == 0) {
         wait_ctl.abort = 0;
         wait_ctl.limit_ns = p.wait_limit_ns;
@@ -753,8 +752,8 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
         bool ok = true;
         int item = blockIdx.x;
         for (int it = 0; ok; ++it) {
-            if (!(ok = post_item(bar, items, it, item, lane, abortp)) || item >= total) break;
             const DkvItem I(p, item);
+            if (!(ok = post_item(bar, items, it, I, lane, abortp)) || I.E < 0) break;
             if (I.E > 0) {
                 // the previous item's K and V have had their last reader when its last dP^T is complete
                 if (filled > 0 && !mbar_wait_warp(&bar.fixed_free, (uint32_t)(filled - 1) & 1u, abortp)) { ok = false; break; }
@@ -819,9 +818,8 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
         int n_out = 0;
         bool ok = true;
         for (int it = 0; ok; ++it) {
-            int item;
-            if (!(ok = take_item(bar, items, it, item, lane, abortp)) || item >= total) break;
-            const DkvItem I(p, item);
+            DkvItem I;
+            if (!(ok = take_item(bar, items, it, I, lane, abortp)) || I.E < 0) break;
             const float* src = (is_d ? p.statD : pick3(p.statB, I.lvl)) + ((long long)I.b * p.H + (long long)I.h * p.kv_group) * p.Tpad +
                                (long long)I.first * kBlk + 4 * lane;
             int eq = 0;
@@ -879,9 +877,9 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
             int g = 0, filled = 0;
             bool ok = true;
             for (int it = 0; ok; ++it) {
-                int item;
-                if (!(ok = take_item(bar, items, it, item, lane, abortp)) || item >= total) break;
-                const int E = DkvItem(p, item).E;
+                DkvItem I;
+                if (!(ok = take_item(bar, items, it, I, lane, abortp)) || I.E < 0) break;
+                const int E = I.E;
                 if (E == 0) continue;
                 // S^T(0) and dP^T(0) of this item run while the element-wise threads still store the previous one's dK and
                 // dV: the accumulators are not touched before those threads hand over the first P^T.
@@ -891,20 +889,24 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
                 issue_s(g);
                 if (!issue_dp(g)) { ok = false; break; }
                 if (E == 1) mma_commit_elect(&bar.fixed_free);
+                auto wait_q = [&](int gq) { return mbar_wait_warp(&bar.a_full[gq % C::kStages], (uint32_t)(gq / C::kStages) & 1u, abortp); };
+                if (kTwoS && E > 1) {
+                    if (!wait_q(g + 1)) { ok = false; break; }
+                    issue_s(g + 1);
+                }
                 for (int e = 0; e < E && ok; ++e, ++g) {
                     const uint32_t s_col = (g & 1) ? kColS1 : kColS;
-                    if (kTwoS && e + 1 < E) {              // its columns: P^T(g-1) was consumed by dV(g-1), issued before
-                        if (!mbar_wait_warp(&bar.a_full[(g + 1) % C::kStages], (uint32_t)((g + 1) / C::kStages) & 1u, abortp)) { ok = false; break; }
-                        issue_s(g + 1);
-                    }
                     const int s = g % C::kStages;
                     const uint32_t qta = qt_lo + s * (C::kTile >> 4), gta = gt_lo + s * (C::kTile >> 4);
                     // dV += P^T(e) dO(e) and dK += dS^T(e) Q(e), each in the two parts in which the element-wise threads
                     // hand their 64 columns over (K-steps {0, 1, 4, 5}, then {2, 3, 6, 7})
 #pragma unroll
                     for (int part = 0; part < 2; ++part) {
-                        if (!mbar_wait_warp(&bar.p_part[part], (uint32_t)g & 1u, abortp)) { ok = false; break; }
-                        tc_fence_after();
+                        // (with two S^T the element-wise threads are ahead: one wait, for the second part, costs less than two)
+                        if (!kTwoS || part == 0) {
+                            if (!mbar_wait_warp(&bar.p_part[kTwoS ? 1 : part], (uint32_t)g & 1u, abortp)) { ok = false; break; }
+                            tc_fence_after();
+                        }
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
                             const int k = C::kstep(part, i);
@@ -932,7 +934,23 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
                                          (e > 0 || part > 0 || i > 0) ? 1u : 0u);
                         }
                     };
-                    if (!kTwoS && e + 1 < E) {
+                    if constexpr (kTwoS) {
+                        // S^T(g+1) is long there; behind dK(g) follow dP^T(g+1) and S^T(g+2), whose columns dV(g) has read
+                        if (!mbar_wait_warp(&bar.ds_part[1], phg, abortp)) { ok = false; break; }
+                        issue_dk(0);
+                        issue_dk(1);
+                        mma_commit_elect(&bar.a_empty[s]);
+                        if (e + 1 < E) {
+                            if (!issue_dp(g + 1)) { ok = false; break; }
+                            if (e + 2 == E) mma_commit_elect(&bar.fixed_free);
+                        }
+                        if (e + 2 < E) {
+                            if (!wait_q(g + 2)) { ok = false; break; }
+                            issue_s(g + 2);
+                        }
+                        continue;
+                    }
+                    if (e + 1 < E) {
                         const int first = poll_two(q_bar, q_ph, &bar.ds_part[0], phg, abortp);
                         if (first < 0) { ok = false; break; }
                         if (first == 0) {
@@ -980,9 +998,8 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
         int g = 0, filled = 0;
 #pragma unroll 1
         for (int it = 0; ok; ++it) {
-        int item;
-        if (!(ok = take_item(bar, items, it, item, lane, abortp)) || item >= total) break;
-        const DkvItem I(p, item);
+        DkvItem I;
+        if (!(ok = take_item(bar, items, it, I, lane, abortp)) || I.E < 0) break;
         const int lvl = I.lvl, E = I.E, Eq = I.Eq, first = I.first;
         const long long j0 = I.j0, j_last = I.j_last, j = j0 + r;
         const bool row_valid = j < I.n;
@@ -1078,8 +1095,9 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
             const bool is_k = w < C::kGroups / 2;
             constexpr int kOut = 2 * DH / C::kGroups;
             const int c_first = (is_k ? w : w - C::kGroups / 2) * kOut;
+            const int first_row = (warp & 3) * 32;                     // of this warp, within the tile
             const LevelGradDev dL = p.dL[lvl];
-            __nv_bfloat16* out = static_cast<__nv_bfloat16*>(is_k ? dL.dk : dL.dv) + I.b * dL.sb + I.h * dL.sh + j * dL.sn;
+            __nv_bfloat16* out = static_cast<__nv_bfloat16*>(is_k ? dL.dk : dL.dv) + I.b * dL.sb + I.h * dL.sh + (j0 + first_row) * dL.sn;
             const float mul = is_k ? p.scale : 1.f;
 #pragma unroll
             for (int c0 = c_first; c0 < c_first + kOut; c0 += 32) {
@@ -1091,7 +1109,7 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
 #pragma unroll
                     for (int i = 0; i < 32; ++i) o[i] = 0u;
                 }
-                if (row_valid) store_row_bf16(out + c0, o, mul);
+                store_rows_bf16<32>(out + c0, dL.sn, (int)min(32LL, (long long)I.n - j0 - first_row), o, mul, lane);
             }
         }
         }   // items

@@ -706,29 +706,21 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
             float l_row = l_run;
             if constexpr (C::kSplit == 2) l_row += lsum[q][half ^ 1][row_in_tile];
             const float inv = l_row > 0.f ? 1.f / l_row : 0.f;   // rows with nothing visible: exact zeros
-            __nv_bfloat16* Orow = p.O + (((long long)b * p.H + h) * p.T + t) * DH + half * (DH / C::kSplit);
+            const int first_row = (warp & 3) * 32;                       // of this warp, within the query tile
+            __nv_bfloat16* out = p.O + (((long long)b * p.H + h) * p.T + tq0 + first_row) * DH + half * (DH / C::kSplit);
+            const int rows_here = (int)max(0LL, min(32LL, p.T - tq0 - first_row));
 #pragma unroll 1
             for (int c0 = 0; c0 < DH / C::kSplit; c0 += 32) {
                 uint32_t o[32];
                 if (E > 0) {
                     tmem_ld32(o_addr + c0, o);
                     tmem_ld_wait();
-                } else {
+                }
+                if (E == 0 || !(inv > 0.f)) {
 #pragma unroll
                     for (int i = 0; i < 32; ++i) o[i] = 0u;
                 }
-                if (row_valid) {
-#pragma unroll
-                    for (int i = 0; i < 32; i += 8) {
-                        uint4 v;
-                        const float z = inv;
-                        v.x = pack_bf16(z > 0.f ? __uint_as_float(o[i]) * z : 0.f, z > 0.f ? __uint_as_float(o[i + 1]) * z : 0.f);
-                        v.y = pack_bf16(z > 0.f ? __uint_as_float(o[i + 2]) * z : 0.f, z > 0.f ? __uint_as_float(o[i + 3]) * z : 0.f);
-                        v.z = pack_bf16(z > 0.f ? __uint_as_float(o[i + 4]) * z : 0.f, z > 0.f ? __uint_as_float(o[i + 5]) * z : 0.f);
-                        v.w = pack_bf16(z > 0.f ? __uint_as_float(o[i + 6]) * z : 0.f, z > 0.f ? __uint_as_float(o[i + 7]) * z : 0.f);
-                        *reinterpret_cast<uint4*>(Orow + c0 + i) = v;
-                    }
-                }
+                store_rows_bf16<32>(out + c0, DH, rows_here, o, inv, lane);
             }
             if (row_valid && half == 0 && p.LSE)
                 p.LSE[((long long)b * p.H + h) * p.T + t] = l_row > 0.f ? (m_run + log2f(l_row)) * kLn2 : -INFINITY;

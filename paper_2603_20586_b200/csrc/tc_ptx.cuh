@@ -206,6 +206,43 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return r;
 }
 
+// Stores N = 16 or 32 consecutive columns of the warp's 32 rows (thread = row) as bf16.  A thread's own 16-byte pieces lie a
+// row apart from its neighbours', so stored as they are every instruction touches 32 lines and the store unit takes one
+// cycle for each; the lanes of a group first exchange pieces so that the group writes one row's N * 2 bytes at a
+// time.  `row0` points at the first column of the warp's first row, `rows` of which (at most 32) exist.
+template <int N>
+__device__ __forceinline__ void store_rows_bf16(__nv_bfloat16* row0, long long stride, int rows, const uint32_t* o, float mul, int lane) {
+    constexpr int C = N / 8;                             // pieces of a row, lanes of a group
+    static_assert(C == 2 || C == 4, "16 or 32 columns");
+    uint4 v[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        v[c].x = pack_bf16(__uint_as_float(o[8 * c]) * mul, __uint_as_float(o[8 * c + 1]) * mul);
+        v[c].y = pack_bf16(__uint_as_float(o[8 * c + 2]) * mul, __uint_as_float(o[8 * c + 3]) * mul);
+        v[c].z = pack_bf16(__uint_as_float(o[8 * c + 4]) * mul, __uint_as_float(o[8 * c + 5]) * mul);
+        v[c].w = pack_bf16(__uint_as_float(o[8 * c + 6]) * mul, __uint_as_float(o[8 * c + 7]) * mul);
+    }
+    // transposition of the group's C x C pieces: lane g ends with piece g of every row of the group
+#pragma unroll
+    for (int bit = 1; bit < C; bit <<= 1) {
+        const bool up = (lane & bit) != 0;
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            if (c & bit) continue;
+            uint4 &lo = v[c], &hi = v[c | bit];
+            const uint4 give = up ? lo : hi;
+            uint4 got;
+            got.x = __shfl_xor_sync(0xffffffffu, give.x, bit); got.y = __shfl_xor_sync(0xffffffffu, give.y, bit);
+            got.z = __shfl_xor_sync(0xffffffffu, give.z, bit); got.w = __shfl_xor_sync(0xffffffffu, give.w, bit);
+            if (up) lo = got; else hi = got;
+        }
+    }
+    const int r0 = lane & ~(C - 1);
+    __nv_bfloat16* at = row0 + (long long)r0 * stride + (lane & (C - 1)) * 8;
+#pragma unroll
+    for (int i = 0; i < C; ++i)
+        if (r0 + i < rows) *reinterpret_cast<uint4*>(at + i * stride) = v[i];
+}
 
 // Host side: tensor map of a [B, H, rows, d] bf16 tensor with element strides (sb, sh, sn, 1) whose box
 // is 64 columns x box_rows rows, 128-byte swizzled (one shared-memory panel per box).
