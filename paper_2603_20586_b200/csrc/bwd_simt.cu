@@ -1,63 +1,64 @@
 // CUDA-core backward of Eq. 5 (derived by differentiating it; the paper prints no backward).
 // With p = lambda exp(s - LSE) on the visible set, D_t = dO_t . O_t and dS = p (dO_t . v - D_t):
-//   kernel delta : D[b,h,t]
-//   kernel dq    : dQ_t = tau sum_{l,j} dS k_{l,j};  per-head gate-logit gradient G[b,h,t,l] = sum_j dS
-//   kernel dkv   : dK_{l,j} = tau sum_t dS q_t;  dV_{l,j} = sum_t p dO_t       (one launch per level)
+//   kernel dq    : dQ_t = tau sum_{l,j} dS k_{l,j};  per-head gate-logit gradient G[b,h,t,l] = sum_j dS;  D[b,h,t]
+//   kernel dkv   : dK_{l,j} = tau sum_t dS q_t;  dV_{l,j} = sum_t p dO_t       (one launch for the three levels)
 //   kernel dgate : dG[b,t,l] = sum_h G[b,h,t,l]                               (fixed order)
-// Every output element is produced by exactly one thread in a fixed summation order, so the result is
-// deterministic.  fp32 arithmetic; tiles of 32 x 32 (query x key) staged in shared memory.
-#include "common.cuh"
+// Every output element is produced by exactly one CTA in a fixed summation order, so the result is
+// deterministic.  fp32 arithmetic; 16 rows against tiles of 32, see simt.cuh.
+#include "simt.cuh"
 
 namespace mka {
 namespace {
 
-constexpr int kRows = 32, kKeys = 32, kWarpRows = 4, kThreads = 256;
-
 template <typename T, int DH>
-__global__ void __launch_bounds__(256) bwd_delta_kernel(const T* __restrict__ O, const T* __restrict__ dO,
-                                                        long long rows, float* __restrict__ delta) {
-    const int lane = threadIdx.x & 31;
-    const long long row = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (row >= rows) return;
-    float s = 0.f;
-    for (int c = lane; c < DH; c += 32) s = fmaf(Elem<T>::ld(O + row * DH + c), Elem<T>::ld(dO + row * DH + c), s);
-    s = warp_sum(s);
-    if (lane == 0) delta[row] = s;
-}
-
-template <typename T, int DH>
-__global__ void __launch_bounds__(kThreads) bwd_dq_kernel(const BwdParams p) {
-    constexpr int CPL = (DH + 31) / 32, LD = DH + 1;
-    extern __shared__ float smem[];
-    float* qs = smem;                 // [kRows][DH]  tau * q
-    float* gs = qs + kRows * DH;      // [kRows][DH]  dO
-    float* ks = gs + kRows * DH;      // [kKeys][LD]
-    float* vs = ks + kKeys * LD;      // [kKeys][LD]
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__global__ void __launch_bounds__(kSimtThreads) bwd_dq_kernel(const BwdParams p, const int vec) {
+    constexpr int CPL = DH / 32, LD = DH + 4, kTileFloats = kSimtTile * LD, R = kSimtWarpRows;
+    extern __shared__ __align__(16) float smem[];
+    float* qs = smem;                            // [16][DH]  tau * q
+    float* gs = qs + kSimtRows * DH;             // [16][DH]  dO
+    float* ps = gs + kSimtRows * DH;             // [16 warps][4 rows][32]  dS of the warp's tile
+    float* tiles = ps + 16 * R * 32;             // [4 groups][K, V][32][LD]; at the end [4 groups][16 rows][DH + 6]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp >> 2, wg = warp & 3, gtid = threadIdx.x & 127;
     const int b = blockIdx.z, h = blockIdx.y;
-    const long long t0 = (long long)blockIdx.x * kRows;
+    const long long t0 = (long long)blockIdx.x * kSimtRows;
     const long long bh = (long long)b * p.H + h;
     const T* Q = static_cast<const T*>(p.Q) + bh * p.T * DH;
     const T* dO = static_cast<const T*>(p.dO) + bh * p.T * DH;
-    for (int i = threadIdx.x; i < kRows * DH; i += kThreads) {
-        long long t = t0 + i / DH;
-        qs[i] = t < p.T ? Elem<T>::ld(Q + t * DH + (i % DH)) * p.scale : 0.f;
-        gs[i] = t < p.T ? Elem<T>::ld(dO + t * DH + (i % DH)) : 0.f;
+    for (int i = threadIdx.x * 4; i < kSimtRows * DH; i += kSimtThreads * 4) {
+        const long long t = t0 + i / DH;
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
+        if (t < p.T) {
+            x = Fetch4<T>::at(Q + t * DH + i % DH, (vec & 8) != 0);
+            y = Fetch4<T>::at(dO + t * DH + i % DH, (vec & 8) != 0);
+        }
+        qs[i] = x.x * p.scale; qs[i + 1] = x.y * p.scale; qs[i + 2] = x.z * p.scale; qs[i + 3] = x.w * p.scale;
+        *reinterpret_cast<float4*>(gs + i) = y;
     }
-    float lse[kWarpRows], dlt[kWarpRows], acc[kWarpRows][CPL];
-    float Ap[kWarpRows][3], Sp[kWarpRows][3];   // per level: sum_j p dP and sum_j p (for the gate gradient)
+    __syncthreads();
+    float lse[R], dlt[R], acc[R][CPL];
+    float Ap[R][3], Sp[R][3];                    // per level, this lane's keys: sum_j p dP and sum_j p (for the gate gradient)
 #pragma unroll
-    for (int r = 0; r < kWarpRows; ++r) {
-        long long t = t0 + warp * kWarpRows + r;
-        long long tc = t < p.T ? t : p.T - 1;
+    for (int r = 0; r < R; ++r) {
+        const long long t = t0 + wg * R + r, tc = t < p.T ? t : p.T - 1;
         lse[r] = p.LSE[bh * p.T + tc];
-        dlt[r] = p.delta[bh * p.T + tc];
+        // D_t = dO_t . O_t, left for the dK/dV kernel too
+        float d = 0.f;
+#pragma unroll
+        for (int k = 0; k < CPL; ++k)
+            d = fmaf(Elem<T>::ld(static_cast<const T*>(p.O) + (bh * p.T + tc) * DH + lane + 32 * k), gs[(wg * R + r) * DH + lane + 32 * k], d);
+        dlt[r] = warp_sum(d);
+        if (group == 0 && lane == 0 && t < p.T) p.delta[bh * p.T + t] = dlt[r];
 #pragma unroll
         for (int k = 0; k < CPL; ++k) acc[r][k] = 0.f;
         Ap[r][0] = Ap[r][1] = Ap[r][2] = 0.f;
         Sp[r][0] = Sp[r][1] = Sp[r][2] = 0.f;
     }
-    const long long t_last = (t0 + kRows - 1 < p.T ? t0 + kRows - 1 : p.T - 1);
+    float* ks = tiles + group * 2 * kTileFloats;
+    float* vs = ks + kTileFloats;
+    float* pw = ps + warp * R * 32;
+    const float* qw = qs + wg * R * DH;
+    const float* gw = gs + wg * R * DH;
+    const long long t_last = (t0 + kSimtRows - 1 < p.T ? t0 + kSimtRows - 1 : p.T - 1);
 #pragma unroll
     for (int lvl = 0; lvl < 3; ++lvl) {
         const LevelDev L = p.L[lvl];
@@ -68,213 +69,237 @@ __global__ void __launch_bounds__(kThreads) bwd_dq_kernel(const BwdParams p) {
         const long long lo = lo_f, hi = hi_l > hi_f ? hi_l : hi_f;
         const T* Kp = static_cast<const T*>(L.k) + b * L.sb + (h / p.kv_group) * L.sh;
         const T* Vp = static_cast<const T*>(L.v) + b * L.sb + (h / p.kv_group) * L.sh;
-        float lam[kWarpRows];
-        long long rlo[kWarpRows], rhi[kWarpRows];
+        float lam[R];
+        long long rlo[R], rhi[R];
 #pragma unroll
-        for (int r = 0; r < kWarpRows; ++r) {
-            long long t = t0 + warp * kWarpRows + r;
-            long long tc = t < p.T ? t : p.T - 1;
+        for (int r = 0; r < R; ++r) {
+            const long long t = t0 + wg * R + r, tc = t < p.T ? t : p.T - 1;
             lam[r] = p.gate[((long long)b * p.T + tc) * 3 + lvl];
             visible_range(lvl, tc + p.q_offset, p.window, L.n, 0, rlo[r], rhi[r]);
             if (t >= p.T) rhi[r] = rlo[r];
         }
-        for (long long j0 = (lo / kKeys) * kKeys; j0 < hi; j0 += kKeys) {
-            __syncthreads();
-            for (int i = threadIdx.x; i < kKeys * DH; i += kThreads) {
-                int jr = i / DH, c = i % DH;
-                long long j = j0 + jr;
-                float kv = 0.f, vv = 0.f;
-                if (j < L.n) { kv = Elem<T>::ld(Kp + j * L.sn + c); vv = Elem<T>::ld(Vp + j * L.sn + c); }
-                ks[jr * LD + c] = kv;
-                vs[jr * LD + c] = vv;
-            }
-            __syncthreads();
-            float s[kWarpRows], dp[kWarpRows];
+        for (long long j0 = (lo / kSimtTile + group) * kSimtTile; j0 < hi; j0 += kSimtGroups * kSimtTile) {
+            group_sync(group);
+            load_pair<T, DH>(ks, vs, Kp, Vp, j0, L.n, L.sn, (vec >> lvl) & 1, gtid);
+            group_sync(group);
+            float s[R], dp[R];
 #pragma unroll
-            for (int r = 0; r < kWarpRows; ++r) s[r] = dp[r] = 0.f;
+            for (int r = 0; r < R; ++r) s[r] = dp[r] = 0.f;
             const float* kr = ks + lane * LD;
             const float* vr = vs + lane * LD;
-            const float* qw = qs + warp * kWarpRows * DH;
-            const float* gw = gs + warp * kWarpRows * DH;
-#pragma unroll 4
-            for (int c = 0; c < DH; ++c) {
-                float kv = kr[c], vv = vr[c];
+#pragma unroll 2
+            for (int c = 0; c < DH; c += 4) {
+                const float4 kv = *reinterpret_cast<const float4*>(kr + c), vv = *reinterpret_cast<const float4*>(vr + c);
 #pragma unroll
-                for (int r = 0; r < kWarpRows; ++r) {
-                    s[r] = fmaf(qw[r * DH + c], kv, s[r]);
-                    dp[r] = fmaf(gw[r * DH + c], vv, dp[r]);
+                for (int r = 0; r < R; ++r) {
+                    const float4 q = *reinterpret_cast<const float4*>(qw + r * DH + c), g = *reinterpret_cast<const float4*>(gw + r * DH + c);
+                    s[r] = fmaf(q.x, kv.x, s[r]); s[r] = fmaf(q.y, kv.y, s[r]); s[r] = fmaf(q.z, kv.z, s[r]); s[r] = fmaf(q.w, kv.w, s[r]);
+                    dp[r] = fmaf(g.x, vv.x, dp[r]); dp[r] = fmaf(g.y, vv.y, dp[r]); dp[r] = fmaf(g.z, vv.z, dp[r]); dp[r] = fmaf(g.w, vv.w, dp[r]);
                 }
             }
             const long long j = j0 + lane;
-            float ds[kWarpRows];
 #pragma unroll
-            for (int r = 0; r < kWarpRows; ++r) {
+            for (int r = 0; r < R; ++r) {
                 const bool vis = (j >= rlo[r]) && (j < rhi[r]) && lam[r] > 0.f;
                 const float pr = vis ? lam[r] * expf(s[r] - lse[r]) : 0.f;
-                ds[r] = pr * (dp[r] - dlt[r]);
+                pw[r * 32 + lane] = pr * (dp[r] - dlt[r]);
                 Ap[r][lvl] = fmaf(pr, dp[r], Ap[r][lvl]);
                 Sp[r][lvl] += pr;
             }
-#pragma unroll 4
-            for (int jj = 0; jj < kKeys; ++jj) {
-                float dj[kWarpRows];
+            __syncwarp();
+#pragma unroll 2
+            for (int jj = 0; jj < kSimtTile; jj += 4) {
+                float4 e[R];
 #pragma unroll
-                for (int r = 0; r < kWarpRows; ++r) dj[r] = __shfl_sync(0xffffffffu, ds[r], jj);
+                for (int r = 0; r < R; ++r) e[r] = *reinterpret_cast<const float4*>(pw + r * 32 + jj);
 #pragma unroll
                 for (int k = 0; k < CPL; ++k) {
-                    int c = lane + 32 * k;
-                    float kv = c < DH ? ks[jj * LD + c] : 0.f;
+                    const float* v = ks + jj * LD + lane + 32 * k;
+                    const float v0 = v[0], v1 = v[LD], v2 = v[2 * LD], v3 = v[3 * LD];
 #pragma unroll
-                    for (int r = 0; r < kWarpRows; ++r) acc[r][k] = fmaf(dj[r], kv, acc[r][k]);
+                    for (int r = 0; r < R; ++r) {
+                        acc[r][k] = fmaf(e[r].x, v0, acc[r][k]); acc[r][k] = fmaf(e[r].y, v1, acc[r][k]);
+                        acc[r][k] = fmaf(e[r].z, v2, acc[r][k]); acc[r][k] = fmaf(e[r].w, v3, acc[r][k]);
+                    }
                 }
             }
+            __syncwarp();
         }
     }
+    // merge the groups: warp w adds up row w
+    __syncthreads();
+    constexpr int kState = DH + 6;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        float* o = tiles + (group * kSimtRows + wg * R + r) * kState;
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+            const float a = warp_sum(Ap[r][l]), sp = warp_sum(Sp[r][l]);
+            if (lane == 0) { o[l] = a; o[3 + l] = sp; }
+        }
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) o[6 + lane + 32 * k] = acc[r][k];
+    }
+    __syncthreads();
+    const long long t = t0 + warp;
+    if (t >= p.T) return;
+    const float* o = tiles + warp * kState;
+    auto total = [&](int i) {
+        float v = o[i];
+#pragma unroll
+        for (int g = 1; g < kSimtGroups; ++g) v += o[g * kSimtRows * kState + i];
+        return v;
+    };
     T* dQ = static_cast<T*>(p.dQ) + bh * p.T * DH;
 #pragma unroll
-    for (int r = 0; r < kWarpRows; ++r) {
-        long long t = t0 + warp * kWarpRows + r;
-        if (t >= p.T) continue;
+    for (int k = 0; k < CPL; ++k) Elem<T>::st(dQ + t * DH + lane + 32 * k, total(6 + lane + 32 * k) * p.scale);
+    // Gate-logit gradient G_l = sum_{j in l} p (dP - D).  Here D is taken as sum_{l,j} p dP / sum p, which
+    // equals dO.O exactly in real arithmetic but does not inherit the rounding of O to its storage
+    // type, so that sum_l G_l = 0 holds to fp32 accuracy.
+    float a[3], sp[3];
 #pragma unroll
-        for (int k = 0; k < CPL; ++k) {
-            int c = lane + 32 * k;
-            if (c < DH) Elem<T>::st(dQ + t * DH + c, acc[r][k] * p.scale);
-        }
-        // Gate-logit gradient G_l = sum_{j in l} p (dP - D).  Here D is taken as sum_{l,j} p dP / sum p, which
-        // equals dO.O exactly in real arithmetic but does not inherit the rounding of O to its storage
-        // type, so that sum_l G_l = 0 holds to fp32 accuracy.
-        float a[3], sp[3];
+    for (int l = 0; l < 3; ++l) { a[l] = total(l); sp[l] = total(3 + l); }
+    const float stot = sp[0] + sp[1] + sp[2];
+    const float dd = stot > 0.f ? (a[0] + a[1] + a[2]) / stot : 0.f;
 #pragma unroll
-        for (int l = 0; l < 3; ++l) { a[l] = warp_sum(Ap[r][l]); sp[l] = warp_sum(Sp[r][l]); }
-        const float stot = sp[0] + sp[1] + sp[2];
-        const float dd = stot > 0.f ? (a[0] + a[1] + a[2]) / stot : 0.f;
-#pragma unroll
-        for (int l = 0; l < 3; ++l)
-            if (lane == 0) p.Gpart[(bh * p.T + t) * 3 + l] = a[l] - sp[l] * dd;
-    }
+    for (int l = 0; l < 3; ++l)
+        if (lane == 0) p.Gpart[(bh * p.T + t) * 3 + l] = a[l] - sp[l] * dd;
 }
 
-// One CTA = 32 key rows of one level of one (batch, head); loops over the query tiles that see them.
+// One CTA = 16 key rows of one level of one (batch, KV head); its groups share the query tiles that see them.  One launch
+// covers the three levels: blockIdx.x runs through L1's, L2's and L3's key tiles.
 template <typename T, int DH>
-__global__ void __launch_bounds__(kThreads) bwd_dkv_kernel(const BwdParams p, const int lvl) {
-    constexpr int CPL = (DH + 31) / 32, LD = DH + 1;
-    extern __shared__ float smem[];
-    float* ksm = smem;                // [kKeys][DH]  tau * k   (this CTA's key rows)
-    float* vsm = ksm + kKeys * DH;    // [kKeys][DH]
-    float* qs = vsm + kKeys * DH;     // [kRows][LD]  query tile
-    float* gs = qs + kRows * LD;      // [kRows][LD]  dO tile
-    __shared__ float s_lse[kRows], s_dlt[kRows], s_lam[kRows];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__global__ void __launch_bounds__(kSimtThreads) bwd_dkv_kernel(const BwdParams p, const int vec) {
+    constexpr int CPL = DH / 32, LD = DH + 4, kTileFloats = kSimtTile * LD, R = kSimtWarpRows;
+    extern __shared__ __align__(16) float smem[];
+    float* ksm = smem;                           // [16][DH]  tau * k   (this CTA's key rows)
+    float* vsm = ksm + kSimtRows * DH;           // [16][DH]
+    float* ps = vsm + kSimtRows * DH;            // [16 warps][p, dS][4 rows][32]
+    float* tiles = ps + 16 * 2 * R * 32;         // [4 groups][Q, dO][32][LD]; at the end [4 groups][16 rows][2 DH]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp >> 2, wg = warp & 3, gtid = threadIdx.x & 127;
     const int b = blockIdx.z, h = blockIdx.y;               // h: KV head; its query heads h * G .. h * G + G - 1 are summed
+    int lvl = 0;
+    long long kt = blockIdx.x;
+    while (kt >= (p.L[lvl].n + kSimtRows - 1) / kSimtRows) { kt -= (p.L[lvl].n + kSimtRows - 1) / kSimtRows; ++lvl; }
     const LevelDev L = p.L[lvl];
     const LevelGradDev dL = p.dL[lvl];
-    const long long j0 = (long long)blockIdx.x * kKeys;
+    const long long j0 = kt * kSimtRows;
     const T* Kp = static_cast<const T*>(L.k) + b * L.sb + h * L.sh;
     const T* Vp = static_cast<const T*>(L.v) + b * L.sb + h * L.sh;
-    for (int i = threadIdx.x; i < kKeys * DH; i += kThreads) {
-        long long j = j0 + i / DH;
-        ksm[i] = j < L.n ? Elem<T>::ld(Kp + j * L.sn + (i % DH)) * p.scale : 0.f;
-        vsm[i] = j < L.n ? Elem<T>::ld(Vp + j * L.sn + (i % DH)) : 0.f;
+    for (int i = threadIdx.x * 4; i < kSimtRows * DH; i += kSimtThreads * 4) {
+        const long long j = j0 + i / DH;
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
+        if (j < L.n) {
+            x = Fetch4<T>::at(Kp + j * L.sn + i % DH, (vec >> lvl) & 1);
+            y = Fetch4<T>::at(Vp + j * L.sn + i % DH, (vec >> lvl) & 1);
+        }
+        ksm[i] = x.x * p.scale; ksm[i + 1] = x.y * p.scale; ksm[i + 2] = x.z * p.scale; ksm[i + 3] = x.w * p.scale;
+        *reinterpret_cast<float4*>(vsm + i) = y;
     }
-    float accK[kWarpRows][CPL], accV[kWarpRows][CPL];
+    __syncthreads();
+    float accK[R][CPL], accV[R][CPL];
 #pragma unroll
-    for (int r = 0; r < kWarpRows; ++r)
+    for (int r = 0; r < R; ++r)
 #pragma unroll
         for (int k = 0; k < CPL; ++k) accK[r][k] = accV[r][k] = 0.f;
     // queries that can see any of this CTA's keys: positions p = t + q_offset with
     //   L1: j <= p <= j + W - 1   L2: p >= j   L3: all
-    const long long j_last = (j0 + kKeys - 1 < L.n ? j0 + kKeys - 1 : L.n - 1);
+    const long long j_last = (j0 + kSimtRows - 1 < L.n ? j0 + kSimtRows - 1 : L.n - 1);
     long long t_lo = 0, t_hi = p.T;
     if (lvl == 0) { t_lo = j0 - p.q_offset; t_hi = j_last + p.window - p.q_offset; }
     else if (lvl == 1) { t_lo = j0 - p.q_offset; }
     if (t_lo < 0) t_lo = 0;
     if (t_hi > p.T) t_hi = p.T;
-    for (int gq = 0; gq < p.kv_group; ++gq) {
-    const long long bh = (long long)b * p.H + (long long)h * p.kv_group + gq;
-    const T* Q = static_cast<const T*>(p.Q) + bh * p.T * DH;
-    const T* dO = static_cast<const T*>(p.dO) + bh * p.T * DH;
-    for (long long tt = (t_lo / kRows) * kRows; tt < t_hi; tt += kRows) {
-        __syncthreads();
-        for (int i = threadIdx.x; i < kRows * DH; i += kThreads) {
-            int r = i / DH, c = i % DH;
-            long long t = tt + r;
-            qs[r * LD + c] = t < p.T ? Elem<T>::ld(Q + t * DH + c) : 0.f;
-            gs[r * LD + c] = t < p.T ? Elem<T>::ld(dO + t * DH + c) : 0.f;
-        }
-        if (threadIdx.x < kRows) {
-            long long t = tt + threadIdx.x;
-            bool ok = t < p.T;
-            s_lse[threadIdx.x] = ok ? p.LSE[bh * p.T + t] : 0.f;
-            s_dlt[threadIdx.x] = ok ? p.delta[bh * p.T + t] : 0.f;
-            s_lam[threadIdx.x] = ok ? p.gate[((long long)b * p.T + t) * 3 + lvl] : 0.f;
-        }
-        __syncthreads();
-        // lane = query of the tile; warp rows = keys
-        const long long t = tt + lane;
+    const long long first = t_lo / kSimtTile, per_head = t_hi > t_lo ? (t_hi + kSimtTile - 1) / kSimtTile - first : 0;
+    float* qs = tiles + group * 2 * kTileFloats;
+    float* gs = qs + kTileFloats;
+    float* pw = ps + warp * 2 * R * 32;
+    const float* kw = ksm + wg * R * DH;
+    const float* vw = vsm + wg * R * DH;
+    for (long long i = group; i < per_head * p.kv_group; i += kSimtGroups) {     // head by head, each head's tiles in order
+        const long long bh = (long long)b * p.H + (long long)h * p.kv_group + i / per_head;
+        const long long tt = (first + i % per_head) * kSimtTile, t = tt + lane;   // lane = query of the tile; warp rows = keys
+        const T* Q = static_cast<const T*>(p.Q) + bh * p.T * DH;
+        const T* dO = static_cast<const T*>(p.dO) + bh * p.T * DH;
+        const long long tc = t < p.T ? t : p.T - 1;
+        const float lse = p.LSE[bh * p.T + tc], dlt = p.delta[bh * p.T + tc], lam = p.gate[((long long)b * p.T + tc) * 3 + lvl];
+        group_sync(group);
+        load_pair<T, DH>(qs, gs, Q, dO, tt, p.T, DH, (vec & 8) != 0, gtid);
+        group_sync(group);
         long long vlo, vhi;
         visible_range(lvl, t + p.q_offset, p.window, L.n, 0, vlo, vhi);
         if (t >= p.T) vhi = vlo;
-        const float lam = s_lam[lane], lse = s_lse[lane], dlt = s_dlt[lane];
-        float s[kWarpRows], dp[kWarpRows];
+        float s[R], dp[R];
 #pragma unroll
-        for (int r = 0; r < kWarpRows; ++r) s[r] = dp[r] = 0.f;
+        for (int r = 0; r < R; ++r) s[r] = dp[r] = 0.f;
         const float* qr = qs + lane * LD;
         const float* gr = gs + lane * LD;
-        const float* kw = ksm + warp * kWarpRows * DH;
-        const float* vw = vsm + warp * kWarpRows * DH;
-#pragma unroll 4
-        for (int c = 0; c < DH; ++c) {
-            float qv = qr[c], gv = gr[c];
+#pragma unroll 2
+        for (int c = 0; c < DH; c += 4) {
+            const float4 qv = *reinterpret_cast<const float4*>(qr + c), gv = *reinterpret_cast<const float4*>(gr + c);
 #pragma unroll
-            for (int r = 0; r < kWarpRows; ++r) {
-                s[r] = fmaf(kw[r * DH + c], qv, s[r]);
-                dp[r] = fmaf(vw[r * DH + c], gv, dp[r]);
+            for (int r = 0; r < R; ++r) {
+                const float4 k = *reinterpret_cast<const float4*>(kw + r * DH + c), v = *reinterpret_cast<const float4*>(vw + r * DH + c);
+                s[r] = fmaf(k.x, qv.x, s[r]); s[r] = fmaf(k.y, qv.y, s[r]); s[r] = fmaf(k.z, qv.z, s[r]); s[r] = fmaf(k.w, qv.w, s[r]);
+                dp[r] = fmaf(v.x, gv.x, dp[r]); dp[r] = fmaf(v.y, gv.y, dp[r]); dp[r] = fmaf(v.z, gv.z, dp[r]); dp[r] = fmaf(v.w, gv.w, dp[r]);
             }
         }
-        float pr[kWarpRows], ds[kWarpRows];
 #pragma unroll
-        for (int r = 0; r < kWarpRows; ++r) {
-            const long long j = j0 + warp * kWarpRows + r;
+        for (int r = 0; r < R; ++r) {
+            const long long j = j0 + wg * R + r;
             const bool vis = (j >= vlo) && (j < vhi) && lam > 0.f;
-            pr[r] = vis ? lam * expf(s[r] - lse) : 0.f;
-            ds[r] = pr[r] * (dp[r] - dlt);
+            const float pr = vis ? lam * expf(s[r] - lse) : 0.f;
+            pw[r * 32 + lane] = pr;
+            pw[(R + r) * 32 + lane] = pr * (dp[r] - dlt);
         }
-#pragma unroll 4
-        for (int q = 0; q < kRows; ++q) {
-            float pj[kWarpRows], dj[kWarpRows];
+        __syncwarp();
+#pragma unroll 2
+        for (int q = 0; q < kSimtTile; q += 4) {
+            float4 pj[R], dj[R];
 #pragma unroll
-            for (int r = 0; r < kWarpRows; ++r) {
-                pj[r] = __shfl_sync(0xffffffffu, pr[r], q);
-                dj[r] = __shfl_sync(0xffffffffu, ds[r], q);
+            for (int r = 0; r < R; ++r) {
+                pj[r] = *reinterpret_cast<const float4*>(pw + r * 32 + q);
+                dj[r] = *reinterpret_cast<const float4*>(pw + (R + r) * 32 + q);
             }
 #pragma unroll
             for (int k = 0; k < CPL; ++k) {
-                int c = lane + 32 * k;
-                float qv = c < DH ? qs[q * LD + c] : 0.f;
-                float gv = c < DH ? gs[q * LD + c] : 0.f;
+                const float* qc = qs + q * LD + lane + 32 * k;
+                const float* gc = gs + q * LD + lane + 32 * k;
+                const float q0 = qc[0], q1 = qc[LD], q2 = qc[2 * LD], q3 = qc[3 * LD];
+                const float g0 = gc[0], g1 = gc[LD], g2 = gc[2 * LD], g3 = gc[3 * LD];
 #pragma unroll
-                for (int r = 0; r < kWarpRows; ++r) {
-                    accK[r][k] = fmaf(dj[r], qv, accK[r][k]);
-                    accV[r][k] = fmaf(pj[r], gv, accV[r][k]);
+                for (int r = 0; r < R; ++r) {
+                    accK[r][k] = fmaf(dj[r].x, q0, accK[r][k]); accK[r][k] = fmaf(dj[r].y, q1, accK[r][k]);
+                    accK[r][k] = fmaf(dj[r].z, q2, accK[r][k]); accK[r][k] = fmaf(dj[r].w, q3, accK[r][k]);
+                    accV[r][k] = fmaf(pj[r].x, g0, accV[r][k]); accV[r][k] = fmaf(pj[r].y, g1, accV[r][k]);
+                    accV[r][k] = fmaf(pj[r].z, g2, accV[r][k]); accV[r][k] = fmaf(pj[r].w, g3, accV[r][k]);
                 }
             }
         }
+        __syncwarp();
     }
-    }   // query heads of the group
-    T* dKp = static_cast<T*>(dL.dk) + b * dL.sb + h * dL.sh;
-    T* dVp = static_cast<T*>(dL.dv) + b * dL.sb + h * dL.sh;
+    // merge the groups: warp w adds up key row w
+    __syncthreads();
 #pragma unroll
-    for (int r = 0; r < kWarpRows; ++r) {
-        long long j = j0 + warp * kWarpRows + r;
-        if (j >= L.n) continue;
+    for (int r = 0; r < R; ++r) {
+        float* o = tiles + (group * kSimtRows + wg * R + r) * 2 * DH;
 #pragma unroll
-        for (int k = 0; k < CPL; ++k) {
-            int c = lane + 32 * k;
-            if (c < DH) {
-                Elem<T>::st(dKp + j * dL.sn + c, accK[r][k] * p.scale);
-                Elem<T>::st(dVp + j * dL.sn + c, accV[r][k]);
-            }
-        }
+        for (int k = 0; k < CPL; ++k) { o[lane + 32 * k] = accK[r][k]; o[DH + lane + 32 * k] = accV[r][k]; }
+    }
+    __syncthreads();
+    const long long j = j0 + warp;
+    if (j >= L.n) return;
+    const float* o = tiles + warp * 2 * DH;
+    T* dKp = static_cast<T*>(dL.dk) + b * dL.sb + h * dL.sh + j * dL.sn;
+    T* dVp = static_cast<T*>(dL.dv) + b * dL.sb + h * dL.sh + j * dL.sn;
+#pragma unroll
+    for (int k = 0; k < CPL; ++k) {
+        const int c = lane + 32 * k;
+        float dk = o[c], dv = o[DH + c];
+#pragma unroll
+        for (int g = 1; g < kSimtGroups; ++g) { dk += o[g * kSimtRows * 2 * DH + c]; dv += o[g * kSimtRows * 2 * DH + DH + c]; }
+        Elem<T>::st(dKp + c, dk * p.scale);
+        Elem<T>::st(dVp + c, dv);
     }
 }
 
@@ -300,28 +325,24 @@ namespace {
 
 template <typename T, int DH>
 cudaError_t launch_t(const BwdParams& p, cudaStream_t st) {
-    const long long rows = (long long)p.B * p.H * p.T;
+    const int vec = simt_vec_bits(p.L, p.Q, p.O, p.dO, sizeof(T) == 2 ? MKA_BF16 : MKA_F32);
+    const size_t tiles_floats = (size_t)kSimtGroups * 2 * kSimtTile * (DH + 4);
     cudaError_t e;
-    bwd_delta_kernel<T, DH><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(static_cast<const T*>(p.O), static_cast<const T*>(p.dO), rows, p.delta);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     {
-        size_t smem = sizeof(float) * (2 * kRows * DH + 2 * kKeys * (DH + 1));
+        const size_t smem = sizeof(float) * (2 * kSimtRows * DH + 16 * kSimtWarpRows * 32 + tiles_floats);
         e = cudaFuncSetAttribute(bwd_dq_kernel<T, DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        dim3 grid((p.T + kRows - 1) / kRows, p.H, p.B);
-        bwd_dq_kernel<T, DH><<<grid, kThreads, smem, st>>>(p);
+        bwd_dq_kernel<T, DH><<<dim3((p.T + kSimtRows - 1) / kSimtRows, p.H, p.B), kSimtThreads, smem, st>>>(p, vec);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    {
-        size_t smem = sizeof(float) * (2 * kKeys * DH + 2 * kRows * (DH + 1));
+    long long key_tiles = 0;
+    for (int l = 0; l < 3; ++l) key_tiles += (p.L[l].n + kSimtRows - 1) / kSimtRows;
+    if (key_tiles > 0) {
+        const size_t smem = sizeof(float) * (2 * kSimtRows * DH + 16 * 2 * kSimtWarpRows * 32 + tiles_floats);
         e = cudaFuncSetAttribute(bwd_dkv_kernel<T, DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        for (int lvl = 0; lvl < 3; ++lvl) {
-            if (p.L[lvl].n == 0) continue;
-            dim3 grid((unsigned)((p.L[lvl].n + kKeys - 1) / kKeys), p.H / (p.kv_group > 0 ? p.kv_group : 1), p.B);
-            bwd_dkv_kernel<T, DH><<<grid, kThreads, smem, st>>>(p, lvl);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        }
+        bwd_dkv_kernel<T, DH><<<dim3((unsigned)key_tiles, p.H / (p.kv_group > 0 ? p.kv_group : 1), p.B), kSimtThreads, smem, st>>>(p, vec);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return launch_bwd_dgate(p.Gpart, p.B, p.H, p.T, p.dG, st);
 }

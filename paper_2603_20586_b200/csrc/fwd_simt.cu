@@ -4,51 +4,52 @@
 //                  32 rows as in Alg. 3, rescale of Eq. 13-14 applied on every block).
 //   MKA_MODE_FULL: Alg. 1 -- one softmax state per level, outputs mixed by the gate at the end.
 // fp32 arithmetic throughout, so this is the kernel for fp32 problems (tolerance 1e-4) and the
-// on-GPU cross-check of the tensor-core kernel.  One CTA = 32 query rows of one (batch, head); each of
-// its 8 warps owns 4 rows; a key tile of 32 rows is staged in shared memory as fp32 and each lane
-// scores one key of the tile.
-#include "common.cuh"
+// on-GPU cross-check of the tensor-core kernel.  One CTA = 16 query rows of one (batch, head), see simt.cuh; a key tile of
+// 32 rows is staged in shared memory as fp32 and each lane scores one key of the tile, four columns at a time.
+#include "simt.cuh"
 
 namespace mka {
 namespace {
 
-constexpr int kRows = 32;        // query rows per CTA
-constexpr int kKeys = 32;        // key rows per shared-memory tile
-constexpr int kWarpRows = 4;
-constexpr int kThreads = 256;
-
 template <typename T, int DH, int MODE>
-__global__ void __launch_bounds__(kThreads) fwd_simt_kernel(const FwdParams p) {
+__global__ void __launch_bounds__(kSimtThreads) fwd_simt_kernel(const FwdParams p, const int vec) {
     constexpr int NS = MODE == MKA_MODE_FULL ? 3 : 1;    // softmax states
-    constexpr int CPL = (DH + 31) / 32;                  // output columns per lane
-    constexpr int LD = DH + 1;                           // padded row pitch (floats)
-    extern __shared__ float smem[];
-    float* qs = smem;                    // [kRows][DH]
-    float* ks = qs + kRows * DH;         // [kKeys][LD]
-    float* vs = ks + kKeys * LD;         // [kKeys][LD]
+    constexpr int CPL = DH / 32;                         // output columns per lane
+    constexpr int LD = DH + 4, kTileFloats = kSimtTile * LD, R = kSimtWarpRows;
+    extern __shared__ __align__(16) float smem[];
+    float* qs = smem;                                    // [16][DH]  tau * q
+    float* ps = qs + kSimtRows * DH;                     // [16 warps][4 rows][32]  weights of the warp's tile
+    float* tiles = ps + 16 * R * 32;                     // [4 groups][K, V][32][LD]; at the end [4 groups][16 rows][NS][DH + 2]
 
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp >> 2, wg = warp & 3, gtid = threadIdx.x & 127;
     const int b = blockIdx.z, h = blockIdx.y;
-    const long long t0 = (long long)blockIdx.x * kRows;
+    const long long t0 = (long long)blockIdx.x * kSimtRows;
     const T* Q = static_cast<const T*>(p.Q) + (((long long)b * p.H + h) * p.T) * DH;
     T* O = static_cast<T*>(p.O) + (((long long)b * p.H + h) * p.T) * DH;
 
-    for (int i = threadIdx.x; i < kRows * DH; i += kThreads) {
-        long long t = t0 + i / DH;
-        qs[i] = t < p.T ? Elem<T>::ld(Q + t * DH + (i % DH)) * p.scale : 0.f;   // tau folded into q
+    for (int i = threadIdx.x * 4; i < kSimtRows * DH; i += kSimtThreads * 4) {
+        const long long t = t0 + i / DH;
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (t < p.T) x = Fetch4<T>::at(Q + t * DH + i % DH, (vec & 8) != 0);
+        qs[i] = x.x * p.scale; qs[i + 1] = x.y * p.scale; qs[i + 2] = x.z * p.scale; qs[i + 3] = x.w * p.scale;   // tau folded into q
     }
+    __syncthreads();
 
-    float m[NS][kWarpRows], z[NS][kWarpRows], acc[NS][kWarpRows][CPL];
+    float m[NS][R], z[NS][R], acc[NS][R][CPL];           // z: this lane's keys only
 #pragma unroll
     for (int s = 0; s < NS; ++s)
 #pragma unroll
-        for (int r = 0; r < kWarpRows; ++r) {
+        for (int r = 0; r < R; ++r) {
             m[s][r] = -INFINITY; z[s][r] = 0.f;
 #pragma unroll
             for (int k = 0; k < CPL; ++k) acc[s][r][k] = 0.f;
         }
 
-    const long long t_last = (t0 + kRows - 1 < p.T ? t0 + kRows - 1 : p.T - 1);
+    float* ks = tiles + group * 2 * kTileFloats;
+    float* vs = ks + kTileFloats;
+    float* pw = ps + warp * R * 32;
+    const float* qw = qs + wg * R * DH;
+    const long long t_last = (t0 + kSimtRows - 1 < p.T ? t0 + kSimtRows - 1 : p.T - 1);
 #pragma unroll
     for (int lvl = 0; lvl < 3; ++lvl) {
         const int st = MODE == MKA_MODE_FULL ? lvl : 0;
@@ -61,115 +62,126 @@ __global__ void __launch_bounds__(kThreads) fwd_simt_kernel(const FwdParams p) {
         const long long lo = lo_first, hi = hi_last > hi_first ? hi_last : hi_first;
         const T* Kp = static_cast<const T*>(L.k) + b * L.sb + (h / p.kv_group) * L.sh;
         const T* Vp = static_cast<const T*>(L.v) + b * L.sb + (h / p.kv_group) * L.sh;
-        float lam[kWarpRows];
-        long long rlo[kWarpRows], rhi[kWarpRows];
+        float lam[R];
+        long long rlo[R], rhi[R];
 #pragma unroll
-        for (int r = 0; r < kWarpRows; ++r) {
-            long long t = t0 + warp * kWarpRows + r;
-            long long tc = t < p.T ? t : p.T - 1;
+        for (int r = 0; r < R; ++r) {
+            const long long t = t0 + wg * R + r, tc = t < p.T ? t : p.T - 1;
             lam[r] = p.gate[((long long)b * p.T + tc) * 3 + lvl];
             visible_range(lvl, tc + p.q_offset, p.window, L.n, p.decode, rlo[r], rhi[r]);
             if (t >= p.T) rhi[r] = rlo[r];
         }
-        for (long long j0 = (lo / kKeys) * kKeys; j0 < hi; j0 += kKeys) {
-            __syncthreads();
-            for (int i = threadIdx.x; i < kKeys * DH; i += kThreads) {
-                int jr = i / DH, c = i % DH;
-                long long j = j0 + jr;
-                float kv = 0.f, vv = 0.f;
-                if (j < L.n) { kv = Elem<T>::ld(Kp + j * L.sn + c); vv = Elem<T>::ld(Vp + j * L.sn + c); }
-                ks[jr * LD + c] = kv;
-                vs[jr * LD + c] = vv;
-            }
-            __syncthreads();
-            float s[kWarpRows];
+        for (long long j0 = (lo / kSimtTile + group) * kSimtTile; j0 < hi; j0 += kSimtGroups * kSimtTile) {
+            group_sync(group);                           // the group's previous tile has been read
+            load_pair<T, DH>(ks, vs, Kp, Vp, j0, L.n, L.sn, (vec >> lvl) & 1, gtid);
+            group_sync(group);
+            float s[R];
 #pragma unroll
-            for (int r = 0; r < kWarpRows; ++r) s[r] = 0.f;
+            for (int r = 0; r < R; ++r) s[r] = 0.f;
             const float* kr = ks + lane * LD;
-            const float* qw = qs + warp * kWarpRows * DH;
-#pragma unroll 8
-            for (int c = 0; c < DH; ++c) {
-                float kv = kr[c];
+#pragma unroll 4
+            for (int c = 0; c < DH; c += 4) {
+                const float4 kv = *reinterpret_cast<const float4*>(kr + c);
 #pragma unroll
-                for (int r = 0; r < kWarpRows; ++r) s[r] = fmaf(qw[r * DH + c], kv, s[r]);
+                for (int r = 0; r < R; ++r) {
+                    const float4 q = *reinterpret_cast<const float4*>(qw + r * DH + c);
+                    s[r] = fmaf(q.x, kv.x, s[r]); s[r] = fmaf(q.y, kv.y, s[r]); s[r] = fmaf(q.z, kv.z, s[r]); s[r] = fmaf(q.w, kv.w, s[r]);
+                }
             }
             const long long j = j0 + lane;
-            float pw[kWarpRows];
 #pragma unroll
-            for (int r = 0; r < kWarpRows; ++r) {
+            for (int r = 0; r < R; ++r) {
                 const bool vis = (j >= rlo[r]) && (j < rhi[r]) && (MODE == MKA_MODE_FULL || lam[r] > 0.f);
-                float x = vis ? s[r] : -INFINITY;
-                float mx = warp_max(x);
-                float m_new = fmaxf(m[st][r], mx);
+                const float x = vis ? s[r] : -INFINITY;
+                const float m_new = fmaxf(m[st][r], warp_max(x));
                 float e = (m_new == -INFINITY) ? 0.f : expf(x - m_new);   // masked: exp(-inf) = 0
-                float resc = (m[st][r] == -INFINITY) ? 0.f : expf(m[st][r] - m_new);
+                const float resc = (m[st][r] == -INFINITY) ? 0.f : expf(m[st][r] - m_new);
                 if (MODE == MKA_MODE_FAST) e *= lam[r];
-                z[st][r] = z[st][r] * resc + warp_sum(e);
+                z[st][r] = z[st][r] * resc + e;
 #pragma unroll
                 for (int k = 0; k < CPL; ++k) acc[st][r][k] *= resc;
                 m[st][r] = m_new;
-                pw[r] = e;
+                pw[r * 32 + lane] = e;
             }
-#pragma unroll 4
-            for (int jj = 0; jj < kKeys; ++jj) {
-                float pj[kWarpRows];
+            __syncwarp();
+#pragma unroll 2
+            for (int jj = 0; jj < kSimtTile; jj += 4) {
+                float4 e[R];
 #pragma unroll
-                for (int r = 0; r < kWarpRows; ++r) pj[r] = __shfl_sync(0xffffffffu, pw[r], jj);
+                for (int r = 0; r < R; ++r) e[r] = *reinterpret_cast<const float4*>(pw + r * 32 + jj);
 #pragma unroll
                 for (int k = 0; k < CPL; ++k) {
-                    int c = lane + 32 * k;
-                    float vv = c < DH ? vs[jj * LD + c] : 0.f;
+                    const float* v = vs + jj * LD + lane + 32 * k;
+                    const float v0 = v[0], v1 = v[LD], v2 = v[2 * LD], v3 = v[3 * LD];
 #pragma unroll
-                    for (int r = 0; r < kWarpRows; ++r) acc[st][r][k] = fmaf(pj[r], vv, acc[st][r][k]);
+                    for (int r = 0; r < R; ++r) {
+                        acc[st][r][k] = fmaf(e[r].x, v0, acc[st][r][k]); acc[st][r][k] = fmaf(e[r].y, v1, acc[st][r][k]);
+                        acc[st][r][k] = fmaf(e[r].z, v2, acc[st][r][k]); acc[st][r][k] = fmaf(e[r].w, v3, acc[st][r][k]);
+                    }
                 }
             }
+            __syncwarp();
         }
     }
 
+    // merge the groups: every group leaves (max, sum, acc) of its tiles, warp w then finishes row w
+    __syncthreads();
+    constexpr int kState = DH + 2;
 #pragma unroll
-    for (int r = 0; r < kWarpRows; ++r) {
-        long long t = t0 + warp * kWarpRows + r;
-        if (t >= p.T) continue;
-        float out[CPL];
+    for (int s = 0; s < NS; ++s)
 #pragma unroll
-        for (int k = 0; k < CPL; ++k) out[k] = 0.f;
+        for (int r = 0; r < R; ++r) {
+            float* o = tiles + ((group * kSimtRows + wg * R + r) * NS + s) * kState;
+            const float zr = warp_sum(z[s][r]);
+            if (lane == 0) { o[0] = m[s][r]; o[1] = zr; }
+#pragma unroll
+            for (int k = 0; k < CPL; ++k) o[2 + lane + 32 * k] = acc[s][r][k];
+        }
+    __syncthreads();
+    const long long t = t0 + warp;
+    if (t >= p.T) return;
+    float out[CPL];
+#pragma unroll
+    for (int k = 0; k < CPL; ++k) out[k] = 0.f;
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+        const float* o = tiles + (warp * NS + s) * kState;
+        constexpr int kGroupFloats = kSimtRows * NS * kState;
+        float M = -INFINITY, Z = 0.f, A[CPL];
+#pragma unroll
+        for (int g = 0; g < kSimtGroups; ++g) M = fmaxf(M, o[g * kGroupFloats]);
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) A[k] = 0.f;
+#pragma unroll
+        for (int g = 0; g < kSimtGroups; ++g) {
+            const float mg = o[g * kGroupFloats], f = mg == -INFINITY ? 0.f : expf(mg - M);
+            Z = fmaf(o[g * kGroupFloats + 1], f, Z);
+#pragma unroll
+            for (int k = 0; k < CPL; ++k) A[k] = fmaf(o[g * kGroupFloats + 2 + lane + 32 * k], f, A[k]);
+        }
+        float w;
         if (MODE == MKA_MODE_FAST) {
-            float inv = z[0][r] > 0.f ? 1.f / z[0][r] : 0.f;
-#pragma unroll
-            for (int k = 0; k < CPL; ++k) out[k] = acc[0][r][k] * inv;
-            if (p.LSE && lane == 0)
-                p.LSE[((long long)b * p.H + h) * p.T + t] = z[0][r] > 0.f ? m[0][r] + logf(z[0][r]) : -INFINITY;
+            w = Z > 0.f ? 1.f / Z : 0.f;
+            if (p.LSE && lane == 0) p.LSE[((long long)b * p.H + h) * p.T + t] = Z > 0.f ? M + logf(Z) : -INFINITY;
         } else {
-#pragma unroll
-            for (int s = 0; s < NS; ++s) {
-                float lam = p.gate[((long long)b * p.T + t) * 3 + s];
-                float w = z[s][r] > 0.f ? lam / z[s][r] : 0.f;
-#pragma unroll
-                for (int k = 0; k < CPL; ++k) out[k] = fmaf(acc[s][r][k], w, out[k]);
-            }
+            w = Z > 0.f ? p.gate[((long long)b * p.T + t) * 3 + s] / Z : 0.f;
         }
 #pragma unroll
-        for (int k = 0; k < CPL; ++k) {
-            int c = lane + 32 * k;
-            if (c < DH) Elem<T>::st(O + t * DH + c, out[k]);
-        }
+        for (int k = 0; k < CPL; ++k) out[k] = fmaf(A[k], w, out[k]);
     }
+#pragma unroll
+    for (int k = 0; k < CPL; ++k) Elem<T>::st(O + t * DH + lane + 32 * k, out[k]);
 }
 
 template <typename T, int DH>
 cudaError_t launch_t(const FwdParams& p, cudaStream_t st) {
-    dim3 grid((p.T + kRows - 1) / kRows, p.H, p.B), block(kThreads);
-    size_t smem = sizeof(float) * (kRows * DH + 2 * kKeys * (DH + 1));
-    cudaError_t e;
-    if (p.mode == MKA_MODE_FULL) {
-        e = cudaFuncSetAttribute(fwd_simt_kernel<T, DH, MKA_MODE_FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        fwd_simt_kernel<T, DH, MKA_MODE_FULL><<<grid, block, smem, st>>>(p);
-    } else {
-        e = cudaFuncSetAttribute(fwd_simt_kernel<T, DH, MKA_MODE_FAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        fwd_simt_kernel<T, DH, MKA_MODE_FAST><<<grid, block, smem, st>>>(p);
-    }
+    const dim3 grid((p.T + kSimtRows - 1) / kSimtRows, p.H, p.B);
+    const size_t smem = sizeof(float) * (kSimtRows * DH + 16 * kSimtWarpRows * 32 + kSimtGroups * 2 * kSimtTile * (DH + 4));
+    const int vec = simt_vec_bits(p.L, p.Q, nullptr, nullptr, sizeof(T) == 2 ? MKA_BF16 : MKA_F32);
+    auto kern = p.mode == MKA_MODE_FULL ? fwd_simt_kernel<T, DH, MKA_MODE_FULL> : fwd_simt_kernel<T, DH, MKA_MODE_FAST>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<grid, kSimtThreads, smem, st>>>(p, vec);
     return cudaGetLastError();
 }
 

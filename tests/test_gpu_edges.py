@@ -80,3 +80,40 @@ def test_router_gradient_splits(mka, orc, dtype, B, T, D):
     mag = np.abs(np64(P["X"]).reshape(-1, D)).T @ np.abs(dG.reshape(-1, 3))
     assert (np.abs(np64(g["dW_r"]) - dW) <= (B * T + 130) * 6e-8 * mag + 1e-30).all()
     assert (np.abs(np64(g["db_r"]) - db) <= 6e-8 * np.abs(db) + 1e-15 * np.abs(dG).sum() * B * T).all()
+
+
+@pytest.mark.parametrize("d,dtype,shift", [(32, torch.float32, 0), (64, torch.float32, 1), (96, torch.float32, 0), (128, torch.float32, 3),
+                                           (96, torch.bfloat16, 0), (32, torch.bfloat16, 0)])
+@pytest.mark.parametrize("T,W,q_off,N", [(1, 1, 0, (1, 1, 0)), (17, 5, 300, (317, 317, 33)), (130, 64, 0, (130, 100, 31))])
+def test_cuda_core_tiles(mka, orc, d, dtype, shift, T, W, q_off, N):
+    """CUDA-core kernels: rows and tiles that are not full, groups without a tile, float tensors that allow no 16-byte load."""
+    B, H = 2, 3
+    P = problem(23, B, H, T, d, N, 64, dtype, router_std=0.5, with_dO=True)
+
+    def moved(x):                       # the same values at an address `shift` floats off
+        if not shift:
+            return x
+        buf = torch.empty(x.numel() + shift, dtype=x.dtype, device=x.device)
+        out = buf[shift:].view(x.shape)
+        return out.copy_(x)
+
+    Q, dO, K, V = moved(P["Q"]), moved(P["dO"]), [moved(k) for k in P["K"]], [moved(v) for v in P["V"]]
+    gate = mka.mka_router(P["X"], P["W_r"], None)
+    mk = lambda mode: mka.make_shape(B, H, T, d, 64, W, q_off, dtype=mka.binding.MKA_BF16 if dtype == torch.bfloat16 else mka.binding.MKA_F32,  # noqa: E731
+                                     mode=mode)
+    shape, full = mk(mka.binding.MKA_MODE_FAST), mk(mka.binding.MKA_MODE_FULL)
+    assert mka.mka_fwd_kernel_kind(shape, K, V) == 0
+    O, LSE = mka.mka_fwd(shape, Q, K, V, gate)
+    g64 = np64(gate)
+    Or, Lr = orc.fwd(P["Q"], P["K"], P["V"], g64, W, q_off)
+    check(O, Or, dtype, "O")
+    assert err(LSE, Lr)[0] <= 1e-4
+    check(mka.mka_fwd(full, Q, K, V, gate)[0], orc.fwd(P["Q"], P["K"], P["V"], g64, W, q_off, mode="full")[0], dtype, "O of the per-level form")
+    g = mka.mka_bwd(shape, Q, K, V, gate, O, LSE, dO, R=P["X"])
+    r = orc.bwd(P["Q"], P["K"], P["V"], g64, P["dO"], W, q_off)
+    check(g["dQ"], r["dQ"], dtype, "dQ")
+    for l in range(3):
+        if N[l]:
+            check(g["dK"][l], r["dK"][l], dtype, f"dK{l}")
+            check(g["dV"][l], r["dV"][l], dtype, f"dV{l}")
+    check(g["dG"], r["dG"], dtype, "dG")
