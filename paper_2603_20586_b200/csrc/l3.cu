@@ -13,7 +13,7 @@ namespace mka {
 namespace {
 
 constexpr int kIdxThreads = 128;
-constexpr int kIdxPairs = 32;                         // (page, head) pairs per batch of a CTA: one per lane in the projections
+constexpr int kIdxPairs = 64;                         // (page, head) pairs per batch of a CTA: two per lane in the projections
 constexpr int kIdxBitsPerWarp = 16;                   // code bits one warp works out per pass
 
 struct L3IndexParams {
@@ -24,108 +24,168 @@ struct L3IndexParams {
     int H_kv, page_rows, d, bits;
 };
 
-// Dynamic shared memory: projT [d][bits + 4] floats (16 consecutive bits of one column are one broadcast read), then
-// s [kIdxPairs][d + 1] floats (the key sums; the odd pitch keeps the lanes of a warp on different banks).
-// A batch = 32 (page, head) pairs.  Loading: 16 threads cover one 256-byte row, a thread sums its eight columns row by
-// row.  Projections: lane = pair, warp = 16 bits; column i costs one read of s, four broadcast reads of projT and 16
-// fmaf, so the arithmetic, not shared memory, is what the projections wait for.
+// Dynamic shared memory: projT [d][bits + 4] floats (16 consecutive bits of one column are four broadcast reads), then two
+// buffers s [kIdxPairs][d + 1] floats (the key sums; the odd pitch keeps the lanes of a warp on different banks).
+// A batch = 64 (page, head) pairs.  The first four warps load: 16 threads cover one 256-byte row, a thread sums its eight
+// columns row by row, with up to 24 loads in flight across items and batches.  The other four project: lane = two pairs,
+// warp = 16 bits; column i costs two reads of s, four broadcast reads of projT and 32 fmaf.  The two halves work on different batches,
+// so the loads of one run under the projections of the other.  As two phases of the same warps, and with one pair to a
+// lane, the shared-memory pipe was busy for 78 us and HBM idle half of the time: 147 us (3.6 TB/s) for [32769 pages, 4 heads, 16
+// rows, 128] at 64 bits, 123 us now (4.4 TB/s).  Registers are moved from the projecting to the loading warps.
 template <int DH>
-__global__ void __launch_bounds__(kIdxThreads, 4) l3_index_kernel(const L3IndexParams p) {
+__global__ void __launch_bounds__(2 * kIdxThreads, 2) l3_index_kernel(const L3IndexParams p) {
     extern __shared__ __align__(16) float sm[];
     const int ppitch = p.bits + 4;                             // floats between columns of projT (keeps the fill off one bank)
+    constexpr int pitch = DH + 1, kSumFloats = kIdxPairs * pitch;
     float* projT = sm;
-    float* s = sm + (size_t)DH * ppitch;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int pitch = DH + 1;
-    for (int e = tid; e < DH * p.bits; e += kIdxThreads) {     // e = j * d + i: coalesced reads of proj
+    float* sums = sm + (size_t)DH * ppitch;
+    const int tid = threadIdx.x & (kIdxThreads - 1), lane = tid & 31, warp = tid >> 5;
+    for (int e = threadIdx.x; e < DH * p.bits; e += 2 * kIdxThreads) {     // e = j * d + i: coalesced reads of proj
         const int j = e / DH, i = e % DH;
         projT[i * ppitch + j] = p.proj[e];
     }
+    __syncthreads();
     constexpr int vecs = DH / 8;                               // 16-byte pieces of a row: 16 (d = 128) or 8 (d = 64)
-    constexpr int items = kIdxPairs * vecs;                    // (pair, piece) items of a batch
-    constexpr int kPerThread = items / kIdxThreads;            // 4 or 2: taken two at a time, 16 loads in flight
+    constexpr int kPerThread = kIdxPairs * vecs / kIdxThreads; // (pair, piece) items of a thread in a batch: 8 or 4
+    constexpr int kSlotStep = kIdxThreads / vecs;              // pairs between a thread's items
     const long long pairs = p.n_pages * p.H_kv;
     const int words = p.bits / 32;
-    unsigned short* codes16 = reinterpret_cast<unsigned short*>(p.codes);
-    for (long long base = (long long)blockIdx.x * kIdxPairs; base < pairs; base += (long long)gridDim.x * kIdxPairs) {
-        __syncthreads();                                       // projT is there; the previous batch is done with s
-        // ---- sums of the pages' keys, row by row
-#pragma unroll
-        for (int k0 = 0; k0 < kPerThread; k0 += 2) {
-            float acc[2][8];
-            const __nv_bfloat16* src[2];
-            bool live[2];
-            int slot[2], piece[2];
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const int it = tid + (k0 + q) * kIdxThreads;
-                slot[q] = it / vecs; piece[q] = it % vecs;
-                const long long pair = base + slot[q];
-                live[q] = pair < pairs;
-                const long long pc = live[q] ? pair : 0;
-                src[q] = p.k + (pc / p.H_kv) * p.sp + (pc % p.H_kv) * p.sh + piece[q] * 8;
-#pragma unroll
-                for (int i = 0; i < 8; ++i) acc[q][i] = 0.f;
+    const long long step = (long long)gridDim.x * kIdxPairs, first = (long long)blockIdx.x * kIdxPairs;
+    // barriers 1, 2: buffer 0 / 1 is filled;  3, 4: it is free again (256 threads: one half arrives, the other waits)
+    auto arrive = [](int id) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(2 * kIdxThreads) : "memory"); };
+    auto wait = [](int id) { asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(2 * kIdxThreads) : "memory"); };
+    if (threadIdx.x < kIdxThreads) {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 152;");  // 256 threads x 128 registers at launch = 128 x 152 + 128 x 104
+        const int slot0 = tid / vecs, piece = tid % vecs;
+        constexpr int kDepth = 3;
+        uint4 u[kDepth][8];
+        // the next eight rows to ask for
+        long long f_base = first;
+        int f_item = 0, f_row = 0;
+        const __nv_bfloat16* f_src = nullptr;                  // null: the pair does not exist
+        auto locate = [&] {
+            const long long pair = f_base + slot0 + f_item * kSlotStep;
+            f_src = nullptr;
+            if (pair < pairs) {
+                const long long page = pair <= 0x7fffffffLL ? (long long)((unsigned)pair / (unsigned)p.H_kv) : pair / p.H_kv;
+                f_src = p.k + page * p.sp + (pair - page * p.H_kv) * p.sh + piece * 8;
             }
-            for (int r0 = 0; r0 < p.page_rows; r0 += 8) {
-                uint4 u[2][8];
+        };
+        locate();
+        auto fetch = [&](uint4 (&to)[8]) {
+            if (f_base >= pairs) return;
+            if (f_src) {
+                if (f_row + 8 <= p.page_rows) {
 #pragma unroll
-                for (int q = 0; q < 2; ++q)
+                    for (int r = 0; r < 8; ++r) to[r] = __ldg(reinterpret_cast<const uint4*>(f_src + r * p.sn));
+                } else {
 #pragma unroll
                     for (int r = 0; r < 8; ++r)
-                        u[q][r] = (live[q] && r0 + r < p.page_rows)
-                                      ? __ldg(reinterpret_cast<const uint4*>(src[q] + (long long)(r0 + r) * p.sn))
-                                      : make_uint4(0u, 0u, 0u, 0u);
+                        if (f_row + r < p.page_rows) to[r] = __ldg(reinterpret_cast<const uint4*>(f_src + r * p.sn));
+                }
+                f_src += 8 * p.sn;
+            }
+            f_row += 8;
+            if (f_row >= p.page_rows) {
+                f_row = 0;
+                if (++f_item == kPerThread) { f_item = 0; f_base += step; }
+                locate();
+            }
+        };
+#pragma unroll
+        for (int i = 0; i < kDepth; ++i) fetch(u[i]);
+        unsigned long long acc[4];                             // eight columns as packed pairs (add.rn.f32x2: two plain sums)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[i] = 0ull;
+        auto add_row = [&](const uint4& v) {
+            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                unsigned long long x2;
+                asm("mov.b64 %0, {%1, %2};" : "=l"(x2) : "r"(w[i] << 16), "r"(w[i] & 0xffff0000u));
+                asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc[i]) : "l"(x2));
+            }
+        };
+        long long base = first;
+        int n = 0, item = 0, row = 0;
+        while (base < pairs) {
+#pragma unroll
+            for (int x = 0; x < kDepth; ++x) {
+                if (base >= pairs) break;
+                if (row + 8 <= p.page_rows) {
+#pragma unroll
+                    for (int r = 0; r < 8; ++r) add_row(u[x][r]);
+                } else {
+#pragma unroll
+                    for (int r = 0; r < 8; ++r)
+                        if (row + r < p.page_rows) add_row(u[x][r]);   // rows past the page add nothing, not even +0
+                }
+                fetch(u[x]);
+                row += 8;
+                if (row >= p.page_rows) {
+                    if (item == 0 && n >= 2) wait(3 + (n & 1));            // the batch before last has been projected
+                    float* s = sums + (n & 1) * kSumFloats + (slot0 + item * kSlotStep) * pitch + piece * 8;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        asm("mov.b64 {%0, %1}, %2;" : "=f"(s[2 * i]), "=f"(s[2 * i + 1]) : "l"(acc[i]));
+                        acc[i] = 0ull;
+                    }
+                    row = 0;
+                    if (++item == kPerThread) {
+                        arrive(1 + (n & 1));
+                        item = 0; ++n; base += step;
+                    }
+                }
+            }
+        }
+    } else {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
+        unsigned short* codes16 = reinterpret_cast<unsigned short*>(p.codes);
+        int n = 0;
+        for (long long base = first; base < pairs; base += step, ++n) {
+            // ---- projections: one fmaf chain per (pair, bit) over the columns 0..d-1
+            wait(1 + (n & 1));
+            const float* sv = sums + (n & 1) * kSumFloats + lane * pitch;
+            for (int j0 = warp * kIdxBitsPerWarp; j0 < p.bits; j0 += (kIdxThreads / 32) * kIdxBitsPerWarp) {
+                // two chains per instruction (fma.rn.f32x2: each half is the same correctly rounded fma as fmaf)
+                unsigned long long a2[2][kIdxBitsPerWarp / 2];
 #pragma unroll
                 for (int q = 0; q < 2; ++q)
 #pragma unroll
-                    for (int r = 0; r < 8; ++r) {
-                        if (r0 + r < p.page_rows) {                // rows past the page add nothing, not even +0
-                            const uint32_t w[4] = {u[q][r].x, u[q][r].y, u[q][r].z, u[q][r].w};
+                    for (int j = 0; j < kIdxBitsPerWarp / 2; ++j) a2[q][j] = 0ull;          // two +0.f
+                const float* pj = projT + j0;
+#pragma unroll 4
+                for (int i = 0; i < DH; ++i) {
+                    const float xa = sv[i], xb = sv[32 * pitch + i];
+                    unsigned long long x2[2];
+                    asm("mov.b64 %0, {%1, %1};" : "=l"(x2[0]) : "f"(xa));
+                    asm("mov.b64 %0, {%1, %1};" : "=l"(x2[1]) : "f"(xb));
 #pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                acc[q][2 * i] = acc[q][2 * i] + __uint_as_float(w[i] << 16);
-                                acc[q][2 * i + 1] = acc[q][2 * i + 1] + __uint_as_float(w[i] & 0xffff0000u);
-                            }
+                    for (int v = 0; v < kIdxBitsPerWarp / 4; ++v) {
+                        const ulonglong2 pr = *reinterpret_cast<const ulonglong2*>(pj + (size_t)i * ppitch + 4 * v);   // bits 4v..4v+3 of column i
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a2[q][2 * v]) : "l"(pr.x), "l"(x2[q]));
+                            asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a2[q][2 * v + 1]) : "l"(pr.y), "l"(x2[q]));
                         }
                     }
-            }
+                }
 #pragma unroll
-            for (int q = 0; q < 2; ++q)
+                for (int q = 0; q < 2; ++q) {
+                    unsigned half = 0u;
 #pragma unroll
-                for (int i = 0; i < 8; ++i) s[slot[q] * pitch + piece[q] * 8 + i] = acc[q][i];
-        }
-        __syncthreads();
-        // ---- projections: one fmaf chain per (pair, bit) over the columns 0..d-1
-        const long long pair = base + lane;
-        const float* sv = s + lane * pitch;
-        for (int j0 = warp * kIdxBitsPerWarp; j0 < p.bits; j0 += (kIdxThreads / 32) * kIdxBitsPerWarp) {
-            // two chains per instruction (fma.rn.f32x2: each half is the same correctly rounded fma as fmaf)
-            unsigned long long a2[kIdxBitsPerWarp / 2];
-#pragma unroll
-            for (int j = 0; j < kIdxBitsPerWarp / 2; ++j) a2[j] = 0ull;          // two +0.f
-            const float* pj = projT + j0;
-            for (int i = 0; i < DH; ++i) {
-                const float x = sv[i];
-                unsigned long long x2;
-                asm("mov.b64 %0, {%1, %1};" : "=l"(x2) : "f"(x));
-#pragma unroll
-                for (int v = 0; v < kIdxBitsPerWarp / 4; ++v) {
-                    const ulonglong2 pr = *reinterpret_cast<const ulonglong2*>(pj + (size_t)i * ppitch + 4 * v);   // bits 4v..4v+3 of column i
-                    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a2[2 * v]) : "l"(pr.x), "l"(x2));
-                    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a2[2 * v + 1]) : "l"(pr.y), "l"(x2));
+                    for (int j = 0; j < kIdxBitsPerWarp / 2; ++j) {
+                        float lo, hi;
+                        asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a2[q][j]));
+                        half |= (lo >= 0.f ? 1u : 0u) << (2 * j);
+                        half |= (hi >= 0.f ? 1u : 0u) << (2 * j + 1);
+                    }
+                    // bits j0..j0+15 are one 16-bit half of word j0 / 32 (low half first)
+                    const long long pair = base + q * 32 + lane;
+                    if (pair < pairs) codes16[(pair * words) * 2 + j0 / 16] = (unsigned short)half;
                 }
             }
-            unsigned half = 0u;
-#pragma unroll
-            for (int j = 0; j < kIdxBitsPerWarp / 2; ++j) {
-                float lo, hi;
-                asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a2[j]));
-                half |= (lo >= 0.f ? 1u : 0u) << (2 * j);
-                half |= (hi >= 0.f ? 1u : 0u) << (2 * j + 1);
-            }
-            // bits j0..j0+15 are one 16-bit half of word j0 / 32 (low half first)
-            if (pair < pairs) codes16[(pair * words) * 2 + j0 / 16] = (unsigned short)half;
+            if (base + 2 * step < pairs) arrive(3 + (n & 1));  // (nobody waits for the last two)
         }
     }
 }
@@ -258,18 +318,18 @@ cudaError_t launch_l3_index(const void* k, long long n_pages, int H_kv, int page
     L3IndexParams p;
     p.k = static_cast<const __nv_bfloat16*>(k); p.proj = proj; p.codes = codes;
     p.n_pages = n_pages; p.sp = sp; p.sh = sh; p.sn = sn; p.H_kv = H_kv; p.page_rows = page_rows; p.d = d; p.bits = bits;
-    const size_t smem = ((size_t)d * (bits + 4) + (size_t)kIdxPairs * (d + 1)) * sizeof(float);
+    const size_t smem = ((size_t)d * (bits + 4) + 2 * (size_t)kIdxPairs * (d + 1)) * sizeof(float);
     auto kern = d == 128 ? l3_index_kernel<128> : l3_index_kernel<64>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const long long batches = (n_pages * H_kv + kIdxPairs - 1) / kIdxPairs;
-    const long long per_sm = smem > 110 * 1024 ? 1 : (smem > 72 * 1024 ? 2 : (smem > 54 * 1024 ? 3 : 4));
+    const long long per_sm = smem > 112 * 1024 ? 1 : 2;
     const long long resident = 148LL * per_sm;
     // persistent CTAs: every CTA transposes the projection into shared memory once and then walks its batches
     // (the grid is shrunk so that all CTAs get the same number of batches)
     const long long per_cta = (batches + resident - 1) / resident;
     const long long grid = (batches + per_cta - 1) / per_cta;
-    kern<<<(unsigned)grid, kIdxThreads, smem, st>>>(p);
+    kern<<<(unsigned)grid, 2 * kIdxThreads, smem, st>>>(p);
     return cudaGetLastError();
 }
 

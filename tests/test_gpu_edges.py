@@ -117,3 +117,14 @@ def test_cuda_core_tiles(mka, orc, d, dtype, shift, T, W, q_off, N):
             check(g["dK"][l], r["dK"][l], dtype, f"dK{l}")
             check(g["dV"][l], r["dV"][l], dtype, f"dV{l}")
     check(g["dG"], r["dG"], dtype, "dG")
+
+
+@pytest.mark.parametrize("d,bits", [(64, 32), (128, 64), (128, 256)])
+@pytest.mark.parametrize("pages,H_kv,page", [(1, 1, 16), (21, 3, 8), (300, 4, 5), (1201, 4, 24)])
+def test_recall_codes_batches(mka, orc, d, bits, pages, H_kv, page):
+    """Recall codes: a batch with one pair, a last batch that is not full, pages of no whole number of eight rows, several batches a CTA."""
+    g = torch.Generator().manual_seed(3)
+    pool = torch.randn(pages, H_kv, page, d, generator=g).bfloat16().cuda()
+    proj = torch.randn(bits, d, generator=g).cuda()
+    codes = mka.mka_l3_index(pool, proj)
+    assert np.array_equal(codes.cpu().numpy().view(np.uint32), orc.l3_index(pool.float().cpu().numpy(), proj.cpu().numpy()))
