@@ -81,33 +81,33 @@ def _load() -> ctypes.CDLL:
     lib.mka_workspace_bytes.argtypes = [ctypes.POINTER(mka_shape), ctypes.POINTER(ctypes.c_int64), ctypes.c_int32]
     vp, i32, i64 = ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64
     lib.mka_router.argtypes = [vp, vp, vp, i64, i32, i32, i32, vp, vp, vp, vp]
-    lib.mka_fwd.argtypes = [ctypes.POINTER(mka_shape), vp, ctypes.POINTER(mka_level), vp, vp, vp, vp, ctypes.c_size_t, vp]
+    lib.mka_fwd.argtypes = [ctypes.POINTER(mka_shape), vp, vp, vp, vp, vp, vp, ctypes.c_size_t, vp]
     lib.mka_decode.argtypes = lib.mka_fwd.argtypes
-    lib.mka_bwd.argtypes = [ctypes.POINTER(mka_shape), vp, ctypes.POINTER(mka_level), vp, vp, vp, vp, vp, i32, vp,
+    lib.mka_bwd.argtypes = [ctypes.POINTER(mka_shape), vp, vp, vp, vp, vp, vp, vp, i32, vp,
                             ctypes.POINTER(mka_level_grad), vp, vp, vp, vp, ctypes.c_size_t, vp]
     lib.mka_decode_plan.argtypes = [ctypes.POINTER(ctypes.c_int64), i32, i32, i32, ctypes.POINTER(mka_decode_plan_t)]
     lib.mka_fwd_tile_range.argtypes = [ctypes.POINTER(mka_shape), ctypes.POINTER(ctypes.c_int64), i32, i64,
                                        ctypes.POINTER(mka_tile_range)]
     lib.mka_device_status.argtypes = [vp, vp]
-    lib.mka_decode_static.argtypes = [ctypes.POINTER(mka_shape), vp, ctypes.POINTER(mka_level), vp, vp, vp, vp]
+    lib.mka_decode_static.argtypes = [ctypes.POINTER(mka_shape), vp, vp, vp, vp, vp, vp]
     lib.mka_decode_static_max_bytes.restype = ctypes.c_size_t
     lib.mka_decode_static_max_bytes.argtypes = []
-    lib.mka_fwd_kernel_kind.argtypes = [ctypes.POINTER(mka_shape), ctypes.POINTER(mka_level)]
-    lib.mka_fuse_kv.argtypes = [i32, i32, i64, i32, i32, ctypes.POINTER(mka_level), vp, ctypes.POINTER(mka_level_grad), i64, vp]
+    lib.mka_fwd_kernel_kind.argtypes = [ctypes.POINTER(mka_shape), vp]
+    lib.mka_fuse_kv.argtypes = [i32, i32, i64, i32, i32, vp, vp, ctypes.POINTER(mka_level_grad), i64, vp]
     lib.mka_l2_summary_workspace_bytes.restype = ctypes.c_size_t
     lib.mka_l2_summary_workspace_bytes.argtypes = [i32, i64, i32, i32]
     lib.mka_decode_paged_workspace_bytes.restype = ctypes.c_size_t
     lib.mka_decode_paged_workspace_bytes.argtypes = [ctypes.POINTER(mka_shape), i32, ctypes.POINTER(ctypes.c_int64)]
-    lib.mka_decode_paged.argtypes = [ctypes.POINTER(mka_shape), i32, vp, ctypes.POINTER(mka_paged_level), vp, vp, vp, vp,
+    lib.mka_decode_paged.argtypes = [ctypes.POINTER(mka_shape), i32, vp, vp, vp, vp, vp, vp,
                                      ctypes.c_size_t, vp]
     lib.mka_fwd_paged.argtypes = lib.mka_decode_paged.argtypes
-    lib.mka_fuse_kv_paged.argtypes = [i32, i32, i64, i32, i32, ctypes.POINTER(mka_level), vp, ctypes.POINTER(mka_paged_level), i64,
+    lib.mka_fuse_kv_paged.argtypes = [i32, i32, i64, i32, i32, vp, vp, ctypes.POINTER(mka_paged_level), i64,
                                       vp, vp]
     lib.mka_l3_index.argtypes = [vp, i64, i32, i32, i32, i64, i64, i64, vp, i32, vp, vp]
     lib.mka_l3_retrieve.argtypes = [vp, i32, i32, i32, i32, vp, i32, vp, vp, vp, i64, i32, i32, i32, vp, vp, vp, vp]
     lib.mka_l2_summary_kernel_kind.argtypes = [i32, i64, i32, i32, ctypes.c_size_t]
     lib.mka_l2_summary.argtypes = [vp, i32, i64, i32, i32, i32, ctypes.c_float, vp, i64, vp, vp, ctypes.c_size_t, vp]
-    lib.mka_bwd_kernel_kind.argtypes = [ctypes.POINTER(mka_shape), ctypes.POINTER(mka_level), vp]
+    lib.mka_bwd_kernel_kind.argtypes = [ctypes.POINTER(mka_shape), vp, vp]
     lib.mka_set_wait_limit_us.argtypes = [ctypes.c_uint32]
     for name in EXPORTS:
         if name not in ("mka_status_str", "mka_workspace_bytes", "mka_decode_static_max_bytes", "mka_l2_summary_workspace_bytes",
@@ -137,14 +137,15 @@ def _dt(t: torch.Tensor) -> int:
     raise TypeError(f"unsupported dtype {t.dtype}")
 
 
+# A small call (one decode step, a short prompt) is over sooner on the GPU than its arguments used to be marshalled here, so
+# pointers travel as plain ints, a call's levels as one array of 64-bit words (both are what the declared argument types and
+# the struct layouts say), and the current stream is asked for without building a Stream object.
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+def _stream(stream) -> int:
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()) if stream is None else stream.cuda_stream
 
 
 def _n_level(n) -> ctypes.Array:
@@ -156,16 +157,23 @@ def make_shape(B, H, T, d, D=0, window=1, q_offset=0, scale=0.0, dtype=MKA_BF16,
     return mka_shape(B, H, T, d, D, window, q_offset, scale, dtype, mode, flags, kv_heads)
 
 
+_LevelWords = ctypes.c_int64 * 18        # mka_level[3]: k, v, n, stride_b, stride_h, stride_n
+_PagedWords = ctypes.c_int64 * 36        # mka_paged_level[3]: twelve 8-byte slots each (page_rows is the low half of its own)
+_NO_LEVEL = (0,) * 6
+_NO_PAGED_LEVEL = (0,) * 7 + (1, 0, 0, 0, 0)
+
+
 def _levels(K: Sequence[Optional[torch.Tensor]], V: Sequence[Optional[torch.Tensor]]):
-    arr = (mka_level * 3)()
+    words = ()
     for l in range(3):
         k, v = K[l], V[l]
         if k is None or k.shape[2] == 0:
-            arr[l] = mka_level(None, None, 0, 0, 0, 0)
+            words += _NO_LEVEL
             continue
-        assert k.dim() == 4 and k.stride(3) == 1 and v.stride() == k.stride() and v.shape == k.shape
-        arr[l] = mka_level(k.data_ptr(), v.data_ptr(), k.shape[2], k.stride(0), k.stride(1), k.stride(2))
-    return arr
+        shape, stride = k.shape, k.stride()
+        assert len(shape) == 4 and stride[3] == 1 and v.stride() == stride and v.shape == shape
+        words += (k.data_ptr(), v.data_ptr(), shape[2]) + stride[:3]
+    return _LevelWords(*words)
 
 
 def mka_workspace_bytes(shape: mka_shape, n_level, which: int) -> int:
@@ -210,9 +218,8 @@ def mka_fwd(shape: mka_shape, Q, K, V, gate, O=None, LSE=None, ws=None, stream=N
         O = torch.empty_like(Q)
     if LSE is None and want_lse and shape.mode == MKA_MODE_FAST:
         LSE = torch.empty(Q.shape[:3], dtype=torch.float32, device=Q.device)
-    n = [0 if k is None else k.shape[2] for k in K]
     if ws is None:
-        ws = alloc_workspace(shape, n, MKA_WS_FWD, Q.device)
+        ws = alloc_workspace(shape, [0 if k is None else k.shape[2] for k in K], MKA_WS_FWD, Q.device)
     _check(lib.mka_fwd(ctypes.byref(shape), _ptr(Q), _levels(K, V), _ptr(gate), _ptr(O), _ptr(LSE), _ptr(ws),
                        ws.numel(), _stream(stream)), "mka_fwd")
     return O, LSE
@@ -224,32 +231,32 @@ def mka_decode(shape: mka_shape, q, K, V, gate, O=None, LSE=None, ws=None, strea
         O = torch.empty_like(q)
     if LSE is None:
         LSE = torch.empty(q.shape[:2], dtype=torch.float32, device=q.device)
-    n = [0 if k is None else k.shape[2] for k in K]
     if ws is None:
-        ws = alloc_workspace(shape, n, MKA_WS_DECODE, q.device)
+        ws = alloc_workspace(shape, [0 if k is None else k.shape[2] for k in K], MKA_WS_DECODE, q.device)
     _check(lib.mka_decode(ctypes.byref(shape), _ptr(q), _levels(K, V), _ptr(gate), _ptr(O), _ptr(LSE), _ptr(ws),
                           ws.numel(), _stream(stream)), "mka_decode")
     return O, LSE
 
 
 def _paged_levels(pools_k, pools_v, tables, rows, n):
-    arr = (mka_paged_level * 3)()
+    words = ()
     for l in range(3):
         k, v = pools_k[l], pools_v[l]
         if k is None or n[l] == 0:
-            arr[l] = mka_paged_level(None, None, None, None, 0, 0, 0, 1, 0, 0, 0, 0)
+            words += _NO_PAGED_LEVEL
             continue
         # pools [pages, H_kv, page_rows, d]; any strides with d contiguous
-        assert k.dim() == 4 and k.stride(3) == 1 and v.stride() == k.stride() and v.shape == k.shape
+        shape, stride = k.shape, k.stride()
+        assert len(shape) == 4 and stride[3] == 1 and v.stride() == stride and v.shape == shape
         tab = tables[l]
         # [B, pages]: one table per sequence; [B, H_kv, pages]: one per (sequence, KV head)
-        assert tab.dtype == torch.int32 and tab.dim() in (2, 3) and tab.stride(-1) == 1
+        ts = tab.stride()
+        assert tab.dtype == torch.int32 and len(ts) in (2, 3) and ts[-1] == 1
         r = None if rows is None else rows[l]
         assert r is None or (r.dtype == torch.int32 and r.is_contiguous())
-        arr[l] = mka_paged_level(k.data_ptr(), v.data_ptr(), tab.data_ptr(), _ptr(r), int(n[l]), tab.stride(0),
-                                 tab.stride(1) if tab.dim() == 3 else 0, k.shape[2], k.stride(0), k.stride(1), k.stride(2),
-                                 k.shape[0])
-    return arr
+        words += (k.data_ptr(), v.data_ptr(), tab.data_ptr(), 0 if r is None else r.data_ptr(), int(n[l]), ts[0],
+                  ts[1] if len(ts) == 3 else 0, shape[2]) + stride[:3] + (shape[0],)
+    return _PagedWords(*words)
 
 
 def mka_fuse_kv_paged(K, V, gate, pool_k, pool_v, table, dst_offset=0, dst_offsets=None, stream=None):
@@ -378,9 +385,8 @@ def mka_bwd(shape: mka_shape, Q, K, V, gate, O, LSE, dO, R=None, dQ=None, dK=Non
             g = dK[l]
             assert g.stride(3) == 1 and dV[l].stride() == g.stride()
             grads[l] = mka_level_grad(g.data_ptr(), dV[l].data_ptr(), g.shape[2], g.stride(0), g.stride(1), g.stride(2))
-    n = [0 if k is None else k.shape[2] for k in K]
     if ws is None:
-        ws = alloc_workspace(shape, n, MKA_WS_BWD, dev)
+        ws = alloc_workspace(shape, [0 if k is None else k.shape[2] for k in K], MKA_WS_BWD, dev)
     _check(lib.mka_bwd(ctypes.byref(shape), _ptr(Q), _levels(K, V), _ptr(gate), _ptr(O), _ptr(LSE), _ptr(dO),
                        _ptr(R), _dt(R) if R is not None else MKA_F32, _ptr(dQ), grads, _ptr(dG), _ptr(dW_r),
                        _ptr(db_r), _ptr(ws), ws.numel(), _stream(stream)), "mka_bwd")
