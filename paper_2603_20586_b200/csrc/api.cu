@@ -199,12 +199,14 @@ mka_status mka_fwd(const mka_shape* s, const void* Q, const mka_level L[3], cons
     p.mode = s->mode; p.decode = 0; p.kv_group = kv_group_of(s);
     p.test_stall = (s->flags & MKA_FLAG_TEST_STALL) ? 1 : 0;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(ws, 0, 16, cs) != cudaSuccess) return MKA_ERR_CUDA;
+    p.status = static_cast<unsigned int*>(ws);
     cudaError_t e;
-    if (!(s->flags & MKA_FLAG_FORCE_SIMT) && s->mode == MKA_MODE_FAST && fwd_tc_eligible(p, s->dtype))
+    if (!(s->flags & MKA_FLAG_FORCE_SIMT) && s->mode == MKA_MODE_FAST && fwd_tc_eligible(p, s->dtype)) {
+        if (cudaMemsetAsync(ws, 0, 16, cs) != cudaSuccess) return MKA_ERR_CUDA;
         e = launch_fwd_tc(p, static_cast<unsigned int*>(ws), cs);
-    else
+    } else {
         e = launch_fwd_simt(p, s->dtype, cs);
+    }
     if (e == cudaErrorNotSupported) return MKA_ERR_UNSUPPORTED;
     return e == cudaSuccess ? MKA_OK : MKA_ERR_CUDA;
 }
@@ -272,7 +274,7 @@ mka_status mka_decode(const mka_shape* s, const void* q, const mka_level L[3], c
     for (int l = 0; l < 3; ++l) p.n_chunks[l] = plan.n_chunks[l];
     p.total_chunks = plan.total_chunks;
     p.partial = reinterpret_cast<float*>(static_cast<char*>(ws) + kWsHeader);
-    if (cudaMemsetAsync(ws, 0, 16, cs) != cudaSuccess) return MKA_ERR_CUDA;
+    p.status = static_cast<unsigned int*>(ws);
     cudaError_t e = launch_decode(p, cs);
     if (e == cudaErrorNotSupported) return MKA_ERR_UNSUPPORTED;
     return e == cudaSuccess ? MKA_OK : MKA_ERR_CUDA;
@@ -503,7 +505,7 @@ mka_status mka_bwd(const mka_shape* s, const void* Q, const mka_level L[3], cons
     p.test_stall = (s->flags & MKA_FLAG_TEST_STALL) ? 1 : 0;
     const bool tc = !(s->flags & MKA_FLAG_FORCE_SIMT) && bwd_tc_eligible(p, s->dtype);
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(ws, 0, 16, cs) != cudaSuccess) return MKA_ERR_CUDA;
+    p.status = static_cast<unsigned int*>(ws);
     cudaError_t e;
     if (tc)
         e = launch_bwd_tc(p, static_cast<unsigned int*>(ws), cs);

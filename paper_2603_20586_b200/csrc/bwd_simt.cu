@@ -24,6 +24,7 @@ __global__ void __launch_bounds__(kSimtThreads) bwd_dq_kernel(const BwdParams p,
     const long long bh = (long long)b * p.H + h;
     const T* Q = static_cast<const T*>(p.Q) + bh * p.T * DH;
     const T* dO = static_cast<const T*>(p.dO) + bh * p.T * DH;
+    if (threadIdx.x < 4 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) p.status[threadIdx.x] = 0u;
     for (int i = threadIdx.x * 4; i < kSimtRows * DH; i += kSimtThreads * 4) {
         const long long t = t0 + i / DH;
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;

@@ -205,7 +205,9 @@ template <int DH>
 __global__ void __launch_bounds__(256) bwd_prep_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfloat16* __restrict__ dO,
                                                        const float* __restrict__ LSE, const float* __restrict__ gate, int H,
                                                        int T, int Tpad, float* __restrict__ sD,
-                                                       float* __restrict__ b0, float* __restrict__ b1, float* __restrict__ b2) {
+                                                       float* __restrict__ b0, float* __restrict__ b1, float* __restrict__ b2,
+                                                       unsigned int* __restrict__ header) {
+    if (threadIdx.x < 4 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) header[threadIdx.x] = 0u;   // status word and tickets of the kernels that follow
     constexpr int LPR = DH / 8;                            // lanes per row: 16 or 8
     constexpr int RPW = 32 / LPR;                          // rows per warp and pass
     constexpr int kPasses = 4;
@@ -1134,7 +1136,7 @@ cudaError_t launch_t(const BwdParams& bp, unsigned int* status_word, cudaStream_
     constexpr int kPrepRowsPerBlock = 8 * (32 / (DH / 8)) * 4;          // 8 warps x rows per pass x passes
     bwd_prep_kernel<DH><<<dim3((Tpad + kPrepRowsPerBlock - 1) / kPrepRowsPerBlock, bp.H, bp.B), 256, 0, st>>>(
         static_cast<const __nv_bfloat16*>(bp.O), static_cast<const __nv_bfloat16*>(bp.dO), bp.LSE, bp.gate, bp.H, bp.T, Tpad,
-        statD, statB[0], statB[1], statB[2]);
+        statD, statB[0], statB[1], statB[2], status_word);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
 

@@ -45,6 +45,7 @@ struct FwdParams {
     int decode;         // every row visible
     int kv_group;       // query heads per KV head (>= 1): head h reads KV head h / kv_group
     int test_stall;     // MKA_FLAG_TEST_STALL (tensor-core forward, dense levels)
+    unsigned int* status;   // device status word; the CUDA-core kernel, which waits for nothing, writes MKA_OK itself
     const PagedLevelDev* paged;   // host array of 3, or null: the levels are page pools (tensor-core forward only; L[l].n still holds the rows)
 };
 
@@ -102,6 +103,7 @@ struct DecodeParams {
     long long n_chunks[3];
     long long total_chunks;
     float* partial;      // [B*H, total_chunks, d+2]
+    unsigned int* status;   // device status word that the combine kernel sets to MKA_OK, or null (kernels before it may wait and set it)
 };
 cudaError_t launch_decode(const DecodeParams& p, cudaStream_t st);
 cudaError_t launch_decode_combine(const DecodeParams& p, cudaStream_t st);   // second kernel alone (gate, n_chunks, partial, O, LSE)
@@ -150,6 +152,7 @@ struct BwdParams {
     int window, q_offset;
     float scale;
     int kv_group;     // query heads per KV head (>= 1); > 1 only on the tensor-core path
+    unsigned int* status;   // first 16 bytes of the workspace (status word, tickets): cleared by the first kernel of the call
     int test_stall;   // MKA_FLAG_TEST_STALL (tensor-core path): the dK/dV kernel's loader leaves out its last query tile
 };
 cudaError_t launch_bwd_simt(const BwdParams& p, int dtype, cudaStream_t st);

@@ -9,12 +9,13 @@
 //   O = sum_c lam_{l(c)} 2^{m_c-M} acc_c / sum_c lam_{l(c)} 2^{m_c-M} z_c.
 #include <mutex>
 
-#include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace mka {
 namespace {
 
 constexpr int kWarps = 8;
+constexpr int kMaxCluster = 8;   // CTAs of a cluster (the portable limit)
 constexpr int kUnroll = 8;   // independent 16-byte loads in flight per lane, per stream (K and V)
 
 __device__ __forceinline__ uint4 ld_stream(const void* p) {
@@ -30,6 +31,42 @@ __device__ __forceinline__ void unpack8(const uint4& u, float (&x)[8]) {
     for (int i = 0; i < 4; ++i) {
         x[2 * i] = __uint_as_float(w[i] << 16);
         x[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+    }
+}
+
+// Merges the lane groups of a warp (lanes that hold the same column slice).
+template <int LPR>
+__device__ __forceinline__ void merge_groups(float& m, float& z, float (&acc)[8]) {
+#pragma unroll
+    for (int o = 16; o >= LPR; o >>= 1) {
+        const float m_o = __shfl_xor_sync(0xffffffffu, m, o);
+        const float z_o = __shfl_xor_sync(0xffffffffu, z, o);
+        const float m_n = fmaxf(m, m_o);
+        const float a = m_n > -INFINITY ? exp2f(m - m_n) : 0.f;
+        const float c = m_n > -INFINITY ? exp2f(m_o - m_n) : 0.f;
+        z = z * a + z_o * c;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float acc_o = __shfl_xor_sync(0xffffffffu, acc[i], o);
+            acc[i] = acc[i] * a + acc_o * c;
+        }
+        m = m_n;
+    }
+}
+
+// Column threadIdx.x of the CTA's warps together.
+template <int DH>
+__device__ __forceinline__ void merge_warps(const float (&sm_m)[kWarps], const float (&sm_z)[kWarps], const float (&sm_acc)[kWarps][DH], float& M,
+                                            float& Z, float& A) {
+    M = -INFINITY;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) M = fmaxf(M, sm_m[w]);
+    Z = 0.f; A = 0.f;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+        const float f = M > -INFINITY ? exp2f(sm_m[w] - M) : 0.f;
+        Z = fmaf(sm_z[w], f, Z);
+        A = fmaf(sm_acc[w][threadIdx.x], f, A);
     }
 }
 
@@ -118,22 +155,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) decode_partial_kernel(const De
         }
     }
 
-    // merge the lane groups of a warp (lanes that hold the same column slice)
-#pragma unroll
-    for (int o = 16; o >= LPR; o >>= 1) {
-        const float m_o = __shfl_xor_sync(0xffffffffu, m, o);
-        const float z_o = __shfl_xor_sync(0xffffffffu, z, o);
-        const float m_n = fmaxf(m, m_o);
-        const float a = m_n > -INFINITY ? exp2f(m - m_n) : 0.f;
-        const float c = m_n > -INFINITY ? exp2f(m_o - m_n) : 0.f;
-        z = z * a + z_o * c;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const float acc_o = __shfl_xor_sync(0xffffffffu, acc[i], o);
-            acc[i] = acc[i] * a + acc_o * c;
-        }
-        m = m_n;
-    }
+    merge_groups<LPR>(m, z, acc);
     // merge the warps of the CTA
     __shared__ float sm_m[kWarps], sm_z[kWarps], sm_acc[kWarps][DH];
     if (grp == 0) {
@@ -143,20 +165,138 @@ __global__ void __launch_bounds__(kWarps * 32, 2) decode_partial_kernel(const De
     }
     __syncthreads();
     if (threadIdx.x < DH) {
-        float M = -INFINITY;
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) M = fmaxf(M, sm_m[w]);
-        float Z = 0.f, A = 0.f;
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) {
-            const float f = M > -INFINITY ? exp2f(sm_m[w] - M) : 0.f;
-            Z = fmaf(sm_z[w], f, Z);
-            A = fmaf(sm_acc[w][threadIdx.x], f, A);
-        }
+        float M, Z, A;
+        merge_warps<DH>(sm_m, sm_z, sm_acc, M, Z, A);
         float* out = p.partial + (long long)blockIdx.x * (DH + 2);
         out[2 + threadIdx.x] = A;
         if (threadIdx.x == 0) { out[0] = M; out[1] = Z; }
     }
+}
+
+// Short caches: ONE kernel.  The CTAs of a cluster share a (batch, head); the slabs of its three levels are dealt over all of
+// their warps, the gate enters as log2(gate) in the exponent, and the CTAs' (max, sum, accumulator) meet in distributed
+// shared memory.  A split into chunks has nothing to gain there, and the second kernel costs a launch and its latency: one
+// sequence with 32 heads and 512 + 1000 + 64 rows took 12.1 us in two kernels, 9.7 here.
+template <int DH>
+__global__ void __launch_bounds__(kWarps * 32, 2) decode_cluster_kernel(const DecodeParams p) {
+    constexpr int LPR = DH / 8, RPI = 32 / LPR, SLAB = RPI * kUnroll;
+    __shared__ float sm_m[kWarps], sm_z[kWarps], sm_acc[kWarps][DH];
+    __shared__ float cta_m, cta_z, cta_acc[DH];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int sub = lane % LPR, grp = lane / LPR;
+    int rank, size;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(size));
+    const long long bh = blockIdx.x / size;
+    const int b = (int)(bh / p.H), h = (int)(bh % p.H);
+    float q[8];
+    {
+        const uint4 u = *reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(p.q) + bh * DH + sub * 8);
+        unpack8(u, q);
+        const float c = p.scale * kLog2e;     // scores in the base-2 domain
+#pragma unroll
+        for (int i = 0; i < 8; ++i) q[i] *= c;
+    }
+    float lam[3];
+    long long end[3];                         // slabs of the levels, running total
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+        lam[l] = p.gate[b * 3 + l];
+        end[l] = (l ? end[l - 1] : 0) + (p.L[l].n + SLAB - 1) / SLAB;
+    }
+    float m = -INFINITY, z = 0.f, acc[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] = 0.f;
+    for (long long slab = (long long)warp * size + rank; slab < end[2]; slab += (long long)kWarps * size) {
+        const int l = slab < end[0] ? 0 : (slab < end[1] ? 1 : 2);
+        const float g = l == 0 ? lam[0] : (l == 1 ? lam[1] : lam[2]);
+        if (!(g > 0.f)) continue;                          // hard routing switched this level off: do not read it
+        const LevelDev& L = l == 0 ? p.L[0] : (l == 1 ? p.L[1] : p.L[2]);
+        const long long r0 = (slab - (l == 0 ? 0 : (l == 1 ? end[0] : end[1]))) * SLAB;
+        const long long base = b * L.sb + (h / p.kv_group) * L.sh + sub * 8;
+        const __nv_bfloat16* Kp = static_cast<const __nv_bfloat16*>(L.k) + base;
+        const __nv_bfloat16* Vp = static_cast<const __nv_bfloat16*>(L.v) + base;
+        uint4 kk[kUnroll], vv[kUnroll];
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+            const long long r = r0 + u * RPI + grp;
+            kk[u] = ld_stream(Kp + (r < L.n ? r : L.n - 1) * L.sn);        // a tail lane re-reads the last row
+        }
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+            const long long r = r0 + u * RPI + grp;
+            vv[u] = ld_stream(Vp + (r < L.n ? r : L.n - 1) * L.sn);
+        }
+        const float bias = log2f(g);
+        float s[kUnroll], smax = -INFINITY;
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+            float x[8];
+            unpack8(kk[u], x);
+            float d0 = 0.f;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) d0 = fmaf(q[i], x[i], d0);
+#pragma unroll
+            for (int o = LPR / 2; o > 0; o >>= 1) d0 += __shfl_xor_sync(0xffffffffu, d0, o);
+            s[u] = r0 + u * RPI + grp < L.n ? d0 + bias : -INFINITY;
+            smax = fmaxf(smax, s[u]);
+        }
+        const float m_new = fmaxf(m, smax);
+        if (m_new > -INFINITY) {
+            const float resc = exp2f(m - m_new);             // m = -inf gives 0
+            z *= resc;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) acc[i] *= resc;
+#pragma unroll
+            for (int u = 0; u < kUnroll; ++u) {
+                const float e = exp2f(s[u] - m_new);         // masked rows: exp2(-inf) = 0
+                z += e;
+                float x[8];
+                unpack8(vv[u], x);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc[i] = fmaf(e, x[i], acc[i]);
+            }
+            m = m_new;
+        }
+    }
+    merge_groups<LPR>(m, z, acc);
+    if (grp == 0) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) sm_acc[warp][sub * 8 + i] = acc[i];
+        if (sub == 0) { sm_m[warp] = m; sm_z[warp] = z; }
+    }
+    __syncthreads();
+    if (threadIdx.x < DH) {
+        float M, Z, A;
+        merge_warps<DH>(sm_m, sm_z, sm_acc, M, Z, A);
+        cta_acc[threadIdx.x] = A;
+        if (threadIdx.x == 0) { cta_m = M; cta_z = Z; }
+    }
+    cluster_sync();
+    // every CTA finishes its share of the columns; the second barrier keeps its shared memory alive for the others
+    const int per = (DH + size - 1) / size, c = rank * per + (int)threadIdx.x;
+    if ((int)threadIdx.x < per && c < DH) {
+        float M = -INFINITY, Z = 0.f, A = 0.f;
+        float mi[kMaxCluster];
+#pragma unroll
+        for (int i = 0; i < kMaxCluster; ++i) {
+            mi[i] = i < size ? ld_cluster(smem_u32(&cta_m), i) : -INFINITY;
+            M = fmaxf(M, mi[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < kMaxCluster; ++i) {
+            if (i >= size) break;
+            const float f = M > -INFINITY ? exp2f(mi[i] - M) : 0.f;
+            Z = fmaf(ld_cluster(smem_u32(&cta_z), i), f, Z);
+            A = fmaf(ld_cluster(smem_u32(&cta_acc[c]), i), f, A);
+        }
+        static_cast<__nv_bfloat16*>(p.O)[bh * DH + c] = __float2bfloat16_rn(Z > 0.f ? A / Z : 0.f);
+        if (c == 0) {
+            if (p.LSE) p.LSE[bh] = Z > 0.f ? (M + log2f(Z)) * kLn2 : -INFINITY;
+            if (p.status && bh == 0) *p.status = MKA_OK;
+        }
+    }
+    cluster_sync();
 }
 
 template <int DH>
@@ -224,13 +364,38 @@ __global__ void __launch_bounds__(DH) decode_combine_kernel(const DecodeParams p
     for (int w = 0; w < DH / 32; ++w) Z += sz[w];
     __nv_bfloat16* O = static_cast<__nv_bfloat16*>(p.O) + bh * DH;
     O[tid] = __float2bfloat16_rn(Z > 0.f ? A / Z : 0.f);
+    if (p.status && bh == 0 && tid == 0) *p.status = MKA_OK;
     if (p.LSE && tid == 0) p.LSE[bh] = Z > 0.f ? (M + log2f(Z)) * kLn2 : -INFINITY;
+}
+
+// CTAs per (batch, head) of the one-kernel form, 0 = the split form.  As many as keep all clusters resident at once (296 CTAs);
+// more only add rounds.  Long lists stay with the split form, whose chunks fill the last round, and so do middling ones
+// where the clusters would leave a third of the slots empty.  Split form / clusters of 1 / 2 / 4 / 8 in us, chosen in brackets:
+//   32 pairs x 1576 rows, d = 128    12.1 / 27.4 / 16.5 / 11.8 / [9.7]     128 pairs x 1576 rows    28.2 / 30.6 / [22.4] / 26.5 / 35.4
+//   32 pairs x 7548 rows             32.9 / 118 / 62 / 35.0 / [25.9]       64 pairs x 16,096 rows   90.2 / 237 / 128 / [86.8] / 90.7
+//   512 pairs x 772 rows             44.2 / [41.3] / 49.1 / 62.3 / 96.4    256 pairs x 4524 rows    100.7 / [97.5] / 101 / 107 / 128
+int cluster_rule(const DecodeParams& p) {
+    const long long rows = p.L[0].n + p.L[1].n + p.L[2].n, bh = (long long)p.B * p.H;
+    int size = 1;
+    while (size < kMaxCluster && bh * size * 2 <= 296) size *= 2;
+    const long long per_cta = rows / size;
+    if (bh * size > 0x7fffffffLL || per_cta > 4096 || (per_cta > 2048 && bh * size < 192)) return 0;
+    return size;
 }
 
 template <int DH>
 cudaError_t launch_t(const DecodeParams& p, cudaStream_t st) {
     const long long bh = (long long)p.B * p.H;
     if (bh == 0) return cudaSuccess;
+    if (const int size = cluster_rule(p)) {
+        cudaLaunchAttribute at;
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = size; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(bh * size)); cfg.blockDim = dim3(kWarps * 32); cfg.stream = st;
+        cfg.attrs = &at; cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, decode_cluster_kernel<DH>, p);
+    }
     if (p.total_chunks > 0) {
         decode_partial_kernel<DH><<<(unsigned)(bh * p.total_chunks), kWarps * 32, 0, st>>>(p);
         cudaError_t e = cudaGetLastError();
@@ -347,6 +512,7 @@ extern "C" mka_status mka_decode_static(const mka_shape* s, const void* q, const
     // Nothing in the array has to start at zero: the partial kernel writes every slot that the combine
     // kernel of the same call reads, so whatever an earlier call left behind is never looked at.
     p.partial = scratch;
+    p.status = nullptr;
     cudaError_t e = launch_decode(p, static_cast<cudaStream_t>(stream));
     if (e == cudaErrorNotSupported) return MKA_ERR_UNSUPPORTED;
     return e == cudaSuccess ? MKA_OK : MKA_ERR_CUDA;

@@ -27,6 +27,7 @@ __global__ void __launch_bounds__(kSimtThreads) fwd_simt_kernel(const FwdParams 
     const T* Q = static_cast<const T*>(p.Q) + (((long long)b * p.H + h) * p.T) * DH;
     T* O = static_cast<T*>(p.O) + (((long long)b * p.H + h) * p.T) * DH;
 
+    if (p.status && threadIdx.x == 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) *p.status = MKA_OK;
     for (int i = threadIdx.x * 4; i < kSimtRows * DH; i += kSimtThreads * 4) {
         const long long t = t0 + i / DH;
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);

@@ -116,24 +116,6 @@ struct Cfg {
 constexpr int kMaxQ = 2;
 constexpr int kMaxSplit = 8;              // CTAs of a cluster (the portable limit)
 
-// Value at shared-memory address `addr` (of this CTA's layout) in CTA `rank` of the cluster.
-__device__ __forceinline__ float ld_cluster(uint32_t addr, int rank) {
-    uint32_t remote;
-    float v;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(remote) : "memory");
-    return v;
-}
-__device__ __forceinline__ float4 ld_cluster4(uint32_t addr, int rank) {
-    uint32_t remote;
-    float4 v;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(remote) : "memory");
-    return v;
-}
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
-}
 
 struct Barriers {
     uint64_t q_full;

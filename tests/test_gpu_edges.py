@@ -128,3 +128,27 @@ def test_recall_codes_batches(mka, orc, d, bits, pages, H_kv, page):
     proj = torch.randn(bits, d, generator=g).cuda()
     codes = mka.mka_l3_index(pool, proj)
     assert np.array_equal(codes.cpu().numpy().view(np.uint32), orc.l3_index(pool.float().cpu().numpy(), proj.cpu().numpy()))
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("B,H,N", [
+    (1, 1, (1, 1, 0)),                 # eight CTAs, two rows
+    (1, 3, (17, 300, 31)),             # slabs that are not full, levels that end inside a round
+    (1, 3, (100, 16500, 200)),         # clusters of eight with about 2100 rows a CTA: the split form
+    (3, 40, (600, 40, 33)),            # clusters of two
+    (2, 150, (130, 0, 5)),             # one CTA a pair, more CTAs than fit at once
+])
+def test_decode_one_kernel_or_two(mka, orc, d, B, H, N):
+    P = problem(37, B, H, 1, d, N, 64, torch.bfloat16, router_std=0.5)
+    q = P["Q"][:, :, 0].contiguous()
+    shape = mka.make_shape(B, H, 1, d, 64)
+    for route in (mka.binding.MKA_ROUTE_SOFT, mka.binding.MKA_ROUTE_TOP1):      # TOP1: levels that are not read
+        gate = mka.mka_router(P["X"], P["W_r"], None, route=route).view(B, 3)
+        ws = torch.full((mka.mka_workspace_bytes(shape, N, mka.binding.MKA_WS_DECODE),), 255, dtype=torch.uint8, device="cuda")
+        O, LSE = mka.mka_decode(shape, q, P["K"], P["V"], gate, ws=ws)
+        assert mka.mka_device_status(ws) == 0
+        Or, Lr = orc.fwd(P["Q"], P["K"], P["V"], np64(gate).reshape(B, 1, 3), 1, decode=True)
+        check(O, Or[:, :, 0], torch.bfloat16, "O")
+        finite = np.isfinite(Lr[:, :, 0])
+        assert np.array_equal(np.isfinite(np64(LSE)), finite)
+        assert not finite.any() or np.abs(np64(LSE)[finite] - Lr[:, :, 0][finite]).max() <= 1e-4
