@@ -201,112 +201,175 @@ struct L3RetrieveParams {
     int* rows;                    // [B] or null: n_sel * page_rows
     long long bank_stride;
     int B, H, H_kv, d, bits, R, page_rows, max_bank;
+    int stage_proj;               // the projection is staged in shared memory (it fits beside the scores and is 16-byte aligned)
 };
 
 constexpr int kRetThreads = 1024;
-constexpr int kMaxR = 64;
-constexpr unsigned short kTaken = 0xffffu;
+constexpr int kRetWarps = kRetThreads / 32;
 
-// dynamic shared memory: unsigned short score[max_bank]
+// Sum of v over the CTA, the same in every thread; `part` is reused by the next call but one.
+__device__ __forceinline__ int cta_sum(int v, int* part, int warp, int lane) {
+    v = __reduce_add_sync(0xffffffffu, v);
+    if (lane == 0) part[warp] = v;
+    __syncthreads();
+    return __reduce_add_sync(0xffffffffu, part[lane]);
+}
+
+// One CTA per (sequence, KV head).  Everything here is latency: the code words of the bank are asked for before the query's
+// code is worked out, and the R best are not picked one after the other (a pass over the bank and two barriers each, 28 us
+// for 8 of 8192 chunks) but cut off at once: a binary search over the score finds the R-th best, one pass in bank order
+// counts what each group of 32 chunks contributes, and a scan of those counts tells every recalled chunk its place in
+// the list.  15 us now.
+// Dynamic shared memory: unsigned short score[max_bank], int before[max_bank / 32 rounded up to whole CTAs], the projection.
 __global__ void __launch_bounds__(kRetThreads) l3_retrieve_kernel(const L3RetrieveParams p) {
     extern __shared__ __align__(16) unsigned short score[];
-    __shared__ float qs[256];
+    __shared__ __align__(16) float qs[256];
     __shared__ unsigned int qcode[8];
-    __shared__ unsigned long long red[kRetThreads / 32];
-    __shared__ int sel[kMaxR];
+    __shared__ int part[2][kRetWarps];
+    int* before = reinterpret_cast<int*>(score + (p.max_bank + 7) / 8 * 8);
+    float* projs = reinterpret_cast<float*>(before + (p.max_bank + kRetThreads - 1) / kRetThreads * kRetWarps);   // [bits][d + 4]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = blockIdx.x / p.H_kv, kvh = blockIdx.x % p.H_kv;
     const int G = p.H / p.H_kv, words = p.bits / 32;
+    int n = p.bank_len[b];
+    n = n < 0 ? 0 : (n > p.max_bank ? p.max_bank : n);
+    const int* bank = p.bank + (long long)b * p.bank_stride;
+    // 64-bit codes: the first eight chunks of a thread, page numbers first, then all code words
+    constexpr int kAhead = 8;
+    uint2 ahead[kAhead];
+    if (words == 2) {
+        int page[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const int c = tid + u * kRetThreads;
+            page[u] = c < n ? bank[c] : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u)
+            ahead[u] = page[u] >= 0 ? __ldg(reinterpret_cast<const uint2*>(p.codes + ((long long)page[u] * p.H_kv + kvh) * 2)) : make_uint2(0u, 0u);
+    }
+    // the projection, where there is room for it: its rows are read by one thread each, four columns at a time
+    const int pitch = p.d + 4;
+    if (p.stage_proj)
+        for (int e = tid * 4; e < p.bits * p.d; e += kRetThreads * 4)
+            *reinterpret_cast<float4*>(projs + (e / p.d) * pitch + e % p.d) = __ldg(reinterpret_cast<const float4*>(p.proj + e));
     // query of the KV head: the group's heads summed in head order, fp32
     if (tid < p.d) {
         const __nv_bfloat16* q0 = p.q + ((long long)b * p.H + (long long)kvh * G) * p.d + tid;
         float acc = 0.f;
-        for (int g = 0; g < G; ++g) acc = acc + __bfloat162float(q0[(long long)g * p.d]);
+        for (int g0 = 0; g0 < G; g0 += 8) {
+            float x[8];
+#pragma unroll
+            for (int g = 0; g < 8; ++g) x[g] = g0 + g < G ? __bfloat162float(q0[(long long)(g0 + g) * p.d]) : 0.f;
+#pragma unroll
+            for (int g = 0; g < 8; ++g)
+                if (g0 + g < G) acc = acc + x[g];
+        }
         qs[tid] = acc;
     }
-    if (tid < 8) qcode[tid] = 0u;
     __syncthreads();
-    if (tid < p.bits) {
+    if (tid < p.bits) {                                        // whole warps: bits is a multiple of 32
         const float* pr = p.proj + (long long)tid * p.d;
         float acc = 0.f;
-        for (int i = 0; i < p.d; ++i) acc = fmaf(pr[i], qs[i], acc);
-        if (acc >= 0.f) atomicOr(&qcode[tid >> 5], 1u << (tid & 31));
+        if (p.stage_proj) {
+#pragma unroll 8
+            for (int i = 0; i < p.d; i += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(projs + tid * pitch + i), x = *reinterpret_cast<const float4*>(qs + i);
+                acc = fmaf(v.x, x.x, acc); acc = fmaf(v.y, x.y, acc); acc = fmaf(v.z, x.z, acc); acc = fmaf(v.w, x.w, acc);
+            }
+        } else {
+            for (int i = 0; i < p.d; ++i) acc = fmaf(pr[i], qs[i], acc);
+        }
+        const unsigned int word = __ballot_sync(0xffffffffu, acc >= 0.f);
+        if (lane == 0) qcode[warp] = word;
     }
     __syncthreads();
-    int n = p.bank_len[b];
-    n = n < 0 ? 0 : (n > p.max_bank ? p.max_bank : n);
-    const int* bank = p.bank + (long long)b * p.bank_stride;
-    // eight chunks per thread at a time: the page numbers first, then all their code words, so that the two dependent
-    // gathers cost two round trips per eight chunks and not two per chunk
-    for (int c0 = tid; c0 < n; c0 += 8 * kRetThreads) {
-        int page[8];
+    // agreement of every chunk's code with the query's: 0..bits (<= 256)
+    if (words == 2) {
+        const unsigned int q0 = qcode[0], q1 = qcode[1];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const int c = tid + u * kRetThreads;
+            if (c < n) score[c] = (unsigned short)(p.bits - __popc(ahead[u].x ^ q0) - __popc(ahead[u].y ^ q1));
+        }
+    }
+    for (int c0 = tid + (words == 2 ? kAhead * kRetThreads : 0); c0 < n; c0 += 8 * kRetThreads) {
+        int page[8], dist[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int c = c0 + u * kRetThreads;
             page[u] = c < n ? bank[c] : 0;
+            dist[u] = 0;
         }
-        if (words == 2) {                                      // 64-bit codes: one 8-byte load per chunk
-            uint2 w[8];
+        for (int w = 0; w < words; ++w)
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
-                w[u] = __ldg(reinterpret_cast<const uint2*>(p.codes + ((long long)page[u] * p.H_kv + kvh) * 2));
+            for (int u = 0; u < 8; ++u) dist[u] += __popc(__ldg(p.codes + ((long long)page[u] * p.H_kv + kvh) * words + w) ^ qcode[w]);
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int c = c0 + u * kRetThreads;
-                if (c < n) score[c] = (unsigned short)(p.bits - __popc(w[u].x ^ qcode[0]) - __popc(w[u].y ^ qcode[1]));
-            }
-        } else {
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int c = c0 + u * kRetThreads;
-                if (c >= n) continue;
-                const unsigned int* code = p.codes + ((long long)page[u] * p.H_kv + kvh) * words;
-                int dist = 0;
-                for (int w = 0; w < words; ++w) dist += __popc(__ldg(code + w) ^ qcode[w]);
-                score[c] = (unsigned short)(p.bits - dist);    // agreement: 0..bits (<= 256)
-            }
+        for (int u = 0; u < 8; ++u) {
+            const int c = c0 + u * kRetThreads;
+            if (c < n) score[c] = (unsigned short)(p.bits - dist[u]);
         }
+    }
+    // (a thread reads back only the scores it wrote, up to the barriers below)
+    const int k = p.R < n ? p.R : n;
+    const int rounds = (n + kRetThreads - 1) / kRetThreads;
+    // the largest score t that at least k chunks reach: all above it are recalled, and the earliest of those at it
+    int lo = 0, hi = p.bits + 1, above = 0, flip = 0;          // at least k chunks reach lo, fewer (above) reach hi
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) / 2;
+        int mine = 0;
+        for (int r = 0; r < rounds; ++r) {
+            const int c = r * kRetThreads + tid;
+            mine += c < n && score[c] >= mid ? 1 : 0;
+        }
+        const int reach = cta_sum(mine, part[flip ^= 1], warp, lane);
+        if (reach >= k) lo = mid;
+        else { hi = mid; above = reach; }
+    }
+    const int at_cut = k - above;                              // how many of the chunks with score lo are recalled
+    // per group of 32 chunks, in bank order: chunks above the cut (low half) and at it (high half)
+    for (int r = 0; r < rounds; ++r) {
+        const int c = r * kRetThreads + tid;
+        const int sc = c < n ? score[c] : -1;
+        const unsigned int gt = __ballot_sync(0xffffffffu, sc > lo), eq = __ballot_sync(0xffffffffu, sc == lo);
+        if (lane == 0) before[r * kRetWarps + warp] = __popc(gt) | (__popc(eq) << 16);
     }
     __syncthreads();
-    const int k = p.R < n ? p.R : n;
-    for (int r = 0; r < k; ++r) {
-        // key = agreement in the high half, inverted position in the low half: the maximum is the best score, earliest chunk
-        unsigned long long best = 0ull;
-        for (int c = tid; c < n; c += kRetThreads) {
-            const unsigned short sc = score[c];
-            if (sc == kTaken) continue;
-            const unsigned long long key = ((unsigned long long)(sc + 1u) << 32) | (unsigned)(0x7fffffff - c);
-            best = key > best ? key : best;
-        }
+    // what comes before each group (fewer than 64 above the cut; at it: saturated at k): a warp scans the groups of one round,
+    // then every warp adds up the rounds before its own
+    __shared__ int total_gt[96], total_eq[96];                 // (at most 96 rounds: 98304 chunks)
+    for (int r = warp; r < rounds; r += kRetWarps) {
+        const int v = before[r * kRetWarps + lane];
+        int gt = v & 0xffff, eq = v >> 16;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
-            best = other > best ? other : best;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int g = __shfl_up_sync(0xffffffffu, gt, o), e = __shfl_up_sync(0xffffffffu, eq, o);
+            if (lane >= o) { gt += g; eq += e; }
         }
-        if (lane == 0) red[warp] = best;
-        __syncthreads();
-        if (tid == 0) {
-            unsigned long long m = red[0];
-            for (int w = 1; w < kRetThreads / 32; ++w) m = red[w] > m ? red[w] : m;
-            const int c = 0x7fffffff - (int)(m & 0xffffffffu);
-            sel[r] = c;
-            score[c] = kTaken;
-        }
-        __syncthreads();
+        if (lane == 31) { total_gt[r] = gt; total_eq[r] = eq; }
+        const int eq_before = eq - (v >> 16);
+        before[r * kRetWarps + lane] = (gt - (v & 0xffff)) | ((eq_before < k ? eq_before : k) << 16);
     }
-    if (tid == 0) {
-        for (int i = 1; i < k; ++i) {                           // bank (time) order
-            const int v = sel[i];
-            int j = i - 1;
-            while (j >= 0 && sel[j] > v) { sel[j + 1] = sel[j]; --j; }
-            sel[j + 1] = v;
-        }
-        int* out = p.table + ((long long)b * p.H_kv + kvh) * p.R;
-        for (int i = 0; i < p.R; ++i) out[i] = i < k ? bank[sel[i]] : 0;
-        if (kvh == 0) {
-            if (p.n_sel) p.n_sel[b] = k;
-            if (p.rows) p.rows[b] = k * p.page_rows;
-        }
+    __syncthreads();
+    int* out = p.table + ((long long)b * p.H_kv + kvh) * p.R;
+    int run_gt = 0, run_eq = 0;
+    for (int r = 0; r < rounds; ++r) {
+        const int c = r * kRetThreads + tid;
+        const int sc = c < n ? score[c] : -1;
+        const unsigned int gt = __ballot_sync(0xffffffffu, sc > lo), eq = __ballot_sync(0xffffffffu, sc == lo);
+        const int round_gt = run_gt, round_eq = run_eq;
+        run_gt += total_gt[r];
+        run_eq += total_eq[r];
+        if (sc < lo) continue;
+        const unsigned int below = (1u << lane) - 1u;
+        const int v = before[r * kRetWarps + warp];
+        const int gt_before = round_gt + (v & 0xffff) + __popc(gt & below), eq_before = round_eq + (v >> 16) + __popc(eq & below);
+        if (sc > lo || eq_before < at_cut) out[gt_before + (eq_before < at_cut ? eq_before : at_cut)] = bank[c];   // bank (time) order
+    }
+    for (int i = k + tid; i < p.R; i += kRetThreads) out[i] = 0;
+    if (tid == 0 && kvh == 0) {
+        if (p.n_sel) p.n_sel[b] = k;
+        if (p.rows) p.rows[b] = k * p.page_rows;
     }
 }
 
@@ -341,7 +404,11 @@ cudaError_t launch_l3_retrieve(const void* q, int B, int H, int H_kv, int d, con
     p.q = static_cast<const __nv_bfloat16*>(q); p.proj = proj; p.codes = codes; p.bank = bank; p.bank_len = bank_len;
     p.table = table; p.n_sel = n_sel; p.rows = rows; p.bank_stride = bank_stride;
     p.B = B; p.H = H; p.H_kv = H_kv; p.d = d; p.bits = bits; p.R = R; p.page_rows = page_rows; p.max_bank = max_bank;
-    const size_t smem = ((size_t)(max_bank > 0 ? max_bank : 1) * sizeof(unsigned short) + 15) / 16 * 16;
+    size_t smem = ((size_t)max_bank + 7) / 8 * 8 * sizeof(unsigned short) +
+                  ((size_t)max_bank + kRetThreads - 1) / kRetThreads * kRetWarps * sizeof(int) + 16;
+    const size_t with_proj = smem + (size_t)bits * (d + 4) * sizeof(float);
+    p.stage_proj = with_proj <= 220 * 1024 && (reinterpret_cast<uintptr_t>(proj) & 15) == 0;
+    if (p.stage_proj) smem = with_proj;
     cudaError_t e = cudaFuncSetAttribute(l3_retrieve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     l3_retrieve_kernel<<<(unsigned)(B * H_kv), kRetThreads, smem, st>>>(p);

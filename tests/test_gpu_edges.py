@@ -152,3 +152,32 @@ def test_decode_one_kernel_or_two(mka, orc, d, B, H, N):
         finite = np.isfinite(Lr[:, :, 0])
         assert np.array_equal(np.isfinite(np64(LSE)), finite)
         assert not finite.any() or np.abs(np64(LSE)[finite] - Lr[:, :, 0][finite]).max() <= 1e-4
+
+
+@pytest.mark.parametrize("bits,n,R", [(32, 1, 8), (64, 31, 64), (64, 8191, 8), (64, 8193, 16), (128, 1025, 7), (256, 2050, 64), (32, 9000, 64)])
+def test_recall_lists(mka, orc, bits, n, R):
+    """Recall lists: fewer chunks than asked for, banks around a thread's chunks, few code bits (long runs of ties), a sequence with no bank."""
+    B, H, H_kv, d = 3, 6, 2, 64
+    g = torch.Generator().manual_seed(bits + n)
+    q = torch.randn(B, H, d, generator=g).bfloat16().cuda()
+    proj = torch.randn(bits, d, generator=g).cuda()
+    pages = n + 5
+    codes = torch.randint(-2**31, 2**31, (pages, H_kv, bits // 32), generator=g, dtype=torch.int64).to(torch.int32).cuda()
+    bank = torch.stack([torch.randperm(pages, generator=g)[:n] for _ in range(B)]).to(torch.int32).cuda()
+    lens = torch.tensor([n, max(1, n // 3), 0], dtype=torch.int32).cuda()
+    for pj in (proj, torch.cat([proj.new_zeros(1), proj.flatten()])[1:].view(bits, d)):          # and a projection that allows no 16-byte load
+        table, n_sel, rows = mka.mka_l3_retrieve(q, H_kv, pj, codes, bank, lens, R, 16)
+        words = codes.cpu().numpy().view(np.uint32)
+        for b in range(B):
+            m = int(lens[b])
+            k = min(R, m)
+            assert int(n_sel[b]) == k and int(rows[b]) == 16 * k
+            for h in range(H_kv):
+                qsum = orc.sum_rows_f32(q[b, h * 3:(h + 1) * 3].float().cpu().numpy())
+                qc = orc.srp_code(qsum, proj.cpu().numpy())
+                own = bank[b, :m].cpu().numpy()
+                agree = bits - np.array([sum(bin(int(a ^ c)).count("1") for a, c in zip(words[pg, h], qc)) for pg in own], dtype=np.int64)
+                best = sorted(sorted(range(m), key=lambda i: (-agree[i], i))[:k])
+                want = np.zeros(R, dtype=np.int64)
+                want[:k] = own[best]
+                assert np.array_equal(table[b, h].cpu().numpy(), want)
