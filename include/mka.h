@@ -162,8 +162,8 @@ mka_status mka_fwd(const mka_shape* shape, const void* Q, const mka_level L[3], 
 
 /*
  * Split-KV single-token decode: Eq. 5 for T == 1 where EVERY cached row of every level is visible
- * (window and q_offset are ignored).  Each chunk of the split table produces an un-gated partial
- * (max, sum, accumulator); a second kernel combines them with the gate in log-sum-exp form.
+ * (window and q_offset are ignored).  Short caches are finished by one kernel; otherwise each chunk of the split table produces
+ * an un-gated partial (max, sum, accumulator) and a second kernel combines them with the gate in log-sum-exp form.
  *   q [B, H, d];  gate [B, 3] f32;  O [B, H, d];  LSE [B, H] f32 or NULL.
  * With shape->kv_heads < H (at most 16 query heads per KV head) the grouped-query kernel of mka_decode_paged runs on the
  * dense levels and reads every cached row once per KV head; ask mka_workspace_bytes with the same shape.
@@ -195,8 +195,9 @@ typedef struct mka_paged_level {
  * (head h reads KV head h / (H / H_kv)); H must be a multiple of H_kv with at most 16 query heads per KV head.
  * Every cached row is read once per KV head.  A level whose gate is exactly 0 for a sequence is not read.
  *   q [B, H, d] bf16;  gate [B, 3] f32;  O [B, H, d] bf16;  LSE [B, H] f32 or NULL
- *   ws: mka_decode_paged_workspace_bytes(shape, H_kv, n_level) bytes, n_level[l] = L[l].n.  The levels are split into
- *       chunks of a multiple of 128 rows (at most 8192), chosen so that the grid makes few rounds of the resident CTAs
+ *   ws: mka_decode_paged_workspace_bytes(shape, H_kv, n_level) bytes, n_level[l] = L[l].n.  The rows that the sequences really
+ *       have are cut into equal shares on the device, one per resident CTA (pages under 8 rows, or more than 512
+ *       sequences: chunks of a multiple of 128 rows, chosen on the host)
  * d must be 64 or 128; pools 16-byte aligned with strides that are multiples of 8 elements.
  * Levels whose pages hold at least 8 rows (and dense levels, see mka_decode) are streamed by the copy engine: a
  * producing warp issues one tensor-map copy per page and 64-column panel, the computing warps wait on barriers for

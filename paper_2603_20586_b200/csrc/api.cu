@@ -142,6 +142,9 @@ mka_status mka_fwd_tile_range(const mka_shape* s, const int64_t n_level[3], int3
 }
 
 static mka_status paged_plan(const int64_t n_level[3], int32_t B, int32_t H_kv, mka_decode_plan_t* plan);
+static size_t paged_partial_bytes(const int64_t n_level[3], int32_t B, int32_t H, int32_t H_kv, int32_t d, const mka_decode_plan_t& plan);
+static mka_status run_decode_paged(DecodePagedParams& p, DecodeParams& c, const int64_t n_level[3], const mka_decode_plan_t& plan, void* ws,
+                                   cudaStream_t cs);
 
 // Grouped heads in the dense decode run the grouped-query kernel (every cached row read once per KV head).
 static bool decode_uses_grouped_kernel(const mka_shape* s) {
@@ -155,6 +158,7 @@ size_t mka_workspace_bytes(const mka_shape* s, const int64_t n_level[3], int32_t
         mka_decode_plan_t plan;
         if (decode_uses_grouped_kernel(s)) {
             if (paged_plan(n_level, s->B, s->kv_heads, &plan) != MKA_OK) return 0;
+            return kWsHeader + paged_partial_bytes(n_level, s->B, s->H, s->kv_heads, s->d, plan);
         } else if (mka_decode_plan(n_level, s->B, s->H, s->d, &plan) != MKA_OK) {
             return 0;
         }
@@ -245,22 +249,12 @@ mka_status mka_decode(const mka_shape* s, const void* q, const mka_level L[3], c
             pp.L[l].k = L[l].k; pp.L[l].v = L[l].v; pp.L[l].table = nullptr; pp.L[l].rows = nullptr; pp.L[l].n = L[l].n;
             pp.L[l].sp = L[l].stride_b; pp.L[l].sh = L[l].stride_h; pp.L[l].sn = L[l].stride_n;
             pp.L[l].page_shift = 40;
-            pp.n_chunks[l] = plan.n_chunks[l];
         }
         pp.q = q; pp.gate = gate; pp.B = s->B; pp.H = s->H; pp.H_kv = s->kv_heads; pp.d = s->d; pp.scale = resolve_scale(s);
-        pp.chunk_rows = plan.chunk_rows; pp.total_chunks = plan.total_chunks;
-        pp.partial = reinterpret_cast<float*>(static_cast<char*>(ws) + kWsHeader);
-        pp.status = static_cast<unsigned int*>(ws); pp.wait_limit_ns = wait_limit_ns();
         DecodeParams c;
         memset(&c, 0, sizeof(c));
         c.O = O; c.LSE = LSE; c.gate = gate; c.B = s->B; c.H = s->H; c.d = s->d;
-        c.total_chunks = plan.total_chunks; c.partial = pp.partial;
-        for (int l = 0; l < 3; ++l) c.n_chunks[l] = plan.n_chunks[l];
-        if (cudaMemsetAsync(ws, 0, 16, cs) != cudaSuccess) return MKA_ERR_CUDA;
-        cudaError_t e = launch_decode_paged(pp, cs);
-        if (e == cudaSuccess) e = launch_decode_combine(c, cs);
-        if (e == cudaErrorNotSupported) return MKA_ERR_UNSUPPORTED;
-        return e == cudaSuccess ? MKA_OK : MKA_ERR_CUDA;
+        return run_decode_paged(pp, c, n_level, plan, ws, cs);
     }
     mka_decode_plan_t plan;
     mka_decode_plan(n_level, s->B, s->H, s->d, &plan);
@@ -309,6 +303,45 @@ static mka_status paged_plan(const int64_t n_level[3], int32_t B, int32_t H_kv, 
         plan->total_chunks += plan->n_chunks[l];
     }
     return MKA_OK;
+}
+
+// Entries per query head of the copy-engine form: a count, and one partial for every share that a list can touch.  The H_kv lists
+// of one sequence are equally long, so a share (all tiles / 296, at least two) is no less than H_kv / 296 of a list.
+static int64_t dealt_slots(const int64_t n_level[3], int32_t H_kv) {
+    int64_t tiles = 0;
+    for (int l = 0; l < 3; ++l) tiles += (n_level[l] + 63) / 64;
+    const int64_t by_share = kDealCtas / H_kv + 2, by_list = tiles / 2 + 2;
+    return 1 + (by_share < by_list ? by_share : by_list);
+}
+
+// Partials' room per query head: the larger of the two forms' (which of them runs hangs on the levels' layout).
+static size_t paged_partial_bytes(const int64_t n_level[3], int32_t B, int32_t H, int32_t H_kv, int32_t d, const mka_decode_plan_t& plan) {
+    const int64_t dealt = dealt_slots(n_level, H_kv);
+    return (size_t)B * H * (size_t)(plan.total_chunks > dealt ? plan.total_chunks : dealt) * (d + 2) * sizeof(float);
+}
+
+// Chooses the form, launches it and the combine kernel.
+static mka_status run_decode_paged(DecodePagedParams& p, DecodeParams& c, const int64_t n_level[3], const mka_decode_plan_t& plan, void* ws,
+                                   cudaStream_t cs) {
+    p.chunk_rows = plan.chunk_rows; p.total_chunks = plan.total_chunks;
+    for (int l = 0; l < 3; ++l) { p.n_chunks[l] = plan.n_chunks[l]; c.n_chunks[l] = plan.n_chunks[l]; }
+    if (plan.total_chunks > 0 && decode_paged_dealt(p)) {
+        p.dealt = c.counted = 1;
+        p.total_chunks = dealt_slots(n_level, p.H_kv);
+    }
+    c.total_chunks = p.total_chunks;
+    p.partial = c.partial = reinterpret_cast<float*>(static_cast<char*>(ws) + kWsHeader);
+    p.status = static_cast<unsigned int*>(ws); p.wait_limit_ns = wait_limit_ns();
+    if (cudaMemsetAsync(ws, 0, 16, cs) != cudaSuccess) return MKA_ERR_CUDA;
+    cudaError_t e = launch_decode_paged(p, cs);
+    if (e == cudaErrorNotSupported && p.dealt) {             // a map could not be encoded: the first form takes any layout
+        p.dealt = c.counted = 0;
+        p.total_chunks = c.total_chunks = plan.total_chunks;
+        e = launch_decode_paged(p, cs);
+    }
+    if (e == cudaSuccess) e = launch_decode_combine(c, cs);
+    if (e == cudaErrorNotSupported) return MKA_ERR_UNSUPPORTED;
+    return e == cudaSuccess ? MKA_OK : MKA_ERR_CUDA;
 }
 
 mka_status mka_fwd_paged(const mka_shape* s, int32_t H_kv, const void* Q, const mka_paged_level L[3], const float* gate,
@@ -364,7 +397,7 @@ size_t mka_decode_paged_workspace_bytes(const mka_shape* s, int32_t H_kv, const 
     if (!s || !n_level || H_kv <= 0 || s->B < 0 || s->H < 0 || s->d <= 0) return 0;
     mka_decode_plan_t plan;
     if (paged_plan(n_level, s->B, H_kv, &plan) != MKA_OK) return 0;
-    return kWsHeader + round_up((size_t)s->B * s->H * plan.total_chunks * (s->d + 2) * sizeof(float), 256);
+    return kWsHeader + paged_partial_bytes(n_level, s->B, s->H, H_kv, s->d, plan);
 }
 
 mka_status mka_decode_paged(const mka_shape* s, int32_t H_kv, const void* q, const mka_paged_level L[3],
@@ -410,20 +443,10 @@ mka_status mka_decode_paged(const mka_shape* s, int32_t H_kv, const void* q, con
     if ((long long)s->B * s->H * plan.total_chunks > 0x7fffffffLL) return MKA_ERR_SHAPE;
     p.q = q; p.gate = gate;
     p.B = s->B; p.H = s->H; p.H_kv = H_kv; p.d = s->d; p.scale = resolve_scale(s);
-    p.chunk_rows = plan.chunk_rows;
-    p.total_chunks = plan.total_chunks;
-    p.partial = reinterpret_cast<float*>(static_cast<char*>(ws) + kWsHeader);
     DecodeParams c;                                    // the combine kernel of the dense decode finishes the job
     memset(&c, 0, sizeof(c));
     c.O = O; c.LSE = LSE; c.gate = gate; c.B = s->B; c.H = s->H; c.d = s->d;
-    c.total_chunks = plan.total_chunks; c.partial = p.partial;
-    for (int l = 0; l < 3; ++l) { p.n_chunks[l] = plan.n_chunks[l]; c.n_chunks[l] = plan.n_chunks[l]; }
-    cudaStream_t cs = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(ws, 0, 16, cs) != cudaSuccess) return MKA_ERR_CUDA;
-    cudaError_t e = launch_decode_paged(p, cs);
-    if (e == cudaSuccess) e = launch_decode_combine(c, cs);
-    if (e == cudaErrorNotSupported) return MKA_ERR_UNSUPPORTED;
-    return e == cudaSuccess ? MKA_OK : MKA_ERR_CUDA;
+    return run_decode_paged(p, c, n_level, plan, ws, static_cast<cudaStream_t>(stream));
 }
 
 mka_status mka_l3_index(const void* k_pool, int64_t n_pages, int32_t H_kv, int32_t page_rows, int32_t d,

@@ -103,6 +103,7 @@ struct DecodeParams {
     long long n_chunks[3];
     long long total_chunks;
     float* partial;      // [B*H, total_chunks, d+2]
+    int counted;         // combine: entry 0 of a (batch, head) holds the number of partials that follow, which carry the gate already
     unsigned int* status;   // device status word that the combine kernel sets to MKA_OK, or null (kernels before it may wait and set it)
 };
 cudaError_t launch_decode(const DecodeParams& p, cudaStream_t st);
@@ -127,9 +128,12 @@ struct DecodePagedParams {
     long long n_chunks[3];
     long long total_chunks;
     float* partial;      // [B*H, total_chunks, d+2]
+    int dealt;                         // the copy-engine form: total_chunks = entries per query head (a count, then the partials)
     unsigned int* status;              // device status word of the call's workspace (bounded waits of the copy-engine form)
     unsigned long long wait_limit_ns;
 };
+constexpr int kDealCtas = 148 * 2;     // CTAs of the copy-engine form: two per SM
+bool decode_paged_dealt(const DecodePagedParams& p);
 cudaError_t launch_decode_paged(const DecodePagedParams& p, cudaStream_t st);
 cudaError_t launch_l3_index(const void* k, long long n_pages, int H_kv, int page_rows, int d, long long sp, long long sh,
                             long long sn, const float* proj, int bits, unsigned int* codes, cudaStream_t st);

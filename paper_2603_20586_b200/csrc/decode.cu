@@ -305,16 +305,32 @@ __global__ void __launch_bounds__(DH) decode_combine_kernel(const DecodeParams p
     const int b = (int)(bh / p.H);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const float* part = p.partial + bh * p.total_chunks * (DH + 2);
-    float lam[3];
+    float lam[3] = {1.f, 1.f, 1.f};
+    long long total = p.total_chunks;
+    if (p.counted) {
+        const float count = part[0];                           // (a call whose waits ran out may not have written it)
+        total = count > 0.f ? (long long)fminf(count, (float)(p.total_chunks - 1)) : 0;
+        part += DH + 2;
+    } else {
 #pragma unroll
-    for (int l = 0; l < 3; ++l) lam[l] = p.gate[b * 3 + l];
+        for (int l = 0; l < 3; ++l) lam[l] = p.gate[b * 3 + l];
+    }
     const long long c1 = p.n_chunks[0], c2 = c1 + p.n_chunks[1];
+    // The kernel is a chain of memory round trips, so the accumulators of the first chunks are asked for along with the
+    // maxima and sums (112 heads x 20 chunks: 8.6 us with three trips one after the other, 6.3 with one).
+    constexpr int kAhead = 32;
+    float ahead[kAhead];
+    const int n_room = (int)(p.total_chunks - (p.counted ? 1 : 0)), n_ahead = total < kAhead ? (int)total : kAhead;
+#pragma unroll
+    for (int j = 0; j < kAhead; ++j) ahead[j] = j < n_room ? part[j * (DH + 2) + 2 + tid] : 0.f;
+    float m_own = -INFINITY, z_own = 0.f;                      // chunk tid's, which the weights need again
     // global maximum over the chunks that count (gate > 0 and something summed): warp shuffles, then
     // one shared-memory hop across the CTA's warps
     float M = -INFINITY;
-    for (long long c = tid; c < p.total_chunks; c += DH) {
+    for (long long c = tid; c < total; c += DH) {
         const float g = c < c1 ? lam[0] : (c < c2 ? lam[1] : lam[2]);
         const float mc = part[c * (DH + 2)], zc = part[c * (DH + 2) + 1];
+        if (c == tid) { m_own = mc; z_own = zc; }
         if (g > 0.f && zc > 0.f) M = fmaxf(M, mc);
     }
     M = warp_max(M);
@@ -330,20 +346,26 @@ __global__ void __launch_bounds__(DH) decode_combine_kernel(const DecodeParams p
     float Z = 0.f, A = 0.f;
     __shared__ float sw[DH];
     if (M > -INFINITY) {
-        for (long long c0 = 0; c0 < p.total_chunks; c0 += DH) {
+        for (long long c0 = 0; c0 < total; c0 += DH) {
             const long long c = c0 + tid;
             float w = 0.f;
-            if (c < p.total_chunks) {
+            if (c < total) {
                 const float g = c < c1 ? lam[0] : (c < c2 ? lam[1] : lam[2]);
-                const float mc = part[c * (DH + 2)], zc = part[c * (DH + 2) + 1];
+                const float mc = c0 == 0 ? m_own : part[c * (DH + 2)], zc = c0 == 0 ? z_own : part[c * (DH + 2) + 1];
                 if (g > 0.f && zc > 0.f) { w = g * exp2f(mc - M); Z = fmaf(w, zc, Z); }
             }
             __syncthreads();                                   // the previous batch has been consumed
             sw[tid] = w;
             __syncthreads();
-            const int nb = p.total_chunks - c0 < DH ? (int)(p.total_chunks - c0) : DH;
+            const int nb = total - c0 < DH ? (int)(total - c0) : DH;
             const float* col = part + c0 * (DH + 2) + 2 + tid;
             int j = 0;
+            if (c0 == 0) {
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u)
+                    if (u < n_ahead) A = fmaf(sw[u], ahead[u], A);
+                j = n_ahead;
+            }
             for (; j + 8 <= nb; j += 8) {
                 float v[8];
 #pragma unroll

@@ -1,7 +1,7 @@
 // Split-KV single-token decode of Eq. 5 over PAGED levels with grouped-query sharing of the KV heads (the serving
 // layout of the paper's inference setup: GQA models, paged KV cache for long contexts).
 //
-// One CTA = (sequence, KV head, chunk of one level).  All G = H / H_kv query heads that share the KV head ride in the
+// Two forms.  The first (any page size): one CTA = (sequence, KV head, chunk of one level).  All G = H / H_kv query heads that share the KV head ride in the
 // 16 rows of one warp-level matrix product, so every cached row is read from HBM once per KV head instead of once
 // per query head.  Rows are found through the page table (row r -> page table[r / page_rows], offset r % page_rows)
 // (the chunk's slice of the table is read into shared memory once) and brought into shared memory with 16-byte
@@ -248,12 +248,18 @@ __global__ void __launch_bounds__(kThreads, 2) decode_paged_kernel(const DecodeP
 }
 
 // ---------------------------------------------------------------------------------------------------------------
-// The same kernel fed by the copy engine.  Where every (page, KV head) block of a level is a box a tensor map can
-// describe (pages of at least 8 rows, or a dense level), a fifth warp produces: lane i owns box i of every 64-row tile
-// (a box = the rows of one page that fall into the tile), looks its page up and issues one TMA copy per 64-column
-// panel of K and of V into 128-byte-swizzled tiles (a ring of three stages, one mbarrier pair per stage).  The four
-// computing warps then issue no load instructions at all; ldmatrix reads the swizzled tiles without bank conflicts.
-// Boxes that start past the chunk's last row are aimed at the chunk's first page (finite data, weights exactly 0);
+// The same products fed by the copy engine, with the work dealt evenly.  Where every (page, KV head) block of a level is a box a
+// tensor map can describe (pages of at least 8 rows, or a dense level), a fifth warp produces: lane i owns box i of every
+// 64-row tile (a box = the rows of one page that fall into the tile), looks its page up one tile ahead and issues one TMA copy
+// per 64-column panel of K and of V into 128-byte-swizzled tiles (a ring of three stages, one mbarrier pair per
+// stage).  The four computing warps then issue no load instructions at all; ldmatrix reads the swizzled tiles without
+// bank conflicts.
+// A list = the tiles of one (sequence, KV head), level after level, as many as the sequence really has (row counts are on the device)
+// and without the levels its gate closes.  All lists laid end to end are cut into equal shares, one per resident CTA; a CTA
+// writes one partial for each list that its share touches.  The gate enters as log2(gate) in the exponent, so a partial may span levels.  Cut
+// into chunks on the host, by the upper bounds of the row counts, a mixed batch left SMs idle while others
+// worked off two full chunks: four sequences of 131072, 79953, 43253 and 114032 rows (790 MB) took 145 us; 127 now.
+// Boxes that start past a level's last row are aimed at the tile's first page (finite data, weights exactly 0);
 // value rows past the last row inside the last box are cleared in shared memory before they are read, so that
 // whatever a partly filled page holds there (NaN included) cannot reach the accumulator through 0 x NaN.
 constexpr int kTmaThreads = 160;
@@ -263,6 +269,61 @@ struct PagedMaps {
     CUtensorMap k[3], v[3];
 };
 
+// Rows of level l that sequence b's list holds: none where the gate is 0.
+__device__ __forceinline__ int list_rows(const DecodePagedParams& p, int b, int l) {
+    const PagedLevelDev& L = p.L[l];
+    if (L.n == 0 || !(p.gate[b * 3 + l] > 0.f)) return 0;
+    const long long n = L.rows ? (long long)L.rows[b] : L.n;
+    return (int)(n < 0 ? 0 : (n > L.n ? L.n : n));
+}
+
+// Walks a CTA's share of the tiles.
+struct TileWalk {
+    const DecodePagedParams& p;
+    const int* tiles;                     // tiles of a list, per sequence
+    int left;                             // tiles of the share still to come
+    int b, kvh, at;                       // list, and the next tile in it
+    int n[3];                             // rows of the list's levels
+    __device__ __forceinline__ TileWalk(const DecodePagedParams& p_, const int* tiles_, const int* before, long long u0, int share)
+        : p(p_), tiles(tiles_), left(share) {
+        // first sequence with tiles past u0 (before[b]: tiles of a list times b's predecessors; H_kv lists each)
+        int lo = 0, hi = p.B - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi) / 2;
+            if ((long long)before[mid + 1] * p.H_kv > u0) hi = mid; else lo = mid + 1;
+        }
+        b = lo;
+        const int in_seq = (int)(u0 - (long long)before[b] * p.H_kv);
+        kvh = in_seq / tiles[b]; at = in_seq - kvh * tiles[b];
+        enter();
+    }
+    __device__ __forceinline__ void enter() {
+#pragma unroll
+        for (int l = 0; l < 3; ++l) n[l] = list_rows(p, b, l);
+    }
+    __device__ __forceinline__ int segment() const { return min(left, tiles[b] - at); }      // tiles of the share in this list
+    // level and first row of tile t of the list
+    __device__ __forceinline__ void locate(int t, int& lvl, int& row0, int& rows) const {
+        const int t0 = (n[0] + kTileRows - 1) / kTileRows, t1 = (n[1] + kTileRows - 1) / kTileRows;
+        lvl = t < t0 ? 0 : (t < t0 + t1 ? 1 : 2);
+        row0 = (t - (lvl > 0 ? t0 : 0) - (lvl > 1 ? t1 : 0)) * kTileRows;
+        rows = lvl == 0 ? n[0] : (lvl == 1 ? n[1] : n[2]);
+    }
+    // past `done` tiles; false when the share is used up
+    __device__ __forceinline__ bool advance(int done) {
+        left -= done; at += done;
+        if (left <= 0) return false;
+        if (at < tiles[b]) return true;
+        at = 0;
+        if (++kvh == p.H_kv) {
+            kvh = 0;
+            do ++b; while (tiles[b] == 0);
+            enter();
+        }
+        return true;
+    }
+};
+
 template <int DH>
 __global__ void __launch_bounds__(kTmaThreads, 2) decode_paged_tma_kernel(const __grid_constant__ PagedMaps maps, const DecodePagedParams p) {
     constexpr int kPanels = DH / 64;
@@ -270,234 +331,285 @@ __global__ void __launch_bounds__(kTmaThreads, 2) decode_paged_tma_kernel(const 
     constexpr int kTileBytes = kPanels * kPanelBytes;       // one of K or V
     constexpr int KS = DH / 16;
     constexpr int NB = DH / 8;
+    constexpr int kState = NB * 4 + 4;                      // one thread's accumulators, maxima and sums
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    float* hand = reinterpret_cast<float*>(smem + kTmaStages * 2 * kTileBytes);      // [kState][32]: one warp's state on its way to warp 0
+    int* tiles = reinterpret_cast<int*>(hand + kState * 32);                         // [B]
+    int* before = tiles + p.B;                                                       // [B + 1]
     __shared__ uint64_t full[kTmaStages], empty[kTmaStages];
     __shared__ WaitCtl ctl;
-    __shared__ int s_pages[kSliceCap];
 
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-    const int g = lane >> 2, t = lane & 3;
     const int G = p.H / p.H_kv;
-    long long chunk = blockIdx.x % p.total_chunks;
-    const long long bk = blockIdx.x / p.total_chunks;
-    const int b = (int)(bk / p.H_kv), kvh = (int)(bk % p.H_kv);
-    const long long chunk_all = chunk;
-    int lvl = 0;
-    while (lvl < 2 && chunk >= p.n_chunks[lvl]) { chunk -= p.n_chunks[lvl]; ++lvl; }
-    const PagedLevelDev L = p.L[lvl];
-    long long n_b = L.rows ? (long long)L.rows[b] : L.n;
-    n_b = n_b < 0 ? 0 : (n_b > L.n ? L.n : n_b);
-    const long long r_begin = chunk * p.chunk_rows;
-    const long long r_end = r_begin + p.chunk_rows < n_b ? r_begin + p.chunk_rows : n_b;
-    const bool skip = p.gate[b * 3 + lvl] == 0.f || r_end <= r_begin;
-    float* part0 = p.partial + (((long long)b * p.H + (long long)kvh * G) * p.total_chunks + chunk_all) * (DH + 2);
-    const long long part_stride = p.total_chunks * (DH + 2);
-    if (skip) {                                                                // nothing to read: empty partials
-        for (int r = 0; r < G; ++r) {
-            float* out = part0 + r * part_stride;
-            for (int i = tid; i < DH + 2; i += kTmaThreads) out[i] = i == 0 ? -INFINITY : 0.f;
-        }
-        return;
-    }
+    const long long slot_floats = DH + 2, list_floats = p.total_chunks * slot_floats;   // entry 0 of a head: how many partials follow
     if (tid == 0) {
         ctl.abort = 0;
         ctl.limit_ns = p.wait_limit_ns;
         for (int i = 0; i < kTmaStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 4); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    const bool dense = L.table == nullptr;                  // one page per sequence: the page is the batch index
-    const int shift = L.page_shift;
-    const long long page_mask = ((long long)1 << shift) - 1;
-    const long long page0 = r_begin >> shift;
-    const int* table = dense ? nullptr : L.table + (long long)b * L.table_stride + (long long)kvh * L.table_head_stride + page0;
-    const long long n_pages = ((r_end - 1) >> shift) - page0 + 1;
-    const bool sliced = !dense && n_pages <= kSliceCap;
-    if (sliced)
-        for (int i = tid; i < (int)n_pages; i += kTmaThreads) s_pages[i] = table[i];
+    for (int b = tid; b < p.B; b += kTmaThreads) {
+        int t = 0;
+#pragma unroll
+        for (int l = 0; l < 3; ++l) t += (list_rows(p, b, l) + kTileRows - 1) / kTileRows;
+        tiles[b] = t;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        int run = 0;
+        for (int b0 = 0; b0 < p.B; b0 += 32) {
+            int t = b0 + lane < p.B ? tiles[b0 + lane] : 0;
+            const int own = t;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int x = __shfl_up_sync(0xffffffffu, t, o);
+                if (lane >= o) t += x;
+            }
+            if (b0 + lane < p.B) before[b0 + lane] = run + t - own;
+            run += __shfl_sync(0xffffffffu, t, 31);
+        }
+        if (lane == 0) before[p.B] = run;
+    }
     __syncthreads();
     volatile WaitCtl* ctlp = &ctl;
-    const long long n_tiles = (r_end - r_begin + kTileRows - 1) / kTileRows;
+    const long long all = (long long)before[p.B] * p.H_kv;
+    const int share = (int)max(2LL, (all + gridDim.x - 1) / gridDim.x);
+    const long long u0 = (long long)blockIdx.x * share;
+    if (blockIdx.x == 0)                                    // sequences without a tile have no partials
+        for (int i = tid; i < p.B * p.H; i += kTmaThreads)
+            if (tiles[i / p.H] == 0) p.partial[i * list_floats] = 0.f;
+    if (u0 >= all) return;
+    TileWalk walk(p, tiles, before, u0, (int)min((long long)share, all - u0));
 
     if (warp == 4) {
         // ------------------------------------------------------------ producer
-        const int box_rows = dense ? kTileRows : (int)(page_mask + 1 < kTileRows ? page_mask + 1 : kTileRows);
-        const int boxes = kTileRows / box_rows;
-        const bool mine = lane < boxes;
-        bool ok = true;
-        for (long long i = 0; i < n_tiles && ok; ++i) {
-            const int st = (int)(i % kTmaStages);
-            long long r0 = r_begin + i * kTileRows + (long long)lane * box_rows;
-            if (r0 >= r_end) r0 = r_begin;                  // a box with no valid row re-reads the chunk's first box
-            int page = b, in_row = (int)r0;
-            if (!dense && mine) {
-                const long long pi = (r0 >> shift) - page0;
-                page = sliced ? s_pages[pi] : table[pi];
-                in_row = (int)(r0 & page_mask);
+        struct Tile { int lvl, row0, rows, b, kvh; };
+        int seg_left = walk.segment(), t = walk.at;
+        bool more = true;
+        auto next = [&](Tile& x) -> bool {
+            if (!more) return false;
+            walk.locate(t, x.lvl, x.row0, x.rows);
+            x.b = walk.b; x.kvh = walk.kvh;
+            ++t;
+            if (--seg_left == 0) {
+                more = walk.advance(walk.segment());
+                if (more) { seg_left = walk.segment(); t = walk.at; }
             }
-            if (!mbar_wait_warp(&empty[st], ((uint32_t)(i / kTmaStages) & 1u) ^ 1u, ctlp)) { ok = false; break; }
+            return true;
+        };
+        auto box_rows_of = [&](int lvl) { return p.L[lvl].table == nullptr || p.L[lvl].page_shift > 5 ? kTileRows : 1 << p.L[lvl].page_shift; };
+        // page and row of this lane's box of a tile; a box with no valid row re-reads the tile's first box
+        auto look_up = [&](const Tile& x, int& page, int& in_row) {
+            const PagedLevelDev& L = p.L[x.lvl];
+            const int box = box_rows_of(x.lvl);
+            int r = x.row0 + lane * box;
+            if (r >= x.rows || lane >= kTileRows / box) r = x.row0;
+            page = x.b; in_row = r;
+            if (L.table != nullptr) {
+                page = L.table[(long long)x.b * L.table_stride + (long long)x.kvh * L.table_head_stride + (r >> L.page_shift)];
+                in_row = r & ((1 << L.page_shift) - 1);
+            }
+        };
+        Tile cur, nxt;
+        int page, in_row, page_n = 0, in_row_n = 0;
+        bool have = next(cur);
+        if (have) look_up(cur, page, in_row);
+        bool ok = true;
+        int issued = 0;
+        while (have) {
+            const bool have_n = next(nxt);
+            if (have_n) look_up(nxt, page_n, in_row_n);
+            const int st = issued % kTmaStages;
+            if (!mbar_wait_warp(&empty[st], ((uint32_t)(issued / kTmaStages) & 1u) ^ 1u, ctlp)) { ok = false; break; }
             if (lane == 0) mbar_expect_tx(&full[st], 2 * kTileBytes);
             __syncwarp();
-            if (mine) {
-                uint8_t* sK = smem + (size_t)st * 2 * kTileBytes + (size_t)lane * box_rows * 128;
+            const int box = box_rows_of(cur.lvl);
+            if (lane < kTileRows / box) {
+                uint8_t* sK = smem + (size_t)st * 2 * kTileBytes + (size_t)lane * box * 128;
 #pragma unroll
                 for (int pn = 0; pn < kPanels; ++pn) {
-                    tma_load_4d(sK + pn * kPanelBytes, &maps.k[lvl], pn * 64, in_row, kvh, page, &full[st]);
-                    tma_load_4d(sK + kTileBytes + pn * kPanelBytes, &maps.v[lvl], pn * 64, in_row, kvh, page, &full[st]);
+                    tma_load_4d(sK + pn * kPanelBytes, &maps.k[cur.lvl], pn * 64, in_row, cur.kvh, page, &full[st]);
+                    tma_load_4d(sK + kTileBytes + pn * kPanelBytes, &maps.v[cur.lvl], pn * 64, in_row, cur.kvh, page, &full[st]);
                 }
             }
+            ++issued;
+            cur = nxt; page = page_n; in_row = in_row_n; have = have_n;
         }
         // the shared memory must not be given up with a copy in flight: wait (bounded) for the stages still out
-        const long long issued = n_tiles;
         if (ok)
-            for (long long i = issued > kTmaStages ? issued - kTmaStages : 0; i < issued; ++i)
+            for (int i = issued > kTmaStages ? issued - kTmaStages : 0; i < issued; ++i)
                 mbar_wait_warp(&full[i % kTmaStages], (uint32_t)(i / kTmaStages) & 1u, ctlp);
         return;
     }
 
     // ---------------------------------------------------------------- computing warps
-    uint32_t qa[KS][4];
-    {
-        const __nv_bfloat16* q0 = static_cast<const __nv_bfloat16*>(p.q) + ((long long)b * p.H + (long long)kvh * G) * DH;
-#pragma unroll
-        for (int ks = 0; ks < KS; ++ks) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int row = g + (i & 1) * 8, col = 16 * ks + (i >> 1) * 8 + 2 * t;
-                qa[ks][i] = row < G ? *reinterpret_cast<const uint32_t*>(q0 + (long long)row * DH + col) : 0u;
-            }
-        }
-    }
+    const int g = lane >> 2, t4 = lane & 3;
     const float c2 = p.scale * kLog2e;
-    float m[2] = {-INFINITY, -INFINITY}, z[2] = {0.f, 0.f};
-    float o[NB][4];
-#pragma unroll
-    for (int nb = 0; nb < NB; ++nb) { o[nb][0] = o[nb][1] = o[nb][2] = o[nb][3] = 0.f; }
     const int kb = warp * 16;                               // this warp's rows of a tile
     const int mi = lane >> 3, l7 = lane & 7;
     // ldmatrix row addresses inside a 128-byte-swizzled panel: row r, 16-byte chunk c sits at r * 128 + ((c ^ (r & 7)) << 4);
     // the rows a lane addresses have r & 7 = lane & 7
     const uint32_t k_row = (uint32_t)(kb + (mi >> 1) * 8 + l7) * 128u;
     const uint32_t v_row = (uint32_t)(kb + (mi & 1) * 8 + l7) * 128u;
-    bool ok = true;
-    for (long long i = 0; i < n_tiles; ++i) {
-        const int st = (int)(i % kTmaStages);
-        ok = mbar_wait_warp(&full[st], (uint32_t)(i / kTmaStages) & 1u, ctlp);
-        if (!ok) break;
-        uint8_t* sK = smem + (size_t)st * 2 * kTileBytes;
-        uint8_t* sV = sK + kTileBytes;
-        const long long tile_base = r_begin + i * kTileRows;
-        if (tile_base + kb + 16 > r_end) {                  // clear this warp's value rows past the chunk's last row
-            const int r_first = (int)max(0LL, r_end - tile_base - kb);       // first row (of the warp's 16) to clear
-            for (int idx = lane; idx < (16 - r_first) * 8 * kPanels; idx += 32) {
-                const int row = kb + r_first + idx / (8 * kPanels), rest = idx % (8 * kPanels);
-                *reinterpret_cast<uint4*>(sV + (rest / 8) * kPanelBytes + row * 128 + (rest % 8) * 16) = make_uint4(0u, 0u, 0u, 0u);
-            }
-            __syncwarp();
-        }
-        float s[2][4];
-#pragma unroll
-        for (int nb = 0; nb < 2; ++nb) { s[nb][0] = s[nb][1] = s[nb][2] = s[nb][3] = 0.f; }
+    int done = 0;                                           // tiles of the share read so far
+    bool more = true;
+    while (more) {
+        const int b = walk.b, kvh = walk.kvh, first = walk.at, count = walk.segment();
+        uint32_t qa[KS][4];
         {
-            const uint32_t a0 = smem_addr(sK) + k_row;
+            const __nv_bfloat16* q0 = static_cast<const __nv_bfloat16*>(p.q) + ((long long)b * p.H + (long long)kvh * G) * DH;
 #pragma unroll
             for (int ks = 0; ks < KS; ++ks) {
-                const int c16 = ks * 2 + (mi & 1);          // 16-byte chunk of the row (0..15 at d = 128)
-                uint32_t r[4];
-                ldmatrix_x4(a0 + (uint32_t)((ks * 2) >> 3) * kPanelBytes + ((uint32_t)((c16 & 7) ^ l7) << 4), r);
-                mma_bf16(s[0], qa[ks], r[0], r[1]);
-                mma_bf16(s[1], qa[ks], r[2], r[3]);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int row = g + (i & 1) * 8, col = 16 * ks + (i >> 1) * 8 + 2 * t4;
+                    qa[ks][i] = row < G ? *reinterpret_cast<const uint32_t*>(q0 + (long long)row * DH + col) : 0u;
+                }
             }
         }
-        const long long row_base = tile_base + kb + 2 * t;
-        float mx[2] = {-INFINITY, -INFINITY};
+        float bias[3];
 #pragma unroll
-        for (int nb = 0; nb < 2; ++nb) {
+        for (int l = 0; l < 3; ++l) bias[l] = log2f(p.gate[b * 3 + l]);           // (a closed level has no tiles)
+        float m[2] = {-INFINITY, -INFINITY}, z[2] = {0.f, 0.f};
+        float o[NB][4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const bool in = row_base + 8 * nb + (j & 1) < r_end;
-                s[nb][j] = in ? s[nb][j] * c2 : -INFINITY;
-                mx[j >> 1] = fmaxf(mx[j >> 1], s[nb][j]);
+        for (int nb = 0; nb < NB; ++nb) { o[nb][0] = o[nb][1] = o[nb][2] = o[nb][3] = 0.f; }
+        bool ok = true;
+        for (int i = 0; i < count; ++i) {
+            const int st = (done + i) % kTmaStages;
+            ok = mbar_wait_warp(&full[st], (uint32_t)((done + i) / kTmaStages) & 1u, ctlp);
+            if (!ok) break;
+            int lvl, tile_base, rows;
+            walk.locate(first + i, lvl, tile_base, rows);
+            const float bl = pick3(bias, lvl);
+            uint8_t* sK = smem + (size_t)st * 2 * kTileBytes;
+            uint8_t* sV = sK + kTileBytes;
+            if (tile_base + kb + 16 > rows) {               // clear this warp's value rows past the level's last row
+                const int r_first = max(0, rows - tile_base - kb);               // first row (of the warp's 16) to clear
+                for (int idx = lane; idx < (16 - r_first) * 8 * kPanels; idx += 32) {
+                    const int row = kb + r_first + idx / (8 * kPanels), rest = idx % (8 * kPanels);
+                    *reinterpret_cast<uint4*>(sV + (rest / 8) * kPanelBytes + row * 128 + (rest % 8) * 16) = make_uint4(0u, 0u, 0u, 0u);
+                }
+                __syncwarp();
             }
-        }
-        uint32_t pa[4];
+            float s[2][4];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
-            mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 2));
-            const float m_new = fmaxf(m[h], mx[h]);
-            const float resc = m_new > -INFINITY ? exp2f(m[h] - m_new) : 1.f;
-            const float sub = m_new > -INFINITY ? m_new : 0.f;
-            m[h] = m_new;
-            z[h] *= resc;
+            for (int nb = 0; nb < 2; ++nb) { s[nb][0] = s[nb][1] = s[nb][2] = s[nb][3] = 0.f; }
+            {
+                const uint32_t a0 = smem_addr(sK) + k_row;
 #pragma unroll
-            for (int nb = 0; nb < NB; ++nb) { o[nb][2 * h] *= resc; o[nb][2 * h + 1] *= resc; }
-            const float p00 = exp2f(s[0][2 * h] - sub), p01 = exp2f(s[0][2 * h + 1] - sub);
-            const float p10 = exp2f(s[1][2 * h] - sub), p11 = exp2f(s[1][2 * h + 1] - sub);
-            z[h] += (p00 + p01) + (p10 + p11);
-            pa[h] = pack2(p00, p01);
-            pa[2 + h] = pack2(p10, p11);
+                for (int ks = 0; ks < KS; ++ks) {
+                    const int c16 = ks * 2 + (mi & 1);      // 16-byte chunk of the row (0..15 at d = 128)
+                    uint32_t r[4];
+                    ldmatrix_x4(a0 + (uint32_t)((ks * 2) >> 3) * kPanelBytes + ((uint32_t)((c16 & 7) ^ l7) << 4), r);
+                    mma_bf16(s[0], qa[ks], r[0], r[1]);
+                    mma_bf16(s[1], qa[ks], r[2], r[3]);
+                }
+            }
+            const int row_base = tile_base + kb + 2 * t4;
+            float mx[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+            for (int nb = 0; nb < 2; ++nb) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const bool in = row_base + 8 * nb + (j & 1) < rows;
+                    s[nb][j] = in ? fmaf(s[nb][j], c2, bl) : -INFINITY;
+                    mx[j >> 1] = fmaxf(mx[j >> 1], s[nb][j]);
+                }
+            }
+            uint32_t pa[4];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
+                mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 2));
+                const float m_new = fmaxf(m[h], mx[h]);
+                const float resc = m_new > -INFINITY ? exp2f(m[h] - m_new) : 1.f;
+                const float sub = m_new > -INFINITY ? m_new : 0.f;
+                m[h] = m_new;
+                z[h] *= resc;
+#pragma unroll
+                for (int nb = 0; nb < NB; ++nb) { o[nb][2 * h] *= resc; o[nb][2 * h + 1] *= resc; }
+                const float p00 = exp2f(s[0][2 * h] - sub), p01 = exp2f(s[0][2 * h + 1] - sub);
+                const float p10 = exp2f(s[1][2 * h] - sub), p11 = exp2f(s[1][2 * h + 1] - sub);
+                z[h] += (p00 + p01) + (p10 + p11);
+                pa[h] = pack2(p00, p01);
+                pa[2 + h] = pack2(p10, p11);
+            }
+            {
+                const uint32_t a0 = smem_addr(sV) + v_row;
+#pragma unroll
+                for (int j = 0; j < NB / 2; ++j) {
+                    const int c16 = j * 2 + (mi >> 1);
+                    uint32_t r[4];
+                    ldmatrix_x4_trans(a0 + (uint32_t)((j * 2) >> 3) * kPanelBytes + ((uint32_t)((c16 & 7) ^ l7) << 4), r);
+                    mma_bf16(o[2 * j], pa, r[0], r[1]);
+                    mma_bf16(o[2 * j + 1], pa, r[2], r[3]);
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&empty[st]);         // this warp has read the stage
         }
+        done += count;
+        // The four warps meet at a named barrier that also carries their "no wait ran out" flags.
         {
-            const uint32_t a0 = smem_addr(sV) + v_row;
-#pragma unroll
-            for (int j = 0; j < NB / 2; ++j) {
-                const int c16 = j * 2 + (mi >> 1);
-                uint32_t r[4];
-                ldmatrix_x4_trans(a0 + (uint32_t)((j * 2) >> 3) * kPanelBytes + ((uint32_t)((c16 & 7) ^ l7) << 4), r);
-                mma_bf16(o[2 * j], pa, r[0], r[1]);
-                mma_bf16(o[2 * j + 1], pa, r[2], r[3]);
+            uint32_t out;
+            asm volatile("{\n.reg .pred pi, po;\nsetp.ne.u32 pi, %1, 0;\nbar.red.and.pred po, 1, 128, pi;\nselp.u32 %0, 1, 0, po;\n}"
+                         : "=r"(out) : "r"((uint32_t)ok) : "memory");
+            if (!out) {
+                if (tid == 0 && p.status) atomicExch(p.status, (unsigned int)MKA_ERR_TIMEOUT);
+                return;
             }
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&empty[st]);             // this warp has read the stage
-    }
-    // The four warps meet at a named barrier that also carries their "no wait ran out" flags (the producer left already).
-    {
-        uint32_t out;
-        asm volatile("{\n.reg .pred pi, po;\nsetp.ne.u32 pi, %1, 0;\nbar.red.and.pred po, 1, 128, pi;\nselp.u32 %0, 1, 0, po;\n}"
-                     : "=r"(out) : "r"((uint32_t)ok) : "memory");
-        if (!out) {
-            if (tid == 0 && p.status) atomicExch(p.status, (unsigned int)MKA_ERR_TIMEOUT);
-            return;
+        // Warp 0 adds up the four warps' states, one after the other through a warp's worth of shared memory (the ring belongs
+        // to the producer, who is ahead): the threads of every warp hold the same elements.
+#pragma unroll 1
+        for (int w = 1; w < 4; ++w) {
+            if (warp == w) {
+#pragma unroll
+                for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) hand[(nb * 4 + j) * 32 + lane] = o[nb][j];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) { hand[(NB * 4 + h) * 32 + lane] = m[h]; hand[(NB * 4 + 2 + h) * 32 + lane] = z[h]; }
+            }
+            asm volatile("bar.sync 1, 128;" ::: "memory");
+            if (warp == 0) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float mo = hand[(NB * 4 + h) * 32 + lane], mn = fmaxf(m[h], mo);
+                    const float a = mn > -INFINITY ? exp2f(m[h] - mn) : 0.f, c = mn > -INFINITY ? exp2f(mo - mn) : 0.f;
+                    m[h] = mn;
+                    z[h] = z[h] * a + hand[(NB * 4 + 2 + h) * 32 + lane] * c;
+#pragma unroll
+                    for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) o[nb][2 * h + j] = o[nb][2 * h + j] * a + hand[(nb * 4 + 2 * h + j) * 32 + lane] * c;
+                }
+            }
+            asm volatile("bar.sync 1, 128;" ::: "memory");
         }
-    }
-    // merge the four warps: per query head (row) M, Z and the accumulator row (the tiles are done with: reuse the memory)
+        if (warp == 0) {
+            // this share is the list's partial number slot; the share with the list's first tile also says how many there are
+            const long long list0 = (long long)before[b] * p.H_kv + (long long)kvh * tiles[b];
+            const int first_share = (int)(list0 / share), slot = (int)blockIdx.x - first_share;
+            const int n_slots = (int)((list0 + tiles[b] - 1) / share) - first_share + 1;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        z[h] += __shfl_xor_sync(0xffffffffu, z[h], 1);
-        z[h] += __shfl_xor_sync(0xffffffffu, z[h], 2);
-    }
-    float* sm_o = reinterpret_cast<float*>(smem);           // [4 warps][16 rows][DH]
-    float* sm_m = sm_o + 4 * 16 * DH;                       // [4][16]
-    float* sm_z = sm_m + 4 * 16;
+            for (int h = 0; h < 2; ++h) {
+                z[h] += __shfl_xor_sync(0xffffffffu, z[h], 1);
+                z[h] += __shfl_xor_sync(0xffffffffu, z[h], 2);
+                const int row = g + 8 * h;
+                if (row >= G) continue;
+                float* head = p.partial + ((long long)b * p.H + (long long)kvh * G + row) * list_floats;
+                if (slot == 0 && t4 == 0) head[0] = (float)n_slots;
+                float* out = head + (1 + slot) * slot_floats;
+                if (t4 == 0) { out[0] = m[h]; out[1] = z[h]; }
 #pragma unroll
-    for (int nb = 0; nb < NB; ++nb) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            sm_o[((warp * 16) + g + (j >> 1) * 8) * DH + nb * 8 + 2 * t + (j & 1)] = o[nb][j];
-    }
-    if (t == 0) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) { sm_m[warp * 16 + g + 8 * h] = m[h]; sm_z[warp * 16 + g + 8 * h] = z[h]; }
-    }
-    asm volatile("bar.sync 1, 128;" ::: "memory");
-    for (int idx = tid; idx < G * DH; idx += 128) {
-        const int r = idx / DH, col = idx % DH;
-        float M = -INFINITY;
-#pragma unroll
-        for (int w = 0; w < 4; ++w) M = fmaxf(M, sm_m[w * 16 + r]);
-        float Z = 0.f, A = 0.f;
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-            const float f = M > -INFINITY ? exp2f(sm_m[w * 16 + r] - M) : 0.f;
-            Z = fmaf(sm_z[w * 16 + r], f, Z);
-            A = fmaf(sm_o[(w * 16 + r) * DH + col], f, A);
+                for (int nb = 0; nb < NB; ++nb) { out[2 + nb * 8 + 2 * t4] = o[nb][2 * h]; out[3 + nb * 8 + 2 * t4] = o[nb][2 * h + 1]; }
+            }
         }
-        float* out = part0 + r * part_stride;
-        out[2 + col] = A;
-        if (col == 0) { out[0] = M; out[1] = Z; }
+        more = walk.advance(count);
     }
 }
 
@@ -533,26 +645,11 @@ cudaError_t launch_tma(const DecodePagedParams& p, cudaStream_t st) {
     for (int l = 0; l < 3; ++l) if (p.L[l].n > 0) { first_real = l; break; }
     if (first_real < 0) return cudaSuccess;
     for (int l = 0; l < 3; ++l) if (p.L[l].n == 0) { maps.k[l] = maps.k[first_real]; maps.v[l] = maps.v[first_real]; }
-    const long long ctas = (long long)p.B * p.H_kv * p.total_chunks;
-    const size_t smem = (size_t)kTmaStages * 2 * kTileRows * DH * 2 + 1024;
+    const size_t smem = (size_t)kTmaStages * 2 * kTileRows * DH * 2 + 1024 + (DH / 8 * 4 + 4) * 32 * sizeof(float) + (2 * (size_t)p.B + 1) * sizeof(int);
     cudaError_t e = cudaFuncSetAttribute(decode_paged_tma_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    decode_paged_tma_kernel<DH><<<(unsigned)ctas, kTmaThreads, smem, st>>>(maps, p);
+    decode_paged_tma_kernel<DH><<<kDealCtas, kTmaThreads, smem, st>>>(maps, p);
     return cudaGetLastError();
-}
-
-bool tma_eligible(const DecodePagedParams& p) {
-    if (!tensor_map_encoder_available()) return false;
-    for (int l = 0; l < 3; ++l) {
-        const PagedLevelDev& L = p.L[l];
-        if (L.n == 0) continue;
-        if (L.table != nullptr && (L.page_shift < 3 || L.page_shift > 30)) return false;     // pages of 8 rows at least
-        if (L.sn <= 0 || L.sn % 8 || L.sh % 8 || L.sp % 8 || L.sp < 0) return false;
-        if (L.sp == 0 && (L.table != nullptr || p.B > 1)) return false;
-        if (p.H_kv > 1 && L.sh <= 0) return false;
-        if (L.n > 0x7fffffffLL) return false;
-    }
-    return true;
 }
 
 template <int DH>
@@ -568,13 +665,26 @@ cudaError_t launch_t(const DecodePagedParams& p, cudaStream_t st) {
 
 }  // namespace
 
+// Levels that the copy-engine form takes (and their sequences' lists fit beside its ring).
+bool decode_paged_dealt(const DecodePagedParams& p) {
+    if (p.B > 512 || (p.d != 64 && p.d != 128)) return false;
+    if (!tensor_map_encoder_available()) return false;
+    for (int l = 0; l < 3; ++l) {
+        const PagedLevelDev& L = p.L[l];
+        if (L.n == 0) continue;
+        if (L.table != nullptr && (L.page_shift < 3 || L.page_shift > 30)) return false;     // pages of 8 rows at least
+        if (L.sn <= 0 || L.sn % 8 || L.sh % 8 || L.sp % 8 || L.sp < 0) return false;
+        if (L.sp == 0 && (L.table != nullptr || p.B > 1)) return false;
+        if (p.H_kv > 1 && L.sh <= 0) return false;
+        if (L.n > 0x7fffffffLL) return false;
+    }
+    return true;
+}
+
 cudaError_t launch_decode_paged(const DecodePagedParams& p, cudaStream_t st) {
     if ((long long)p.B * p.H_kv * p.total_chunks == 0) return cudaSuccess;
     if (p.d != 128 && p.d != 64) return cudaErrorNotSupported;
-    if (tma_eligible(p)) {
-        const cudaError_t e = p.d == 128 ? launch_tma<128>(p, st) : launch_tma<64>(p, st);
-        if (e != cudaErrorNotSupported) return e;           // a map could not be encoded: the first form takes any layout
-    }
+    if (p.dealt) return p.d == 128 ? launch_tma<128>(p, st) : launch_tma<64>(p, st);
     return p.d == 128 ? launch_t<128>(p, st) : launch_t<64>(p, st);
 }
 

@@ -181,3 +181,49 @@ def test_recall_lists(mka, orc, bits, n, R):
                 want = np.zeros(R, dtype=np.int64)
                 want[:k] = own[best]
                 assert np.array_equal(table[b, h].cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("B,H,H_kv,N,page", [
+    (1, 16, 1, (64, 1, 0), 8),             # two tiles: one share
+    (37, 4, 2, (40, 130, 3), 16),          # shares that end inside lists and reach over several sequences
+    (3, 14, 2, (300, 9000, 70), 64),       # lists of dozens of shares
+    (513, 2, 1, (20, 33, 0), 16),          # more sequences than the dealt form takes
+])
+def test_decode_paged_shares(mka, orc, d, B, H, H_kv, N, page):
+    """Paged decode against the dense oracle: mixed lengths, sequences without a row, levels that a gate closes."""
+    P = problem(41, B, H, 1, d, N, 64, torch.bfloat16, router_std=0.5)
+    q = P["Q"][:, :, 0].contiguous()
+    gate = mka.mka_router(P["X"], P["W_r"], None).view(B, 3).clone()
+    gate[B // 2, 1] = 0.0
+    g = torch.Generator().manual_seed(5)
+    rows = [torch.randint(0, n + 1, (B,), generator=g, dtype=torch.int32) for n in N]
+    for r, n in zip(rows, N):
+        r[0] = n
+    if B > 2:
+        for r in rows:
+            r[B - 1] = 0
+    K, V = ([x[:, :H_kv].contiguous() for x in P[k]] for k in ("K", "V"))
+    pk, pv, tabs = [], [], []
+    for l, n in enumerate(N):
+        width = max(1, -(-n // page))
+        tab = torch.randperm(B * width + 2, generator=g)[:B * width].view(B, width).to(torch.int32)
+        a, b = (torch.full((B * width + 2, H_kv, page, d), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        for s in range(B):
+            for j in range(-(-int(rows[l][s]) // page)):
+                m = min(page, int(rows[l][s]) - j * page)
+                a[tab[s, j], :, :m] = K[l][s, :, j * page:j * page + m]
+                b[tab[s, j], :, :m] = V[l][s, :, j * page:j * page + m]
+        pk.append(a), pv.append(b), tabs.append(tab.cuda())
+    shape = mka.make_shape(B, H, 1, d, 64)
+    ws = torch.full((mka.mka_decode_paged_workspace_bytes(shape, H_kv, N),), 255, dtype=torch.uint8, device="cuda")
+    O, LSE = mka.mka_decode_paged(shape, H_kv, q, pk, pv, tabs, N, gate, rows=[r.cuda() for r in rows], ws=ws)
+    assert mka.mka_device_status(ws) == 0
+    for s in sorted({0, 1 % B, B // 2, B - 2 if B > 2 else 0, B - 1}):
+        ks, vs = ([x[l][s:s + 1, :, :int(rows[l][s])].repeat_interleave(H // H_kv, 1) for l in range(3)] for x in (K, V))
+        Or, Lr = orc.fwd(P["Q"][s:s + 1], ks, vs, np64(gate[s:s + 1]).reshape(1, 1, 3), 1, decode=True)
+        seen = np.isfinite(Lr[0, 0, 0])
+        check(O[s:s + 1], Or[:, :, 0] if seen else np.zeros_like(Or[:, :, 0]), torch.bfloat16, f"O of sequence {s}")
+        got = np64(LSE[s:s + 1])
+        assert np.isfinite(got).all() == seen
+        assert not seen or np.abs(got - Lr[:, :, 0]).max() <= 1e-4
