@@ -21,20 +21,23 @@
 // biases and 64 D_t per tile from shared memory (which the tensor pipe saturates).  They enter through the tensor pipe
 // instead: both score products get a ninth K-step whose key-side operand is ones and whose query-side operand holds
 // bias_t / scale (for S^T) or -D_t (for dP^T), each split into three bf16 terms, so S^T + bias / scale and dP^T - D arrive
-// in TMEM ready-made.  The producing warp writes those 4 KB operand slabs (no swizzle) from the statistics of the prep
+// in TMEM ready-made.  Two warps of their own write those 4 KB operand slabs (no swizzle) from the statistics of the prep
 // kernel, fetched one tile ahead.  Q tiles and dO tiles travel in rings of their own: dO(e) is free again after dV(e),
 // Q(e) only after dK(e), and Q(e+1) is what the next score product waits for.  Half of the exponentials of that kernel
 // run as a cubic on the FMA pipe (exp2_pair_fma).
 //
-// Warp roles (320 threads): warps 0-7 are the element-wise ("softmax") threads: thread i of either
-// warpgroup owns TMEM lane i & 127 (a query row in the dQ kernel, a key row in the dK/dV kernel);
-// warpgroup 0 takes columns 0-63 of a tile and warpgroup 1 columns 64-127.  Their work on a tile has
+// CTAs are persistent: they take output tiles (items) from a ticket counter, and the next item's copies and first products run
+// under the element-wise threads' stores of the previous one.
+//
+// Warp roles: the first eight warps (d = 64: sixteen) are the element-wise ("softmax") threads: thread i of a
+// warpgroup owns TMEM lane i & 127 (a query row in the dQ kernel, a key row in the dK/dV kernel) and the
+// warpgroup's share of a tile's columns (64, d = 64: 32).  Their work on a tile has
 // two phases so that it overlaps the tensor pipe: phase 1 needs only S (p = 2^(s*scale + bias), kept in
 // registers) and runs while dP is still being multiplied; phase 2 reads dP, forms dS = p (dP - D) and
-// writes it (bf16) over the columns of dP it has just read.  Warp 8 issues the TMA loads (lane 0);
-// warp 9 issues every tcgen05.mma, running its loop converged with one elected lane issuing.
+// writes it (bf16) over the columns of dP it has just read.  The next warp issues the TMA loads; the one
+// after it issues every tcgen05.mma, running its loop converged with one elected lane issuing; two more write the slabs (dK/dV).
 // TMEM (512 columns), dQ kernel: S ping [0,128), S pong [128,256), dP/dS [256,384), dQ [384,384+d).
-//                     dK/dV kernel: S^T/P^T [0,128), dP^T/dS^T [128,256), dK [256,256+d), dV [256+d,256+2d).
+//                     dK/dV kernel: S^T/P^T [0,128), dP^T/dS^T [128,256), dK [256,256+d), dV [256+d,256+2d), d = 64: second S^T [384,512).
 // Every mbarrier wait is bounded; on expiry the CTA raises a flag, drains and reports MKA_ERR_TIMEOUT.
 #include "tc_ptx.cuh"
 
