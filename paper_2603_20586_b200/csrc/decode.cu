@@ -519,7 +519,7 @@ extern "C" mka_status mka_decode_static(const mka_shape* s, const void* q, const
     if (slots * (unsigned long long)(s->d + 2) > kStaticScratchFloats) return MKA_ERR_WORKSPACE;
     float* scratch = nullptr;
     if (static_scratch_address(&scratch) != cudaSuccess) return MKA_ERR_CUDA;
-    DecodeParams p;
+    DecodeParams p = {};                 // (no partial counts, no status word)
     p.q = q; p.O = O; p.LSE = LSE; p.gate = gate;
     for (int l = 0; l < 3; ++l) {
         p.L[l].k = L[l].k; p.L[l].v = L[l].v; p.L[l].n = L[l].n;
@@ -534,7 +534,6 @@ extern "C" mka_status mka_decode_static(const mka_shape* s, const void* q, const
     // Nothing in the array has to start at zero: the partial kernel writes every slot that the combine
     // kernel of the same call reads, so whatever an earlier call left behind is never looked at.
     p.partial = scratch;
-    p.status = nullptr;
     cudaError_t e = launch_decode(p, static_cast<cudaStream_t>(stream));
     if (e == cudaErrorNotSupported) return MKA_ERR_UNSUPPORTED;
     return e == cudaSuccess ? MKA_OK : MKA_ERR_CUDA;
