@@ -137,7 +137,7 @@ struct BwdBarriers {
     uint64_t b_full[kMaxStages], b_empty[kMaxStages];     // second streamed ring (dQ kernel: V tiles; dK/dV kernel: dO tiles + D slabs)
     uint64_t s_full[2];                                   // S landed in TMEM (dQ kernel: ping, pong)
     uint64_t dp_full;                                     // dP landed in TMEM
-    uint64_t p_part[2];                                   // phase 1 (dK/dV kernel): the first / second 32 columns of every thread's P^T are written
+    uint64_t p_part[2];                                   // phase 1 (dK/dV kernel): the first / second half of every thread's P^T columns is written; with two S^T: all of the P^T over S^T buffer 0 / 1
     uint64_t ds_part[2];                                  // phase 2: the same for dS
     uint64_t acc_done;                                    // per item: its accumulators are complete
     uint64_t fixed_free;                                  // per item: its own tiles have had their last reader
@@ -907,9 +907,9 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
                     // hand their 64 columns over (K-steps {0, 1, 4, 5}, then {2, 3, 6, 7})
 #pragma unroll
                     for (int part = 0; part < 2; ++part) {
-                        // (with two S^T the element-wise threads are ahead: one wait, for the second part, costs less than two)
+                        // (with two S^T the element-wise threads are ahead: one wait, for the whole tile, costs less than two)
                         if (!kTwoS || part == 0) {
-                            if (!mbar_wait_warp(&bar.p_part[kTwoS ? 1 : part], (uint32_t)g & 1u, abortp)) { ok = false; break; }
+                            if (!mbar_wait_warp(&bar.p_part[kTwoS ? g & 1 : part], (uint32_t)(kTwoS ? g >> 1 : g) & 1u, abortp)) { ok = false; break; }
                             tc_fence_after();
                         }
 #pragma unroll
@@ -1061,10 +1061,13 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
             p_cols(0, kHalf);
             tmem_store_part<kHalf>(s_addr, pk);
             p_cols(kHalf, kHalf + kHalf / 2);
-            hand_over(&bar.p_part[0]);
+            if constexpr (!kTwoS) hand_over(&bar.p_part[0]);
             p_cols(kHalf + kHalf / 2, C::kCols);
             tmem_store_part<kHalf>(s_addr + kHalf / 2, pk + kHalf / 2);
-            hand_over(&bar.p_part[1]);
+            // With two S^T a warp may reach this line for tile g+1 while another has not yet for tile g (S^T(g+1) waits for nobody
+            // here), and an mbarrier counts arrivals, not warps: each buffer has a barrier of its own.  S^T(g+2) is issued behind
+            // dV(g), so no warp arrives twice in one phase.
+            hand_over(&bar.p_part[kTwoS ? g & 1 : 1]);
             // phase 2: dS^T = P^T (dP^T - D_t), written over the columns just read; the difference comes from the tensor pipe
             ok = mbar_wait(&bar.dp_full, (uint32_t)g & 1u, abortp);
             ok = __all_sync(0xffffffffu, ok);

@@ -64,6 +64,43 @@ def test_fwd_key_tiles_split_between_ctas(mka, orc, d, B, H, Hkv, T, W, q_off, N
         assert torch.equal(O, again)
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("B,H,Hkv,T,W,q_off,N", [
+    (4, 16, 4, 700, 64, 600, (1300, 1600, 40)),          # keys that no query sees (left of every window, past the last query): items without a tile
+    (5, 8, 8, 1100, 200, 0, (1100, 1100, 300)),          # one and more tiles to an item, last tiles that are not full
+])
+def test_bwd_items_carried_over(mka, orc, d, B, H, Hkv, T, W, q_off, N):
+    """More than two output tiles to every CTA of the dQ and the dK/dV kernel: rings, buffers and barriers go on from item to item.
+    The result may not change from call to call either: a tile read before every warp has written its part would."""
+    assert B * H * -(-T // 128) > 296 and B * Hkv * sum(-(-n // 128) for n in N) > 296
+    P = problem(43, B, H, T, d, N, 64, torch.bfloat16, router_std=0.5, with_dO=True)
+    K, V = ([x[:, :Hkv].contiguous() for x in P[k]] for k in ("K", "V"))
+    shape = mka.make_shape(B, H, T, d, 64, W, q_off, kv_heads=Hkv)
+    assert mka.mka_bwd_kernel_kind(shape, K, V) == 1
+    gate = mka.mka_router(P["X"], P["W_r"], None)
+    O, LSE = mka.mka_fwd(shape, P["Q"], K, V, gate)
+    ws = mka.alloc_workspace(shape, N, mka.MKA_WS_BWD, "cuda")
+    run = lambda: mka.mka_bwd(shape, P["Q"], K, V, gate, O, LSE, P["dO"], R=P["X"], ws=ws)  # noqa: E731
+    g = run()
+    assert mka.mka_device_status(ws) == 0
+    for _ in range(20):
+        again = run()
+        assert torch.equal(g["dQ"], again["dQ"])
+        for l in range(3):
+            assert torch.equal(g["dK"][l], again["dK"][l]) and torch.equal(g["dV"][l], again["dV"][l])
+    G = H // Hkv
+    rep = [[x.repeat_interleave(G, 1) for x in t] for t in (K, V)]
+    r = orc.bwd(P["Q"], rep[0], rep[1], np64(gate), P["dO"], W, q_off)
+    check(g["dQ"], r["dQ"], torch.bfloat16, "dQ")
+    for l in range(3):
+        for name in ("dK", "dV"):
+            want = r[name][l].reshape(B, Hkv, G, N[l], d).sum(2)
+            # one rounding to bf16 of a sum over the group's heads and up to T queries: half a step of the largest value, on top of the contract's bound
+            mx, mean = err(g[name][l], want)
+            assert mx <= 2e-2 + np.abs(want).max() / 256 and mean <= 2e-3 + np.abs(want).mean() / 256, (name, l, mx, mean)
+    check(g["dG"], r["dG"], torch.bfloat16, "dG")
+
+
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("B,T,D", [(1, 1, 64), (1, 127, 264), (2, 300, 2048), (3, 1111, 1000), (1, 5000, 256), (2, 70, 100)])
 def test_router_gradient_splits(mka, orc, dtype, B, T, D):
