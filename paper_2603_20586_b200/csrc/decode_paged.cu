@@ -492,6 +492,9 @@ __global__ void __launch_bounds__(kTmaThreads, 2) decode_paged_tma_kernel(const 
                     const int row = kb + r_first + idx / (8 * kPanels), rest = idx % (8 * kPanels);
                     *reinterpret_cast<uint4*>(sV + (rest / 8) * kPanelBytes + row * 128 + (rest % 8) * 16) = make_uint4(0u, 0u, 0u, 0u);
                 }
+                // the share goes on behind this tile: the copy engine writes the same bytes again once the stage is free, and the
+                // mbarrier alone does not order these stores before its writes
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
             }
             float s[2][4];

@@ -225,6 +225,7 @@ def test_recall_lists(mka, orc, bits, n, R):
     (1, 16, 1, (64, 1, 0), 8),             # two tiles: one share
     (37, 4, 2, (40, 130, 3), 16),          # shares that end inside lists and reach over several sequences
     (3, 14, 2, (300, 9000, 70), 64),       # lists of dozens of shares
+    (150, 4, 2, (70, 129, 200), 16),       # shares of nine tiles, every third one ragged: stages refilled behind rows that were cleared
     (513, 2, 1, (20, 33, 0), 16),          # more sequences than the dealt form takes
 ])
 def test_decode_paged_shares(mka, orc, d, B, H, H_kv, N, page):
@@ -256,6 +257,9 @@ def test_decode_paged_shares(mka, orc, d, B, H, H_kv, N, page):
     ws = torch.full((mka.mka_decode_paged_workspace_bytes(shape, H_kv, N),), 255, dtype=torch.uint8, device="cuda")
     O, LSE = mka.mka_decode_paged(shape, H_kv, q, pk, pv, tabs, N, gate, rows=[r.cuda() for r in rows], ws=ws)
     assert mka.mka_device_status(ws) == 0
+    for _ in range(30):                    # (a row cleared or copied too late would not come out the same every time)
+        again, _ = mka.mka_decode_paged(shape, H_kv, q, pk, pv, tabs, N, gate, rows=[r.cuda() for r in rows], ws=ws)
+        assert torch.equal(O, again)
     for s in sorted({0, 1 % B, B // 2, B - 2 if B > 2 else 0, B - 1}):
         ks, vs = ([x[l][s:s + 1, :, :int(rows[l][s])].repeat_interleave(H // H_kv, 1) for l in range(3)] for x in (K, V))
         Or, Lr = orc.fwd(P["Q"][s:s + 1], ks, vs, np64(gate[s:s + 1]).reshape(1, 1, 3), 1, decode=True)
