@@ -69,8 +69,9 @@ typedef enum { MKA_ROUTE_SOFT = 0, MKA_ROUTE_UNIFORM = 1, MKA_ROUTE_TOP1 = 2, MK
                                            the status word; O and LSE of such a call are invalid.  In mka_bwd
                                            (tensor-core kernels) the loader of every CTA of the dK/dV kernel leaves
                                            out its last query tile, with the same end; the gradients of such a call
-                                           are invalid.  Exists so that the give-up path can be exercised without a
-                                           fault or a hang. */
+                                           are invalid.  In mka_decode_paged (copy-engine form) the loader of every CTA
+                                           leaves out the last tile of its share; O and LSE are invalid.  Exists so
+                                           that the give-up path can be exercised without a fault or a hang. */
 
 /* which = argument of mka_workspace_bytes */
 #define MKA_WS_FWD 0

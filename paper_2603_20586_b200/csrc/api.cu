@@ -443,6 +443,7 @@ mka_status mka_decode_paged(const mka_shape* s, int32_t H_kv, const void* q, con
     if ((long long)s->B * s->H * plan.total_chunks > 0x7fffffffLL) return MKA_ERR_SHAPE;
     p.q = q; p.gate = gate;
     p.B = s->B; p.H = s->H; p.H_kv = H_kv; p.d = s->d; p.scale = resolve_scale(s);
+    p.test_stall = (s->flags & MKA_FLAG_TEST_STALL) ? 1 : 0;
     DecodeParams c;                                    // the combine kernel of the dense decode finishes the job
     memset(&c, 0, sizeof(c));
     c.O = O; c.LSE = LSE; c.gate = gate; c.B = s->B; c.H = s->H; c.d = s->d;

@@ -424,11 +424,12 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const 
             item = __shfl_sync(0xffffffffu, item, 0);
         }
         // every copy issued above must have landed before the shared memory can be given up
-        if (filled > 0) mbar_wait_warp(&bar.fixed_full, (uint32_t)(filled - 1) & 1u, abortp);
+        const unsigned long long t_drain = gtimer();
+        if (filled > 0) mbar_drain(&bar.fixed_full, (uint32_t)(filled - 1) & 1u, abortp, t_drain);
         for (int i = issued_k > C::kStagesK ? issued_k - C::kStagesK : 0; i < issued_k; ++i)
-            mbar_wait_warp(&bar.a_full[i % C::kStagesK], (uint32_t)(i / C::kStagesK) & 1u, abortp);
+            mbar_drain(&bar.a_full[i % C::kStagesK], (uint32_t)(i / C::kStagesK) & 1u, abortp, t_drain);
         for (int i = issued_v > C::kStages ? issued_v - C::kStages : 0; i < issued_v; ++i)
-            mbar_wait_warp(&bar.b_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
+            mbar_drain(&bar.b_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp, t_drain);
     } else if (warp == C::kMmaWarp) {
         {   // every lane runs the issue loop (converged); elect.sync inside the wrappers picks the issuing lane
             // low descriptor words of the operands (see make_desc): K-major views for S and dP, MN-major view of K for dQ
@@ -806,12 +807,14 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
             if (lane == 0) item = (int)gridDim.x + (int)atomicAdd(p.dkv_ticket, 1u);
             item = __shfl_sync(0xffffffffu, item, 0);
         }
-        // every copy issued above must have landed before the shared memory can be given up
-        if (filled > 0) mbar_wait_warp(&bar.fixed_full, (uint32_t)(filled - 1) & 1u, abortp);
+        // every copy issued above must have landed before the shared memory can be given up (a stage that a slab warp gave up
+        // before writing does not complete: the limit, one for all of these waits, ends it)
+        const unsigned long long t_drain = gtimer();
+        if (filled > 0) mbar_drain(&bar.fixed_full, (uint32_t)(filled - 1) & 1u, abortp, t_drain);
         for (int i = issued > C::kStages ? issued - C::kStages : 0; i < issued; ++i)
-            mbar_wait_warp(&bar.a_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
+            mbar_drain(&bar.a_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp, t_drain);
         for (int i = issued_b > C::kStages ? issued_b - C::kStages : 0; i < issued_b; ++i)
-            mbar_wait_warp(&bar.b_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
+            mbar_drain(&bar.b_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp, t_drain);
     } else if (warp == C::kSlabWarp || warp == C::kSlabWarp + 1) {
         // The operand slabs of the ninth K-step: the first of these warps writes the bias slabs (ring of the Q tiles), the second
         // the D slabs (ring of the dO tiles), four queries a lane, fetched one tile ahead.  Warps of their own: when the

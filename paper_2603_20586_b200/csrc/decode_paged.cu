@@ -416,13 +416,13 @@ __global__ void __launch_bounds__(kTmaThreads, 2) decode_paged_tma_kernel(const 
         int page, in_row, page_n = 0, in_row_n = 0;
         bool have = next(cur);
         if (have) look_up(cur, page, in_row);
-        bool ok = true;
         int issued = 0;
         while (have) {
             const bool have_n = next(nxt);
+            if (p.test_stall && !have_n) break;             // test hook: the last tile of the share never arrives
             if (have_n) look_up(nxt, page_n, in_row_n);
             const int st = issued % kTmaStages;
-            if (!mbar_wait_warp(&empty[st], ((uint32_t)(issued / kTmaStages) & 1u) ^ 1u, ctlp)) { ok = false; break; }
+            if (!mbar_wait_warp(&empty[st], ((uint32_t)(issued / kTmaStages) & 1u) ^ 1u, ctlp)) break;
             if (lane == 0) mbar_expect_tx(&full[st], 2 * kTileBytes);
             __syncwarp();
             const int box = box_rows_of(cur.lvl);
@@ -437,10 +437,10 @@ __global__ void __launch_bounds__(kTmaThreads, 2) decode_paged_tma_kernel(const 
             ++issued;
             cur = nxt; page = page_n; in_row = in_row_n; have = have_n;
         }
-        // the shared memory must not be given up with a copy in flight: wait (bounded) for the stages still out
-        if (ok)
-            for (int i = issued > kTmaStages ? issued - kTmaStages : 0; i < issued; ++i)
-                mbar_wait_warp(&full[i % kTmaStages], (uint32_t)(i / kTmaStages) & 1u, ctlp);
+        // the shared memory must not be given up with a copy in flight, whoever gave up: wait (bounded) for the stages still out
+        const unsigned long long t0 = gtimer();
+        for (int i = issued > kTmaStages ? issued - kTmaStages : 0; i < issued; ++i)
+            mbar_drain(&full[i % kTmaStages], (uint32_t)(i / kTmaStages) & 1u, ctlp, t0);
         return;
     }
 

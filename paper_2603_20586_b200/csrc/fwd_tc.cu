@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
                                     &bar.k_full[s]);
                 }
                 if (!mbar_wait_warp(&bar.v_empty[s], ph ^ 1u, abortp)) {           // gave up with this stage's K copies in flight
-                    mbar_wait_warp(&bar.k_full[s], ph, abortp);
+                    mbar_drain(&bar.k_full[s], ph, abortp, gtimer());
                     ok = false;
                     break;
                 }
@@ -294,10 +294,11 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
         }
         // Before leaving, make sure every copy issued has landed (bounded): the shared memory must not be handed to
         // another CTA with a bulk copy still in flight.  (A stage whose wait failed got no copies.)
-        mbar_wait_warp(&bar.q_full, 0, abortp);
+        const unsigned long long t_drain = gtimer();
+        mbar_drain(&bar.q_full, 0, abortp, t_drain);
         for (int i = issued > C::kStages ? issued - C::kStages : 0; i < issued; ++i) {
-            mbar_wait_warp(&bar.k_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
-            mbar_wait_warp(&bar.v_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
+            mbar_drain(&bar.k_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp, t_drain);
+            mbar_drain(&bar.v_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp, t_drain);
         }
     } else if (warp == C::kProducerWarp) {
         // Dense levels: the warp waits converged and one lane issues (inside an `if (lane == 0)` around the whole loop the
@@ -329,7 +330,7 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
                 }
                 __syncwarp();
                 if (!mbar_wait_warp(&bar.v_empty[s], ph ^ 1u, abortp)) {           // gave up with this stage's K copies in flight
-                    mbar_wait_warp(&bar.k_full[s], ph, abortp);
+                    mbar_drain(&bar.k_full[s], ph, abortp, gtimer());
                     ok = false;
                     break;
                 }
@@ -345,10 +346,11 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
         }
         // Before leaving, make sure every copy issued has landed (bounded): the shared memory must not be handed to
         // another CTA with a bulk copy still in flight.  (A stage whose wait failed got no copies.)
-        mbar_wait_warp(&bar.q_full, 0, abortp);
+        const unsigned long long t_drain = gtimer();
+        mbar_drain(&bar.q_full, 0, abortp, t_drain);
         for (int i = issued > C::kStages ? issued - C::kStages : 0; i < issued; ++i) {
-            mbar_wait_warp(&bar.k_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
-            mbar_wait_warp(&bar.v_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp);
+            mbar_drain(&bar.k_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp, t_drain);
+            mbar_drain(&bar.v_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp, t_drain);
         }
     } else if (warp == C::kMmaWarp) {
         {   // every lane runs the issue loop (converged); elect.sync inside the wrappers picks the issuing lane

@@ -115,9 +115,9 @@ __global__ void __launch_bounds__(kSumThreads, 3) l2_summary_kernel(const __grid
     }
     const bool fresh_ema = kEma && !p.use_state;      // the first token of the session initialises the average
     bool ok = true;
-    int s = 0;
+    int s = 0, i = 0;
     uint32_t phase = 0;                               // ring slot of tile i and the parity of its use
-    for (int i = 0; i < ntiles; ++i) {
+    for (; i < ntiles; ++i) {
         ok = mbar_wait(&full[s], phase, abortp);
         if (!__syncthreads_and(ok)) { ok = false; break; }
         const P2* tile = reinterpret_cast<const P2*>(ring + (size_t)s * kTileBytes) + (size_t)g * RG * kNP + c;
@@ -195,7 +195,8 @@ __global__ void __launch_bounds__(kSumThreads, 3) l2_summary_kernel(const __grid
     }
     if (!ok && tid == 0) {
         // copies issued but not consumed must land before the shared memory is given up (bounded)
-        for (int s = 0; s < kSumStages; ++s) mbar_wait(&full[s], 0, abortp), mbar_wait(&full[s], 1, abortp);
+        const unsigned long long t0 = gtimer();
+        for (int j = i; j < ntiles && j < i + kSumStages; ++j) mbar_drain(&full[j % kSumStages], (uint32_t)(j / kSumStages) & 1u, abortp, t0);
         if (p.status) atomicExch(p.status, (unsigned int)MKA_ERR_TIMEOUT);
     }
     __syncthreads();

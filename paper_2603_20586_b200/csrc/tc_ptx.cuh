@@ -51,6 +51,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile
         if (gtimer() - t0 > ctl->limit_ns) { ctl->abort = 1; return false; }
     }
 }
+// Waits for a copy that was issued.  Unlike mbar_wait it goes on when another role gave up: a CTA must not hand its shared memory
+// back with a copy in flight.  Bounded by the same limit, counted from `t0`, so that several of these in a row have one limit.
+__device__ __forceinline__ void mbar_drain(uint64_t* b, uint32_t parity, volatile WaitCtl* ctl, unsigned long long t0) {
+    while (!mbar_try(b, parity))
+        if (gtimer() - t0 > ctl->limit_ns) { ctl->abort = 1; return; }
+}
 __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, int x, int y, int z, int w, uint64_t* bar) {
     asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
                  ::"r"(smem_u32(dst)), "l"(map), "r"(x), "r"(y), "r"(z), "r"(w), "r"(smem_u32(bar)) : "memory");

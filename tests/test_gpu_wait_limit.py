@@ -1,9 +1,9 @@
 """The give-up path of the kernels' bounded waits, exercised without a fault or a hang.
 
-Every wait inside the tensor-core forward and backward and the segmented summary has a wall-clock limit.  Here the
-limit is set to a few milliseconds and a test hook withholds something a wait needs (the forward's last key tile; the
-last query tile of the backward's dK/dV kernel, whose issuing warp polls two barriers in a loop of its own; one
-segment's carried state): the wait runs out, every role of the CTA drains, tensor memory is freed, the kernel RETURNS, and the
+Every wait inside the tensor-core forward and backward, the paged decode and the segmented summary has a wall-clock limit.
+Here the limit is set to a few milliseconds and a test hook withholds something a wait needs (the forward's last key tile;
+the last query tile of the backward's dK/dV kernel, whose issuing warp polls two barriers in a loop of its own; the last
+tile of a share of the paged decode; one segment's carried state): the wait runs out, every role of the CTA drains, tensor memory is freed, the kernel RETURNS, and the
 status word of the workspace reads MKA_ERR_TIMEOUT.  The next ordinary call on the same stream must then match the
 oracle, which shows that the context and the library are still healthy.
 """
@@ -79,6 +79,61 @@ def test_backward_wait_runs_out_and_the_next_call_is_correct(mka, orc, short_lim
     for l in range(3):
         check(g["dK"][l], ref["dK"][l], torch.bfloat16, f"dK{l} after a timed-out call")
         check(g["dV"][l], ref["dV"][l], torch.bfloat16, f"dV{l} after a timed-out call")
+
+
+@pytest.mark.parametrize("d", [128, 64])
+def test_backward_wait_runs_out_in_a_later_item(mka, orc, short_limit, d):
+    """160 key tiles on 148 CTAs, only the newest of them seen by a query: every CTA's first item has no tile, and the wait
+    that runs out is one of a CTA's second item."""
+    B, H, T, W, N = 1, 1, 300, 96, (20480, 0, 0)
+    P = problem(94, B, H, T, d, N, 32, torch.bfloat16, router_std=0.3, with_dO=True)
+    gate = mka.mka_router(P["X"], P["W_r"], None)
+    mk = lambda flags: mka.make_shape(B, H, T, d, 32, W, q_offset=N[0] - T, flags=flags)  # noqa: E731
+    shape, stalled = mk(0), mk(mka.MKA_FLAG_TEST_STALL)
+    O, LSE = mka.mka_fwd(shape, P["Q"], P["K"], P["V"], gate)
+    assert mka.mka_bwd_kernel_kind(shape, P["K"], P["V"]) == 1
+    ws = mka.alloc_workspace(shape, N, mka.MKA_WS_BWD, "cuda")
+    mka.mka_bwd(stalled, P["Q"], P["K"], P["V"], gate, O, LSE, P["dO"], ws=ws)
+    assert mka.mka_device_status(ws) == MKA_ERR_TIMEOUT
+    g = mka.mka_bwd(shape, P["Q"], P["K"], P["V"], gate, O, LSE, P["dO"], ws=ws)
+    assert mka.mka_device_status(ws) == 0
+    ref = orc.bwd(P["Q"], P["K"], P["V"], np64(gate), P["dO"], W, q_offset=N[0] - T)
+    check(g["dQ"], ref["dQ"], torch.bfloat16, "dQ after a timed-out call")
+    check(g["dK"][0], ref["dK"][0], torch.bfloat16, "dK after a timed-out call")
+    check(g["dV"][0], ref["dV"][0], torch.bfloat16, "dV after a timed-out call")
+    assert not g["dK"][0][:, :, :N[0] - T - W].any()             # the items without a tile are written, as zeros
+
+
+@pytest.mark.parametrize("d", [128, 64])
+def test_paged_decode_wait_runs_out_and_the_next_call_is_correct(mka, orc, short_limit, d):
+    """The last tile of every CTA's share never arrives: the computing warps give up with other copies of the ring in flight."""
+    B, H, Hkv, N, page = 2, 4, 2, (300, 70000, 100), 16
+    P = problem(95, B, H, 1, d, N, 64, torch.bfloat16, router_std=0.3)
+    gate = mka.mka_router(P["X"], P["W_r"], None).view(B, 3)
+    q = P["Q"][:, :, 0].contiguous()
+    pools, tabs = ([], []), []
+    for l, n in enumerate(N):
+        width = -(-n // page)
+        tab = torch.randperm(B * width, generator=torch.Generator().manual_seed(l)).view(B, width).to(torch.int32).cuda()
+        for dst, src in zip(pools, (P["K"][l][:, :Hkv], P["V"][l][:, :Hkv])):
+            rows = torch.nn.functional.pad(src, (0, 0, 0, width * page - n)).view(B, Hkv, width, page, d).transpose(1, 2)
+            dst.append(torch.empty(B * width, Hkv, page, d, dtype=src.dtype, device="cuda"))
+            dst[-1][tab.long().flatten()] = rows.reshape(B * width, Hkv, page, d)
+        tabs.append(tab)
+    shape, stalled = mka.make_shape(B, H, 1, d), mka.make_shape(B, H, 1, d, flags=mka.MKA_FLAG_TEST_STALL)
+    ws = torch.zeros(mka.mka_decode_paged_workspace_bytes(shape, Hkv, N), dtype=torch.uint8, device="cuda")
+    t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    t0.record()
+    mka.mka_decode_paged(stalled, Hkv, q, *pools, tabs, N, gate, ws=ws)
+    t1.record()
+    assert mka.mka_device_status(ws) == MKA_ERR_TIMEOUT
+    assert t0.elapsed_time(t1) < 1000.0
+    O, LSE = mka.mka_decode_paged(shape, Hkv, q, *pools, tabs, N, gate, ws=ws)
+    assert mka.mka_device_status(ws) == 0
+    rep = [[x[:, :Hkv].repeat_interleave(H // Hkv, 1) for x in P[k]] for k in ("K", "V")]
+    Or, Lr = orc.fwd(P["Q"], *rep, np64(gate).reshape(B, 1, 3), 1, decode=True)
+    check(O, Or[:, :, 0], torch.bfloat16, "paged decode after a timed-out call")
+    assert np.abs(np64(LSE) - Lr[:, :, 0]).max() <= 2e-3
 
 
 def test_summary_look_back_runs_out_and_the_next_call_is_correct(mka, orc, short_limit):
