@@ -2,6 +2,8 @@
 // (Alg. 1 step 12 / Alg. 2 step 5), plus the hard top-1 / top-2 and uniform routing variants
 // (Table 10).  HBM-bound for many rows, latency-bound for few: every row of R is read exactly once with 16-byte loads.
 // Also the router's backward: dW_r = R^T dG, db_r = sum dG (two deterministic passes).
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace mka {
@@ -72,6 +74,21 @@ template <> struct Vec8<float> {
     static __device__ __forceinline__ void widen(const Raw& u, float (&x)[8]) {
         x[0] = u.a.x; x[1] = u.a.y; x[2] = u.a.z; x[3] = u.a.w; x[4] = u.b.x; x[5] = u.b.y; x[6] = u.b.z; x[7] = u.b.w;
     }
+};
+
+template <typename T, int N> struct Cols : Vec8<T> {};   // N consecutive elements as floats
+template <> struct Cols<__nv_bfloat16, 4> {
+    using Raw = uint2;
+    static __device__ __forceinline__ Raw fetch(const __nv_bfloat16* p) { return __ldg(reinterpret_cast<const uint2*>(p)); }
+    static __device__ __forceinline__ void widen(const Raw& u, float (&x)[4]) {
+        x[0] = __uint_as_float(u.x << 16); x[1] = __uint_as_float(u.x & 0xffff0000u);
+        x[2] = __uint_as_float(u.y << 16); x[3] = __uint_as_float(u.y & 0xffff0000u);
+    }
+};
+template <> struct Cols<float, 4> {
+    using Raw = float4;
+    static __device__ __forceinline__ Raw fetch(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+    static __device__ __forceinline__ void widen(const Raw& u, float (&x)[4]) { x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w; }
 };
 
 // Sums of ROWS rows x 3 logits over a warp: while a lane holds several rows it hands half of them to its partner and adds
@@ -238,11 +255,43 @@ router_any_kernel(const T* __restrict__ R, const float* __restrict__ W_r, const 
     }
 }
 
+// Sum of rows [r0, r1) of a [rows, 3] array by the 256 threads of a CTA, valid in thread 0.
+template <typename V>
+__device__ __forceinline__ void sum_dG(const V* __restrict__ x, long long r0, long long r1, double (&sm)[256][3], double (&a)[3]) {
+    a[0] = a[1] = a[2] = 0.0;
+    for (long long r = r0 + threadIdx.x; r < r1; r += 256)
+#pragma unroll
+        for (int l = 0; l < 3; ++l) a[l] += (double)x[r * 3 + l];
+#pragma unroll
+    for (int l = 0; l < 3; ++l) sm[threadIdx.x][l] = a[l];
+    __syncthreads();
+    for (int s = 128; s > 0; s >>= 1) {
+        if (threadIdx.x < s)
+#pragma unroll
+            for (int l = 0; l < 3; ++l) sm[threadIdx.x][l] += sm[threadIdx.x + s][l];
+        __syncthreads();
+    }
+#pragma unroll
+    for (int l = 0; l < 3; ++l) a[l] = sm[0][l];
+}
+
+// The CTAs of the first column block also add up their chunk's rows of dG for db_r, in 64 bits because the rows' terms cancel
+// (one CTA over all rows took 22 us at 32768 rows).
+__device__ __forceinline__ void chunk_db(const float* __restrict__ dG, long long r0, long long r1, int chunk, double* __restrict__ db_partial) {
+    if (blockIdx.x != 0 || !db_partial) return;
+    __shared__ double sm[256][3];
+    double b[3];
+    sum_dG(dG, r0, r1, sm, b);
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int l = 0; l < 3; ++l) db_partial[chunk * 3 + l] = b[l];
+}
+
 // dW_r partials: CTA (row chunk, column block); thread = one column of R, loops over the chunk's rows.
 template <typename T>
 __global__ void __launch_bounds__(256)
 router_bwd_partial_kernel(const T* __restrict__ R, const float* __restrict__ dG, long long rows, int D,
-                          int n_row_chunks, float* __restrict__ partial) {
+                          int n_row_chunks, float* __restrict__ partial, double* __restrict__ db_partial) {
     const int c = blockIdx.x * 256 + threadIdx.x;
     const int chunk = blockIdx.y;
     const long long per = (rows + n_row_chunks - 1) / n_row_chunks;
@@ -268,71 +317,51 @@ router_bwd_partial_kernel(const T* __restrict__ R, const float* __restrict__ dG,
         float* o = partial + ((long long)chunk * D + c) * 3;
         o[0] = a0; o[1] = a1; o[2] = a2;
     }
+    chunk_db(dG, r0, r1, chunk, db_partial);
 }
 
-// Sum of rows [r0, r1) of a [rows, 3] array by the 256 threads of a CTA, valid in thread 0.
-template <typename V>
-__device__ __forceinline__ void sum_dG(const V* __restrict__ x, long long r0, long long r1, double (&sm)[256][3], double (&a)[3]) {
-    a[0] = a[1] = a[2] = 0.0;
-    for (long long r = r0 + threadIdx.x; r < r1; r += 256)
-#pragma unroll
-        for (int l = 0; l < 3; ++l) a[l] += (double)x[r * 3 + l];
-#pragma unroll
-    for (int l = 0; l < 3; ++l) sm[threadIdx.x][l] = a[l];
-    __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-        if (threadIdx.x < s)
-#pragma unroll
-            for (int l = 0; l < 3; ++l) sm[threadIdx.x][l] += sm[threadIdx.x + s][l];
-        __syncthreads();
-    }
-#pragma unroll
-    for (int l = 0; l < 3; ++l) a[l] = sm[0][l];
-}
-
-// The same with eight consecutive columns per lane (16-byte loads of bf16): a warp takes every eighth row of the chunk, and
+// The same with N = 8 or 4 consecutive columns per lane (16- or 8-byte loads of bf16): a warp takes every eighth row of the chunk, and
 // the next eight rows' loads are in flight while the current eight are added (without that the kernel waits for
-// loads most of the time: 2 TB/s); the eight warps' sums meet in shared memory.  Used when D is a multiple of 8 and R is
-// 16-byte aligned.  The CTAs of the first column block also add up the chunk's rows of dG for db_r, in 64 bits because the
-// rows' terms cancel (one CTA over all rows took 22 us at 32768 rows).
-template <typename T>
+// loads most of the time: 2 TB/s); the eight warps' sums meet in shared memory.  Used when D is a multiple of N and R is
+// 16-byte aligned.
+template <typename T, int N>
 __global__ void __launch_bounds__(256, 2)
-router_bwd_partial8_kernel(const T* __restrict__ R, const float* __restrict__ dG, long long rows, int D,
+router_bwd_partial_vec_kernel(const T* __restrict__ R, const float* __restrict__ dG, long long rows, int D,
                            int n_row_chunks, float* __restrict__ partial, double* __restrict__ db_partial) {
-    constexpr int kBatch = sizeof(T) == 2 ? 8 : 4;             // rows of a batch: 16-byte loads in flight a lane = 8
-    __shared__ float sum[8][24][33];
+    constexpr int kBatch = N * sizeof(T) <= 16 ? 8 : 4;        // rows of a batch: loads in flight a lane = 8
+    __shared__ float sum[8][3 * N][33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int c = blockIdx.x * 256 + lane * 8;
+    const int c = blockIdx.x * (32 * N) + lane * N;
     const int chunk = blockIdx.y;
     const long long per = (rows + n_row_chunks - 1) / n_row_chunks;
     const long long r0 = chunk * per, r1 = r0 + per < rows ? r0 + per : rows;
-    float a[24];
+    float a[3 * N];
 #pragma unroll
-    for (int j = 0; j < 24; ++j) a[j] = 0.f;
-    typename Vec8<T>::Raw x[2][kBatch];
+    for (int j = 0; j < 3 * N; ++j) a[j] = 0.f;
+    typename Cols<T, N>::Raw x[2][kBatch];
     float g[2];
     // rows rb, rb + 8, ..; a row past the chunk's end reads row rb again and weighs 0.  Lane 3u + l fetches dG[row u][l].
-    auto fetch = [&](long long rb, typename Vec8<T>::Raw (&to)[kBatch], float& gv) {
+    auto fetch = [&](long long rb, typename Cols<T, N>::Raw (&to)[kBatch], float& gv) {
         if (rb >= r1) return;
         if (c < D)
 #pragma unroll
-            for (int u = 0; u < kBatch; ++u) to[u] = Vec8<T>::fetch(R + (rb + 8 * u < r1 ? rb + 8 * u : rb) * (long long)D + c);
+            for (int u = 0; u < kBatch; ++u) to[u] = Cols<T, N>::fetch(R + (rb + 8 * u < r1 ? rb + 8 * u : rb) * (long long)D + c);
         const long long gr = rb + 8 * (lane / 3);
         gv = lane < 3 * kBatch && gr < r1 ? __ldg(dG + gr * 3 + lane % 3) : 0.f;
     };
-    auto add = [&](long long rb, const typename Vec8<T>::Raw (&from)[kBatch], float gv) {
+    auto add = [&](long long rb, const typename Cols<T, N>::Raw (&from)[kBatch], float gv) {
         if (rb >= r1) return;
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) {
             const bool in = rb + 8 * u < r1;                   // (a repeated row weighs 0, but 0 x inf would not be 0)
-            float f[8];
-            Vec8<T>::widen(from[u], f);
+            float f[N];
+            Cols<T, N>::widen(from[u], f);
 #pragma unroll
             for (int l = 0; l < 3; ++l) {
                 const float gl = __shfl_sync(0xffffffffu, gv, 3 * u + l);
                 if (in)
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) a[j * 3 + l] = fmaf(f[j], gl, a[j * 3 + l]);
+                    for (int j = 0; j < N; ++j) a[j * 3 + l] = fmaf(f[j], gl, a[j * 3 + l]);
             }
         }
     };
@@ -344,23 +373,16 @@ router_bwd_partial8_kernel(const T* __restrict__ R, const float* __restrict__ dG
         add(rb + 8 * kBatch, x[1], g[1]);
     }
 #pragma unroll
-    for (int j = 0; j < 24; ++j) sum[warp][j][lane] = a[j];
+    for (int j = 0; j < 3 * N; ++j) sum[warp][j][lane] = a[j];
     __syncthreads();
-    const int cols = min(256, D - (int)blockIdx.x * 256) * 3;
+    const int cols = min(32 * N, D - (int)blockIdx.x * (32 * N)) * 3;
     for (int i = threadIdx.x; i < cols; i += 256) {
         float s = 0.f;
 #pragma unroll
-        for (int w = 0; w < 8; ++w) s += sum[w][i % 24][i / 24];
-        partial[((long long)chunk * D + blockIdx.x * 256) * 3 + i] = s;
+        for (int w = 0; w < 8; ++w) s += sum[w][i % (3 * N)][i / (3 * N)];
+        partial[((long long)chunk * D + blockIdx.x * (32 * N)) * 3 + i] = s;
     }
-    if (blockIdx.x == 0 && db_partial) {
-        __shared__ double sm[256][3];
-        double b[3];
-        sum_dG(dG, r0, r1, sm, b);
-        if (threadIdx.x == 0)
-#pragma unroll
-            for (int l = 0; l < 3; ++l) db_partial[chunk * 3 + l] = b[l];
-    }
+    chunk_db(dG, r0, r1, chunk, db_partial);
 }
 
 // dW_r = sum of the chunks' partials (32 outputs to a CTA, eight threads to an output: the loads of one output are eight
@@ -434,22 +456,25 @@ cudaError_t launch_router(const void* R, const float* W_r, const float* b_r, lon
 
 cudaError_t launch_router_bwd(const void* R, int r_dtype, const float* dG, long long rows, int D, float* dW_r,
                               float* db_r, float* partial, double* db_partial, int n_row_chunks, cudaStream_t st) {
-    // as many row chunks as fill the chip's CTA slots once (two to an SM), at most the caller's
-    const int col_blocks = (D + 255) / 256;
-    if (n_row_chunks > 296 / col_blocks) n_row_chunks = 296 / col_blocks > 0 ? 296 / col_blocks : 1;
-    const bool vec = dW_r && D % 8 == 0 && (reinterpret_cast<uintptr_t>(R) & 15) == 0;
-    double* db_part = vec && db_r ? db_partial : nullptr;
+    // Columns a lane: eight where D and R allow it, else four, else one.  The vector kernels keep their own loads in flight and take
+    // as many row chunks as fill the chip's CTA slots once (two to an SM).  A thread of the one-column kernel has one load in
+    // flight and lives on the number of CTAs: it takes all of the caller's chunks.  Both kernels together, 32768 rows of bf16:
+    // D = 4096 (eight columns) 69 us; D = 4100 87 us with four columns, 702 with one and few chunks; D = 2050 54 us with
+    // all chunks, 397 with few; D = 4096 at an address that allows no vector 94 us, 697 with few.
+    const bool aligned = (reinterpret_cast<uintptr_t>(R) & 15) == 0;
+    const int cols = aligned && D % 8 == 0 ? 8 : (aligned && D % 4 == 0 ? 4 : 1);
+    const int col_blocks = cols == 1 ? (D + 255) / 256 : (D + 32 * cols - 1) / (32 * cols);
+    if (cols > 1 && n_row_chunks > 296 / col_blocks) n_row_chunks = 296 / col_blocks > 0 ? 296 / col_blocks : 1;
+    double* db_part = dW_r && db_r ? db_partial : nullptr;
     if (dW_r) {
         const dim3 grid(col_blocks, n_row_chunks);
-        if (r_dtype == MKA_BF16) {
-            auto* r = static_cast<const __nv_bfloat16*>(R);
-            if (vec) router_bwd_partial8_kernel<<<grid, 256, 0, st>>>(r, dG, rows, D, n_row_chunks, partial, db_part);
-            else router_bwd_partial_kernel<<<grid, 256, 0, st>>>(r, dG, rows, D, n_row_chunks, partial);
-        } else {
-            auto* r = static_cast<const float*>(R);
-            if (vec) router_bwd_partial8_kernel<<<grid, 256, 0, st>>>(r, dG, rows, D, n_row_chunks, partial, db_part);
-            else router_bwd_partial_kernel<<<grid, 256, 0, st>>>(r, dG, rows, D, n_row_chunks, partial);
-        }
+        auto launch = [&](const auto* r) {
+            using T = std::remove_cv_t<std::remove_pointer_t<decltype(r)>>;
+            auto kern = cols == 8 ? router_bwd_partial_vec_kernel<T, 8> : (cols == 4 ? router_bwd_partial_vec_kernel<T, 4> : router_bwd_partial_kernel<T>);
+            kern<<<grid, 256, 0, st>>>(r, dG, rows, D, n_row_chunks, partial, db_part);
+        };
+        if (r_dtype == MKA_BF16) launch(static_cast<const __nv_bfloat16*>(R));
+        else launch(static_cast<const float*>(R));
     }
     const int blocks = (dW_r ? (D * 3 + 31) / 32 : 0) + (db_r ? 1 : 0);
     if (blocks) router_bwd_reduce_kernel<<<blocks, 256, 0, st>>>(partial, dG, rows, D, n_row_chunks, db_part, dW_r, db_r);
