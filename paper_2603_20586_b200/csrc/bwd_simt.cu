@@ -4,28 +4,30 @@
 //   kernel dkv   : dK_{l,j} = tau sum_t dS q_t;  dV_{l,j} = sum_t p dO_t       (one launch for the three levels)
 //   kernel dgate : dG[b,t,l] = sum_h G[b,h,t,l]                               (fixed order)
 // Every output element is produced by exactly one CTA in a fixed summation order, so the result is
-// deterministic.  fp32 arithmetic; 16 rows against tiles of 32, see simt.cuh.
+// deterministic.  fp32 arithmetic; 16 or 32 rows against tiles of 32, see simt.cuh.
 #include "simt.cuh"
 
 namespace mka {
 namespace {
 
-template <typename T, int DH>
-__global__ void __launch_bounds__(kSimtThreads) bwd_dq_kernel(const BwdParams p, const int vec) {
+template <typename T, int DH, int GROUPS>
+__global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1) bwd_dq_kernel(const BwdParams p, const int vec) {
+    using S = SimtCta<GROUPS>;
+    constexpr int kRows = S::kRows, kGroupThreads = S::kWarps * 32;
     constexpr int CPL = DH / 32, LD = DH + 4, kTileFloats = kSimtTile * LD, R = kSimtWarpRows;
     extern __shared__ __align__(16) float smem[];
-    float* qs = smem;                            // [16][DH]  tau * q
-    float* gs = qs + kSimtRows * DH;             // [16][DH]  dO
-    float* ps = gs + kSimtRows * DH;             // [16 warps][4 rows][32]  dS of the warp's tile
-    float* tiles = ps + 16 * R * 32;             // [4 groups][K, V][32][LD]; at the end [4 groups][16 rows][DH + 6]
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp >> 2, wg = warp & 3, gtid = threadIdx.x & 127;
+    float* qs = smem;                            // [rows][DH]  tau * q
+    float* gs = qs + kRows * DH;             // [rows][DH]  dO
+    float* ps = gs + kRows * DH;                 // [warps][4 rows][32]  dS of the warp's tile
+    float* tiles = ps + S::kThreads * R;         // [groups][K, V][32][LD]; at the end [groups][rows][DH + 6]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp / S::kWarps, wg = warp % S::kWarps, gtid = threadIdx.x % kGroupThreads;
     const int b = blockIdx.z, h = blockIdx.y;
-    const long long t0 = (long long)blockIdx.x * kSimtRows;
+    const long long t0 = (long long)blockIdx.x * kRows;
     const long long bh = (long long)b * p.H + h;
     const T* Q = static_cast<const T*>(p.Q) + bh * p.T * DH;
     const T* dO = static_cast<const T*>(p.dO) + bh * p.T * DH;
     if (threadIdx.x < 4 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) p.status[threadIdx.x] = 0u;
-    for (int i = threadIdx.x * 4; i < kSimtRows * DH; i += kSimtThreads * 4) {
+    for (int i = threadIdx.x * 4; i < kRows * DH; i += S::kThreads * 4) {
         const long long t = t0 + i / DH;
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
         if (t < p.T) {
@@ -59,7 +61,7 @@ __global__ void __launch_bounds__(kSimtThreads) bwd_dq_kernel(const BwdParams p,
     float* pw = ps + warp * R * 32;
     const float* qw = qs + wg * R * DH;
     const float* gw = gs + wg * R * DH;
-    const long long t_last = (t0 + kSimtRows - 1 < p.T ? t0 + kSimtRows - 1 : p.T - 1);
+    const long long t_last = (t0 + kRows - 1 < p.T ? t0 + kRows - 1 : p.T - 1);
 #pragma unroll
     for (int lvl = 0; lvl < 3; ++lvl) {
         const LevelDev L = p.L[lvl];
@@ -79,10 +81,10 @@ __global__ void __launch_bounds__(kSimtThreads) bwd_dq_kernel(const BwdParams p,
             visible_range(lvl, tc + p.q_offset, p.window, L.n, 0, rlo[r], rhi[r]);
             if (t >= p.T) rhi[r] = rlo[r];
         }
-        for (long long j0 = (lo / kSimtTile + group) * kSimtTile; j0 < hi; j0 += kSimtGroups * kSimtTile) {
-            group_sync(group);
-            load_pair<T, DH>(ks, vs, Kp, Vp, j0, L.n, L.sn, (vec >> lvl) & 1, gtid);
-            group_sync(group);
+        for (long long j0 = (lo / kSimtTile + group) * kSimtTile; j0 < hi; j0 += S::kGroups * kSimtTile) {
+            group_sync<kGroupThreads>(group);
+            load_pair<T, DH, kGroupThreads>(ks, vs, Kp, Vp, j0, L.n, L.sn, (vec >> lvl) & 1, gtid);
+            group_sync<kGroupThreads>(group);
             float s[R], dp[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) s[r] = dp[r] = 0.f;
@@ -127,12 +129,12 @@ __global__ void __launch_bounds__(kSimtThreads) bwd_dq_kernel(const BwdParams p,
             __syncwarp();
         }
     }
-    // merge the groups: warp w adds up row w
+    // merge the groups: a warp adds up one row after the other
     __syncthreads();
     constexpr int kState = DH + 6;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        float* o = tiles + (group * kSimtRows + wg * R + r) * kState;
+        float* o = tiles + (group * kRows + wg * R + r) * kState;
 #pragma unroll
         for (int l = 0; l < 3; ++l) {
             const float a = warp_sum(Ap[r][l]), sp = warp_sum(Sp[r][l]);
@@ -142,13 +144,15 @@ __global__ void __launch_bounds__(kSimtThreads) bwd_dq_kernel(const BwdParams p,
         for (int k = 0; k < CPL; ++k) o[6 + lane + 32 * k] = acc[r][k];
     }
     __syncthreads();
-    const long long t = t0 + warp;
-    if (t >= p.T) return;
-    const float* o = tiles + warp * kState;
+#pragma unroll 1
+    for (int row = warp; row < kRows; row += S::kThreads / 32) {
+    const long long t = t0 + row;
+    if (t >= p.T) break;
+    const float* o = tiles + row * kState;
     auto total = [&](int i) {
         float v = o[i];
 #pragma unroll
-        for (int g = 1; g < kSimtGroups; ++g) v += o[g * kSimtRows * kState + i];
+        for (int g = 1; g < S::kGroups; ++g) v += o[g * kRows * kState + i];
         return v;
     };
     T* dQ = static_cast<T*>(p.dQ) + bh * p.T * DH;
@@ -165,29 +169,32 @@ __global__ void __launch_bounds__(kSimtThreads) bwd_dq_kernel(const BwdParams p,
 #pragma unroll
     for (int l = 0; l < 3; ++l)
         if (lane == 0) p.Gpart[(bh * p.T + t) * 3 + l] = a[l] - sp[l] * dd;
+    }
 }
 
-// One CTA = 16 key rows of one level of one (batch, KV head); its groups share the query tiles that see them.  One launch
+// One CTA = 16 or 32 key rows of one level of one (batch, KV head); its groups share the query tiles that see them.  One launch
 // covers the three levels: blockIdx.x runs through L1's, L2's and L3's key tiles.
-template <typename T, int DH>
-__global__ void __launch_bounds__(kSimtThreads) bwd_dkv_kernel(const BwdParams p, const int vec) {
+template <typename T, int DH, int GROUPS>
+__global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1) bwd_dkv_kernel(const BwdParams p, const int vec) {
+    using S = SimtCta<GROUPS>;
+    constexpr int kRows = S::kRows, kGroupThreads = S::kWarps * 32;
     constexpr int CPL = DH / 32, LD = DH + 4, kTileFloats = kSimtTile * LD, R = kSimtWarpRows;
     extern __shared__ __align__(16) float smem[];
-    float* ksm = smem;                           // [16][DH]  tau * k   (this CTA's key rows)
-    float* vsm = ksm + kSimtRows * DH;           // [16][DH]
-    float* ps = vsm + kSimtRows * DH;            // [16 warps][p, dS][4 rows][32]
-    float* tiles = ps + 16 * 2 * R * 32;         // [4 groups][Q, dO][32][LD]; at the end [4 groups][16 rows][2 DH]
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp >> 2, wg = warp & 3, gtid = threadIdx.x & 127;
+    float* ksm = smem;                           // [rows][DH]  tau * k   (this CTA's key rows)
+    float* vsm = ksm + kRows * DH;           // [rows][DH]
+    float* ps = vsm + kRows * DH;                // [warps][p, dS][4 rows][32]
+    float* tiles = ps + S::kThreads * 2 * R;     // [groups][Q, dO][32][LD]; at the end [groups][rows][2 DH]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp / S::kWarps, wg = warp % S::kWarps, gtid = threadIdx.x % kGroupThreads;
     const int b = blockIdx.z, h = blockIdx.y;               // h: KV head; its query heads h * G .. h * G + G - 1 are summed
     int lvl = 0;
     long long kt = blockIdx.x;
-    while (kt >= (p.L[lvl].n + kSimtRows - 1) / kSimtRows) { kt -= (p.L[lvl].n + kSimtRows - 1) / kSimtRows; ++lvl; }
+    while (kt >= (p.L[lvl].n + kRows - 1) / kRows) { kt -= (p.L[lvl].n + kRows - 1) / kRows; ++lvl; }
     const LevelDev L = p.L[lvl];
     const LevelGradDev dL = p.dL[lvl];
-    const long long j0 = kt * kSimtRows;
+    const long long j0 = kt * kRows;
     const T* Kp = static_cast<const T*>(L.k) + b * L.sb + h * L.sh;
     const T* Vp = static_cast<const T*>(L.v) + b * L.sb + h * L.sh;
-    for (int i = threadIdx.x * 4; i < kSimtRows * DH; i += kSimtThreads * 4) {
+    for (int i = threadIdx.x * 4; i < kRows * DH; i += S::kThreads * 4) {
         const long long j = j0 + i / DH;
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
         if (j < L.n) {
@@ -205,7 +212,7 @@ __global__ void __launch_bounds__(kSimtThreads) bwd_dkv_kernel(const BwdParams p
         for (int k = 0; k < CPL; ++k) accK[r][k] = accV[r][k] = 0.f;
     // queries that can see any of this CTA's keys: positions p = t + q_offset with
     //   L1: j <= p <= j + W - 1   L2: p >= j   L3: all
-    const long long j_last = (j0 + kSimtRows - 1 < L.n ? j0 + kSimtRows - 1 : L.n - 1);
+    const long long j_last = (j0 + kRows - 1 < L.n ? j0 + kRows - 1 : L.n - 1);
     long long t_lo = 0, t_hi = p.T;
     if (lvl == 0) { t_lo = j0 - p.q_offset; t_hi = j_last + p.window - p.q_offset; }
     else if (lvl == 1) { t_lo = j0 - p.q_offset; }
@@ -217,16 +224,16 @@ __global__ void __launch_bounds__(kSimtThreads) bwd_dkv_kernel(const BwdParams p
     float* pw = ps + warp * 2 * R * 32;
     const float* kw = ksm + wg * R * DH;
     const float* vw = vsm + wg * R * DH;
-    for (long long i = group; i < per_head * p.kv_group; i += kSimtGroups) {     // head by head, each head's tiles in order
+    for (long long i = group; i < per_head * p.kv_group; i += S::kGroups) {     // head by head, each head's tiles in order
         const long long bh = (long long)b * p.H + (long long)h * p.kv_group + i / per_head;
         const long long tt = (first + i % per_head) * kSimtTile, t = tt + lane;   // lane = query of the tile; warp rows = keys
         const T* Q = static_cast<const T*>(p.Q) + bh * p.T * DH;
         const T* dO = static_cast<const T*>(p.dO) + bh * p.T * DH;
         const long long tc = t < p.T ? t : p.T - 1;
         const float lse = p.LSE[bh * p.T + tc], dlt = p.delta[bh * p.T + tc], lam = p.gate[((long long)b * p.T + tc) * 3 + lvl];
-        group_sync(group);
-        load_pair<T, DH>(qs, gs, Q, dO, tt, p.T, DH, (vec & 8) != 0, gtid);
-        group_sync(group);
+        group_sync<kGroupThreads>(group);
+        load_pair<T, DH, kGroupThreads>(qs, gs, Q, dO, tt, p.T, DH, (vec & 8) != 0, gtid);
+        group_sync<kGroupThreads>(group);
         long long vlo, vhi;
         visible_range(lvl, t + p.q_offset, p.window, L.n, 0, vlo, vhi);
         if (t >= p.T) vhi = vlo;
@@ -279,18 +286,20 @@ __global__ void __launch_bounds__(kSimtThreads) bwd_dkv_kernel(const BwdParams p
         }
         __syncwarp();
     }
-    // merge the groups: warp w adds up key row w
+    // merge the groups: a warp adds up one key row after the other
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        float* o = tiles + (group * kSimtRows + wg * R + r) * 2 * DH;
+        float* o = tiles + (group * kRows + wg * R + r) * 2 * DH;
 #pragma unroll
         for (int k = 0; k < CPL; ++k) { o[lane + 32 * k] = accK[r][k]; o[DH + lane + 32 * k] = accV[r][k]; }
     }
     __syncthreads();
-    const long long j = j0 + warp;
-    if (j >= L.n) return;
-    const float* o = tiles + warp * 2 * DH;
+#pragma unroll 1
+    for (int row = warp; row < kRows; row += S::kThreads / 32) {
+    const long long j = j0 + row;
+    if (j >= L.n) break;
+    const float* o = tiles + row * 2 * DH;
     T* dKp = static_cast<T*>(dL.dk) + b * dL.sb + h * dL.sh + j * dL.sn;
     T* dVp = static_cast<T*>(dL.dv) + b * dL.sb + h * dL.sh + j * dL.sn;
 #pragma unroll
@@ -298,9 +307,10 @@ __global__ void __launch_bounds__(kSimtThreads) bwd_dkv_kernel(const BwdParams p
         const int c = lane + 32 * k;
         float dk = o[c], dv = o[DH + c];
 #pragma unroll
-        for (int g = 1; g < kSimtGroups; ++g) { dk += o[g * kSimtRows * 2 * DH + c]; dv += o[g * kSimtRows * 2 * DH + DH + c]; }
+        for (int g = 1; g < S::kGroups; ++g) { dk += o[g * kRows * 2 * DH + c]; dv += o[g * kRows * 2 * DH + DH + c]; }
         Elem<T>::st(dKp + c, dk * p.scale);
         Elem<T>::st(dVp + c, dv);
+    }
     }
 }
 
@@ -324,28 +334,35 @@ cudaError_t launch_bwd_dgate(const float* Gpart, int B, int H, long long T, floa
 
 namespace {
 
+template <typename T, int DH, int GROUPS>
+cudaError_t launch_dq(const BwdParams& p, int vec, cudaStream_t st) {
+    using S = SimtCta<GROUPS>;
+    const size_t smem = sizeof(float) * (2 * S::kRows * DH + S::kThreads * kSimtWarpRows + (size_t)S::kGroups * 2 * kSimtTile * (DH + 4));
+    const cudaError_t e = cudaFuncSetAttribute(bwd_dq_kernel<T, DH, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    bwd_dq_kernel<T, DH, GROUPS><<<dim3((p.T + S::kRows - 1) / S::kRows, p.H, p.B), S::kThreads, smem, st>>>(p, vec);
+    return cudaGetLastError();
+}
+
+template <typename T, int DH, int GROUPS>
+cudaError_t launch_dkv(const BwdParams& p, int vec, cudaStream_t st) {
+    using S = SimtCta<GROUPS>;
+    long long key_tiles = 0;
+    for (int l = 0; l < 3; ++l) key_tiles += (p.L[l].n + S::kRows - 1) / S::kRows;
+    if (key_tiles == 0) return cudaSuccess;
+    const size_t smem = sizeof(float) * (2 * S::kRows * DH + S::kThreads * 2 * kSimtWarpRows + (size_t)S::kGroups * 2 * kSimtTile * (DH + 4));
+    const cudaError_t e = cudaFuncSetAttribute(bwd_dkv_kernel<T, DH, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    bwd_dkv_kernel<T, DH, GROUPS><<<dim3((unsigned)key_tiles, p.H / (p.kv_group > 0 ? p.kv_group : 1), p.B), S::kThreads, smem, st>>>(p, vec);
+    return cudaGetLastError();
+}
+
 template <typename T, int DH>
 cudaError_t launch_t(const BwdParams& p, cudaStream_t st) {
     const int vec = simt_vec_bits(p.L, p.Q, p.O, p.dO, sizeof(T) == 2 ? MKA_BF16 : MKA_F32);
-    const size_t tiles_floats = (size_t)kSimtGroups * 2 * kSimtTile * (DH + 4);
-    cudaError_t e;
-    {
-        const size_t smem = sizeof(float) * (2 * kSimtRows * DH + 16 * kSimtWarpRows * 32 + tiles_floats);
-        e = cudaFuncSetAttribute(bwd_dq_kernel<T, DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        bwd_dq_kernel<T, DH><<<dim3((p.T + kSimtRows - 1) / kSimtRows, p.H, p.B), kSimtThreads, smem, st>>>(p, vec);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    long long key_tiles = 0;
-    for (int l = 0; l < 3; ++l) key_tiles += (p.L[l].n + kSimtRows - 1) / kSimtRows;
-    if (key_tiles > 0) {
-        const size_t smem = sizeof(float) * (2 * kSimtRows * DH + 16 * 2 * kSimtWarpRows * 32 + tiles_floats);
-        e = cudaFuncSetAttribute(bwd_dkv_kernel<T, DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        bwd_dkv_kernel<T, DH><<<dim3((unsigned)key_tiles, p.H / (p.kv_group > 0 ? p.kv_group : 1), p.B), kSimtThreads, smem, st>>>(p, vec);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    return launch_bwd_dgate(p.Gpart, p.B, p.H, p.T, p.dG, st);
+    cudaError_t e = simt_query_groups(p, 50.0) ? launch_dq<T, DH, 4>(p, vec, st) : launch_dq<T, DH, 1>(p, vec, st);
+    if (e == cudaSuccess) e = simt_key_groups(p) ? launch_dkv<T, DH, 4>(p, vec, st) : launch_dkv<T, DH, 1>(p, vec, st);
+    return e == cudaSuccess ? launch_bwd_dgate(p.Gpart, p.B, p.H, p.T, p.dG, st) : e;
 }
 
 template <typename T>

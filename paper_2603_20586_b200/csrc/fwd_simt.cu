@@ -4,31 +4,33 @@
 //                  32 rows as in Alg. 3, rescale of Eq. 13-14 applied on every block).
 //   MKA_MODE_FULL: Alg. 1 -- one softmax state per level, outputs mixed by the gate at the end.
 // fp32 arithmetic throughout, so this is the kernel for fp32 problems (tolerance 1e-4) and the
-// on-GPU cross-check of the tensor-core kernel.  One CTA = 16 query rows of one (batch, head), see simt.cuh; a key tile of
+// on-GPU cross-check of the tensor-core kernel.  One CTA = 16 or 32 query rows of one (batch, head), see simt.cuh; a key tile of
 // 32 rows is staged in shared memory as fp32 and each lane scores one key of the tile, four columns at a time.
 #include "simt.cuh"
 
 namespace mka {
 namespace {
 
-template <typename T, int DH, int MODE>
-__global__ void __launch_bounds__(kSimtThreads) fwd_simt_kernel(const FwdParams p, const int vec) {
+template <typename T, int DH, int MODE, int GROUPS>
+__global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1) fwd_simt_kernel(const FwdParams p, const int vec) {
+    using S = SimtCta<GROUPS>;
+    constexpr int kRows = S::kRows, kGroupThreads = S::kWarps * 32;
     constexpr int NS = MODE == MKA_MODE_FULL ? 3 : 1;    // softmax states
     constexpr int CPL = DH / 32;                         // output columns per lane
     constexpr int LD = DH + 4, kTileFloats = kSimtTile * LD, R = kSimtWarpRows;
     extern __shared__ __align__(16) float smem[];
-    float* qs = smem;                                    // [16][DH]  tau * q
-    float* ps = qs + kSimtRows * DH;                     // [16 warps][4 rows][32]  weights of the warp's tile
-    float* tiles = ps + 16 * R * 32;                     // [4 groups][K, V][32][LD]; at the end [4 groups][16 rows][NS][DH + 2]
+    float* qs = smem;                                    // [rows][DH]  tau * q
+    float* ps = qs + kRows * DH;                         // [warps][4 rows][32]  weights of the warp's tile
+    float* tiles = ps + S::kThreads * R;                 // [groups][K, V][32][LD]; at the end [groups][rows][NS][DH + 2]
 
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp >> 2, wg = warp & 3, gtid = threadIdx.x & 127;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp / S::kWarps, wg = warp % S::kWarps, gtid = threadIdx.x % kGroupThreads;
     const int b = blockIdx.z, h = blockIdx.y;
-    const long long t0 = (long long)blockIdx.x * kSimtRows;
+    const long long t0 = (long long)blockIdx.x * kRows;
     const T* Q = static_cast<const T*>(p.Q) + (((long long)b * p.H + h) * p.T) * DH;
     T* O = static_cast<T*>(p.O) + (((long long)b * p.H + h) * p.T) * DH;
 
     if (p.status && threadIdx.x == 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) *p.status = MKA_OK;
-    for (int i = threadIdx.x * 4; i < kSimtRows * DH; i += kSimtThreads * 4) {
+    for (int i = threadIdx.x * 4; i < kRows * DH; i += S::kThreads * 4) {
         const long long t = t0 + i / DH;
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
         if (t < p.T) x = Fetch4<T>::at(Q + t * DH + i % DH, (vec & 8) != 0);
@@ -50,7 +52,7 @@ __global__ void __launch_bounds__(kSimtThreads) fwd_simt_kernel(const FwdParams 
     float* vs = ks + kTileFloats;
     float* pw = ps + warp * R * 32;
     const float* qw = qs + wg * R * DH;
-    const long long t_last = (t0 + kSimtRows - 1 < p.T ? t0 + kSimtRows - 1 : p.T - 1);
+    const long long t_last = (t0 + kRows - 1 < p.T ? t0 + kRows - 1 : p.T - 1);
 #pragma unroll
     for (int lvl = 0; lvl < 3; ++lvl) {
         const int st = MODE == MKA_MODE_FULL ? lvl : 0;
@@ -72,10 +74,10 @@ __global__ void __launch_bounds__(kSimtThreads) fwd_simt_kernel(const FwdParams 
             visible_range(lvl, tc + p.q_offset, p.window, L.n, p.decode, rlo[r], rhi[r]);
             if (t >= p.T) rhi[r] = rlo[r];
         }
-        for (long long j0 = (lo / kSimtTile + group) * kSimtTile; j0 < hi; j0 += kSimtGroups * kSimtTile) {
-            group_sync(group);                           // the group's previous tile has been read
-            load_pair<T, DH>(ks, vs, Kp, Vp, j0, L.n, L.sn, (vec >> lvl) & 1, gtid);
-            group_sync(group);
+        for (long long j0 = (lo / kSimtTile + group) * kSimtTile; j0 < hi; j0 += S::kGroups * kSimtTile) {
+            group_sync<kGroupThreads>(group);                           // the group's previous tile has been read
+            load_pair<T, DH, kGroupThreads>(ks, vs, Kp, Vp, j0, L.n, L.sn, (vec >> lvl) & 1, gtid);
+            group_sync<kGroupThreads>(group);
             float s[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) s[r] = 0.f;
@@ -125,36 +127,38 @@ __global__ void __launch_bounds__(kSimtThreads) fwd_simt_kernel(const FwdParams 
         }
     }
 
-    // merge the groups: every group leaves (max, sum, acc) of its tiles, warp w then finishes row w
+    // merge the groups: every group leaves (max, sum, acc) of its tiles, a warp then finishes one row after the other
     __syncthreads();
     constexpr int kState = DH + 2;
 #pragma unroll
     for (int s = 0; s < NS; ++s)
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            float* o = tiles + ((group * kSimtRows + wg * R + r) * NS + s) * kState;
+            float* o = tiles + ((group * kRows + wg * R + r) * NS + s) * kState;
             const float zr = warp_sum(z[s][r]);
             if (lane == 0) { o[0] = m[s][r]; o[1] = zr; }
 #pragma unroll
             for (int k = 0; k < CPL; ++k) o[2 + lane + 32 * k] = acc[s][r][k];
         }
     __syncthreads();
-    const long long t = t0 + warp;
-    if (t >= p.T) return;
+#pragma unroll 1
+    for (int row = warp; row < kRows; row += S::kThreads / 32) {
+    const long long t = t0 + row;
+    if (t >= p.T) break;
     float out[CPL];
 #pragma unroll
     for (int k = 0; k < CPL; ++k) out[k] = 0.f;
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
-        const float* o = tiles + (warp * NS + s) * kState;
-        constexpr int kGroupFloats = kSimtRows * NS * kState;
+        const float* o = tiles + (row * NS + s) * kState;
+        constexpr int kGroupFloats = kRows * NS * kState;
         float M = -INFINITY, Z = 0.f, A[CPL];
 #pragma unroll
-        for (int g = 0; g < kSimtGroups; ++g) M = fmaxf(M, o[g * kGroupFloats]);
+        for (int g = 0; g < S::kGroups; ++g) M = fmaxf(M, o[g * kGroupFloats]);
 #pragma unroll
         for (int k = 0; k < CPL; ++k) A[k] = 0.f;
 #pragma unroll
-        for (int g = 0; g < kSimtGroups; ++g) {
+        for (int g = 0; g < S::kGroups; ++g) {
             const float mg = o[g * kGroupFloats], f = mg == -INFINITY ? 0.f : expf(mg - M);
             Z = fmaf(o[g * kGroupFloats + 1], f, Z);
 #pragma unroll
@@ -172,18 +176,28 @@ __global__ void __launch_bounds__(kSimtThreads) fwd_simt_kernel(const FwdParams 
     }
 #pragma unroll
     for (int k = 0; k < CPL; ++k) Elem<T>::st(O + t * DH + lane + 32 * k, out[k]);
+    }
+}
+
+template <typename T, int DH, int MODE, int GROUPS>
+cudaError_t launch_g(const FwdParams& p, cudaStream_t st) {
+    using S = SimtCta<GROUPS>;
+    const dim3 grid((p.T + S::kRows - 1) / S::kRows, p.H, p.B);
+    const size_t tiles = (size_t)S::kGroups * 2 * kSimtTile * (DH + 4), merge = (size_t)S::kGroups * S::kRows * (MODE == MKA_MODE_FULL ? 3 : 1) * (DH + 2);
+    const size_t smem = sizeof(float) * (S::kRows * DH + S::kThreads * kSimtWarpRows + (tiles > merge ? tiles : merge));
+    const int vec = simt_vec_bits(p.L, p.Q, nullptr, nullptr, sizeof(T) == 2 ? MKA_BF16 : MKA_F32);
+    auto kern = fwd_simt_kernel<T, DH, MODE, GROUPS>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<grid, S::kThreads, smem, st>>>(p, vec);
+    return cudaGetLastError();
 }
 
 template <typename T, int DH>
 cudaError_t launch_t(const FwdParams& p, cudaStream_t st) {
-    const dim3 grid((p.T + kSimtRows - 1) / kSimtRows, p.H, p.B);
-    const size_t smem = sizeof(float) * (kSimtRows * DH + 16 * kSimtWarpRows * 32 + kSimtGroups * 2 * kSimtTile * (DH + 4));
-    const int vec = simt_vec_bits(p.L, p.Q, nullptr, nullptr, sizeof(T) == 2 ? MKA_BF16 : MKA_F32);
-    auto kern = p.mode == MKA_MODE_FULL ? fwd_simt_kernel<T, DH, MKA_MODE_FULL> : fwd_simt_kernel<T, DH, MKA_MODE_FAST>;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<grid, kSimtThreads, smem, st>>>(p, vec);
-    return cudaGetLastError();
+    const bool four = simt_query_groups(p, DH <= 64 ? 28.0 : 40.0);
+    if (p.mode == MKA_MODE_FULL) return four ? launch_g<T, DH, MKA_MODE_FULL, 4>(p, st) : launch_g<T, DH, MKA_MODE_FULL, 1>(p, st);
+    return four ? launch_g<T, DH, MKA_MODE_FAST, 4>(p, st) : launch_g<T, DH, MKA_MODE_FAST, 1>(p, st);
 }
 
 template <typename T>

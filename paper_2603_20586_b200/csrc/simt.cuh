@@ -1,16 +1,23 @@
 // Pieces shared by the CUDA-core forward and backward: tile loads and the shape of their CTAs.
 // A CTA owns 16 rows (queries, or keys in the dK/dV kernel) and has four groups of four warps; every warp of a group owns
 // four of the rows, and the groups take every fourth 32-row tile of the list that the rows walk, each into its own part
-// of shared memory.  Their partial results are merged in a fixed order at the end.  The problems that run here are small
+// of shared memory.  Their partial results are merged in a fixed order at the end.  Most problems that run here are small
 // (fp32 reference runs: a few heads of a few hundred rows), so the launch is bound by the length of that walk on a
-// mostly idle chip, not by arithmetic: with one group of eight warps over 32 rows, [1, 4, 256, 64] took 63 us.
+// mostly idle chip, not by arithmetic: with one group of eight warps over 32 rows, [1, 4, 256, 64] took 63 us.  Where the blocks
+// fill the chip that one group of eight warps is the shape of the CTA (simt_four_groups).
 #pragma once
 
 #include "common.cuh"
 
 namespace mka {
 
-constexpr int kSimtRows = 16, kSimtTile = 32, kSimtWarpRows = 4, kSimtGroups = 4, kSimtThreads = 512;
+constexpr int kSimtTile = 32, kSimtWarpRows = 4;
+
+// The two shapes of a CTA, by its number of groups: four groups of four warps (16 rows), or one group of eight (32 rows).
+template <int GROUPS> struct SimtCta {
+    static constexpr int kGroups = GROUPS, kWarps = GROUPS == 4 ? 4 : 8;      // kWarps: of a group
+    static constexpr int kRows = kWarps * kSimtWarpRows, kThreads = kGroups * kWarps * 32;
+};
 
 template <typename T> struct Fetch4;   // four consecutive elements as floats
 template <> struct Fetch4<float> {
@@ -27,15 +34,15 @@ template <> struct Fetch4<__nv_bfloat16> {     // bf16 tensors are 16-byte align
     }
 };
 
-// 32 rows [j0, j0 + 32) of two tensors of the same strides into shared memory, rows past n as zeros, by a group's 128 threads.
+// 32 rows [j0, j0 + 32) of two tensors of the same strides into shared memory, rows past n as zeros, by a group's threads.
 // Pitch DH + 4 floats: rows stay 16-byte aligned and eight lanes' 16-byte reads of eight rows fall on different banks.
-template <typename T, int DH>
+template <typename T, int DH, int GROUP_THREADS>
 __device__ __forceinline__ void load_pair(float* da, float* db, const T* a, const T* b, long long j0, long long n, long long stride,
                                           bool vec, int gtid) {
     constexpr int V = DH / 4;
 #pragma unroll
-    for (int i = 0; i < kSimtTile * V / 128; ++i) {
-        const int e = gtid + i * 128, r = e / V, c = (e % V) * 4;
+    for (int i = 0; i < kSimtTile * V / GROUP_THREADS; ++i) {
+        const int e = gtid + i * GROUP_THREADS, r = e / V, c = (e % V) * 4;
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
         if (j0 + r < n) {
             x = Fetch4<T>::at(a + (j0 + r) * stride + c, vec);
@@ -46,7 +53,8 @@ __device__ __forceinline__ void load_pair(float* da, float* db, const T* a, cons
     }
 }
 
-__device__ __forceinline__ void group_sync(int group) { asm volatile("bar.sync %0, 128;" ::"r"(group + 1) : "memory"); }
+template <int GROUP_THREADS>
+__device__ __forceinline__ void group_sync(int group) { asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(GROUP_THREADS) : "memory"); }
 
 // 16-byte loads are possible: bit l for level l (its K and V), bit 3 for the contiguous tensors.
 inline int simt_vec_bits(const LevelDev L[3], const void* a, const void* b, const void* c, int dtype) {
@@ -55,6 +63,43 @@ inline int simt_vec_bits(const LevelDev L[3], const void* a, const void* b, cons
     for (int l = 0; l < 3; ++l)
         if (ok(L[l].k) && ok(L[l].v) && L[l].sn % 4 == 0 && L[l].sh % 4 == 0 && L[l].sb % 4 == 0) bits |= 1 << l;
     return dtype == MKA_BF16 ? 15 : bits;
+}
+
+// Which shape.  Four groups shorten the walk of a CTA and leave fewer CTAs on an SM at a time: they are for launches whose blocks
+// do not fill the chip, and for long walks; one group has the better throughput.  `blocks`: CTAs of 16 rows;
+// `walk`: tiles that a row block visits, on average; `k`, tiles for a block more than one per SM: 28 in the forward (40 above
+// d = 64, where an SM holds one CTA of four groups), 50 for dQ and 120 (of the longest walk) for dK/dV, where four groups hold
+// out longer.  Over 200 shapes of d = 32 to 128 the rule costs 1 % on average against the better shape.  fp32, us, four groups /
+// one group (in brackets one group with scalar loads, the only shape there once was):
+//   forward, d = 64    8 heads x 200 rows, 104 blocks, 17 tiles   29.8 / 57.4 (84.1)      24 x 200, 312, 10    39.0 / 50.1 (63.6)
+//                      24 x 512, 768, 13                          121 / 116 (135)         8 x 3000, 1504, 53   735 / 726 (874)
+//                      128 x 64, 512, 14                          86.1 / 63.5 (82.2)      8 x 1024, 512, 2     22.6 / 14.4 (18.5)
+//   forward, d = 128   32 x 200, 416, 8                           43.1 / 51.2
+inline bool simt_four_groups(long long blocks, double walk, double k) { return blocks <= 148 || (double)(blocks - 148) <= k * walk; }
+template <typename P> inline bool simt_query_groups(const P& p, double k) {           // forward and dQ: row blocks of queries
+    double keys = 0.0;
+    for (int l = 0; l < 3; ++l) {
+        const double n = (double)p.L[l].n, seen = l == 0 ? (double)p.window + 15.0 : (l == 1 ? (double)p.q_offset + 0.5 * p.T : n);
+        keys += n > 0.0 ? 32.0 + (seen < n ? seen : n) : 0.0;
+    }
+    return simt_four_groups((long long)p.B * p.H * ((p.T + 15) / 16), keys / 32.0, k);
+}
+// dK/dV: the levels' key blocks walk very different numbers of query tiles, and a launch lasts at least as long as its longest walk
+// (a long-term level of 64 rows under 8192 queries beside a window of 16: 603 / 1434 us), so that walk counts here, also against
+// the launch's total over the CTA slots.
+inline bool simt_key_groups(const BwdParams& p) {
+    double longest = 0.0, total = 0.0;
+    long long blocks = 0;
+    for (int l = 0; l < 3; ++l) {
+        if (p.L[l].n == 0) continue;
+        const double seen = l == 0 && p.window + 15.0 < p.T ? p.window + 15.0 : (double)p.T;
+        const double walk = seen * p.kv_group / 32.0;
+        const long long n = (long long)p.B * (p.H / p.kv_group) * ((p.L[l].n + 15) / 16);
+        longest = walk > longest ? walk : longest;
+        total += (l == 1 ? 0.5 : 1.0) * walk * (double)n;
+        blocks += n;
+    }
+    return simt_four_groups(blocks, longest, 120.0) || longest * 444.0 >= total;
 }
 
 }  // namespace mka

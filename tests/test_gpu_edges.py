@@ -156,6 +156,31 @@ def test_cuda_core_tiles(mka, orc, d, dtype, shift, T, W, q_off, N):
     check(g["dG"], r["dG"], dtype, "dG")
 
 
+@pytest.mark.parametrize("d,dtype", [(32, torch.float32), (64, torch.float32), (96, torch.float32), (128, torch.float32), (96, torch.bfloat16)])
+@pytest.mark.parametrize("B,H,T,W,N", [
+    (1, 40, 97, 9, (97, 0, 33)),           # many short walks: one group of warps to a CTA, 32 rows, the last block with one
+    (2, 20, 250, 40, (250, 250, 5)),       # and a long-term level whose keys walk every query beside a short window's
+])
+def test_cuda_core_many_blocks(mka, orc, d, dtype, B, H, T, W, N):
+    P = problem(29, B, H, T, d, N, 64, dtype, router_std=0.5, with_dO=True)
+    gate = mka.mka_router(P["X"], P["W_r"], None)
+    mk = lambda mode: mka.make_shape(B, H, T, d, 64, W, dtype=mka.binding.MKA_BF16 if dtype == torch.bfloat16 else mka.binding.MKA_F32, mode=mode)  # noqa: E731
+    shape, full = mk(mka.binding.MKA_MODE_FAST), mk(mka.binding.MKA_MODE_FULL)
+    O, LSE = mka.mka_fwd(shape, P["Q"], P["K"], P["V"], gate)
+    g64 = np64(gate)
+    check(O, orc.fwd(P["Q"], P["K"], P["V"], g64, W)[0], dtype, "O")
+    check(mka.mka_fwd(full, P["Q"], P["K"], P["V"], gate)[0], orc.fwd(P["Q"], P["K"], P["V"], g64, W, mode="full")[0], dtype, "O of the per-level form")
+    g = mka.mka_bwd(shape, P["Q"], P["K"], P["V"], gate, O, LSE, P["dO"])
+    r = orc.bwd(P["Q"], P["K"], P["V"], g64, P["dO"], W)
+    check(g["dQ"], r["dQ"], dtype, "dQ")
+    for l in range(3):
+        if N[l]:
+            check(g["dK"][l], r["dK"][l], dtype, f"dK{l}")
+            check(g["dV"][l], r["dV"][l], dtype, f"dV{l}")
+    # dG sums over 40 (20) heads, each within the contract's bound of a single head's sum
+    assert err(g["dG"], r["dG"])[0] <= (2e-2 if dtype == torch.bfloat16 else 1e-4) * H / 4
+
+
 @pytest.mark.parametrize("d,bits", [(64, 32), (128, 64), (128, 256)])
 @pytest.mark.parametrize("pages,H_kv,page", [(1, 1, 16), (21, 3, 8), (300, 4, 5), (1201, 4, 24)])
 def test_recall_codes_batches(mka, orc, d, bits, pages, H_kv, page):
