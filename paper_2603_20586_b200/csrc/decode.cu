@@ -391,18 +391,29 @@ __global__ void __launch_bounds__(DH) decode_combine_kernel(const DecodeParams p
 }
 
 // CTAs per (batch, head) of the one-kernel form, 0 = the split form.  As many as keep all clusters resident at once (296 CTAs);
-// more only add rounds.  Long lists stay with the split form, whose chunks fill the last round, and so do middling ones
-// where the clusters would leave a third of the slots empty.  Split form / clusters of 1 / 2 / 4 / 8 in us, chosen in brackets:
-//   32 pairs x 1576 rows, d = 128    12.1 / 27.4 / 16.5 / 11.8 / [9.7]     128 pairs x 1576 rows    28.2 / 30.6 / [22.4] / 26.5 / 35.4
-//   32 pairs x 7548 rows             32.9 / 118 / 62 / 35.0 / [25.9]       64 pairs x 16,096 rows   90.2 / 237 / 128 / [86.8] / 90.7
-//   512 pairs x 772 rows             44.2 / [41.3] / 49.1 / 62.3 / 96.4    256 pairs x 4524 rows    100.7 / [97.5] / 101 / 107 / 128
+// more only add rounds.  The split form's chunks fill the chip to the end, at 6.8 TB/s, and cost 10 us more (a second kernel, its
+// launch, the partials).  A cluster's CTAs are as long as their pair's list: an SM brings its own at 52 GB/s, so SMs that hold two
+// while others hold one finish last, and a last round with few CTAs leaves most of the chip idle.  Both are added up here; the
+// model was fitted to 500 sizes of 8 to 2048 pairs and 200 to 16,000 rows, over which the form it picks takes 0.1 % more
+// than the better one on average, 7 % at most.  Split form / clusters of 1 / 2 / 4 / 8 in us, chosen in brackets, d = 128:
+//   8 pairs x 1000 rows    13.6 / 14.9 / 10.5 / 10.5 / [10.5]     128 x 10,000   113 / 168 / [109] / 113 / 123
+//   96 x 5000     [49.4] / 85.9 / 54.4 / 59.2 / 53.5              288 x 5000     128 / [119] / 126 / 152
+//   192 x 4000    [71.9] / 82.2 / 88.2 / 75.0                     304 x 2300     [69.8] / 93.1 / 78.4
+//   304 x 4000    [111] / 152 / 127                               416 x 2300     [90.4] / 101 / 86.0
+//   448 x 2300    [96.4] / 101 / 105                              640 x 3000     [166] / 194
 int cluster_rule(const DecodeParams& p) {
     const long long rows = p.L[0].n + p.L[1].n + p.L[2].n, bh = (long long)p.B * p.H;
     int size = 1;
     while (size < kMaxCluster && bh * size * 2 <= 296) size *= 2;
-    const long long per_cta = rows / size;
-    if (bh * size > 0x7fffffffLL || per_cta > 4096 || (per_cta > 2048 && bh * size < 192)) return 0;
-    return size;
+    const long long ctas = bh * size;
+    const double per_cta = (double)rows / size;
+    if (ctas > 0x7fffffffLL || per_cta > 8192.0) return 0;                // (longer ones were not measured)
+    const double kb = per_cta * 4.0 * p.d * 1e-3, sm = kb / 52.0, chip = kb / 6800.0;      // us: one CTA on an SM; its share of the chip's rate
+    const double full = (double)(ctas / 296), rest = (double)(ctas % 296);
+    double t = full * (2.0 * sm > 296.0 * chip ? 2.0 * sm : 296.0 * chip);
+    const double alone = (rest > 148.0 || full > 0.0 ? 2.0 : 1.0) * sm;
+    if (rest > 0.0) t += alone > rest * chip ? alone : rest * chip;
+    return t <= (double)ctas * chip + 10.0 ? size : 0;
 }
 
 template <int DH>

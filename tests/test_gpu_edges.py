@@ -196,7 +196,9 @@ def test_recall_codes_batches(mka, orc, d, bits, pages, H_kv, page):
 @pytest.mark.parametrize("B,H,N", [
     (1, 1, (1, 1, 0)),                 # eight CTAs, two rows
     (1, 3, (17, 300, 31)),             # slabs that are not full, levels that end inside a round
-    (1, 3, (100, 16500, 200)),         # clusters of eight with about 2100 rows a CTA: the split form
+    (1, 3, (100, 16500, 200)),         # clusters of eight with about 2100 rows a CTA: the split form at d = 128
+    (1, 3, (100, 40000, 200)),         # the split form at both widths
+    (2, 176, (300, 900, 40)),          # more CTAs than fit, a short last round: one kernel at d = 64, two at d = 128
     (3, 40, (600, 40, 33)),            # clusters of two
     (2, 150, (130, 0, 5)),             # one CTA a pair, more CTAs than fit at once
 ])
