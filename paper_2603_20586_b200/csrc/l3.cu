@@ -14,6 +14,7 @@ namespace {
 
 constexpr int kIdxThreads = 128;
 constexpr int kIdxPairs = 64;                         // (page, head) pairs per batch of a CTA: two per lane in the projections
+constexpr int kPhasePairs = 32;                       // the same in the two-phase form: one per lane
 constexpr int kIdxBitsPerWarp = 16;                   // code bits one warp works out per pass
 
 struct L3IndexParams {
@@ -186,6 +187,111 @@ __global__ void __launch_bounds__(2 * kIdxThreads, 2) l3_index_kernel(const L3In
                 }
             }
             if (base + 2 * step < pairs) arrive(3 + (n & 1));  // (nobody waits for the last two)
+        }
+    }
+}
+
+// The same in two phases: all 128 threads load and sum a batch of 32 pairs, then all project it, lane = pair.  No thread is set aside for
+// projections and up to four CTAs share an SM, so this form is for pools with few code bits to a key row and for small ones
+// (see launch_l3_index).
+// Dynamic shared memory: projT [d][bits + 4] floats, then s [kPhasePairs][d + 1] floats.
+template <int DH>
+__global__ void __launch_bounds__(kIdxThreads, 4) l3_index_phases_kernel(const L3IndexParams p) {
+    extern __shared__ __align__(16) float sm[];
+    const int ppitch = p.bits + 4;                             // floats between columns of projT (keeps the fill off one bank)
+    float* projT = sm;
+    float* s = sm + (size_t)DH * ppitch;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int pitch = DH + 1;
+    for (int e = tid; e < DH * p.bits; e += kIdxThreads) {     // e = j * d + i: coalesced reads of proj
+        const int j = e / DH, i = e % DH;
+        projT[i * ppitch + j] = p.proj[e];
+    }
+    constexpr int vecs = DH / 8;                               // 16-byte pieces of a row: 16 (d = 128) or 8 (d = 64)
+    constexpr int items = kPhasePairs * vecs;                    // (pair, piece) items of a batch
+    constexpr int kPerThread = items / kIdxThreads;            // 4 or 2: taken two at a time, 16 loads in flight
+    const long long pairs = p.n_pages * p.H_kv;
+    const int words = p.bits / 32;
+    unsigned short* codes16 = reinterpret_cast<unsigned short*>(p.codes);
+    for (long long base = (long long)blockIdx.x * kPhasePairs; base < pairs; base += (long long)gridDim.x * kPhasePairs) {
+        __syncthreads();                                       // projT is there; the previous batch is done with s
+        // ---- sums of the pages' keys, row by row
+#pragma unroll
+        for (int k0 = 0; k0 < kPerThread; k0 += 2) {
+            float acc[2][8];
+            const __nv_bfloat16* src[2];
+            bool live[2];
+            int slot[2], piece[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int it = tid + (k0 + q) * kIdxThreads;
+                slot[q] = it / vecs; piece[q] = it % vecs;
+                const long long pair = base + slot[q];
+                live[q] = pair < pairs;
+                const long long pc = live[q] ? pair : 0;
+                src[q] = p.k + (pc / p.H_kv) * p.sp + (pc % p.H_kv) * p.sh + piece[q] * 8;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc[q][i] = 0.f;
+            }
+            for (int r0 = 0; r0 < p.page_rows; r0 += 8) {
+                uint4 u[2][8];
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+#pragma unroll
+                    for (int r = 0; r < 8; ++r)
+                        u[q][r] = (live[q] && r0 + r < p.page_rows)
+                                      ? __ldg(reinterpret_cast<const uint4*>(src[q] + (long long)(r0 + r) * p.sn))
+                                      : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+#pragma unroll
+                    for (int r = 0; r < 8; ++r) {
+                        if (r0 + r < p.page_rows) {                // rows past the page add nothing, not even +0
+                            const uint32_t w[4] = {u[q][r].x, u[q][r].y, u[q][r].z, u[q][r].w};
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                acc[q][2 * i] = acc[q][2 * i] + __uint_as_float(w[i] << 16);
+                                acc[q][2 * i + 1] = acc[q][2 * i + 1] + __uint_as_float(w[i] & 0xffff0000u);
+                            }
+                        }
+                    }
+            }
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) s[slot[q] * pitch + piece[q] * 8 + i] = acc[q][i];
+        }
+        __syncthreads();
+        // ---- projections: one fmaf chain per (pair, bit) over the columns 0..d-1
+        const long long pair = base + lane;
+        const float* sv = s + lane * pitch;
+        for (int j0 = warp * kIdxBitsPerWarp; j0 < p.bits; j0 += (kIdxThreads / 32) * kIdxBitsPerWarp) {
+            // two chains per instruction (fma.rn.f32x2: each half is the same correctly rounded fma as fmaf)
+            unsigned long long a2[kIdxBitsPerWarp / 2];
+#pragma unroll
+            for (int j = 0; j < kIdxBitsPerWarp / 2; ++j) a2[j] = 0ull;          // two +0.f
+            const float* pj = projT + j0;
+            for (int i = 0; i < DH; ++i) {
+                const float x = sv[i];
+                unsigned long long x2;
+                asm("mov.b64 %0, {%1, %1};" : "=l"(x2) : "f"(x));
+#pragma unroll
+                for (int v = 0; v < kIdxBitsPerWarp / 4; ++v) {
+                    const ulonglong2 pr = *reinterpret_cast<const ulonglong2*>(pj + (size_t)i * ppitch + 4 * v);   // bits 4v..4v+3 of column i
+                    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a2[2 * v]) : "l"(pr.x), "l"(x2));
+                    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a2[2 * v + 1]) : "l"(pr.y), "l"(x2));
+                }
+            }
+            unsigned half = 0u;
+#pragma unroll
+            for (int j = 0; j < kIdxBitsPerWarp / 2; ++j) {
+                float lo, hi;
+                asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a2[j]));
+                half |= (lo >= 0.f ? 1u : 0u) << (2 * j);
+                half |= (hi >= 0.f ? 1u : 0u) << (2 * j + 1);
+            }
+            // bits j0..j0+15 are one 16-bit half of word j0 / 32 (low half first)
+            if (pair < pairs) codes16[(pair * words) * 2 + j0 / 16] = (unsigned short)half;
         }
     }
 }
@@ -373,6 +479,21 @@ __global__ void __launch_bounds__(kRetThreads) l3_retrieve_kernel(const L3Retrie
     }
 }
 
+// Which form of the index kernel.  The one with projecting warps of its own wins where projections are a good part of the work and
+// there are batches enough for all SMs; where a key row carries few code bits (its projecting half idles; at 32 bits two of those four
+// warps never have work, at 128 bits and d = 128 one CTA fits an SM) and for small pools the two-phase form does.  Time of the
+// first over that of the second, [5 .. 500 MB of keys], 4 KV heads:
+//   d = 64    32 bits, pages of 1 to 128 rows    1.04 .. 1.9            d = 128    32 bits    1.03 .. 1.9
+//             64 bits, 8 / 16 rows               0.75 / 0.96 (large)               64 bits, 8 / 16 rows     0.71 / 0.81 (large)
+//             64 bits, 24 / 32 / 64 rows         1.09 / 1.19 / 1.34                64 bits, 24 / 32 / 64    0.92 .. 1.10 / 0.97 .. 1.14 / 1.01 .. 1.25
+//             128 bits, 24 / 32 / 64 rows        0.88 / 0.98 .. 1.13 / 1.20        128 bits, 16 / 32 / 64   0.84 / 1.16 / 1.49
+//             256 bits, 16 / 64 rows             0.63 / 0.79                       256 bits, 16 / 64        0.57 / 0.97
+//   pools of at most 74 batches of 64 pairs, at any width (138 sizes): 0.95 .. 1.9
+bool two_phases(const L3IndexParams& p) {
+    if (p.bits == 32 || p.n_pages * p.H_kv <= 74 * kIdxPairs) return true;
+    return (p.bits == 64 && p.page_rows >= 24) || (p.bits == 128 && p.page_rows >= 32);
+}
+
 }  // namespace
 
 cudaError_t launch_l3_index(const void* k, long long n_pages, int H_kv, int page_rows, int d, long long sp, long long sh,
@@ -381,19 +502,22 @@ cudaError_t launch_l3_index(const void* k, long long n_pages, int H_kv, int page
     L3IndexParams p;
     p.k = static_cast<const __nv_bfloat16*>(k); p.proj = proj; p.codes = codes;
     p.n_pages = n_pages; p.sp = sp; p.sh = sh; p.sn = sn; p.H_kv = H_kv; p.page_rows = page_rows; p.d = d; p.bits = bits;
-    const size_t smem = ((size_t)d * (bits + 4) + 2 * (size_t)kIdxPairs * (d + 1)) * sizeof(float);
-    auto kern = d == 128 ? l3_index_kernel<128> : l3_index_kernel<64>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    const long long batches = (n_pages * H_kv + kIdxPairs - 1) / kIdxPairs;
-    const long long per_sm = smem > 112 * 1024 ? 1 : 2;
-    const long long resident = 148LL * per_sm;
     // persistent CTAs: every CTA transposes the projection into shared memory once and then walks its batches
     // (the grid is shrunk so that all CTAs get the same number of batches)
-    const long long per_cta = (batches + resident - 1) / resident;
-    const long long grid = (batches + per_cta - 1) / per_cta;
-    kern<<<(unsigned)grid, 2 * kIdxThreads, smem, st>>>(p);
-    return cudaGetLastError();
+    auto launch = [&](auto kern, int batch, int buffers, int threads, auto ctas_per_sm) {
+        const size_t smem = ((size_t)d * (bits + 4) + (size_t)buffers * batch * (d + 1)) * sizeof(float);
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        const long long batches = (n_pages * H_kv + batch - 1) / batch, resident = 148LL * ctas_per_sm(smem);
+        const long long per_cta = (batches + resident - 1) / resident, grid = (batches + per_cta - 1) / per_cta;
+        kern<<<(unsigned)grid, threads, smem, st>>>(p);
+        return cudaGetLastError();
+    };
+    if (two_phases(p))
+        return launch(d == 128 ? l3_index_phases_kernel<128> : l3_index_phases_kernel<64>, kPhasePairs, 1, kIdxThreads,
+                      [](size_t smem) { return smem > 110 * 1024 ? 1 : (smem > 72 * 1024 ? 2 : (smem > 54 * 1024 ? 3 : 4)); });
+    return launch(d == 128 ? l3_index_kernel<128> : l3_index_kernel<64>, kIdxPairs, 2, 2 * kIdxThreads,
+                  [](size_t smem) { return smem > 112 * 1024 ? 1 : 2; });
 }
 
 cudaError_t launch_l3_retrieve(const void* q, int B, int H, int H_kv, int d, const float* proj, int bits,

@@ -181,10 +181,11 @@ def test_cuda_core_many_blocks(mka, orc, d, dtype, B, H, T, W, N):
     assert err(g["dG"], r["dG"])[0] <= (2e-2 if dtype == torch.bfloat16 else 1e-4) * H / 4
 
 
-@pytest.mark.parametrize("d,bits", [(64, 32), (128, 64), (128, 256)])
-@pytest.mark.parametrize("pages,H_kv,page", [(1, 1, 16), (21, 3, 8), (300, 4, 5), (1201, 4, 24)])
+@pytest.mark.parametrize("d,bits", [(64, 32), (64, 64), (128, 64), (128, 128), (128, 256)])
+@pytest.mark.parametrize("pages,H_kv,page", [(1, 1, 16), (21, 3, 8), (300, 4, 5), (1201, 4, 24), (1184, 4, 16), (1185, 4, 16), (1185, 4, 32), (20001, 2, 3)])
 def test_recall_codes_batches(mka, orc, d, bits, pages, H_kv, page):
-    """Recall codes: a batch with one pair, a last batch that is not full, pages of no whole number of eight rows, several batches a CTA."""
+    """Recall codes: a batch with one pair, a last batch that is not full, pages of no whole number of eight rows, several batches a CTA,
+    both forms of the kernel on either side of every line between them."""
     g = torch.Generator().manual_seed(3)
     pool = torch.randn(pages, H_kv, page, d, generator=g).bfloat16().cuda()
     proj = torch.randn(bits, d, generator=g).cuda()
