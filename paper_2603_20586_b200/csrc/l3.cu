@@ -308,6 +308,7 @@ struct L3RetrieveParams {
     long long bank_stride;
     int B, H, H_kv, d, bits, R, page_rows, max_bank;
     int stage_proj;               // the projection is staged in shared memory (it fits beside the scores and is 16-byte aligned)
+    int code_vec;                 // code words fetched by one load: 4 (16-byte aligned codes of 128 or 256 bits), 2 (64 bits, 8-byte aligned) or 1
 };
 
 constexpr int kRetThreads = 1024;
@@ -330,7 +331,7 @@ __device__ __forceinline__ int cta_sum(int v, int* part, int warp, int lane) {
 __global__ void __launch_bounds__(kRetThreads) l3_retrieve_kernel(const L3RetrieveParams p) {
     extern __shared__ __align__(16) unsigned short score[];
     __shared__ __align__(16) float qs[256];
-    __shared__ unsigned int qcode[8];
+    __shared__ __align__(16) unsigned int qcode[8];
     __shared__ int part[2][kRetWarps];
     int* before = reinterpret_cast<int*>(score + (p.max_bank + 7) / 8 * 8);
     float* projs = reinterpret_cast<float*>(before + (p.max_bank + kRetThreads - 1) / kRetThreads * kRetWarps);   // [bits][d + 4]
@@ -340,10 +341,11 @@ __global__ void __launch_bounds__(kRetThreads) l3_retrieve_kernel(const L3Retrie
     int n = p.bank_len[b];
     n = n < 0 ? 0 : (n > p.max_bank ? p.max_bank : n);
     const int* bank = p.bank + (long long)b * p.bank_stride;
-    // 64-bit codes: the first eight chunks of a thread, page numbers first, then all code words
+    // 64-bit codes: the first eight chunks of a thread, page numbers first, then all code words.  (Wider codes would need 32 and
+    // 64 registers for that, half or all of what a thread has here; theirs are asked for after the query's code.)
     constexpr int kAhead = 8;
     uint2 ahead[kAhead];
-    if (words == 2) {
+    if (p.code_vec == 2) {
         int page[kAhead];
 #pragma unroll
         for (int u = 0; u < kAhead; ++u) {
@@ -391,7 +393,7 @@ __global__ void __launch_bounds__(kRetThreads) l3_retrieve_kernel(const L3Retrie
     }
     __syncthreads();
     // agreement of every chunk's code with the query's: 0..bits (<= 256)
-    if (words == 2) {
+    if (p.code_vec == 2) {
         const unsigned int q0 = qcode[0], q1 = qcode[1];
 #pragma unroll
         for (int u = 0; u < kAhead; ++u) {
@@ -399,21 +401,49 @@ __global__ void __launch_bounds__(kRetThreads) l3_retrieve_kernel(const L3Retrie
             if (c < n) score[c] = (unsigned short)(p.bits - __popc(ahead[u].x ^ q0) - __popc(ahead[u].y ^ q1));
         }
     }
-    for (int c0 = tid + (words == 2 ? kAhead * kRetThreads : 0); c0 < n; c0 += 8 * kRetThreads) {
-        int page[8], dist[8];
+    // All words of a code lie in one sector, so they are fetched together: word by word over eight chunks, a CTA's 8192 sectors had
+    // left its L1 before the next word (whole kernel, 256 bits, 40,000 chunks: 366 us; one after the other and 32 bits a load 221; now 110).
+    const unsigned int* codes = p.codes + (long long)kvh * words;
+    const long long page_words = (long long)p.H_kv * words;
+    for (int c0 = tid + (p.code_vec == 2 ? kAhead * kRetThreads : 0); c0 < n; c0 += 8 * kRetThreads) {
+        int page[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int c = c0 + u * kRetThreads;
             page[u] = c < n ? bank[c] : 0;
-            dist[u] = 0;
         }
-        for (int w = 0; w < words; ++w)
-#pragma unroll
-            for (int u = 0; u < 8; ++u) dist[u] += __popc(__ldg(p.codes + ((long long)page[u] * p.H_kv + kvh) * words + w) ^ qcode[w]);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
+        auto put = [&](int u, int dist) {
             const int c = c0 + u * kRetThreads;
-            if (c < n) score[c] = (unsigned short)(p.bits - dist[u]);
+            if (c < n) score[c] = (unsigned short)(p.bits - dist);
+        };
+        if (p.code_vec == 4) {
+            const uint4 qa = *reinterpret_cast<const uint4*>(qcode), qb = *reinterpret_cast<const uint4*>(qcode + 4);
+            auto differ = [](const uint4& x, const uint4& y) { return __popc(x.x ^ y.x) + __popc(x.y ^ y.y) + __popc(x.z ^ y.z) + __popc(x.w ^ y.w); };
+#pragma unroll
+            for (int u0 = 0; u0 < 8; u0 += 4) {
+                uint4 a[4], b[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const uint4* at = reinterpret_cast<const uint4*>(codes + page[u0 + u] * page_words);
+                    a[u] = __ldg(at);
+                    b[u] = words == 8 ? __ldg(at + 1) : qb;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) put(u0 + u, differ(a[u], qa) + differ(b[u], qb));
+            }
+        } else if (p.code_vec == 2) {
+            uint2 w[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) w[u] = __ldg(reinterpret_cast<const uint2*>(codes + page[u] * page_words));
+#pragma unroll
+            for (int u = 0; u < 8; ++u) put(u, __popc(w[u].x ^ qcode[0]) + __popc(w[u].y ^ qcode[1]));
+        } else {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                int dist = 0;
+                for (int w = 0; w < words; ++w) dist += __popc(__ldg(codes + page[u] * page_words + w) ^ qcode[w]);
+                put(u, dist);
+            }
         }
     }
     // (a thread reads back only the scores it wrote, up to the barriers below)
@@ -531,6 +561,8 @@ cudaError_t launch_l3_retrieve(const void* q, int B, int H, int H_kv, int d, con
     size_t smem = ((size_t)max_bank + 7) / 8 * 8 * sizeof(unsigned short) +
                   ((size_t)max_bank + kRetThreads - 1) / kRetThreads * kRetWarps * sizeof(int) + 16;
     const size_t with_proj = smem + (size_t)bits * (d + 4) * sizeof(float);
+    const uintptr_t at = reinterpret_cast<uintptr_t>(codes);
+    p.code_vec = bits >= 128 && at % 16 == 0 ? 4 : (bits == 64 && at % 8 == 0 ? 2 : 1);
     p.stage_proj = with_proj <= 220 * 1024 && (reinterpret_cast<uintptr_t>(proj) & 15) == 0;
     if (p.stage_proj) smem = with_proj;
     cudaError_t e = cudaFuncSetAttribute(l3_retrieve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -219,7 +219,7 @@ def test_decode_one_kernel_or_two(mka, orc, d, B, H, N):
         assert not finite.any() or np.abs(np64(LSE)[finite] - Lr[:, :, 0][finite]).max() <= 1e-4
 
 
-@pytest.mark.parametrize("bits,n,R", [(32, 1, 8), (64, 31, 64), (64, 8191, 8), (64, 8193, 16), (128, 1025, 7), (256, 2050, 64), (32, 9000, 64)])
+@pytest.mark.parametrize("bits,n,R", [(32, 1, 8), (64, 31, 64), (64, 8191, 8), (64, 8193, 16), (128, 1025, 7), (256, 2050, 64), (32, 9000, 64), (128, 9001, 8), (256, 40000, 8)])
 def test_recall_lists(mka, orc, bits, n, R):
     """Recall lists: fewer chunks than asked for, banks around a thread's chunks, few code bits (long runs of ties), a sequence with no bank."""
     B, H, H_kv, d = 3, 6, 2, 64
@@ -230,8 +230,9 @@ def test_recall_lists(mka, orc, bits, n, R):
     codes = torch.randint(-2**31, 2**31, (pages, H_kv, bits // 32), generator=g, dtype=torch.int64).to(torch.int32).cuda()
     bank = torch.stack([torch.randperm(pages, generator=g)[:n] for _ in range(B)]).to(torch.int32).cuda()
     lens = torch.tensor([n, max(1, n // 3), 0], dtype=torch.int32).cuda()
-    for pj in (proj, torch.cat([proj.new_zeros(1), proj.flatten()])[1:].view(bits, d)):          # and a projection that allows no 16-byte load
-        table, n_sel, rows = mka.mka_l3_retrieve(q, H_kv, pj, codes, bank, lens, R, 16)
+    off = lambda x: torch.cat([x.new_zeros(1), x.flatten()])[1:].view(x.shape)                  # noqa: E731  the same values at an address that allows no vector load
+    for pj, cd in ((proj, codes), (off(proj), codes), (proj, off(codes))):
+        table, n_sel, rows = mka.mka_l3_retrieve(q, H_kv, pj, cd, bank, lens, R, 16)
         words = codes.cpu().numpy().view(np.uint32)
         for b in range(B):
             m = int(lens[b])
