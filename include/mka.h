@@ -197,8 +197,8 @@ typedef struct mka_paged_level {
  * Every cached row is read once per KV head.  A level whose gate is exactly 0 for a sequence is not read.
  *   q [B, H, d] bf16;  gate [B, 3] f32;  O [B, H, d] bf16;  LSE [B, H] f32 or NULL
  *   ws: mka_decode_paged_workspace_bytes(shape, H_kv, n_level) bytes, n_level[l] = L[l].n.  The rows that the sequences really
- *       have are cut into equal shares on the device, one per resident CTA (pages under 8 rows, or more than 512
- *       sequences: chunks of a multiple of 128 rows, chosen on the host)
+ *       have are cut into equal shares on the device, one per resident CTA (pages under 8 rows: chunks
+ *       of a multiple of 128 rows, chosen on the host)
  * d must be 64 or 128; pools 16-byte aligned with strides that are multiples of 8 elements.
  * Levels whose pages hold at least 8 rows (and dense levels, see mka_decode) are streamed by the copy engine: a
  * producing warp issues one tensor-map copy per page and 64-column panel, the computing warps wait on barriers for

@@ -130,6 +130,7 @@ struct DecodePagedParams {
     float* partial;      // [B*H, total_chunks, d+2]
     int test_stall;                    // MKA_FLAG_TEST_STALL (copy-engine form): every CTA's producer leaves out the last tile of its share
     int dealt;                         // the copy-engine form: total_chunks = entries per query head (a count, then the partials)
+    int deal_shift;                    // copy-engine form: log2 of the sequences in a block of its sums
     unsigned int* status;              // device status word of the call's workspace (bounded waits of the copy-engine form)
     unsigned long long wait_limit_ns;
 };

@@ -277,31 +277,65 @@ __device__ __forceinline__ int list_rows(const DecodePagedParams& p, int b, int 
     return (int)(n < 0 ? 0 : (n > L.n ? L.n : n));
 }
 
+// Tiles of one list of sequence b.
+__device__ __forceinline__ int list_tiles(const DecodePagedParams& p, int b) {
+    int t = 0;
+#pragma unroll
+    for (int l = 0; l < 3; ++l) t += (list_rows(p, b, l) + kTileRows - 1) / kTileRows;
+    return t;
+}
+
+// Where the shares begin is found from sums over blocks of 2^shift consecutive sequences, as many as keep the blocks within
+// kDealBlocks: any batch fits, and up to kDealBlocks sequences every sequence is a block.
+constexpr int kDealBlocks = 512;
+
 // Walks a CTA's share of the tiles.
 struct TileWalk {
     const DecodePagedParams& p;
-    const int* tiles;                     // tiles of a list, per sequence
     int left;                             // tiles of the share still to come
     int b, kvh, at;                       // list, and the next tile in it
     int n[3];                             // rows of the list's levels
-    __device__ __forceinline__ TileWalk(const DecodePagedParams& p_, const int* tiles_, const int* before, long long u0, int share)
-        : p(p_), tiles(tiles_), left(share) {
-        // first sequence with tiles past u0 (before[b]: tiles of a list times b's predecessors; H_kv lists each)
-        int lo = 0, hi = p.B - 1;
+    int tiles, ahead;                     // tiles of the list, and of one list of each of b's predecessors
+    // before[i]: tiles of one list of each sequence in front of block i.  Called by whole warps.
+    __device__ __forceinline__ TileWalk(const DecodePagedParams& p_, const int* before, int blocks, int shift, long long u0, int share, int lane)
+        : p(p_), left(share) {
+        int lo = 0, hi = blocks - 1;      // first block with tiles past u0 (H_kv lists to a sequence)
         while (lo < hi) {
             const int mid = (lo + hi) / 2;
             if ((long long)before[mid + 1] * p.H_kv > u0) hi = mid; else lo = mid + 1;
         }
-        b = lo;
-        const int in_seq = (int)(u0 - (long long)before[b] * p.H_kv);
-        kvh = in_seq / tiles[b]; at = in_seq - kvh * tiles[b];
+        ahead = before[lo];
+        b = lo << shift;
+        if (shift > 0) {                  // and the sequence in it, 32 at a time
+            const int end = min(p.B, (lo + 1) << shift);
+            for (;; b += 32) {
+                const int own = b + lane < end ? list_tiles(p, b + lane) : 0;
+                int sum = own;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int x = __shfl_up_sync(0xffffffffu, sum, o);
+                    if (lane >= o) sum += x;
+                }
+                const unsigned int past = __ballot_sync(0xffffffffu, (long long)(ahead + sum) * p.H_kv > u0);
+                if (past) {
+                    const int i = __ffs(past) - 1;
+                    b += i;
+                    ahead += __shfl_sync(0xffffffffu, sum - own, i);
+                    break;
+                }
+                ahead += __shfl_sync(0xffffffffu, sum, 31);
+            }
+        }
         enter();
+        const int in_seq = (int)(u0 - (long long)ahead * p.H_kv);
+        kvh = in_seq / tiles; at = in_seq - kvh * tiles;
     }
     __device__ __forceinline__ void enter() {
+        tiles = 0;
 #pragma unroll
-        for (int l = 0; l < 3; ++l) n[l] = list_rows(p, b, l);
+        for (int l = 0; l < 3; ++l) { n[l] = list_rows(p, b, l); tiles += (n[l] + kTileRows - 1) / kTileRows; }
     }
-    __device__ __forceinline__ int segment() const { return min(left, tiles[b] - at); }      // tiles of the share in this list
+    __device__ __forceinline__ int segment() const { return min(left, tiles - at); }      // tiles of the share in this list
     // level and first row of tile t of the list
     __device__ __forceinline__ void locate(int t, int& lvl, int& row0, int& rows) const {
         const int t0 = (n[0] + kTileRows - 1) / kTileRows, t1 = (n[1] + kTileRows - 1) / kTileRows;
@@ -313,12 +347,11 @@ struct TileWalk {
     __device__ __forceinline__ bool advance(int done) {
         left -= done; at += done;
         if (left <= 0) return false;
-        if (at < tiles[b]) return true;
+        if (at < tiles) return true;
         at = 0;
         if (++kvh == p.H_kv) {
             kvh = 0;
-            do ++b; while (tiles[b] == 0);
-            enter();
+            do { ahead += tiles; ++b; enter(); } while (tiles == 0);
         }
         return true;
     }
@@ -335,8 +368,7 @@ __global__ void __launch_bounds__(kTmaThreads, 2) decode_paged_tma_kernel(const 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     float* hand = reinterpret_cast<float*>(smem + kTmaStages * 2 * kTileBytes);      // [kState][32]: one warp's state on its way to warp 0
-    int* tiles = reinterpret_cast<int*>(hand + kState * 32);                         // [B]
-    int* before = tiles + p.B;                                                       // [B + 1]
+    int* before = reinterpret_cast<int*>(hand + kState * 32);                        // [blocks + 1]
     __shared__ uint64_t full[kTmaStages], empty[kTmaStages];
     __shared__ WaitCtl ctl;
 
@@ -350,38 +382,45 @@ __global__ void __launch_bounds__(kTmaThreads, 2) decode_paged_tma_kernel(const 
         for (int i = 0; i < kTmaStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 4); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (int b = tid; b < p.B; b += kTmaThreads) {
-        int t = 0;
+    const int shift = p.deal_shift, blocks = (p.B + (1 << shift) - 1) >> shift;
+    for (int i = tid; i <= blocks; i += kTmaThreads) before[i] = 0;
+    __syncthreads();
+    for (int b0 = tid; b0 < p.B; b0 += 4 * kTmaThreads) {   // four sequences' row counts and gates in flight
+        int t[4];
 #pragma unroll
-        for (int l = 0; l < 3; ++l) t += (list_rows(p, b, l) + kTileRows - 1) / kTileRows;
-        tiles[b] = t;
+        for (int u = 0; u < 4; ++u) t[u] = b0 + u * kTmaThreads < p.B ? list_tiles(p, b0 + u * kTmaThreads) : 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int b = b0 + u * kTmaThreads;
+            if (b >= p.B) break;
+            if (t[u]) atomicAdd(&before[b >> shift], t[u]);
+            else if (b % gridDim.x == blockIdx.x)           // a sequence without a tile has no partials
+                for (int h = 0; h < p.H; ++h) p.partial[((long long)b * p.H + h) * list_floats] = 0.f;
+        }
     }
     __syncthreads();
-    if (warp == 0) {
+    if (warp == 0) {                                        // sums in front of each block
         int run = 0;
-        for (int b0 = 0; b0 < p.B; b0 += 32) {
-            int t = b0 + lane < p.B ? tiles[b0 + lane] : 0;
+        for (int b0 = 0; b0 < blocks; b0 += 32) {
+            int t = b0 + lane < blocks ? before[b0 + lane] : 0;
             const int own = t;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const int x = __shfl_up_sync(0xffffffffu, t, o);
                 if (lane >= o) t += x;
             }
-            if (b0 + lane < p.B) before[b0 + lane] = run + t - own;
+            if (b0 + lane < blocks) before[b0 + lane] = run + t - own;
             run += __shfl_sync(0xffffffffu, t, 31);
         }
-        if (lane == 0) before[p.B] = run;
+        if (lane == 0) before[blocks] = run;
     }
     __syncthreads();
     volatile WaitCtl* ctlp = &ctl;
-    const long long all = (long long)before[p.B] * p.H_kv;
+    const long long all = (long long)before[blocks] * p.H_kv;
     const int share = (int)max(2LL, (all + gridDim.x - 1) / gridDim.x);
     const long long u0 = (long long)blockIdx.x * share;
-    if (blockIdx.x == 0)                                    // sequences without a tile have no partials
-        for (int i = tid; i < p.B * p.H; i += kTmaThreads)
-            if (tiles[i / p.H] == 0) p.partial[i * list_floats] = 0.f;
     if (u0 >= all) return;
-    TileWalk walk(p, tiles, before, u0, (int)min((long long)share, all - u0));
+    TileWalk walk(p, before, blocks, shift, u0, (int)min((long long)share, all - u0), lane);
 
     if (warp == 4) {
         // ------------------------------------------------------------ producer
@@ -595,9 +634,9 @@ __global__ void __launch_bounds__(kTmaThreads, 2) decode_paged_tma_kernel(const 
         }
         if (warp == 0) {
             // this share is the list's partial number slot; the share with the list's first tile also says how many there are
-            const long long list0 = (long long)before[b] * p.H_kv + (long long)kvh * tiles[b];
+            const long long list0 = (long long)walk.ahead * p.H_kv + (long long)kvh * walk.tiles;
             const int first_share = (int)(list0 / share), slot = (int)blockIdx.x - first_share;
-            const int n_slots = (int)((list0 + tiles[b] - 1) / share) - first_share + 1;
+            const int n_slots = (int)((list0 + walk.tiles - 1) / share) - first_share + 1;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 z[h] += __shfl_xor_sync(0xffffffffu, z[h], 1);
@@ -619,7 +658,9 @@ __global__ void __launch_bounds__(kTmaThreads, 2) decode_paged_tma_kernel(const 
 // The copy-engine form needs every non-empty level to be describable by a tensor map: a dense level, or pages of at
 // least 8 rows; strides are multiples of 8 elements already.
 template <int DH>
-cudaError_t launch_tma(const DecodePagedParams& p, cudaStream_t st) {
+cudaError_t launch_tma(DecodePagedParams p, cudaStream_t st) {
+    p.deal_shift = 0;
+    while (((p.B - 1) >> p.deal_shift) >= kDealBlocks) ++p.deal_shift;
     PagedMaps maps;
     for (int l = 0; l < 3; ++l) {
         const PagedLevelDev& L = p.L[l];
@@ -648,7 +689,7 @@ cudaError_t launch_tma(const DecodePagedParams& p, cudaStream_t st) {
     for (int l = 0; l < 3; ++l) if (p.L[l].n > 0) { first_real = l; break; }
     if (first_real < 0) return cudaSuccess;
     for (int l = 0; l < 3; ++l) if (p.L[l].n == 0) { maps.k[l] = maps.k[first_real]; maps.v[l] = maps.v[first_real]; }
-    const size_t smem = (size_t)kTmaStages * 2 * kTileRows * DH * 2 + 1024 + (DH / 8 * 4 + 4) * 32 * sizeof(float) + (2 * (size_t)p.B + 1) * sizeof(int);
+    const size_t smem = (size_t)kTmaStages * 2 * kTileRows * DH * 2 + 1024 + (DH / 8 * 4 + 4) * 32 * sizeof(float) + (kDealBlocks + 1) * sizeof(int);
     cudaError_t e = cudaFuncSetAttribute(decode_paged_tma_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     decode_paged_tma_kernel<DH><<<kDealCtas, kTmaThreads, smem, st>>>(maps, p);
@@ -668,9 +709,9 @@ cudaError_t launch_t(const DecodePagedParams& p, cudaStream_t st) {
 
 }  // namespace
 
-// Levels that the copy-engine form takes (and their sequences' lists fit beside its ring).
+// Levels that the copy-engine form takes.
 bool decode_paged_dealt(const DecodePagedParams& p) {
-    if (p.B > 512 || (p.d != 64 && p.d != 128)) return false;
+    if (p.d != 64 && p.d != 128) return false;
     if (!tensor_map_encoder_available()) return false;
     for (int l = 0; l < 3; ++l) {
         const PagedLevelDev& L = p.L[l];

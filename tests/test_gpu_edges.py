@@ -255,7 +255,9 @@ def test_recall_lists(mka, orc, bits, n, R):
     (37, 4, 2, (40, 130, 3), 16),          # shares that end inside lists and reach over several sequences
     (3, 14, 2, (300, 9000, 70), 64),       # lists of dozens of shares
     (150, 4, 2, (70, 129, 200), 16),       # shares of nine tiles, every third one ragged: stages refilled behind rows that were cleared
-    (513, 2, 1, (20, 33, 0), 16),          # more sequences than the dealt form takes
+    (513, 2, 1, (20, 33, 0), 16),          # shares found through blocks of two sequences
+    (2500, 2, 2, (9, 70, 0), 16),          # of eight
+    (20000, 1, 1, (1, 3, 0), 8),           # and of 64, with sequences without a row among them
 ])
 def test_decode_paged_shares(mka, orc, d, B, H, H_kv, N, page):
     """Paged decode against the dense oracle: mixed lengths, sequences without a row, levels that a gate closes."""
