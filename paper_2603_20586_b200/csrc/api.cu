@@ -528,6 +528,7 @@ mka_status mka_bwd(const mka_shape* s, const void* Q, const mka_level L[3], cons
     p.window = s->window; p.q_offset = s->q_offset; p.scale = resolve_scale(s); p.kv_group = kv_group_of(s);
     p.test_stall = (s->flags & MKA_FLAG_TEST_STALL) ? 1 : 0;
     const bool tc = !(s->flags & MKA_FLAG_FORCE_SIMT) && bwd_tc_eligible(p, s->dtype);
+    if (tc && !aligned16(ws)) return MKA_ERR_ALIGN;          // its statistics are read 16 bytes at a time
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     p.status = static_cast<unsigned int*>(ws);
     cudaError_t e;
@@ -539,7 +540,8 @@ mka_status mka_bwd(const mka_shape* s, const void* Q, const mka_level L[3], cons
     if (e != cudaSuccess) return MKA_ERR_CUDA;
     if (dW_r || db_r) {
         // the statistics have had their last reader: their room takes the chunks' sums of dG
-        double* db_part = bwd_stats_bytes(s) >= kRouterBwdChunks * 3 * sizeof(double) ? reinterpret_cast<double*>(p.stats) : nullptr;
+        const bool room = bwd_stats_bytes(s) >= kRouterBwdChunks * 3 * sizeof(double) && (reinterpret_cast<uintptr_t>(p.stats) & 7u) == 0;
+        double* db_part = room ? reinterpret_cast<double*>(p.stats) : nullptr;
         e = launch_router_bwd(R, r_dtype, dG, (long long)s->B * s->T, s->D, dW_r, db_r, rpart, db_part, kRouterBwdChunks, cs);
         if (e != cudaSuccess) return MKA_ERR_CUDA;
     }

@@ -119,6 +119,29 @@ def test_router_gradient_splits(mka, orc, dtype, B, T, D):
     assert (np.abs(np64(g["db_r"]) - db) <= 6e-8 * np.abs(db) + 1e-15 * np.abs(dG).sum() * B * T).all()
 
 
+def test_bwd_workspace_alignment(mka, orc):
+    """fp32 takes a workspace at any word; the tensor-core kernels read their statistics 16 bytes at a time and refuse what allows none."""
+    B, H, T, d, N, D = 1, 2, 130, 64, (130, 130, 40), 72
+    for dtype in (torch.float32, torch.bfloat16):
+        P = problem(18, B, H, T, d, N, D, dtype, router_std=0.3, with_dO=True)
+        gate = mka.mka_router(P["X"], P["W_r"], None)
+        shape = mka.make_shape(B, H, T, d, D, 32, dtype=mka.binding.MKA_BF16 if dtype == torch.bfloat16 else mka.binding.MKA_F32)
+        O, LSE = mka.mka_fwd(shape, P["Q"], P["K"], P["V"], gate)
+        ws = mka.alloc_workspace(shape, N, mka.MKA_WS_BWD, "cuda")
+        off = torch.zeros(ws.numel() + 4, dtype=torch.uint8, device="cuda")[4:]
+        run = lambda w: mka.mka_bwd(shape, P["Q"], P["K"], P["V"], gate, O, LSE, P["dO"], R=P["X"], ws=w)  # noqa: E731
+        want = run(ws)
+        if dtype == torch.bfloat16:
+            with pytest.raises(RuntimeError, match="align"):
+                run(off)
+            continue
+        got = run(off)
+        for k in ("dQ", "dG", "dW_r"):
+            assert torch.equal(got[k], want[k])
+        # one CTA's sum of dG in place of the chunks' sums, both in 64 bits: one rounding apart at most
+        assert err(got["db_r"], np64(want["db_r"]))[0] <= 1.2e-7 * np.abs(np64(want["db_r"])).max()
+
+
 @pytest.mark.parametrize("d,dtype,shift", [(32, torch.float32, 0), (64, torch.float32, 1), (96, torch.float32, 0), (128, torch.float32, 3),
                                            (96, torch.bfloat16, 0), (32, torch.bfloat16, 0)])
 @pytest.mark.parametrize("T,W,q_off,N", [(1, 1, 0, (1, 1, 0)), (17, 5, 300, (317, 317, 33)), (130, 64, 0, (130, 100, 31))])
