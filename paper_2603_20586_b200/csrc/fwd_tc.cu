@@ -817,7 +817,7 @@ int resident_clusters(int split) {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<DH>::kSmemBytes) != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
         cudaGetLastError();
-        n = 0;
+        return 0;                                             // not split this time; only answers are remembered
     }
     known[dev][split].store(n + 1, std::memory_order_relaxed);
     return n;
