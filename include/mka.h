@@ -28,6 +28,8 @@
  *     is launched, and nothing is launched when validation fails.  No entry point aborts or traps.
  *   - Head width d must be 32, 64, 96 or 128 (decode and the tensor-core forward: 64 or 128).  bf16 tensors
  *     need 16-byte aligned base pointers and strides that are multiples of 8 elements.
+ *   - A call's results are the same bits every time.  The low bits of a row may change with what else is in the call: sums are
+ *     split by the number of rows, heads and sequences (and, in the paged decode, by all sequences' row counts).
  *   - There is no CPU fallback: without a CUDA device every compute entry point returns MKA_ERR_CUDA.
  */
 #ifndef MKA_H_
@@ -268,7 +270,8 @@ mka_status mka_l3_retrieve(const void* q, int32_t B, int32_t H, int32_t H_kv, in
  * and a caller training that variant passes dW_r = db_r = NULL.
  * bf16 with d in {64,128} runs the TMA + tcgen05 kernels (one pass that owns query tiles for dQ and dG, one
  * pass that owns key tiles for dK and dV; scores are recomputed in each, nothing is accumulated atomically);
- * f32, other head widths and MKA_FLAG_FORCE_SIMT run the CUDA-core kernels.  Both are deterministic.
+ * f32, other head widths and MKA_FLAG_FORCE_SIMT run the CUDA-core kernels.  Both are deterministic.  The tensor-core
+ * kernels want ws 16-byte aligned (MKA_ERR_ALIGN otherwise).
  */
 mka_status mka_bwd(const mka_shape* shape, const void* Q, const mka_level L[3], const float* gate,
                    const void* O, const float* LSE, const void* dO, const void* R, int32_t r_dtype,

@@ -474,8 +474,8 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const 
                     mma_commit_elect(&bar.b_empty[sv]);
                     if (e + 1 == E) mma_commit_elect(&bar.fixed_free);
                     if (e + 1 < E && !issue_s(g + 1)) { ok = false; break; }
-                    // dQ += dS(e) K(e), in the two parts in which the element-wise threads hand dS over (32 of each thread's
-                    // 64 columns: K-steps {0, 1, 4, 5}, then {2, 3, 6, 7}), so that the first half runs under the second
+                    // dQ += dS(e) K(e), in the two parts in which the element-wise threads hand dS over (half of each thread's
+                    // columns: at d = 128 K-steps {0, 1, 4, 5}, then {2, 3, 6, 7}), so that the first half runs under the second
 #pragma unroll
                     for (int part = 0; part < 2; ++part) {
                         if (!mbar_wait_warp(&bar.ds_part[part], (uint32_t)g & 1u, abortp)) { ok = false; break; }
@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const 
             }
         }
     } else {
-        // ------------------------------------------------------------ element-wise warpgroups (thread = query row, 64 of the 128 columns)
+        // ------------------------------------------------------------ element-wise warpgroups (thread = query row, 64 of the 128 columns; d = 64: 32)
         const int w = warp >> 2;
         const int r = tid & 127;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
@@ -539,7 +539,7 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const 
             const float bl = bias[l];
             const uint64_t scale2 = pack2(p.scale_log2, p.scale_log2), bl2 = pack2(bl, bl), negD2 = pack2(-Dt, -Dt);
             for (int kt = I.first[l]; kt < I.end[l]; ++kt, ++g) {
-                // phase 1: p = 2^(s * scale + bias) for this thread's 64 columns (needs S only)
+                // phase 1: p = 2^(s * scale + bias) for this thread's columns (needs S only)
                 ok = mbar_wait(&bar.s_full[g & 1], (uint32_t)(g >> 1) & 1u, abortp);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
@@ -907,7 +907,7 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
                     const int s = g % C::kStages;
                     const uint32_t qta = qt_lo + s * (C::kTile >> 4), gta = gt_lo + s * (C::kTile >> 4);
                     // dV += P^T(e) dO(e) and dK += dS^T(e) Q(e), each in the two parts in which the element-wise threads
-                    // hand their 64 columns over (K-steps {0, 1, 4, 5}, then {2, 3, 6, 7})
+                    // hand their columns over (d = 128: K-steps {0, 1, 4, 5}, then {2, 3, 6, 7}; d = 64: the whole tile at once for dV)
 #pragma unroll
                     for (int part = 0; part < 2; ++part) {
                         // (with two S^T the element-wise threads are ahead: one wait, for the whole tile, costs less than two)
@@ -997,7 +997,7 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
             }
         }
     } else {
-        // ------------------------------------------------------------ element-wise warpgroups (thread = key row, 64 of the 128 query columns)
+        // ------------------------------------------------------------ element-wise warpgroups (thread = key row, 64 of the 128 query columns; d = 64: 32)
         const int w = warp >> 2;
         const int r = tid & 127;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
@@ -1020,7 +1020,7 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
         for (int e = 0; e < E; ++e, ++g) {
             const long long tt = (long long)(first + eq) * kBlk;       // first query of the tile
             if (++eq == Eq) eq = 0;
-            // phase 1: P^T = 2^(scale * (s + bias_t / scale)) for this thread's 64 query columns; the sum comes from the tensor pipe
+            // phase 1: P^T = 2^(scale * (s + bias_t / scale)) for this thread's query columns; the sum comes from the tensor pipe
             ok = kTwoS ? mbar_wait(&bar.s_full[g & 1], (uint32_t)(g >> 1) & 1u, abortp) : mbar_wait(&bar.s_full[0], (uint32_t)g & 1u, abortp);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;

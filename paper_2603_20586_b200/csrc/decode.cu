@@ -1,5 +1,7 @@
 // Split-KV single-token decode of Eq. 5 (all cached rows of the three levels visible).
 //
+// Two forms (cluster_rule).  Short and evenly dealt caches: one kernel, decode_cluster_kernel, whose clusters finish a (batch, head)
+// each.  Otherwise the split form, two kernels; the paged and grouped decode (decode_paged.cu) ends with the second of them:
 // Kernel 1 (HBM-bound, streams K and V exactly once): grid = (batch*head) x chunks of the split
 // table.  A row of d bf16 values is covered by d/8 lanes with one 16-byte load each, so a warp reads
 // 32*16 contiguous bytes per instruction; each lane group keeps its own running (max, sum, acc) in the

@@ -6,7 +6,7 @@
 // Code bits are decided by fp32 arithmetic, so its order is fixed: sums run row by row, a projection is one fmaf
 // chain over the columns.
 //   l3_index_kernel     HBM-bound: reads every key of the pool once, writes bits/8 bytes per (page, KV head)
-//   l3_retrieve_kernel  one CTA per (sequence, KV head): query code, Hamming scores of the bank, R selection rounds
+//   l3_retrieve_kernel  one CTA per (sequence, KV head): query code, Hamming scores of the bank, a binary search for the R-th best
 #include "common.cuh"
 
 namespace mka {

@@ -84,6 +84,46 @@ def test_planted_chunk_is_recalled_and_dominates_the_decode(mka, orc):
     assert np.abs(np64(LSE) - Lr).max() <= 2e-3
 
 
+@pytest.mark.parametrize("bits,page,d", [(64, 16, 128), (128, 32, 64)])
+def test_serving_step_against_64_bits(mka, orc, bits, page, d):
+    """One token per sequence of a serving engine: gate, append of the fused row, recall, decode over window, session and recalled
+    chunks.  Which chunks are recalled hangs on single code bits (they are compared elsewhere, bit for bit), so the recalled
+    table is an input of the 64-bit decode here."""
+    B, H, Hkv, D, R, n, bank = 4, 12, 4, 96, 8, (300, 2000, 8 * page), 150
+    g = torch.Generator(device="cuda").manual_seed(bits)
+    rn = lambda *s, dt=torch.bfloat16: torch.randn(*s, device="cuda", generator=g, dtype=dt)  # noqa: E731
+    pk, pv, tab = [], [], []
+    for rows in (n[0], n[1], bank * page):
+        width = -(-rows // page)
+        pk.append(rn(B * width + 3, Hkv, page, d)), pv.append(rn(B * width + 3, Hkv, page, d))
+        tab.append(torch.randperm(B * width + 3, device="cuda", generator=g)[:B * width].view(B, width).to(torch.int32).contiguous())
+    len2 = torch.tensor([n[1], 1220, 40, 1], dtype=torch.int32, device="cuda")
+    len1, bank_len = len2.clamp(max=n[0]), torch.tensor([bank, 91, 3, 0], dtype=torch.int32, device="cuda")
+    X, W, q, proj = rn(B, 1, D), rn(D, 3, dt=torch.float32) * 0.1, rn(B, H, d), rn(bits, d, dt=torch.float32)
+    newK, newV = ([rn(B, Hkv, 1, d) for _ in range(3)] for _ in range(2))
+    codes = mka.mka_l3_index(pk[2], proj)
+    gate = mka.mka_router(X, W, None)
+    g64 = orc.router(np64(X).reshape(B, D), np64(W))[0]
+    assert np.abs(np64(gate).reshape(B, 3) - g64).max() <= 2e-6
+    mka.mka_fuse_kv_paged(newK, newV, gate, pk[1], pv[1], tab[1], dst_offsets=len2 - 1)
+    for pool, new in ((pk[1], newK), (pv[1], newV)):
+        for b in range(B):
+            r = int(len2[b]) - 1
+            want = sum(g64[b, l] * np64(new[l][b, :, 0]) for l in range(3))
+            assert np.abs(np64(pool[int(tab[1][b, r // page]), :, r % page]) - want).max() <= np.abs(want).max() / 256      # one rounding to bf16
+    table, n_sel, rows3 = mka.mka_l3_retrieve(q, Hkv, proj, codes, tab[2], bank_len, R, page)
+    assert n_sel.tolist() == [R, R, 3, 0]
+    shape = mka.make_shape(B, H, 1, d, D)
+    ws = torch.zeros(mka.mka_decode_paged_workspace_bytes(shape, Hkv, n), dtype=torch.uint8, device="cuda")
+    O, LSE = mka.mka_decode_paged(shape, Hkv, q, pk, pv, (tab[0], tab[1], table), n, gate.view(B, 3), rows=(len1, len2, rows3), ws=ws)
+    assert mka.mka_device_status(ws) == 0
+    ints = lambda t: t.cpu().numpy().astype(np.int64)  # noqa: E731
+    Or, Lr = orc.decode_paged(np64(q), [np64(k) for k in pk], [np64(v) for v in pv], [ints(tab[0]), ints(tab[1]), ints(table)],
+                              [ints(len1), ints(len2), ints(rows3)], page, g64)
+    check(O, Or, torch.bfloat16, "O of the serving step")
+    assert np.abs(np64(LSE) - Lr).max() <= 2e-3
+
+
 def test_l3_rejects_bad_arguments(mka):
     cfg = RecallConfig("t_bad", 37, 1, 8, 2, 64, 20, 8, 64, 4)
     P = make_recall(cfg, "cuda")
