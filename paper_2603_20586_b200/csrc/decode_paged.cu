@@ -308,7 +308,7 @@ struct TileWalk {
         b = lo << shift;
         if (shift > 0) {                  // and the sequence in it, 32 at a time
             const int end = min(p.B, (lo + 1) << shift);
-            for (;; b += 32) {
+            for (; b < end; b += 32) {
                 const int own = b + lane < end ? list_tiles(p, b + lane) : 0;
                 int sum = own;
 #pragma unroll
@@ -325,10 +325,11 @@ struct TileWalk {
                 }
                 ahead += __shfl_sync(0xffffffffu, sum, 31);
             }
+            b = min(b, end - 1);          // (row counts that change under the call may lead past the block: the walk ends all the same)
         }
         enter();
         const int in_seq = (int)(u0 - (long long)ahead * p.H_kv);
-        kvh = in_seq / tiles; at = in_seq - kvh * tiles;
+        kvh = min(in_seq / max(tiles, 1), p.H_kv - 1); at = in_seq - kvh * tiles;
     }
     __device__ __forceinline__ void enter() {
         tiles = 0;
@@ -351,7 +352,11 @@ struct TileWalk {
         at = 0;
         if (++kvh == p.H_kv) {
             kvh = 0;
-            do { ahead += tiles; ++b; enter(); } while (tiles == 0);
+            do {
+                if (++b == p.B) { b = p.B - 1; return false; }
+                ahead += tiles;
+                enter();
+            } while (tiles == 0);
         }
         return true;
     }
