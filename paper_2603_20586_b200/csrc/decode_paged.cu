@@ -269,12 +269,13 @@ struct PagedMaps {
     CUtensorMap k[3], v[3];
 };
 
-// Rows of level l that sequence b's list holds: none where the gate is 0.
+// Rows of level l that sequence b's list holds: none where the gate is 0.  No load hangs on another: asked for one after the other
+// (the row count only where the gate is open, level after level) the six of a sequence were six round trips at the start of every CTA.
 __device__ __forceinline__ int list_rows(const DecodePagedParams& p, int b, int l) {
     const PagedLevelDev& L = p.L[l];
-    if (L.n == 0 || !(p.gate[b * 3 + l] > 0.f)) return 0;
+    const float gate = p.gate[b * 3 + l];
     const long long n = L.rows ? (long long)L.rows[b] : L.n;
-    return (int)(n < 0 ? 0 : (n > L.n ? L.n : n));
+    return L.n == 0 || !(gate > 0.f) ? 0 : (int)(n < 0 ? 0 : (n > L.n ? L.n : n));
 }
 
 // Tiles of one list of sequence b.
@@ -328,6 +329,7 @@ struct TileWalk {
             b = min(b, end - 1);          // (row counts that change under the call may lead past the block: the walk ends all the same)
         }
         enter();
+        if (shift == 0) tiles = before[b + 1] - ahead;        // (no need to wait for the row counts)
         const int in_seq = (int)(u0 - (long long)ahead * p.H_kv);
         kvh = min(in_seq / max(tiles, 1), p.H_kv - 1); at = in_seq - kvh * tiles;
     }
@@ -388,8 +390,10 @@ __global__ void __launch_bounds__(kTmaThreads, 2) decode_paged_tma_kernel(const 
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     const int shift = p.deal_shift, blocks = (p.B + (1 << shift) - 1) >> shift;
-    for (int i = tid; i <= blocks; i += kTmaThreads) before[i] = 0;
-    __syncthreads();
+    if (shift > 0) {
+        for (int i = tid; i < blocks; i += kTmaThreads) before[i] = 0;
+        __syncthreads();
+    }
     for (int b0 = tid; b0 < p.B; b0 += 4 * kTmaThreads) {   // four sequences' row counts and gates in flight
         int t[4];
 #pragma unroll
@@ -398,8 +402,9 @@ __global__ void __launch_bounds__(kTmaThreads, 2) decode_paged_tma_kernel(const 
         for (int u = 0; u < 4; ++u) {
             const int b = b0 + u * kTmaThreads;
             if (b >= p.B) break;
-            if (t[u]) atomicAdd(&before[b >> shift], t[u]);
-            else if (b % gridDim.x == blockIdx.x)           // a sequence without a tile has no partials
+            if (shift == 0) before[b] = t[u];
+            else atomicAdd(&before[b >> shift], t[u]);
+            if (t[u] == 0 && b % gridDim.x == blockIdx.x)   // a sequence without a tile has no partials
                 for (int h = 0; h < p.H; ++h) p.partial[((long long)b * p.H + h) * list_floats] = 0.f;
         }
     }
