@@ -54,15 +54,15 @@ def load_peaks():
 # as it was when the counters were taken: when the file has changed since, the figure is reported as null ("stale").
 NCU_TRAFFIC = {
     # kernel@workload: (bytes in the capture, units of the capture, summary file under profiles/, source file, its digest)
-    "fwd_tc_kernel@c3": (376.523776e6 + 61.946368e6, 1 * 8, "fwd_tc_kernel_c3p.md", "fwd_tc.cu", "58f08d0c47e4"),
-    "fwd_tc_kernel64@c2": (204.546304e6 + 28.208640e6, 8 * 16, "fwd_tc_kernel64_c2.md", "fwd_tc.cu", "58f08d0c47e4"),   # the whole configuration
-    "decode_partial_kernel@c4": (1.476476e9 + 5.132288e6, 2 * 32, "decode_partial_kernel_c4p.md", "decode.cu", "ed9d09920f1b"),
-    "bwd_dq_tc_kernel@c5": (220.275200e6 + 27.056128e6, 1 * 16, "bwd_tc_kernels_c5p.md", "bwd_tc.cu", "5b543af267de"),
-    "bwd_dkv_tc_kernel@c5": (220.271872e6 + 114.367232e6, 1 * 16, "bwd_tc_kernels_c5p.md", "bwd_tc.cu", "5b543af267de"),
+    "fwd_tc_kernel@c3": (376.073216e6 + 57.210112e6, 1 * 8, "fwd_tc_kernel_c3p.md", "fwd_tc.cu", "266857ed858f"),
+    "fwd_tc_kernel64@c2": (204.392704e6 + 27.338752e6, 8 * 16, "fwd_tc_kernel64_c2.md", "fwd_tc.cu", "266857ed858f"),   # the whole configuration
+    "decode_partial_kernel@c4": (1.476515e9 + 3.866880e6, 2 * 32, "decode_partial_kernel_c4p.md", "decode.cu", "93b91a32241a"),
+    "bwd_dq_tc_kernel@c5": (220.267264e6 + 26.553088e6, 1 * 16, "bwd_tc_kernels_c5p.md", "bwd_tc.cu", "62205ef506c5"),
+    "bwd_dkv_tc_kernel@c5": (220.343808e6 + 116.964864e6, 1 * 16, "bwd_tc_kernels_c5p.md", "bwd_tc.cu", "62205ef506c5"),
     "l2_summary_seg_kernel@s3": (101.000704e6 + 55.384064e6, 12288.0 / 32768.0, "l2_summary_seg_kernel_s3p.md", "summary_seg.cu", "6e2dcc00fbde"),   # 12288 of the 32768 tokens
     "fuse_kv_kernel@f3": (403.137024e6 + 83.414784e6, 1 * 8, "fuse_kv_kernel_f3p.md", "fuse_kv.cu", "3becacc721a4"),
-    "decode_paged_kernel@g4": (293.682688e6 + 3.988480e6, 1 * 4, "decode_paged_kernel_g4p.md", "decode_paged.cu", "712e1e791061"),   # one of the four sequences (g4p)
-    "l3_index_kernel@r3": (134.301696e6 + 3.607552e6, 1, "l3_index_kernel_r3p.md", "l3.cu", "6e05d1bc7821"),            # one of the four sequences (r3p)
+    "decode_paged_kernel@g4": (293.738240e6 + 3.420928e6, 1 * 4, "decode_paged_kernel_g4p.md", "decode_paged.cu", "f1544adcf30a"),   # one of the four sequences (g4p)
+    "l3_index_kernel@r3": (134.313728e6 + 3.178496e6, 1, "l3_index_kernel_r3p.md", "l3.cu", "feaf0bd07ff1"),            # one of the four sequences (r3p)
 }
 
 
