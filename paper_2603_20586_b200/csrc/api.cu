@@ -206,7 +206,6 @@ mka_status mka_fwd(const mka_shape* s, const void* Q, const mka_level L[3], cons
     p.status = static_cast<unsigned int*>(ws);
     cudaError_t e;
     if (!(s->flags & MKA_FLAG_FORCE_SIMT) && s->mode == MKA_MODE_FAST && fwd_tc_eligible(p, s->dtype)) {
-        if (cudaMemsetAsync(ws, 0, 16, cs) != cudaSuccess) return MKA_ERR_CUDA;
         e = launch_fwd_tc(p, static_cast<unsigned int*>(ws), cs);
     } else {
         e = launch_fwd_simt(p, s->dtype, cs);
@@ -332,7 +331,7 @@ static mka_status run_decode_paged(DecodePagedParams& p, DecodeParams& c, const 
     c.total_chunks = p.total_chunks;
     p.partial = c.partial = reinterpret_cast<float*>(static_cast<char*>(ws) + kWsHeader);
     p.status = static_cast<unsigned int*>(ws); p.wait_limit_ns = wait_limit_ns();
-    if (cudaMemsetAsync(ws, 0, 16, cs) != cudaSuccess) return MKA_ERR_CUDA;
+    if (plan.total_chunks == 0) c.status = p.status;         // only the combine kernel runs
     cudaError_t e = launch_decode_paged(p, cs);
     if (e == cudaErrorNotSupported && p.dealt) {             // a map could not be encoded: the first form takes any layout
         p.dealt = c.counted = 0;
@@ -387,7 +386,6 @@ mka_status mka_fwd_paged(const mka_shape* s, int32_t H_kv, const void* Q, const 
     p.window = s->window; p.q_offset = s->q_offset; p.scale = resolve_scale(s);
     p.mode = s->mode; p.decode = 0; p.kv_group = s->H / H_kv; p.paged = P;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(ws, 0, 16, cs) != cudaSuccess) return MKA_ERR_CUDA;
     cudaError_t e = launch_fwd_tc(p, static_cast<unsigned int*>(ws), cs);
     if (e == cudaErrorNotSupported) return MKA_ERR_UNSUPPORTED;
     return e == cudaSuccess ? MKA_OK : MKA_ERR_CUDA;

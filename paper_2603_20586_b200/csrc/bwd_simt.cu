@@ -12,6 +12,7 @@ namespace {
 
 template <typename T, int DH, int GROUPS>
 __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1) bwd_dq_kernel(const BwdParams p, const int vec) {
+    chain_enter();
     using S = SimtCta<GROUPS>;
     constexpr int kRows = S::kRows, kGroupThreads = S::kWarps * 32;
     constexpr int CPL = DH / 32, LD = DH + 4, kTileFloats = kSimtTile * LD, R = kSimtWarpRows;
@@ -176,6 +177,7 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
 // covers the three levels: blockIdx.x runs through L1's, L2's and L3's key tiles.
 template <typename T, int DH, int GROUPS>
 __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1) bwd_dkv_kernel(const BwdParams p, const int vec) {
+    chain_enter();
     using S = SimtCta<GROUPS>;
     constexpr int kRows = S::kRows, kGroupThreads = S::kWarps * 32;
     constexpr int CPL = DH / 32, LD = DH + 4, kTileFloats = kSimtTile * LD, R = kSimtWarpRows;
@@ -315,6 +317,7 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
 }
 
 __global__ void bwd_dgate_kernel(const float* __restrict__ Gpart, int B, int H, long long T, float* __restrict__ dG) {
+    chain_enter();
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;   // over B*T*3
     if (i >= (long long)B * T * 3) return;
     long long b = i / (T * 3), rem = i % (T * 3);
@@ -328,8 +331,7 @@ __global__ void bwd_dgate_kernel(const float* __restrict__ Gpart, int B, int H, 
 cudaError_t launch_bwd_dgate(const float* Gpart, int B, int H, long long T, float* dG, cudaStream_t st) {
     const long long n = (long long)B * T * 3;
     if (n == 0) return cudaSuccess;
-    bwd_dgate_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(Gpart, B, H, T, dG);
-    return cudaGetLastError();
+    return launch_chained(bwd_dgate_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, 0, Gpart, B, H, T, dG);
 }
 
 namespace {
@@ -340,8 +342,7 @@ cudaError_t launch_dq(const BwdParams& p, int vec, cudaStream_t st) {
     const size_t smem = sizeof(float) * (2 * S::kRows * DH + S::kThreads * kSimtWarpRows + (size_t)S::kGroups * 2 * kSimtTile * (DH + 4));
     const cudaError_t e = cudaFuncSetAttribute(bwd_dq_kernel<T, DH, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    bwd_dq_kernel<T, DH, GROUPS><<<dim3((p.T + S::kRows - 1) / S::kRows, p.H, p.B), S::kThreads, smem, st>>>(p, vec);
-    return cudaGetLastError();
+    return launch_chained(bwd_dq_kernel<T, DH, GROUPS>, dim3((p.T + S::kRows - 1) / S::kRows, p.H, p.B), dim3(S::kThreads), smem, st, 0, p, vec);
 }
 
 template <typename T, int DH, int GROUPS>
@@ -353,8 +354,8 @@ cudaError_t launch_dkv(const BwdParams& p, int vec, cudaStream_t st) {
     const size_t smem = sizeof(float) * (2 * S::kRows * DH + S::kThreads * 2 * kSimtWarpRows + (size_t)S::kGroups * 2 * kSimtTile * (DH + 4));
     const cudaError_t e = cudaFuncSetAttribute(bwd_dkv_kernel<T, DH, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    bwd_dkv_kernel<T, DH, GROUPS><<<dim3((unsigned)key_tiles, p.H / (p.kv_group > 0 ? p.kv_group : 1), p.B), S::kThreads, smem, st>>>(p, vec);
-    return cudaGetLastError();
+    return launch_chained(bwd_dkv_kernel<T, DH, GROUPS>, dim3((unsigned)key_tiles, p.H / (p.kv_group > 0 ? p.kv_group : 1), p.B), dim3(S::kThreads), smem, st, 0, p,
+                          vec);
 }
 
 template <typename T, int DH>

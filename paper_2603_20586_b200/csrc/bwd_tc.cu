@@ -210,6 +210,7 @@ __global__ void __launch_bounds__(256) bwd_prep_kernel(const __nv_bfloat16* __re
                                                        int T, int Tpad, float* __restrict__ sD,
                                                        float* __restrict__ b0, float* __restrict__ b1, float* __restrict__ b2,
                                                        unsigned int* __restrict__ header) {
+    chain_enter();
     if (threadIdx.x < 4 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) header[threadIdx.x] = 0u;   // status word and tickets of the kernels that follow
     constexpr int LPR = DH / 8;                            // lanes per row: 16 or 8
     constexpr int RPW = 32 / LPR;                          // rows per warp and pass
@@ -360,6 +361,7 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const 
         for (int i = 0; i < 2; ++i) { mbar_init(&bar.item_full[i], 1); mbar_init(&bar.item_free[i], 1 + C::kEw); }   // the issuing warp and the element-wise warps
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    chain_enter();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -743,6 +745,7 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
     __syncthreads();
     if (tid < kBlk) *reinterpret_cast<uint4*>(sAugK + (tid & 7) * 16 + (tid >> 3) * 256) = make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    chain_enter();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -1143,10 +1146,9 @@ cudaError_t launch_t(const BwdParams& bp, unsigned int* status_word, cudaStream_
     const long long sq_n = DH, sq_h = (long long)bp.T * DH, sq_b = (long long)bp.H * bp.T * DH;
 
     constexpr int kPrepRowsPerBlock = 8 * (32 / (DH / 8)) * 4;          // 8 warps x rows per pass x passes
-    bwd_prep_kernel<DH><<<dim3((Tpad + kPrepRowsPerBlock - 1) / kPrepRowsPerBlock, bp.H, bp.B), 256, 0, st>>>(
-        static_cast<const __nv_bfloat16*>(bp.O), static_cast<const __nv_bfloat16*>(bp.dO), bp.LSE, bp.gate, bp.H, bp.T, Tpad,
-        statD, statB[0], statB[1], statB[2], status_word);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_chained(bwd_prep_kernel<DH>, dim3((Tpad + kPrepRowsPerBlock - 1) / kPrepRowsPerBlock, bp.H, bp.B), dim3(256), 0, st, 0,
+                                   static_cast<const __nv_bfloat16*>(bp.O), static_cast<const __nv_bfloat16*>(bp.dO), bp.LSE, bp.gate, bp.H, bp.T,
+                                   Tpad, statD, statB[0], statB[1], statB[2], status_word);
     if (e != cudaSuccess) return e;
 
     BwdTcParams p;
@@ -1183,8 +1185,8 @@ cudaError_t launch_t(const BwdParams& bp, unsigned int* status_word, cudaStream_
         if (e != cudaSuccess) return e;
         p.dq_items = (long long)(Tpad / kBlk) * bp.H * bp.B;
         p.dq_ticket = status_word + 2;
-        bwd_dq_tc_kernel<DH><<<(unsigned)(p.dq_items < 148 ? p.dq_items : 148), C::kThreads, C::kSmemDq, st>>>(m, p);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = launch_chained(bwd_dq_tc_kernel<DH>, dim3((unsigned)(p.dq_items < 148 ? p.dq_items : 148)), dim3(C::kThreads), C::kSmemDq, st, 0, m, p);
+        if (e != cudaSuccess) return e;
     }
     const int tiles = p.kv_tiles[0] + p.kv_tiles[1] + p.kv_tiles[2];
     if (tiles > 0) {
@@ -1202,8 +1204,8 @@ cudaError_t launch_t(const BwdParams& bp, unsigned int* status_word, cudaStream_
         if (e != cudaSuccess) return e;
         p.dkv_items = (long long)tiles * H_kv * bp.B;
         p.dkv_ticket = status_word + 1;
-        bwd_dkv_tc_kernel<DH><<<(unsigned)(p.dkv_items < 148 ? p.dkv_items : 148), C::kThreadsDkv, C::kSmemDkv, st>>>(m, p);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = launch_chained(bwd_dkv_tc_kernel<DH>, dim3((unsigned)(p.dkv_items < 148 ? p.dkv_items : 148)), dim3(C::kThreadsDkv), C::kSmemDkv, st, 0, m, p);
+        if (e != cudaSuccess) return e;
     }
     return launch_bwd_dgate(bp.Gpart, bp.B, bp.H, bp.T, bp.dG, st);
 }

@@ -74,6 +74,7 @@ __device__ __forceinline__ void merge_warps(const float (&sm_m)[kWarps], const f
 
 template <int DH>
 __global__ void __launch_bounds__(kWarps * 32, 2) decode_partial_kernel(const DecodeParams p) {
+    chain_enter();
     constexpr int LPR = DH / 8;          // lanes per row
     constexpr int RPI = 32 / LPR;        // rows per warp-wide load instruction
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -181,6 +182,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) decode_partial_kernel(const De
 // sequence with 32 heads and 512 + 1000 + 64 rows took 12.1 us in two kernels, 9.7 here.
 template <int DH>
 __global__ void __launch_bounds__(kWarps * 32, 2) decode_cluster_kernel(const DecodeParams p) {
+    chain_enter();
     constexpr int LPR = DH / 8, RPI = 32 / LPR, SLAB = RPI * kUnroll;
     __shared__ float sm_m[kWarps], sm_z[kWarps], sm_acc[kWarps][DH];
     __shared__ float cta_m, cta_z, cta_acc[DH];
@@ -303,6 +305,7 @@ __global__ void __launch_bounds__(kWarps * 32, 2) decode_cluster_kernel(const De
 
 template <int DH>
 __global__ void __launch_bounds__(DH) decode_combine_kernel(const DecodeParams p) {
+    chain_enter();
     const long long bh = blockIdx.x;
     const int b = (int)(bh / p.H);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -422,22 +425,13 @@ template <int DH>
 cudaError_t launch_t(const DecodeParams& p, cudaStream_t st) {
     const long long bh = (long long)p.B * p.H;
     if (bh == 0) return cudaSuccess;
-    if (const int size = cluster_rule(p)) {
-        cudaLaunchAttribute at;
-        at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim.x = size; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(bh * size)); cfg.blockDim = dim3(kWarps * 32); cfg.stream = st;
-        cfg.attrs = &at; cfg.numAttrs = 1;
-        return cudaLaunchKernelEx(&cfg, decode_cluster_kernel<DH>, p);
-    }
+    if (const int size = cluster_rule(p))
+        return launch_chained(decode_cluster_kernel<DH>, dim3((unsigned)(bh * size)), dim3(kWarps * 32), 0, st, size, p);
     if (p.total_chunks > 0) {
-        decode_partial_kernel<DH><<<(unsigned)(bh * p.total_chunks), kWarps * 32, 0, st>>>(p);
-        cudaError_t e = cudaGetLastError();
+        cudaError_t e = launch_chained(decode_partial_kernel<DH>, dim3((unsigned)(bh * p.total_chunks)), dim3(kWarps * 32), 0, st, 0, p);
         if (e != cudaSuccess) return e;
     }
-    decode_combine_kernel<DH><<<(unsigned)bh, DH, 0, st>>>(p);
-    return cudaGetLastError();
+    return launch_chained(decode_combine_kernel<DH>, dim3((unsigned)bh), dim3(DH), 0, st, 0, p);
 }
 
 }  // namespace
@@ -445,10 +439,8 @@ cudaError_t launch_t(const DecodeParams& p, cudaStream_t st) {
 cudaError_t launch_decode_combine(const DecodeParams& p, cudaStream_t st) {
     const long long bh = (long long)p.B * p.H;
     if (bh == 0) return cudaSuccess;
-    if (p.d == 128) decode_combine_kernel<128><<<(unsigned)bh, 128, 0, st>>>(p);
-    else if (p.d == 64) decode_combine_kernel<64><<<(unsigned)bh, 64, 0, st>>>(p);
-    else return cudaErrorNotSupported;
-    return cudaGetLastError();
+    if (p.d != 128 && p.d != 64) return cudaErrorNotSupported;
+    return launch_chained(p.d == 128 ? decode_combine_kernel<128> : decode_combine_kernel<64>, dim3((unsigned)bh), dim3(p.d), 0, st, 0, p);
 }
 
 cudaError_t launch_decode(const DecodeParams& p, cudaStream_t st) {

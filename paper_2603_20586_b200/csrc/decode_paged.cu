@@ -49,6 +49,8 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
 
 template <int DH>
 __global__ void __launch_bounds__(kThreads, 2) decode_paged_kernel(const DecodePagedParams p) {
+    chain_enter();
+    if (blockIdx.x == 0 && threadIdx.x == 0 && p.status) *p.status = MKA_OK;
     constexpr int kPitch = DH * 2 + 16;                     // bytes between rows in shared memory: ldmatrix hits every bank once
     constexpr int kTileBytes = kTileRows * kPitch;          // one of K or V
     constexpr int kVecPerRow = DH / 8;                      // 16-byte pieces of a row
@@ -389,6 +391,8 @@ __global__ void __launch_bounds__(kTmaThreads, 2) decode_paged_tma_kernel(const 
         for (int i = 0; i < kTmaStages; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 4); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    chain_enter();
+    if (blockIdx.x == 0 && tid == 0 && p.status) atomicExch(p.status, (unsigned int)MKA_OK);   // (see fwd_tc_kernel)
     const int shift = p.deal_shift, blocks = (p.B + (1 << shift) - 1) >> shift;
     if (shift > 0) {
         for (int i = tid; i < blocks; i += kTmaThreads) before[i] = 0;
@@ -702,8 +706,7 @@ cudaError_t launch_tma(DecodePagedParams p, cudaStream_t st) {
     const size_t smem = (size_t)kTmaStages * 2 * kTileRows * DH * 2 + 1024 + (DH / 8 * 4 + 4) * 32 * sizeof(float) + (kDealBlocks + 1) * sizeof(int);
     cudaError_t e = cudaFuncSetAttribute(decode_paged_tma_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    decode_paged_tma_kernel<DH><<<kDealCtas, kTmaThreads, smem, st>>>(maps, p);
-    return cudaGetLastError();
+    return launch_chained(decode_paged_tma_kernel<DH>, dim3(kDealCtas), dim3(kTmaThreads), smem, st, 0, maps, p);
 }
 
 template <int DH>
@@ -713,8 +716,7 @@ cudaError_t launch_t(const DecodePagedParams& p, cudaStream_t st) {
     const size_t smem = (size_t)kStages * 2 * kTileRows * (DH * 2 + 16);
     cudaError_t e = cudaFuncSetAttribute(decode_paged_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    decode_paged_kernel<DH><<<(unsigned)ctas, kThreads, smem, st>>>(p);
-    return cudaGetLastError();
+    return launch_chained(decode_paged_kernel<DH>, dim3((unsigned)ctas), dim3(kThreads), smem, st, 0, p);
 }
 
 }  // namespace

@@ -64,6 +64,7 @@ struct FuseParams {
 
 template <typename T>
 __global__ void __launch_bounds__(256) fuse_kv_kernel(const FuseParams p, const long long total_vecs) {
+    chain_enter();
     constexpr int E = Vec<T>::kElems;
     const int vpr = p.d / E;                                     // vectors per row
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total_vecs; i += (long long)gridDim.x * blockDim.x) {
@@ -122,9 +123,8 @@ cudaError_t launch_fuse_kv(const LevelDev L[3], const LevelGradDev& out, const f
     long long blocks = (total + 255) / 256;
     const long long cap = 148LL * 8 * 8;                          // a few waves of resident CTAs; the loop strides over the rest
     if (blocks > cap) blocks = cap;
-    if (dtype == MKA_BF16) fuse_kv_kernel<__nv_bfloat16><<<(unsigned)blocks, 256, 0, st>>>(p, total);
-    else fuse_kv_kernel<float><<<(unsigned)blocks, 256, 0, st>>>(p, total);
-    return cudaGetLastError();
+    return launch_chained(dtype == MKA_BF16 ? fuse_kv_kernel<__nv_bfloat16> : fuse_kv_kernel<float>, dim3((unsigned)blocks), dim3(256), 0, st, 0, p,
+                          total);
 }
 
 }  // namespace mka

@@ -13,6 +13,7 @@ namespace {
 
 template <typename T, int DH, int MODE, int GROUPS>
 __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1) fwd_simt_kernel(const FwdParams p, const int vec) {
+    chain_enter();
     using S = SimtCta<GROUPS>;
     constexpr int kRows = S::kRows, kGroupThreads = S::kWarps * 32;
     constexpr int NS = MODE == MKA_MODE_FULL ? 3 : 1;    // softmax states
@@ -189,8 +190,7 @@ cudaError_t launch_g(const FwdParams& p, cudaStream_t st) {
     auto kern = fwd_simt_kernel<T, DH, MODE, GROUPS>;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<grid, S::kThreads, smem, st>>>(p, vec);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, dim3(S::kThreads), smem, st, 0, p, vec);
 }
 
 template <typename T, int DH>

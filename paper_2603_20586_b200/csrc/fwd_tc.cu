@@ -190,6 +190,10 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    chain_enter();
+    // The status word starts at OK.  CTAs start in the order of their numbers and none gives up before the wait limit (100 us at
+    // least) has passed, so the first one clears it before any other can have something to report.
+    if (tid == 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) atomicExch(p.status, (unsigned int)MKA_OK);
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(C::kTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -917,14 +921,7 @@ cudaError_t launch_t(const FwdParams& fp, unsigned int* status_word, cudaStream_
                          : (split > 1 ? fwd_tc_kernel<DH, false, true> : fwd_tc_kernel<DH, false, false>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<DH>::kSmemBytes);
     if (e != cudaSuccess) return e;
-    if (split > 1) {
-        cudaLaunchAttribute at;
-        const cudaLaunchConfig_t cfg = cluster_config<DH>(split, dim3(q_blocks * split, fp.H, fp.B), st, &at);
-        return cudaLaunchKernelEx(&cfg, kern, maps, p);
-    }
-    dim3 grid(q_blocks, fp.H, fp.B);
-    kern<<<grid, Cfg<DH>::kThreads, Cfg<DH>::kSmemBytes, st>>>(maps, p);
-    return cudaGetLastError();
+    return launch_chained(kern, dim3(q_blocks * split, fp.H, fp.B), dim3(Cfg<DH>::kThreads), Cfg<DH>::kSmemBytes, st, split > 1 ? split : 0, maps, p);
 }
 
 }  // namespace

@@ -35,6 +35,7 @@ struct L3IndexParams {
 // rows, 128] at 64 bits, 123 us now (4.4 TB/s).  Registers are moved from the projecting to the loading warps.
 template <int DH>
 __global__ void __launch_bounds__(2 * kIdxThreads, 2) l3_index_kernel(const L3IndexParams p) {
+    chain_enter();
     extern __shared__ __align__(16) float sm[];
     const int ppitch = p.bits + 4;                             // floats between columns of projT (keeps the fill off one bank)
     constexpr int pitch = DH + 1, kSumFloats = kIdxPairs * pitch;
@@ -197,6 +198,7 @@ __global__ void __launch_bounds__(2 * kIdxThreads, 2) l3_index_kernel(const L3In
 // Dynamic shared memory: projT [d][bits + 4] floats, then s [kPhasePairs][d + 1] floats.
 template <int DH>
 __global__ void __launch_bounds__(kIdxThreads, 4) l3_index_phases_kernel(const L3IndexParams p) {
+    chain_enter();
     extern __shared__ __align__(16) float sm[];
     const int ppitch = p.bits + 4;                             // floats between columns of projT (keeps the fill off one bank)
     float* projT = sm;
@@ -329,6 +331,7 @@ __device__ __forceinline__ int cta_sum(int v, int* part, int warp, int lane) {
 // the list.  15 us now.
 // Dynamic shared memory: unsigned short score[max_bank], int before[max_bank / 32 rounded up to whole CTAs], the projection.
 __global__ void __launch_bounds__(kRetThreads) l3_retrieve_kernel(const L3RetrieveParams p) {
+    chain_enter();
     extern __shared__ __align__(16) unsigned short score[];
     __shared__ __align__(16) float qs[256];
     __shared__ __align__(16) unsigned int qcode[8];
@@ -540,8 +543,7 @@ cudaError_t launch_l3_index(const void* k, long long n_pages, int H_kv, int page
         if (e != cudaSuccess) return e;
         const long long batches = (n_pages * H_kv + batch - 1) / batch, resident = 148LL * ctas_per_sm(smem);
         const long long per_cta = (batches + resident - 1) / resident, grid = (batches + per_cta - 1) / per_cta;
-        kern<<<(unsigned)grid, threads, smem, st>>>(p);
-        return cudaGetLastError();
+        return launch_chained(kern, dim3((unsigned)grid), dim3(threads), smem, st, 0, p);
     };
     if (two_phases(p))
         return launch(d == 128 ? l3_index_phases_kernel<128> : l3_index_phases_kernel<64>, kPhasePairs, 1, kIdxThreads,
@@ -567,8 +569,7 @@ cudaError_t launch_l3_retrieve(const void* q, int B, int H, int H_kv, int d, con
     if (p.stage_proj) smem = with_proj;
     cudaError_t e = cudaFuncSetAttribute(l3_retrieve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    l3_retrieve_kernel<<<(unsigned)(B * H_kv), kRetThreads, smem, st>>>(p);
-    return cudaGetLastError();
+    return launch_chained(l3_retrieve_kernel, dim3((unsigned)(B * H_kv)), dim3(kRetThreads), smem, st, 0, p);
 }
 
 }  // namespace mka

@@ -126,6 +126,7 @@ router_kernel(const T* __restrict__ R, const float* __restrict__ W_r, const floa
               long long rows, int D, int route, float* __restrict__ gate, float* __restrict__ log2_gate,
               int8_t* __restrict__ idx) {
     __shared__ float part[kMaxThreads / 32][ROWS * 3];
+    chain_enter();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long row0 = (long long)blockIdx.x * ROWS;
     const long long last = rows - 1 - row0;                       // a row past the end reads the last one again
@@ -178,6 +179,7 @@ __global__ void __launch_bounds__(kWarps * 32)
 router_rows_kernel(const T* __restrict__ R, const float* __restrict__ W_r, const float* __restrict__ b_r,
                    long long rows, int D, int route, float* __restrict__ gate, float* __restrict__ log2_gate,
                    int8_t* __restrict__ idx) {
+    chain_enter();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long row0 = ((long long)blockIdx.x * kWarps + warp) * kRowsPerWarp;
     if (row0 >= rows) return;
@@ -219,6 +221,7 @@ __global__ void __launch_bounds__(kWarps * 32)
 router_any_kernel(const T* __restrict__ R, const float* __restrict__ W_r, const float* __restrict__ b_r,
                   long long rows, int D, int route, float* __restrict__ gate, float* __restrict__ log2_gate,
                   int8_t* __restrict__ idx) {
+    chain_enter();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long row0 = ((long long)blockIdx.x * kWarps + warp) * kRowsPerWarp;
     if (row0 >= rows) return;
@@ -292,6 +295,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 router_bwd_partial_kernel(const T* __restrict__ R, const float* __restrict__ dG, long long rows, int D,
                           int n_row_chunks, float* __restrict__ partial, double* __restrict__ db_partial) {
+    chain_enter();
     const int c = blockIdx.x * 256 + threadIdx.x;
     const int chunk = blockIdx.y;
     const long long per = (rows + n_row_chunks - 1) / n_row_chunks;
@@ -330,6 +334,7 @@ router_bwd_partial_vec_kernel(const T* __restrict__ R, const float* __restrict__
                            int n_row_chunks, float* __restrict__ partial, double* __restrict__ db_partial) {
     constexpr int kBatch = N * sizeof(T) <= 16 ? 8 : 4;        // rows of a batch: loads in flight a lane = 8
     __shared__ float sum[8][3 * N][33];
+    chain_enter();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int c = blockIdx.x * (32 * N) + lane * N;
     const int chunk = blockIdx.y;
@@ -390,6 +395,7 @@ router_bwd_partial_vec_kernel(const T* __restrict__ R, const float* __restrict__
 __global__ void __launch_bounds__(256) router_bwd_reduce_kernel(const float* __restrict__ partial, const float* __restrict__ dG, long long rows,
                                                                 int D, int n_row_chunks, const double* __restrict__ db_partial,
                                                                 float* __restrict__ dW_r, float* __restrict__ db_r) {
+    chain_enter();
     if (db_r && blockIdx.x == gridDim.x - 1) {
         __shared__ double sm[256][3];
         double b[3];
@@ -419,39 +425,34 @@ __global__ void __launch_bounds__(256) router_bwd_reduce_kernel(const float* __r
 
 namespace {
 template <typename T>
-void router_t(const T* R, const float* W_r, const float* b_r, long long rows, int D, int route, float* gate, float* log2_gate,
+cudaError_t router_t(const T* R, const float* W_r, const float* b_r, long long rows, int D, int route, float* gate, float* log2_gate,
               int8_t* idx, cudaStream_t st) {
     if (D % 8 || (uintptr_t)R % 16 || (uintptr_t)W_r % 16) {
         const long long rows_per_cta = kWarps * kRowsPerWarp;
-        router_any_kernel<T><<<(unsigned)((rows + rows_per_cta - 1) / rows_per_cta), kWarps * 32, 0, st>>>(
-            R, W_r, b_r, rows, D, route, gate, log2_gate, idx);
-        return;
+        return launch_chained(router_any_kernel<T>, dim3((unsigned)((rows + rows_per_cta - 1) / rows_per_cta)), dim3(kWarps * 32), 0, st, 0,
+                              R, W_r, b_r, rows, D, route, gate, log2_gate, idx);
     }
     // Up to two rows per SM: one row to a CTA, for the shortest chain; to eight per SM: two; below 32 a row is still better
     // split over a CTA (2000 rows of 2048 bf16: 5.2 us against 8.4), above it the warps have enough to do on their own
     // (32768 rows: 28 us against 51; loads ahead of the sums and W_r in shared memory were slower too, 35 and 44 us).
     if (rows >= 32 * 148) {
         const long long rows_per_cta = kWarps * kRowsPerWarp;
-        router_rows_kernel<T><<<(unsigned)((rows + rows_per_cta - 1) / rows_per_cta), kWarps * 32, 0, st>>>(
-            R, W_r, b_r, rows, D, route, gate, log2_gate, idx);
-        return;
+        return launch_chained(router_rows_kernel<T>, dim3((unsigned)((rows + rows_per_cta - 1) / rows_per_cta)), dim3(kWarps * 32), 0, st, 0,
+                              R, W_r, b_r, rows, D, route, gate, log2_gate, idx);
     }
     const int threads = D >= 8 * kMaxThreads ? kMaxThreads : (D / 8 + 31) / 32 * 32;
-    if (rows >= 8 * 148)
-        router_kernel<T, 8><<<(unsigned)((rows + 7) / 8), threads, 0, st>>>(R, W_r, b_r, rows, D, route, gate, log2_gate, idx);
-    else if (rows >= 2 * 148)
-        router_kernel<T, 2><<<(unsigned)((rows + 1) / 2), threads, 0, st>>>(R, W_r, b_r, rows, D, route, gate, log2_gate, idx);
-    else
-        router_kernel<T, 1><<<(unsigned)rows, threads, 0, st>>>(R, W_r, b_r, rows, D, route, gate, log2_gate, idx);
+    const int per_cta = rows >= 8 * 148 ? 8 : (rows >= 2 * 148 ? 2 : 1);
+    auto kern = per_cta == 8 ? router_kernel<T, 8> : (per_cta == 2 ? router_kernel<T, 2> : router_kernel<T, 1>);
+    return launch_chained(kern, dim3((unsigned)((rows + per_cta - 1) / per_cta)), dim3(threads), 0, st, 0, R, W_r, b_r, rows, D, route, gate,
+                          log2_gate, idx);
 }
 }  // namespace
 
 cudaError_t launch_router(const void* R, const float* W_r, const float* b_r, long long rows, int D, int r_dtype,
                           int route, float* gate, float* log2_gate, int8_t* idx, cudaStream_t st) {
     if (rows == 0) return cudaSuccess;
-    if (r_dtype == MKA_BF16) router_t(static_cast<const __nv_bfloat16*>(R), W_r, b_r, rows, D, route, gate, log2_gate, idx, st);
-    else router_t(static_cast<const float*>(R), W_r, b_r, rows, D, route, gate, log2_gate, idx, st);
-    return cudaGetLastError();
+    if (r_dtype == MKA_BF16) return router_t(static_cast<const __nv_bfloat16*>(R), W_r, b_r, rows, D, route, gate, log2_gate, idx, st);
+    return router_t(static_cast<const float*>(R), W_r, b_r, rows, D, route, gate, log2_gate, idx, st);
 }
 
 cudaError_t launch_router_bwd(const void* R, int r_dtype, const float* dG, long long rows, int D, float* dW_r,
@@ -466,19 +467,20 @@ cudaError_t launch_router_bwd(const void* R, int r_dtype, const float* dG, long 
     const int col_blocks = cols == 1 ? (D + 255) / 256 : (D + 32 * cols - 1) / (32 * cols);
     if (cols > 1 && n_row_chunks > 296 / col_blocks) n_row_chunks = 296 / col_blocks > 0 ? 296 / col_blocks : 1;
     double* db_part = dW_r && db_r ? db_partial : nullptr;
+    cudaError_t e = cudaSuccess;
     if (dW_r) {
         const dim3 grid(col_blocks, n_row_chunks);
         auto launch = [&](const auto* r) {
             using T = std::remove_cv_t<std::remove_pointer_t<decltype(r)>>;
             auto kern = cols == 8 ? router_bwd_partial_vec_kernel<T, 8> : (cols == 4 ? router_bwd_partial_vec_kernel<T, 4> : router_bwd_partial_kernel<T>);
-            kern<<<grid, 256, 0, st>>>(r, dG, rows, D, n_row_chunks, partial, db_part);
+            e = launch_chained(kern, grid, dim3(256), 0, st, 0, r, dG, rows, D, n_row_chunks, partial, db_part);
         };
         if (r_dtype == MKA_BF16) launch(static_cast<const __nv_bfloat16*>(R));
         else launch(static_cast<const float*>(R));
     }
     const int blocks = (dW_r ? (D * 3 + 31) / 32 : 0) + (db_r ? 1 : 0);
-    if (blocks) router_bwd_reduce_kernel<<<blocks, 256, 0, st>>>(partial, dG, rows, D, n_row_chunks, db_part, dW_r, db_r);
-    return cudaGetLastError();
+    if (e != cudaSuccess || !blocks) return e;
+    return launch_chained(router_bwd_reduce_kernel, dim3(blocks), dim3(256), 0, st, 0, partial, dG, rows, D, n_row_chunks, db_part, dW_r, db_r);
 }
 
 }  // namespace mka
