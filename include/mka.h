@@ -159,7 +159,15 @@ size_t mka_workspace_bytes(const mka_shape* shape, const int64_t n_level[3], int
  *        not written in MKA_MODE_FULL
  * bf16 with d in {64,128} runs the TMA + tcgen05 kernel; f32, MKA_MODE_FULL and MKA_FLAG_FORCE_SIMT
  * run the CUDA-core kernel.
+ *
+ * mka_fwd_with_scratch: the same with room for partial results, `scratch_bytes` at `scratch` (device, 16-byte aligned;
+ * NULL and 0: none).  Where few blocks of query rows would leave SMs idle, the forward then cuts their key lists evenly
+ * over all SMs; mka_fwd_scratch_bytes says how much room that takes for a shape (H_kv as in mka_fwd_paged, 0: the shape's own;
+ * result 0: the call has no use for scratch; with less it runs as mka_fwd does).  The scratch is used between the call's kernels only.
  */
+size_t mka_fwd_scratch_bytes(const mka_shape* shape, int32_t H_kv, const int64_t n_level[3]);
+mka_status mka_fwd_with_scratch(const mka_shape* shape, const void* Q, const mka_level L[3], const float* gate,
+                                void* O, float* LSE, void* ws, size_t ws_bytes, void* scratch, size_t scratch_bytes, void* stream);
 mka_status mka_fwd(const mka_shape* shape, const void* Q, const mka_level L[3], const float* gate,
                    void* O, float* LSE, void* ws, size_t ws_bytes, void* stream);
 
@@ -220,7 +228,11 @@ mka_status mka_decode_paged(const mka_shape* shape, int32_t H_kv, const void* q,
  * the product reads them.  Pages with no valid row are never read.
  * bf16, MKA_MODE_FAST, d in {64, 128} only (the TMA + tcgen05 kernel; a 128-row key tile is assembled from one box
  * per page); anything else returns MKA_ERR_UNSUPPORTED.  ws: at least 256 bytes (status word).
+ * mka_fwd_paged_with_scratch: as mka_fwd_with_scratch (levels with a row count per sequence have no use for scratch).
  */
+mka_status mka_fwd_paged_with_scratch(const mka_shape* shape, int32_t H_kv, const void* Q, const mka_paged_level L[3],
+                                      const float* gate, void* O, float* LSE, void* ws, size_t ws_bytes, void* scratch,
+                                      size_t scratch_bytes, void* stream);
 mka_status mka_fwd_paged(const mka_shape* shape, int32_t H_kv, const void* Q, const mka_paged_level L[3],
                          const float* gate, void* O, float* LSE, void* ws, size_t ws_bytes, void* stream);
 

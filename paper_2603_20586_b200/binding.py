@@ -28,7 +28,8 @@ TILE = 128
 EXPORTS = ["mka_status_str", "mka_router", "mka_workspace_bytes", "mka_fwd", "mka_decode", "mka_bwd",
            "mka_decode_plan", "mka_fwd_tile_range", "mka_device_status", "mka_fwd_kernel_kind",
            "mka_bwd_kernel_kind", "mka_fuse_kv", "mka_l2_summary", "mka_l2_summary_workspace_bytes", "mka_l2_summary_kernel_kind", "mka_decode_static", "mka_decode_static_max_bytes",
-           "mka_decode_paged", "mka_decode_paged_workspace_bytes", "mka_l3_index", "mka_l3_retrieve", "mka_fwd_paged", "mka_fuse_kv_paged", "mka_set_wait_limit_us"]
+           "mka_decode_paged", "mka_decode_paged_workspace_bytes", "mka_l3_index", "mka_l3_retrieve", "mka_fwd_paged", "mka_fuse_kv_paged", "mka_set_wait_limit_us",
+           "mka_fwd_scratch_bytes", "mka_fwd_with_scratch", "mka_fwd_paged_with_scratch"]
 
 
 class MkaError(RuntimeError):
@@ -83,6 +84,9 @@ def _load() -> ctypes.CDLL:
     lib.mka_router.argtypes = [vp, vp, vp, i64, i32, i32, i32, vp, vp, vp, vp]
     lib.mka_fwd.argtypes = [ctypes.POINTER(mka_shape), vp, vp, vp, vp, vp, vp, ctypes.c_size_t, vp]
     lib.mka_decode.argtypes = lib.mka_fwd.argtypes
+    lib.mka_fwd_scratch_bytes.restype = ctypes.c_size_t
+    lib.mka_fwd_scratch_bytes.argtypes = [ctypes.POINTER(mka_shape), i32, ctypes.POINTER(ctypes.c_int64)]
+    lib.mka_fwd_with_scratch.argtypes = [ctypes.POINTER(mka_shape), vp, vp, vp, vp, vp, vp, ctypes.c_size_t, vp, ctypes.c_size_t, vp]
     lib.mka_bwd.argtypes = [ctypes.POINTER(mka_shape), vp, vp, vp, vp, vp, vp, vp, i32, vp,
                             ctypes.POINTER(mka_level_grad), vp, vp, vp, vp, ctypes.c_size_t, vp]
     lib.mka_decode_plan.argtypes = [ctypes.POINTER(ctypes.c_int64), i32, i32, i32, ctypes.POINTER(mka_decode_plan_t)]
@@ -101,6 +105,7 @@ def _load() -> ctypes.CDLL:
     lib.mka_decode_paged.argtypes = [ctypes.POINTER(mka_shape), i32, vp, vp, vp, vp, vp, vp,
                                      ctypes.c_size_t, vp]
     lib.mka_fwd_paged.argtypes = lib.mka_decode_paged.argtypes
+    lib.mka_fwd_paged_with_scratch.argtypes = [ctypes.POINTER(mka_shape), i32, vp, vp, vp, vp, vp, vp, ctypes.c_size_t, vp, ctypes.c_size_t, vp]
     lib.mka_fuse_kv_paged.argtypes = [i32, i32, i64, i32, i32, vp, vp, ctypes.POINTER(mka_paged_level), i64,
                                       vp, vp]
     lib.mka_l3_index.argtypes = [vp, i64, i32, i32, i32, i64, i64, i64, vp, i32, vp, vp]
@@ -111,7 +116,7 @@ def _load() -> ctypes.CDLL:
     lib.mka_set_wait_limit_us.argtypes = [ctypes.c_uint32]
     for name in EXPORTS:
         if name not in ("mka_status_str", "mka_workspace_bytes", "mka_decode_static_max_bytes", "mka_l2_summary_workspace_bytes",
-                        "mka_decode_paged_workspace_bytes", "mka_set_wait_limit_us"):
+                        "mka_decode_paged_workspace_bytes", "mka_set_wait_limit_us", "mka_fwd_scratch_bytes"):
             getattr(lib, name).restype = ctypes.c_int
     lib.mka_set_wait_limit_us.restype = ctypes.c_uint32
     return lib
@@ -157,6 +162,7 @@ def make_shape(B, H, T, d, D=0, window=1, q_offset=0, scale=0.0, dtype=MKA_BF16,
     return mka_shape(B, H, T, d, D, window, q_offset, scale, dtype, mode, flags, kv_heads)
 
 
+_Rows = ctypes.c_int64 * 3
 _LevelWords = ctypes.c_int64 * 18        # mka_level[3]: k, v, n, stride_b, stride_h, stride_n
 _PagedWords = ctypes.c_int64 * 36        # mka_paged_level[3]: twelve 8-byte slots each (page_rows is the low half of its own)
 _NO_LEVEL = (0,) * 6
@@ -212,16 +218,30 @@ def alloc_workspace(shape: mka_shape, n_level, which: int, device) -> torch.Tens
     return torch.empty(mka_workspace_bytes(shape, n_level, which), dtype=torch.uint8, device=device)
 
 
+def _fwd_scratch(shape: mka_shape, H_kv: int, n_level, device) -> Optional[torch.Tensor]:
+    """Room for the forward's partial results, from the caller's stream like its outputs, or None where it has no use for any."""
+    q_tiles = shape.B * shape.H * ((shape.T + 127) // 128)
+    if q_tiles > 4 * 148 * 2 or q_tiles * sum(n_level) < 148 * 4 * 128:      # many blocks, or little to share out: not worth the question
+        return None
+    nbytes = lib.mka_fwd_scratch_bytes(shape, H_kv, n_level)
+    try:
+        return torch.empty(nbytes, dtype=torch.uint8, device=device) if nbytes else None
+    except torch.OutOfMemoryError:                                           # the call runs without, as it would have
+        return None
+
+
 def mka_fwd(shape: mka_shape, Q, K, V, gate, O=None, LSE=None, ws=None, stream=None, want_lse=True):
     assert Q.is_contiguous() and gate.is_contiguous() and gate.dtype == torch.float32
     if O is None:
         O = torch.empty_like(Q)
     if LSE is None and want_lse and shape.mode == MKA_MODE_FAST:
         LSE = torch.empty(Q.shape[:3], dtype=torch.float32, device=Q.device)
+    n = [0 if k is None else k.shape[2] for k in K]
     if ws is None:
-        ws = alloc_workspace(shape, [0 if k is None else k.shape[2] for k in K], MKA_WS_FWD, Q.device)
-    _check(lib.mka_fwd(ctypes.byref(shape), _ptr(Q), _levels(K, V), _ptr(gate), _ptr(O), _ptr(LSE), _ptr(ws),
-                       ws.numel(), _stream(stream)), "mka_fwd")
+        ws = alloc_workspace(shape, n, MKA_WS_FWD, Q.device)
+    tmp = _fwd_scratch(shape, 0, _Rows(*n), Q.device) if stream is None else None
+    _check(lib.mka_fwd_with_scratch(ctypes.byref(shape), _ptr(Q), _levels(K, V), _ptr(gate), _ptr(O), _ptr(LSE), _ptr(ws), ws.numel(),
+                                    _ptr(tmp), 0 if tmp is None else tmp.numel(), _stream(stream)), "mka_fwd")
     return O, LSE
 
 
@@ -288,8 +308,10 @@ def mka_fwd_paged(shape: mka_shape, H_kv: int, Q, pools_k, pools_v, tables, n, g
         LSE = torch.empty(B, H, T, dtype=torch.float32, device=Q.device)
     if ws is None:
         ws = torch.zeros(256, dtype=torch.uint8, device=Q.device)
-    _check(lib.mka_fwd_paged(ctypes.byref(shape), H_kv, _ptr(Q), _paged_levels(pools_k, pools_v, tables, rows, n), _ptr(gate),
-                             _ptr(O), _ptr(LSE), _ptr(ws), ws.numel(), _stream(stream)), "mka_fwd_paged")
+    tmp = _fwd_scratch(shape, H_kv, _n_level(n), Q.device) if stream is None and (rows is None or not any(r is not None for r in rows)) else None
+    _check(lib.mka_fwd_paged_with_scratch(ctypes.byref(shape), H_kv, _ptr(Q), _paged_levels(pools_k, pools_v, tables, rows, n), _ptr(gate),
+                                          _ptr(O), _ptr(LSE), _ptr(ws), ws.numel(), _ptr(tmp), 0 if tmp is None else tmp.numel(),
+                                          _stream(stream)), "mka_fwd_paged")
     return O, LSE
 
 

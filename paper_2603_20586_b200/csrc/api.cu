@@ -185,8 +185,27 @@ mka_status mka_router(const void* R, const float* W_r, const float* b_r, int64_t
     return e == cudaSuccess ? MKA_OK : MKA_ERR_CUDA;
 }
 
+size_t mka_fwd_scratch_bytes(const mka_shape* s, int32_t H_kv, const int64_t n_level[3]) {
+    if (check_shape(s, false) != MKA_OK || !n_level || H_kv < 0 || (H_kv > 0 && s->H % H_kv)) return 0;
+    if (s->dtype != MKA_BF16 || s->mode != MKA_MODE_FAST || (s->d != 64 && s->d != 128) || (s->flags & MKA_FLAG_FORCE_SIMT)) return 0;
+    FwdParams p;
+    memset(&p, 0, sizeof(p));
+    for (int l = 0; l < 3; ++l) {
+        if (n_level[l] < 0 || n_level[l] > 0x7fffffffLL) return 0;
+        p.L[l].n = n_level[l];
+    }
+    p.B = s->B; p.H = s->H; p.T = s->T; p.d = s->d; p.window = s->window; p.q_offset = s->q_offset;
+    p.kv_group = H_kv > 0 && s->H > 0 ? s->H / H_kv : kv_group_of(s);
+    return fwd_tc_scratch_bytes(p);
+}
+
 mka_status mka_fwd(const mka_shape* s, const void* Q, const mka_level L[3], const float* gate, void* O, float* LSE,
                    void* ws, size_t ws_bytes, void* stream) {
+    return mka_fwd_with_scratch(s, Q, L, gate, O, LSE, ws, ws_bytes, nullptr, 0, stream);
+}
+
+mka_status mka_fwd_with_scratch(const mka_shape* s, const void* Q, const mka_level L[3], const float* gate, void* O, float* LSE,
+                                void* ws, size_t ws_bytes, void* scratch, size_t scratch_bytes, void* stream) {
     mka_status st = check_shape(s, false);
     if (st != MKA_OK) return st;
     if ((st = check_levels(s, L)) != MKA_OK) return st;
@@ -201,6 +220,7 @@ mka_status mka_fwd(const mka_shape* s, const void* Q, const mka_level L[3], cons
     p.B = s->B; p.H = s->H; p.T = s->T; p.d = s->d;
     p.window = s->window; p.q_offset = s->q_offset; p.scale = resolve_scale(s);
     p.mode = s->mode; p.decode = 0; p.kv_group = kv_group_of(s);
+    p.scratch = scratch; p.scratch_bytes = scratch_bytes;
     p.test_stall = (s->flags & MKA_FLAG_TEST_STALL) ? 1 : 0;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     p.status = static_cast<unsigned int*>(ws);
@@ -345,6 +365,12 @@ static mka_status run_decode_paged(DecodePagedParams& p, DecodeParams& c, const 
 
 mka_status mka_fwd_paged(const mka_shape* s, int32_t H_kv, const void* Q, const mka_paged_level L[3], const float* gate,
                          void* O, float* LSE, void* ws, size_t ws_bytes, void* stream) {
+    return mka_fwd_paged_with_scratch(s, H_kv, Q, L, gate, O, LSE, ws, ws_bytes, nullptr, 0, stream);
+}
+
+mka_status mka_fwd_paged_with_scratch(const mka_shape* s, int32_t H_kv, const void* Q, const mka_paged_level L[3], const float* gate,
+                                      void* O, float* LSE, void* ws, size_t ws_bytes, void* scratch, size_t scratch_bytes,
+                                      void* stream) {
     mka_status st = check_shape(s, false);
     if (st != MKA_OK) return st;
     if (s->dtype != MKA_BF16 || s->mode != MKA_MODE_FAST || (s->flags & MKA_FLAG_FORCE_SIMT)) return MKA_ERR_UNSUPPORTED;
@@ -385,6 +411,7 @@ mka_status mka_fwd_paged(const mka_shape* s, int32_t H_kv, const void* Q, const 
     p.B = s->B; p.H = s->H; p.T = s->T; p.d = s->d;
     p.window = s->window; p.q_offset = s->q_offset; p.scale = resolve_scale(s);
     p.mode = s->mode; p.decode = 0; p.kv_group = s->H / H_kv; p.paged = P;
+    p.scratch = scratch; p.scratch_bytes = scratch_bytes;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     cudaError_t e = launch_fwd_tc(p, static_cast<unsigned int*>(ws), cs);
     if (e == cudaErrorNotSupported) return MKA_ERR_UNSUPPORTED;

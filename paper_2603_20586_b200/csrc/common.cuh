@@ -70,6 +70,8 @@ struct FwdParams {
     int kv_group;       // query heads per KV head (>= 1): head h reads KV head h / kv_group
     int test_stall;     // MKA_FLAG_TEST_STALL (tensor-core forward, dense levels)
     unsigned int* status;   // device status word; the CUDA-core kernel, which waits for nothing, writes MKA_OK itself
+    void* scratch;          // room for partial results (tensor-core forward), or null
+    size_t scratch_bytes;
     const PagedLevelDev* paged;   // host array of 3, or null: the levels are page pools (tensor-core forward only; L[l].n still holds the rows)
 };
 
@@ -205,5 +207,6 @@ bool bwd_tc_eligible(const BwdParams& p, int dtype);
 // Tensor-core (TMA + tcgen05) forward; returns cudaErrorNotSupported when the shape is not eligible.
 cudaError_t launch_fwd_tc(const FwdParams& p, unsigned int* status_word, cudaStream_t st);
 bool fwd_tc_eligible(const FwdParams& p, int dtype);
+size_t fwd_tc_scratch_bytes(const FwdParams& p);      // scratch with which the call would run faster, 0: none
 
 }  // namespace mka

@@ -1,16 +1,14 @@
 // Tensor-core forward of Eq. 5 for bf16 on sm_100a: TMA -> shared memory -> tcgen05.mma -> TMEM.
 //
-// A CTA owns 128-row query tiles of one (batch, head) -- two of them ("ping" and "pong", 256 rows) at d = 128, one at
-// d = 64, where two CTAs share an SM -- and walks ONE level-ordered list of 128-row key tiles: all visible L1 tiles,
-// then L2, then L3.  A single running (max, sum) per row spans the three levels (the max shift of Eq. 11-14); the gate
-// enters as a per-row, per-level additive bias log2(lambda) inside the exponent, so that
+// A CTA works on a block: 128-row query tiles -- two of them ("ping" and "pong": 256 rows of a head, or 128 rows of two heads of
+// a group) at d = 128, one at d = 64, where two CTAs share an SM -- and ONE level-ordered list of 128-row key tiles: all
+// visible L1 tiles, then L2, then L3.  A single running (max, sum) per row spans the three levels (the max shift of
+// Eq. 11-14); the gate enters as a per-row, per-level additive bias log2(lambda) inside the exponent, so that
 //     p = 2^(s * tau * log2(e) + log2(lambda_l) - m)  =  lambda_l * exp(s*tau - m')
 // which is exactly the gated, un-normalised weight of Eq. 5.  One normalisation at the end.
 //
-// Warp roles (384 threads):
-//   softmax warps    thread = one query row (TMEM lane) x 128 key columns at d = 128 (four warps per query tile), x 64
-//                    columns at d = 64 (eight warps: warp = (column half, lane quarter); the two threads of a row agree
-//                    on the row maximum through shared memory and a 256-thread barrier).  Reads S from TMEM, applies
+// Warp roles (d = 128: 384 threads, d = 64: 256):
+//   softmax warps    four per query tile, thread = one query row (TMEM lane) x 128 key columns.  Reads S from TMEM, applies
 //                    bias and masks, running max, exp2, packs the weights to bf16 and writes them to TMEM in parts of
 //                    32 keys (at d = 128 over the columns S occupied), rescales the O accumulator when the running
 //                    maximum grows by more than 2^8 (lazy rescale), and does the epilogue.
@@ -22,8 +20,9 @@
 //                    memory, N-major) in pieces that follow the parts of P, so that most of the product runs under the
 //                    remaining exponentials.  At d = 128 the order is  S0(e)  O1(e-1)  S1(e)  O0(e):  each tile's
 //                    softmax overlaps the other tile's products.
-//   last two warps   idle: they complete the last warpgroup, so that registers can be moved from it to the softmax
-//                    warpgroups (setmaxnreg): a launch leaves 168 (d = 64, two CTAs per SM: 80) registers per thread.
+//   next warp        deals: works out the CTA's items (blocks, or pieces of their tile lists).
+//   last warp        idle: it completes the last warpgroup, so that registers can be moved from it to the softmax
+//                    warpgroups (setmaxnreg): a launch leaves 168 (d = 64, two CTAs per SM: 128) registers per thread.
 // TMEM: S tiles first (128 columns each), then the O accumulators (d columns each); at d = 64 a P region of 64 columns
 // per query tile follows, and S_q(e+1) is multiplied while the softmax of S_q(e) runs (the hand-off is "S is in
 // registers", not "P has been consumed").  d = 128 uses all 512 columns, d = 64 256.
@@ -69,33 +68,39 @@ struct TcParams {
     long long table_stride[3], table_head_stride[3];
     int page_shift[3], box_rows[3], pool_pages[3];
     const int* rows[3];      // per-sequence rows of a level (clamped to [0, n]), or null
-    int deal;                // (batch, head) pairs per group of blocks dealt by query block (1 = pair by pair)
+    int deal;                // lines per group of blocks dealt by query block (1 = line by line)
+    // A block = query tiles that walk one key-tile list.  d = 64: one tile.  d = 128: two, either 256 consecutive rows of one head, or
+    // (pair_heads) the same 128 rows of two heads that share a KV head.  A "line" = what the blocks of one column of rows belong
+    // to: a (batch, head), or a (batch, pair of heads).
+    int pair_heads;
+    int block_rows;          // rows that a block moves down by: 128 or 256
+    int lines, q_blocks;     // lines, and blocks of one
+    int line_units;          // kStream: units of one line
+    int range, longer;       // kStream: units of a CTA's range; the first `longer` CTAs have one more
+    float* slots;            // kStream: two partial results per CTA
 };
 
 template <int DH>
 struct Cfg {
-    // d = 128: one CTA per SM with two query tiles (all 512 TMEM columns); a softmax thread owns a whole query row
-    // (128 key columns).
-    // d = 64: the scores of one key tile cost the special-function unit as much as at d = 128 but only half the
+    // A softmax thread owns a whole query row (128 key columns).  d = 128: one CTA per SM with two query tiles (all 512 TMEM
+    // columns).  d = 64: the scores of one key tile cost the special-function unit as much as at d = 128 but only half the
     // tensor work, and the tile lists of the training shapes are short; there a CTA takes ONE query tile (256 TMEM
-    // columns) and two CTAs share the SM, so that one CTA's start-up, waits and epilogue run under the other's steady
-    // state.  Two CTAs leave 80 registers per thread, so a row is split between two threads (64 columns each), and
-    // registers are moved from the last warpgroup to the softmax warpgroups.
+    // columns) and two CTAs share the SM, so that one CTA's waits and epilogue run under the other's steady state.  With
+    // two threads to a row (64 columns each, sixteen softmax warps on the SM) the exchange of the row maximum put a barrier of
+    // all eight warps into every tile: [8, 16, 2048, 64] (window 512, 1024 slots) took 288 us against 258.
     static constexpr int kNumQ = DH == 128 ? 2 : 1;
     static constexpr int kCtasPerSm = DH == 128 ? 1 : 2;
-    static constexpr int kSplit = DH == 128 ? 1 : 2;           // threads per query row
-    static constexpr int kCols = kTileN / kSplit;             // key columns of one softmax thread
-    static constexpr int kMergeCols = DH == 128 ? 16 : 8;      // columns of a row that a thread merges at a time (kSplitKeys)
-    static constexpr int kParts = kCols / 32;                 // the weights of a tile are handed over in parts of 32 keys per thread
-    static constexpr int kRowWarps = 4 * kSplit;              // softmax warps per query tile
+    static constexpr int kMergeCols = DH == 128 ? 16 : 8;      // columns of a row that a thread merges at a time (kCluster)
+    static constexpr int kParts = kTileN / 32;                // the weights of a tile are handed over in parts of 32 keys
+    static constexpr int kRowWarps = 4;                       // softmax warps per query tile
     static constexpr int kSoftmaxWarps = kRowWarps * kNumQ;
-    // The registers are re-divided between the warpgroups (setmaxnreg, a warpgroup-wide instruction: two idle warps
-    // complete the last one).  At d = 128 a thread's 128 scores need more than the 168 registers that a launch gives.
+    // The registers are re-divided between the warpgroups (setmaxnreg, a warpgroup-wide instruction: an idle warp
+    // completes the last one).  A thread's 128 scores need more than the 168 (d = 64: 128) registers that a launch gives.
     static constexpr int kThreads = (kSoftmaxWarps + 4) * 32;
-    static constexpr int kProducerWarp = kSoftmaxWarps, kMmaWarp = kSoftmaxWarps + 1;
+    static constexpr int kProducerWarp = kSoftmaxWarps, kMmaWarp = kSoftmaxWarps + 1, kDealWarp = kSoftmaxWarps + 2;
     // What the warpgroups hold after the move must not exceed what the launch gave the CTA, or the increase would
-    // wait forever:  d = 128: 384 threads x 168 registers at launch = 256 x 216 + 128 x 72;  d = 64: 384 x 80 = 256 x 104 + 128 x 32.
-    static constexpr int kRegsLaunch = DH == 128 ? 168 : 80, kRegsSoftmax = DH == 128 ? 216 : 104, kRegsOther = DH == 128 ? 72 : 32;
+    // wait forever:  d = 128: 384 threads x 168 registers at launch = 256 x 216 + 128 x 72;  d = 64: 256 x 128 = 128 x 200 + 128 x 56.
+    static constexpr int kRegsLaunch = DH == 128 ? 168 : 128, kRegsSoftmax = DH == 128 ? 216 : 200, kRegsOther = DH == 128 ? 72 : 56;
     static_assert(kSoftmaxWarps * 32 * kRegsSoftmax + 4 * 32 * kRegsOther <= kThreads * kRegsLaunch, "register pool of the CTA exceeded");
     static_assert(kThreads * kCtasPerSm * (kRegsLaunch + 8) > 65536, "the launch would get more than kRegsLaunch registers per thread");
     static constexpr int kPanels = DH / 64;
@@ -111,6 +116,7 @@ struct Cfg {
     static constexpr uint32_t kTmemCols = DH == 128 ? 512u : 256u;
     static_assert(kColP + (kSeparateP ? kNumQ * (kTileN / 2) : 0) <= kTmemCols, "TMEM columns exceeded");
     static constexpr uint32_t kIdescPV = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(DH >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
+    static constexpr int kSlotFloats = kNumQ * kTileM * (DH + 2);   // a partial result of a block: O as [columns / 4][rows][4], then (max, sum) of every row
 };
 
 constexpr int kMaxQ = 2;
@@ -120,8 +126,18 @@ constexpr int kMaxSplit = 8;              // CTAs of a cluster (the portable lim
 struct Barriers {
     uint64_t q_full;
     uint64_t k_full[4], k_empty[4], v_full[4], v_empty[4];
-    uint64_t s_full[kMaxQ], p_part[kMaxQ][4], pv_done[kMaxQ];   // p_part: the first / second 32 keys of both column halves are written
+    uint64_t s_full[kMaxQ], p_part[kMaxQ][4], pv_done[kMaxQ];   // p_part: that part of 32 keys is written
     uint64_t s_free[kMaxQ];   // d = 64 only: the warpgroup has read S(e) into registers, S(e+1) may overwrite it
+    uint64_t q_empty;         // the item's Q tiles have had their last reader
+    uint64_t item_full[2], item_free[2];
+};
+
+// A block of query rows, or a part of its key-tile list, with the rows of the levels it sees.
+struct Item {
+    int b, kvh, E;            // E: key tiles; -1: there is no further item
+    int slot;                 // where the partial result goes; -1: the item is a whole block
+    int h[kMaxQ], m[kMaxQ];   // head and first row of each query tile
+    int first[3], end[3], n[3];
 };
 
 // Key-tile range [first, end) of a block of query rows [r0, r1] (inclusive) on one level.
@@ -136,10 +152,92 @@ __host__ __device__ __forceinline__ void tile_range(int level, long long r0, lon
     end = (int)((hi + kTileN - 1) / kTileN);
 }
 
-// kSplitKeys: the CTAs of a cluster share one block of query rows and split its key-tile list between them (see split_rule).
-// Each ends with its own un-normalised O and (max, sum); they meet in distributed shared memory, so no scratch memory
-// and no second launch is needed.
-template <int DH, bool kPaged, bool kSplitKeys>
+// N (a multiple of 8) consecutive columns of one row as bf16.
+template <int N>
+__device__ __forceinline__ void store_cols_bf16(__nv_bfloat16* out, const float (&x)[N]) {
+#pragma unroll
+    for (int c = 0; c < N; c += 8) {
+        uint4 v;
+        v.x = pack_bf16(x[c], x[c + 1]); v.y = pack_bf16(x[c + 2], x[c + 3]);
+        v.z = pack_bf16(x[c + 4], x[c + 5]); v.w = pack_bf16(x[c + 6], x[c + 7]);
+        *reinterpret_cast<uint4*>(out + c) = v;
+    }
+}
+
+// How the work is dealt to the CTAs:
+//   kWhole    a CTA takes one block of query rows.
+//   kCluster  the CTAs of a cluster share one block and split its key-tile list between them (see form_rule).  Each ends with its
+//             own un-normalised O and (max, sum); they meet in distributed shared memory, so no scratch memory is needed.
+//   kStream   the key tiles of all blocks, laid end to end, are cut into equal ranges, one per resident CTA.  A CTA works off the pieces of
+//             blocks in its range one after the other: the next piece's copies and first products run under the epilogue of
+//             the one before.  Pieces of cut blocks go to scratch memory and fwd_merge_kernel adds them up.
+enum { kWhole = 0, kCluster = 1, kStream = 2 };
+constexpr int kStreamRounds = 4;    // kStream is looked at up to this many rounds of resident CTAs
+constexpr int kBlockUnits = 2;      // kStream: a block counts as its key tiles and this many more (its epilogue)
+
+// Units of block `qb` of every line.
+__host__ __device__ __forceinline__ int block_units(int qb, int rows, int T, int q_offset, int window, const long long (&n)[3]) {
+    const long long r0 = (long long)qb * rows, r1 = r0 + rows - 1;
+    int units = kBlockUnits;
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+        int first = 0, end = 0;
+        if (n[l] > 0) tile_range(l, r0, r1 < T - 1 ? r1 : T - 1, q_offset, window, n[l], first, end);
+        units += end - first;
+    }
+    return units;
+}
+
+// Heads and first rows of the query tiles of block qb of a line.  A tile without a partner head starts past the last row.
+template <int DH>
+__device__ __forceinline__ void block_tiles_of(const TcParams& p, int line, int qb, int& b, int& kvh, int (&h)[kMaxQ], int (&m)[kMaxQ]) {
+    const int H_kv = p.H / p.kv_group;
+    if (DH == 128 && p.pair_heads) {
+        const int per = (p.kv_group + 1) / 2, bk = line / per, j = 2 * (line - bk * per);
+        b = bk / H_kv; kvh = bk - b * H_kv;
+        h[0] = kvh * p.kv_group + j;
+        m[0] = qb * kTileM;
+        h[1] = j + 1 < p.kv_group ? h[0] + 1 : h[0];
+        m[1] = j + 1 < p.kv_group ? m[0] : p.T;
+        return;
+    }
+    b = line / p.H;
+    h[0] = h[1] = line - b * p.H;
+    kvh = h[0] / p.kv_group;
+    m[0] = qb * Cfg<DH>::kNumQ * kTileM;
+    m[1] = m[0] + kTileM;
+}
+
+// kStream: first unit of CTA i's range, and the CTA whose range holds unit u.
+__device__ __forceinline__ int range_start(const TcParams& p, int i) { return i * p.range + min(i, p.longer); }
+__device__ __forceinline__ int range_of(const TcParams& p, int u) {
+    const int head = p.longer * (p.range + 1);
+    return u < head ? u / (p.range + 1) : p.longer + (u - head) / p.range;
+}
+
+// Block that holds unit u of a line, and its first unit.  Called by a whole warp.
+__device__ __forceinline__ void find_block(const TcParams& p, int u, int lane, int& qb, int& unit0) {
+    int before = 0;
+    for (int q0 = 0;; q0 += 32) {
+        const int own = q0 + lane < p.q_blocks ? block_units(q0 + lane, p.block_rows, p.T, p.q_offset, p.window, p.n) : 0;
+        int sum = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, sum, o);
+            if (lane >= o) sum += x;
+        }
+        const unsigned int past = __ballot_sync(0xffffffffu, before + sum > u);
+        if (past || q0 + 32 >= p.q_blocks) {
+            const int i = past ? __ffs(past) - 1 : min(31, p.q_blocks - 1 - q0);
+            qb = q0 + i;
+            unit0 = before + __shfl_sync(0xffffffffu, sum - own, i);
+            return;
+        }
+        before += __shfl_sync(0xffffffffu, sum, 31);
+    }
+}
+
+template <int DH, bool kPaged, int kForm>
 __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc_kernel(const __grid_constant__ TcMaps maps, const TcParams p) {
     using C = Cfg<DH>;
     extern __shared__ uint8_t smem_raw[];
@@ -150,30 +248,68 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
     __shared__ Barriers bar;
     __shared__ uint32_t tmem_base_slot;
     __shared__ WaitCtl wait_ctl;
-    __shared__ float xmax[2][C::kNumQ][C::kSplit][kTileM];           // row maxima of the two column halves, double-buffered by tile parity
-    __shared__ float lsum[C::kNumQ][C::kSplit][kTileM];              // row sums of the two column halves (epilogue)
-    __shared__ float cl_max[kSplitKeys ? C::kNumQ : 1][kTileM], cl_sum[kSplitKeys ? C::kNumQ : 1][kTileM];   // this CTA's (max, sum) of every row, for its cluster
+    __shared__ Item items[2];
+    __shared__ float cl_max[kForm == kCluster ? C::kNumQ : 1][kTileM], cl_sum[kForm == kCluster ? C::kNumQ : 1][kTileM];   // this CTA's (max, sum) of every row, for its cluster
 
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // tid >> 5, but provably warp-uniform for the compiler
-    // Blocks start in the order of their linear index.  Within a group of p.deal (batch, head) pairs the blocks are
-    // dealt by query block, heaviest (latest rows) first for every pair of the group, then the next lighter one: the
-    // launch then ends with the group's lightest blocks instead of the last head's heaviest.
     int crank = 0, csize = 1;                                 // this CTA's place in its cluster
-    if constexpr (kSplitKeys) {
+    if constexpr (kForm == kCluster) {
         asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
         asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(csize));
     }
-    const int grid_x = (int)gridDim.x / csize;                // blocks of query rows
-    const int lin = (int)blockIdx.x / csize + grid_x * (blockIdx.y + gridDim.y * blockIdx.z);      // fewer than 2^31 blocks
-    const int per_group = p.deal * grid_x;
-    const int grp = lin / per_group, in_grp = lin - grp * per_group;
-    const int pairs_here = min(p.deal, (int)(gridDim.y * gridDim.z) - grp * p.deal);
-    const int hb = grp * p.deal + in_grp % pairs_here;
-    const int b = hb / (int)gridDim.y, h = hb - b * (int)gridDim.y;
-    const int qpair = grid_x - 1 - in_grp / pairs_here;
-    const long long m0 = (long long)qpair * (C::kNumQ * kTileM);
-    const long long m_last = (m0 + C::kNumQ * kTileM - 1 < p.T - 1) ? m0 + C::kNumQ * kTileM - 1 : p.T - 1;
+    // The whole block `qb` of a line.
+    auto block_of = [&](int line, int qb, Item& it) {
+        block_tiles_of<DH>(p, line, qb, it.b, it.kvh, it.h, it.m);
+        it.slot = -1; it.E = 0;
+        const long long m_last = min((long long)it.m[0] + p.block_rows - 1, (long long)p.T - 1);
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+            long long n = p.n[l];
+            if (kPaged && p.rows[l]) {                        // rows of the level for this sequence
+                const long long r = p.rows[l][it.b];
+                n = r < 0 ? 0 : (r < n ? r : n);
+            }
+            it.n[l] = (int)n;
+            if (n > 0) tile_range(l, it.m[0], m_last, p.q_offset, p.window, n, it.first[l], it.end[l]);
+            else it.first[l] = it.end[l] = 0;
+            it.E += it.end[l] - it.first[l];
+        }
+    };
+    // Tiles [t0, t1) of the level-ordered list.
+    auto cut = [&](Item& it, int t0, int t1) {
+        int base = 0;
+        it.E = 0;
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+            const int cnt = it.end[l] - it.first[l];
+            const int a = min(max(t0 - base, 0), cnt), z = min(max(t1 - base, 0), cnt);
+            it.end[l] = it.first[l] + z;
+            it.first[l] += a;
+            it.E += z - a;
+            base += cnt;
+        }
+    };
+    // kStream: the next piece of this CTA's range [u, u1) that holds tiles (or the start of a block without tiles).
+    int u = 0, u1 = 0, unit0 = 0;                             // unit0: first unit of block (line, qb)  (fewer than 2^30 units)
+    int line = 0, qb = 0;
+    auto next_piece = [&](Item& it) {
+        while (u < u1) {
+            block_of(line, qb, it);
+            const int E = it.E;
+            const int t0 = u - unit0, t1 = min(E, u1 - unit0);
+            u = unit0 + E + kBlockUnits;
+            unit0 = u;
+            if (++qb == p.q_blocks) { qb = 0; ++line; }
+            if (E == 0 ? t0 > 0 : t0 >= t1) continue;         // nothing but the block's epilogue, which goes with its last tile
+            if (t0 > 0 || t1 < E) {
+                cut(it, t0, t1);
+                it.slot = 2 * (int)blockIdx.x + (t0 > 0 ? 0 : 1);
+            }
+            return;
+        }
+        it.E = -1;
+    };
 
     if (tid == 0) {
         wait_ctl.abort = 0;
@@ -188,9 +324,39 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
             for (int i = 0; i < 4; ++i) mbar_init(&bar.p_part[q][i], C::kRowWarps);   // one arrival per softmax warp
             mbar_init(&bar.s_free[q], C::kRowWarps);
         }
+        mbar_init(&bar.q_empty, 1);
+        for (int i = 0; i < 2; ++i) { mbar_init(&bar.item_full[i], 1); mbar_init(&bar.item_free[i], 2 + C::kSoftmaxWarps); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    chain_enter();
+    auto first_item = [&] {
+        Item it;
+        if constexpr (kForm == kStream) {
+            u = range_start(p, blockIdx.x); u1 = range_start(p, blockIdx.x + 1);
+            line = u / p.line_units;
+            int in_line;
+            find_block(p, u - line * p.line_units, lane, qb, in_line);
+            unit0 = line * p.line_units + in_line;
+            next_piece(it);
+        } else {
+            // Blocks start in the order of their linear index.  Within a group of p.deal lines the blocks are
+            // dealt by query block, heaviest (latest rows) first for every line of the group, then the next lighter one: the
+            // launch then ends with the group's lightest blocks instead of the last head's heaviest.
+            const int lin = (int)blockIdx.x / csize;          // fewer than 2^31 blocks
+            const int per_group = p.deal * p.q_blocks;
+            const int grp = lin / per_group, in_grp = lin - grp * per_group;
+            const int lines_here = min(p.deal, p.lines - grp * p.deal);
+            block_of(grp * p.deal + in_grp % lines_here, p.q_blocks - 1 - in_grp / lines_here, it);
+            if constexpr (kForm == kCluster) {                // this CTA's share of the list
+                const int total = it.E;
+                cut(it, (int)((long long)total * crank / csize), (int)((long long)total * (crank + 1) / csize));
+            }
+        }
+        if (lane == 0) items[0] = it;
+    };
+    chain_trigger();
+    if (kForm == kStream && warp == C::kDealWarp) first_item();              // (from the call's arguments alone)
+    chain_wait();
+    if (kForm != kStream && warp == C::kDealWarp) first_item();
     // The status word starts at OK.  CTAs start in the order of their numbers and none gives up before the wait limit (100 us at
     // least) has passed, so the first one clears it before any other can have something to report.
     if (tid == 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) atomicExch(p.status, (unsigned int)MKA_OK);
@@ -204,162 +370,119 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
     const uint32_t tmem = tmem_base_slot;
     volatile WaitCtl* abortp = &wait_ctl;
 
-    // rows of the three levels for this sequence
-    long long nl[3];
-#pragma unroll
-    for (int l = 0; l < 3; ++l) {
-        nl[l] = p.n[l];
-        if (kPaged && p.rows[l]) {
-            const long long r = p.rows[l][b];
-            nl[l] = r < 0 ? 0 : (r < p.n[l] ? r : p.n[l]);
+    // Item number i is in items[i & 1]: the first from the start, the others once the dealing warp has posted them.  A warp that
+    // is done with one says so.
+    auto has_item = [&](int i) -> bool {
+        if (i > 0) {
+            if (kForm != kStream || !mbar_wait_warp(&bar.item_full[i & 1], (uint32_t)((i - 1) >> 1) & 1u, abortp)) return false;
         }
-    }
-    // the CTA's level-ordered key-tile list (same closed form in every role)
-    int first[3], end[3];
-#pragma unroll
-    for (int l = 0; l < 3; ++l) {
-        if (nl[l] > 0) tile_range(l, m0, m_last, p.q_offset, p.window, nl[l], first[l], end[l]);
-        else first[l] = end[l] = 0;
-    }
-    if constexpr (kSplitKeys) {                               // this CTA's share of the list: tiles [g0, g1)
-        const int total = (end[0] - first[0]) + (end[1] - first[1]) + (end[2] - first[2]);
-        const int g0 = (int)((long long)total * crank / csize), g1 = (int)((long long)total * (crank + 1) / csize);
-        int base = 0;
-#pragma unroll
-        for (int l = 0; l < 3; ++l) {
-            const int cnt = end[l] - first[l];
-            const int a = min(max(g0 - base, 0), cnt), z = min(max(g1 - base, 0), cnt);
-            end[l] = first[l] + z;
-            first[l] += a;
-            base += cnt;
+        return items[i & 1].E >= 0;
+    };
+    auto done_item = [&](int i) {
+        if constexpr (kForm == kStream) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar.item_free[i & 1]);
         }
-    }
-    const int E = (end[0] - first[0]) + (end[1] - first[1]) + (end[2] - first[2]);
+    };
 
     if (warp >= C::kSoftmaxWarps) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::kRegsOther));
-    if (warp == C::kProducerWarp && kPaged) {
+    if (warp == C::kProducerWarp) {
+        // The warp waits converged.  Dense levels: one lane issues (inside an `if (lane == 0)` around the whole loop the
+        // kernel keeps its loop state in local memory: 1.63 us per key tile instead of 1.49 at d = 128).
         // Paged levels: the whole warp produces.  Lane i owns box i of every key tile (a box = the rows of one page
         // that fall into the tile): it looks its page up while the warp waits for the stage to drain and issues its
         // own copies, so a tile costs one table round trip (overlapped) and four warp-wide copy instructions.
-        if (lane == 0) {
-            mbar_expect_tx(&bar.q_full, C::kNumQ * C::kTileBytes);
-#pragma unroll
-            for (int q = 0; q < C::kNumQ; ++q)
-#pragma unroll
-                for (int pn = 0; pn < C::kPanels; ++pn)
-                    tma_load_4d(sQ + q * C::kTileBytes + pn * kPanelBytes, &maps.q, pn * 64, (int)(m0 + q * kTileM), h, b, &bar.q_full);
-        }
-        int issued = 0;
+        int issued = 0, it = 0;                               // key tiles and items
         bool ok = true;
-        const int kvh = h / p.kv_group;
-#pragma unroll 1
-        for (int l = 0; l < 3 && ok; ++l) {
-            const int kt_first = pick3(first, l), kt_end = pick3(end, l);
-            if (kt_first >= kt_end) continue;
-            const long long n_here = pick3(nl, l);
-            const int* tab = p.table[l] + (long long)b * p.table_stride[l] + (long long)kvh * p.table_head_stride[l];
-            const int rpb = p.box_rows[l];
-            const bool mine = lane < kTileN / rpb;
-            const int in_mask = (1 << p.page_shift[l]) - 1;
-            for (int kt = kt_first; kt < kt_end; ++kt) {
-                const int s = issued % C::kStages;
-                const uint32_t ph = (uint32_t)(issued / C::kStages) & 1u;
-                // a box past the level's last row is aimed past the pool, where the copy engine fills zeros as it does
-                // past a dense level's end
-                const long long row = (long long)kt * kTileN + lane * rpb;
-                int page = p.pool_pages[l];
-                if (mine && row < n_here) page = tab[row >> p.page_shift[l]];
-                const int in_row = (int)(row & in_mask);
-                if (!mbar_wait_warp(&bar.k_empty[s], ph ^ 1u, abortp)) { ok = false; break; }
-                if (lane == 0) mbar_expect_tx(&bar.k_full[s], C::kTileBytes);
-                __syncwarp();
-                if (mine) {
+        for (; ok && has_item(it); ++it) {
+            const Item& I = items[it & 1];
+            const int b = I.b, kvh = I.kvh;
+            if (it > 0 && !mbar_wait_warp(&bar.q_empty, (uint32_t)(it - 1) & 1u, abortp)) break;
+            if (lane == 0) {
+                mbar_expect_tx(&bar.q_full, C::kNumQ * C::kTileBytes);
+#pragma unroll
+                for (int q = 0; q < C::kNumQ; ++q)
 #pragma unroll
                     for (int pn = 0; pn < C::kPanels; ++pn)
-                        tma_load_4d(sK + s * C::kTileBytes + pn * kPanelBytes + lane * rpb * 128, &maps.k[l], pn * 64, in_row, kvh, page,
-                                    &bar.k_full[s]);
-                }
-                if (!mbar_wait_warp(&bar.v_empty[s], ph ^ 1u, abortp)) {           // gave up with this stage's K copies in flight
-                    mbar_drain(&bar.k_full[s], ph, abortp, gtimer());
-                    ok = false;
-                    break;
-                }
-                if (lane == 0) mbar_expect_tx(&bar.v_full[s], C::kTileBytes);
-                __syncwarp();
-                if (mine) {
-#pragma unroll
-                    for (int pn = 0; pn < C::kPanels; ++pn)
-                        tma_load_4d(sV + s * C::kTileBytes + pn * kPanelBytes + lane * rpb * 128, &maps.v[l], pn * 64, in_row, kvh, page,
-                                    &bar.v_full[s]);
-                }
-                ++issued;
+                        tma_load_4d(sQ + q * C::kTileBytes + pn * kPanelBytes, &maps.q, pn * 64, I.m[q], I.h[q], b, &bar.q_full);
             }
+            __syncwarp();
+            int left = I.E;
+#pragma unroll 1
+            for (int l = 0; l < 3 && ok; ++l) {
+                const int kt_first = I.first[l], kt_end = I.end[l];
+                if (kt_first >= kt_end) continue;
+                const long long n_here = I.n[l];
+                const int* tab = kPaged ? p.table[l] + (long long)b * p.table_stride[l] + (long long)kvh * p.table_head_stride[l] : nullptr;
+                const int rpb = kPaged ? p.box_rows[l] : kTileN;
+                const bool mine = lane < kTileN / rpb;
+                const int in_mask = kPaged ? (1 << p.page_shift[l]) - 1 : 0;
+                for (int kt = kt_first; kt < kt_end; ++kt) {
+                    if (!kPaged && p.test_stall && --left == 0) { ok = false; break; }     // test hook: the item's last tile never arrives
+                    const int s = issued % C::kStages;
+                    const uint32_t ph = (uint32_t)(issued / C::kStages) & 1u;
+                    // a box past the level's last row is aimed past the pool, where the copy engine fills zeros as it does
+                    // past a dense level's end
+                    int z = kt * kTileN, w = b;                        // dense: row in the level, batch; paged: row in the page, page
+                    if constexpr (kPaged) {
+                        const long long row = (long long)kt * kTileN + lane * rpb;
+                        w = p.pool_pages[l];
+                        if (mine && row < n_here) w = tab[row >> p.page_shift[l]];
+                        z = (int)(row & in_mask);
+                    }
+                    if (!mbar_wait_warp(&bar.k_empty[s], ph ^ 1u, abortp)) { ok = false; break; }
+                    if (lane == 0) mbar_expect_tx(&bar.k_full[s], C::kTileBytes);
+                    __syncwarp();
+                    if (mine) {
+#pragma unroll
+                        for (int pn = 0; pn < C::kPanels; ++pn)
+                            tma_load_4d(sK + s * C::kTileBytes + pn * kPanelBytes + lane * rpb * 128, &maps.k[l], pn * 64, z, kvh, w, &bar.k_full[s]);
+                    }
+                    __syncwarp();
+                    if (!mbar_wait_warp(&bar.v_empty[s], ph ^ 1u, abortp)) {           // gave up with this stage's K copies in flight
+                        mbar_drain(&bar.k_full[s], ph, abortp, gtimer());
+                        ok = false;
+                        break;
+                    }
+                    if (lane == 0) mbar_expect_tx(&bar.v_full[s], C::kTileBytes);
+                    __syncwarp();
+                    if (mine) {
+#pragma unroll
+                        for (int pn = 0; pn < C::kPanels; ++pn)
+                            tma_load_4d(sV + s * C::kTileBytes + pn * kPanelBytes + lane * rpb * 128, &maps.v[l], pn * 64, z, kvh, w, &bar.v_full[s]);
+                    }
+                    __syncwarp();
+                    ++issued;
+                }
+            }
+            if (!ok) { ++it; break; }                         // its Q was asked for
+            done_item(it);
         }
         // Before leaving, make sure every copy issued has landed (bounded): the shared memory must not be handed to
         // another CTA with a bulk copy still in flight.  (A stage whose wait failed got no copies.)
         const unsigned long long t_drain = gtimer();
-        mbar_drain(&bar.q_full, 0, abortp, t_drain);
+        if (it > 0) mbar_drain(&bar.q_full, (uint32_t)(it - 1) & 1u, abortp, t_drain);
         for (int i = issued > C::kStages ? issued - C::kStages : 0; i < issued; ++i) {
             mbar_drain(&bar.k_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp, t_drain);
             mbar_drain(&bar.v_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp, t_drain);
         }
-    } else if (warp == C::kProducerWarp) {
-        // Dense levels: the warp waits converged and one lane issues (inside an `if (lane == 0)` around the whole loop the
-        // kernel keeps its loop state in local memory: 1.63 us per key tile instead of 1.49 at d = 128).
-        if (lane == 0) {
-            mbar_expect_tx(&bar.q_full, C::kNumQ * C::kTileBytes);
-#pragma unroll
-            for (int q = 0; q < C::kNumQ; ++q)
-#pragma unroll
-                for (int pn = 0; pn < C::kPanels; ++pn)
-                    tma_load_4d(sQ + q * C::kTileBytes + pn * kPanelBytes, &maps.q, pn * 64, (int)(m0 + q * kTileM), h, b, &bar.q_full);
-        }
-        int issued = 0;
-        bool ok = true;
-        const int kvh = h / p.kv_group;
-#pragma unroll 1
-        for (int l = 0; l < 3 && ok; ++l) {
-            const int kt_end = pick3(end, l);
-            for (int kt = pick3(first, l); kt < kt_end; ++kt) {
-                if (p.test_stall && issued == E - 1) break;        // test hook: the last tile never arrives
-                const int s = issued % C::kStages;
-                const uint32_t ph = (uint32_t)(issued / C::kStages) & 1u;
-                if (!mbar_wait_warp(&bar.k_empty[s], ph ^ 1u, abortp)) { ok = false; break; }
+    } else if (warp == C::kDealWarp) {
+        if constexpr (kForm == kStream) {
+            for (int it = 1;; ++it) {
+                Item next;
+                next_piece(next);
+                if (it >= 2 && !mbar_wait_warp(&bar.item_free[it & 1], (uint32_t)((it - 2) >> 1) & 1u, abortp)) break;
                 if (lane == 0) {
-                    mbar_expect_tx(&bar.k_full[s], C::kTileBytes);
-#pragma unroll
-                    for (int pn = 0; pn < C::kPanels; ++pn)
-                        tma_load_4d(sK + s * C::kTileBytes + pn * kPanelBytes, &maps.k[l], pn * 64, kt * kTileN, kvh, b, &bar.k_full[s]);
+                    items[it & 1] = next;
+                    mbar_arrive(&bar.item_full[it & 1]);
                 }
                 __syncwarp();
-                if (!mbar_wait_warp(&bar.v_empty[s], ph ^ 1u, abortp)) {           // gave up with this stage's K copies in flight
-                    mbar_drain(&bar.k_full[s], ph, abortp, gtimer());
-                    ok = false;
-                    break;
-                }
-                if (lane == 0) {
-                    mbar_expect_tx(&bar.v_full[s], C::kTileBytes);
-#pragma unroll
-                    for (int pn = 0; pn < C::kPanels; ++pn)
-                        tma_load_4d(sV + s * C::kTileBytes + pn * kPanelBytes, &maps.v[l], pn * 64, kt * kTileN, kvh, b, &bar.v_full[s]);
-                }
-                __syncwarp();
-                ++issued;
+                if (next.E < 0) break;
             }
-        }
-        // Before leaving, make sure every copy issued has landed (bounded): the shared memory must not be handed to
-        // another CTA with a bulk copy still in flight.  (A stage whose wait failed got no copies.)
-        const unsigned long long t_drain = gtimer();
-        mbar_drain(&bar.q_full, 0, abortp, t_drain);
-        for (int i = issued > C::kStages ? issued - C::kStages : 0; i < issued; ++i) {
-            mbar_drain(&bar.k_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp, t_drain);
-            mbar_drain(&bar.v_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp, t_drain);
         }
     } else if (warp == C::kMmaWarp) {
         {   // every lane runs the issue loop (converged); elect.sync inside the wrappers picks the issuing lane
-            bool ok = mbar_wait_warp(&bar.q_full, 0, abortp);
-            tc_fence_after();
             // low descriptor words of the operands (see make_desc)
             const uint32_t q_lo = desc_lo_kmajor(smem_u32(sQ)), k_lo = desc_lo_kmajor(smem_u32(sK));
             const uint32_t v_lo = desc_lo_mnmajor(smem_u32(sV), kPanelBytes);
@@ -371,6 +494,32 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
                            C::kIdescQK, k > 0);
                 mma_commit_elect(&bar.s_full[q]);
             };
+            auto k_ready = [&](int g) { return mbar_wait_warp(&bar.k_full[g % C::kStages], (uint32_t)(g / C::kStages) & 1u, abortp); };
+            auto v_ready = [&](int g) { return mbar_wait_warp(&bar.v_full[g % C::kStages], (uint32_t)(g / C::kStages) & 1u, abortp); };
+            // O_q += P_q V in parts: the softmax warps hand over the weights of 32 keys at a time (K-steps 2 part,
+            // 2 part + 1), so that the product runs under the remaining exponentials.
+            auto issue_pv = [&](int q, int g, bool accumulate) -> bool {
+                const uint32_t va = v_lo + (g % C::kStages) * (C::kTileBytes >> 4);
+                const uint32_t pa = tmem + (C::kSeparateP ? C::kColP + q * (kTileN / 2) : q * kTileN);
+#pragma unroll
+                for (int part = 0; part < C::kParts; ++part) {
+                    if (!mbar_wait_warp(&bar.p_part[q][part], (uint32_t)g & 1u, abortp)) return false;
+                    tc_fence_after();
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        const int k = part * 2 + i;
+                        mma_ts_elect(tmem + C::kColO + q * DH, pa + k * 8, make_desc(va + k * (2048 >> 4)), C::kIdescPV,
+                                     (accumulate || part > 0 || i > 0) ? 1u : 0u);
+                    }
+                }
+                mma_commit_elect(&bar.pv_done[q]);
+                return true;
+            };
+            int g = 0;                                        // key tiles of the CTA, across its items
+            bool ok = true;
+            for (int it = 0; ok && has_item(it); ++it) {
+            const Item& I = items[it & 1];
+            const int E = __shfl_sync(0xffffffffu, I.E, 0);   // warp-uniform for the compiler too
             // Paged levels: the page that holds a level's last row is copied whole, so the rows after that row arrive
             // with whatever the pool holds there (a recycled page, never-written memory).  Their weights are exactly 0,
             // but 0 x NaN or 0 x Inf would still poison the accumulator: those V rows are cleared here, after the
@@ -380,9 +529,9 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
                 int e0 = 0;
 #pragma unroll
                 for (int l = 0; l < 3; ++l) {
-                    const int tiles = end[l] - first[l];
-                    const int tail = (int)(nl[l] % kTileN);
-                    if (tiles > 0 && tail != 0 && (long long)end[l] * kTileN > nl[l]) {
+                    const int tiles = I.end[l] - I.first[l];
+                    const int tail = I.n[l] % kTileN;
+                    if (tiles > 0 && tail != 0 && (long long)I.end[l] * kTileN > I.n[l]) {
                         const int rpb = p.box_rows[l];
                         scrub_e[l] = e0 + tiles - 1;
                         scrub_r0[l] = tail;
@@ -406,185 +555,157 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
                 }
                 }
             };
-            // O_q += P_q V in parts: the softmax warps hand over the weights of 32 keys per thread at a time (K-steps
-            // 2 part, 2 part + 1 of every thread's columns), so that the product runs under the remaining exponentials.
-            auto issue_pv = [&](int q, int s, int e, bool accumulate) -> bool {
-                const uint32_t va = v_lo + s * (C::kTileBytes >> 4);
-                const uint32_t pa = tmem + (C::kSeparateP ? C::kColP + q * (kTileN / 2) : q * kTileN);
-#pragma unroll
-                for (int part = 0; part < C::kParts; ++part) {
-                    if (!mbar_wait_warp(&bar.p_part[q][part], (uint32_t)e & 1u, abortp)) return false;
-                    tc_fence_after();
-#pragma unroll
-                    for (int i = 0; i < 2 * C::kSplit; ++i) {
-                        const int k = (i >> 1) * (8 / C::kSplit) + part * 2 + (i & 1);
-                        mma_ts_elect(tmem + C::kColO + q * DH, pa + k * 8, make_desc(va + k * (2048 >> 4)), C::kIdescPV,
-                                     (accumulate || part > 0 || i > 0) ? 1u : 0u);
-                    }
-                }
-                mma_commit_elect(&bar.pv_done[q]);
-                return true;
-            };
+            if (!(ok = mbar_wait_warp(&bar.q_full, (uint32_t)it & 1u, abortp))) break;
+            tc_fence_after();
+            if (E == 0) {
+                mma_commit_elect(&bar.q_empty);
+                done_item(it);
+                continue;
+            }
+            if (!(ok = k_ready(g))) break;
             if (C::kSeparateP) {
                 // S_q(e+1) is issued as soon as the warpgroup has S_q(e) in registers; O_q += P_q(e) V(e) when P_q(e) is written.
-                if (ok && E > 0) ok = mbar_wait_warp(&bar.k_full[0], 0, abortp);
-                if (ok && E > 0) {
+                for (int q = 0; q < C::kNumQ && ok; ++q) {
+                    if (g > 0 && !mbar_wait_warp(&bar.s_free[q], (uint32_t)(g - 1) & 1u, abortp)) { ok = false; break; }
                     tc_fence_after();
-                    issue_qk(0, 0);
-                    issue_qk(1, 0);
-                    mma_commit_elect(&bar.k_empty[0]);
+                    issue_qk(q, g % C::kStages);
                 }
-                for (int e = 0; e < E && ok; ++e) {
-                    const int s = e % C::kStages, sn = (e + 1) % C::kStages;
+                if (!ok) break;
+                mma_commit_elect(&bar.k_empty[g % C::kStages]);
+                if (E == 1) mma_commit_elect(&bar.q_empty);
+                for (int e = 0; e < E && ok; ++e, ++g) {
+                    const int s = g % C::kStages, sn = (g + 1) % C::kStages;
                     if (e + 1 < E) {
-                        if (!mbar_wait_warp(&bar.k_full[sn], (uint32_t)((e + 1) / C::kStages) & 1u, abortp)) { ok = false; break; }
+                        if (!k_ready(g + 1)) { ok = false; break; }
 #pragma unroll
                         for (int q = 0; q < C::kNumQ; ++q) {
-                            if (!mbar_wait_warp(&bar.s_free[q], (uint32_t)e & 1u, abortp)) { ok = false; break; }
+                            if (!mbar_wait_warp(&bar.s_free[q], (uint32_t)g & 1u, abortp)) { ok = false; break; }
                             tc_fence_after();
                             issue_qk(q, sn);
                         }
                         if (!ok) break;
                         mma_commit_elect(&bar.k_empty[sn]);
+                        if (e + 2 == E) mma_commit_elect(&bar.q_empty);
                     }
-                    if (!mbar_wait_warp(&bar.v_full[s], (uint32_t)(e / C::kStages) & 1u, abortp)) { ok = false; break; }
+                    if (!v_ready(g)) { ok = false; break; }
                     scrub_v(e, s);
 #pragma unroll
                     for (int q = 0; q < C::kNumQ; ++q) {
-                        if (!issue_pv(q, s, e, e > 0)) { ok = false; break; }
+                        if (!issue_pv(q, g, e > 0)) { ok = false; break; }
                     }
                     if (!ok) break;
                     mma_commit_elect(&bar.v_empty[s]);
                 }
             } else {
-            // The wait for K(e+1) is taken before the wait for P_0(e), so that S_0(e+1) follows O_0(e) at once: that
-            // pair of products is what query tile 0's softmax threads are waiting for.
-            if (ok && E > 0) ok = mbar_wait_warp(&bar.k_full[0], 0, abortp);
-            for (int e = 0; e < E && ok; ++e) {
-                const int s = e % C::kStages;
-                const uint32_t ph = (uint32_t)(e / C::kStages) & 1u;
-                tc_fence_after();
-                issue_qk(0, s);
-                if (e > 0) {
-                    const int sp = (e - 1) % C::kStages;
-                    if (!issue_pv(1, sp, e - 1, e - 1 > 0)) { ok = false; break; }
-                    mma_commit_elect(&bar.v_empty[sp]);
+                // The wait for K(e+1) is taken before the wait for P_0(e), so that S_0(e+1) follows O_0(e) at once: that
+                // pair of products is what query tile 0's softmax threads are waiting for.
+                for (int e = 0; e < E && ok; ++e, ++g) {
+                    const int s = g % C::kStages;
+                    tc_fence_after();
+                    issue_qk(0, s);
+                    if (e > 0) {
+                        if (!issue_pv(1, g - 1, e - 1 > 0)) { ok = false; break; }
+                        mma_commit_elect(&bar.v_empty[(g - 1) % C::kStages]);
+                    }
+                    issue_qk(1, s);
+                    mma_commit_elect(&bar.k_empty[s]);
+                    if (e + 1 == E) mma_commit_elect(&bar.q_empty);
+                    if (!v_ready(g)) { ok = false; break; }
+                    scrub_v(e, s);
+                    if (e + 1 < E && !k_ready(g + 1)) { ok = false; break; }
+                    if (!issue_pv(0, g, e > 0)) { ok = false; break; }
                 }
-                issue_qk(1, s);
-                mma_commit_elect(&bar.k_empty[s]);
-                if (!mbar_wait_warp(&bar.v_full[s], ph, abortp)) { ok = false; break; }
-                scrub_v(e, s);
-                if (e + 1 < E && !mbar_wait_warp(&bar.k_full[(e + 1) % C::kStages], (uint32_t)((e + 1) / C::kStages) & 1u, abortp)) { ok = false; break; }
-                if (!issue_pv(0, s, e, e > 0)) { ok = false; break; }
+                if (!ok) break;
+                if (!(ok = issue_pv(1, g - 1, E > 1))) break;
+                mma_commit_elect(&bar.v_empty[(g - 1) % C::kStages]);
             }
-            if (ok && E > 0) {
-                const int sp = (E - 1) % C::kStages;
-                if (issue_pv(1, sp, E - 1, E - 1 > 0)) mma_commit_elect(&bar.v_empty[sp]);
+            done_item(it);
             }
-            }   // !kSeparateP
         }
     }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(C::kRegsSoftmax));
         // ------------------------------------------------------------ softmax warps
-        // warp = (query tile, column part, lane quarter); thread = one query row (TMEM lane) x kCols key columns.
-        // With two threads per row (d = 64) they agree on the row maximum through shared memory at a 256-thread barrier
-        // that also carries their "no wait has run out" flags, so that the 256 threads always leave together.
-        const int q = warp / C::kRowWarps, half = (warp >> 2) % C::kSplit;
+        // warp = (query tile, lane quarter); thread = one query row (TMEM lane)
+        const int q = warp / C::kRowWarps;
         const int row_in_tile = (warp & 3) * 32 + lane;
-        const int t = (int)m0 + q * kTileM + row_in_tile;    // T < 2^31
-        const bool row_valid = t < p.T;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        const uint32_t s_addr = tmem + lane_base + q * kTileN + half * C::kCols;
-        const uint32_t o_addr = tmem + lane_base + C::kColO + q * DH + half * (DH / C::kSplit);
+        const uint32_t s_addr = tmem + lane_base + q * kTileN;
+        const uint32_t o_addr = tmem + lane_base + C::kColO + q * DH;
         // where this thread's weights go as bf16 pairs
-        const uint32_t p_addr = (C::kSeparateP ? tmem + lane_base + C::kColP + q * (kTileN / 2) : tmem + lane_base + q * kTileN) + half * (C::kCols / 2);
-        const long long tq0 = m0 + (long long)q * kTileM;                      // first row of this query tile
-        const long long tq1 = (tq0 + kTileM - 1 < p.T - 1) ? tq0 + kTileM - 1 : p.T - 1;
-        auto row_all = [&](bool flag) -> bool {                                 // AND over the threads of the query tile
-            if constexpr (C::kSplit == 1) return flag;
-            uint32_t out;
-            asm volatile("{\n.reg .pred pi, po;\nsetp.ne.u32 pi, %1, 0;\nbar.red.and.pred po, %2, 256, pi;\nselp.u32 %0, 1, 0, po;\n}"
-                         : "=r"(out) : "r"((uint32_t)flag), "r"(1 + q) : "memory");
-            return out != 0;
-        };
-
-        float m_run = -INFINITY, l_run = 0.f;                                    // l_run: this thread's columns only
-        bool ok = true, all_ok = true;                                           // ok is warp-uniform
+        const uint32_t p_addr = C::kSeparateP ? tmem + lane_base + C::kColP + q * (kTileN / 2) : tmem + lane_base + q * kTileN;
+        bool ok = true;                                                          // warp-uniform
+        int g = 0;                                                               // key tiles of the CTA, across its items
+#pragma unroll 1
+        for (int it = 0; ok && has_item(it); ++it) {
+        const Item& I = items[it & 1];
+        const int tq0 = I.m[q];                                                  // first row of this query tile
+        const int t = tq0 + row_in_tile;                                         // T < 2^31 - 256
+        const bool row_valid = t < p.T;
+        float m_run = -INFINITY, l_run = 0.f;
         int e = 0;
 #pragma unroll 1
-        for (int l = 0; l < 3 && all_ok; ++l) {
-            const int kt_first = pick3(first, l), kt_end = pick3(end, l);
+        for (int l = 0; l < 3 && ok; ++l) {
+            const int kt_first = I.first[l], kt_end = I.end[l];
             if (kt_first == kt_end) continue;
-            const long long n_here = pick3(nl, l);
+            const long long n_here = I.n[l];
             float bias = -INFINITY;
             int lo = 0, hi = 0;                              // visible rows of this level (levels hold fewer than 2^31 rows)
             // A row past T has a bias of -inf, so its weights are 0 whatever it sees: it takes the last row's range and
             // costs its warp no mask of its own.
             if (row_valid) {
-                const float g = p.gate[((long long)b * p.T + t) * 3 + l];
-                bias = g > 0.f ? log2f(g) : -INFINITY;
+                const float gt = p.gate[((long long)I.b * p.T + t) * 3 + l];
+                bias = gt > 0.f ? log2f(gt) : -INFINITY;
             }
             // key tiles visible to every row of THIS query tile need no element mask
             int full_first = 0, full_end = 0x7fffffff;                     // (a tile without a row inside T masks nothing)
-            if (tq0 <= tq1) {
+            if (tq0 < p.T) {
+                const int tq1 = min(tq0 + kTileM - 1, p.T - 1);
                 {
                     long long lo64, hi64;
                     visible_range(l, (row_valid ? (long long)t : tq1) + p.q_offset, p.window, n_here, 0, lo64, hi64);
                     lo = (int)lo64; hi = (int)hi64;
                 }
                 long long lo_f, hi_f, lo_l, hi_l;
-                visible_range(l, tq0 + p.q_offset, p.window, n_here, 0, lo_f, hi_f);
-                visible_range(l, tq1 + p.q_offset, p.window, n_here, 0, lo_l, hi_l);
+                visible_range(l, (long long)tq0 + p.q_offset, p.window, n_here, 0, lo_f, hi_f);
+                visible_range(l, (long long)tq1 + p.q_offset, p.window, n_here, 0, lo_l, hi_l);
                 full_first = (int)((lo_l + kTileN - 1) / kTileN);
                 full_end = (int)(hi_f / kTileN);
             }
-            for (int kt = kt_first; kt < kt_end; ++kt, ++e) {
-                if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&bar.s_full[q], (uint32_t)e & 1u, abortp));
-                float s[C::kCols];
-                float mx = -INFINITY;
-                if (ok) {
-                    tc_fence_after();
+            for (int kt = kt_first; kt < kt_end; ++kt, ++e, ++g) {
+                if (!(ok = __all_sync(0xffffffffu, mbar_wait(&bar.s_full[q], (uint32_t)g & 1u, abortp)))) break;
+                float s[kTileN];
+                tc_fence_after();
 #pragma unroll
-                    for (int c0 = 0; c0 < C::kCols; c0 += 32) tmem_ld32(s_addr + c0, reinterpret_cast<uint32_t*>(s) + c0);
-                    tmem_ld_wait();
-                    if (C::kSeparateP) {                     // S(e) is in registers: its TMEM columns may be reused
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&bar.s_free[q]);
-                    }
-                    const bool need_mask = !(kt >= full_first && kt < full_end);
-                    if (need_mask) {
-                        const long long col0 = (long long)kt * kTileN + half * C::kCols;
-                        const int c_lo = (int)max(0LL, min((long long)lo - col0, (long long)C::kCols));
-                        const int c_hi = (int)max(0LL, min((long long)hi - col0, (long long)C::kCols));
-                        // One bit per column: the bits of 32 columns come from two shifts and each costs a test and a select.
-                        // Two comparisons per column made a masked tile take 3.6 us against 1.6 (now 2.1).
-#pragma unroll
-                        for (int c0 = 0; c0 < C::kCols; c0 += 32) {      // 32 columns that no row of the warp masks are passed over
-                            const uint32_t vis = low_bits(c_hi - c0) & ~low_bits(c_lo - c0);
-                            if (__all_sync(0xffffffffu, vis == 0xffffffffu)) continue;
-#pragma unroll
-                            for (int i = 0; i < 32; ++i) s[c0 + i] = (vis >> i) & 1u ? s[c0 + i] : -INFINITY;
-                        }
-                    }
-                    float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-                    for (int c = 0; c < C::kCols; c += 8) {
-                        mx4[0] = max3(mx4[0], s[c], s[c + 1]); mx4[1] = max3(mx4[1], s[c + 2], s[c + 3]);
-                        mx4[2] = max3(mx4[2], s[c + 4], s[c + 5]); mx4[3] = max3(mx4[3], s[c + 6], s[c + 7]);
-                    }
-                    mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+                for (int c0 = 0; c0 < kTileN; c0 += 32) tmem_ld32(s_addr + c0, reinterpret_cast<uint32_t*>(s) + c0);
+                tmem_ld_wait();
+                if (C::kSeparateP) {                         // S(e) is in registers: its TMEM columns may be reused
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&bar.s_free[q]);
                 }
-                if constexpr (C::kSplit == 2) {
-                    xmax[e & 1][q][half][row_in_tile] = mx;
-                    all_ok = row_all(ok);
-                    if (!all_ok) break;
-                    mx = fmaxf(mx, xmax[e & 1][q][half ^ 1][row_in_tile]);
-                } else {
-                    all_ok = ok;
-                    if (!all_ok) break;
+                const bool need_mask = !(kt >= full_first && kt < full_end);
+                if (need_mask) {
+                    const long long col0 = (long long)kt * kTileN;
+                    const int c_lo = (int)max(0LL, min((long long)lo - col0, (long long)kTileN));
+                    const int c_hi = (int)max(0LL, min((long long)hi - col0, (long long)kTileN));
+                    // One bit per column: the bits of 32 columns come from two shifts and each costs a test and a select.
+                    // Two comparisons per column made a masked tile take 3.6 us against 1.6 (now 2.1).
+#pragma unroll
+                    for (int c0 = 0; c0 < kTileN; c0 += 32) {        // 32 columns that no row of the warp masks are passed over
+                        const uint32_t vis = low_bits(c_hi - c0) & ~low_bits(c_lo - c0);
+                        if (__all_sync(0xffffffffu, vis == 0xffffffffu)) continue;
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) s[c0 + i] = (vis >> i) & 1u ? s[c0 + i] : -INFINITY;
+                    }
                 }
+                float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+                for (int c = 0; c < kTileN; c += 8) {
+                    mx4[0] = max3(mx4[0], s[c], s[c + 1]); mx4[1] = max3(mx4[1], s[c + 2], s[c + 3]);
+                    mx4[2] = max3(mx4[2], s[c + 4], s[c + 5]); mx4[3] = max3(mx4[3], s[c + 6], s[c + 7]);
+                }
+                const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
                 const float x_max = fmaf(mx, p.scale_log2, bias);            // -inf when the whole row is masked
                 const float m_new = fmaxf(m_run, x_max);
                 const bool grow = m_new > m_run + kRescaleThreshold;         // also true for the first finite max
@@ -597,84 +718,75 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
                 // P(e-1) must have been consumed before P(e) replaces it (d = 64), and before O is rescaled
                 const bool rescale = e > 0 && __any_sync(0xffffffffu, alpha != 1.f);
                 if ((C::kSeparateP || rescale) && e > 0) {
-                    ok = __all_sync(0xffffffffu, mbar_wait(&bar.pv_done[q], (uint32_t)(e - 1) & 1u, abortp));
-                    if (ok) tc_fence_after();
+                    if (!(ok = __all_sync(0xffffffffu, mbar_wait(&bar.pv_done[q], (uint32_t)(g - 1) & 1u, abortp)))) break;
+                    tc_fence_after();
                 }
-                if (ok) {
-                    if (rescale) {                           // some row of this warp moved its reference maximum
+                if (rescale) {                               // some row of this warp moved its reference maximum
 #pragma unroll 1
-                        for (int c0 = 0; c0 < DH / C::kSplit; c0 += 32) {
-                            uint32_t o[32];
-                            tmem_ld32(o_addr + c0, o);
-                            tmem_ld_wait();
+                    for (int c0 = 0; c0 < DH; c0 += 32) {
+                        uint32_t o[32];
+                        tmem_ld32(o_addr + c0, o);
+                        tmem_ld_wait();
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-                            tmem_st32(o_addr + c0, o);
-                        }
+                        for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+                        tmem_st32(o_addr + c0, o);
                     }
-                    // The weights leave in parts of 32 columns (16 packed pairs, one store each).  A part is handed to
-                    // the issuing warp in the middle of the next part's exponentials, when its store has long completed.
-                    // Scale, shift and the row sum work on packed pairs: one instruction for two columns.
-                    const uint64_t scale2 = pack2(p.scale_log2, p.scale_log2), shift2 = pack2(shift, shift);
-                    uint64_t sum_a = pack2(0.f, 0.f), sum_b = sum_a;
-                    uint32_t pk[16];
-                    auto weights = [&](int c_from, int c_to, int c_base) {
-#pragma unroll
-                        for (int c = c_from; c < c_to; c += 4) {
-                            float x0, x1, x2, x3;
-                            unpack2(fma2(pack2(s[c], s[c + 1]), scale2, shift2), x0, x1);
-                            unpack2(fma2(pack2(s[c + 2], s[c + 3]), scale2, shift2), x2, x3);
-                            const float p0 = ex2(x0), p1 = ex2(x1), p2 = ex2(x2), p3 = ex2(x3);
-                            sum_a = add2(sum_a, pack2(p0, p1));
-                            sum_b = add2(sum_b, pack2(p2, p3));
-                            pk[(c - c_base) / 2] = pack_bf16(p0, p1);
-                            pk[(c - c_base) / 2 + 1] = pack_bf16(p2, p3);
-                        }
-                    };
-                    auto hand_over = [&](int part) {         // the part (and a rescaled accumulator) is in TMEM
-                        tmem_st_wait();
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&bar.p_part[q][part]);
-                    };
-#pragma unroll
-                    for (int part = 0; part < C::kParts; ++part) {
-                        weights(32 * part, 32 * part + 16, 32 * part);
-                        if (part > 0) hand_over(part - 1);
-                        weights(32 * part + 16, 32 * part + 32, 32 * part);
-                        tmem_st16(p_addr + 16 * part, pk);
-                    }
-                    {
-                        float a0, a1;
-                        unpack2(add2(sum_a, sum_b), a0, a1);
-                        l_run += a0 + a1;
-                    }
-                    hand_over(C::kParts - 1);
                 }
+                // The weights leave in parts of 32 columns (16 packed pairs, one store each).  A part is handed to
+                // the issuing warp in the middle of the next part's exponentials, when its store has long completed.
+                // Scale, shift and the row sum work on packed pairs: one instruction for two columns.
+                const uint64_t scale2 = pack2(p.scale_log2, p.scale_log2), shift2 = pack2(shift, shift);
+                uint64_t sum_a = pack2(0.f, 0.f), sum_b = sum_a;
+                uint32_t pk[16];
+                auto weights = [&](int c_from, int c_to, int c_base) {
+#pragma unroll
+                    for (int c = c_from; c < c_to; c += 4) {
+                        float x0, x1, x2, x3;
+                        unpack2(fma2(pack2(s[c], s[c + 1]), scale2, shift2), x0, x1);
+                        unpack2(fma2(pack2(s[c + 2], s[c + 3]), scale2, shift2), x2, x3);
+                        const float p0 = ex2(x0), p1 = ex2(x1), p2 = ex2(x2), p3 = ex2(x3);
+                        sum_a = add2(sum_a, pack2(p0, p1));
+                        sum_b = add2(sum_b, pack2(p2, p3));
+                        pk[(c - c_base) / 2] = pack_bf16(p0, p1);
+                        pk[(c - c_base) / 2 + 1] = pack_bf16(p2, p3);
+                    }
+                };
+                auto hand_over = [&](int part) {             // the part (and a rescaled accumulator) is in TMEM
+                    tmem_st_wait();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&bar.p_part[q][part]);
+                };
+#pragma unroll
+                for (int part = 0; part < C::kParts; ++part) {
+                    weights(32 * part, 32 * part + 16, 32 * part);
+                    if (part > 0) hand_over(part - 1);
+                    weights(32 * part + 16, 32 * part + 32, 32 * part);
+                    tmem_st16(p_addr + 16 * part, pk);
+                }
+                {
+                    float a0, a1;
+                    unpack2(add2(sum_a, sum_b), a0, a1);
+                    l_run += a0 + a1;
+                }
+                hand_over(C::kParts - 1);
             }
         }
         // ------------------------------------------------------------ epilogue
-        if (all_ok) {
-            if (ok && E > 0) ok = __all_sync(0xffffffffu, mbar_wait(&bar.pv_done[q], (uint32_t)(E - 1) & 1u, abortp));
-            if constexpr (C::kSplit == 2) lsum[q][half][row_in_tile] = l_run;   // the row's sum is the sum of its two halves
-            all_ok = row_all(ok);
-        }
-        if constexpr (kSplitKeys) {
+        const int E = I.E;
+        if (ok && E > 0) ok = __all_sync(0xffffffffu, mbar_wait(&bar.pv_done[q], (uint32_t)(g - 1) & 1u, abortp));
+        if constexpr (kForm == kCluster) {
             // Every operand tile has been read when all softmax warps have seen their last product (and no copy is in
             // flight then), so O may lie over the K and V rings: four columns of all 128 rows, then the next four.
-            if (half == 0) {
-                const bool any = all_ok && E > 0;
-                cl_max[q][row_in_tile] = any ? m_run : -INFINITY;
-                float l_row = l_run;
-                if constexpr (C::kSplit == 2) l_row += lsum[q][1][row_in_tile];
-                cl_sum[q][row_in_tile] = any ? l_row : 0.f;
-            }
+            const bool any = ok && E > 0;
+            cl_max[q][row_in_tile] = any ? m_run : -INFINITY;
+            cl_sum[q][row_in_tile] = any ? l_run : 0.f;
             asm volatile("bar.sync 4, %0;" ::"n"(C::kSoftmaxWarps * 32) : "memory");
-            if (all_ok && !abortp->abort) {
+            if (ok && !abortp->abort) {
                 tc_fence_after();
-                float4* so = reinterpret_cast<float4*>(sK) + (q * DH + half * (DH / C::kSplit)) / 4 * kTileM + row_in_tile;
+                float4* so = reinterpret_cast<float4*>(sK) + q * DH / 4 * kTileM + row_in_tile;
 #pragma unroll 1
-                for (int c0 = 0; c0 < DH / C::kSplit; c0 += 32) {
+                for (int c0 = 0; c0 < DH; c0 += 32) {
                     uint32_t o[32];
                     if (E > 0) {
                         tmem_ld32(o_addr + c0, o);
@@ -688,17 +800,30 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
                         so[(c0 + i) / 4 * kTileM] = make_float4(__uint_as_float(o[i]), __uint_as_float(o[i + 1]), __uint_as_float(o[i + 2]), __uint_as_float(o[i + 3]));
                 }
             }
-        }
-        if (!kSplitKeys && all_ok) {
+        } else if (kForm == kStream && ok && I.slot >= 0) {
+            // a piece of a cut block: its accumulator as it is, rows next to each other (a warp stores 512 bytes at a time)
             tc_fence_after();
-            float l_row = l_run;
-            if constexpr (C::kSplit == 2) l_row += lsum[q][half ^ 1][row_in_tile];
-            const float inv = l_row > 0.f ? 1.f / l_row : 0.f;   // rows with nothing visible: exact zeros
-            const int first_row = (warp & 3) * 32;                       // of this warp, within the query tile
-            __nv_bfloat16* out = p.O + (((long long)b * p.H + h) * p.T + tq0 + first_row) * DH + half * (DH / C::kSplit);
-            const int rows_here = (int)max(0LL, min(32LL, p.T - tq0 - first_row));
+            float* slot = p.slots + (long long)I.slot * C::kSlotFloats;
+            float4* so = reinterpret_cast<float4*>(slot) + q * DH / 4 * kTileM + row_in_tile;
 #pragma unroll 1
-            for (int c0 = 0; c0 < DH / C::kSplit; c0 += 32) {
+            for (int c0 = 0; c0 < DH; c0 += 32) {
+                uint32_t o[32];
+                tmem_ld32(o_addr + c0, o);
+                tmem_ld_wait();
+#pragma unroll
+                for (int i = 0; i < 32; i += 4)
+                    so[(c0 + i) / 4 * kTileM] = make_float4(__uint_as_float(o[i]), __uint_as_float(o[i + 1]), __uint_as_float(o[i + 2]), __uint_as_float(o[i + 3]));
+            }
+            reinterpret_cast<float2*>(slot + C::kNumQ * kTileM * DH)[q * kTileM + row_in_tile] = make_float2(m_run, l_run);
+        } else if (ok) {
+            tc_fence_after();
+            const float inv = l_run > 0.f ? 1.f / l_run : 0.f;           // rows with nothing visible: exact zeros
+            const int first_row = (warp & 3) * 32;                       // of this warp, within the query tile
+            const long long bh = (long long)I.b * p.H + I.h[q];
+            __nv_bfloat16* out = p.O + (bh * p.T + tq0 + first_row) * DH;
+            const int rows_here = max(0, min(32, p.T - tq0 - first_row));
+#pragma unroll 1
+            for (int c0 = 0; c0 < DH; c0 += 32) {
                 uint32_t o[32];
                 if (E > 0) {
                     tmem_ld32(o_addr + c0, o);
@@ -710,12 +835,13 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
                 }
                 store_rows_bf16<32>(out + c0, DH, rows_here, o, inv, lane);
             }
-            if (row_valid && half == 0 && p.LSE)
-                p.LSE[((long long)b * p.H + h) * p.T + t] = l_row > 0.f ? (m_run + log2f(l_row)) * kLn2 : -INFINITY;
+            if (row_valid && p.LSE) p.LSE[bh * p.T + t] = l_run > 0.f ? (m_run + log2f(l_run)) * kLn2 : -INFINITY;
+        }
+        done_item(it);
         }
     }
 
-    if constexpr (kSplitKeys) {
+    if constexpr (kForm == kCluster) {
         // Merge: every CTA takes its share of the block's columns, a few at a time, and adds the cluster's parts with the
         // weights 2^(max_i - max) / sum.  The second barrier keeps a CTA's shared memory alive until all have read it.
         __syncwarp();
@@ -727,7 +853,8 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
             int have_q = -1;
             for (int u = crank * (C::kSoftmaxWarps / 4) + (warp >> 2); u < C::kNumQ * DH / C::kMergeCols; u += csize * (C::kSoftmaxWarps / 4)) {
                 const int q = u / (DH / C::kMergeCols), c0 = (u % (DH / C::kMergeCols)) * C::kMergeCols;
-                const int t = (int)m0 + q * kTileM + row_in_tile;
+                const int t = items[0].m[q] + row_in_tile;
+                const long long bh = (long long)items[0].b * p.H + items[0].h[q];
                 if (t >= p.T) continue;
                 if (q != have_q || c0 == 0) {
                     float mi[kMaxSplit], mx = -INFINITY, sum = 0.f;
@@ -745,7 +872,7 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
 #pragma unroll
                     for (int i = 0; i < kMaxSplit; ++i) w[i] = inv > 0.f ? w[i] * inv : 0.f;
                     have_q = inv > 0.f ? q : kMaxQ + q;
-                    if (c0 == 0 && p.LSE) p.LSE[((long long)b * p.H + h) * p.T + t] = sum > 0.f ? (mx + log2f(sum)) * kLn2 : -INFINITY;
+                    if (c0 == 0 && p.LSE) p.LSE[bh * p.T + t] = sum > 0.f ? (mx + log2f(sum)) * kLn2 : -INFINITY;
                 }
                 float acc[C::kMergeCols];
 #pragma unroll
@@ -772,14 +899,7 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
                         }
                     }
                 }
-                __nv_bfloat16* out = p.O + (((long long)b * p.H + h) * p.T + t) * DH + c0;
-#pragma unroll
-                for (int c = 0; c < C::kMergeCols; c += 8) {
-                    uint4 v;
-                    v.x = pack_bf16(acc[c], acc[c + 1]); v.y = pack_bf16(acc[c + 2], acc[c + 3]);
-                    v.z = pack_bf16(acc[c + 4], acc[c + 5]); v.w = pack_bf16(acc[c + 6], acc[c + 7]);
-                    *reinterpret_cast<uint4*>(out + c) = v;
-                }
+                store_cols_bf16<C::kMergeCols>(p.O + (bh * p.T + t) * DH + c0, acc);
             }
         }
         __syncwarp();
@@ -789,6 +909,71 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
     __syncthreads();
     if (tid == 0 && wait_ctl.abort) atomicExch(p.status, (unsigned int)MKA_ERR_TIMEOUT);
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::kTmemCols) : "memory");
+}
+
+// kStream, second kernel: adds up the pieces of the cut blocks.  Boundary i = blockIdx.x + 1 lies between the ranges of CTAs i - 1 and i
+// of the first kernel; the first boundary inside a block's tiles does the whole block, eight columns of 128 rows to a warpgroup.
+// Its bytes come from the L2 cache: two pieces of 128 KB (d = 128) at most per CTA.
+constexpr int kMergeThreads = 256, kMergeAhead = 4;
+template <int DH>
+__global__ void __launch_bounds__(kMergeThreads, 4) fwd_merge_kernel(const TcParams p) {
+    using C = Cfg<DH>;
+    chain_trigger();
+    const int lane = threadIdx.x & 31;
+    const int cut = range_start(p, blockIdx.x + 1);                       // first unit of CTA blockIdx.x + 1
+    const int line = cut / p.line_units;
+    int qb, unit0;
+    find_block(p, cut - line * p.line_units, lane, qb, unit0);
+    const int E = block_units(qb, p.block_rows, p.T, p.q_offset, p.window, p.n) - kBlockUnits;
+    const int at = line * p.line_units + unit0;                           // the block's first unit
+    chain_wait();                                                         // (every CTA: what follows this kernel relies on it for the first one too)
+    if (cut <= at || cut >= at + E) return;                               // between two blocks
+    const int i0 = range_of(p, at), parts = range_of(p, at + E - 1) - i0 + 1;
+    if (i0 != (int)blockIdx.x) return;                                    // not the block's first boundary
+    int b, kvh, h[kMaxQ], m[kMaxQ];
+    block_tiles_of<DH>(p, line, qb, b, kvh, h, m);
+    // CTA i0 holds the block's first tiles in its second slot, the others theirs in their first
+    const float* s0 = p.slots + (long long)(2 * i0 + 1) * C::kSlotFloats;
+    const long long step = 2LL * C::kSlotFloats;
+    const int row = threadIdx.x & 127;
+    for (int c8 = blockIdx.y * (kMergeThreads / 128) + (threadIdx.x >> 7); c8 < C::kNumQ * DH / 8; c8 += gridDim.y * (kMergeThreads / 128)) {
+    const int q = c8 / (DH / 8), c0 = (c8 % (DH / 8)) * 8;
+    const int t = (q == 0 ? m[0] : m[1]) + row;
+    if (t >= p.T) continue;
+    const int ml_at = C::kNumQ * kTileM * DH + (q * kTileM + row) * 2, o_at = ((q * DH + c0) / 4 * kTileM + row) * 4;
+    float mx = -INFINITY, sum = 0.f, acc[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) acc[c] = 0.f;
+    for (int i = 0; i < parts; i += kMergeAhead) {                        // the loads of several pieces are in flight together
+        float2 ml[kMergeAhead];
+        float4 lo[kMergeAhead], hi[kMergeAhead];
+#pragma unroll
+        for (int j = 0; j < kMergeAhead; ++j) {
+            const int k = min(i + j, parts - 1);
+            const float* sl = k == 0 ? s0 : s0 + k * step - C::kSlotFloats;
+            ml[j] = *reinterpret_cast<const float2*>(sl + ml_at);
+            lo[j] = *reinterpret_cast<const float4*>(sl + o_at);
+            hi[j] = *reinterpret_cast<const float4*>(sl + o_at + kTileM * 4);
+        }
+#pragma unroll
+        for (int j = 0; j < kMergeAhead; ++j) {
+            if (i + j >= parts || ml[j].x == -INFINITY) continue;         // (a row that sees none of the piece's tiles)
+            const float m_new = fmaxf(mx, ml[j].x);
+            const float keep = mx == -INFINITY ? 0.f : ex2(mx - m_new), w = ex2(ml[j].x - m_new);
+            mx = m_new;
+            sum = fmaf(w, ml[j].y, sum * keep);
+            const float v[8] = {lo[j].x, lo[j].y, lo[j].z, lo[j].w, hi[j].x, hi[j].y, hi[j].z, hi[j].w};
+#pragma unroll
+            for (int c = 0; c < 8; ++c) acc[c] = fmaf(w, v[c], acc[c] * keep);
+        }
+    }
+    const float inv = sum > 0.f ? 1.f / sum : 0.f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) acc[c] = inv > 0.f ? acc[c] * inv : 0.f;
+    const long long at_row = ((long long)b * p.H + (q == 0 ? h[0] : h[1])) * p.T + t;
+    store_cols_bf16<8>(p.O + at_row * DH + c0, acc);
+    if (c0 == 0 && p.LSE) p.LSE[at_row] = sum > 0.f ? (mx + log2f(sum)) * kLn2 : -INFINITY;
+    }
 }
 
 inline bool make_map(CUtensorMap* map, const void* base, int d, long long rows, int H, int B, long long sn, long long sh, long long sb) {
@@ -815,7 +1000,7 @@ int resident_clusters(int split) {
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
     int n = known[dev][split].load(std::memory_order_relaxed);
     if (n) return n - 1;
-    auto kern = fwd_tc_kernel<DH, false, true>;
+    auto kern = fwd_tc_kernel<DH, false, kCluster>;
     cudaLaunchAttribute at;
     const cudaLaunchConfig_t cfg = cluster_config<DH>(split, dim3(split), nullptr, &at);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<DH>::kSmemBytes) != cudaSuccess ||
@@ -827,47 +1012,100 @@ int resident_clusters(int split) {
     return n;
 }
 
-// Key tiles of one block of query rows (device row counts of paged levels are not known here: n bounds them).
-template <int DH>
-int block_tiles(const FwdParams& fp, long long q_block) {
-    const long long r0 = q_block * Cfg<DH>::kNumQ * kTileM;
-    const long long r1 = r0 + Cfg<DH>::kNumQ * kTileM - 1 < fp.T - 1 ? r0 + Cfg<DH>::kNumQ * kTileM - 1 : fp.T - 1;
-    int tiles = 0;
-    for (int l = 0; l < 3; ++l) {
-        int first = 0, end = 0;
-        if (fp.L[l].n > 0) tile_range(l, r0, r1, fp.q_offset, fp.window, fp.L[l].n, first, end);
-        tiles += end - first;
-    }
-    return tiles;
+// How the query tiles are put into blocks.
+struct Blocks {
+    int pair_heads, rows;         // see TcParams
+    long long lines;
+    int per_line;
+};
+
+// Key tiles of one block (device row counts of paged levels are not known here: n bounds them).
+int block_tiles(const FwdParams& fp, const Blocks& bl, long long q_block) {
+    const long long n[3] = {fp.L[0].n, fp.L[1].n, fp.L[2].n};
+    return block_units((int)q_block, bl.rows, fp.T, fp.q_offset, fp.window, n) - kBlockUnits;
 }
 
-// CTAs that share a block of query rows.  A launch with fewer blocks than the chip holds CTAs (a chunk of a prompt, short
-// sequences) leaves SMs idle while every block walks its whole tile list; splitting the list between the CTAs of a cluster
-// costs each of them its start-up and the merge.  Counted in key tiles (1.5 us at d = 128): 3 for start-up and epilogue,
-// 7 with the merge; blocks start heaviest first, so round r of the resident clusters lasts as long as its first block, and
-// two CTAs on one SM (d = 64) take 1.3 times as long each.  A split has to promise 15 % (below that the model is no better
-// than a coin).  Measured, forward alone, unsplit / split by 2 / 3 / 4 / 5 / 8, chosen in brackets:
-//   d = 128, 28 heads, 512 rows at 15,000 rows of context    263 / [144] / 199 / 160 / 197 / 197 us  (56 blocks, 160 tiles)
-//   d = 128, 12 heads, 700 rows at 6000 rows                 121 / 72 / [56] / 86 / 77 / 91 us       (36 blocks, 71 tiles)
-//   d = 128, 32 heads, 100 rows at 1500 rows                 50 / 34 / 28 / [25] / 43 / 53 us        (32 blocks, 24 tiles)
-//   d = 128, 16 heads, 1500 rows                             [96] / 102 / 109 / 103 / 121 / 167 us   (96 blocks, 36 to 54 tiles)
-//   d = 64, 28 heads, 1500 rows                              [57] / 61 / 75 / 80 / 95 / 138 us       (336 blocks)
+// d = 128: 256 consecutive rows of a head, or 128 rows of two heads of a group where that makes fewer key tiles to walk (a last
+// block with 128 rows or fewer is half empty; two heads see exactly the same keys).  2 x 69 rows at 5467, 32 heads on 8, in
+// clusters, the better size for each: 82 us in blocks of one head, 49 in pairs.
 template <int DH>
-int split_rule(const FwdParams& fp, int q_blocks) {
-    const long long pairs = (long long)fp.B * fp.H, blocks = pairs * q_blocks;
+Blocks make_blocks(const FwdParams& fp) {
+    Blocks bl;
+    bl.pair_heads = 0; bl.rows = Cfg<DH>::kNumQ * kTileM;
+    bl.lines = (long long)fp.B * fp.H;
+    bl.per_line = (fp.T + bl.rows - 1) / bl.rows;
+    if (DH != 128 || fp.kv_group < 2 || bl.per_line > 32) return bl;
+    Blocks two = {1, kTileM, bl.lines / fp.kv_group * ((fp.kv_group + 1) / 2), (fp.T + kTileM - 1) / kTileM};
+    double t1 = 0.0, t2 = 0.0;
+    for (int i = 0; i < bl.per_line; ++i) t1 += block_tiles(fp, bl, i) + kBlockUnits;
+    for (int i = 0; i < two.per_line; ++i) t2 += block_tiles(fp, two, i) + kBlockUnits;
+    return t2 * (double)two.lines < 0.97 * t1 * (double)bl.lines ? two : bl;
+}
+
+// Which form.  A launch whose blocks do not fill the chip, or fill it a little more than once, leaves SMs idle while others walk whole
+// lists.  Cluster or equal ranges then share the lists out; the first costs its merge and whole clusters per GPC, the second a pass
+// of partial results through the L2 cache, and its CTAs, each in another place of the keys, find less of them there.  All are added
+// up in us: a round of resident CTAs lasts as long as its first (heaviest) block.  The constants were fitted to 34 sizes (8 to 1600
+// blocks, 4 to 490 tiles a block), over which the pick takes 0.7 % more than the best form on average, 10 % at most.  Whole / clusters of 2 / 3 /
+// 4 / 8 / ranges, chosen in brackets:
+//   d = 128, 28 heads on 4, 512 rows at 15,000 rows of context      265 / 144 / 195 / 155 / 191 / [124] us   (56 blocks, 160 tiles)
+//   d = 128, 12 on 4, 949 rows at 3804                              93 / 59 / 79 / 69 / 101 / [51] us        (48 blocks, 61 tiles)
+//   d = 128, 12 on 4, 175 rows at 4662                              90 / 53 / 40 / 34 / [25] / 33 us         (12 blocks, 54 tiles)
+//   d = 128, 12 on 4, 124 rows at 36,735                            452 / 234 / 161 / 124 / 73 / [55] us     (8 blocks, 295 tiles)
+//   d = 128, 32 on 8, 2 x 69 rows at 5467                           127 / 83 / 58 / [49] / 84 / 63 us        (32 blocks, 75 tiles)
+//   d = 128, 16 heads, 3078 rows                                    164 / 170 / 194 / 228 / 347 / [155] us   (208 blocks)
+//   d = 128, 2 x 16 heads, 1000 rows                                [35] / 51 / 63 / 80 / 149 / 56 us        (128 blocks)
+//   d = 64, 2 x 32 heads, 627 rows, 7815 slots                      179 / 157 / 159 / 164 / 205 / [137] us   (320 blocks)
+//   d = 64, 16 heads, 777 rows                                      [19] / 17 / 23 / 24 / 41 / 23 us         (112 blocks)
+struct FormChoice { int form, ctas; };       // kCluster: CTAs of a cluster; kStream: CTAs of the grid
+template <int DH>
+FormChoice form_rule(const FwdParams& fp, const Blocks& bl, bool scratch) {
+    const long long lines = bl.lines, blocks = lines * bl.per_line;
     const int slots = 148 * Cfg<DH>::kCtasPerSm;
-    if (blocks > slots) return 1;
-    int best = 1;
-    double best_cost = 0.85 * (block_tiles<DH>(fp, q_blocks - 1) + 3) * (blocks > 148 ? 1.3 : 1.0);
-    for (int split = 2; split <= kMaxSplit; ++split) {
-        const int fit = resident_clusters<DH>(split);
-        if (fit < 1) continue;
-        double cost = 0.0;
-        for (long long blk = 0; blk < blocks && cost < best_cost; blk += fit)
-            cost += ((double)block_tiles<DH>(fp, q_blocks - 1 - blk / pairs) / split + 7) * (blocks * split > 148 ? (DH == 64 ? 1.3 : 1.0) : 1.0);
-        if (cost < best_cost) { best = split; best_cost = cost; }
+    const double tile = DH == 128 ? 1.54 : 0.93;                            // us for a CTA that has its SM to itself
+    auto shared = [](long long ctas) { return DH == 64 && ctas > 148 ? 1.36 : 1.0; };
+    FormChoice best = {kWhole, 1};
+    if (blocks > kStreamRounds * slots) return best;                         // whole blocks fill the chip evenly enough
+    double best_us = 0.0;
+    for (long long blk = 0; blk < blocks; blk += slots)
+        best_us += block_tiles(fp, bl, bl.per_line - 1 - blk / lines) * tile * shared(blocks - blk) + (blk == 0 ? 7.0 : 4.5);
+    best_us *= 0.97;                                                         // (what the model can tell apart)
+    if (blocks <= slots) {
+        for (int split = 2; split <= kMaxSplit; ++split) {
+            const int fit = resident_clusters<DH>(split);
+            if (fit < 1) continue;
+            double us = 0.0;
+            for (long long blk = 0; blk < blocks && us < best_us; blk += fit)
+                us += block_tiles(fp, bl, bl.per_line - 1 - blk / lines) * tile * 1.03 / split * shared((blocks - blk < fit ? blocks - blk : fit) * split) +
+                      (blk == 0 ? 14.5 : 11.5);
+            if (us < best_us) { best = {kCluster, split}; best_us = us; }
+        }
+    }
+    if (scratch) {
+        double units = 0.0, mbytes = 0.0;
+        for (int qb = 0; qb < bl.per_line; ++qb) units += block_tiles(fp, bl, qb) + kBlockUnits;
+        units *= (double)lines;
+        for (int l = 0; l < 3; ++l) {
+            const double seen = l == 0 ? (double)fp.window + fp.T : 1e18;
+            mbytes += ((double)fp.L[l].n < seen ? (double)fp.L[l].n : seen) * fp.B * (fp.H / fp.kv_group) * (DH * 4e-6);
+        }
+        const double us = units / slots * tile * 1.18 * shared(slots) + 17.5 + 0.35 * slots / (double)blocks + (mbytes > 100.0 ? 0.068 * (mbytes - 100.0) : 0.0);
+        if (units >= slots && units < 1e9 && us < best_us) best = {kStream, slots};
     }
     return best;
+}
+
+template <int DH>
+bool known_rows(const FwdParams& fp) {       // kStream cuts by the levels' lengths, which a row count per sequence may undercut
+    for (int l = 0; l < 3; ++l) if (fp.paged && fp.L[l].n > 0 && fp.paged[l].rows) return false;
+    return true;
+}
+template <int DH>
+size_t scratch_bytes_t(const FwdParams& fp) {
+    const Blocks bl = make_blocks<DH>(fp);
+    if (bl.lines * bl.per_line > kStreamRounds * 148 * Cfg<DH>::kCtasPerSm || !known_rows<DH>(fp)) return 0;
+    const FormChoice c = form_rule<DH>(fp, bl, true);
+    return c.form == kStream ? (size_t)2 * c.ctas * Cfg<DH>::kSlotFloats * sizeof(float) : 0;
 }
 
 template <int DH>
@@ -906,25 +1144,46 @@ cudaError_t launch_t(const FwdParams& fp, unsigned int* status_word, cudaStream_
     p.status = status_word;
     p.wait_limit_ns = wait_limit_ns();
     p.test_stall = fp.test_stall;
-    {   // as many (batch, head) pairs per group as keep the group's K and V (48 MB at most) in the L2 cache while
+    const Blocks bl = make_blocks<DH>(fp);
+    {   // as many lines per group as keep the group's K and V (48 MB at most) in the L2 cache while
         // its blocks, dealt by query block, re-read them
         double pair_bytes = 0.0;
         for (int l = 0; l < 3; ++l) pair_bytes += (double)fp.L[l].n * DH * 4.0;
-        pair_bytes /= fp.kv_group;
-        const double pairs = (double)fp.B * fp.H;
-        const double fit = pair_bytes > 0.0 ? 48.0 * 1024 * 1024 / pair_bytes : pairs;
-        p.deal = fit < 1.0 ? 1 : (fit > pairs ? (int)pairs : (int)fit);
+        pair_bytes /= bl.pair_heads ? (fp.kv_group + 1) / 2 : fp.kv_group;
+        const double lines = (double)bl.lines;
+        const double fit = pair_bytes > 0.0 ? 48.0 * 1024 * 1024 / pair_bytes : lines;
+        p.deal = fit < 1.0 ? 1 : (fit > lines ? (int)lines : (int)fit);
     }
-    const int q_blocks = (fp.T + Cfg<DH>::kNumQ * kTileM - 1) / (Cfg<DH>::kNumQ * kTileM);
-    const int split = split_rule<DH>(fp, q_blocks);
-    auto kern = fp.paged ? (split > 1 ? fwd_tc_kernel<DH, true, true> : fwd_tc_kernel<DH, true, false>)
-                         : (split > 1 ? fwd_tc_kernel<DH, false, true> : fwd_tc_kernel<DH, false, false>);
+    p.pair_heads = bl.pair_heads; p.block_rows = bl.rows; p.lines = (int)bl.lines; p.q_blocks = bl.per_line;
+    const bool scratch = fp.scratch && (reinterpret_cast<uintptr_t>(fp.scratch) & 15) == 0 && known_rows<DH>(fp);
+    FormChoice form = form_rule<DH>(fp, bl, scratch);
+    if (form.form == kStream && fp.scratch_bytes < (size_t)2 * form.ctas * Cfg<DH>::kSlotFloats * sizeof(float)) form = form_rule<DH>(fp, bl, false);
+    auto kern = form.form == kStream    ? (fp.paged ? fwd_tc_kernel<DH, true, kStream> : fwd_tc_kernel<DH, false, kStream>)
+                : form.form == kCluster ? (fp.paged ? fwd_tc_kernel<DH, true, kCluster> : fwd_tc_kernel<DH, false, kCluster>)
+                                        : (fp.paged ? fwd_tc_kernel<DH, true, kWhole> : fwd_tc_kernel<DH, false, kWhole>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<DH>::kSmemBytes);
     if (e != cudaSuccess) return e;
-    return launch_chained(kern, dim3(q_blocks * split, fp.H, fp.B), dim3(Cfg<DH>::kThreads), Cfg<DH>::kSmemBytes, st, split > 1 ? split : 0, maps, p);
+    const long long blocks = bl.lines * bl.per_line;
+    if (form.form != kStream) {
+        if (blocks * form.ctas > 0x7fffffffLL) return cudaErrorInvalidValue;
+        return launch_chained(kern, dim3((unsigned)(blocks * form.ctas)), dim3(Cfg<DH>::kThreads), Cfg<DH>::kSmemBytes, st,
+                              form.form == kCluster ? form.ctas : 0, maps, p);
+    }
+    for (int qb = 0; qb < bl.per_line; ++qb) p.line_units += block_units(qb, bl.rows, p.T, p.q_offset, p.window, p.n);
+    const int units = p.lines * p.line_units;
+    p.range = units / form.ctas; p.longer = units % form.ctas;
+    p.slots = static_cast<float*>(fp.scratch);
+    e = launch_chained(kern, dim3(form.ctas), dim3(Cfg<DH>::kThreads), Cfg<DH>::kSmemBytes, st, 0, maps, p);
+    if (e != cudaSuccess) return e;
+    return launch_chained(fwd_merge_kernel<DH>, dim3(form.ctas - 1, DH == 128 ? 4 : 2), dim3(kMergeThreads), 0, st, 0, p);
 }
 
 }  // namespace
+
+size_t fwd_tc_scratch_bytes(const FwdParams& p) {
+    if (p.B == 0 || p.H == 0 || p.T == 0) return 0;
+    return p.d == 128 ? scratch_bytes_t<128>(p) : scratch_bytes_t<64>(p);
+}
 
 bool fwd_tc_eligible(const FwdParams& p, int dtype) {
     if (dtype != MKA_BF16 || p.mode != MKA_MODE_FAST || p.decode) return false;
