@@ -677,10 +677,10 @@ mka_status mka_l2_summary(const void* X, int32_t B, int64_t T, int32_t D, int32_
     if (!aligned16(X) || !aligned16(M2)) return MKA_ERR_ALIGN;
     if (ws && ws_bytes < kWsHeader) return MKA_ERR_WORKSPACE;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
-    if (ws && cudaMemsetAsync(ws, 0, 16, cs) != cudaSuccess) return MKA_ERR_CUDA;
     // With enough scratch the segmented (look-back) form cuts the sequences into 256-row segments, which keeps the GPU
     // busy however few column strips there are; otherwise one CTA walks each strip from end to end.
     const bool segmented = ws && (reinterpret_cast<uintptr_t>(ws) & 15) == 0 && mka_l2_summary_kernel_kind(B, T, D, dtype, ws_bytes) == 1;
+    if (ws && !segmented && cudaMemsetAsync(ws, 0, 16, cs) != cudaSuccess) return MKA_ERR_CUDA;      // (the segmented form clears its scratch itself)
     cudaError_t e = segmented
         ? launch_l2_summary_seg(X, M2, state, n_prev > 0 ? 1 : 0, n_prev, B, T, D, dtype, kind | stall, beta,
                                 static_cast<unsigned int*>(ws), static_cast<char*>(ws) + kWsHeader, cs)

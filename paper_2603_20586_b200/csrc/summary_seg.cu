@@ -344,8 +344,193 @@ __global__ void __launch_bounds__(kSegThreads, kSegCtasPerSm) l2_summary_seg_ker
     }
 }
 
+// The same tiles, one CTA to a strip: where the strips alone fill most of the chip, the segments of a strip are dealt to the groups
+// of four warps of one CTA, and the carried state goes from group to group through shared memory.  Nothing is published, polled
+// or cleared in global memory; a hand-over costs some 200 cycles where a look-back waits for an L2 round trip or two, and a group scans
+// and stores its tile while the others load theirs.  Every state is folded as in the form above, in the same order.
+// [1, 32768, 4096] bf16, 128 strips of 64 bytes: 98 us against 107 with the look-back and its two clears of scratch.
+constexpr int kPipeGroups = 6;                       // one 32 KB tile each
+
 template <typename T, bool kEma, int WB>
-cudaError_t launch_w(const void* X, SegParams p, cudaStream_t st) {
+__global__ void __launch_bounds__(kPipeGroups * kSegThreads, 1) l2_summary_pipe_kernel(const __grid_constant__ CUtensorMap map, const SegParams p) {
+    using P2 = typename Pair2<T>::type;
+    using V8 = typename Oct<T>::type;
+    constexpr int kSegRows = kSegTileBytes / WB, kNC = WB / (int)sizeof(T), kNP = kNC / 2, CW = Oct<T>::kCols;
+    constexpr int kNL = kNC / CW, G = kSegThreads / kNL, RG = kSegRows / G;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~static_cast<uintptr_t>(127));
+    __shared__ float part[kPipeGroups][G][kNC];
+    __shared__ float2 handed[kPipeGroups][kNP];                // the state entering a group's tile, from the group before it
+    __shared__ float2 carry[kPipeGroups][kNP];                 // the same for all of the group's warps
+    __shared__ float a_pow[RG + 1];                            // beta^j, j = 0..RG (EMA)
+    __shared__ uint64_t full[kPipeGroups], entered[kPipeGroups];
+    __shared__ WaitCtl wait_ctl;
+
+    const int tid = threadIdx.x % kSegThreads, wg = __shfl_sync(0xffffffffu, (int)threadIdx.x / kSegThreads, 0), lane = tid & 31;
+    const int c = tid % kNL, g = tid / kNL;
+    const int Tn = (int)p.T;
+    const float beta = p.beta, omb = 1.f - p.beta;
+    volatile WaitCtl* abortp = &wait_ctl;
+    float a_rg = 1.f, a_full = 1.f;                            // beta^RG, beta^kSegRows
+    if (kEma) {
+#pragma unroll
+        for (int k = 0; k < RG; ++k) a_rg *= beta;
+#pragma unroll
+        for (int k = 0; k < G; ++k) a_full *= a_rg;
+    }
+    if (kEma && threadIdx.x <= RG) {
+        float a = 1.f;
+        for (int j = 0; j < (int)threadIdx.x; ++j) a *= beta;
+        a_pow[threadIdx.x] = a;
+    }
+    if (threadIdx.x == 0) {
+        wait_ctl.abort = 0;
+        wait_ctl.limit_ns = p.wait_limit_ns;
+        for (int i = 0; i < kPipeGroups; ++i) { mbar_init(&full[i], 1); mbar_init(&entered[i], 1); }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    chain_enter();
+    if (threadIdx.x == 0 && blockIdx.x == 0 && p.status) atomicExch(p.status, (unsigned int)MKA_OK);      // (before any wait can run out)
+    __syncthreads();
+    const int b = blockIdx.x / p.strips, col0 = (blockIdx.x % p.strips) * kNC;
+    uint8_t* tile_bytes = smem + wg * kSegTileBytes;
+    const P2* tile = reinterpret_cast<const P2*>(tile_bytes);                    // [kSegRows][kNP]
+    auto load = [&](int seg) {
+        mbar_expect_tx(&full[wg], kSegTileBytes);
+#pragma unroll
+        for (int bx = 0; bx < kSegRows / kSegBoxRows; ++bx)
+            tma_load_3d(tile_bytes + (size_t)bx * kSegBoxRows * WB, &map, col0, seg * kSegRows + bx * kSegBoxRows, b, &full[wg]);
+    };
+    auto group_and = [&](bool flag) -> bool {                  // the group's barrier; true when the flag is for all of its threads
+        uint32_t out;
+        asm volatile("{\n.reg .pred pi, po;\nsetp.ne.u32 pi, %1, 0;\nbar.red.and.pred po, %2, %3, pi;\nselp.u32 %0, 1, 0, po;\n}"
+                     : "=r"(out) : "r"((uint32_t)flag), "r"(1 + wg), "n"(kSegThreads) : "memory");
+        return out != 0;
+    };
+    int loads = 0;                                             // of the group (thread 0)
+    if (tid == 0 && wg < p.S) { load(wg); ++loads; }
+    int n = 0;                                                 // the group's tiles so far
+    for (int seg = wg; seg < p.S; seg += kPipeGroups, ++n) {
+        const int row0 = seg * kSegRows;
+        bool ok = mbar_wait(&full[wg], n & 1, abortp);
+        // ---- 1. totals of this thread's rows (zero incoming state)
+        const int t0 = row0 + g * RG;
+        const int left = Tn - t0;
+        const int nv = left >= RG ? RG : (left > 0 ? left : 0);
+        const V8* trow = reinterpret_cast<const V8*>(tile) + (size_t)g * RG * kNL + c;
+        float r[CW];
+#pragma unroll
+        for (int j = 0; j < CW; ++j) r[j] = 0.f;
+        if (ok) {
+#pragma unroll
+            for (int k = 0; k < RG; ++k) {
+                float x[CW];
+                Oct<T>::unpack(trow[k * kNL], x);
+                if (nv == RG || k < nv) {
+#pragma unroll
+                    for (int j = 0; j < CW; ++j) r[j] = kEma ? fmaf(beta, r[j], omb * x[j]) : r[j] + x[j];
+                }
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < CW; ++j) part[wg][g][c * CW + j] = r[j];
+        const int seg_rows = Tn - row0 >= kSegRows ? kSegRows : Tn - row0;      // valid rows of this segment (>= 1)
+        auto group_a = [&](int gg) -> float {                                    // a of row group gg of this segment
+            if (!kEma) return 1.f;
+            const int l2 = Tn - (row0 + gg * RG);
+            return a_pow[l2 >= RG ? RG : (l2 > 0 ? l2 : 0)];
+        };
+        if (!group_and(ok)) break;
+        // ---- 2. the group's first warp: segment aggregate, state entering and leaving.  Lane = column pair (kNP <= 32).
+        if (tid < 32) {
+            const bool col_ok = lane < kNP && col0 + 2 * lane < p.D;
+            float2 tot = make_float2(0.f, 0.f), in = tot;
+            if (lane < kNP) {
+#pragma unroll
+                for (int gg = 0; gg < G; ++gg) {
+                    const float a = group_a(gg);
+                    const float2 pt = *reinterpret_cast<const float2*>(&part[wg][gg][2 * lane]);
+                    tot.x = kEma ? fmaf(a, tot.x, pt.x) : tot.x + pt.x;
+                    tot.y = kEma ? fmaf(a, tot.y, pt.y) : tot.y + pt.y;
+                }
+            }
+            float a_seg = a_full;                                                // beta^(rows of this segment)
+            if (kEma && seg_rows != kSegRows) {
+                a_seg = 1.f;
+                for (int gg = 0; gg < G; ++gg) a_seg *= group_a(gg);
+            }
+            bool wok = true;
+            if (seg == 0) {
+                if (lane < kNP) {
+                    if (p.use_state) {
+                        if (col_ok) in = *reinterpret_cast<const float2*>(p.state + (long long)b * p.D + col0 + 2 * lane);
+                    } else if (kEma) {
+                        Pair2<T>::unpack(tile[lane], in.x, in.y);                // m_{-1} := x_0 makes m_0 = x_0
+                    }
+                }
+            } else {
+                wok = mbar_wait_warp(&entered[wg], (uint32_t)(wg == 0 ? n - 1 : n) & 1u, abortp);
+                if (wok && lane < kNP) in = handed[wg][lane];
+            }
+            if (wok) {
+                const float2 out_state = make_float2(fmaf(a_seg, in.x, tot.x), fmaf(a_seg, in.y, tot.y));
+                if (seg + 1 < p.S && !(p.test_stall && seg == 1)) {
+                    // the next group has taken its last state: it could not have handed its own on, nor this tile come, otherwise
+                    const int to = wg + 1 < kPipeGroups ? wg + 1 : 0;
+                    if (lane < kNP) handed[to][lane] = out_state;
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&entered[to]);
+                }
+                if (col_ok && seg == p.S - 1 && p.state) *reinterpret_cast<float2*>(p.state + (long long)b * p.D + col0 + 2 * lane) = out_state;
+                if (lane < kNP) carry[wg][lane] = in;
+            }
+        }
+        if (!group_and(!abortp->abort)) break;
+        // ---- 3. scan again from the true incoming state and store: the lanes of a row cover its WB bytes
+        {
+            float m[CW];
+#pragma unroll
+            for (int j = 0; j < CW; ++j) m[j] = reinterpret_cast<const float*>(carry[wg])[c * CW + j];
+#pragma unroll
+            for (int gg = 0; gg < G; ++gg) {
+                if (gg < g) {
+                    const float a = group_a(gg);
+#pragma unroll
+                    for (int j = 0; j < CW; ++j) m[j] = kEma ? fmaf(a, m[j], part[wg][gg][c * CW + j]) : m[j] + part[wg][gg][c * CW + j];
+                }
+            }
+            float cnt = (float)(p.n_prev + (long long)t0 + 1);
+            V8* orow = reinterpret_cast<V8*>(static_cast<T*>(p.M2) + ((long long)b * p.T + t0) * p.D + col0) + c;
+            const long long ostride = p.D / CW;                                  // row pitch in 8-byte units
+            const bool col_ok = col0 + CW * c < p.D;
+#pragma unroll
+            for (int k = 0; k < RG; ++k) {
+                float x[CW], v[CW];
+                Oct<T>::unpack(trow[k * kNL], x);
+                if (kEma) {
+#pragma unroll
+                    for (int j = 0; j < CW; ++j) { m[j] = fmaf(beta, m[j], omb * x[j]); v[j] = m[j]; }
+                } else {
+                    const float inv = __fdividef(1.f, cnt);
+                    cnt += 1.f;
+#pragma unroll
+                    for (int j = 0; j < CW; ++j) { m[j] += x[j]; v[j] = m[j] * inv; }
+                }
+                if (col_ok && (nv == RG || k < nv)) orow[k * ostride] = Oct<T>::pack(v);
+            }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");           // the next load into the tile follows these reads
+        group_and(true);
+        if (tid == 0 && seg + kPipeGroups < p.S) { load(seg + kPipeGroups); ++loads; }
+    }
+    // A group that gave up may still have a load in flight: wait for it (bounded) before the shared memory goes away.
+    if (tid == 0 && wait_ctl.abort && loads > 0) mbar_drain(&full[wg], (uint32_t)(loads - 1) & 1u, abortp, gtimer());
+    __syncthreads();
+    if (threadIdx.x == 0 && wait_ctl.abort && p.status) atomicExch(p.status, (unsigned int)MKA_ERR_TIMEOUT);
+}
+
+template <typename T, bool kEma, int WB>
+cudaError_t launch_w(const void* X, SegParams p, bool one_cta_per_strip, cudaStream_t st) {
     constexpr int kNC = WB / (int)sizeof(T);
     constexpr int kRows = kSegTileBytes / WB;
     p.S = (int)((p.T + kRows - 1) / kRows);
@@ -354,9 +539,15 @@ cudaError_t launch_w(const void* X, SegParams p, cudaStream_t st) {
     if (tiles > 0x7fffffffLL) return cudaErrorNotSupported;
     CUtensorMap map;
     if (!make_strip_map(&map, X, sizeof(T) == 2, p.D, p.T, p.B, kNC, kSegBoxRows)) return cudaErrorNotSupported;
+    if (one_cta_per_strip) {
+        const size_t smem = (size_t)kPipeGroups * kSegTileBytes + 128;
+        cudaError_t e = cudaFuncSetAttribute(l2_summary_pipe_kernel<T, kEma, WB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        return launch_chained(l2_summary_pipe_kernel<T, kEma, WB>, dim3(p.strips * p.B), dim3(kPipeGroups * kSegThreads), smem, st, 0, map, p);
+    }
     const size_t smem = (size_t)kSegTileBytes + 128;
-    // the ticket counter and the records this launch will use start at zero
-    cudaError_t e = cudaMemsetAsync(p.ticket, 0, 256 + (size_t)p.B * p.S * p.D * sizeof(unsigned long long), st);
+    // the status word, the ticket counter and the records this launch will use start at zero
+    cudaError_t e = cudaMemsetAsync(p.status, 0, kWsHeader + 256 + (size_t)p.B * p.S * p.D * sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(l2_summary_seg_kernel<T, kEma, WB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -365,12 +556,24 @@ cudaError_t launch_w(const void* X, SegParams p, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// Strip width: 128 bytes when all sequences together offer about 200 strips, else 64.
+// Form and strip width.  One CTA to a strip (one round of them: 148 strips at most) costs each its strip's length, 2.4 us per 1000 rows
+// of 64 bytes, 4.5 of 128, and some more the more of them share the memory; the look-back form fills the chip whatever the
+// strips, at 5.5 TB/s, and costs the clears and the waits of its first segments.  us, look-back / strips of 64 / 128 bytes, bf16:
+//   [1,   600, 2048]  9.9 / [6.5] / 6.1     [1,  4000, 2048] [12.6] / 15.4 / 20.1     [1, 16000, 3072] [47] / 50 / 78
+//   [1,  4000, 4096]  21 / [16.4] / 21.2    [1, 16000, 4096] 56 / [54.6] / 80.6       [1, 65536, 4096] 191 / [184] / 290
+//   [2,  4000, 3584]  29 / - / [27.6]       [3, 16000, 2048] [77] / - / 85            [1, 65536, 3584] [172] / 177 / 281
+// Look-back strips: 128 bytes when all sequences together offer about 200, else 64.
 template <typename T, bool kEma>
 cudaError_t launch_k(const void* X, const SegParams& p, cudaStream_t st) {
-    const long long strips128 = (long long)p.B * ((p.D * (long long)sizeof(T) + 127) / 128);
-    if (strips128 >= 192) return launch_w<T, kEma, 128>(X, p, st);
-    return launch_w<T, kEma, 64>(X, p, st);          // 32-byte strips were measured too: they lose more in DRAM efficiency than they gain
+    auto strips = [&](int wb) { return (long long)p.B * ((p.D * (long long)sizeof(T) + wb - 1) / wb); };
+    const long long strips128 = strips(128), strips64 = strips(64);
+    const double look_back = 7.5 + 2.0 * p.B * p.T * p.D * sizeof(T) / 5.5e6;
+    const double in64 = strips64 > 148 ? 1e30 : 4.9 + p.T * (2.35e-3 + 0.65e-3 * strips64 / 128);
+    const double in128 = strips128 > 148 ? 1e30 : 4.9 + p.T * (4.45e-3 + 0.75e-3 * strips128 / 112);
+    if (in64 <= in128 && in64 < look_back) return launch_w<T, kEma, 64>(X, p, true, st);
+    if (in128 < look_back) return launch_w<T, kEma, 128>(X, p, true, st);
+    if (strips128 >= 192) return launch_w<T, kEma, 128>(X, p, false, st);
+    return launch_w<T, kEma, 64>(X, p, false, st);          // 32-byte strips were measured too: they lose more in DRAM efficiency than they gain
 }
 
 }  // namespace
