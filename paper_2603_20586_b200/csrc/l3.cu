@@ -7,7 +7,7 @@
 // chain over the columns.
 //   l3_index_kernel     HBM-bound: reads every key of the pool once, writes bits/8 bytes per (page, KV head)
 //   l3_retrieve_kernel  one CTA per (sequence, KV head): query code, Hamming scores of the bank, a binary search for the R-th best
-#include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace mka {
 namespace {
@@ -309,6 +309,7 @@ struct L3RetrieveParams {
     int* rows;                    // [B] or null: n_sel * page_rows
     long long bank_stride;
     int B, H, H_kv, d, bits, R, page_rows, max_bank;
+    int per_cta;                  // chunks that a CTA of the cluster takes at most
     int stage_proj;               // the projection is staged in shared memory (it fits beside the scores and is 16-byte aligned)
     int code_vec;                 // code words fetched by one load: 4 (16-byte aligned codes of 128 or 256 bits), 2 (64 bits, 8-byte aligned) or 1
 };
@@ -316,34 +317,36 @@ struct L3RetrieveParams {
 constexpr int kRetThreads = 1024;
 constexpr int kRetWarps = kRetThreads / 32;
 
-// Sum of v over the CTA, the same in every thread; `part` is reused by the next call but one.
-__device__ __forceinline__ int cta_sum(int v, int* part, int warp, int lane) {
-    v = __reduce_add_sync(0xffffffffu, v);
-    if (lane == 0) part[warp] = v;
-    __syncthreads();
-    return __reduce_add_sync(0xffffffffu, part[lane]);
-}
+constexpr int kRetMaxCluster = 8;
 
-// One CTA per (sequence, KV head).  Everything here is latency: the code words of the bank are asked for before the query's
-// code is worked out, and the R best are not picked one after the other (a pass over the bank and two barriers each, 28 us
-// for 8 of 8192 chunks) but cut off at once: a binary search over the score finds the R-th best, one pass in bank order
-// counts what each group of 32 chunks contributes, and a scan of those counts tells every recalled chunk its place in
-// the list.  15 us now.
-// Dynamic shared memory: unsigned short score[max_bank], int before[max_bank / 32 rounded up to whole CTAs], the projection.
+// A cluster of CTAs per (sequence, KV head), each with a stretch of the bank.  Everything here is latency: the code words are asked for
+// before the query's code is worked out; the R best are not picked one after the other but cut off at once.  A CTA counts its
+// chunks by score, the counts of the cluster meet in distributed shared memory, and the R-th best score, what lies above it and
+// how much of both the CTAs in front hold come from one scan over them; inside a CTA per-group counts and their scan give every
+// recalled chunk its place in bank order.  The gather of the codes is one sector a chunk, which a single SM's L1 works off one a
+// cycle: with one CTA and a binary search over the scores (a pass and a barrier each step), 8 of 8192 chunks took 15 us.
+// Dynamic shared memory: unsigned short score[per_cta], int before[per_cta / 32 rounded up to whole rounds], the projection.
 __global__ void __launch_bounds__(kRetThreads) l3_retrieve_kernel(const L3RetrieveParams p) {
-    chain_enter();
     extern __shared__ __align__(16) unsigned short score[];
     __shared__ __align__(16) float qs[256];
     __shared__ __align__(16) unsigned int qcode[8];
-    __shared__ int part[2][kRetWarps];
-    int* before = reinterpret_cast<int*>(score + (p.max_bank + 7) / 8 * 8);
-    float* projs = reinterpret_cast<float*>(before + (p.max_bank + kRetThreads - 1) / kRetThreads * kRetWarps);   // [bits][d + 4]
+    __shared__ int hist[257], total[257], lower[257];          // chunks by score: this CTA's, the cluster's, those of the CTAs in front
+    __shared__ int cut_s[4];
+    chain_enter();
+    int rank, size;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(size));
+    int* before = reinterpret_cast<int*>(score + (p.per_cta + 7) / 8 * 8);
+    float* projs = reinterpret_cast<float*>(before + (p.per_cta + kRetThreads - 1) / kRetThreads * kRetWarps);   // [bits][d + 4]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int b = blockIdx.x / p.H_kv, kvh = blockIdx.x % p.H_kv;
+    const int list = blockIdx.x / size, b = list / p.H_kv, kvh = list % p.H_kv;
     const int G = p.H / p.H_kv, words = p.bits / 32;
-    int n = p.bank_len[b];
-    n = n < 0 ? 0 : (n > p.max_bank ? p.max_bank : n);
-    const int* bank = p.bank + (long long)b * p.bank_stride;
+    int n_bank = p.bank_len[b];
+    n_bank = n_bank < 0 ? 0 : (n_bank > p.max_bank ? p.max_bank : n_bank);
+    const int per = ((n_bank + size - 1) / size + 31) / 32 * 32;            // at most per_cta
+    const int c_first = min(rank * per, n_bank), n = min(per, n_bank - c_first);   // this CTA's chunks, from here on counted from its first
+    const int* bank = p.bank + (long long)b * p.bank_stride + c_first;
+    for (int i = tid; i <= p.bits; i += kRetThreads) hist[i] = 0;
     // 64-bit codes: the first eight chunks of a thread, page numbers first, then all code words.  (Wider codes would need 32 and
     // 64 registers for that, half or all of what a thread has here; theirs are asked for after the query's code.)
     constexpr int kAhead = 8;
@@ -401,7 +404,10 @@ __global__ void __launch_bounds__(kRetThreads) l3_retrieve_kernel(const L3Retrie
 #pragma unroll
         for (int u = 0; u < kAhead; ++u) {
             const int c = tid + u * kRetThreads;
-            if (c < n) score[c] = (unsigned short)(p.bits - __popc(ahead[u].x ^ q0) - __popc(ahead[u].y ^ q1));
+            if (c >= n) continue;
+            const int sc = p.bits - __popc(ahead[u].x ^ q0) - __popc(ahead[u].y ^ q1);
+            score[c] = (unsigned short)sc;
+            atomicAdd(&hist[sc], 1);
         }
     }
     // All words of a code lie in one sector, so they are fetched together: word by word over eight chunks, a CTA's 8192 sectors had
@@ -417,7 +423,9 @@ __global__ void __launch_bounds__(kRetThreads) l3_retrieve_kernel(const L3Retrie
         }
         auto put = [&](int u, int dist) {
             const int c = c0 + u * kRetThreads;
-            if (c < n) score[c] = (unsigned short)(p.bits - dist);
+            if (c >= n) return;
+            score[c] = (unsigned short)(p.bits - dist);
+            atomicAdd(&hist[p.bits - dist], 1);
         };
         if (p.code_vec == 4) {
             const uint4 qa = *reinterpret_cast<const uint4*>(qcode), qb = *reinterpret_cast<const uint4*>(qcode + 4);
@@ -450,22 +458,47 @@ __global__ void __launch_bounds__(kRetThreads) l3_retrieve_kernel(const L3Retrie
         }
     }
     // (a thread reads back only the scores it wrote, up to the barriers below)
-    const int k = p.R < n ? p.R : n;
+    const int k = p.R < n_bank ? p.R : n_bank;
     const int rounds = (n + kRetThreads - 1) / kRetThreads;
-    // the largest score t that at least k chunks reach: all above it are recalled, and the earliest of those at it
-    int lo = 0, hi = p.bits + 1, above = 0, flip = 0;          // at least k chunks reach lo, fewer (above) reach hi
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) / 2;
-        int mine = 0;
-        for (int r = 0; r < rounds; ++r) {
-            const int c = r * kRetThreads + tid;
-            mine += c < n && score[c] >= mid ? 1 : 0;
+    __syncthreads();
+    cluster_sync();                                            // every CTA's counts are there
+    for (int i = tid; i <= p.bits; i += kRetThreads) {
+        int sum = 0, front = 0;
+#pragma unroll
+        for (int r = 0; r < kRetMaxCluster; ++r) {
+            const int v = r < size ? __float_as_int(ld_cluster(smem_u32(&hist[i]), r)) : 0;
+            sum += v;
+            front += r < rank ? v : 0;
         }
-        const int reach = cta_sum(mine, part[flip ^= 1], warp, lane);
-        if (reach >= k) lo = mid;
-        else { hi = mid; above = reach; }
+        total[i] = sum; lower[i] = front;
     }
-    const int at_cut = k - above;                              // how many of the chunks with score lo are recalled
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");           // (waited for at the end: nobody leaves while its counts are read)
+    __syncthreads();
+    // the largest score that at least k chunks reach, how many are above it, and how many above and at it the CTAs in front hold
+    if (warp == 0) {
+        int above = 0, above_front = 0;
+        for (int top = p.bits; top >= 0; top -= 32) {          // lane = score top - lane
+            const int at = top - lane, own = at >= 0 ? total[at] : 0, own_front = at >= 0 ? lower[at] : 0;
+            int sum = own, front = own_front;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int x = __shfl_up_sync(0xffffffffu, sum, o), y = __shfl_up_sync(0xffffffffu, front, o);
+                if (lane >= o) { sum += x; front += y; }
+            }
+            const unsigned int reach = __ballot_sync(0xffffffffu, above + sum >= k);
+            if (reach) {
+                if (lane == __ffs(reach) - 1) {
+                    cut_s[0] = at; cut_s[1] = above + sum - own;
+                    cut_s[2] = above_front + front - own_front; cut_s[3] = own_front;
+                }
+                break;
+            }
+            above += __shfl_sync(0xffffffffu, sum, 31);
+            above_front += __shfl_sync(0xffffffffu, front, 31);
+        }
+    }
+    __syncthreads();
+    const int lo = cut_s[0], at_cut = k - cut_s[1];            // the cut, and how many of the chunks at it are recalled
     // per group of 32 chunks, in bank order: chunks above the cut (low half) and at it (high half)
     for (int r = 0; r < rounds; ++r) {
         const int c = r * kRetThreads + tid;
@@ -491,7 +524,7 @@ __global__ void __launch_bounds__(kRetThreads) l3_retrieve_kernel(const L3Retrie
     }
     __syncthreads();
     int* out = p.table + ((long long)b * p.H_kv + kvh) * p.R;
-    int run_gt = 0, run_eq = 0;
+    int run_gt = cut_s[2], run_eq = min(cut_s[3], at_cut);     // (past at_cut the exact number does not matter)
     for (int r = 0; r < rounds; ++r) {
         const int c = r * kRetThreads + tid;
         const int sc = c < n ? score[c] : -1;
@@ -505,11 +538,13 @@ __global__ void __launch_bounds__(kRetThreads) l3_retrieve_kernel(const L3Retrie
         const int gt_before = round_gt + (v & 0xffff) + __popc(gt & below), eq_before = round_eq + (v >> 16) + __popc(eq & below);
         if (sc > lo || eq_before < at_cut) out[gt_before + (eq_before < at_cut ? eq_before : at_cut)] = bank[c];   // bank (time) order
     }
-    for (int i = k + tid; i < p.R; i += kRetThreads) out[i] = 0;
-    if (tid == 0 && kvh == 0) {
+    if (rank == 0)
+        for (int i = k + tid; i < p.R; i += kRetThreads) out[i] = 0;
+    if (tid == 0 && kvh == 0 && rank == 0) {
         if (p.n_sel) p.n_sel[b] = k;
         if (p.rows) p.rows[b] = k * p.page_rows;
     }
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
 // Which form of the index kernel.  The one with projecting warps of its own wins where projections are a good part of the work and
@@ -560,8 +595,12 @@ cudaError_t launch_l3_retrieve(const void* q, int B, int H, int H_kv, int d, con
     p.q = static_cast<const __nv_bfloat16*>(q); p.proj = proj; p.codes = codes; p.bank = bank; p.bank_len = bank_len;
     p.table = table; p.n_sel = n_sel; p.rows = rows; p.bank_stride = bank_stride;
     p.B = B; p.H = H; p.H_kv = H_kv; p.d = d; p.bits = bits; p.R = R; p.page_rows = page_rows; p.max_bank = max_bank;
-    size_t smem = ((size_t)max_bank + 7) / 8 * 8 * sizeof(unsigned short) +
-                  ((size_t)max_bank + kRetThreads - 1) / kRetThreads * kRetWarps * sizeof(int) + 16;
+    // CTAs of a cluster: a bank of a few thousand chunks is spread until a CTA has about a thousand, while all CTAs fit the chip at once
+    int size = 1;
+    while (size < kRetMaxCluster && size * 1024 < max_bank && (long long)B * H_kv * size * 2 <= 148) size *= 2;
+    p.per_cta = ((max_bank + size - 1) / size + 31) / 32 * 32;
+    size_t smem = ((size_t)p.per_cta + 7) / 8 * 8 * sizeof(unsigned short) +
+                  ((size_t)p.per_cta + kRetThreads - 1) / kRetThreads * kRetWarps * sizeof(int) + 16;
     const size_t with_proj = smem + (size_t)bits * (d + 4) * sizeof(float);
     const uintptr_t at = reinterpret_cast<uintptr_t>(codes);
     p.code_vec = bits >= 128 && at % 16 == 0 ? 4 : (bits == 64 && at % 8 == 0 ? 2 : 1);
@@ -569,7 +608,7 @@ cudaError_t launch_l3_retrieve(const void* q, int B, int H, int H_kv, int d, con
     if (p.stage_proj) smem = with_proj;
     cudaError_t e = cudaFuncSetAttribute(l3_retrieve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    return launch_chained(l3_retrieve_kernel, dim3((unsigned)(B * H_kv)), dim3(kRetThreads), smem, st, 0, p);
+    return launch_chained(l3_retrieve_kernel, dim3((unsigned)(B * H_kv * size)), dim3(kRetThreads), smem, st, size, p);
 }
 
 }  // namespace mka
