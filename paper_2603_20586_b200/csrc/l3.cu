@@ -12,10 +12,18 @@
 namespace mka {
 namespace {
 
-constexpr int kIdxThreads = 128;
+constexpr int kIdxThreads = 128;                      // threads that project; the two-phase form: all threads
 constexpr int kIdxPairs = 64;                         // (page, head) pairs per batch of a CTA: two per lane in the projections
 constexpr int kPhasePairs = 32;                       // the same in the two-phase form: one per lane
 constexpr int kIdxBitsPerWarp = 16;                   // code bits one warp works out per pass
+
+// 16 bytes that nobody reads again: they leave the L1 to the loads in flight (109 us with plain loads in the form for large pools; the
+// other forms, whose pools may still lie in the L2 cache, gain nothing).
+__device__ __forceinline__ uint4 ld_once(const void* p) {
+    uint4 v;
+    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
 
 struct L3IndexParams {
     const __nv_bfloat16* k;
@@ -27,39 +35,41 @@ struct L3IndexParams {
 
 // Dynamic shared memory: projT [d][bits + 4] floats (16 consecutive bits of one column are four broadcast reads), then two
 // buffers s [kIdxPairs][d + 1] floats (the key sums; the odd pitch keeps the lanes of a warp on different banks).
-// A batch = 64 (page, head) pairs.  The first four warps load: 16 threads cover one 256-byte row, a thread sums its eight
-// columns row by row, with up to 24 loads in flight across items and batches.  The other four project: lane = two pairs,
-// warp = 16 bits; column i costs two reads of s, four broadcast reads of projT and 32 fmaf.  The two halves work on different batches,
+// A batch = 64 (page, head) pairs.  The first LOADERS threads load: 16 of them cover one 256-byte row, a thread sums its eight
+// columns row by row, with up to 24 (512 loaders: 16) loads in flight across items and batches.  Four more warps project: lane = two pairs,
+// warp = 16 bits; column i costs two reads of s, four broadcast reads of projT and 32 fmaf.  The two sides work on different batches,
 // so the loads of one run under the projections of the other.  As two phases of the same warps, and with one pair to a
 // lane, the shared-memory pipe was busy for 78 us and HBM idle half of the time: 147 us (3.6 TB/s) for [32769 pages, 4 heads, 16
-// rows, 128] at 64 bits, 123 us now (4.4 TB/s).  Registers are moved from the projecting to the loading warps.
-template <int DH>
-__global__ void __launch_bounds__(2 * kIdxThreads, 2) l3_index_kernel(const L3IndexParams p) {
+// rows, 128] at 64 bits, 123 us with four loading warps in each of two CTAs (registers moved to them from the projecting ones);
+// sixteen in one CTA: see many_loaders.
+template <int DH, int LOADERS>
+__global__ void __launch_bounds__(LOADERS + kIdxThreads, LOADERS == 128 ? 2 : 1) l3_index_kernel(const L3IndexParams p) {
     chain_enter();
     extern __shared__ __align__(16) float sm[];
     const int ppitch = p.bits + 4;                             // floats between columns of projT (keeps the fill off one bank)
     constexpr int pitch = DH + 1, kSumFloats = kIdxPairs * pitch;
     float* projT = sm;
     float* sums = sm + (size_t)DH * ppitch;
-    const int tid = threadIdx.x & (kIdxThreads - 1), lane = tid & 31, warp = tid >> 5;
-    for (int e = threadIdx.x; e < DH * p.bits; e += 2 * kIdxThreads) {     // e = j * d + i: coalesced reads of proj
+    const bool loads = threadIdx.x < LOADERS;
+    const int tid = loads ? threadIdx.x : threadIdx.x - LOADERS, lane = tid & 31, warp = tid >> 5;
+    for (int e = threadIdx.x; e < DH * p.bits; e += LOADERS + kIdxThreads) {     // e = j * d + i: coalesced reads of proj
         const int j = e / DH, i = e % DH;
         projT[i * ppitch + j] = p.proj[e];
     }
     __syncthreads();
     constexpr int vecs = DH / 8;                               // 16-byte pieces of a row: 16 (d = 128) or 8 (d = 64)
-    constexpr int kPerThread = kIdxPairs * vecs / kIdxThreads; // (pair, piece) items of a thread in a batch: 8 or 4
-    constexpr int kSlotStep = kIdxThreads / vecs;              // pairs between a thread's items
+    constexpr int kPerThread = kIdxPairs * vecs / LOADERS; // (pair, piece) items of a thread in a batch: 8 or 4 (512 loaders: 2 or 1)
+    constexpr int kSlotStep = LOADERS / vecs;              // pairs between a thread's items
     const long long pairs = p.n_pages * p.H_kv;
     const int words = p.bits / 32;
     const long long step = (long long)gridDim.x * kIdxPairs, first = (long long)blockIdx.x * kIdxPairs;
-    // barriers 1, 2: buffer 0 / 1 is filled;  3, 4: it is free again (256 threads: one half arrives, the other waits)
-    auto arrive = [](int id) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(2 * kIdxThreads) : "memory"); };
-    auto wait = [](int id) { asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(2 * kIdxThreads) : "memory"); };
-    if (threadIdx.x < kIdxThreads) {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 152;");  // 256 threads x 128 registers at launch = 128 x 152 + 128 x 104
+    // barriers 1, 2: buffer 0 / 1 is filled;  3, 4: it is free again (one side arrives, the other waits)
+    auto arrive = [](int id) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(LOADERS + kIdxThreads) : "memory"); };
+    auto wait = [](int id) { asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(LOADERS + kIdxThreads) : "memory"); };
+    if (loads) {
+        if constexpr (LOADERS == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 152;");  // 256 threads x 128 registers at launch = 128 x 152 + 128 x 104
         const int slot0 = tid / vecs, piece = tid % vecs;
-        constexpr int kDepth = 3;
+        constexpr int kDepth = LOADERS == 128 ? 3 : 2;
         uint4 u[kDepth][8];
         // the next eight rows to ask for
         long long f_base = first;
@@ -74,16 +84,20 @@ __global__ void __launch_bounds__(2 * kIdxThreads, 2) l3_index_kernel(const L3In
             }
         };
         locate();
+        auto load = [](const __nv_bfloat16* src) {
+            if constexpr (LOADERS == 512) return ld_once(src);
+            else return __ldg(reinterpret_cast<const uint4*>(src));
+        };
         auto fetch = [&](uint4 (&to)[8]) {
             if (f_base >= pairs) return;
             if (f_src) {
                 if (f_row + 8 <= p.page_rows) {
 #pragma unroll
-                    for (int r = 0; r < 8; ++r) to[r] = __ldg(reinterpret_cast<const uint4*>(f_src + r * p.sn));
+                    for (int r = 0; r < 8; ++r) to[r] = load(f_src + r * p.sn);
                 } else {
 #pragma unroll
                     for (int r = 0; r < 8; ++r)
-                        if (f_row + r < p.page_rows) to[r] = __ldg(reinterpret_cast<const uint4*>(f_src + r * p.sn));
+                        if (f_row + r < p.page_rows) to[r] = load(f_src + r * p.sn);
                 }
                 f_src += 8 * p.sn;
             }
@@ -141,7 +155,7 @@ __global__ void __launch_bounds__(2 * kIdxThreads, 2) l3_index_kernel(const L3In
             }
         }
     } else {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
+        if constexpr (LOADERS == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
         unsigned short* codes16 = reinterpret_cast<unsigned short*>(p.codes);
         int n = 0;
         for (long long base = first; base < pairs; base += step, ++n) {
@@ -547,6 +561,19 @@ __global__ void __launch_bounds__(kRetThreads) l3_retrieve_kernel(const L3Retrie
     asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
+// Sixteen loading warps in a CTA that has its SM to itself, instead of eight in two CTAs: half of the warp cycles of the eight went
+// into the adds' latencies with their loads not yet asked for again (DRAM 53 % busy), and the two CTAs' copies of the projection take
+// the room of loads in flight.  The four projecting warps then serve twice the rows, so the form is for pools that come from
+// memory and for few code bits to a row.  Time of the better of the two other forms over its, 300 MB of keys, pages of 16 / 32 / 64 rows:
+//   d = 64    32 bits 1.04 / 1.09 / 1.02    64 bits 1.12 / 1.20 / 1.07    128 bits 0.88 / 1.26 / 1.18    256 bits 0.86 / 1.00 / 1.42
+//   d = 128           1.09 / 1.10 / 1.09            1.22 / 1.41 / 1.52             1.19 / 1.54 / 1.53             0.92 / 1.23 / 1.79
+//   pages of 8 rows 0.8 .. 0.9;  pools of 40 MB 0.7 .. 1.2, of 60 MB 0.91 .. 1.22, of 90 MB and more 1.02 .. 1.44 (32 bits: 0.8 .. 1.03)
+// [32769 pages, 4 heads, 16 rows, 128], 64 bits: 119.5 us before, 106 now (5.1 TB/s).
+bool many_loaders(const L3IndexParams& p) {
+    return p.page_rows >= 16 && p.bits <= (p.d == 128 ? 8 : 4) * p.page_rows &&
+           (double)p.n_pages * p.H_kv * p.page_rows * p.d * 2.0 >= (p.bits == 32 ? 200e6 : 80e6);
+}
+
 // Which form of the index kernel.  The one with projecting warps of its own wins where projections are a good part of the work and
 // there are batches enough for all SMs; where a key row carries few code bits (its projecting half idles; at 32 bits two of those four
 // warps never have work, at 128 bits and d = 128 one CTA fits an SM) and for small pools the two-phase form does.  Time of the
@@ -580,10 +607,12 @@ cudaError_t launch_l3_index(const void* k, long long n_pages, int H_kv, int page
         const long long per_cta = (batches + resident - 1) / resident, grid = (batches + per_cta - 1) / per_cta;
         return launch_chained(kern, dim3((unsigned)grid), dim3(threads), smem, st, 0, p);
     };
+    if (many_loaders(p))
+        return launch(d == 128 ? l3_index_kernel<128, 512> : l3_index_kernel<64, 512>, kIdxPairs, 2, 512 + kIdxThreads, [](size_t) { return 1; });
     if (two_phases(p))
         return launch(d == 128 ? l3_index_phases_kernel<128> : l3_index_phases_kernel<64>, kPhasePairs, 1, kIdxThreads,
                       [](size_t smem) { return smem > 110 * 1024 ? 1 : (smem > 72 * 1024 ? 2 : (smem > 54 * 1024 ? 3 : 4)); });
-    return launch(d == 128 ? l3_index_kernel<128> : l3_index_kernel<64>, kIdxPairs, 2, 2 * kIdxThreads,
+    return launch(d == 128 ? l3_index_kernel<128, 128> : l3_index_kernel<64, 128>, kIdxPairs, 2, 2 * kIdxThreads,
                   [](size_t smem) { return smem > 112 * 1024 ? 1 : 2; });
 }
 
