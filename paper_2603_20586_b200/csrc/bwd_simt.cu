@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
 }
 
 // One CTA = 16 or 32 key rows of one level of one (batch, KV head); its groups share the query tiles that see them.  One launch
-// covers the three levels: blockIdx.x runs through L1's, L2's and L3's key tiles.
+// covers the three levels: blockIdx.x runs through L3's, L2's and L1's key tiles, the longest walks first.
 template <typename T, int DH, int GROUPS>
 __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1) bwd_dkv_kernel(const BwdParams p, const int vec) {
     chain_enter();
@@ -188,9 +188,9 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
     float* tiles = ps + S::kThreads * 2 * R;     // [groups][Q, dO][32][LD]; at the end [groups][rows][2 DH]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = warp / S::kWarps, wg = warp % S::kWarps, gtid = threadIdx.x % kGroupThreads;
     const int b = blockIdx.z, h = blockIdx.y;               // h: KV head; its query heads h * G .. h * G + G - 1 are summed
-    int lvl = 0;
+    int lvl = 2;
     long long kt = blockIdx.x;
-    while (kt >= (p.L[lvl].n + kRows - 1) / kRows) { kt -= (p.L[lvl].n + kRows - 1) / kRows; ++lvl; }
+    while (kt >= (p.L[lvl].n + kRows - 1) / kRows) { kt -= (p.L[lvl].n + kRows - 1) / kRows; --lvl; }
     const LevelDev L = p.L[lvl];
     const LevelGradDev dL = p.dL[lvl];
     const long long j0 = kt * kRows;
@@ -361,7 +361,10 @@ cudaError_t launch_dkv(const BwdParams& p, int vec, cudaStream_t st) {
 template <typename T, int DH>
 cudaError_t launch_t(const BwdParams& p, cudaStream_t st) {
     const int vec = simt_vec_bits(p.L, p.Q, p.O, p.dO, sizeof(T) == 2 ? MKA_BF16 : MKA_F32);
-    cudaError_t e = simt_query_groups(p, 50.0) ? launch_dq<T, DH, 4>(p, vec, st) : launch_dq<T, DH, 1>(p, vec, st);
+    const int groups = simt_query_groups(p, 50.0);
+    cudaError_t e;
+    if constexpr (DH < 128) e = groups == 8 ? launch_dq<T, DH, 8>(p, vec, st) : (groups == 4 ? launch_dq<T, DH, 4>(p, vec, st) : launch_dq<T, DH, 1>(p, vec, st));
+    else e = groups == 4 ? launch_dq<T, DH, 4>(p, vec, st) : launch_dq<T, DH, 1>(p, vec, st);
     if (e == cudaSuccess) e = simt_key_groups(p) ? launch_dkv<T, DH, 4>(p, vec, st) : launch_dkv<T, DH, 1>(p, vec, st);
     return e == cudaSuccess ? launch_bwd_dgate(p.Gpart, p.B, p.H, p.T, p.dG, st) : e;
 }

@@ -13,9 +13,10 @@ namespace mka {
 
 constexpr int kSimtTile = 32, kSimtWarpRows = 4;
 
-// The two shapes of a CTA, by its number of groups: four groups of four warps (16 rows), or one group of eight (32 rows).
+// The shapes of a CTA, by its number of groups: eight groups of two warps (8 rows), four groups of four (16 rows), or one group of
+// eight (32 rows).
 template <int GROUPS> struct SimtCta {
-    static constexpr int kGroups = GROUPS, kWarps = GROUPS == 4 ? 4 : 8;      // kWarps: of a group
+    static constexpr int kGroups = GROUPS, kWarps = GROUPS == 8 ? 2 : (GROUPS == 4 ? 4 : 8);      // kWarps: of a group
     static constexpr int kRows = kWarps * kSimtWarpRows, kThreads = kGroups * kWarps * 32;
 };
 
@@ -76,13 +77,23 @@ inline int simt_vec_bits(const LevelDev L[3], const void* a, const void* b, cons
 //                      128 x 64, 512, 14                          86.1 / 63.5 (82.2)      8 x 1024, 512, 2     22.6 / 14.4 (18.5)
 //   forward, d = 128   32 x 200, 416, 8                           43.1 / 51.2
 inline bool simt_four_groups(long long blocks, double walk, double k) { return blocks <= 148 || (double)(blocks - 148) <= k * walk; }
-template <typename P> inline bool simt_query_groups(const P& p, double k) {           // forward and dQ: row blocks of queries
+template <typename P> inline double simt_query_walk(const P& p) {                     // forward and dQ: row blocks of queries
     double keys = 0.0;
     for (int l = 0; l < 3; ++l) {
         const double n = (double)p.L[l].n, seen = l == 0 ? (double)p.window + 15.0 : (l == 1 ? (double)p.q_offset + 0.5 * p.T : n);
         keys += n > 0.0 ? 32.0 + (seen < n ? seen : n) : 0.0;
     }
-    return simt_four_groups((long long)p.B * p.H * ((p.T + 15) / 16), keys / 32.0, k);
+    return keys / 32.0;
+}
+template <typename P> inline int simt_query_groups(const P& p, double k) {
+    const long long blocks = (long long)p.B * p.H * ((p.T + 15) / 16);
+    const double walk = simt_query_walk(p);
+    // Half as many rows to a CTA where even twice the blocks find an SM each and every group still has a tile: an SM's shared-memory
+    // reads, which bound a step of the walk, are the same, but a step covers eight tiles.  [1, 4, 256, 64] (window 64, 128 slots): both
+    // forwards and the backward together 106 us in four groups, 94 in eight and with the longest key blocks of dK/dV first (clusters of
+    // two to four CTAs of four groups instead: 118).
+    if (p.d < 128 && blocks * 2 <= 148 && walk >= 8.0) return 8;
+    return simt_four_groups(blocks, walk, k) ? 4 : 1;
 }
 // dK/dV: the levels' key blocks walk very different numbers of query tiles, and a launch lasts at least as long as its longest walk
 // (a long-term level of 64 rows under 8192 queries beside a window of 16: 603 / 1434 us), so that walk counts here, also against
