@@ -12,6 +12,12 @@ from typing import Optional, Sequence
 
 import torch
 
+try:
+    from . import _host_args
+except ImportError as e:
+    raise ImportError("the binding's host module is missing: build it with `python -m paper_2603_20586_b200.build` "
+                      "(there is no fallback path)") from e
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libmka_b200.so")
 
@@ -88,7 +94,7 @@ def _load() -> ctypes.CDLL:
     lib.mka_fwd_scratch_bytes.argtypes = [ctypes.POINTER(mka_shape), i32, ctypes.POINTER(ctypes.c_int64)]
     lib.mka_fwd_with_scratch.argtypes = [ctypes.POINTER(mka_shape), vp, vp, vp, vp, vp, vp, ctypes.c_size_t, vp, ctypes.c_size_t, vp]
     lib.mka_bwd.argtypes = [ctypes.POINTER(mka_shape), vp, vp, vp, vp, vp, vp, vp, i32, vp,
-                            ctypes.POINTER(mka_level_grad), vp, vp, vp, vp, ctypes.c_size_t, vp]
+                            vp, vp, vp, vp, vp, ctypes.c_size_t, vp]
     lib.mka_decode_plan.argtypes = [ctypes.POINTER(ctypes.c_int64), i32, i32, i32, ctypes.POINTER(mka_decode_plan_t)]
     lib.mka_fwd_tile_range.argtypes = [ctypes.POINTER(mka_shape), ctypes.POINTER(ctypes.c_int64), i32, i64,
                                        ctypes.POINTER(mka_tile_range)]
@@ -106,8 +112,7 @@ def _load() -> ctypes.CDLL:
                                      ctypes.c_size_t, vp]
     lib.mka_fwd_paged.argtypes = lib.mka_decode_paged.argtypes
     lib.mka_fwd_paged_with_scratch.argtypes = [ctypes.POINTER(mka_shape), i32, vp, vp, vp, vp, vp, vp, ctypes.c_size_t, vp, ctypes.c_size_t, vp]
-    lib.mka_fuse_kv_paged.argtypes = [i32, i32, i64, i32, i32, vp, vp, ctypes.POINTER(mka_paged_level), i64,
-                                      vp, vp]
+    lib.mka_fuse_kv_paged.argtypes = [i32, i32, i64, i32, i32, vp, vp, vp, i64, vp, vp]
     lib.mka_l3_index.argtypes = [vp, i64, i32, i32, i32, i64, i64, i64, vp, i32, vp, vp]
     lib.mka_l3_retrieve.argtypes = [vp, i32, i32, i32, i32, vp, i32, vp, vp, vp, i64, i32, i32, i32, vp, vp, vp, vp]
     lib.mka_l2_summary_kernel_kind.argtypes = [i32, i64, i32, i32, ctypes.c_size_t]
@@ -143,14 +148,14 @@ def _dt(t: torch.Tensor) -> int:
 
 
 # A small call (one decode step, a short prompt) is over sooner on the GPU than its arguments used to be marshalled here, so
-# pointers travel as plain ints, a call's levels as one array of 64-bit words (both are what the declared argument types and
-# the struct layouts say), and the current stream is asked for without building a Stream object.
+# pointers travel as plain ints, a call's levels as one array of 64-bit words that native code fills in (both are what the
+# declared argument types and the struct layouts say), and the current stream is asked for without building a Stream object.
 def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else t.data_ptr()
 
 
 def _stream(stream) -> int:
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()) if stream is None else stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) if stream is None else stream.cuda_stream
 
 
 def _n_level(n) -> ctypes.Array:
@@ -163,23 +168,10 @@ def make_shape(B, H, T, d, D=0, window=1, q_offset=0, scale=0.0, dtype=MKA_BF16,
 
 
 _Rows = ctypes.c_int64 * 3
-_LevelWords = ctypes.c_int64 * 18        # mka_level[3]: k, v, n, stride_b, stride_h, stride_n
-_PagedWords = ctypes.c_int64 * 36        # mka_paged_level[3]: twelve 8-byte slots each (page_rows is the low half of its own)
-_NO_LEVEL = (0,) * 6
-_NO_PAGED_LEVEL = (0,) * 7 + (1, 0, 0, 0, 0)
-
-
-def _levels(K: Sequence[Optional[torch.Tensor]], V: Sequence[Optional[torch.Tensor]]):
-    words = ()
-    for l in range(3):
-        k, v = K[l], V[l]
-        if k is None or k.shape[2] == 0:
-            words += _NO_LEVEL
-            continue
-        shape, stride = k.shape, k.stride()
-        assert len(shape) == 4 and stride[3] == 1 and v.stride() == stride and v.shape == shape
-        words += (k.data_ptr(), v.data_ptr(), shape[2]) + stride[:3]
-    return _LevelWords(*words)
+_levels = _host_args.levels                # (K, V) -> mka_level[3] as bytes; None or no rows: an absent level
+_paged_levels = _host_args.paged_levels    # (pools_k, pools_v, tables, rows or None, n) -> mka_paged_level[3] as bytes; pools
+                                           # [pages, H_kv, page_rows, d], any strides with d contiguous; tables [B, pages] or [B, H_kv, pages]
+_empty_f32 = _host_args.empty_f32          # (t, keep, extra) -> fp32 tensor of t's first `keep` dimensions (and `extra`)
 
 
 def mka_workspace_bytes(shape: mka_shape, n_level, which: int) -> int:
@@ -206,9 +198,8 @@ def mka_router(R: torch.Tensor, W_r: torch.Tensor, b_r: Optional[torch.Tensor], 
     D = R.shape[-1]
     rows = R.numel() // D if D else 0
     assert R.is_contiguous() and W_r.is_contiguous() and W_r.dtype == torch.float32 and W_r.shape == (D, 3)
-    lead = tuple(R.shape[:-1])
     if gate is None:
-        gate = torch.empty(lead + (3,), dtype=torch.float32, device=R.device)
+        gate = _empty_f32(R, R.dim() - 1, 3)
     _check(lib.mka_router(_ptr(R), _ptr(W_r), _ptr(b_r), rows, D, _dt(R), route, _ptr(gate), _ptr(log2_gate),
                           _ptr(route_idx), _stream(stream)), "mka_router")
     return gate
@@ -235,7 +226,7 @@ def mka_fwd(shape: mka_shape, Q, K, V, gate, O=None, LSE=None, ws=None, stream=N
     if O is None:
         O = torch.empty_like(Q)
     if LSE is None and want_lse and shape.mode == MKA_MODE_FAST:
-        LSE = torch.empty(Q.shape[:3], dtype=torch.float32, device=Q.device)
+        LSE = _empty_f32(Q, 3, 0)
     n = [0 if k is None else k.shape[2] for k in K]
     if ws is None:
         ws = alloc_workspace(shape, n, MKA_WS_FWD, Q.device)
@@ -250,33 +241,12 @@ def mka_decode(shape: mka_shape, q, K, V, gate, O=None, LSE=None, ws=None, strea
     if O is None:
         O = torch.empty_like(q)
     if LSE is None:
-        LSE = torch.empty(q.shape[:2], dtype=torch.float32, device=q.device)
+        LSE = _empty_f32(q, 2, 0)
     if ws is None:
         ws = alloc_workspace(shape, [0 if k is None else k.shape[2] for k in K], MKA_WS_DECODE, q.device)
     _check(lib.mka_decode(ctypes.byref(shape), _ptr(q), _levels(K, V), _ptr(gate), _ptr(O), _ptr(LSE), _ptr(ws),
                           ws.numel(), _stream(stream)), "mka_decode")
     return O, LSE
-
-
-def _paged_levels(pools_k, pools_v, tables, rows, n):
-    words = ()
-    for l in range(3):
-        k, v = pools_k[l], pools_v[l]
-        if k is None or n[l] == 0:
-            words += _NO_PAGED_LEVEL
-            continue
-        # pools [pages, H_kv, page_rows, d]; any strides with d contiguous
-        shape, stride = k.shape, k.stride()
-        assert len(shape) == 4 and stride[3] == 1 and v.stride() == stride and v.shape == shape
-        tab = tables[l]
-        # [B, pages]: one table per sequence; [B, H_kv, pages]: one per (sequence, KV head)
-        ts = tab.stride()
-        assert tab.dtype == torch.int32 and len(ts) in (2, 3) and ts[-1] == 1
-        r = None if rows is None else rows[l]
-        assert r is None or (r.dtype == torch.int32 and r.is_contiguous())
-        words += (k.data_ptr(), v.data_ptr(), tab.data_ptr(), 0 if r is None else r.data_ptr(), int(n[l]), ts[0],
-                  ts[1] if len(ts) == 3 else 0, shape[2]) + stride[:3] + (shape[0],)
-    return _PagedWords(*words)
 
 
 def mka_fuse_kv_paged(K, V, gate, pool_k, pool_v, table, dst_offset=0, dst_offsets=None, stream=None):
@@ -286,12 +256,10 @@ def mka_fuse_kv_paged(K, V, gate, pool_k, pool_v, table, dst_offset=0, dst_offse
     ref = next(k for k in K if k is not None)
     B, H, n, d = ref.shape
     assert gate.is_contiguous() and gate.dtype == torch.float32 and tuple(gate.shape) == (B, n, 3)
-    assert pool_k.dim() == 4 and pool_k.stride(3) == 1 and pool_v.stride() == pool_k.stride() and pool_k.dtype == ref.dtype
-    assert table.dtype == torch.int32 and table.dim() == 2 and table.stride(1) == 1
+    assert pool_k.dtype == ref.dtype
     assert dst_offsets is None or (dst_offsets.dtype == torch.int32 and dst_offsets.is_contiguous())
-    dst = mka_paged_level(pool_k.data_ptr(), pool_v.data_ptr(), table.data_ptr(), None, table.shape[1] * pool_k.shape[2],
-                          table.stride(0), 0, pool_k.shape[2], pool_k.stride(0), pool_k.stride(1), pool_k.stride(2), pool_k.shape[0])
-    _check(lib.mka_fuse_kv_paged(B, H, n, d, _dt(ref), _levels(K, V), _ptr(gate), ctypes.byref(dst), dst_offset, _ptr(dst_offsets),
+    _check(lib.mka_fuse_kv_paged(B, H, n, d, _dt(ref), _levels(K, V), _ptr(gate), _host_args.paged_level(pool_k, pool_v, table), dst_offset,
+                                 _ptr(dst_offsets),
                                  _stream(stream)), "mka_fuse_kv_paged")
     return pool_k, pool_v
 
@@ -305,7 +273,7 @@ def mka_fwd_paged(shape: mka_shape, H_kv: int, Q, pools_k, pools_v, tables, n, g
     if O is None:
         O = torch.empty_like(Q)
     if LSE is None:
-        LSE = torch.empty(B, H, T, dtype=torch.float32, device=Q.device)
+        LSE = _empty_f32(Q, 3, 0)
     if ws is None:
         ws = torch.zeros(256, dtype=torch.uint8, device=Q.device)
     tmp = _fwd_scratch(shape, H_kv, _n_level(n), Q.device) if stream is None and (rows is None or not any(r is not None for r in rows)) else None
@@ -327,7 +295,7 @@ def mka_decode_paged(shape: mka_shape, H_kv: int, q, pools_k, pools_v, tables, n
     if O is None:
         O = torch.empty_like(q)
     if LSE is None:
-        LSE = torch.empty(q.shape[:2], dtype=torch.float32, device=q.device)
+        LSE = _empty_f32(q, 2, 0)
     if ws is None:
         ws = torch.empty(mka_decode_paged_workspace_bytes(shape, H_kv, n), dtype=torch.uint8, device=q.device)
     _check(lib.mka_decode_paged(ctypes.byref(shape), H_kv, _ptr(q), _paged_levels(pools_k, pools_v, tables, rows, n),
@@ -388,25 +356,18 @@ def mka_bwd(shape: mka_shape, Q, K, V, gate, O, LSE, dO, R=None, dQ=None, dK=Non
     if dQ is None:
         dQ = torch.empty_like(Q)
     if dK is None:
-        dK = [None if k is None else torch.empty_like(k) for k in K]
+        dK = _host_args.empties_like(K)
     if dV is None:
-        dV = [None if v is None else torch.empty_like(v) for v in V]
+        dV = _host_args.empties_like(V)
     if dG is None:
-        dG = torch.empty(gate.shape, dtype=torch.float32, device=dev)
+        dG = _empty_f32(gate, gate.dim(), 0)
     if R is not None and want_router_grad:
         assert R.is_contiguous()
         if dW_r is None:
             dW_r = torch.empty((R.shape[-1], 3), dtype=torch.float32, device=dev)
         if db_r is None:
             db_r = torch.empty((3,), dtype=torch.float32, device=dev)
-    grads = (mka_level_grad * 3)()
-    for l in range(3):
-        if K[l] is None or K[l].shape[2] == 0:
-            grads[l] = mka_level_grad(None, None, 0, 0, 0, 0)
-        else:
-            g = dK[l]
-            assert g.stride(3) == 1 and dV[l].stride() == g.stride()
-            grads[l] = mka_level_grad(g.data_ptr(), dV[l].data_ptr(), g.shape[2], g.stride(0), g.stride(1), g.stride(2))
+    grads = _host_args.grads([None if K[l] is None or K[l].shape[2] == 0 else dK[l] for l in range(3)], dV)
     if ws is None:
         ws = alloc_workspace(shape, [0 if k is None else k.shape[2] for k in K], MKA_WS_BWD, dev)
     _check(lib.mka_bwd(ctypes.byref(shape), _ptr(Q), _levels(K, V), _ptr(gate), _ptr(O), _ptr(LSE), _ptr(dO),

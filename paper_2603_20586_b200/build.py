@@ -17,6 +17,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmka_b200.so")
+HOST_SRC, HOST_MODULE = os.path.join(CSRC, "host_args.cpp"), os.path.join(HERE, "_host_args.so")
 OBJ_DIR = os.path.join(HERE, "_build")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -35,6 +36,21 @@ def _stale(target, deps):
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _host_module_cmd(out):
+    """The binding's argument marshalling (host only): a Python module against the installed torch."""
+    import sysconfig
+
+    import torch
+    from torch.utils.cpp_extension import include_paths, library_paths
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I", sysconfig.get_paths()["include"]]
+    for path in include_paths():
+        cmd += ["-isystem", path]
+    for path in library_paths():
+        cmd += ["-L", path]
+    return cmd + [HOST_SRC, "-o", out, "-lc10", "-ltorch_cpu", "-ltorch_python"]
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     headers = glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
     os.makedirs(OBJ_DIR, exist_ok=True)
@@ -51,7 +67,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         if verbose or r.returncode:
             sys.stderr.write(r.stdout + r.stderr)
         if r.returncode:
-            raise RuntimeError("nvcc failed: " + " ".join(cmd))
+            raise RuntimeError("build failed: " + " ".join(cmd))
 
     with ThreadPoolExecutor(max_workers=min(8, max(1, len(jobs)))) as ex:
         list(ex.map(run, jobs))
@@ -59,6 +75,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
         tmp = LIB + f".{os.getpid()}.tmp"
         run([NVCC, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", tmp] + objs + ["-cudart", "static"])
         os.replace(tmp, LIB)
+    if force or _stale(HOST_MODULE, [HOST_SRC]):
+        tmp = HOST_MODULE + f".{os.getpid()}.tmp"
+        run(_host_module_cmd(tmp))
+        os.replace(tmp, HOST_MODULE)
     return LIB
 
 
