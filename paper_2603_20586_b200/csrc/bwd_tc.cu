@@ -202,7 +202,9 @@ template <int kWarps> __device__ __forceinline__ bool softmax_group_all(bool fla
 // D = dO . O and the three exponent biases of every padded row.  DH / 8 lanes share a row (one 16-byte load of O and
 // one of dO each), a warp covers 2 or 4 rows per pass and a thread works on four passes at once, so eight loads are
 // in flight per thread; the row's LSE and gate are fetched with them.  blockIdx.y is the (batch, head): with the row split
-// by 64-bit divisions the arithmetic took most of the time (2.5 TB/s).  Padding rows (t >= T) get a bias of -inf so
+// by 64-bit divisions the arithmetic took most of the time (2.5 TB/s).  Each lane finishes one row: with the row's first lane
+// loading and storing for it, two rows at a time, the pass took 82 us at [1, 32, 32768, 128] and 19 us at [8, 16, 2048, 64],
+// now 53 and 16 (62 registers before, 37 now).  Padding rows (t >= T) get a bias of -inf so
 // that a streamed sub-tile may run past the last query without a mask.
 template <int DH>
 __global__ void __launch_bounds__(256) bwd_prep_kernel(const __nv_bfloat16* __restrict__ O, const __nv_bfloat16* __restrict__ dO,
@@ -214,29 +216,30 @@ __global__ void __launch_bounds__(256) bwd_prep_kernel(const __nv_bfloat16* __re
     if (threadIdx.x < 4 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) header[threadIdx.x] = 0u;   // status word and tickets of the kernels that follow
     constexpr int LPR = DH / 8;                            // lanes per row: 16 or 8
     constexpr int RPW = 32 / LPR;                          // rows per warp and pass
-    constexpr int kPasses = 4;
+    constexpr int kPasses = 4, kRows = RPW * kPasses;      // rows of a warp: 8 or 16
     const int lane = threadIdx.x & 31, sub = lane % LPR, grp = lane / LPR;
     const long long bh = (long long)blockIdx.z * H + blockIdx.y;
-    const int row0 = (blockIdx.x * 8 + (threadIdx.x >> 5)) * (RPW * kPasses) + grp;
+    const int row0 = (blockIdx.x * 8 + (threadIdx.x >> 5)) * kRows;
     const __nv_bfloat16* Ob = O + bh * T * DH + sub * 8;
     const __nv_bfloat16* dOb = dO + bh * T * DH + sub * 8;
     uint4 a[kPasses], g[kPasses];
-    float lse[kPasses], gt[kPasses][3];
 #pragma unroll
     for (int u = 0; u < kPasses; ++u) {
-        const int t = row0 + u * RPW;
+        const int t = row0 + u * RPW + grp;
         a[u] = g[u] = make_uint4(0u, 0u, 0u, 0u);
-        lse[u] = -INFINITY;
-        gt[u][0] = gt[u][1] = gt[u][2] = 0.f;
         if (t < T) {
             a[u] = __ldg(reinterpret_cast<const uint4*>(Ob + (long long)t * DH));
             g[u] = __ldg(reinterpret_cast<const uint4*>(dOb + (long long)t * DH));
-            if (sub == 0) {
-                lse[u] = LSE[bh * T + t];
-                const float* gr = gate + ((long long)blockIdx.z * T + t) * 3;
-                gt[u][0] = gr[0]; gt[u][1] = gr[1]; gt[u][2] = gr[2];
-            }
         }
+    }
+    // lane i < kRows finishes row i of the warp: its LSE and gate on the way in, its four values on the way out, are then
+    // consecutive in memory (by the row's first lane, pass by pass, they were 32 accesses of two rows each)
+    const int t_own = row0 + lane;
+    float lse = -INFINITY, gt[3] = {0.f, 0.f, 0.f}, own = 0.f;
+    if (lane < kRows && t_own < T) {
+        lse = LSE[bh * T + t_own];
+        const float* gr = gate + ((long long)blockIdx.z * T + t_own) * 3;
+        gt[0] = gr[0]; gt[1] = gr[1]; gt[2] = gr[2];
     }
 #pragma unroll
     for (int u = 0; u < kPasses; ++u) {
@@ -249,16 +252,17 @@ __global__ void __launch_bounds__(256) bwd_prep_kernel(const __nv_bfloat16* __re
         }
 #pragma unroll
         for (int o = LPR / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        const int t = row0 + u * RPW;
-        if (sub == 0 && t < Tpad) {
-            const bool live = lse[u] > -INFINITY;
-            const float l2 = lse[u] * kLog2e;
-            const long long at = bh * Tpad + t;
-            sD[at] = s;
-            b0[at] = (live && gt[u][0] > 0.f) ? log2f(gt[u][0]) - l2 : -INFINITY;
-            b1[at] = (live && gt[u][1] > 0.f) ? log2f(gt[u][1]) - l2 : -INFINITY;
-            b2[at] = (live && gt[u][2] > 0.f) ? log2f(gt[u][2]) - l2 : -INFINITY;
-        }
+        const float of_row = __shfl_sync(0xffffffffu, s, (lane % RPW) * LPR);
+        if (lane / RPW == u) own = of_row;
+    }
+    if (lane < kRows && t_own < Tpad) {
+        const bool live = lse > -INFINITY;
+        const float l2 = lse * kLog2e;
+        const long long at = bh * Tpad + t_own;
+        sD[at] = own;
+        b0[at] = (live && gt[0] > 0.f) ? log2f(gt[0]) - l2 : -INFINITY;
+        b1[at] = (live && gt[1] > 0.f) ? log2f(gt[1]) - l2 : -INFINITY;
+        b2[at] = (live && gt[2] > 0.f) ? log2f(gt[2]) - l2 : -INFINITY;
     }
 }
 
