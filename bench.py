@@ -216,7 +216,7 @@ class Leg:
             self.grads = {"dQ": torch.empty_like(self.t["Q"]), "dK": [torch.empty_like(k) for k in self.K],
                           "dV": [torch.empty_like(v) for v in self.V], "dG": torch.empty(B, T, 3, device=device),
                           "dW_r": torch.empty(D, 3, device=device), "db_r": torch.empty(3, device=device)}
-            self.launches_per_step = 1 + 1 + (1 + 1 + 1 + 1) + 2   # router, fwd, bwd(prep,dq,dkv,dgate), router bwd
+            self.launches_per_step = 1 + 1 + (1 + 1 + 1) + 2   # router, fwd, bwd(prep,dq,dkv), router bwd
             self.bwd_executed_ratio = 1.4           # the two-pass backward runs 14 d flops per pair for the method's 10 d
         else:
             self.launches_per_step = 2              # router, fwd

@@ -68,7 +68,8 @@ struct BwdTcParams {
     int H_kv;
     long long dkv_items;      // key tiles of all levels, KV heads and batches
     long long dq_items;       // query tiles of all heads and batches
-    unsigned int *dkv_ticket, *dq_ticket;   // zero at launch
+    unsigned int *dkv_ticket, *dq_ticket, *gate_ticket;   // zero at launch
+    float* dG;
     unsigned int* status;
     unsigned long long wait_limit_ns;
     int test_stall;           // test hook: the dK/dV kernel's loader leaves out the last query tile of every CTA
@@ -203,7 +204,7 @@ template <int kWarps> __device__ __forceinline__ bool softmax_group_all(bool fla
 // one of dO each), a warp covers 2 or 4 rows per pass and a thread works on four passes at once, so eight loads are
 // in flight per thread; the row's LSE and gate are fetched with them.  blockIdx.y is the (batch, head): with the row split
 // by 64-bit divisions the arithmetic took most of the time (2.5 TB/s).  Each lane finishes one row: with the row's first lane
-// loading and storing for it, two rows at a time, the pass took 82 us at [1, 32, 32768, 128] and 19 us at [8, 16, 2048, 64],
+// loading and storing for it, two rows at a time, the pass took 82 us at [4, 16, 8192, 128] and 19 us at [8, 16, 2048, 64],
 // now 53 and 16 (62 registers before, 37 now).  Padding rows (t >= T) get a bias of -inf so
 // that a streamed sub-tile may run past the last query without a mask.
 template <int DH>
@@ -724,6 +725,7 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
     __shared__ uint32_t tmem_base_slot;
     __shared__ WaitCtl wait_ctl;
     __shared__ DkvItem items[2];
+    __shared__ unsigned int gate_chunk;
 
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // tid >> 5, but provably warp-uniform for the compiler
@@ -822,6 +824,7 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
             mbar_drain(&bar.a_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp, t_drain);
         for (int i = issued_b > C::kStages ? issued_b - C::kStages : 0; i < issued_b; ++i)
             mbar_drain(&bar.b_full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, abortp, t_drain);
+        if (lane == 0) gate_chunk = atomicAdd(p.gate_ticket, 1u);
     } else if (warp == C::kSlabWarp || warp == C::kSlabWarp + 1) {
         // The operand slabs of the ninth K-step: the first of these warps writes the bias slabs (ring of the Q tiles), the second
         // the D slabs (ring of the dO tiles), four queries a lane, fetched one tile ahead.  Warps of their own: when the
@@ -1137,6 +1140,18 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
     __syncthreads();
     if (tid == 0 && wait_ctl.abort) atomicExch(p.status, (unsigned int)MKA_ERR_TIMEOUT);
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+    // The gate gradient's sums over the heads, left to the CTAs that are done with their key tiles first: a ticket is a sum per
+    // thread, the first one taken under the epilogue.  As a launch behind this one they took 5 us: a step at [2, 16 on 4, 1000, 128] 140.7 -> 138.0 us,
+    // at [1, 8, 700, 128] 60.0 -> 57.6.
+    const long long per_batch = p.T * 3LL;
+    for (;;) {
+        const long long at = (long long)gate_chunk * C::kThreadsDkv + tid;
+        if (at - tid >= per_batch * p.B) break;
+        if (at < per_batch * p.B) sum_dgate(p.Gpart, p.dG, p.H, p.T, at / per_batch, at % per_batch);
+        __syncthreads();
+        if (tid == 0) gate_chunk = atomicAdd(p.gate_ticket, 1u);
+        __syncthreads();
+    }
 }
 
 template <int DH>
@@ -1208,8 +1223,11 @@ cudaError_t launch_t(const BwdParams& bp, unsigned int* status_word, cudaStream_
         if (e != cudaSuccess) return e;
         p.dkv_items = (long long)tiles * H_kv * bp.B;
         p.dkv_ticket = status_word + 1;
-        e = launch_chained(bwd_dkv_tc_kernel<DH>, dim3((unsigned)(p.dkv_items < 148 ? p.dkv_items : 148)), dim3(C::kThreadsDkv), C::kSmemDkv, st, 0, m, p);
-        if (e != cudaSuccess) return e;
+        p.gate_ticket = status_word + 3;
+        p.dG = bp.dG;
+        const long long ctas = p.dkv_items + ((long long)p.B * p.T * 3 + C::kThreadsDkv - 1) / C::kThreadsDkv;   // key tiles and sums of dG
+        e = launch_chained(bwd_dkv_tc_kernel<DH>, dim3((unsigned)(ctas < 148 ? ctas : 148)), dim3(C::kThreadsDkv), C::kSmemDkv, st, 0, m, p);
+        return e;
     }
     return launch_bwd_dgate(bp.Gpart, bp.B, bp.H, bp.T, bp.dG, st);
 }

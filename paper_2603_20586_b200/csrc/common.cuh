@@ -200,6 +200,13 @@ size_t l2_summary_seg_workspace(int B, long long T, int D, int dtype);
 cudaError_t launch_l2_summary_seg(const void* X, void* M2, float* state, int use_state, long long n_prev, int B, long long T,
                                   int D, int dtype, int kind, float beta, unsigned int* status, void* scratch, cudaStream_t st);
 cudaError_t launch_bwd_dgate(const float* Gpart, int B, int H, long long T, float* dG, cudaStream_t st);
+// dG[b,t,l] = sum_h G[b,h,t,l], added up in the order of the heads; at = t * 3 + l.
+__device__ __forceinline__ void sum_dgate(const float* Gpart, float* dG, int H, long long T, long long b, long long at) {
+    float s = 0.f;
+#pragma unroll 8
+    for (int h = 0; h < H; ++h) s += __ldcg(Gpart + (b * H + h) * T * 3 + at);
+    dG[b * T * 3 + at] = s;
+}
 // Tensor-core (TMA + tcgen05) backward; same contract as the forward below.
 cudaError_t launch_bwd_tc(const BwdParams& p, unsigned int* status_word, cudaStream_t st);
 bool bwd_tc_eligible(const BwdParams& p, int dtype);

@@ -1,0 +1,50 @@
+"""Gate gradient summed over the heads beside dK and dV: more sums than the CTAs of the key tiles take in one round, a remainder of a
+round, one key tile under many queries, and a short level alone."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_helpers import F32_MAX, err, np64, problem
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mka():
+    import paper_2603_20586_b200 as m
+    assert torch.cuda.is_available()
+    return m
+
+
+# B, H, T, d, window, rows of the three levels
+TC = [(1, 3, 40000, 64, 16, (0, 0, 20)), (2, 5, 300, 128, 32, (300, 300, 130)), (1, 32, 1000, 128, 256, (1000, 0, 7)), (3, 2, 129, 64, 129, (129, 129, 0))]
+
+
+@pytest.mark.parametrize("case", TC, ids=lambda c: f"T{c[2]}H{c[1]}d{c[3]}")
+def test_tensor_core_sums_are_those_of_single_heads(mka, case):
+    B, H, T, d, W, N = case
+    P = problem(71, B, H, T, d, N, 64, torch.bfloat16, router_std=0.3, with_dO=True)
+    gate = mka.mka_router(P["X"], P["W_r"], None)
+    K, V = P["K"], P["V"]
+    shape, single = (mka.make_shape(B, n, T, d, 64, W) for n in (H, 1))
+    O, LSE = mka.mka_fwd(shape, P["Q"], K, V, gate)
+    got = mka.mka_bwd(shape, P["Q"], K, V, gate, O, LSE, P["dO"])["dG"]
+    want = torch.zeros_like(got)
+    for h in range(H):
+        one = lambda t: t[:, h:h + 1].contiguous()
+        want += mka.mka_bwd(single, one(P["Q"]), [one(k) for k in K], [one(v) for v in V], gate, one(O), one(LSE), one(P["dO"]))["dG"]
+    assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("case", [(2, 3, 171, 32, 40, (171, 171, 5)), (1, 1, 700, 96, 9, (0, 0, 3)), (3, 7, 1, 64, 1, (1, 1, 40))], ids=lambda c: f"T{c[2]}H{c[1]}")
+def test_cuda_core_sums_match_the_oracle(mka, orc, case):
+    B, H, T, d, W, N = case
+    P = problem(72, B, H, T, d, N, 32, torch.float32, router_std=0.3, with_dO=True)
+    gate = mka.mka_router(P["X"], P["W_r"], None)
+    shape = mka.make_shape(B, H, T, d, 32, W, dtype=mka.binding.MKA_F32)
+    O, LSE = mka.mka_fwd(shape, P["Q"], P["K"], P["V"], gate)
+    got = mka.mka_bwd(shape, P["Q"], P["K"], P["V"], gate, O, LSE, P["dO"])["dG"]
+    rg, _ = orc.router(np64(P["X"]), np64(P["W_r"]))
+    want = orc.bwd(P["Q"], P["K"], P["V"], rg, P["dO"], W)["dG"]
+    # sums of up to T terms and H heads: the contract's bound grows with the largest of them
+    assert err(got, want)[0] <= F32_MAX * max(1.0, np.abs(want).max())
