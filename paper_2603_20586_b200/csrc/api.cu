@@ -66,6 +66,21 @@ void fill_levels(LevelDev out[3], const mka_level L[3]) {
 
 constexpr int kRouterBwdChunks = 128;
 
+// Bytes [lo, hi) that a call reads or writes, for telling a caller that writes a result over an operand.
+struct Span {
+    uintptr_t lo, hi;
+    bool meets(const Span& o) const { return lo < hi && o.lo < o.hi && lo < o.hi && o.lo < hi; }
+    bool meets(const void* x, size_t bytes) const { const uintptr_t at = reinterpret_cast<uintptr_t>(x); return meets(Span{at, at + bytes}); }
+};
+template <typename Level>
+Span level_span(const void* x, const Level& L, const BwdParams& p, size_t elem) {
+    if (L.n <= 0 || !x || p.B <= 0 || p.H <= 0) return {0, 0};
+    const long long steps[3] = {(p.B - 1) * L.sb, (p.H / (p.kv_group > 0 ? p.kv_group : 1) - 1) * L.sh, (L.n - 1) * L.sn};
+    Span r = {reinterpret_cast<uintptr_t>(x), reinterpret_cast<uintptr_t>(x) + p.d * elem};
+    for (const long long step : steps) (step < 0 ? r.lo : r.hi) += step * (long long)elem;
+    return r;
+}
+
 // Per-row statistics of the tensor-core backward: three arrays of [B, H, Tpad] float2, Tpad = T rounded up to 128.
 size_t bwd_stats_bytes(const mka_shape* s) {
     const size_t tpad = ((size_t)s->T + 127) / 128 * 128;
@@ -552,6 +567,12 @@ mka_status mka_bwd(const mka_shape* s, const void* Q, const mka_level L[3], cons
     p.B = s->B; p.H = s->H; p.T = s->T; p.d = s->d;
     p.window = s->window; p.q_offset = s->q_offset; p.scale = resolve_scale(s); p.kv_group = kv_group_of(s);
     p.test_stall = (s->flags & MKA_FLAG_TEST_STALL) ? 1 : 0;
+    const size_t elem = s->dtype == MKA_BF16 ? 2 : 4;
+    const Span dg = {reinterpret_cast<uintptr_t>(dG), reinterpret_cast<uintptr_t>(dG) + (size_t)s->B * s->T * 3 * sizeof(float)};
+    p.dg_last = dg.meets(Q, rows * s->d * elem) || dg.meets(dO, rows * s->d * elem) || dg.meets(LSE, rows * sizeof(float)) ||
+                dg.meets(gate, (size_t)s->B * s->T * 3 * sizeof(float));
+    for (int l = 0; l < 3; ++l)
+        for (const void* x : {p.L[l].k, p.L[l].v}) p.dg_last |= dg.meets(level_span(x, p.L[l], p, elem));
     const bool tc = !(s->flags & MKA_FLAG_FORCE_SIMT) && bwd_tc_eligible(p, s->dtype);
     if (tc && !aligned16(ws)) return MKA_ERR_ALIGN;          // its statistics are read 16 bytes at a time
     cudaStream_t cs = static_cast<cudaStream_t>(stream);

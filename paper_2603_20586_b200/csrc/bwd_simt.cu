@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
     }
 }
 
-// The gate gradient where no level has a key and there is no dK/dV launch to do it.
+// The gate gradient where the dK/dV launch cannot do it: no level has a key, or dG is written over something that launch reads.
 __global__ void bwd_dgate_kernel(const float* Gpart, int B, int H, long long T, float* dG) {
     chain_enter();
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;   // over B*T*3
@@ -355,12 +355,13 @@ cudaError_t launch_dkv(const BwdParams& p, int vec, cudaStream_t st) {
     for (int l = 0; l < 3; ++l) key_tiles += (p.L[l].n + S::kRows - 1) / S::kRows;
     if (key_tiles == 0) return launch_bwd_dgate(p.Gpart, p.B, p.H, p.T, p.dG, st);
     const size_t smem = sizeof(float) * (2 * S::kRows * DH + S::kThreads * 2 * kSimtWarpRows + (size_t)S::kGroups * 2 * kSimtTile * (DH + 4));
-    const cudaError_t e = cudaFuncSetAttribute(bwd_dkv_kernel<T, DH, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(bwd_dkv_kernel<T, DH, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int H_kv = p.H / (p.kv_group > 0 ? p.kv_group : 1);
-    const long long gate_blocks = (p.T * 3LL + S::kThreads - 1) / S::kThreads;       // of a batch, dealt over blockIdx.x and .y
-    return launch_chained(bwd_dkv_kernel<T, DH, GROUPS>, dim3((unsigned)(key_tiles + (gate_blocks + H_kv - 1) / H_kv), H_kv, p.B), dim3(S::kThreads), smem, st, 0,
-                          p, vec, (int)key_tiles);
+    const long long gate_blocks = p.dg_last ? 0 : (p.T * 3LL + S::kThreads - 1) / S::kThreads;       // of a batch, dealt over blockIdx.x and .y
+    e = launch_chained(bwd_dkv_kernel<T, DH, GROUPS>, dim3((unsigned)(key_tiles + (gate_blocks + H_kv - 1) / H_kv), H_kv, p.B), dim3(S::kThreads), smem, st, 0,
+                       p, vec, (int)key_tiles);
+    return e == cudaSuccess && p.dg_last ? launch_bwd_dgate(p.Gpart, p.B, p.H, p.T, p.dG, st) : e;
 }
 
 template <typename T, int DH>

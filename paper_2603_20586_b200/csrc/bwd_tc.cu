@@ -69,7 +69,7 @@ struct BwdTcParams {
     long long dkv_items;      // key tiles of all levels, KV heads and batches
     long long dq_items;       // query tiles of all heads and batches
     unsigned int *dkv_ticket, *dq_ticket, *gate_ticket;   // zero at launch
-    float* dG;
+    float* dG;                // null: not this kernel's
     unsigned int* status;
     unsigned long long wait_limit_ns;
     int test_stall;           // test hook: the dK/dV kernel's loader leaves out the last query tile of every CTA
@@ -1146,7 +1146,7 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
     const long long per_batch = p.T * 3LL;
     for (;;) {
         const long long at = (long long)gate_chunk * C::kThreadsDkv + tid;
-        if (at - tid >= per_batch * p.B) break;
+        if (!p.dG || at - tid >= per_batch * p.B) break;
         if (at < per_batch * p.B) sum_dgate(p.Gpart, p.dG, p.H, p.T, at / per_batch, at % per_batch);
         __syncthreads();
         if (tid == 0) gate_chunk = atomicAdd(p.gate_ticket, 1u);
@@ -1224,10 +1224,10 @@ cudaError_t launch_t(const BwdParams& bp, unsigned int* status_word, cudaStream_
         p.dkv_items = (long long)tiles * H_kv * bp.B;
         p.dkv_ticket = status_word + 1;
         p.gate_ticket = status_word + 3;
-        p.dG = bp.dG;
-        const long long ctas = p.dkv_items + ((long long)p.B * p.T * 3 + C::kThreadsDkv - 1) / C::kThreadsDkv;   // key tiles and sums of dG
+        p.dG = bp.dg_last ? nullptr : bp.dG;
+        const long long ctas = p.dkv_items + (!p.dG ? 0 : (long long)p.B * p.T * 3 + C::kThreadsDkv - 1) / C::kThreadsDkv;   // key tiles and sums of dG
         e = launch_chained(bwd_dkv_tc_kernel<DH>, dim3((unsigned)(ctas < 148 ? ctas : 148)), dim3(C::kThreadsDkv), C::kSmemDkv, st, 0, m, p);
-        return e;
+        if (e != cudaSuccess || p.dG) return e;
     }
     return launch_bwd_dgate(bp.Gpart, bp.B, bp.H, bp.T, bp.dG, st);
 }

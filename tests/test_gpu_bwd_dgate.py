@@ -48,3 +48,18 @@ def test_cuda_core_sums_match_the_oracle(mka, orc, case):
     want = orc.bwd(P["Q"], P["K"], P["V"], rg, P["dO"], W)["dG"]
     # sums of up to T terms and H heads: the contract's bound grows with the largest of them
     assert err(got, want)[0] <= F32_MAX * max(1.0, np.abs(want).max())
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32], ids=["bf16", "f32"])
+@pytest.mark.parametrize("over", ["gate", "LSE"])
+def test_gate_gradient_written_over_an_operand(mka, dtype, over):
+    B, H, T, d, W = 2, 3, 500, 64, 100
+    P = problem(73, B, H, T, d, (T, T, 90), 32, dtype, router_std=0.3, with_dO=True)
+    gate = mka.mka_router(P["X"], P["W_r"], None)
+    shape = mka.make_shape(B, H, T, d, 32, W, dtype=mka.binding.MKA_BF16 if dtype == torch.bfloat16 else mka.binding.MKA_F32)
+    O, LSE = mka.mka_fwd(shape, P["Q"], P["K"], P["V"], gate)
+    apart = mka.mka_bwd(shape, P["Q"], P["K"], P["V"], gate, O, LSE, P["dO"])
+    dG = gate if over == "gate" else LSE.view(-1)[:gate.numel()].view(gate.shape)
+    got = mka.mka_bwd(shape, P["Q"], P["K"], P["V"], gate, O, LSE, P["dO"], dG=dG)
+    assert got["dG"] is dG and torch.equal(dG, apart["dG"]) and torch.equal(got["dQ"], apart["dQ"])
+    for l in range(3): assert torch.equal(got["dK"][l], apart["dK"][l]) and torch.equal(got["dV"][l], apart["dV"][l])
