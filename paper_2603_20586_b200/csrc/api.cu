@@ -572,7 +572,12 @@ mka_status mka_bwd(const mka_shape* s, const void* Q, const mka_level L[3], cons
     p.dg_last = dg.meets(Q, rows * s->d * elem) || dg.meets(dO, rows * s->d * elem) || dg.meets(LSE, rows * sizeof(float)) ||
                 dg.meets(gate, (size_t)s->B * s->T * 3 * sizeof(float));
     for (int l = 0; l < 3; ++l)
-        for (const void* x : {p.L[l].k, p.L[l].v}) p.dg_last |= dg.meets(level_span(x, p.L[l], p, elem));
+        for (const void* x : {p.L[l].k, p.L[l].v}) {
+            const Span rows_of_x = level_span(x, p.L[l], p, elem);
+            p.dg_last |= dg.meets(rows_of_x);
+            for (int m = 0; m < 3; ++m)
+                p.in_place |= p.L[m].n > 0 && (rows_of_x.meets(level_span(p.dL[m].dk, p.dL[m], p, elem)) || rows_of_x.meets(level_span(p.dL[m].dv, p.dL[m], p, elem)));
+        }
     const bool tc = !(s->flags & MKA_FLAG_FORCE_SIMT) && bwd_tc_eligible(p, s->dtype);
     if (tc && !aligned16(ws)) return MKA_ERR_ALIGN;          // its statistics are read 16 bytes at a time
     cudaStream_t cs = static_cast<cudaStream_t>(stream);

@@ -70,6 +70,7 @@ struct BwdTcParams {
     long long dq_items;       // query tiles of all heads and batches
     unsigned int *dkv_ticket, *dq_ticket, *gate_ticket;   // zero at launch
     float* dG;                // null: not this kernel's
+    int in_place;             // a gradient of keys or values is written over keys or values
     unsigned int* status;
     unsigned long long wait_limit_ns;
     int test_stall;           // test hook: the dK/dV kernel's loader leaves out the last query tile of every CTA
@@ -366,7 +367,7 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const 
         for (int i = 0; i < 2; ++i) { mbar_init(&bar.item_full[i], 1); mbar_init(&bar.item_free[i], 1 + C::kEw); }   // the issuing warp and the element-wise warps
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    chain_enter();
+    chain_wait();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -374,6 +375,8 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    // Only now, with the statistics there for whoever comes next: the dK/dV kernel does not wait for this one (see there).
+    chain_trigger();
     const uint32_t tmem = tmem_base_slot;
     volatile WaitCtl* abortp = &wait_ctl;
 
@@ -751,7 +754,13 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
     __syncthreads();
     if (tid < kBlk) *reinterpret_cast<uint4*>(sAugK + (tid & 7) * 16 + (tid >> 3) * 256) = make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    chain_enter();
+    // Nothing that the dQ kernel writes is read here, so this kernel's CTAs start as soon as an SM has no more items of that one, under
+    // its tail, instead of waiting for its end.  What it does read was there before the dQ kernel let it start; the statistics, which
+    // an L1 may still hold from an earlier call, are fetched past it.  The wait for the dQ kernel comes at the end (its sums of dG; and the next kernel
+    // waits for this one only and needs both), or here where dK or dV are written over keys or values that the dQ kernel reads.
+    // Steps: [2, 16 on 4, 1000, 128] 142.8 -> 140.3 us, [8, 16, 2048, 64] 1056 -> 1044, [8, 16, 795, 64] 241.7 -> 232.7, [1, 8, 700, 128] 71.0 -> 60.1.
+    chain_trigger();
+    if (p.in_place) chain_wait();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -842,12 +851,12 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
                                (long long)I.first * kBlk + 4 * lane;
             int eq = 0;
             float4 next = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (I.E > 0) next = *reinterpret_cast<const float4*>(src);
+            if (I.E > 0) next = __ldcg(reinterpret_cast<const float4*>(src));
             for (int e = 0; e < I.E; ++e, ++n_out) {
                 const int s = n_out % C::kStages;
                 const float v[4] = {next.x * mul, next.y * mul, next.z * mul, next.w * mul};
                 if (++eq == I.Eq) { eq = 0; src += p.Tpad; }
-                if (e + 1 < I.E) next = *reinterpret_cast<const float4*>(src + (long long)eq * kBlk);
+                if (e + 1 < I.E) next = __ldcg(reinterpret_cast<const float4*>(src + (long long)eq * kBlk));
                 uint4 row[4];                                        // each value as three bf16 terms
 #pragma unroll
                 for (int i = 0; i < 4; ++i) row[i] = split3_bf16(v[i]);
@@ -1143,6 +1152,7 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
     // The gate gradient's sums over the heads, left to the CTAs that are done with their key tiles first: a ticket is a sum per
     // thread, the first one taken under the epilogue.  As a launch behind this one they took 5 us: a step at [2, 16 on 4, 1000, 128] 140.7 -> 138.0 us,
     // at [1, 8, 700, 128] 60.0 -> 57.6.
+    chain_wait();
     const long long per_batch = p.T * 3LL;
     for (;;) {
         const long long at = (long long)gate_chunk * C::kThreadsDkv + tid;
@@ -1225,6 +1235,7 @@ cudaError_t launch_t(const BwdParams& bp, unsigned int* status_word, cudaStream_
         p.dkv_ticket = status_word + 1;
         p.gate_ticket = status_word + 3;
         p.dG = bp.dg_last ? nullptr : bp.dG;
+        p.in_place = bp.in_place;
         const long long ctas = p.dkv_items + (!p.dG ? 0 : (long long)p.B * p.T * 3 + C::kThreadsDkv - 1) / C::kThreadsDkv;   // key tiles and sums of dG
         e = launch_chained(bwd_dkv_tc_kernel<DH>, dim3((unsigned)(ctas < 148 ? ctas : 148)), dim3(C::kThreadsDkv), C::kSmemDkv, st, 0, m, p);
         if (e != cudaSuccess || p.dG) return e;

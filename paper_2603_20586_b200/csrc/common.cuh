@@ -185,6 +185,7 @@ struct BwdParams {
     float scale;
     int kv_group;     // query heads per KV head (>= 1); > 1 only on the tensor-core path
     unsigned int* status;   // first 16 bytes of the workspace (status word, tickets): cleared by the first kernel of the call
+    int in_place;     // a gradient of keys or values lies in memory of keys or values
     int dg_last;      // dG lies in memory that the call still reads: its sums have to wait for the end of dK and dV
     int test_stall;   // MKA_FLAG_TEST_STALL (tensor-core path): the dK/dV kernel's loader leaves out its last query tile
 };

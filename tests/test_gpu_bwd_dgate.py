@@ -63,3 +63,18 @@ def test_gate_gradient_written_over_an_operand(mka, dtype, over):
     got = mka.mka_bwd(shape, P["Q"], P["K"], P["V"], gate, O, LSE, P["dO"], dG=dG)
     assert got["dG"] is dG and torch.equal(dG, apart["dG"]) and torch.equal(got["dQ"], apart["dQ"])
     for l in range(3): assert torch.equal(got["dK"][l], apart["dK"][l]) and torch.equal(got["dV"][l], apart["dV"][l])
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32], ids=["bf16", "f32"])
+@pytest.mark.parametrize("swap", [False, True], ids=["own", "values_over_keys"])
+def test_key_and_value_gradients_written_over_keys_and_values(mka, dtype, swap):
+    B, H, T, d, W = 2, 6, 700, 64, 100
+    P = problem(74, B, H, T, d, (T, T, 90), 32, dtype, router_std=0.3, with_dO=True)
+    gate = mka.mka_router(P["X"], P["W_r"], None)
+    shape = mka.make_shape(B, H, T, d, 32, W, dtype=mka.binding.MKA_BF16 if dtype == torch.bfloat16 else mka.binding.MKA_F32)
+    O, LSE = mka.mka_fwd(shape, P["Q"], P["K"], P["V"], gate)
+    apart = mka.mka_bwd(shape, P["Q"], P["K"], P["V"], gate, O, LSE, P["dO"])
+    dK, dV = (P["V"], P["K"]) if swap else (P["K"], P["V"])
+    got = mka.mka_bwd(shape, P["Q"], P["K"], P["V"], gate, O, LSE, P["dO"], dK=dK, dV=dV)
+    assert torch.equal(got["dQ"], apart["dQ"]) and torch.equal(got["dG"], apart["dG"])
+    for l in range(3): assert torch.equal(dK[l], apart["dK"][l]) and torch.equal(dV[l], apart["dV"][l])
