@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
     }
 }
 
-// The gate gradient where the dK/dV launch cannot do it: no level has a key, or dG is written over something that launch reads.
+// The gate gradient where the dK/dV launch cannot do it: no level has a key, dG is written over something that launch reads, or dQ comes after it.
 __global__ void bwd_dgate_kernel(const float* Gpart, int B, int H, long long T, float* dG) {
     chain_enter();
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;   // over B*T*3

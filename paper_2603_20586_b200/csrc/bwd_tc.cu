@@ -69,8 +69,8 @@ struct BwdTcParams {
     long long dkv_items;      // key tiles of all levels, KV heads and batches
     long long dq_items;       // query tiles of all heads and batches
     unsigned int *dkv_ticket, *dq_ticket, *gate_ticket;   // zero at launch
-    float* dG;                // null: not this kernel's
-    int in_place;             // a gradient of keys or values is written over keys or values
+    float* dG;                // null: not the dK/dV kernel's
+    int dq_first, in_place;   // order of the two kernels (see launch_t); a gradient of keys or values is written over keys or values
     unsigned int* status;
     unsigned long long wait_limit_ns;
     int test_stall;           // test hook: the dK/dV kernel's loader leaves out the last query tile of every CTA
@@ -367,7 +367,12 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const 
         for (int i = 0; i < 2; ++i) { mbar_init(&bar.item_full[i], 1); mbar_init(&bar.item_free[i], 1 + C::kEw); }   // the issuing warp and the element-wise warps
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    chain_wait();
+    // Neither of the two kernels reads what the other writes, so the second one's CTAs start as soon as an SM has no more items of the
+    // first, under its tail, instead of at its end.  What the second one reads was there before the first let it start (below); the
+    // statistics, which an L1 may still hold from an earlier call, are fetched past it.  Its wait for the first comes at the end: the
+    // next kernel waits for the second only and needs both.
+    if (p.dq_first) chain_wait();
+    else chain_trigger();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -375,15 +380,20 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    // Only now, with the statistics there for whoever comes next: the dK/dV kernel does not wait for this one (see there).
-    chain_trigger();
+    if (p.dq_first) chain_trigger();                      // only now, with the statistics there for whoever comes next
     const uint32_t tmem = tmem_base_slot;
     volatile WaitCtl* abortp = &wait_ctl;
 
     if (warp == C::kProducerWarp) {
         int issued_k = 0, issued_v = 0, filled = 0;          // key tiles requested (per ring), items
         bool ok = true;
+        // (behind the dK/dV kernel some CTAs start late: all items come from the counter then)
+        const int dealt = p.dq_first ? (int)gridDim.x : 0;
         int item = blockIdx.x;
+        if (!p.dq_first) {
+            if (lane == 0) item = (int)atomicAdd(p.dq_ticket, 1u);
+            item = __shfl_sync(0xffffffffu, item, 0);
+        }
         for (int it = 0; ok; ++it) {
             const DqItem I(p, item);
             if (!(ok = post_item(bar, items, it, I, lane, abortp)) || I.E < 0) break;
@@ -430,7 +440,7 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const 
             }
             // The next item is taken only now, with this one's last tiles still in the rings: taken earlier, the items left
             // for a second round would go to whichever CTAs started first, the ones with the longest items among them.
-            if (lane == 0) item = (int)gridDim.x + (int)atomicAdd(p.dq_ticket, 1u);
+            if (lane == 0) item = dealt + (int)atomicAdd(p.dq_ticket, 1u);
             item = __shfl_sync(0xffffffffu, item, 0);
         }
         // every copy issued above must have landed before the shared memory can be given up
@@ -523,10 +533,10 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const 
         const bool row_valid = t < p.T;
         float Dt = 0.f, bias[3] = {-INFINITY, -INFINITY, -INFINITY};
         if (row_valid) {
-            Dt = p.statD[bh * p.Tpad + t];
+            Dt = __ldcg(p.statD + bh * p.Tpad + t);
 #pragma unroll
             for (int l = 0; l < 3; ++l) {
-                bias[l] = p.statB[l][bh * p.Tpad + t];
+                bias[l] = __ldcg(p.statB[l] + bh * p.Tpad + t);
             }
         }
         float Al[3] = {0.f, 0.f, 0.f}, Sl[3] = {0.f, 0.f, 0.f};   // per level: sum p dP and sum p over this thread's columns
@@ -671,6 +681,7 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreads, 1) bwd_dq_tc_kernel(const 
     __syncthreads();
     if (tid == 0 && wait_ctl.abort) atomicExch(p.status, (unsigned int)MKA_ERR_TIMEOUT);
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+    chain_wait();
 }
 
 // ------------------------------------------------------------------------------------------ dK, dV
@@ -754,13 +765,10 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
     __syncthreads();
     if (tid < kBlk) *reinterpret_cast<uint4*>(sAugK + (tid & 7) * 16 + (tid >> 3) * 256) = make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    // Nothing that the dQ kernel writes is read here, so this kernel's CTAs start as soon as an SM has no more items of that one, under
-    // its tail, instead of waiting for its end.  What it does read was there before the dQ kernel let it start; the statistics, which
-    // an L1 may still hold from an earlier call, are fetched past it.  The wait for the dQ kernel comes at the end (its sums of dG; and the next kernel
-    // waits for this one only and needs both), or here where dK or dV are written over keys or values that the dQ kernel reads.
-    // Steps: [2, 16 on 4, 1000, 128] 142.8 -> 140.3 us, [8, 16, 2048, 64] 1056 -> 1044, [8, 16, 795, 64] 241.7 -> 232.7, [1, 8, 700, 128] 71.0 -> 60.1.
-    chain_trigger();
-    if (p.in_place) chain_wait();
+    // (see the dQ kernel; written over keys or values that the dQ kernel reads, dK and dV wait for its end)
+    const bool waits = !p.dq_first || p.in_place;
+    if (waits) chain_wait();
+    else chain_trigger();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)), "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -768,6 +776,7 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (waits) chain_trigger();
     const uint32_t tmem = tmem_base_slot;
     volatile WaitCtl* abortp = &wait_ctl;
 
@@ -1199,48 +1208,44 @@ cudaError_t launch_t(const BwdParams& bp, unsigned int* status_word, cudaStream_
     p.test_stall = bp.test_stall;
 
     // both kernels move 128-row tiles (box = 64 columns x 128 rows)
-    {
-        BwdMaps m;
-        if (!make_bf16_map(&m.q, bp.Q, DH, bp.T, bp.H, bp.B, sq_n, sq_h, sq_b, 128) ||
-            !make_bf16_map(&m.dO, bp.dO, DH, bp.T, bp.H, bp.B, sq_n, sq_h, sq_b, 128))
+    BwdMaps m;
+    if (!make_bf16_map(&m.q, bp.Q, DH, bp.T, bp.H, bp.B, sq_n, sq_h, sq_b, kBlk) ||
+        !make_bf16_map(&m.dO, bp.dO, DH, bp.T, bp.H, bp.B, sq_n, sq_h, sq_b, kBlk))
+        return cudaErrorNotSupported;
+    for (int l = 0; l < 3; ++l) {
+        if (bp.L[l].n == 0) { m.k[l] = m.q; m.v[l] = m.q; continue; }
+        if (!make_bf16_map(&m.k[l], bp.L[l].k, DH, bp.L[l].n, H_kv, bp.B, bp.L[l].sn, bp.L[l].sh, bp.L[l].sb, kBlk) ||
+            !make_bf16_map(&m.v[l], bp.L[l].v, DH, bp.L[l].n, H_kv, bp.B, bp.L[l].sn, bp.L[l].sh, bp.L[l].sb, kBlk))
             return cudaErrorNotSupported;
-        for (int l = 0; l < 3; ++l) {
-            if (bp.L[l].n == 0) { m.k[l] = m.q; m.v[l] = m.q; continue; }
-            if (!make_bf16_map(&m.k[l], bp.L[l].k, DH, bp.L[l].n, H_kv, bp.B, bp.L[l].sn, bp.L[l].sh, bp.L[l].sb, kBlk) ||
-                !make_bf16_map(&m.v[l], bp.L[l].v, DH, bp.L[l].n, H_kv, bp.B, bp.L[l].sn, bp.L[l].sh, bp.L[l].sb, kBlk))
-                return cudaErrorNotSupported;
-        }
+    }
+    p.dq_items = (long long)(Tpad / kBlk) * bp.H * bp.B;
+    p.dq_ticket = status_word + 2;
+    p.dkv_items = (long long)(p.kv_tiles[0] + p.kv_tiles[1] + p.kv_tiles[2]) * H_kv * bp.B;
+    p.dkv_ticket = status_word + 1;
+    p.gate_ticket = status_word + 3;
+    p.in_place = bp.in_place;
+    // Which of the two comes first.  dK/dV has the longer items, up to every query tile of a group of heads; started last, they leave a tail.
+    // Started first, dQ's items fill the SMs beside them, but the gate gradient's sums, which need all of dQ, are then a launch of their
+    // own.  The line lies between these (longest walk in query tiles; us of a step with dQ first / dK and dV first):
+    //   6  [1, 8, 700, 128] 58.8 / 61.6     7  [8, 16, 795, 64] 241.7 / 244.7     16  [8, 16, 2048, 64] 1065 / 1071
+    //   32  [2, 16 on 4, 1000, 128] 138.9 / 130.6     84  [2, 28 on 4, 1500, 128] 350 / 307     96  [4, 8 on 2, 3000, 64] 423 / 387
+    // Written over keys or values that dQ reads, dK and dV come last.
+    const int q_tiles = Tpad / kBlk, window_tiles = (p.window < Tpad ? p.window : Tpad) / kBlk + 2;
+    const long long longest = (long long)(p.n[1] > 0 || p.n[2] > 0 || q_tiles < window_tiles ? q_tiles : window_tiles) * p.kv_group;
+    p.dq_first = p.dkv_items == 0 || bp.in_place || longest < 24;
+    p.dG = p.dq_first && !bp.dg_last && p.dkv_items > 0 ? bp.dG : nullptr;
+    auto launch_dq = [&] {
         e = cudaFuncSetAttribute(bwd_dq_tc_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmemDq);
-        if (e != cudaSuccess) return e;
-        p.dq_items = (long long)(Tpad / kBlk) * bp.H * bp.B;
-        p.dq_ticket = status_word + 2;
-        e = launch_chained(bwd_dq_tc_kernel<DH>, dim3((unsigned)(p.dq_items < 148 ? p.dq_items : 148)), dim3(C::kThreads), C::kSmemDq, st, 0, m, p);
-        if (e != cudaSuccess) return e;
-    }
-    const int tiles = p.kv_tiles[0] + p.kv_tiles[1] + p.kv_tiles[2];
-    if (tiles > 0) {
-        BwdMaps m;
-        if (!make_bf16_map(&m.q, bp.Q, DH, bp.T, bp.H, bp.B, sq_n, sq_h, sq_b, kBlk) ||
-            !make_bf16_map(&m.dO, bp.dO, DH, bp.T, bp.H, bp.B, sq_n, sq_h, sq_b, kBlk))
-            return cudaErrorNotSupported;
-        for (int l = 0; l < 3; ++l) {
-            if (bp.L[l].n == 0) { m.k[l] = m.q; m.v[l] = m.q; continue; }
-            if (!make_bf16_map(&m.k[l], bp.L[l].k, DH, bp.L[l].n, H_kv, bp.B, bp.L[l].sn, bp.L[l].sh, bp.L[l].sb, 128) ||
-                !make_bf16_map(&m.v[l], bp.L[l].v, DH, bp.L[l].n, H_kv, bp.B, bp.L[l].sn, bp.L[l].sh, bp.L[l].sb, 128))
-                return cudaErrorNotSupported;
-        }
+        if (e == cudaSuccess) e = launch_chained(bwd_dq_tc_kernel<DH>, dim3((unsigned)(p.dq_items < 148 ? p.dq_items : 148)), dim3(C::kThreads), C::kSmemDq, st, 0, m, p);
+    };
+    if (p.dq_first) launch_dq();
+    if (e == cudaSuccess && p.dkv_items > 0) {
         e = cudaFuncSetAttribute(bwd_dkv_tc_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmemDkv);
-        if (e != cudaSuccess) return e;
-        p.dkv_items = (long long)tiles * H_kv * bp.B;
-        p.dkv_ticket = status_word + 1;
-        p.gate_ticket = status_word + 3;
-        p.dG = bp.dg_last ? nullptr : bp.dG;
-        p.in_place = bp.in_place;
         const long long ctas = p.dkv_items + (!p.dG ? 0 : (long long)p.B * p.T * 3 + C::kThreadsDkv - 1) / C::kThreadsDkv;   // key tiles and sums of dG
-        e = launch_chained(bwd_dkv_tc_kernel<DH>, dim3((unsigned)(ctas < 148 ? ctas : 148)), dim3(C::kThreadsDkv), C::kSmemDkv, st, 0, m, p);
-        if (e != cudaSuccess || p.dG) return e;
+        if (e == cudaSuccess) e = launch_chained(bwd_dkv_tc_kernel<DH>, dim3((unsigned)(ctas < 148 ? ctas : 148)), dim3(C::kThreadsDkv), C::kSmemDkv, st, 0, m, p);
     }
-    return launch_bwd_dgate(bp.Gpart, bp.B, bp.H, bp.T, bp.dG, st);
+    if (e == cudaSuccess && !p.dq_first) launch_dq();
+    return e != cudaSuccess || p.dG ? e : launch_bwd_dgate(bp.Gpart, bp.B, bp.H, bp.T, bp.dG, st);
 }
 
 }  // namespace

@@ -17,7 +17,7 @@ def mka():
 
 
 # B, H, T, d, window, rows of the three levels
-TC = [(1, 3, 40000, 64, 16, (0, 0, 20)), (2, 5, 300, 128, 32, (300, 300, 130)), (1, 32, 1000, 128, 256, (1000, 0, 7)), (3, 2, 129, 64, 129, (129, 129, 0))]
+TC = [(1, 3, 40000, 64, 16, (0, 0, 20)), (9, 2, 1100, 64, 64, (0, 0, 20)), (2, 5, 300, 128, 32, (300, 300, 130)), (1, 32, 1000, 128, 256, (1000, 0, 7)), (3, 2, 129, 64, 129, (129, 129, 0))]
 
 
 @pytest.mark.parametrize("case", TC, ids=lambda c: f"T{c[2]}H{c[1]}d{c[3]}")
@@ -67,8 +67,9 @@ def test_gate_gradient_written_over_an_operand(mka, dtype, over):
 
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32], ids=["bf16", "f32"])
 @pytest.mark.parametrize("swap", [False, True], ids=["own", "values_over_keys"])
-def test_key_and_value_gradients_written_over_keys_and_values(mka, dtype, swap):
-    B, H, T, d, W = 2, 6, 700, 64, 100
+@pytest.mark.parametrize("T", [700, 3100])                        # 3100: apart, dK and dV come before dQ; in place, behind it
+def test_key_and_value_gradients_written_over_keys_and_values(mka, dtype, swap, T):
+    B, H, d, W = 2, 6, 64, 100
     P = problem(74, B, H, T, d, (T, T, 90), 32, dtype, router_std=0.3, with_dO=True)
     gate = mka.mka_router(P["X"], P["W_r"], None)
     shape = mka.make_shape(B, H, T, d, 32, W, dtype=mka.binding.MKA_BF16 if dtype == torch.bfloat16 else mka.binding.MKA_F32)
