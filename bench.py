@@ -54,15 +54,15 @@ def load_peaks():
 # as it was when the counters were taken: when the file has changed since, the figure is reported as null ("stale").
 NCU_TRAFFIC = {
     # kernel@workload: (bytes in the capture, units of the capture, summary file under profiles/, source file, its digest)
-    "fwd_tc_kernel@c3": (376.073216e6 + 57.210112e6, 1 * 8, "fwd_tc_kernel_c3p.md", "fwd_tc.cu", "266857ed858f"),
-    "fwd_tc_kernel64@c2": (204.392704e6 + 27.338752e6, 8 * 16, "fwd_tc_kernel64_c2.md", "fwd_tc.cu", "266857ed858f"),   # the whole configuration
-    "decode_partial_kernel@c4": (1.476515e9 + 3.866880e6, 2 * 32, "decode_partial_kernel_c4p.md", "decode.cu", "93b91a32241a"),
-    "bwd_dq_tc_kernel@c5": (220.267264e6 + 26.553088e6, 1 * 16, "bwd_tc_kernels_c5p.md", "bwd_tc.cu", "62205ef506c5"),
-    "bwd_dkv_tc_kernel@c5": (220.343808e6 + 116.964864e6, 1 * 16, "bwd_tc_kernels_c5p.md", "bwd_tc.cu", "62205ef506c5"),
-    "l2_summary_seg_kernel@s3": (101.000704e6 + 55.384064e6, 12288.0 / 32768.0, "l2_summary_seg_kernel_s3p.md", "summary_seg.cu", "6e2dcc00fbde"),   # 12288 of the 32768 tokens
-    "fuse_kv_kernel@f3": (403.137024e6 + 83.414784e6, 1 * 8, "fuse_kv_kernel_f3p.md", "fuse_kv.cu", "3becacc721a4"),
-    "decode_paged_kernel@g4": (293.738240e6 + 3.420928e6, 1 * 4, "decode_paged_kernel_g4p.md", "decode_paged.cu", "f1544adcf30a"),   # one of the four sequences (g4p)
-    "l3_index_kernel@r3": (134.313728e6 + 3.178496e6, 1, "l3_index_kernel_r3p.md", "l3.cu", "feaf0bd07ff1"),            # one of the four sequences (r3p)
+    "fwd_tc_kernel@c3": (375.738112e6 + 56.466176e6, 1 * 8, "fwd_tc_kernel_c3p.md", "fwd_tc.cu", "700d68196eb2"),
+    "fwd_tc_kernel64@c2": (204.101888e6 + 25.370112e6, 8 * 16, "fwd_tc_kernel64_c2.md", "fwd_tc.cu", "700d68196eb2"),   # the whole configuration
+    "decode_partial_kernel@c4": (1.476457e9 + 4.163328e6, 2 * 32, "decode_partial_kernel_c4p.md", "decode.cu", "8ff55e2ca41e"),
+    "bwd_dq_tc_kernel@c5": (220.270080e6 + 27.188992e6, 1 * 16, "bwd_tc_kernels_c5p.md", "bwd_tc.cu", "482b3652e285"),
+    "bwd_dkv_tc_kernel@c5": (220.271360e6 + 117.273344e6, 1 * 16, "bwd_tc_kernels_c5p.md", "bwd_tc.cu", "482b3652e285"),
+    "l2_summary_seg_kernel@s3": (100.699392e6 + 54.012160e6, 12288.0 / 32768.0, "l2_summary_seg_kernel_s3p.md", "summary_seg.cu", "f824f10a3d76"),   # 12288 of the 32768 tokens
+    "fuse_kv_kernel@f3": (403.136512e6 + 83.408640e6, 1 * 8, "fuse_kv_kernel_f3p.md", "fuse_kv.cu", "b1ef4c991e47"),
+    "decode_paged_kernel@g4": (293.730304e6 + 3.355136e6, 1 * 4, "decode_paged_kernel_g4p.md", "decode_paged.cu", "929e98e72397"),   # one of the four sequences (g4p)
+    "l3_index_kernel@r3": (134.305792e6 + 4.221696e6, 1, "l3_index_kernel_r3p.md", "l3.cu", "607ee4fa9ab7"),            # one of the four sequences (r3p)
 }
 
 
@@ -216,7 +216,7 @@ class Leg:
             self.grads = {"dQ": torch.empty_like(self.t["Q"]), "dK": [torch.empty_like(k) for k in self.K],
                           "dV": [torch.empty_like(v) for v in self.V], "dG": torch.empty(B, T, 3, device=device),
                           "dW_r": torch.empty(D, 3, device=device), "db_r": torch.empty(3, device=device)}
-            self.launches_per_step = 1 + 1 + (1 + 1 + 1) + 2   # router, fwd, bwd(prep,dq,dkv), router bwd
+            self.launches_per_step = 1 + 1 + (1 + 1 + 1 + 1) + 2   # router, fwd, bwd(prep,dkv,dq,dgate), router bwd
             self.bwd_executed_ratio = 1.4           # the two-pass backward runs 14 d flops per pair for the method's 10 d
         else:
             self.launches_per_step = 2              # router, fwd
