@@ -92,6 +92,12 @@ struct Cfg {
     static constexpr int kCtasPerSm = DH == 128 ? 1 : 2;
     static constexpr int kMergeCols = DH == 128 ? 16 : 8;      // columns of a row that a thread merges at a time (kCluster)
     static constexpr int kParts = kTileN / 32;                // the weights of a tile are handed over in parts of 32 keys
+    // d = 64 sums the weights of keys 0..63 and 64..127 of a tile apart, each with a running sum of its own: in one chain of
+    // all 128 small weights are lost beside large ones earlier (64 weights of 2^-24 after four of 1: LSE short by 9.5e-7 of 1.39, now by a rounding; [8, 16, 2048,
+    // 64] on normal inputs: LSE off by 4.45e-8 in one chain, 4.42e-8 in two).  The parts are taken from the two halves in turn, which adds up O's products
+    // in the order of the sums.
+    static constexpr int kSums = DH == 64 ? 2 : 1;
+    static constexpr __host__ __device__ int part_of(int i) { return kSums == 2 && (i == 1 || i == 2) ? 3 - i : i; }
     static constexpr int kRowWarps = 4;                       // softmax warps per query tile
     static constexpr int kSoftmaxWarps = kRowWarps * kNumQ;
     // The registers are re-divided between the warpgroups (setmaxnreg, a warpgroup-wide instruction: an idle warp
@@ -502,14 +508,14 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
                 const uint32_t va = v_lo + (g % C::kStages) * (C::kTileBytes >> 4);
                 const uint32_t pa = tmem + (C::kSeparateP ? C::kColP + q * (kTileN / 2) : q * kTileN);
 #pragma unroll
-                for (int part = 0; part < C::kParts; ++part) {
-                    if (!mbar_wait_warp(&bar.p_part[q][part], (uint32_t)g & 1u, abortp)) return false;
+                for (int n = 0; n < C::kParts; ++n) {
+                    if (!mbar_wait_warp(&bar.p_part[q][C::part_of(n)], (uint32_t)g & 1u, abortp)) return false;
                     tc_fence_after();
 #pragma unroll
                     for (int i = 0; i < 2; ++i) {
-                        const int k = part * 2 + i;
+                        const int k = C::part_of(n) * 2 + i;
                         mma_ts_elect(tmem + C::kColO + q * DH, pa + k * 8, make_desc(va + k * (2048 >> 4)), C::kIdescPV,
-                                     (accumulate || part > 0 || i > 0) ? 1u : 0u);
+                                     (accumulate || n > 0 || i > 0) ? 1u : 0u);
                     }
                 }
                 mma_commit_elect(&bar.pv_done[q]);
@@ -642,7 +648,7 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
         const int tq0 = I.m[q];                                                  // first row of this query tile
         const int t = tq0 + row_in_tile;                                         // T < 2^31 - 256
         const bool row_valid = t < p.T;
-        float m_run = -INFINITY, l_run = 0.f;
+        float m_run = -INFINITY, l_part[C::kSums] = {};
         int e = 0;
 #pragma unroll 1
         for (int l = 0; l < 3 && ok; ++l) {
@@ -713,7 +719,8 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
                 const float m_eff = m_use == -INFINITY ? 0.f : m_use;
                 const float alpha = grow ? (m_run == -INFINITY ? 0.f : ex2(m_run - m_use)) : 1.f;
                 const float shift = bias - m_eff;
-                l_run *= alpha;
+#pragma unroll
+                for (int i = 0; i < C::kSums; ++i) l_part[i] *= alpha;
                 m_run = m_use;
                 // P(e-1) must have been consumed before P(e) replaces it (d = 64), and before O is rescaled
                 const bool rescale = e > 0 && __any_sync(0xffffffffu, alpha != 1.f);
@@ -736,17 +743,20 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
                 // the issuing warp in the middle of the next part's exponentials, when its store has long completed.
                 // Scale, shift and the row sum work on packed pairs: one instruction for two columns.
                 const uint64_t scale2 = pack2(p.scale_log2, p.scale_log2), shift2 = pack2(shift, shift);
-                uint64_t sum_a = pack2(0.f, 0.f), sum_b = sum_a;
+                uint64_t sum_a[C::kSums], sum_b[C::kSums];
+#pragma unroll
+                for (int i = 0; i < C::kSums; ++i) sum_a[i] = sum_b[i] = pack2(0.f, 0.f);
                 uint32_t pk[16];
                 auto weights = [&](int c_from, int c_to, int c_base) {
+                    const int half = C::kSums == 2 ? c_base / 64 : 0;
 #pragma unroll
                     for (int c = c_from; c < c_to; c += 4) {
                         float x0, x1, x2, x3;
                         unpack2(fma2(pack2(s[c], s[c + 1]), scale2, shift2), x0, x1);
                         unpack2(fma2(pack2(s[c + 2], s[c + 3]), scale2, shift2), x2, x3);
                         const float p0 = ex2(x0), p1 = ex2(x1), p2 = ex2(x2), p3 = ex2(x3);
-                        sum_a = add2(sum_a, pack2(p0, p1));
-                        sum_b = add2(sum_b, pack2(p2, p3));
+                        sum_a[half] = add2(sum_a[half], pack2(p0, p1));
+                        sum_b[half] = add2(sum_b[half], pack2(p2, p3));
                         pk[(c - c_base) / 2] = pack_bf16(p0, p1);
                         pk[(c - c_base) / 2 + 1] = pack_bf16(p2, p3);
                     }
@@ -758,20 +768,23 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
                     if (lane == 0) mbar_arrive(&bar.p_part[q][part]);
                 };
 #pragma unroll
-                for (int part = 0; part < C::kParts; ++part) {
+                for (int n = 0; n < C::kParts; ++n) {
+                    const int part = C::part_of(n);
                     weights(32 * part, 32 * part + 16, 32 * part);
-                    if (part > 0) hand_over(part - 1);
+                    if (n > 0) hand_over(C::part_of(n - 1));
                     weights(32 * part + 16, 32 * part + 32, 32 * part);
                     tmem_st16(p_addr + 16 * part, pk);
                 }
-                {
+#pragma unroll
+                for (int i = 0; i < C::kSums; ++i) {
                     float a0, a1;
-                    unpack2(add2(sum_a, sum_b), a0, a1);
-                    l_run += a0 + a1;
+                    unpack2(add2(sum_a[i], sum_b[i]), a0, a1);
+                    l_part[i] += a0 + a1;
                 }
-                hand_over(C::kParts - 1);
+                hand_over(C::part_of(C::kParts - 1));
             }
         }
+        const float l_run = C::kSums == 2 ? l_part[0] + l_part[C::kSums - 1] : l_part[0];
         // ------------------------------------------------------------ epilogue
         const int E = I.E;
         if (ok && E > 0) ok = __all_sync(0xffffffffu, mbar_wait(&bar.pv_done[q], (uint32_t)(g - 1) & 1u, abortp));

@@ -123,3 +123,19 @@ def test_ranges_long_lists(mka, orc, d):
     Or, Lr = orc.fwd(np64(P["Q"]), [full(k) for k in P["K"]], [full(v) for v in P["V"]], np64(gate), W, q_off)
     check(O, Or, torch.bfloat16, "O")
     assert err(LSE, Lr)[0] <= 2e-3 and (LSE - lse_whole).abs().max().item() <= 1e-4
+
+
+def test_small_weights_of_a_row_are_kept(mka):
+    """d = 64: the weights of keys 0..63 and of keys 64..127 of a tile are added up apart.  Four weights of 1 in the first half, 64 of 2^-24
+    in the second: the sum is 4 + 2^-18 in fp32, and LSE misses it by the roundings of a logarithm and a product (1.5e-7 each at most);
+    added to the ones, each of the small weights is lost and LSE is short by 9.5e-7."""
+    B, H, T, d, n = 1, 2, 130, 64, 128
+    Q, K, V = (torch.zeros(B, H, rows, d, device="cuda", dtype=torch.bfloat16) for rows in (T, n, n))
+    Q[..., 0] = 1.0
+    K[:, :, :64, 0], K[:, :, :4, 0], K[:, :, 64:, 0] = -1000.0, 0.0, -24.0      # log2 of the weights: a scale of ln 2 makes base 2
+    V[..., 3] = 1.0
+    gate = torch.tensor([0.0, 0.0, 1.0], device="cuda").repeat(B, T, 1).contiguous()
+    shape = mka.make_shape(B, H, T, d, 64, 64, scale=float(np.log(2.0)))
+    O, LSE = mka.mka_fwd(shape, Q, [None, None, K], [None, None, V], gate)
+    assert (LSE.double() - np.log(4.0 + 2.0 ** -18)).abs().max().item() <= 4e-7
+    assert torch.equal(O, torch.ones_like(O) * (torch.arange(d, device="cuda") == 3))
