@@ -478,7 +478,10 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
             for (int it = 1;; ++it) {
                 Item next;
                 next_piece(next);
-                if (it >= 2 && !mbar_wait_warp(&bar.item_free[it & 1], (uint32_t)((it - 2) >> 1) & 1u, abortp)) break;
+                // This wait lasts as long as the work on item it - 2, which is in the way: some waits of the other roles for each of its key
+                // tiles, and it is allowed as many limits.  Should one of those run out, it ends this one.  (Counting the tiles as they
+                // are asked for and starting the clock again with each cost a 512-row chunk at 15,000 rows of context 1.5 %.)
+                if (it >= 2 && !mbar_wait_warp(&bar.item_free[it & 1], (uint32_t)((it - 2) >> 1) & 1u, abortp, 8u * (items[it & 1].E + 1))) break;
                 if (lane == 0) {
                     items[it & 1] = next;
                     mbar_arrive(&bar.item_full[it & 1]);

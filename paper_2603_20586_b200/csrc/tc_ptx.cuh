@@ -39,8 +39,8 @@ __device__ __forceinline__ unsigned long long gtimer() {
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
-// Bounded wait: false when the limit expired or another role already gave up.
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile WaitCtl* ctl) {
+// Bounded wait: false when the limit (`limits` of them) expired or another role already gave up.
+__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile WaitCtl* ctl, unsigned int limits = 1) {
     if (mbar_try(b, parity)) return true;
     const unsigned long long t0 = gtimer();
     for (;;) {
@@ -48,7 +48,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile
         for (int i = 0; i < 32; ++i)
             if (mbar_try(b, parity)) return true;
         if (ctl->abort) return false;
-        if (gtimer() - t0 > ctl->limit_ns) { ctl->abort = 1; return false; }
+        if (gtimer() - t0 > limits * ctl->limit_ns) { ctl->abort = 1; return false; }
     }
 }
 // Waits for a copy that was issued.  Unlike mbar_wait it goes on when another role gave up: a CTA must not hand its shared memory
@@ -130,8 +130,8 @@ __device__ __forceinline__ void mma_commit_elect(uint64_t* bar) {
                  ::"r"(smem_u32(bar)) : "memory");
 }
 // Bounded wait executed by every lane of a converged warp; the result is made warp-uniform.
-__device__ __forceinline__ bool mbar_wait_warp(uint64_t* b, uint32_t parity, volatile WaitCtl* ctl) {
-    return __all_sync(0xffffffffu, mbar_wait(b, parity, ctl));
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* b, uint32_t parity, volatile WaitCtl* ctl, unsigned int limits = 1) {
+    return __all_sync(0xffffffffu, mbar_wait(b, parity, ctl, limits));
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }

@@ -7,6 +7,8 @@ tile of a share of the paged decode; one segment's carried state): the wait runs
 status word of the workspace reads MKA_ERR_TIMEOUT.  The next ordinary call on the same stream must then match the
 oracle, which shows that the context and the library are still healthy.
 """
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -148,3 +150,27 @@ def test_summary_look_back_runs_out_and_the_next_call_is_correct(mka, orc, short
     assert mka.mka_device_status(ws) == 0
     ref = orc.l2_summary(np64(X))[0]
     check(M2, ref, torch.bfloat16, "summary after a timed-out call")
+
+
+@pytest.mark.parametrize("d", [128, 64])
+def test_a_low_limit_does_not_end_a_call_whose_pieces_are_long(mka, d):
+    """Equal ranges of key tiles: a CTA works on pieces of some 280 and 240 tiles, each several times as long as the limit, while every wait
+    of its copies and products is over after a tile or two.  Nothing may give up."""
+    B, H, Hkv, T, q_off = 1, 24, 4, 1024, 100000
+    N = (0, q_off + T, 64)
+    g = torch.Generator(device="cuda").manual_seed(96)
+    mk = lambda *n: torch.randn(*n, device="cuda", dtype=torch.bfloat16, generator=g)
+    Q, K, V = mk(B, H, T, d), [mk(B, Hkv, n, d) for n in N], [mk(B, Hkv, n, d) for n in N]
+    gate = torch.softmax(torch.randn(B, T, 3, device="cuda", generator=g), -1).contiguous()
+    shape = mka.make_shape(B, H, T, d, 64, 64, q_off, kv_heads=Hkv)
+    assert mka.lib.mka_fwd_scratch_bytes(ctypes.byref(shape), 0, (ctypes.c_int64 * 3)(*N)) > 0
+    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+    want, want_lse = mka.mka_fwd(shape, Q, K, V, gate, ws=ws)
+    assert mka.mka_device_status(ws) == 0
+    old = mka.mka_set_wait_limit_us(200)
+    try:
+        got, lse = mka.mka_fwd(shape, Q, K, V, gate, ws=ws)
+    finally:
+        mka.mka_set_wait_limit_us(old)
+    assert mka.mka_device_status(ws) == 0
+    assert torch.equal(got, want) and torch.equal(lse, want_lse)
