@@ -425,7 +425,8 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
                 const bool mine = lane < kTileN / rpb;
                 const int in_mask = kPaged ? (1 << p.page_shift[l]) - 1 : 0;
                 for (int kt = kt_first; kt < kt_end; ++kt) {
-                    if (!kPaged && p.test_stall && --left == 0) { ok = false; break; }     // test hook: the item's last tile never arrives
+                    // test hook: the item's last tile never arrives (kStream: of the first item in one half of the CTAs, of the second in the other)
+                    if (!kPaged && p.test_stall && it == (kForm == kStream ? (int)(blockIdx.x & 1) : 0) && --left == 0) { ok = false; break; }
                     const int s = issued % C::kStages;
                     const uint32_t ph = (uint32_t)(issued / C::kStages) & 1u;
                     // a box past the level's last row is aimed past the pool, where the copy engine fills zeros as it does

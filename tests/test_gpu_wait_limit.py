@@ -3,7 +3,7 @@
 Every wait inside the tensor-core forward and backward, the paged decode and the segmented summary has a wall-clock limit.
 Here the limit is set to a few milliseconds and a test hook withholds something a wait needs (the forward's last key tile;
 the last query tile of the backward's dK/dV kernel, whose issuing warp polls two barriers in a loop of its own; the last
-tile of a share of the paged decode; one segment's carried state): the wait runs out, every role of the CTA drains, tensor memory is freed, the kernel RETURNS, and the
+tile of a share of the paged decode; one segment's carried state, in global or in shared memory): the wait runs out, every role of the CTA drains, tensor memory is freed, the kernel RETURNS, and the
 status word of the workspace reads MKA_ERR_TIMEOUT.  The next ordinary call on the same stream must then match the
 oracle, which shows that the context and the library are still healthy.
 """
@@ -174,3 +174,73 @@ def test_a_low_limit_does_not_end_a_call_whose_pieces_are_long(mka, d):
         mka.mka_set_wait_limit_us(old)
     assert mka.mka_device_status(ws) == 0
     assert torch.equal(got, want) and torch.equal(lse, want_lse)
+
+
+@pytest.mark.parametrize("case", [(1, 12, 4, 949, 128, 1750, 3804, 144), (2, 32, 32, 627, 64, 2630, 0, 7815)], ids=["d128", "d64"])
+def test_forward_wait_runs_out_within_ranges(mka, short_limit, case):
+    """Equal ranges of key tiles: half of the CTAs never get the last tile of their first piece, with the dealing warp at its wait, the others
+    that of their second."""
+    B, H, Hkv, T, d, W, q_off, n3 = case
+    N = (q_off + T, q_off + T, n3)
+    g = torch.Generator(device="cuda").manual_seed(97)
+    mk = lambda *n: torch.randn(*n, device="cuda", dtype=torch.bfloat16, generator=g)
+    Q, K, V = mk(B, H, T, d), [mk(B, Hkv, n, d) for n in N], [mk(B, Hkv, n, d) for n in N]
+    gate = torch.softmax(torch.randn(B, T, 3, device="cuda", generator=g), -1).contiguous()
+    shape, stalled = (mka.make_shape(B, H, T, d, 64, W, q_off, flags=f, kv_heads=Hkv) for f in (0, mka.MKA_FLAG_TEST_STALL))
+    assert mka.lib.mka_fwd_scratch_bytes(ctypes.byref(stalled), 0, (ctypes.c_int64 * 3)(*N)) > 0
+    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+    want, want_lse = mka.mka_fwd(shape, Q, K, V, gate, ws=ws)
+    assert mka.mka_device_status(ws) == 0
+    t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    t0.record()
+    mka.mka_fwd(stalled, Q, K, V, gate, ws=ws)
+    t1.record()
+    assert mka.mka_device_status(ws) == MKA_ERR_TIMEOUT
+    assert t0.elapsed_time(t1) < 1000.0
+    got, lse = mka.mka_fwd(shape, Q, K, V, gate, ws=ws)
+    assert mka.mka_device_status(ws) == 0
+    assert torch.equal(got, want) and torch.equal(lse, want_lse)
+
+
+@pytest.mark.parametrize("d", [128, 64])
+def test_backward_wait_runs_out_with_dq_under_it(mka, short_limit, d):
+    """Grouped heads whose key tiles walk 32 query tiles: dK and dV come first, and dQ's items run under their tail, which here is a wait that
+    runs out."""
+    B, H, Hkv, T, W, N = 1, 8, 2, 1000, 96, (1000, 1000, 160)
+    g = torch.Generator(device="cuda").manual_seed(98)
+    mk = lambda *n: torch.randn(*n, device="cuda", dtype=torch.bfloat16, generator=g)
+    Q, dO, K, V = mk(B, H, T, d), mk(B, H, T, d), [mk(B, Hkv, n, d) for n in N], [mk(B, Hkv, n, d) for n in N]
+    gate = torch.softmax(torch.randn(B, T, 3, device="cuda", generator=g), -1).contiguous()
+    shape, stalled = (mka.make_shape(B, H, T, d, 64, W, flags=f, kv_heads=Hkv) for f in (0, mka.MKA_FLAG_TEST_STALL))
+    O, LSE = mka.mka_fwd(shape, Q, K, V, gate)
+    assert mka.mka_bwd_kernel_kind(shape, K, V) == 1
+    ws = mka.alloc_workspace(shape, N, mka.MKA_WS_BWD, "cuda")
+    want = mka.mka_bwd(shape, Q, K, V, gate, O, LSE, dO, ws=ws)
+    assert mka.mka_device_status(ws) == 0
+    t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    t0.record()
+    mka.mka_bwd(stalled, Q, K, V, gate, O, LSE, dO, ws=ws)
+    t1.record()
+    assert mka.mka_device_status(ws) == MKA_ERR_TIMEOUT
+    assert t0.elapsed_time(t1) < 1000.0
+    got = mka.mka_bwd(shape, Q, K, V, gate, O, LSE, dO, ws=ws)
+    assert mka.mka_device_status(ws) == 0
+    assert torch.equal(got["dQ"], want["dQ"]) and torch.equal(got["dG"], want["dG"])
+    for l in range(3): assert torch.equal(got["dK"][l], want["dK"][l]) and torch.equal(got["dV"][l], want["dV"][l])
+
+
+def test_summary_hand_over_runs_out_and_the_next_call_is_correct(mka, orc, short_limit):
+    """128 strips of eight tiles: one CTA to a strip, whose second group never hands its state on.  (This form leaves the scratch alone.)"""
+    B, T, D = 1, 4096, 4096
+    X = torch.randn(B, T, D, device="cuda", dtype=torch.bfloat16, generator=torch.Generator(device="cuda").manual_seed(99))
+    ws = mka.mka_l2_summary_workspace(X).fill_(0x5a)
+    assert mka.mka_l2_summary_kernel_kind(X, ws) == 1
+    t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    t0.record()
+    mka.mka_l2_summary(X, mka.MKA_SUMMARY_MEAN | mka.MKA_SUMMARY_TEST_STALL, ws=ws)
+    t1.record()
+    assert mka.mka_device_status(ws) == MKA_ERR_TIMEOUT
+    assert t0.elapsed_time(t1) < 1000.0
+    M2 = mka.mka_l2_summary(X, mka.MKA_SUMMARY_MEAN, ws=ws)
+    assert mka.mka_device_status(ws) == 0 and bool((ws[256:] == 0x5a).all())
+    check(M2, orc.l2_summary(np64(X))[0], torch.bfloat16, "summary after a timed-out call")
