@@ -1224,15 +1224,26 @@ cudaError_t launch_t(const BwdParams& bp, unsigned int* status_word, cudaStream_
     p.dkv_ticket = status_word + 1;
     p.gate_ticket = status_word + 3;
     p.in_place = bp.in_place;
-    // Which of the two comes first.  dK/dV has the longer items, up to every query tile of a group of heads; started last, they leave a tail.
-    // Started first, dQ's items fill the SMs beside them, but the gate gradient's sums, which need all of dQ, are then a launch of their
-    // own.  The line lies between these (longest walk in query tiles; us of a step with dQ first / dK and dV first):
-    //   6  [1, 8, 700, 128] 58.8 / 61.6     7  [8, 16, 795, 64] 241.7 / 244.7     16  [8, 16, 2048, 64] 1065 / 1071
-    //   32  [2, 16 on 4, 1000, 128] 138.9 / 130.6     84  [2, 28 on 4, 1500, 128] 350 / 307     96  [4, 8 on 2, 3000, 64] 423 / 387
+    // Which of the two comes first: the one with the longer items, which would leave a tail behind the other; the shorter ones then fill the SMs
+    // beside them.  An item of dK/dV walks up to every query tile of a group of heads, one of dQ the key tiles of three levels.  dK and dV
+    // have to be worth it: the gate gradient's sums, which need all of dQ, are a launch of their own behind it.  Nothing is to be gained with few
+    // query tiles or where all items find an SM of their own.  With one or two heads of many tiles dQ's items all start at once,
+    // and the SMs with the longest of them would come last to dK/dV's first.  Longest items in tiles (dK/dV, dQ); us of a backward, dQ first /
+    // dK and dV first, the pick in brackets:
+    //   grouped     [2, 12 on 4, 1100, 64] (27, 13) 86 / [78]        [2, 16 on 4, 1000, 128] (32, 16) 141 / [131]     [1, 16 on 4, 700, 128] (24, 22) 99 / [93]
+    //               [1, 28 on 4, 2000, 128] (112, 21) 294 / [248]    [2, 32 on 8, 4096, 128] (128, 46) 1500 / [1414]  [2, 16 on 8, 1600, 128] (26, 19) 153 / [146]
+    //               [4, 16 on 8, 2048, 64] (32, 30) [354] / 358      [1, 4 on 2, 2048, 128] (32, 24), 136 items [66] / 68
+    //   ungrouped   [1, 8, 3100, 128] (25, 39) [151] / 159           [1, 3, 6000, 64] (47, 61) [116] / 126            [2, 16, 3100, 64] (25, 39) [332] / 342
+    //               [1, 32, 8192, 128] (64, 90) [2784] / 2806        [4, 16, 8192, 128] (64, 90) [5475] / 5580        [1, 3, 4096, 64] (32, 58) [90] / 101
+    //   two heads   [1, 2, 8192, 128] (64, 90) 213 / [188]           [1, 2, 6000, 128] (47, 73) 155 / [139]           [1, 2, 4096, 128] (32, 50) [83] / 92
     // Written over keys or values that dQ reads, dK and dV come last.
     const int q_tiles = Tpad / kBlk, window_tiles = (p.window < Tpad ? p.window : Tpad) / kBlk + 2;
     const long long longest = (long long)(p.n[1] > 0 || p.n[2] > 0 || q_tiles < window_tiles ? q_tiles : window_tiles) * p.kv_group;
-    p.dq_first = p.dkv_items == 0 || bp.in_place || longest < 24;
+    const long long causal_tiles = ((long long)p.q_offset + Tpad + kBlk - 1) / kBlk;
+    const long long dq_longest = (long long)(p.kv_tiles[0] < window_tiles ? p.kv_tiles[0] : window_tiles) +
+                                 (p.kv_tiles[1] < causal_tiles ? p.kv_tiles[1] : causal_tiles) + p.kv_tiles[2];
+    const bool longer = 12 * longest > 13 * dq_longest, two_heads = (long long)p.B * p.H <= 2 && q_tiles >= 40;
+    p.dq_first = p.dkv_items == 0 || bp.in_place || longest < 24 || p.dkv_items + p.dq_items <= 148 || !(longer || two_heads);
     p.dG = p.dq_first && !bp.dg_last && p.dkv_items > 0 ? bp.dG : nullptr;
     auto launch_dq = [&] {
         e = cudaFuncSetAttribute(bwd_dq_tc_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmemDq);

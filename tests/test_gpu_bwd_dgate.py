@@ -67,7 +67,7 @@ def test_gate_gradient_written_over_an_operand(mka, dtype, over):
 
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32], ids=["bf16", "f32"])
 @pytest.mark.parametrize("swap", [False, True], ids=["own", "values_over_keys"])
-@pytest.mark.parametrize("T", [700, 3100])                        # 3100: apart, dK and dV come before dQ; in place, behind it
+@pytest.mark.parametrize("T", [700, 3100])
 def test_key_and_value_gradients_written_over_keys_and_values(mka, dtype, swap, T):
     B, H, d, W = 2, 6, 64, 100
     P = problem(74, B, H, T, d, (T, T, 90), 32, dtype, router_std=0.3, with_dO=True)
@@ -77,5 +77,24 @@ def test_key_and_value_gradients_written_over_keys_and_values(mka, dtype, swap, 
     apart = mka.mka_bwd(shape, P["Q"], P["K"], P["V"], gate, O, LSE, P["dO"])
     dK, dV = (P["V"], P["K"]) if swap else (P["K"], P["V"])
     got = mka.mka_bwd(shape, P["Q"], P["K"], P["V"], gate, O, LSE, P["dO"], dK=dK, dV=dV)
+    assert torch.equal(got["dQ"], apart["dQ"]) and torch.equal(got["dG"], apart["dG"])
+    for l in range(3): assert torch.equal(dK[l], apart["dK"][l]) and torch.equal(dV[l], apart["dV"][l])
+
+
+@pytest.mark.parametrize("case", [(2, 8, 2, 1000, 64, 100, 90), (2, 12, 2, 700, 128, 256, 200), (1, 2, 2, 5200, 64, 64, 40)], ids=["G4", "G6", "two_heads"])
+@pytest.mark.parametrize("swap", [False, True], ids=["own", "values_over_keys"])
+def test_both_orders_of_the_two_kernels_give_the_same_bits(mka, case, swap):
+    """Sizes at which dK and dV come before dQ when they are written apart, and behind it when written over keys or values."""
+    B, H, Hkv, T, d, W, n3 = case
+    g = torch.Generator(device="cuda").manual_seed(75)
+    mk = lambda *n: torch.randn(*n, device="cuda", dtype=torch.bfloat16, generator=g)
+    N = (T, T, n3)
+    Q, dO, K, V = mk(B, H, T, d), mk(B, H, T, d), [mk(B, Hkv, n, d) for n in N], [mk(B, Hkv, n, d) for n in N]
+    gate = torch.softmax(torch.randn(B, T, 3, device="cuda", generator=g), -1).contiguous()
+    shape = mka.make_shape(B, H, T, d, 64, W, kv_heads=Hkv)
+    O, LSE = mka.mka_fwd(shape, Q, K, V, gate)
+    apart = mka.mka_bwd(shape, Q, K, V, gate, O, LSE, dO)
+    dK, dV = (V, K) if swap else (K, V)
+    got = mka.mka_bwd(shape, Q, K, V, gate, O, LSE, dO, dK=dK, dV=dV)
     assert torch.equal(got["dQ"], apart["dQ"]) and torch.equal(got["dG"], apart["dG"])
     for l in range(3): assert torch.equal(dK[l], apart["dK"][l]) and torch.equal(dV[l], apart["dV"][l])

@@ -206,7 +206,7 @@ def test_forward_wait_runs_out_within_ranges(mka, short_limit, case):
 def test_backward_wait_runs_out_with_dq_under_it(mka, short_limit, d):
     """Grouped heads whose key tiles walk 32 query tiles: dK and dV come first, and dQ's items run under their tail, which here is a wait that
     runs out."""
-    B, H, Hkv, T, W, N = 1, 8, 2, 1000, 96, (1000, 1000, 160)
+    B, H, Hkv, T, W, N = 1, 16, 4, 1000, 96, (1000, 1000, 160)
     g = torch.Generator(device="cuda").manual_seed(98)
     mk = lambda *n: torch.randn(*n, device="cuda", dtype=torch.bfloat16, generator=g)
     Q, dO, K, V = mk(B, H, T, d), mk(B, H, T, d), [mk(B, Hkv, n, d) for n in N], [mk(B, Hkv, n, d) for n in N]
