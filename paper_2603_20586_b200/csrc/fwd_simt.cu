@@ -6,6 +6,8 @@
 // fp32 arithmetic throughout, so this is the kernel for fp32 problems (tolerance 1e-4) and the
 // on-GPU cross-check of the tensor-core kernel.  One CTA = 16 or 32 query rows of one (batch, head), see simt.cuh; a key tile of
 // 32 rows is staged in shared memory as fp32 and each lane scores one key of the tile, four columns at a time.
+#include <type_traits>
+
 #include "simt.cuh"
 
 namespace mka {
@@ -153,7 +155,10 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
     for (int s = 0; s < NS; ++s) {
         const float* o = tiles + (row * NS + s) * kState;
         constexpr int kGroupFloats = kRows * NS * kState;
-        float M = -INFINITY, Z = 0.f, A[CPL];
+        // Eight groups' sums are added up in 64 bits, so that LSE is no further off than with the four groups of twice the rows (in 32 bits:
+        // 0.4 to 2.3 % further on average over inputs, now 1.2 to 1.6 % less; nothing to be seen in the time).
+        std::conditional_t<S::kGroups == 8, double, float> sum = 0;
+        float M = -INFINITY, A[CPL];
 #pragma unroll
         for (int g = 0; g < S::kGroups; ++g) M = fmaxf(M, o[g * kGroupFloats]);
 #pragma unroll
@@ -161,10 +166,11 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
 #pragma unroll
         for (int g = 0; g < S::kGroups; ++g) {
             const float mg = o[g * kGroupFloats], f = mg == -INFINITY ? 0.f : expf(mg - M);
-            Z = fmaf(o[g * kGroupFloats + 1], f, Z);
+            sum = fma(static_cast<decltype(sum)>(o[g * kGroupFloats + 1]), static_cast<decltype(sum)>(f), sum);
 #pragma unroll
             for (int k = 0; k < CPL; ++k) A[k] = fmaf(o[g * kGroupFloats + 2 + lane + 32 * k], f, A[k]);
         }
+        const float Z = static_cast<float>(sum);
         float w;
         if (MODE == MKA_MODE_FAST) {
             w = Z > 0.f ? 1.f / Z : 0.f;

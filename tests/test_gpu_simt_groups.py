@@ -45,3 +45,19 @@ def test_forward_and_backward_match_the_oracle(mka, orc, case):
     # gradients sum up to T terms each: the contract's bound grows with the largest of them
     for name, got, want in [("dQ", g["dQ"], ref["dQ"])] + [(f"d{k}{l}", g[f"d{k}"][l], ref[f"d{k}"][l]) for k in "KV" for l in range(3)]:
         assert err(got, want)[0] <= F32_MAX * max(1.0, np.abs(want).max()), name
+
+
+def test_small_sums_of_the_groups_are_kept(mka):
+    """Eight tiles of 32 slots, one to a group: a weight of 1 in the first, one of 0.4 * 2^-23 in each of the others.  Their sum is 1 + 2.8 * 2^-23;
+    the nearest float and its logarithm (an ulp, 6e-8) leave LSE within 1e-7, added up one after the other in fp32 the seven are lost (3.3e-7)."""
+    B, H, T, d, n = 1, 1, 16, 32, 256
+    small = 0.4 * 2.0 ** -23
+    Q, K, V = (torch.zeros(B, H, rows, d, device="cuda") for rows in (T, n, n))
+    Q[..., 0] = 1.0
+    K[..., 0] = -1000.0
+    K[:, :, ::32, 0] = float(np.log(small))
+    K[:, :, 0, 0] = 0.0
+    gate = torch.tensor([0.0, 0.0, 1.0], device="cuda").repeat(B, T, 1).contiguous()
+    shape = mka.make_shape(B, H, T, d, 32, 1, scale=1.0, dtype=mka.binding.MKA_F32)
+    _, LSE = mka.mka_fwd(shape, Q, [None, None, K], [None, None, V], gate)
+    assert (LSE.double() - np.log(1.0 + 7 * small)).abs().max().item() <= 1e-7
