@@ -227,7 +227,7 @@ def mka_fwd(shape: mka_shape, Q, K, V, gate, O=None, LSE=None, ws=None, stream=N
         O = torch.empty_like(Q)
     if LSE is None and want_lse and shape.mode == MKA_MODE_FAST:
         LSE = _empty_f32(Q, 3, 0)
-    n = [0 if k is None else k.shape[2] for k in K]
+    n = [0 if K[l] is None else K[l].shape[2] for l in range(3)]
     if ws is None:
         ws = alloc_workspace(shape, n, MKA_WS_FWD, Q.device)
     tmp = _fwd_scratch(shape, 0, _Rows(*n), Q.device) if stream is None else None
@@ -276,7 +276,9 @@ def mka_fwd_paged(shape: mka_shape, H_kv: int, Q, pools_k, pools_v, tables, n, g
         LSE = _empty_f32(Q, 3, 0)
     if ws is None:
         ws = torch.zeros(256, dtype=torch.uint8, device=Q.device)
-    tmp = _fwd_scratch(shape, H_kv, _n_level(n), Q.device) if stream is None and (rows is None or not any(r is not None for r in rows)) else None
+    tmp = None
+    if stream is None and (rows is None or not any(r is not None for r in rows)):
+        tmp = _fwd_scratch(shape, H_kv, _Rows(*[0 if pools_k[l] is None else int(n[l]) for l in range(3)]), Q.device)
     _check(lib.mka_fwd_paged_with_scratch(ctypes.byref(shape), H_kv, _ptr(Q), _paged_levels(pools_k, pools_v, tables, rows, n), _ptr(gate),
                                           _ptr(O), _ptr(LSE), _ptr(ws), ws.numel(), _ptr(tmp), 0 if tmp is None else tmp.numel(),
                                           _stream(stream)), "mka_fwd_paged")
@@ -367,7 +369,7 @@ def mka_bwd(shape: mka_shape, Q, K, V, gate, O, LSE, dO, R=None, dQ=None, dK=Non
             dW_r = torch.empty((R.shape[-1], 3), dtype=torch.float32, device=dev)
         if db_r is None:
             db_r = torch.empty((3,), dtype=torch.float32, device=dev)
-    grads = _host_args.grads([None if K[l] is None or K[l].shape[2] == 0 else dK[l] for l in range(3)], dV)
+    grads = _host_args.grads(K, dK, dV)
     if ws is None:
         ws = alloc_workspace(shape, [0 if k is None else k.shape[2] for k in K], MKA_WS_BWD, dev)
     _check(lib.mka_bwd(ctypes.byref(shape), _ptr(Q), _levels(K, V), _ptr(gate), _ptr(O), _ptr(LSE), _ptr(dO),

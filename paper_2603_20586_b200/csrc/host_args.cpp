@@ -27,22 +27,43 @@ struct Held {                                        // a reference of our own
     Held(const Held&) = delete;
     Held& operator=(const Held&) = delete;
 };
-struct Seq : Held {                                  // a list or tuple (or what can be made one), held while it is read
-    explicit Seq(PyObject* x) : Held(PySequence_Fast(x, "a sequence of tensors is expected")) {}
-    Py_ssize_t size() const { return PySequence_Fast_GET_SIZE(o); }
-    PyObject* at(Py_ssize_t i) const {
-        if (i >= size()) throw Bad();
-        return PySequence_Fast_GET_ITEM(o, i);
+// Entries of a list or tuple, or of whatever else answers x[i] (then held as long as this is).
+class Seq {
+    PyObject* x_;
+    const bool plain_;
+    std::vector<PyObject*> held_;
+
+  public:
+    explicit Seq(PyObject* x) : x_(x), plain_(PyList_Check(x) || PyTuple_Check(x)) { Py_INCREF(x_); }
+    ~Seq() {
+        for (PyObject* h : held_) Py_DECREF(h);
+        Py_DECREF(x_);
     }
-    const at::Tensor* tensor_at(Py_ssize_t i) const {         // nullptr for None
+    Seq(const Seq&) = delete;
+    Seq& operator=(const Seq&) = delete;
+    PyObject* at(Py_ssize_t i) {
+        if (plain_ && i < PySequence_Fast_GET_SIZE(x_)) return PySequence_Fast_GET_ITEM(x_, i);
+        const Held at(PyLong_FromSsize_t(i));
+        PyObject* item = PyObject_GetItem(x_, at.o);
+        if (!item) throw PyErrSet();
+        held_.push_back(item);
+        return item;
+    }
+    const at::Tensor* tensor_at(Py_ssize_t i) {               // nullptr for None
         PyObject* x = at(i);
         return x == Py_None ? nullptr : &tensor(x);
     }
 };
 
 int64_t address(const at::Tensor& t) { return static_cast<int64_t>(reinterpret_cast<intptr_t>(t.data_ptr())); }
-int64_t integer(PyObject* o) {
-    const int64_t v = PyLong_AsLongLong(o);
+int64_t integer(PyObject* o) {                       // int(o)
+    int64_t v;
+    if (PyLong_CheckExact(o)) {
+        v = PyLong_AsLongLong(o);
+    } else {
+        const Held whole(PyNumber_Long(o));
+        v = PyLong_AsLongLong(whole.o);
+    }
     if (v == -1 && PyErr_Occurred()) throw PyErrSet();
     return v;
 }
@@ -71,42 +92,57 @@ PyObject* guarded(F f) {
     END_HANDLE_TH_ERRORS
 }
 
-// Words of mka_level[3] or mka_level_grad[3]: k, v, n, stride_b, stride_h, stride_n; zeros for a level that is None or has no rows.
-template <typename Check>
-PyObject* three_levels(PyObject* const* a, Py_ssize_t n, Check check) {
+// Words of a level: k, v, n, stride_b, stride_h, stride_n; zeros where keys are None or have no rows.
+void put_level(int64_t* o, const at::Tensor& k, const at::Tensor& v) {
+    o[0] = address(k); o[1] = address(v); o[2] = k.size(2);
+    for (int i = 0; i < 3; ++i) o[3 + i] = k.stride(i);
+}
+PyObject* levels(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
         if (n != 2) throw Bad();
-        const Seq K(a[0]), V(a[1]);
+        Seq K(a[0]), V(a[1]);
         int64_t w[18] = {};
         for (int l = 0; l < 3; ++l) {
             const at::Tensor* k = K.tensor_at(l);
             if (!k || k->size(2) == 0) continue;
             const at::Tensor* v = V.tensor_at(l);
             if (!v) throw Bad();
-            check(*k, *v);
-            int64_t* o = w + 6 * l;
-            o[0] = address(*k); o[1] = address(*v); o[2] = k->size(2);
-            for (int i = 0; i < 3; ++i) o[3 + i] = k->stride(i);
+            check_pair(*k, *v);
+            put_level(w + 6 * l, *k, *v);
         }
         return bytes(w);
     });
 }
-PyObject* levels(PyObject*, PyObject* const* a, Py_ssize_t n) { return three_levels(a, n, check_pair); }
-PyObject* grads(PyObject*, PyObject* const* a, Py_ssize_t n) { return three_levels(a, n, check_layout); }
+PyObject* grads(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    return guarded([&]() -> PyObject* {
+        if (n != 3) throw Bad();
+        Seq K(a[0]), dK(a[1]), dV(a[2]);
+        int64_t w[18] = {};
+        for (int l = 0; l < 3; ++l) {
+            const at::Tensor* k = K.tensor_at(l);
+            if (!k || k->size(2) == 0) continue;
+            const at::Tensor *dk = dK.tensor_at(l), *dv = dV.tensor_at(l);
+            if (!dk || !dv) throw Bad();
+            check_layout(*dk, *dv);
+            put_level(w + 6 * l, *dk, *dv);
+        }
+        return bytes(w);
+    });
+}
 
 PyObject* paged_levels(PyObject*, PyObject* const* a, Py_ssize_t n_args) {
     return guarded([&]() -> PyObject* {
         if (n_args != 5) throw Bad();
-        const Seq K(a[0]), V(a[1]), tabs(a[2]), n(a[4]);
+        Seq K(a[0]), V(a[1]), tabs(a[2]), rows(a[3]), n(a[4]);
         const bool counted = a[3] != Py_None;
-        const Seq rows(counted ? a[3] : a[4]);
         int64_t w[36] = {};
         for (int l = 0; l < 3; ++l) {
             int64_t* o = w + 12 * l;
             o[7] = 1;
-            const int64_t most = integer(n.at(l));
             const at::Tensor* k = K.tensor_at(l);
-            if (!k || most == 0) continue;
+            if (!k) continue;
+            const int64_t most = integer(n.at(l));
+            if (most == 0) continue;
             const at::Tensor *v = V.tensor_at(l), *tab = tabs.tensor_at(l), *r = counted ? rows.tensor_at(l) : nullptr;
             if (!v || !tab) throw Bad();
             check_pair(*k, *v);
@@ -137,12 +173,13 @@ PyObject* paged_level(PyObject*, PyObject* const* a, Py_ssize_t n) {
 PyObject* empties_like(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
         if (n != 1) throw Bad();
-        const Seq in(a[0]);
-        Held out(PyList_New(in.size()));
-        for (Py_ssize_t i = 0; i < in.size(); ++i) {
-            const at::Tensor* t = in.tensor_at(i);
-            PyObject* o = t ? THPVariable_Wrap(at::empty_like(*t)) : Py_None;
-            if (!t) Py_INCREF(o);
+        const Held in(PySequence_Fast(a[0], "a sequence of tensors is expected"));
+        const Py_ssize_t size = PySequence_Fast_GET_SIZE(in.o);
+        Held out(PyList_New(size));
+        for (Py_ssize_t i = 0; i < size; ++i) {
+            PyObject* x = PySequence_Fast_GET_ITEM(in.o, i);
+            PyObject* o = x == Py_None ? Py_None : THPVariable_Wrap(at::empty_like(tensor(x)));
+            if (x == Py_None) Py_INCREF(o);
             PyList_SET_ITEM(out.o, i, o);
         }
         Py_INCREF(out.o);
@@ -167,7 +204,7 @@ template <typename F> PyMethodDef method(const char* name, F f, const char* doc)
 }
 PyMethodDef methods[] = {
     method("levels", levels, "levels(K, V) -> mka_level[3] as bytes; None or no rows: an absent level"),
-    method("grads", grads, "grads(dK, dV) -> mka_level_grad[3] as bytes"),
+    method("grads", grads, "grads(K, dK, dV) -> mka_level_grad[3] as bytes; a level absent from K is absent"),
     method("paged_levels", paged_levels, "paged_levels(pools_k, pools_v, tables, rows or None, n) -> mka_paged_level[3] as bytes"),
     method("paged_level", paged_level, "paged_level(pool_k, pool_v, table) -> one mka_paged_level over the table's width as bytes"),
     method("empties_like", empties_like, "empties_like(tensors) -> list of empty_like, None for None"),

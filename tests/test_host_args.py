@@ -56,3 +56,31 @@ def test_outputs():
     assert mka._empty_f32(q, 0, 0).shape == () and mka._empty_f32(q, 4, 0).dtype == torch.float32
     a, none = mka._host_args.empties_like([q, None])
     assert none is None and a.shape == q.shape and a.dtype == q.dtype and a.stride() == q.stride()
+
+
+def test_what_answers_an_index_is_taken():
+    k, v, tab = _t(2, 3, 40, 64), _t(2, 3, 40, 64), _t(3, 4, dtype=torch.int32)
+    want = mka._levels([k, None, k], [v, None, v])
+    assert mka._levels({0: k, 1: None, 2: k}, {0: v, 2: v}) == want and mka._levels([k, None, k, None], (v, None, v)) == want
+    both = torch.stack([k, k, k])
+    assert _words(mka._levels(both, both))[6] == both[1].data_ptr()
+    with pytest.raises(IndexError):
+        mka._levels([k], [v])
+
+
+def test_rows_of_paged_levels_are_whole_numbers_by_value():
+    pk, pv, tab = _t(9, 2, 16, 64), _t(9, 2, 16, 64), _t(3, 4, dtype=torch.int32)
+    want = mka._paged_levels([pk, None, pk], [pv, None, pv], [tab, None, tab], None, [60, 0, 33])
+    for n in ([60.0, None, 33.9], [torch.tensor(60), "absent", 33], {0: 60, 2: 33}):           # beside a pool of None nothing is looked at
+        assert mka._paged_levels([pk, None, pk], [pv, None, pv], [tab, None, tab], None, n) == want
+    with pytest.raises(TypeError):
+        mka._paged_levels([pk, None, None], [pv, None, None], [tab, None, None], None, [None, 0, 0])
+
+
+def test_gradients_follow_the_keys():
+    k, g, h = _t(2, 3, 40, 64), _t(2, 3, 40, 64), _t(2, 3, 40, 64)
+    w = _words(mka._host_args.grads([k, None, k[:, :, :0]], [g, g, None], [h, h, None]))
+    assert w[:6] == (g.data_ptr(), h.data_ptr(), 40, *g.stride()[:3]) and w[6:] == (0,) * 12
+    for dk, dv in ((None, h), (g, None), (g, h.transpose(2, 3)), (g.transpose(2, 3), h.transpose(2, 3))):
+        with pytest.raises(AssertionError):                                                     # keys without room for their gradients
+            mka._host_args.grads([k, None, None], [dk, None, None], [dv, None, None])
