@@ -7,16 +7,27 @@ library has not been built the import fails, and every call raises ``MkaError`` 
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from typing import Optional, Sequence
 
 import torch
 
-try:
-    from . import _host_args
-except ImportError as e:
-    raise ImportError("the binding's host module is missing: build it with `python -m paper_2603_20586_b200.build` "
-                      "(there is no fallback path)") from e
+from .build import host_module
+
+
+def _load_host_args():
+    path = host_module()
+    if not os.path.exists(path):
+        raise ImportError(f"{path}, the binding's host module for this Python and torch, is missing: build it with "
+                          "`python -m paper_2603_20586_b200.build` (there is no fallback path)")
+    spec = importlib.util.spec_from_file_location(f"{__package__}._host_args", path)
+    module = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(module)
+    return module
+
+
+_host_args = _load_host_args()
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libmka_b200.so")

@@ -17,7 +17,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmka_b200.so")
-HOST_SRC, HOST_MODULE = os.path.join(CSRC, "host_args.cpp"), os.path.join(HERE, "_host_args.so")
+HOST_SRC = os.path.join(CSRC, "host_args.cpp")
 OBJ_DIR = os.path.join(HERE, "_build")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -36,8 +36,14 @@ def _stale(target, deps):
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def host_module() -> str:
+    """Path of the binding's argument marshalling (host only).  It is compiled against torch's and Python's headers, so each of their
+    versions has a file of its own: one that was built for others is neither loaded nor taken for up to date."""
+    import torch
+    return os.path.join(HERE, f"_host_args.{sys.implementation.cache_tag}.torch-{torch.__version__}-{str(torch.version.git_version)[:8]}.so")
+
+
 def _host_module_cmd(out):
-    """The binding's argument marshalling (host only): a Python module against the installed torch."""
     import sysconfig
 
     import torch
@@ -75,10 +81,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
         tmp = LIB + f".{os.getpid()}.tmp"
         run([NVCC, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", tmp] + objs + ["-cudart", "static"])
         os.replace(tmp, LIB)
-    if force or _stale(HOST_MODULE, [HOST_SRC]):
-        tmp = HOST_MODULE + f".{os.getpid()}.tmp"
+    host = host_module()
+    if force or _stale(host, [HOST_SRC]):
+        tmp = host + f".{os.getpid()}.tmp"
         run(_host_module_cmd(tmp))
-        os.replace(tmp, HOST_MODULE)
+        os.replace(tmp, host)
     return LIB
 
 

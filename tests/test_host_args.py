@@ -1,5 +1,6 @@
 """The binding's native marshalling: the words it writes for levels, gradients and paged levels, and what it refuses (no GPU)."""
 import struct
+import sys
 
 import pytest
 import torch
@@ -84,3 +85,16 @@ def test_gradients_follow_the_keys():
     for dk, dv in ((None, h), (g, None), (g, h.transpose(2, 3)), (g.transpose(2, 3), h.transpose(2, 3))):
         with pytest.raises(AssertionError):                                                     # keys without room for their gradients
             mka._host_args.grads([k, None, None], [dk, None, None], [dv, None, None])
+
+
+def test_module_of_another_torch_or_python_is_not_loaded(monkeypatch):
+    from paper_2603_20586_b200 import build
+    own = build.host_module()
+    assert mka._host_args.__file__ == own and not build._stale(own, [build.HOST_SRC])
+    monkeypatch.setattr(torch, "__version__", torch.__version__ + ".later")
+    assert build.host_module() != own and build._stale(build.host_module(), [build.HOST_SRC])
+    with pytest.raises(ImportError, match="later"):
+        mka._load_host_args()
+    monkeypatch.undo()
+    monkeypatch.setattr(sys.implementation, "cache_tag", "cpython-999")
+    assert build.host_module() != own
