@@ -220,19 +220,29 @@ def alloc_workspace(shape: mka_shape, n_level, which: int, device) -> torch.Tens
     return torch.empty(mka_workspace_bytes(shape, n_level, which), dtype=torch.uint8, device=device)
 
 
-def _fwd_scratch(shape: mka_shape, H_kv: int, n_level, device) -> Optional[torch.Tensor]:
-    """Room for the forward's partial results, from the caller's stream like its outputs, or None where it has no use for any."""
+def _fwd_scratch(shape: mka_shape, H_kv: int, n_level, device, stream) -> Optional[torch.Tensor]:
+    """Room for the forward's partial results on the call's stream, or None where it has no use for any."""
     q_tiles = shape.B * shape.H * ((shape.T + 127) // 128)
     if q_tiles > 4 * 148 * 2 or q_tiles * sum(n_level) < 148 * 4 * 128:      # many blocks, or little to share out: not worth the question
         return None
     nbytes = lib.mka_fwd_scratch_bytes(shape, H_kv, n_level)
+    if nbytes == 0:
+        return None
     try:
-        return torch.empty(nbytes, dtype=torch.uint8, device=device) if nbytes else None
+        if stream is None:
+            return torch.empty(nbytes, dtype=torch.uint8, device=device)
+        # from the allocator's blocks of that stream, to which it goes back when the call has been queued there
+        with torch.cuda.stream(stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(stream.cuda_stream, device)):
+            return torch.empty(nbytes, dtype=torch.uint8, device=device)
     except torch.OutOfMemoryError:                                           # the call runs without, as it would have
         return None
 
 
 def mka_fwd(shape: mka_shape, Q, K, V, gate, O=None, LSE=None, ws=None, stream=None, want_lse=True):
+    """Fused forward over dense levels.  Where few blocks of rows would leave SMs idle (short chunks with long caches) the call takes up to 39 MB
+    of scratch memory for partial results from torch's allocator, on the call's stream, and gives it back when it is queued; so a
+    CUDA graph of it is captured with torch.cuda.graph.  Where that memory is not to be had, and through the C entry without scratch, the
+    key lists are cut in another way, and O may differ by a rounding to bf16, LSE by some 1e-7 of its size."""
     assert Q.is_contiguous() and gate.is_contiguous() and gate.dtype == torch.float32
     if O is None:
         O = torch.empty_like(Q)
@@ -241,7 +251,7 @@ def mka_fwd(shape: mka_shape, Q, K, V, gate, O=None, LSE=None, ws=None, stream=N
     n = [0 if K[l] is None else K[l].shape[2] for l in range(3)]
     if ws is None:
         ws = alloc_workspace(shape, n, MKA_WS_FWD, Q.device)
-    tmp = _fwd_scratch(shape, 0, _Rows(*n), Q.device) if stream is None else None
+    tmp = _fwd_scratch(shape, 0, _Rows(*n), Q.device, stream)
     _check(lib.mka_fwd_with_scratch(ctypes.byref(shape), _ptr(Q), _levels(K, V), _ptr(gate), _ptr(O), _ptr(LSE), _ptr(ws), ws.numel(),
                                     _ptr(tmp), 0 if tmp is None else tmp.numel(), _stream(stream)), "mka_fwd")
     return O, LSE
@@ -278,7 +288,7 @@ def mka_fuse_kv_paged(K, V, gate, pool_k, pool_v, table, dst_offset=0, dst_offse
 def mka_fwd_paged(shape: mka_shape, H_kv: int, Q, pools_k, pools_v, tables, n, gate, rows=None, O=None, LSE=None, ws=None,
                   stream=None):
     """mka_fwd over paged levels with grouped-query head sharing (n[l]: upper bound of the rows on level l; rows[l]:
-    int32 [B] rows of every sequence, or None)."""
+    int32 [B] rows of every sequence, or None).  Scratch memory as in mka_fwd."""
     assert Q.is_contiguous() and gate.is_contiguous() and gate.dtype == torch.float32
     B, H, T, d = Q.shape
     if O is None:
@@ -288,8 +298,8 @@ def mka_fwd_paged(shape: mka_shape, H_kv: int, Q, pools_k, pools_v, tables, n, g
     if ws is None:
         ws = torch.zeros(256, dtype=torch.uint8, device=Q.device)
     tmp = None
-    if stream is None and (rows is None or not any(r is not None for r in rows)):
-        tmp = _fwd_scratch(shape, H_kv, _Rows(*[0 if pools_k[l] is None else int(n[l]) for l in range(3)]), Q.device)
+    if rows is None or not any(r is not None for r in rows):
+        tmp = _fwd_scratch(shape, H_kv, _Rows(*[0 if pools_k[l] is None else int(n[l]) for l in range(3)]), Q.device, stream)
     _check(lib.mka_fwd_paged_with_scratch(ctypes.byref(shape), H_kv, _ptr(Q), _paged_levels(pools_k, pools_v, tables, rows, n), _ptr(gate),
                                           _ptr(O), _ptr(LSE), _ptr(ws), ws.numel(), _ptr(tmp), 0 if tmp is None else tmp.numel(),
                                           _stream(stream)), "mka_fwd_paged")

@@ -139,3 +139,32 @@ def test_small_weights_of_a_row_are_kept(mka):
     O, LSE = mka.mka_fwd(shape, Q, [None, None, K], [None, None, V], gate)
     assert (LSE.double() - np.log(4.0 + 2.0 ** -18)).abs().max().item() <= 4e-7
     assert torch.equal(O, torch.ones_like(O) * (torch.arange(d, device="cuda") == 3))
+
+
+def test_a_stream_of_the_callers_gives_the_same_bits(mka):
+    """The partial results of a call on a stream of its own lie in memory of that stream: other streams' allocations do not run into it."""
+    B, H, Hkv, T, d, W, q_off, n3 = RANGES[0]
+    N = (q_off + T, q_off + T, n3)
+    g = torch.Generator(device="cuda").manual_seed(6)
+    mk = lambda *n: torch.randn(*n, device="cuda", dtype=torch.bfloat16, generator=g)
+    Q, K, V = mk(B, H, T, d), [mk(B, Hkv, n, d) for n in N], [mk(B, Hkv, n, d) for n in N]
+    gate = torch.softmax(torch.randn(B, T, 3, device="cuda", generator=g), -1).contiguous()
+    shape = mka.make_shape(B, H, T, d, 64, W, q_off, kv_heads=Hkv)
+    need = _need(mka, shape, N)
+    assert need > 0
+    want, want_lse = mka.mka_fwd(shape, Q, K, V, gate)
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+
+    class Handle:                                                     # anything that has a cuda_stream is a stream to the binding
+        cuda_stream = side.cuda_stream
+
+    for stream in (side, Handle()):
+        outs = [(torch.empty_like(Q), torch.empty_like(want_lse), torch.zeros(256, dtype=torch.uint8, device="cuda")) for _ in range(8)]
+        side.wait_stream(torch.cuda.current_stream())
+        for O, LSE, ws in outs:
+            mka.mka_fwd(shape, Q, K, V, gate, O=O, LSE=LSE, ws=ws, stream=stream)
+            torch.full((need,), 255, dtype=torch.uint8, device="cuda")  # on the current stream, beside the call
+        torch.cuda.synchronize()
+        for O, LSE, ws in outs:
+            assert mka.mka_device_status(ws) == 0 and torch.equal(O, want) and torch.equal(LSE, want_lse)
