@@ -1,4 +1,6 @@
 """GPU parity of the fused forward over paged levels (grouped-query heads) against the oracle, through the C ABI."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -111,3 +113,72 @@ def test_paged_forward_rejects_what_it_does_not_do(mka):
         mka.mka_fwd_paged(mka.make_shape(1, 4, T, 128, 32, 32, flags=1), 2, Q, P["pools_k"], P["pools_v"], P["tables"],
                           list(cfg.N), gate)
     assert e.value.code == 5
+
+
+# B, H, KV heads, T, d, window, q_offset, rows of the long-term level, rows of a page, a table for every KV head
+RANGES = [
+    (1, 12, 4, 949, 128, 1750, 3804, 144, 16, False),
+    (2, 12, 4, 871, 128, 859, 2175, 3765, 256, False),        # pages longer than a tile, two sequences, heads in pairs and one alone
+    (1, 28, 4, 301, 128, 500, 20000, 0, 8, True),             # no long-term level
+    (2, 32, 32, 627, 64, 2630, 0, 7815, 16, True),
+    (2, 32, 32, 627, 64, 2630, 0, 7815, 256, False),
+]
+
+
+@pytest.mark.parametrize("case", RANGES, ids=lambda c: f"d{c[4]}page{c[8]}")
+def test_paged_levels_in_equal_ranges(mka, orc, case):
+    """Sizes at which the key tiles are cut into equal ranges, with scratch memory.  Every row that no sequence owns is NaN, also those after a
+    level's last row in a piece that holds its last tile.  The dense form over the gathered levels makes the same pieces, bit for bit."""
+    B, H, Hkv, T, d, W, q_off, n3, page, per_head = case
+    N = (q_off + T, q_off + T, n3)
+    g = torch.Generator(device="cuda").manual_seed(61)
+    mk = lambda *n: torch.randn(*n, device="cuda", dtype=torch.bfloat16, generator=g)
+    Q, K, V = mk(B, H, T, d), [mk(B, Hkv, n, d) for n in N], [mk(B, Hkv, n, d) for n in N]
+    gate = torch.softmax(torch.randn(B, T, 3, device="cuda", generator=g), -1).contiguous()
+    gate[:, ::7, 0] = 0.0
+    pools, tabs = ([], []), []
+    for l, n in enumerate(N):
+        if n == 0:
+            pools[0].append(None), pools[1].append(None), tabs.append(None)
+            continue
+        width = -(-n // page)
+        lists = Hkv if per_head else 1
+        tab = torch.randperm(B * lists * width + 3, device="cuda", generator=g)[:B * lists * width].view(B, lists, width)
+        for pool, src in zip(pools, (K[l], V[l])):
+            x = torch.full((B, Hkv, width * page, d), float("nan"), device="cuda", dtype=torch.bfloat16)
+            x[:, :, :n] = src
+            x = x.view(B, Hkv, width, page, d)
+            pool.append(torch.full((B * lists * width + 3, Hkv, page, d), float("nan"), device="cuda", dtype=torch.bfloat16))
+            for h in range(Hkv):
+                pool[-1][tab[:, h if per_head else 0].reshape(-1), h] = x[:, h].reshape(-1, page, d)
+        tabs.append((tab if per_head else tab[:, 0]).to(torch.int32).contiguous())
+    shape = mka.make_shape(B, H, T, d, 32, W, q_off)
+    dense = mka.make_shape(B, H, T, d, 32, W, q_off, kv_heads=Hkv)
+    b, rows = mka.binding, (ctypes.c_int64 * 3)(*N)
+    need = int(mka.lib.mka_fwd_scratch_bytes(ctypes.byref(shape), Hkv, rows))
+    assert need > 0 and need == int(mka.lib.mka_fwd_scratch_bytes(ctypes.byref(dense), 0, rows))
+    ws = torch.full((256,), 0x55, dtype=torch.uint8, device="cuda")
+    O, LSE = mka.mka_fwd_paged(shape, Hkv, Q, *pools, tabs, N, gate, ws=ws)
+    assert mka.mka_device_status(ws) == 0
+    Od, Ld = mka.mka_fwd(dense, Q, K, V, gate)
+    assert torch.equal(O, Od) and torch.equal(LSE, Ld)
+
+    def through_c(scratch):                                   # without enough scratch: as without any
+        o, lse, tmp = torch.empty_like(O), torch.empty_like(LSE), torch.full((need,), 255, dtype=torch.uint8, device="cuda")
+        b._check(mka.lib.mka_fwd_paged_with_scratch(ctypes.byref(shape), Hkv, b._ptr(Q), b._paged_levels(*pools, tabs, None, N), b._ptr(gate), b._ptr(o),
+                                                    b._ptr(lse), b._ptr(ws), 256, b._ptr(tmp) if scratch else None, scratch, b._stream(None)), "c")
+        assert mka.mka_device_status(ws) == 0
+        return o, lse
+
+    a, la = through_c(need)
+    c, lc = through_c(0)
+    e, le = through_c(need - 256)
+    assert torch.equal(a, O) and torch.equal(la, LSE) and torch.equal(c, e) and torch.equal(lc, le)
+    # both cuts sum the same products in fp32: O differs by a rounding to bf16 (2^-8 of values below 2), LSE by some 2^-22 of its size
+    assert (a.float() - c.float()).abs().max().item() <= 2.0 ** -7 and (la - lc).abs().max().item() <= 2e-5
+    # and one head's last rows against the oracle
+    h, t0 = H - 1, T - 40
+    one = lambda x: np64(x[:1, h // (H // Hkv):h // (H // Hkv) + 1])
+    Or, Lr = orc.fwd(np64(Q[:1, h:h + 1, t0:]), [one(k) for k in K], [one(v) for v in V], np64(gate[:1, t0:]), W, q_off + t0)
+    check(O[:1, h:h + 1, t0:], Or, torch.bfloat16, "O against the oracle")
+    assert np.abs(np64(LSE[:1, h:h + 1, t0:]) - Lr).max() <= 2e-3
