@@ -1,5 +1,5 @@
-"""Gate gradient summed over the heads beside dK and dV: more sums than the CTAs of the key tiles take in one round, a remainder of a
-round, one key tile under many queries, and a short level alone."""
+"""Gate gradient summed over the heads: by a kernel of its own behind dQ (40,000 queries under one key tile: dK and dV come first), and beside dK
+and dV: a round of the CTAs and part of a second one (MORE), a remainder of a round, and a short level alone."""
 import numpy as np
 import pytest
 import torch
@@ -98,3 +98,25 @@ def test_both_orders_of_the_two_kernels_give_the_same_bits(mka, case, swap):
     got = mka.mka_bwd(shape, Q, K, V, gate, O, LSE, dO, dK=dK, dV=dV)
     assert torch.equal(got["dQ"], apart["dQ"]) and torch.equal(got["dG"], apart["dG"])
     for l in range(3): assert torch.equal(dK[l], apart["dK"][l]) and torch.equal(dV[l], apart["dV"][l])
+
+
+# walks of 20 and 23 query tiles, so dQ comes first; 313 and 218 pieces of sums (384 and 640 threads to a CTA) on 148 CTAs
+MORE = [(16, 2, 2500, 128, 64, (0, 0, 20)), (16, 3, 2900, 64, 64, (0, 0, 130))]
+
+
+@pytest.mark.parametrize("case", MORE, ids=lambda c: f"T{c[2]}H{c[1]}d{c[3]}")
+def test_sums_of_a_second_round_are_taken(mka, case):
+    B, H, T, d, W, N = case
+    g = torch.Generator(device="cuda").manual_seed(76)
+    mk = lambda *n: torch.randn(*n, device="cuda", dtype=torch.bfloat16, generator=g)
+    Q, dO, K, V = mk(B, H, T, d), mk(B, H, T, d), [mk(B, H, n, d) for n in N], [mk(B, H, n, d) for n in N]
+    gate = torch.softmax(torch.randn(B, T, 3, device="cuda", generator=g), -1).contiguous()
+    shape, single = (mka.make_shape(B, n, T, d, 64, W) for n in (H, 1))
+    O, LSE = mka.mka_fwd(shape, Q, K, V, gate)
+    fresh = lambda: torch.full_like(gate, float("nan"))
+    got = mka.mka_bwd(shape, Q, K, V, gate, O, LSE, dO, dG=fresh())["dG"]
+    want = torch.zeros_like(got)
+    for h in range(H):
+        one = lambda t: t[:, h:h + 1].contiguous()
+        want += mka.mka_bwd(single, one(Q), [one(k) for k in K], [one(v) for v in V], gate, one(O), one(LSE), one(dO), dG=fresh())["dG"]
+    assert bool(torch.isfinite(got).all()) and torch.equal(got, want)
