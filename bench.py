@@ -59,7 +59,7 @@ NCU_TRAFFIC = {
     "decode_partial_kernel@c4": (1.476457e9 + 4.163328e6, 2 * 32, "decode_partial_kernel_c4p.md", "decode.cu", "8ff55e2ca41e"),
     "bwd_dq_tc_kernel@c5": (220.270080e6 + 27.188992e6, 1 * 16, "bwd_tc_kernels_c5p.md", "bwd_tc.cu", "482b3652e285"),
     "bwd_dkv_tc_kernel@c5": (220.271360e6 + 117.273344e6, 1 * 16, "bwd_tc_kernels_c5p.md", "bwd_tc.cu", "482b3652e285"),
-    "l2_summary_seg_kernel@s3": (100.699392e6 + 54.012160e6, 12288.0 / 32768.0, "l2_summary_seg_kernel_s3p.md", "summary_seg.cu", "f824f10a3d76"),   # 12288 of the 32768 tokens
+    "l2_summary_pipe_kernel@s3": (100.699392e6 + 54.012160e6, 12288.0 / 32768.0, "l2_summary_seg_kernel_s3p.md", "summary_seg.cu", "f824f10a3d76"),   # 12288 of the 32768 tokens
     "fuse_kv_kernel@f3": (403.136512e6 + 83.408640e6, 1 * 8, "fuse_kv_kernel_f3p.md", "fuse_kv.cu", "b1ef4c991e47"),
     "decode_paged_kernel@g4": (293.730304e6 + 3.355136e6, 1 * 4, "decode_paged_kernel_g4p.md", "decode_paged.cu", "929e98e72397"),   # one of the four sequences (g4p)
     "l3_index_kernel@r3": (134.305792e6 + 4.221696e6, 1, "l3_index_kernel_r3p.md", "l3.cu", "607ee4fa9ab7"),            # one of the four sequences (r3p)
@@ -421,8 +421,8 @@ def leg_report(leg, ms_per_step, n_gpus, peaks):
                          ncu_traffic("decode_paged_kernel@g4", cfg) if tag == "g4" else none)
     elif leg.kind == "summary":
         work, unit, metric = w["summary_bytes"], "GB/s", "l2_summary_hbm_gbs"
-        roof = _hbm_roof("l2_summary_seg_kernel", work / (k["main"] * 1e-3) / 1e9, peaks,
-                         ncu_traffic("l2_summary_seg_kernel@s3", cfg) if tag == "s3" else none)
+        roof = _hbm_roof("l2_summary_pipe_kernel", work / (k["main"] * 1e-3) / 1e9, peaks,
+                         ncu_traffic("l2_summary_pipe_kernel@s3", cfg) if tag == "s3" else none)
     elif leg.kind == "fuse":
         work, unit, metric = w["fuse_bytes"], "GB/s", "route_fuse_hbm_gbs"
         roof = _hbm_roof("fuse_kv_kernel", work / (k["main"] * 1e-3) / 1e9, peaks,

@@ -1159,8 +1159,7 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
     if (tid == 0 && wait_ctl.abort) atomicExch(p.status, (unsigned int)MKA_ERR_TIMEOUT);
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
     // The gate gradient's sums over the heads, left to the CTAs that are done with their key tiles first: a ticket is a sum per
-    // thread, the first one taken under the epilogue.  As a launch behind this one they took 5 us: a step at [2, 16 on 4, 1000, 128] 140.7 -> 138.0 us,
-    // at [1, 8, 700, 128] 60.0 -> 57.6.
+    // thread, the first one taken under the epilogue.  As a launch behind this one they took 5 us: a step at [1, 8, 700, 128] 60.0 -> 57.6.
     chain_wait();
     const long long per_batch = p.T * 3LL;
     for (;;) {

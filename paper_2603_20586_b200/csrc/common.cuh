@@ -10,12 +10,16 @@
 
 namespace mka {
 
-// Every kernel of the library is launched so that it may start while the kernel before it in the stream still runs (programmatic
-// dependent launch): its CTAs take the SMs' free places, set up what needs no memory and wait in chain_wait for the end of that
-// kernel and for its writes.  One after the other a boundary costs about 2 us of drain, launch and set-up (measured between the
+// The kernels of the library are launched so that they may start while the kernel before them in the stream still runs (programmatic
+// dependent launch; not the two forms of the session summary that follow a clearing of their scratch): a kernel's CTAs take the SMs' free
+// places, set up what needs no memory and wait in chain_wait for the end of the kernel before and for its writes.  One after the other a boundary costs about 2 us of drain, launch and set-up (measured between the
 // kernels of a serving step and of a backward), as much as half of the short kernels take.  Nothing in global memory is read or
 // written, and no tensor memory allocated (the kernel before may not have taken its own yet), in front of chain_wait;
 // chain_trigger stands at the start, since a waiting CTA costs nothing: the next kernel starts when all CTAs of this one have.
+// The one exception is the second of the two large backward kernels (tensor cores), which runs beside the first and waits for it at its end
+// only.  It may: the first one lets it start only after its own chain_wait and its allocation of tensor memory, so all that the second
+// one reads was complete by then (the statistics are read past L1, which may hold an earlier call's); neither reads what the other
+// writes, and the forms of a call in which one would (gradients written over keys or values) take the full wait.
 __device__ __forceinline__ void chain_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_enter() { chain_trigger(); chain_wait(); }

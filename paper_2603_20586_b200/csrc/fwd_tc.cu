@@ -1063,7 +1063,7 @@ Blocks make_blocks(const FwdParams& fp) {
 // lists.  Cluster or equal ranges then share the lists out; the first costs its merge and whole clusters per GPC, the second a pass
 // of partial results through the L2 cache, and its CTAs, each in another place of the keys, find less of them there.  All are added
 // up in us: a round of resident CTAs lasts as long as its first (heaviest) block.  The constants were fitted to 34 sizes (8 to 1600
-// blocks, 4 to 490 tiles a block), over which the pick takes 0.7 % more than the best form on average, 10 % at most.  Whole / clusters of 2 / 3 /
+// blocks, 4 to 490 tiles a block), over which the pick takes 0.7 % more than the best form on average, 12 % at most (the last of these).  Whole / clusters of 2 / 3 /
 // 4 / 8 / ranges, chosen in brackets:
 //   d = 128, 28 heads on 4, 512 rows at 15,000 rows of context      265 / 144 / 195 / 155 / 191 / [124] us   (56 blocks, 160 tiles)
 //   d = 128, 12 on 4, 949 rows at 3804                              93 / 59 / 79 / 69 / 101 / [51] us        (48 blocks, 61 tiles)
