@@ -163,7 +163,8 @@ size_t mka_workspace_bytes(const mka_shape* shape, const int64_t n_level[3], int
  * mka_fwd_with_scratch: the same with room for partial results, `scratch_bytes` at `scratch` (device, 16-byte aligned;
  * NULL and 0: none).  Where few blocks of query rows would leave SMs idle, the forward then cuts their key lists evenly
  * over all SMs; mka_fwd_scratch_bytes says how much room that takes for a shape (H_kv as in mka_fwd_paged, 0: the shape's own;
- * result 0: the call has no use for scratch; with less it runs as mka_fwd does).  The scratch is used between the call's kernels only.
+ * result 0: the call has no use for scratch; with less it runs as mka_fwd does: the lists are then cut otherwise, and O may differ
+ * by a rounding to bf16).  The scratch is used between the call's kernels only.
  */
 size_t mka_fwd_scratch_bytes(const mka_shape* shape, int32_t H_kv, const int64_t n_level[3]);
 mka_status mka_fwd_with_scratch(const mka_shape* shape, const void* Q, const mka_level L[3], const float* gate,

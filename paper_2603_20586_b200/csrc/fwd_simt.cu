@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
         const float* o = tiles + (row * NS + s) * kState;
         constexpr int kGroupFloats = kRows * NS * kState;
         // Eight groups' sums are added up in 64 bits, so that LSE is no further off than with the four groups of twice the rows (in 32 bits:
-        // 0.4 to 2.3 % further on average over inputs, now 1.2 to 1.6 % less; nothing to be seen in the time).
+        // 0.6 to 1.8 % further on average over 30 inputs of six sizes, now 1.2 to 1.6 % nearer; fp32 step [1, 4, 256, 64] 81.5 us, now 81.7).
         std::conditional_t<S::kGroups == 8, double, float> sum = 0;
         float M = -INFINITY, A[CPL];
 #pragma unroll
