@@ -38,24 +38,32 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
         qs[i] = x.x * p.scale; qs[i + 1] = x.y * p.scale; qs[i + 2] = x.z * p.scale; qs[i + 3] = x.w * p.scale;
         *reinterpret_cast<float4*>(gs + i) = y;
     }
-    __syncthreads();
-    float lse[R], dlt[R], acc[R][CPL];
+    float lse[R], dlt[R], acc[R][CPL], lam[3][R], o_own[R][CPL];
     float Ap[R][3], Sp[R][3];                    // per level, this lane's keys: sum_j p dP and sum_j p (for the gate gradient)
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const long long t = t0 + wg * R + r, tc = t < p.T ? t : p.T - 1;
         lse[r] = p.LSE[bh * p.T + tc];
-        // D_t = dO_t . O_t, left for the dK/dV kernel too
-        float d = 0.f;
 #pragma unroll
-        for (int k = 0; k < CPL; ++k)
-            d = fmaf(Elem<T>::ld(static_cast<const T*>(p.O) + (bh * p.T + tc) * DH + lane + 32 * k), gs[(wg * R + r) * DH + lane + 32 * k], d);
-        dlt[r] = warp_sum(d);
-        if (group == 0 && lane == 0 && t < p.T) p.delta[bh * p.T + t] = dlt[r];
+        for (int l = 0; l < 3; ++l) lam[l][r] = p.gate[((long long)b * p.T + tc) * 3 + l];
 #pragma unroll
-        for (int k = 0; k < CPL; ++k) acc[r][k] = 0.f;
+        for (int k = 0; k < CPL; ++k) {
+            o_own[r][k] = Elem<T>::ld(static_cast<const T*>(p.O) + (bh * p.T + tc) * DH + lane + 32 * k);
+            acc[r][k] = 0.f;
+        }
         Ap[r][0] = Ap[r][1] = Ap[r][2] = 0.f;
         Sp[r][0] = Sp[r][1] = Sp[r][2] = 0.f;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        // D_t = dO_t . O_t, left for the dK/dV kernel too
+        const long long t = t0 + wg * R + r;
+        float d = 0.f;
+#pragma unroll
+        for (int k = 0; k < CPL; ++k) d = fmaf(o_own[r][k], gs[(wg * R + r) * DH + lane + 32 * k], d);
+        dlt[r] = warp_sum(d);
+        if (group == 0 && lane == 0 && t < p.T) p.delta[bh * p.T + t] = dlt[r];
     }
     float* ks = tiles + group * 2 * kTileFloats;
     float* vs = ks + kTileFloats;
@@ -63,6 +71,7 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
     const float* qw = qs + wg * R * DH;
     const float* gw = gs + wg * R * DH;
     const long long t_last = (t0 + kRows - 1 < p.T ? t0 + kRows - 1 : p.T - 1);
+    int turns = 0;
 #pragma unroll
     for (int lvl = 0; lvl < 3; ++lvl) {
         const LevelDev L = p.L[lvl];
@@ -73,18 +82,22 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
         const long long lo = lo_f, hi = hi_l > hi_f ? hi_l : hi_f;
         const T* Kp = static_cast<const T*>(L.k) + b * L.sb + (h / p.kv_group) * L.sh;
         const T* Vp = static_cast<const T*>(L.v) + b * L.sb + (h / p.kv_group) * L.sh;
-        float lam[R];
         long long rlo[R], rhi[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const long long t = t0 + wg * R + r, tc = t < p.T ? t : p.T - 1;
-            lam[r] = p.gate[((long long)b * p.T + tc) * 3 + lvl];
             visible_range(lvl, tc + p.q_offset, p.window, L.n, 0, rlo[r], rhi[r]);
             if (t >= p.T) rhi[r] = rlo[r];
         }
-        for (long long j0 = (lo / kSimtTile + group) * kSimtTile; j0 < hi; j0 += S::kGroups * kSimtTile) {
+        // the groups take the tiles of the three levels in turn, as one list
+        const long long j_first = lo / kSimtTile * kSimtTile;
+        int turn = group - turns % S::kGroups;
+        if (turn < 0) turn += S::kGroups;
+        if (hi > lo) turns += (int)((hi - j_first + kSimtTile - 1) / kSimtTile % S::kGroups);
+        for (long long j0 = j_first + (long long)turn * kSimtTile; j0 < hi; j0 += S::kGroups * kSimtTile) {
             group_sync<kGroupThreads>(group);
             load_pair<T, DH, kGroupThreads>(ks, vs, Kp, Vp, j0, L.n, L.sn, (vec >> lvl) & 1, gtid);
+            copies_wait<T>();
             group_sync<kGroupThreads>(group);
             float s[R], dp[R];
 #pragma unroll
@@ -104,8 +117,8 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
             const long long j = j0 + lane;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                const bool vis = (j >= rlo[r]) && (j < rhi[r]) && lam[r] > 0.f;
-                const float pr = vis ? lam[r] * expf(s[r] - lse[r]) : 0.f;
+                const bool vis = (j >= rlo[r]) && (j < rhi[r]) && lam[lvl][r] > 0.f;
+                const float pr = vis ? lam[lvl][r] * expf(s[r] - lse[r]) : 0.f;
                 pw[r * 32 + lane] = pr * (dp[r] - dlt[r]);
                 Ap[r][lvl] = fmaf(pr, dp[r], Ap[r][lvl]);
                 Sp[r][lvl] += pr;
@@ -212,7 +225,6 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
         ksm[i] = x.x * p.scale; ksm[i + 1] = x.y * p.scale; ksm[i + 2] = x.z * p.scale; ksm[i + 3] = x.w * p.scale;
         *reinterpret_cast<float4*>(vsm + i) = y;
     }
-    __syncthreads();
     float accK[R][CPL], accV[R][CPL];
 #pragma unroll
     for (int r = 0; r < R; ++r)
@@ -239,9 +251,11 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
         const T* dO = static_cast<const T*>(p.dO) + bh * p.T * DH;
         const long long tc = t < p.T ? t : p.T - 1;
         const float lse = p.LSE[bh * p.T + tc], dlt = p.delta[bh * p.T + tc], lam = p.gate[((long long)b * p.T + tc) * 3 + lvl];
-        group_sync<kGroupThreads>(group);
+        if (i != group) group_sync<kGroupThreads>(group);
         load_pair<T, DH, kGroupThreads>(qs, gs, Q, dO, tt, p.T, DH, (vec & 8) != 0, gtid);
-        group_sync<kGroupThreads>(group);
+        copies_wait<T>();
+        if (i == group) __syncthreads();                                        // the keys and values too
+        else group_sync<kGroupThreads>(group);
         long long vlo, vhi;
         visible_range(lvl, t + p.q_offset, p.window, L.n, 0, vlo, vhi);
         if (t >= p.T) vhi = vlo;
@@ -295,6 +309,7 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
         __syncwarp();
     }
     // merge the groups: a warp adds up one key row after the other
+    if (group >= per_head * p.kv_group) __syncthreads();                        // a group without a tile
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < R; ++r) {

@@ -39,7 +39,14 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
         if (t < p.T) x = Fetch4<T>::at(Q + t * DH + i % DH, (vec & 8) != 0);
         qs[i] = x.x * p.scale; qs[i + 1] = x.y * p.scale; qs[i + 2] = x.z * p.scale; qs[i + 3] = x.w * p.scale;   // tau folded into q
     }
-    __syncthreads();
+    float lam[3][R];
+#pragma unroll
+    for (int lvl = 0; lvl < 3; ++lvl)
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const long long t = t0 + wg * R + r, tc = t < p.T ? t : p.T - 1;
+            lam[lvl][r] = p.gate[((long long)b * p.T + tc) * 3 + lvl];
+        }
 
     float m[NS][R], z[NS][R], acc[NS][R][CPL];           // z: this lane's keys only
 #pragma unroll
@@ -56,6 +63,8 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
     float* pw = ps + warp * R * 32;
     const float* qw = qs + wg * R * DH;
     const long long t_last = (t0 + kRows - 1 < p.T ? t0 + kRows - 1 : p.T - 1);
+    int turns = 0;
+    bool first = true;
 #pragma unroll
     for (int lvl = 0; lvl < 3; ++lvl) {
         const int st = MODE == MKA_MODE_FULL ? lvl : 0;
@@ -68,19 +77,25 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
         const long long lo = lo_first, hi = hi_last > hi_first ? hi_last : hi_first;
         const T* Kp = static_cast<const T*>(L.k) + b * L.sb + (h / p.kv_group) * L.sh;
         const T* Vp = static_cast<const T*>(L.v) + b * L.sb + (h / p.kv_group) * L.sh;
-        float lam[R];
         long long rlo[R], rhi[R];
+        const long long j_first = lo / kSimtTile * kSimtTile;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const long long t = t0 + wg * R + r, tc = t < p.T ? t : p.T - 1;
-            lam[r] = p.gate[((long long)b * p.T + tc) * 3 + lvl];
             visible_range(lvl, tc + p.q_offset, p.window, L.n, p.decode, rlo[r], rhi[r]);
             if (t >= p.T) rhi[r] = rlo[r];
         }
-        for (long long j0 = (lo / kSimtTile + group) * kSimtTile; j0 < hi; j0 += S::kGroups * kSimtTile) {
-            group_sync<kGroupThreads>(group);                           // the group's previous tile has been read
+        // the groups take the tiles of the three levels in turn, as one list
+        int turn = group - turns % S::kGroups;
+        if (turn < 0) turn += S::kGroups;
+        if (hi > lo) turns += (int)((hi - j_first + kSimtTile - 1) / kSimtTile % S::kGroups);
+        for (long long j0 = j_first + (long long)turn * kSimtTile; j0 < hi; j0 += S::kGroups * kSimtTile) {
+            if (!first) group_sync<kGroupThreads>(group);               // the group's previous tile has been read
             load_pair<T, DH, kGroupThreads>(ks, vs, Kp, Vp, j0, L.n, L.sn, (vec >> lvl) & 1, gtid);
-            group_sync<kGroupThreads>(group);
+            copies_wait<T>();
+            if (first) __syncthreads();                                 // the queries too
+            else group_sync<kGroupThreads>(group);
+            first = false;
             float s[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) s[r] = 0.f;
@@ -97,12 +112,12 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
             const long long j = j0 + lane;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                const bool vis = (j >= rlo[r]) && (j < rhi[r]) && (MODE == MKA_MODE_FULL || lam[r] > 0.f);
+                const bool vis = (j >= rlo[r]) && (j < rhi[r]) && (MODE == MKA_MODE_FULL || lam[lvl][r] > 0.f);
                 const float x = vis ? s[r] : -INFINITY;
                 const float m_new = fmaxf(m[st][r], warp_max(x));
                 float e = (m_new == -INFINITY) ? 0.f : expf(x - m_new);   // masked: exp(-inf) = 0
                 const float resc = (m[st][r] == -INFINITY) ? 0.f : expf(m[st][r] - m_new);
-                if (MODE == MKA_MODE_FAST) e *= lam[r];
+                if (MODE == MKA_MODE_FAST) e *= lam[lvl][r];
                 z[st][r] = z[st][r] * resc + e;
 #pragma unroll
                 for (int k = 0; k < CPL; ++k) acc[st][r][k] *= resc;
@@ -131,6 +146,7 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
     }
 
     // merge the groups: every group leaves (max, sum, acc) of its tiles, a warp then finishes one row after the other
+    if (first) __syncthreads();                                         // a group without a tile
     __syncthreads();
     constexpr int kState = DH + 2;
 #pragma unroll
