@@ -98,6 +98,14 @@ struct Cfg {
     // in the order of the sums.
     static constexpr int kSums = DH == 64 ? 2 : 1;
     static constexpr __host__ __device__ int part_of(int i) { return kSums == 2 && (i == 1 || i == 2) ? 3 - i : i; }
+    // A pair of weights in every poly_every() groups of four is formed on the FMA pipe (exp2_pair_poly, as exact as the special-function unit's):
+    // d = 64 keeps that unit busy 84 % of a CTA's steady state, and d = 128 runs at the power cap, where a quarter of the weights on
+    // the other pipe cost less than they save.  us, none / every 8th / 4th / 3rd / 2nd group / every group:
+    //   [1, 32, 32768, 128] whole blocks    12,747 / 12,747 / 12,550 / 12,400 / [12,383] / 13,785      [8, 16, 2048, 64]    272 / 268 / [269] / 269 / 268 / 320
+    //   [4, 16, 8192, 128]                  1777 / 1744 / 1740 / 1724 / [1720] / 1913                  [1, 16, 777, 64]     22.2 / 22.1 / [21.8] / 21.8 / 21.7 / -
+    // Cut lists at d = 128 (clusters, equal ranges) end before the power cap is reached, and there the longer chain shows: a 512-row chunk at
+    // 15,000 rows of context 150.7, with every 3rd group 152.6, every 2nd 157.6.
+    static constexpr __host__ __device__ int poly_every(int form) { return DH == 64 ? 4 : (form == 0 ? 2 : 0); }
     static constexpr int kRowWarps = 4;                       // softmax warps per query tile
     static constexpr int kSoftmaxWarps = kRowWarps * kNumQ;
     // The registers are re-divided between the warpgroups (setmaxnreg, a warpgroup-wide instruction: an idle warp
@@ -751,6 +759,7 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
 #pragma unroll
                 for (int i = 0; i < C::kSums; ++i) sum_a[i] = sum_b[i] = pack2(0.f, 0.f);
                 uint32_t pk[16];
+                constexpr int kPoly = C::poly_every(kForm);
                 auto weights = [&](int c_from, int c_to, int c_base) {
                     const int half = C::kSums == 2 ? c_base / 64 : 0;
 #pragma unroll
@@ -758,7 +767,10 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
                         float x0, x1, x2, x3;
                         unpack2(fma2(pack2(s[c], s[c + 1]), scale2, shift2), x0, x1);
                         unpack2(fma2(pack2(s[c + 2], s[c + 3]), scale2, shift2), x2, x3);
-                        const float p0 = ex2(x0), p1 = ex2(x1), p2 = ex2(x2), p3 = ex2(x3);
+                        const float p0 = ex2(x0), p1 = ex2(x1);
+                        float p2, p3;
+                        if (kPoly && (c / 4) % (kPoly ? kPoly : 1) == 0) exp2_pair_poly(x2, x3, p2, p3);
+                        else p2 = ex2(x2), p3 = ex2(x3);
                         sum_a[half] = add2(sum_a[half], pack2(p0, p1));
                         sum_b[half] = add2(sum_b[half], pack2(p2, p3));
                         pk[(c - c_base) / 2] = pack_bf16(p0, p1);
