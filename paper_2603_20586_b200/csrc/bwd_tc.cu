@@ -23,8 +23,8 @@
 // bias_t / scale (for S^T) or -D_t (for dP^T), each split into three bf16 terms, so S^T + bias / scale and dP^T - D arrive
 // in TMEM ready-made.  Two warps of their own write those 4 KB operand slabs (no swizzle) from the statistics of the prep
 // kernel, fetched one tile ahead.  Q tiles and dO tiles travel in rings of their own: dO(e) is free again after dV(e),
-// Q(e) only after dK(e), and Q(e+1) is what the next score product waits for.  Half of the exponentials of that kernel
-// run as a cubic on the FMA pipe (exp2_pair_fma).
+// Q(e) only after dK(e), and Q(e+1) is what the next score product waits for.  At d = 128 a quarter of the exponentials of that
+// kernel run as a cubic on the FMA pipe (exp2_pair_fma).
 //
 // CTAs are persistent: they take output tiles (items) from a ticket counter, and the next item's copies and first products run
 // under the element-wise threads' stores of the previous one.
@@ -1073,10 +1073,13 @@ __global__ void __launch_bounds__(BCfg<DH>::kThreadsDkv, 1) bwd_dkv_tc_kernel(co
                 for (int c = c_from; c < c_to; c += 2) {
                     float x0, x1;
                     unpack2(mul2(pack2(pr[c], pr[c + 1]), scale2), x0, x1);
-                    // Every other pair on the FMA pipe: the hand-over of P^T, not these threads' total work, is what the
-                    // next score product waits for, and the special-function unit alone is the slower way there.
+                    // d = 128: every fourth pair on the FMA pipe: the hand-over of P^T, not these threads' total work, is what the
+                    // next score product waits for, and the special-function unit alone is the slower way there.  With two S^T it is not
+                    // waited for, and the sixteen warps are short of issue slots (65 % used, the special-function unit 25 %, with every
+                    // other pair on the FMA pipe).  Backward, us, every other / third / fourth / no pair: [4, 16, 8192, 128] 5622 / 5560 / [5564] / 5709,
+                    // [2, 16 on 4, 1000, 128] 96.1 / 94.6 / [95.0] / 95.6; [8, 16, 2048, 64] 803 / - / 791 / [786].
                     float p0, p1;
-                    if ((c >> 1) & 1) { p0 = ex2(x0); p1 = ex2(x1); }
+                    if (kTwoS || (c >> 1) % 4 != 0) { p0 = ex2(x0); p1 = ex2(x1); }
                     else exp2_pair_fma(x0, x1, p0, p1);
                     pk[c / 2] = pack_bf16(p0, p1);
                 }
