@@ -33,11 +33,13 @@ struct L3IndexParams {
     int H_kv, page_rows, d, bits;
 };
 
+constexpr __host__ __device__ int idx_pitch(int d) { return d + 4; }
+
 // Dynamic shared memory: projT [d][bits + 4] floats (16 consecutive bits of one column are four broadcast reads), then two
-// buffers s [kIdxPairs][d + 1] floats (the key sums; the odd pitch keeps the lanes of a warp on different banks).
+// buffers s [kIdxPairs][d + 4] floats (the key sums; with that pitch the 16-byte reads of eight lanes fall on different banks).
 // A batch = 64 (page, head) pairs.  The first LOADERS threads load: 16 of them cover one 256-byte row, a thread sums its eight
 // columns row by row, with up to 24 (512 loaders: 16) loads in flight across items and batches.  Four more warps project: lane = two pairs,
-// warp = 16 bits; column i costs two reads of s, four broadcast reads of projT and 32 fmaf.  The two sides work on different batches,
+// warp = 16 bits; four columns cost two 16-byte reads of s, 16 broadcast reads of projT and 128 fmaf.  The two sides work on different batches,
 // so the loads of one run under the projections of the other.  As two phases of the same warps, and with one pair to a
 // lane, the shared-memory pipe was busy for 78 us and HBM idle half of the time: 147 us (3.6 TB/s) for [32769 pages, 4 heads, 16
 // rows, 128] at 64 bits, 123 us with four loading warps in each of two CTAs (registers moved to them from the projecting ones);
@@ -47,7 +49,7 @@ __global__ void __launch_bounds__(LOADERS + kIdxThreads, LOADERS == 128 ? 2 : 1)
     chain_enter();
     extern __shared__ __align__(16) float sm[];
     const int ppitch = p.bits + 4;                             // floats between columns of projT (keeps the fill off one bank)
-    constexpr int pitch = DH + 1, kSumFloats = kIdxPairs * pitch;
+    constexpr int pitch = idx_pitch(DH), kSumFloats = kIdxPairs * pitch;
     float* projT = sm;
     float* sums = sm + (size_t)DH * ppitch;
     const bool loads = threadIdx.x < LOADERS;
@@ -141,11 +143,10 @@ __global__ void __launch_bounds__(LOADERS + kIdxThreads, LOADERS == 128 ? 2 : 1)
                 if (row >= p.page_rows) {
                     if (item == 0 && n >= 2) wait(3 + (n & 1));            // the batch before last has been projected
                     float* s = sums + (n & 1) * kSumFloats + (slot0 + item * kSlotStep) * pitch + piece * 8;
+                    *reinterpret_cast<ulonglong2*>(s) = make_ulonglong2(acc[0], acc[1]);
+                    *reinterpret_cast<ulonglong2*>(s + 4) = make_ulonglong2(acc[2], acc[3]);
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        asm("mov.b64 {%0, %1}, %2;" : "=f"(s[2 * i]), "=f"(s[2 * i + 1]) : "l"(acc[i]));
-                        acc[i] = 0ull;
-                    }
+                    for (int i = 0; i < 4; ++i) acc[i] = 0ull;
                     row = 0;
                     if (++item == kPerThread) {
                         arrive(1 + (n & 1));
@@ -170,19 +171,27 @@ __global__ void __launch_bounds__(LOADERS + kIdxThreads, LOADERS == 128 ? 2 : 1)
 #pragma unroll
                     for (int j = 0; j < kIdxBitsPerWarp / 2; ++j) a2[q][j] = 0ull;          // two +0.f
                 const float* pj = projT + j0;
-#pragma unroll 4
-                for (int i = 0; i < DH; ++i) {
-                    const float xa = sv[i], xb = sv[32 * pitch + i];
-                    unsigned long long x2[2];
-                    asm("mov.b64 %0, {%1, %1};" : "=l"(x2[0]) : "f"(xa));
-                    asm("mov.b64 %0, {%1, %1};" : "=l"(x2[1]) : "f"(xb));
+                // 32 columns to a turn: a warp has its scheduler's share to itself and waits for the reads at the start of each turn (the loading warps never
+                // wait for long: they ran out of buffers for 2 % of the time, these warps of sums for 0.1 %).  Turns of 4 / 8 / 16 / 32 columns:
+                // [32769 pages, 4 heads, 16 rows, 128], 64 bits 118 / 111 / 111 / 109.5 us; 128 bits [20000, 8, 16, 128] 204 / 190 / 183 / 182;
+                // 256 bits [20000, 2, 8, 128] 93.0 / 89.3 / 85.4 / 81.9.
+#pragma unroll 8
+                for (int i4 = 0; i4 < DH; i4 += 4) {
+                    const float4 xa4 = *reinterpret_cast<const float4*>(sv + i4), xb4 = *reinterpret_cast<const float4*>(sv + 32 * pitch + i4);
+                    const float xa[4] = {xa4.x, xa4.y, xa4.z, xa4.w}, xb[4] = {xb4.x, xb4.y, xb4.z, xb4.w};
 #pragma unroll
-                    for (int v = 0; v < kIdxBitsPerWarp / 4; ++v) {
-                        const ulonglong2 pr = *reinterpret_cast<const ulonglong2*>(pj + (size_t)i * ppitch + 4 * v);   // bits 4v..4v+3 of column i
+                    for (int k = 0; k < 4; ++k) {
+                        unsigned long long x2[2];
+                        asm("mov.b64 %0, {%1, %1};" : "=l"(x2[0]) : "f"(xa[k]));
+                        asm("mov.b64 %0, {%1, %1};" : "=l"(x2[1]) : "f"(xb[k]));
 #pragma unroll
-                        for (int q = 0; q < 2; ++q) {
-                            asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a2[q][2 * v]) : "l"(pr.x), "l"(x2[q]));
-                            asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a2[q][2 * v + 1]) : "l"(pr.y), "l"(x2[q]));
+                        for (int v = 0; v < kIdxBitsPerWarp / 4; ++v) {
+                            const ulonglong2 pr = *reinterpret_cast<const ulonglong2*>(pj + (size_t)(i4 + k) * ppitch + 4 * v);   // bits 4v..4v+3 of the column
+#pragma unroll
+                            for (int q = 0; q < 2; ++q) {
+                                asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a2[q][2 * v]) : "l"(pr.x), "l"(x2[q]));
+                                asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a2[q][2 * v + 1]) : "l"(pr.y), "l"(x2[q]));
+                            }
                         }
                     }
                 }
@@ -568,7 +577,7 @@ __global__ void __launch_bounds__(kRetThreads) l3_retrieve_kernel(const L3Retrie
 //   d = 64    32 bits 1.04 / 1.09 / 1.02    64 bits 1.12 / 1.20 / 1.07    128 bits 0.88 / 1.26 / 1.18    256 bits 0.86 / 1.00 / 1.42
 //   d = 128           1.09 / 1.10 / 1.09            1.22 / 1.41 / 1.52             1.19 / 1.54 / 1.53             0.92 / 1.23 / 1.79
 //   pages of 8 rows 0.8 .. 0.9;  pools of 40 MB 0.7 .. 1.2, of 60 MB 0.91 .. 1.22, of 90 MB and more 1.02 .. 1.44 (32 bits: 0.8 .. 1.03)
-// [32769 pages, 4 heads, 16 rows, 128], 64 bits: 119.5 us before, 106 now (5.1 TB/s).
+// [32769 pages, 4 heads, 16 rows, 128], 64 bits: 119.5 us with eight loading warps, 106 with sixteen (109.5 against 117.6 on another day with longer turns of the projecting warps).
 bool many_loaders(const L3IndexParams& p) {
     return p.page_rows >= 16 && p.bits <= (p.d == 128 ? 8 : 4) * p.page_rows &&
            (double)p.n_pages * p.H_kv * p.page_rows * p.d * 2.0 >= (p.bits == 32 ? 200e6 : 80e6);
@@ -600,7 +609,7 @@ cudaError_t launch_l3_index(const void* k, long long n_pages, int H_kv, int page
     // persistent CTAs: every CTA transposes the projection into shared memory once and then walks its batches
     // (the grid is shrunk so that all CTAs get the same number of batches)
     auto launch = [&](auto kern, int batch, int buffers, int threads, auto ctas_per_sm) {
-        const size_t smem = ((size_t)d * (bits + 4) + (size_t)buffers * batch * (d + 1)) * sizeof(float);
+        const size_t smem = ((size_t)d * (bits + 4) + (size_t)buffers * batch * (buffers == 2 ? idx_pitch(d) : d + 1)) * sizeof(float);
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         const long long batches = (n_pages * H_kv + batch - 1) / batch, resident = 148LL * ctas_per_sm(smem);
