@@ -1075,7 +1075,8 @@ Blocks make_blocks(const FwdParams& fp) {
 // lists.  Cluster or equal ranges then share the lists out; the first costs its merge and whole clusters per GPC, the second a pass
 // of partial results through the L2 cache, and its CTAs, each in another place of the keys, find less of them there.  All are added
 // up in us: a round of resident CTAs lasts as long as its first (heaviest) block.  The constants were fitted to 34 sizes (8 to 1600
-// blocks, 4 to 490 tiles a block), over which the pick takes 0.7 % more than the best form on average, 12 % at most (the last of these).  Whole / clusters of 2 / 3 /
+// blocks, 4 to 490 tiles a block), over which the pick takes 0.7 % more than the best form on average, and for d = 64 again to 40 (with a cluster's
+// start and merge at 14.5 us as for d = 128 the pick took 3.6 % more there, 22 % at most; now 1.6 %).  Whole / clusters of 2 / 3 /
 // 4 / 8 / ranges, chosen in brackets:
 //   d = 128, 28 heads on 4, 512 rows at 15,000 rows of context      265 / 144 / 195 / 155 / 191 / [124] us   (56 blocks, 160 tiles)
 //   d = 128, 12 on 4, 949 rows at 3804                              93 / 59 / 79 / 69 / 101 / [51] us        (48 blocks, 61 tiles)
@@ -1085,28 +1086,34 @@ Blocks make_blocks(const FwdParams& fp) {
 //   d = 128, 16 heads, 3078 rows                                    164 / 170 / 194 / 228 / 347 / [155] us   (208 blocks)
 //   d = 128, 2 x 16 heads, 1000 rows                                [35] / 51 / 63 / 80 / 149 / 56 us        (128 blocks)
 //   d = 64, 2 x 32 heads, 627 rows, 7815 slots                      179 / 157 / 159 / 164 / 205 / [137] us   (320 blocks)
-//   d = 64, 16 heads, 777 rows                                      [19] / 17 / 23 / 24 / 41 / 23 us         (112 blocks)
+//   d = 64, 16 heads, 777 rows                                      19 / [17] / 23 / 24 / 41 / 21 us         (112 blocks)
+//   d = 64, 32 heads on 8, 479 rows, 1698 slots                     29 / [25] / 34 / 32 / 51 / 30 us         (128 blocks)
 struct FormChoice { int form, ctas; };       // kCluster: CTAs of a cluster; kStream: CTAs of the grid
 template <int DH>
 FormChoice form_rule(const FwdParams& fp, const Blocks& bl, bool scratch) {
     const long long lines = bl.lines, blocks = lines * bl.per_line;
     const int slots = 148 * Cfg<DH>::kCtasPerSm;
     const double tile = DH == 128 ? 1.54 : 0.93;                            // us for a CTA that has its SM to itself
+    const double whole_first = DH == 128 ? 7.0 : 6.5, whole_next = DH == 128 ? 4.5 : 3.0;           // a round's start and end
+    const double cluster_first = DH == 128 ? 14.5 : 9.5, cluster_next = DH == 128 ? 11.5 : 13.0;
+    const double ranges_first = DH == 128 ? 17.5 : 16.5, ranges_tile = DH == 128 ? 1.18 : 1.14;
     auto shared = [](long long ctas) { return DH == 64 && ctas > 148 ? 1.36 : 1.0; };
     FormChoice best = {kWhole, 1};
     if (blocks > kStreamRounds * slots) return best;                         // whole blocks fill the chip evenly enough
     double best_us = 0.0;
     for (long long blk = 0; blk < blocks; blk += slots)
-        best_us += block_tiles(fp, bl, bl.per_line - 1 - blk / lines) * tile * shared(blocks - blk) + (blk == 0 ? 7.0 : 4.5);
+        best_us += block_tiles(fp, bl, bl.per_line - 1 - blk / lines) * tile * shared(blocks - blk) + (blk == 0 ? whole_first : whole_next);
     best_us *= 0.97;                                                         // (what the model can tell apart)
     if (blocks <= slots) {
         for (int split = 2; split <= kMaxSplit; ++split) {
+            // d = 64: three tiles to a CTA at least (2 x 16 heads on 4, 220 rows, 5 tiles: 11.2 us whole, 13.9 in clusters of 4)
+            if (DH == 64 && 3 * split > block_tiles(fp, bl, bl.per_line - 1)) break;
             const int fit = resident_clusters<DH>(split);
             if (fit < 1) continue;
             double us = 0.0;
             for (long long blk = 0; blk < blocks && us < best_us; blk += fit)
                 us += block_tiles(fp, bl, bl.per_line - 1 - blk / lines) * tile * 1.03 / split * shared((blocks - blk < fit ? blocks - blk : fit) * split) +
-                      (blk == 0 ? 14.5 : 11.5);
+                      (blk == 0 ? cluster_first : cluster_next);
             if (us < best_us) { best = {kCluster, split}; best_us = us; }
         }
     }
@@ -1118,7 +1125,7 @@ FormChoice form_rule(const FwdParams& fp, const Blocks& bl, bool scratch) {
             const double seen = l == 0 ? (double)fp.window + fp.T : 1e18;
             mbytes += ((double)fp.L[l].n < seen ? (double)fp.L[l].n : seen) * fp.B * (fp.H / fp.kv_group) * (DH * 4e-6);
         }
-        const double us = units / slots * tile * 1.18 * shared(slots) + 17.5 + 0.35 * slots / (double)blocks + (mbytes > 100.0 ? 0.068 * (mbytes - 100.0) : 0.0);
+        const double us = units / slots * tile * ranges_tile * shared(slots) + ranges_first + 0.35 * slots / (double)blocks + (mbytes > 100.0 ? 0.068 * (mbytes - 100.0) : 0.0);
         if (units >= slots && units < 1e9 && us < best_us) best = {kStream, slots};
     }
     return best;
