@@ -183,6 +183,17 @@ _levels = _host_args.levels                # (K, V) -> mka_level[3] as bytes; No
 _paged_levels = _host_args.paged_levels    # (pools_k, pools_v, tables, rows or None, n) -> mka_paged_level[3] as bytes; pools
                                            # [pages, H_kv, page_rows, d], any strides with d contiguous; tables [B, pages] or [B, H_kv, pages]
 _empty_f32 = _host_args.empty_f32          # (t, keep, extra) -> fp32 tensor of t's first `keep` dimensions (and `extra`)
+_empty_like = _host_args.empty_like
+_row_counts = _host_args.row_counts        # (K) -> the rows of three levels, 0 for None
+
+
+def _address(function) -> int:
+    return ctypes.cast(function, ctypes.c_void_p).value
+
+
+# The entry points that short steps consist of are called from native code too: tensors, None and ints go in as they are.
+_router, _fwd, _fwd_paged = _address(lib.mka_router), _address(lib.mka_fwd_with_scratch), _address(lib.mka_fwd_paged_with_scratch)
+_decode, _decode_paged, _bwd = _address(lib.mka_decode), _address(lib.mka_decode_paged), _address(lib.mka_bwd)
 
 
 def mka_workspace_bytes(shape: mka_shape, n_level, which: int) -> int:
@@ -211,8 +222,7 @@ def mka_router(R: torch.Tensor, W_r: torch.Tensor, b_r: Optional[torch.Tensor], 
     assert R.is_contiguous() and W_r.is_contiguous() and W_r.dtype == torch.float32 and W_r.shape == (D, 3)
     if gate is None:
         gate = _empty_f32(R, R.dim() - 1, 3)
-    _check(lib.mka_router(_ptr(R), _ptr(W_r), _ptr(b_r), rows, D, _dt(R), route, _ptr(gate), _ptr(log2_gate),
-                          _ptr(route_idx), _stream(stream)), "mka_router")
+    _check(_host_args.call_router(_router, R, W_r, b_r, rows, D, _dt(R), route, gate, log2_gate, route_idx, _stream(stream)), "mka_router")
     return gate
 
 
@@ -225,7 +235,7 @@ def _fwd_scratch(shape: mka_shape, H_kv: int, n_level, device, stream) -> Option
     q_tiles = shape.B * shape.H * ((shape.T + 127) // 128)
     if q_tiles > 4 * 148 * 2 or q_tiles * sum(n_level) < 148 * 4 * 128:      # many blocks, or little to share out: not worth the question
         return None
-    nbytes = lib.mka_fwd_scratch_bytes(shape, H_kv, n_level)
+    nbytes = lib.mka_fwd_scratch_bytes(shape, H_kv, _Rows(*n_level))
     if nbytes == 0:
         return None
     try:
@@ -245,15 +255,15 @@ def mka_fwd(shape: mka_shape, Q, K, V, gate, O=None, LSE=None, ws=None, stream=N
     key lists are cut in another way, and O may differ by a rounding to bf16, LSE by some 1e-7 of its size."""
     assert Q.is_contiguous() and gate.is_contiguous() and gate.dtype == torch.float32
     if O is None:
-        O = torch.empty_like(Q)
+        O = _empty_like(Q)
     if LSE is None and want_lse and shape.mode == MKA_MODE_FAST:
         LSE = _empty_f32(Q, 3, 0)
-    n = [0 if K[l] is None else K[l].shape[2] for l in range(3)]
+    n = _row_counts(K)
     if ws is None:
         ws = alloc_workspace(shape, n, MKA_WS_FWD, Q.device)
-    tmp = _fwd_scratch(shape, 0, _Rows(*n), Q.device, stream)
-    _check(lib.mka_fwd_with_scratch(ctypes.byref(shape), _ptr(Q), _levels(K, V), _ptr(gate), _ptr(O), _ptr(LSE), _ptr(ws), ws.numel(),
-                                    _ptr(tmp), 0 if tmp is None else tmp.numel(), _stream(stream)), "mka_fwd")
+    tmp = _fwd_scratch(shape, 0, n, Q.device, stream)
+    _check(_host_args.call_fwd(_fwd, shape, Q, _levels(K, V), gate, O, LSE, ws, ws.numel(), tmp, 0 if tmp is None else tmp.numel(),
+                               _stream(stream)), "mka_fwd")
     return O, LSE
 
 
@@ -265,8 +275,7 @@ def mka_decode(shape: mka_shape, q, K, V, gate, O=None, LSE=None, ws=None, strea
         LSE = _empty_f32(q, 2, 0)
     if ws is None:
         ws = alloc_workspace(shape, [0 if k is None else k.shape[2] for k in K], MKA_WS_DECODE, q.device)
-    _check(lib.mka_decode(ctypes.byref(shape), _ptr(q), _levels(K, V), _ptr(gate), _ptr(O), _ptr(LSE), _ptr(ws),
-                          ws.numel(), _stream(stream)), "mka_decode")
+    _check(_host_args.call_decode(_decode, shape, q, _levels(K, V), gate, O, LSE, ws, ws.numel(), _stream(stream)), "mka_decode")
     return O, LSE
 
 
@@ -299,10 +308,9 @@ def mka_fwd_paged(shape: mka_shape, H_kv: int, Q, pools_k, pools_v, tables, n, g
         ws = torch.zeros(256, dtype=torch.uint8, device=Q.device)
     tmp = None
     if rows is None or not any(r is not None for r in rows):
-        tmp = _fwd_scratch(shape, H_kv, _Rows(*[0 if pools_k[l] is None else int(n[l]) for l in range(3)]), Q.device, stream)
-    _check(lib.mka_fwd_paged_with_scratch(ctypes.byref(shape), H_kv, _ptr(Q), _paged_levels(pools_k, pools_v, tables, rows, n), _ptr(gate),
-                                          _ptr(O), _ptr(LSE), _ptr(ws), ws.numel(), _ptr(tmp), 0 if tmp is None else tmp.numel(),
-                                          _stream(stream)), "mka_fwd_paged")
+        tmp = _fwd_scratch(shape, H_kv, [0 if pools_k[l] is None else int(n[l]) for l in range(3)], Q.device, stream)
+    _check(_host_args.call_fwd_paged(_fwd_paged, shape, H_kv, Q, _paged_levels(pools_k, pools_v, tables, rows, n), gate, O, LSE, ws, ws.numel(),
+                                     tmp, 0 if tmp is None else tmp.numel(), _stream(stream)), "mka_fwd_paged")
     return O, LSE
 
 
@@ -321,8 +329,8 @@ def mka_decode_paged(shape: mka_shape, H_kv: int, q, pools_k, pools_v, tables, n
         LSE = _empty_f32(q, 2, 0)
     if ws is None:
         ws = torch.empty(mka_decode_paged_workspace_bytes(shape, H_kv, n), dtype=torch.uint8, device=q.device)
-    _check(lib.mka_decode_paged(ctypes.byref(shape), H_kv, _ptr(q), _paged_levels(pools_k, pools_v, tables, rows, n),
-                                _ptr(gate), _ptr(O), _ptr(LSE), _ptr(ws), ws.numel(), _stream(stream)), "mka_decode_paged")
+    _check(_host_args.call_decode_paged(_decode_paged, shape, H_kv, q, _paged_levels(pools_k, pools_v, tables, rows, n), gate, O, LSE, ws, ws.numel(),
+                                        _stream(stream)), "mka_decode_paged")
     return O, LSE
 
 
@@ -393,9 +401,8 @@ def mka_bwd(shape: mka_shape, Q, K, V, gate, O, LSE, dO, R=None, dQ=None, dK=Non
     grads = _host_args.grads(K, dK, dV)
     if ws is None:
         ws = alloc_workspace(shape, [0 if k is None else k.shape[2] for k in K], MKA_WS_BWD, dev)
-    _check(lib.mka_bwd(ctypes.byref(shape), _ptr(Q), _levels(K, V), _ptr(gate), _ptr(O), _ptr(LSE), _ptr(dO),
-                       _ptr(R), _dt(R) if R is not None else MKA_F32, _ptr(dQ), grads, _ptr(dG), _ptr(dW_r),
-                       _ptr(db_r), _ptr(ws), ws.numel(), _stream(stream)), "mka_bwd")
+    _check(_host_args.call_bwd(_bwd, shape, Q, _levels(K, V), gate, O, LSE, dO, R, _dt(R) if R is not None else MKA_F32, dQ, grads, dG, dW_r,
+                               db_r, ws, ws.numel(), _stream(stream)), "mka_bwd")
     return {"dQ": dQ, "dK": dK, "dV": dV, "dG": dG, "dW_r": dW_r, "db_r": db_r}
 
 

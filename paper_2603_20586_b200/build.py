@@ -49,7 +49,7 @@ def _host_module_cmd(out):
     import torch
     from torch.utils.cpp_extension import include_paths, library_paths
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared",
-           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I", sysconfig.get_paths()["include"]]
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I", sysconfig.get_paths()["include"], "-I", os.path.join(ROOT, "include")]
     for path in include_paths():
         cmd += ["-isystem", path]
     for path in library_paths():
@@ -82,7 +82,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         run([NVCC, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", tmp] + objs + ["-cudart", "static"])
         os.replace(tmp, LIB)
     host = host_module()
-    if force or _stale(host, [HOST_SRC]):
+    if force or _stale(host, [HOST_SRC] + glob.glob(os.path.join(ROOT, "include", "*.h"))):
         tmp = host + f".{os.getpid()}.tmp"
         run(_host_module_cmd(tmp))
         os.replace(tmp, host)

@@ -1,14 +1,20 @@
 // Host side of the binding: the levels of a call as the array of 64-bit words that mka_level[3], mka_level_grad[3] and
-// mka_paged_level[3] are, and the call's small outputs.  Asked for one by one from Python, the pointers, shapes and strides of the
-// six tensors of a call took longer than a short decode takes on the GPU (6.3 us; 0.2 us here).
+// mka_paged_level[3] are, the call's small outputs, and the calls of the library that short steps consist of.  Asked for one by one from Python, the
+// pointers, shapes and strides of the six tensors of a call took longer than a short decode takes on the GPU (6.3 us; 0.2 us here); the
+// rest of a call's arguments through ctypes took 1.7 us of a router's 4.6, and of a forward's 12.2 (a short prompt is over in 17) 7.7.
 #include <ATen/ops/empty.h>
 #include <ATen/ops/empty_like.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <Python.h>
 #include <stdint.h>
+#include <string.h>
 
+#include <tuple>
+#include <utility>
 #include <vector>
+
+#include "mka.h"
 
 namespace {
 
@@ -199,6 +205,114 @@ PyObject* empty_f32(PyObject*, PyObject* const* a, Py_ssize_t n) {
     });
 }
 
+// A C argument from a Python object; what was taken out of the object lives as long as this.
+template <typename P> struct Arg;
+template <> struct Arg<int64_t> {
+    int64_t v;
+    explicit Arg(PyObject* o) : v(0) {
+        if (!PyLong_Check(o)) {
+            PyErr_SetString(PyExc_TypeError, "an int is expected");
+            throw PyErrSet();
+        }
+        v = PyLong_AsLongLong(o);
+        if (v == -1 && PyErr_Occurred()) throw PyErrSet();
+    }
+};
+template <> struct Arg<int32_t> {
+    int32_t v;
+    explicit Arg(PyObject* o) : v(static_cast<int32_t>(Arg<int64_t>(o).v)) {}
+};
+template <> struct Arg<size_t> {
+    size_t v;
+    explicit Arg(PyObject* o) : v(static_cast<size_t>(Arg<int64_t>(o).v)) {}
+};
+template <typename T> struct Arg<T*> {               // a tensor's memory, an address, or None
+    T* v;
+    explicit Arg(PyObject* o) : v(nullptr) {
+        if (o == Py_None) return;
+        if (PyLong_Check(o)) {
+            v = static_cast<T*>(PyLong_AsVoidPtr(o));
+            if (!v && PyErr_Occurred()) throw PyErrSet();
+        } else {
+            v = static_cast<T*>(tensor(o).data_ptr());
+        }
+    }
+};
+template <typename T> struct Levels {                // three levels as `levels`, `grads` or `paged_levels` returned them
+    const T* v;
+    explicit Levels(PyObject* o) : v(nullptr) {
+        if (!PyBytes_Check(o) || PyBytes_GET_SIZE(o) != static_cast<Py_ssize_t>(3 * sizeof(T))) throw Bad();
+        v = reinterpret_cast<const T*>(PyBytes_AS_STRING(o));
+    }
+};
+template <> struct Arg<const mka_level*> : Levels<mka_level> { using Levels::Levels; };
+template <> struct Arg<const mka_level_grad*> : Levels<mka_level_grad> { using Levels::Levels; };
+template <> struct Arg<const mka_paged_level*> : Levels<mka_paged_level> { using Levels::Levels; };
+template <> struct Arg<const mka_shape*> {
+    mka_shape copy;
+    const mka_shape* v;
+    explicit Arg(PyObject* o) : v(&copy) {
+        Py_buffer view;
+        if (PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) != 0) throw PyErrSet();
+        const bool fits = view.len == static_cast<Py_ssize_t>(sizeof(mka_shape));
+        if (fits) memcpy(&copy, view.buf, sizeof(mka_shape));
+        PyBuffer_Release(&view);
+        if (!fits) {
+            PyErr_SetString(PyExc_TypeError, "an mka_shape is expected");
+            throw PyErrSet();
+        }
+    }
+    Arg(const Arg&) = delete;
+};
+
+// The library's function at address a[0] (of the type of the declaration named) with the other arguments; its status.  Other threads run meanwhile.
+template <typename R, typename... P, size_t... I>
+PyObject* invoke(R (*)(P...), PyObject* const* a, std::index_sequence<I...>) {
+    const auto f = reinterpret_cast<R (*)(P...)>(Arg<void*>(a[0]).v);
+    if (!f) throw Bad();
+    const std::tuple<Arg<P>...> args{a[1 + I]...};
+    R status;
+    Py_BEGIN_ALLOW_THREADS
+    status = f(std::get<I>(args).v...);
+    Py_END_ALLOW_THREADS
+    return PyLong_FromLongLong(static_cast<long long>(status));
+}
+template <typename R, typename... P>
+PyObject* call(R (*declared)(P...), PyObject* const* a, Py_ssize_t n) {
+    return guarded([&]() -> PyObject* {
+        if (n != static_cast<Py_ssize_t>(1 + sizeof...(P))) throw Bad();
+        return invoke(declared, a, std::index_sequence_for<P...>());
+    });
+}
+#define MKA_CALL(name) \
+    PyObject* call_##name(PyObject*, PyObject* const* a, Py_ssize_t n) { return call(static_cast<decltype(&mka_##name)>(nullptr), a, n); }
+MKA_CALL(router)
+MKA_CALL(fwd_with_scratch)
+MKA_CALL(fwd_paged_with_scratch)
+MKA_CALL(decode)
+MKA_CALL(decode_paged)
+MKA_CALL(bwd)
+#undef MKA_CALL
+
+PyObject* empty_like(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    return guarded([&]() -> PyObject* {
+        if (n != 1) throw Bad();
+        return THPVariable_Wrap(at::empty_like(tensor(a[0])));
+    });
+}
+PyObject* row_counts(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    return guarded([&]() -> PyObject* {
+        if (n != 1) throw Bad();
+        Seq K(a[0]);
+        int64_t rows[3];
+        for (int l = 0; l < 3; ++l) {
+            const at::Tensor* k = K.tensor_at(l);
+            rows[l] = k ? k->size(2) : 0;
+        }
+        return Py_BuildValue("LLL", static_cast<long long>(rows[0]), static_cast<long long>(rows[1]), static_cast<long long>(rows[2]));
+    });
+}
+
 template <typename F> PyMethodDef method(const char* name, F f, const char* doc) {
     return {name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(f)), METH_FASTCALL, doc};
 }
@@ -209,6 +323,14 @@ PyMethodDef methods[] = {
     method("paged_level", paged_level, "paged_level(pool_k, pool_v, table) -> one mka_paged_level over the table's width as bytes"),
     method("empties_like", empties_like, "empties_like(tensors) -> list of empty_like, None for None"),
     method("empty_f32", empty_f32, "empty_f32(t, keep, extra) -> fp32 tensor of t's first `keep` dimensions, then `extra` if not 0"),
+    method("empty_like", empty_like, "empty_like(t)"),
+    method("row_counts", row_counts, "row_counts(K) -> the rows of three levels, 0 for None"),
+    method("call_router", call_router, "call_router(address, arguments of mka_router...) -> its status"),
+    method("call_fwd", call_fwd_with_scratch, "the same for mka_fwd_with_scratch"),
+    method("call_fwd_paged", call_fwd_paged_with_scratch, "the same for mka_fwd_paged_with_scratch"),
+    method("call_decode", call_decode, "the same for mka_decode"),
+    method("call_decode_paged", call_decode_paged, "the same for mka_decode_paged"),
+    method("call_bwd", call_bwd, "the same for mka_bwd"),
     {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_host_args", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
