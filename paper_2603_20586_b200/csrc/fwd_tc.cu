@@ -1020,6 +1020,12 @@ cudaLaunchConfig_t cluster_config(int split, dim3 grid, cudaStream_t st, cudaLau
     return cfg;
 }
 
+// A kernel of the forward's shape (threads, shared memory) and CTAs per SM, asked about in its place: for a kernel that moves registers
+// between its warps the occupancy query finds one CTA to an SM at d = 64, where two run (112 clusters of two CTAs, which it
+// takes for two rounds of 74, end after 15.8 us; a whole block of theirs after 18.3).
+template <int DH>
+__global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_shape_kernel() {}
+
 // Clusters of `split` CTAs that the device keeps resident at a time (a cluster stays within one GPC, so this is less than
 // the number of CTAs / split); asked once per device and size.
 template <int DH>
@@ -1029,7 +1035,7 @@ int resident_clusters(int split) {
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
     int n = known[dev][split].load(std::memory_order_relaxed);
     if (n) return n - 1;
-    auto kern = fwd_tc_kernel<DH, false, kCluster>;
+    auto kern = fwd_shape_kernel<DH>;
     cudaLaunchAttribute at;
     const cudaLaunchConfig_t cfg = cluster_config<DH>(split, dim3(split), nullptr, &at);
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<DH>::kSmemBytes) != cudaSuccess ||
@@ -1075,8 +1081,8 @@ Blocks make_blocks(const FwdParams& fp) {
 // lists.  Cluster or equal ranges then share the lists out; the first costs its merge and whole clusters per GPC, the second a pass
 // of partial results through the L2 cache, and its CTAs, each in another place of the keys, find less of them there.  All are added
 // up in us: a round of resident CTAs lasts as long as its first (heaviest) block.  The constants were fitted to 34 sizes (8 to 1600
-// blocks, 4 to 490 tiles a block), over which the pick takes 0.7 % more than the best form on average, and for d = 64 again to 40 (with a cluster's
-// start and merge at 14.5 us as for d = 128 the pick took 3.6 % more there, 22 % at most; now 1.6 %).  Whole / clusters of 2 / 3 /
+// blocks, 4 to 490 tiles a block), over which the pick takes 0.7 % more than the best form on average, and for d = 64 again to 40, where it took
+// 3.2 % more with one cluster CTA counted to an SM, now 1.5 % (CTAs of clusters share SMs from about 96 on).  Whole / clusters of 2 / 3 /
 // 4 / 8 / ranges, chosen in brackets:
 //   d = 128, 28 heads on 4, 512 rows at 15,000 rows of context      265 / 144 / 195 / 155 / 191 / [124] us   (56 blocks, 160 tiles)
 //   d = 128, 12 on 4, 949 rows at 3804                              93 / 59 / 79 / 69 / 101 / [51] us        (48 blocks, 61 tiles)
@@ -1095,9 +1101,10 @@ FormChoice form_rule(const FwdParams& fp, const Blocks& bl, bool scratch) {
     const int slots = 148 * Cfg<DH>::kCtasPerSm;
     const double tile = DH == 128 ? 1.54 : 0.93;                            // us for a CTA that has its SM to itself
     const double whole_first = DH == 128 ? 7.0 : 6.5, whole_next = DH == 128 ? 4.5 : 3.0;           // a round's start and end
-    const double cluster_first = DH == 128 ? 14.5 : 9.5, cluster_next = DH == 128 ? 11.5 : 13.0;
+    const double cluster_first = DH == 128 ? 14.5 : 9.2, cluster_next = DH == 128 ? 11.5 : 9.0;
+    const double cluster_tile = DH == 128 ? 1.03 : 1.1;
     const double ranges_first = DH == 128 ? 17.5 : 16.5, ranges_tile = DH == 128 ? 1.18 : 1.14;
-    auto shared = [](long long ctas) { return DH == 64 && ctas > 148 ? 1.36 : 1.0; };
+    auto shared = [](long long ctas, long long sms = 148) { return DH == 64 && ctas > sms ? 1.28 : 1.0; };
     FormChoice best = {kWhole, 1};
     if (blocks > kStreamRounds * slots) return best;                         // whole blocks fill the chip evenly enough
     double best_us = 0.0;
@@ -1112,7 +1119,7 @@ FormChoice form_rule(const FwdParams& fp, const Blocks& bl, bool scratch) {
             if (fit < 1) continue;
             double us = 0.0;
             for (long long blk = 0; blk < blocks && us < best_us; blk += fit)
-                us += block_tiles(fp, bl, bl.per_line - 1 - blk / lines) * tile * 1.03 / split * shared((blocks - blk < fit ? blocks - blk : fit) * split) +
+                us += block_tiles(fp, bl, bl.per_line - 1 - blk / lines) * tile * cluster_tile / split * shared((blocks - blk < fit ? blocks - blk : fit) * split, 96) +
                       (blk == 0 ? cluster_first : cluster_next);
             if (us < best_us) { best = {kCluster, split}; best_us = us; }
         }
