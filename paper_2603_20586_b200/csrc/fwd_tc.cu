@@ -98,14 +98,15 @@ struct Cfg {
     // in the order of the sums.
     static constexpr int kSums = DH == 64 ? 2 : 1;
     static constexpr __host__ __device__ int part_of(int i) { return kSums == 2 && (i == 1 || i == 2) ? 3 - i : i; }
-    // A pair of weights in every poly_every() groups of four is formed on the FMA pipe (exp2_pair_poly, as exact as the special-function unit's):
-    // d = 64 keeps that unit busy 84 % of a CTA's steady state, and d = 128 runs at the power cap, where a quarter of the weights on
+    // A pair of weights in every poly_every()-th group of four is formed on the FMA pipe (exp2_pair_poly, as exact as the special-function unit's):
+    // d = 64 keeps that unit busy 84 % of a CTA's steady state, and d = 128 runs at the power cap, where a sixth of the weights on
     // the other pipe cost less than they save.  us, none / every 8th / 4th / 3rd / 2nd group / every group:
-    //   [1, 32, 32768, 128] whole blocks    12,747 / 12,747 / 12,550 / 12,400 / [12,383] / 13,785      [8, 16, 2048, 64]    272 / 268 / [269] / 269 / 268 / 320
-    //   [4, 16, 8192, 128]                  1777 / 1744 / 1740 / 1724 / [1720] / 1913                  [1, 16, 777, 64]     22.2 / 22.1 / [21.8] / 21.8 / 21.7 / -
-    // Cut lists at d = 128 (clusters, equal ranges) end before the power cap is reached, and there the longer chain shows: a 512-row chunk at
-    // 15,000 rows of context 150.7, with every 3rd group 152.6, every 2nd 157.6.
-    static constexpr __host__ __device__ int poly_every(int form) { return DH == 64 ? 4 : (form == 0 ? 2 : 0); }
+    //   [1, 32, 32768, 128] whole blocks    12,747 / 12,747 / 12,550 / [12,400] / 12,383 / 13,785      [8, 16, 2048, 64]    272 / 268 / [269] / 269 / 268 / 320
+    //   [4, 16, 8192, 128]                  1777 / 1744 / 1740 / [1724] / 1720 / 1913                  [1, 16, 777, 64]     22.2 / 22.1 / [21.8] / 21.8 / 21.7 / -
+    // (whole blocks of 30 to 2000 us at d = 128: 0.96 to 1.00 of the time without; over paged levels, which give the dense form's bits, every 3rd 0.98 to
+    // 1.00, every 2nd up to 1.02).  Cut lists at d = 128 (clusters, equal ranges) end before the power cap is reached, and there the longer chain
+    // shows: a 512-row chunk at 15,000 rows of context 150.7, with every 3rd group 152.6, every 2nd 157.6.
+    static constexpr __host__ __device__ int poly_every(int form) { return DH == 64 ? 4 : (form == 0 ? 3 : 0); }
     static constexpr int kRowWarps = 4;                       // softmax warps per query tile
     static constexpr int kSoftmaxWarps = kRowWarps * kNumQ;
     // The registers are re-divided between the warpgroups (setmaxnreg, a warpgroup-wide instruction: an idle warp
