@@ -361,6 +361,7 @@ static mka_status run_decode_paged(DecodePagedParams& p, DecodeParams& c, const 
     for (int l = 0; l < 3; ++l) { p.n_chunks[l] = plan.n_chunks[l]; c.n_chunks[l] = plan.n_chunks[l]; }
     if (plan.total_chunks > 0 && decode_paged_dealt(p)) {
         p.dealt = c.counted = 1;
+        c.expected = kDealCtas / (p.B * p.H_kv) + 1;
         p.total_chunks = dealt_slots(n_level, p.H_kv);
     }
     c.total_chunks = p.total_chunks;

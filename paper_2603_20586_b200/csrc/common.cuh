@@ -134,6 +134,7 @@ struct DecodeParams {
     long long total_chunks;
     float* partial;      // [B*H, total_chunks, d+2]
     int counted;         // combine: entry 0 of a (batch, head) holds the number of partials that follow, which carry the gate already
+    int expected;        // counted: partials of a (batch, head) in a batch of equal lengths
     unsigned int* status;   // device status word that the combine kernel sets to MKA_OK, or null (kernels before it may wait and set it)
 };
 cudaError_t launch_decode(const DecodeParams& p, cudaStream_t st);
@@ -160,6 +161,7 @@ struct DecodePagedParams {
     float* partial;      // [B*H, total_chunks, d+2]
     int test_stall;                    // MKA_FLAG_TEST_STALL (copy-engine form): every CTA's producer leaves out the last tile of its share
     int dealt;                         // the copy-engine form: total_chunks = entries per query head (a count, then the partials)
+    int few;                           // copy-engine form: few enough sequences and tiles for the short way to a CTA's share
     int deal_shift;                    // copy-engine form: log2 of the sequences in a block of its sums
     unsigned int* status;              // device status word of the call's workspace (bounded waits of the copy-engine form)
     unsigned long long wait_limit_ns;

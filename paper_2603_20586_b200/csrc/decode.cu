@@ -303,55 +303,59 @@ __global__ void __launch_bounds__(kWarps * 32, 2) decode_cluster_kernel(const De
     cluster_sync();
 }
 
-template <int DH>
-__global__ void __launch_bounds__(DH) decode_combine_kernel(const DecodeParams p) {
+// GROUPS > 1: many chunks, dealt in turn to that many groups of DH threads (a thread per column each).
+template <int DH, int GROUPS>
+__global__ void __launch_bounds__(DH * GROUPS) decode_combine_kernel(const DecodeParams p) {
     chain_enter();
+    constexpr int kThreads = DH * GROUPS;
     const long long bh = blockIdx.x;
     const int b = (int)(bh / p.H);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, col = tid % DH, grp = tid / DH;
     const float* part = p.partial + bh * p.total_chunks * (DH + 2);
     float lam[3] = {1.f, 1.f, 1.f};
-    long long total = p.total_chunks;
+    // The kernel is a chain of memory round trips, so all that may be needed is asked for at once, bounded by the room that there is: the
+    // number of partials, the maxima and sums, and the accumulators of the first chunks.  (112 heads x 20 chunks: 8.6 us with three trips
+    // one after the other, 6.3 with two.  28 heads x 56 chunks: 5.5 us with two and a third for the chunks past 32, now 3.6.)
+    constexpr int kAhead = GROUPS == 1 ? 32 : 16;
+    const int n_room = (int)(p.total_chunks - (p.counted ? 1 : 0));
+    float count = 0.f;
     if (p.counted) {
-        const float count = part[0];                           // (a call whose waits ran out may not have written it)
-        total = count > 0.f ? (long long)fminf(count, (float)(p.total_chunks - 1)) : 0;
+        count = part[0];
         part += DH + 2;
     } else {
 #pragma unroll
         for (int l = 0; l < 3; ++l) lam[l] = p.gate[b * 3 + l];
     }
-    const long long c1 = p.n_chunks[0], c2 = c1 + p.n_chunks[1];
-    // The kernel is a chain of memory round trips, so the accumulators of the first chunks are asked for along with the
-    // maxima and sums (112 heads x 20 chunks: 8.6 us with three trips one after the other, 6.3 with one).
-    constexpr int kAhead = 32;
+    float m_own = -INFINITY, z_own = 0.f;                      // chunk tid's
+    if (tid < n_room) { m_own = part[(long long)tid * (DH + 2)]; z_own = part[(long long)tid * (DH + 2) + 1]; }
     float ahead[kAhead];
-    const int n_room = (int)(p.total_chunks - (p.counted ? 1 : 0)), n_ahead = total < kAhead ? (int)total : kAhead;
 #pragma unroll
-    for (int j = 0; j < kAhead; ++j) ahead[j] = j < n_room ? part[j * (DH + 2) + 2 + tid] : 0.f;
-    float m_own = -INFINITY, z_own = 0.f;                      // chunk tid's, which the weights need again
+    for (int j = 0; j < kAhead; ++j) ahead[j] = grp + j * GROUPS < n_room ? part[(long long)(grp + j * GROUPS) * (DH + 2) + 2 + col] : 0.f;
+    // (a call whose waits ran out may not have written the count)
+    const long long total = !p.counted ? p.total_chunks : (count > 0.f ? (long long)fminf(count, (float)n_room) : 0);
+    const long long c1 = p.n_chunks[0], c2 = c1 + p.n_chunks[1];
     // global maximum over the chunks that count (gate > 0 and something summed): warp shuffles, then
     // one shared-memory hop across the CTA's warps
     float M = -INFINITY;
-    for (long long c = tid; c < total; c += DH) {
+    for (long long c = tid; c < total; c += kThreads) {
         const float g = c < c1 ? lam[0] : (c < c2 ? lam[1] : lam[2]);
-        const float mc = part[c * (DH + 2)], zc = part[c * (DH + 2) + 1];
-        if (c == tid) { m_own = mc; z_own = zc; }
+        const float mc = c == tid ? m_own : part[c * (DH + 2)], zc = c == tid ? z_own : part[c * (DH + 2) + 1];
         if (g > 0.f && zc > 0.f) M = fmaxf(M, mc);
     }
     M = warp_max(M);
-    __shared__ float sm[DH / 32];
+    __shared__ float sm[kThreads / 32];
     if (lane == 0) sm[warp] = M;
     __syncthreads();
     M = sm[0];
 #pragma unroll
-    for (int w = 1; w < DH / 32; ++w) M = fmaxf(M, sm[w]);
+    for (int w = 1; w < kThreads / 32; ++w) M = fmaxf(M, sm[w]);
 
-    // Weights of a batch of DH chunks are worked out side by side (one chunk per thread) and parked in shared
+    // Weights of a batch of kThreads chunks are worked out side by side (one chunk per thread) and parked in shared
     // memory; the accumulation over the batch then runs without a branch, its loads independent of each other.
     float Z = 0.f, A = 0.f;
-    __shared__ float sw[DH];
+    __shared__ float sw[kThreads];
     if (M > -INFINITY) {
-        for (long long c0 = 0; c0 < total; c0 += DH) {
+        for (long long c0 = 0; c0 < total; c0 += kThreads) {
             const long long c = c0 + tid;
             float w = 0.f;
             if (c < total) {
@@ -362,37 +366,51 @@ __global__ void __launch_bounds__(DH) decode_combine_kernel(const DecodeParams p
             __syncthreads();                                   // the previous batch has been consumed
             sw[tid] = w;
             __syncthreads();
-            const int nb = total - c0 < DH ? (int)(total - c0) : DH;
-            const float* col = part + c0 * (DH + 2) + 2 + tid;
-            int j = 0;
+            const int nb = total - c0 < kThreads ? (int)(total - c0) : kThreads;
+            const float* at = part + c0 * (DH + 2) + 2 + col;
+            int j = grp;
             if (c0 == 0) {
 #pragma unroll
                 for (int u = 0; u < kAhead; ++u)
-                    if (u < n_ahead) A = fmaf(sw[u], ahead[u], A);
-                j = n_ahead;
+                    if (grp + u * GROUPS < nb) A = fmaf(sw[grp + u * GROUPS], ahead[u], A);
+                j += kAhead * GROUPS;
             }
-            for (; j + 8 <= nb; j += 8) {
+            for (; j + 7 * GROUPS < nb; j += 8 * GROUPS) {
                 float v[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = col[(long long)(j + u) * (DH + 2)];
+                for (int u = 0; u < 8; ++u) v[u] = at[(long long)(j + u * GROUPS) * (DH + 2)];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) A = fmaf(sw[j + u], v[u], A);
+                for (int u = 0; u < 8; ++u) A = fmaf(sw[j + u * GROUPS], v[u], A);
             }
-            for (; j < nb; ++j) A = fmaf(sw[j], col[(long long)j * (DH + 2)], A);
+            for (; j < nb; j += GROUPS) A = fmaf(sw[j], at[(long long)j * (DH + 2)], A);
         }
     }
     // Z: every thread holds the share of its own chunks
     Z = warp_sum(Z);
-    __shared__ float sz[DH / 32];
+    __shared__ float sz[kThreads / 32], sa[GROUPS > 1 ? GROUPS - 1 : 1][DH];
     if (lane == 0) sz[warp] = Z;
+    if (GROUPS > 1 && grp > 0) sa[grp - 1][col] = A;
     __syncthreads();
+    if (grp > 0) return;
     Z = 0.f;
 #pragma unroll
-    for (int w = 0; w < DH / 32; ++w) Z += sz[w];
+    for (int w = 0; w < kThreads / 32; ++w) Z += sz[w];
+#pragma unroll
+    for (int g = 1; g < GROUPS; ++g) A += sa[g - 1][col];
     __nv_bfloat16* O = static_cast<__nv_bfloat16*>(p.O) + bh * DH;
-    O[tid] = __float2bfloat16_rn(Z > 0.f ? A / Z : 0.f);
+    O[col] = __float2bfloat16_rn(Z > 0.f ? A / Z : 0.f);
     if (p.status && bh == 0 && tid == 0) *p.status = MKA_OK;
     if (p.LSE && tid == 0) p.LSE[bh] = Z > 0.f ? (M + log2f(Z)) * kLn2 : -INFINITY;
+}
+
+// Four groups where a thread would have many chunks and the CTAs leave SMs idle; at d = 64, where a group is two warps, for more than it
+// asks for at once.  Router and decode, us, one group / four: 4 x 28 heads on 4 at 6500 rows, d = 128 (19 partials) 25.1 / [23.3]; at 10,500 rows,
+// d = 64 [18.2] / 18.9; 28 heads on 4 at 10,500 rows, d = 128 (56 partials) 20.8 with a third round trip, [16.8].
+template <int DH>
+cudaError_t launch_combine(const DecodeParams& p, cudaStream_t st) {
+    const dim3 grid((unsigned)((long long)p.B * p.H));
+    if ((p.counted ? p.expected > (DH == 128 ? 8 : 32) : p.total_chunks > 32) && grid.x <= 296) return launch_chained(decode_combine_kernel<DH, 4>, grid, dim3(DH * 4), 0, st, 0, p);
+    return launch_chained(decode_combine_kernel<DH, 1>, grid, dim3(DH), 0, st, 0, p);
 }
 
 // CTAs per (batch, head) of the one-kernel form, 0 = the split form.  As many as keep all clusters resident at once (296 CTAs);
@@ -431,7 +449,7 @@ cudaError_t launch_t(const DecodeParams& p, cudaStream_t st) {
         cudaError_t e = launch_chained(decode_partial_kernel<DH>, dim3((unsigned)(bh * p.total_chunks)), dim3(kWarps * 32), 0, st, 0, p);
         if (e != cudaSuccess) return e;
     }
-    return launch_chained(decode_combine_kernel<DH>, dim3((unsigned)bh), dim3(DH), 0, st, 0, p);
+    return launch_combine<DH>(p, st);
 }
 
 }  // namespace
@@ -440,7 +458,7 @@ cudaError_t launch_decode_combine(const DecodeParams& p, cudaStream_t st) {
     const long long bh = (long long)p.B * p.H;
     if (bh == 0) return cudaSuccess;
     if (p.d != 128 && p.d != 64) return cudaErrorNotSupported;
-    return launch_chained(p.d == 128 ? decode_combine_kernel<128> : decode_combine_kernel<64>, dim3((unsigned)bh), dim3(p.d), 0, st, 0, p);
+    return p.d == 128 ? launch_combine<128>(p, st) : launch_combine<64>(p, st);
 }
 
 cudaError_t launch_decode(const DecodeParams& p, cudaStream_t st) {
