@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(DH * GROUPS) decode_combine_kernel(const Decod
     float lam[3] = {1.f, 1.f, 1.f};
     // The kernel is a chain of memory round trips, so all that may be needed is asked for at once, bounded by the room that there is: the
     // number of partials, the maxima and sums, and the accumulators of the first chunks.  (112 heads x 20 chunks: 8.6 us with three trips
-    // one after the other, 6.3 with two.  28 heads x 56 chunks: 5.5 us with two and a third for the chunks past 32, now 3.6.)
+    // one after the other, 6.3 with two.  28 heads x 56 chunks: 5.5 us with two and a third for the chunks past 32.)
     constexpr int kAhead = GROUPS == 1 ? 32 : 16;
     const int n_room = (int)(p.total_chunks - (p.counted ? 1 : 0));
     float count = 0.f;
