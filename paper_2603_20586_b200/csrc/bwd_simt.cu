@@ -5,6 +5,8 @@
 //   dG[b,t,l] = sum_h G[b,h,t,l] (fixed order): blocks of the dK/dV launch beside those of the key tiles
 // Every output element is produced by exactly one CTA in a fixed summation order, so the result is
 // deterministic.  fp32 arithmetic; 16 or 32 rows against tiles of 32, see simt.cuh.
+#include <type_traits>
+
 #include "simt.cuh"
 
 namespace mka {
@@ -175,14 +177,20 @@ __global__ void __launch_bounds__(SimtCta<GROUPS>::kThreads, GROUPS == 1 ? 2 : 1
     // Gate-logit gradient G_l = sum_{j in l} p (dP - D).  Here D is taken as sum_{l,j} p dP / sum p, which
     // equals dO.O exactly in real arithmetic but does not inherit the rounding of O to its storage
     // type, so that sum_l G_l = 0 holds to fp32 accuracy.
-    float a[3], sp[3];
+    // (eight groups' sums in 64 bits, as in the forward)
+    using Sum = std::conditional_t<S::kGroups == 8, double, float>;
+    Sum a[3], sp[3];
 #pragma unroll
-    for (int l = 0; l < 3; ++l) { a[l] = total(l); sp[l] = total(3 + l); }
-    const float stot = sp[0] + sp[1] + sp[2];
-    const float dd = stot > 0.f ? (a[0] + a[1] + a[2]) / stot : 0.f;
+    for (int l = 0; l < 3; ++l) {
+        a[l] = o[l]; sp[l] = o[3 + l];
+#pragma unroll
+        for (int g = 1; g < S::kGroups; ++g) { a[l] += o[g * kRows * kState + l]; sp[l] += o[g * kRows * kState + 3 + l]; }
+    }
+    const Sum stot = sp[0] + sp[1] + sp[2];
+    const Sum dd = stot > 0 ? (a[0] + a[1] + a[2]) / stot : 0;
 #pragma unroll
     for (int l = 0; l < 3; ++l)
-        if (lane == 0) p.Gpart[(bh * p.T + t) * 3 + l] = a[l] - sp[l] * dd;
+        if (lane == 0) p.Gpart[(bh * p.T + t) * 3 + l] = static_cast<float>(a[l] - sp[l] * dd);
     }
 }
 

@@ -281,18 +281,19 @@ __global__ void __launch_bounds__(kWarps * 32, 2) decode_cluster_kernel(const De
     const int per = (DH + size - 1) / size, c = rank * per + (int)threadIdx.x;
     if ((int)threadIdx.x < per && c < DH) {
         float M = -INFINITY, Z = 0.f, A = 0.f;
-        float mi[kMaxCluster];
+        // All reads at once, a missing CTA's from the first one: a branch for each made them follow one another.
+        float mi[kMaxCluster], zi[kMaxCluster], ai[kMaxCluster];
 #pragma unroll
         for (int i = 0; i < kMaxCluster; ++i) {
-            mi[i] = i < size ? ld_cluster(smem_u32(&cta_m), i) : -INFINITY;
-            M = fmaxf(M, mi[i]);
+            const int from = i < size ? i : 0;
+            mi[i] = ld_cluster(smem_u32(&cta_m), from); zi[i] = ld_cluster(smem_u32(&cta_z), from); ai[i] = ld_cluster(smem_u32(&cta_acc[c]), from);
         }
 #pragma unroll
+        for (int i = 0; i < kMaxCluster; ++i) M = fmaxf(M, mi[i]);
+#pragma unroll
         for (int i = 0; i < kMaxCluster; ++i) {
-            if (i >= size) break;
-            const float f = M > -INFINITY ? exp2f(mi[i] - M) : 0.f;
-            Z = fmaf(ld_cluster(smem_u32(&cta_z), i), f, Z);
-            A = fmaf(ld_cluster(smem_u32(&cta_acc[c]), i), f, A);
+            const float f = i < size && M > -INFINITY ? exp2f(mi[i] - M) : 0.f;
+            if (i < size) { Z = fmaf(zi[i], f, Z); A = fmaf(ai[i], f, A); }
         }
         static_cast<__nv_bfloat16*>(p.O)[bh * DH + c] = __float2bfloat16_rn(Z > 0.f ? A / Z : 0.f);
         if (c == 0) {

@@ -487,11 +487,13 @@ __global__ void __launch_bounds__(kRetThreads) l3_retrieve_kernel(const L3Retrie
     cluster_sync();                                            // every CTA's counts are there
     for (int i = tid; i <= p.bits; i += kRetThreads) {
         int sum = 0, front = 0;
+        int v[kRetMaxCluster];                                 // all reads at once, a missing CTA's from the first one
+#pragma unroll
+        for (int r = 0; r < kRetMaxCluster; ++r) v[r] = __float_as_int(ld_cluster(smem_u32(&hist[i]), r < size ? r : 0));
 #pragma unroll
         for (int r = 0; r < kRetMaxCluster; ++r) {
-            const int v = r < size ? __float_as_int(ld_cluster(smem_u32(&hist[i]), r)) : 0;
-            sum += v;
-            front += r < rank ? v : 0;
+            sum += r < size ? v[r] : 0;
+            front += r < rank ? v[r] : 0;
         }
         total[i] = sum; lower[i] = front;
     }
