@@ -54,15 +54,15 @@ def load_peaks():
 # as it was when the counters were taken: when the file has changed since, the figure is reported as null ("stale").
 NCU_TRAFFIC = {
     # kernel@workload: (bytes in the capture, units of the capture, summary file under profiles/, source file, its digest)
-    "fwd_tc_kernel@c3": (375.181056e6 + 56.532736e6, 1 * 8, "fwd_tc_kernel_c3p.md", "fwd_tc.cu", "095d5fd190c0"),
-    "fwd_tc_kernel64@c2": (204.155136e6 + 25.436160e6, 8 * 16, "fwd_tc_kernel64_c2.md", "fwd_tc.cu", "095d5fd190c0"),   # the whole configuration
-    "decode_partial_kernel@c4": (1.476457e9 + 4.163328e6, 2 * 32, "decode_partial_kernel_c4p.md", "decode.cu", "8ff55e2ca41e"),
-    "bwd_dq_tc_kernel@c5": (220.371456e6 + 26.972160e6, 1 * 16, "bwd_tc_kernels_c5p.md", "bwd_tc.cu", "0f66e669b095"),
-    "bwd_dkv_tc_kernel@c5": (221.904384e6 + 118.048512e6, 1 * 16, "bwd_tc_kernels_c5p.md", "bwd_tc.cu", "0f66e669b095"),
+    "fwd_tc_kernel@c3": (375.179264e6 + 56.739328e6, 1 * 8, "fwd_tc_kernel_c3p.md", "fwd_tc.cu", "4c90380f91c4"),
+    "fwd_tc_kernel64@c2": (206.649344e6 + 27.328256e6, 8 * 16, "fwd_tc_kernel64_c2.md", "fwd_tc.cu", "4c90380f91c4"),   # the whole configuration
+    "decode_partial_kernel@c4": (1.476449e9 + 4.224768e6, 2 * 32, "decode_partial_kernel_c4p.md", "decode.cu", "502997e1c1d8"),
+    "bwd_dq_tc_kernel@c5": (220.644864e6 + 26.942464e6, 1 * 16, "bwd_tc_kernels_c5p.md", "bwd_tc.cu", "1809b0267c2d"),
+    "bwd_dkv_tc_kernel@c5": (221.846528e6 + 118.659072e6, 1 * 16, "bwd_tc_kernels_c5p.md", "bwd_tc.cu", "1809b0267c2d"),
     "l2_summary_pipe_kernel@s3": (100.699392e6 + 54.012160e6, 12288.0 / 32768.0, "l2_summary_seg_kernel_s3p.md", "summary_seg.cu", "f824f10a3d76"),   # 12288 of the 32768 tokens
     "fuse_kv_kernel@f3": (403.136512e6 + 83.408640e6, 1 * 8, "fuse_kv_kernel_f3p.md", "fuse_kv.cu", "b1ef4c991e47"),
-    "decode_paged_kernel@g4": (293.730304e6 + 3.355136e6, 1 * 4, "decode_paged_kernel_g4p.md", "decode_paged.cu", "929e98e72397"),   # one of the four sequences (g4p)
-    "l3_index_kernel@r3": (134.305792e6 + 4.221696e6, 1, "l3_index_kernel_r3p.md", "l3.cu", "607ee4fa9ab7"),            # one of the four sequences (r3p)
+    "decode_paged_kernel@g4": (293.750528e6 + 3.454976e6, 1 * 4, "decode_paged_kernel_g4p.md", "decode_paged.cu", "0d8f44cbc542"),   # one of the four sequences (g4p)
+    "l3_index_kernel@r3": (134.585856e6 + 3.313920e6, 1, "l3_index_kernel_r3p.md", "l3.cu", "00671588e2bc"),            # one of the four sequences (r3p)
 }
 
 
