@@ -11,7 +11,6 @@ namespace {
 
 constexpr int kRowsPerWarp = 4;
 constexpr int kWarps = 8;
-constexpr int kMaxThreads = 256;
 
 __device__ __forceinline__ void finish_row(float g0, float g1, float g2, int route, long long row, float* gate,
                                            float* log2_gate, int8_t* idx) {
@@ -92,7 +91,7 @@ template <> struct Cols<float, 4> {
 };
 
 // Sums of ROWS rows x 3 logits over a warp: while a lane holds several rows it hands half of them to its partner and adds
-// the partner's other half, so that eight rows cost 27 shuffles instead of 120.  The lanes of group `row` (32 / ROWS of
+// the partner's other half, so that four rows cost 18 shuffles instead of 60.  The lanes of group `row` (32 / ROWS of
 // them) end with that row's sums in acc[0..2].
 template <int ROWS>
 __device__ __forceinline__ void sum_rows(float (&acc)[ROWS * 3], int lane, int& row) {
@@ -116,16 +115,20 @@ __device__ __forceinline__ void sum_rows(float (&acc)[ROWS * 3], int lane, int& 
         for (int l = 0; l < 3; ++l) acc[l] += __shfl_xor_sync(0xffffffffu, acc[l], off);
 }
 
-// One CTA takes ROWS rows and spreads D over its threads (eight columns each per pass), so the loads of a row are 16 bytes
-// a thread and independent of each other: ROWS of them are in flight, whatever the number of rows.  The kernel is bound by
+// One CTA takes ROWS rows and spreads D over its THREADS threads (COLS columns each per pass), so that the loads of a row are
+// independent of each other: ROWS of them are in flight, whatever the number of rows.  The kernel is bound by
 // one load's latency: a warp that walks four rows by itself took 11 us for ONE row of D = 4096.  With thousands of rows
-// the order turns round (see router_rows_kernel).
-template <typename T, int ROWS>
-__global__ void __launch_bounds__(kMaxThreads)
+// the order turns round (see router_rows_kernel).  A thread's columns of W_r lie 12 COLS bytes from its neighbour's, so a 16-byte read by a warp
+// touches 24 lines at eight columns and 12 at four, and all of W_r (48 KB at D = 4096) goes through each CTA's L1: with four columns and
+// twice the threads one row of 4096 takes 2.30 us instead of 2.56, 512 rows of 3584 3.84 instead of 4.78.  From 8 rows per SM on it is the
+// rows' own loads that count, and they shrink to 8 bytes: eight columns and 256 threads there (2000 rows of 2048: 4.1 us against 5.9).
+template <typename T, int ROWS, int COLS, int THREADS>
+__global__ void __launch_bounds__(THREADS)
 router_kernel(const T* __restrict__ R, const float* __restrict__ W_r, const float* __restrict__ b_r,
               long long rows, int D, int route, float* __restrict__ gate, float* __restrict__ log2_gate,
               int8_t* __restrict__ idx) {
-    __shared__ float part[kMaxThreads / 32][ROWS * 3];
+    using V = Cols<T, COLS>;
+    __shared__ float part[THREADS / 32][ROWS * 3];
     chain_enter();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long row0 = (long long)blockIdx.x * ROWS;
@@ -134,23 +137,25 @@ router_kernel(const T* __restrict__ R, const float* __restrict__ W_r, const floa
 #pragma unroll
     for (int i = 0; i < ROWS * 3; ++i) acc[i] = 0.f;
     const T* base = R + row0 * (long long)D;
-    for (int c = threadIdx.x * 8; c < D; c += blockDim.x * 8) {
-        typename Vec8<T>::Raw x[ROWS];
+    constexpr int kUnroll = ROWS == 2 ? 2 : 1;                // both passes of D = 4096 at once: 512 rows of 3584 3.84 us against 4.01; one row, four rows: nothing, or slower
+#pragma unroll kUnroll
+    for (int c = threadIdx.x * COLS; c < D; c += blockDim.x * COLS) {
+        typename V::Raw x[ROWS];
 #pragma unroll
-        for (int r = 0; r < ROWS; ++r) x[r] = Vec8<T>::fetch(base + (r <= last ? r : last) * D + c);
-        float w[24];
+        for (int r = 0; r < ROWS; ++r) x[r] = V::fetch(base + (r <= last ? r : last) * D + c);
+        float w[3 * COLS];
         const float4* wp = reinterpret_cast<const float4*>(W_r + (long long)c * 3);
 #pragma unroll
-        for (int i = 0; i < 6; ++i) {
+        for (int i = 0; i < 3 * COLS / 4; ++i) {
             const float4 v = __ldg(wp + i);
             w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
         }
 #pragma unroll
         for (int r = 0; r < ROWS; ++r) {
-            float f[8];
-            Vec8<T>::widen(x[r], f);
+            float f[COLS];
+            V::widen(x[r], f);
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
+            for (int i = 0; i < COLS; ++i)
 #pragma unroll
                 for (int l = 0; l < 3; ++l) acc[r * 3 + l] = fmaf(f[i], w[3 * i + l], acc[r * 3 + l]);
         }
@@ -432,19 +437,26 @@ cudaError_t router_t(const T* R, const float* W_r, const float* b_r, long long r
         return launch_chained(router_any_kernel<T>, dim3((unsigned)((rows + rows_per_cta - 1) / rows_per_cta)), dim3(kWarps * 32), 0, st, 0,
                               R, W_r, b_r, rows, D, route, gate, log2_gate, idx);
     }
-    // Up to two rows per SM: one row to a CTA, for the shortest chain; to eight per SM: two; below 32 a row is still better
-    // split over a CTA (2000 rows of 2048 bf16: 5.2 us against 8.4), above it the warps have enough to do on their own
-    // (32768 rows: 28 us against 51; loads ahead of the sums and W_r in shared memory were slower too, 35 and 44 us).
-    if (rows >= 32 * 148) {
+    // Up to two rows per SM: one row to a CTA, for the shortest chain; to four per SM: two; above: four (777 rows of 1024: 2.56 us, 2.9 with two;
+    // 1000 rows of 4096: 4.5 against 4.7; 512 rows of 3584: two 3.84, four 5.0; 2000 rows of 2048: four 4.1, eight 4.6; 4700 of 4096: 10.8, 12.9).
+    // With many rows the warps have enough to do on their own, a row each: the sooner the shorter the rows (a CTA's time against the
+    // warps': 4800 rows of 768 4.10 us, 4.95, 9400 of 256 4.4, 3.7 and of 768 6.4, 6.0; 8192 of 1024 6.7, 7.5, 9400 of 1536 10.4, 10.1; 5000 of 4096 12.4, 20.7,
+    // 16384 of 1024 10.8, 9.0, 32768 of 2048 36, 28; loads ahead of the sums and W_r in shared memory were slower too, 35 and 44 us).
+    const int warps_from = D >= 2048 ? 64 : (D >= 1024 ? 56 : (D >= 768 ? 40 : 32));   // rows per SM
+    if (rows >= warps_from * 148) {
         const long long rows_per_cta = kWarps * kRowsPerWarp;
         return launch_chained(router_rows_kernel<T>, dim3((unsigned)((rows + rows_per_cta - 1) / rows_per_cta)), dim3(kWarps * 32), 0, st, 0,
                               R, W_r, b_r, rows, D, route, gate, log2_gate, idx);
     }
-    const int threads = D >= 8 * kMaxThreads ? kMaxThreads : (D / 8 + 31) / 32 * 32;
-    const int per_cta = rows >= 8 * 148 ? 8 : (rows >= 2 * 148 ? 2 : 1);
-    auto kern = per_cta == 8 ? router_kernel<T, 8> : (per_cta == 2 ? router_kernel<T, 2> : router_kernel<T, 1>);
-    return launch_chained(kern, dim3((unsigned)((rows + per_cta - 1) / per_cta)), dim3(threads), 0, st, 0, R, W_r, b_r, rows, D, route, gate,
-                          log2_gate, idx);
+    auto go = [&](auto kern, int per_cta, int cols, int most) {
+        const int threads = D >= cols * most ? most : (D / cols + 31) / 32 * 32;
+        return launch_chained(kern, dim3((unsigned)((rows + per_cta - 1) / per_cta)), dim3(threads), 0, st, 0, R, W_r, b_r, rows, D, route, gate,
+                              log2_gate, idx);
+    };
+    if (rows >= 8 * 148) return go(router_kernel<T, 4, 8, 256>, 4, 8, 256);
+    if (rows >= 4 * 148) return go(router_kernel<T, 4, 4, 512>, 4, 4, 512);
+    if (rows >= 2 * 148) return go(router_kernel<T, 2, 4, 512>, 2, 4, 512);
+    return go(router_kernel<T, 1, 4, 512>, 1, 4, 512);
 }
 }  // namespace
 
