@@ -191,7 +191,8 @@ def _address(function) -> int:
     return ctypes.cast(function, ctypes.c_void_p).value
 
 
-# The entry points that short steps consist of are called from native code too: tensors, None and ints go in as they are.
+# The entry points that short steps consist of are called from native code too: tensors, None and ints go in as they are (an int
+# only as a count or the stream, never in a tensor's place).
 _router, _fwd, _fwd_paged = _address(lib.mka_router), _address(lib.mka_fwd_with_scratch), _address(lib.mka_fwd_paged_with_scratch)
 _decode, _decode_paged, _bwd = _address(lib.mka_decode), _address(lib.mka_decode_paged), _address(lib.mka_bwd)
 

@@ -11,6 +11,7 @@
 #include <string.h>
 
 #include <tuple>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -226,16 +227,19 @@ template <> struct Arg<size_t> {
     size_t v;
     explicit Arg(PyObject* o) : v(static_cast<size_t>(Arg<int64_t>(o).v)) {}
 };
-template <typename T> struct Arg<T*> {               // a tensor's memory, an address, or None
+template <typename T> struct Arg<T*> {               // a tensor's memory, or None; no int, as True in an output's place would be address 1
     T* v;
     explicit Arg(PyObject* o) : v(nullptr) {
+        if (o != Py_None) v = static_cast<T*>(tensor(o).data_ptr());
+    }
+};
+struct Address {                                     // of a function, or a stream's handle
+    void* v;
+    explicit Address(PyObject* o) : v(nullptr) {
         if (o == Py_None) return;
-        if (PyLong_Check(o)) {
-            v = static_cast<T*>(PyLong_AsVoidPtr(o));
-            if (!v && PyErr_Occurred()) throw PyErrSet();
-        } else {
-            v = static_cast<T*>(tensor(o).data_ptr());
-        }
+        if (!PyLong_Check(o)) throw Bad();
+        v = PyLong_AsVoidPtr(o);
+        if (!v && PyErr_Occurred()) throw PyErrSet();
     }
 };
 template <typename T> struct Levels {                // three levels as `levels`, `grads` or `paged_levels` returned them
@@ -265,12 +269,13 @@ template <> struct Arg<const mka_shape*> {
     Arg(const Arg&) = delete;
 };
 
-// The library's function at address a[0] (of the type of the declaration named) with the other arguments; its status.  Other threads run meanwhile.
+// The library's function at address a[0] (of the type of the declaration named) with the other arguments, the last of which is the stream; its
+// status.  Other threads run meanwhile.
 template <typename R, typename... P, size_t... I>
 PyObject* invoke(R (*)(P...), PyObject* const* a, std::index_sequence<I...>) {
-    const auto f = reinterpret_cast<R (*)(P...)>(Arg<void*>(a[0]).v);
+    const auto f = reinterpret_cast<R (*)(P...)>(Address(a[0]).v);
     if (!f) throw Bad();
-    const std::tuple<Arg<P>...> args{a[1 + I]...};
+    const std::tuple<std::conditional_t<I + 1 == sizeof...(P), Address, Arg<P>>...> args{a[1 + I]...};
     R status;
     Py_BEGIN_ALLOW_THREADS
     status = f(std::get<I>(args).v...);

@@ -36,7 +36,7 @@ def test_status_is_the_librarys():
 
 @pytest.mark.parametrize("args,error", [
     ((1,), AssertionError),                                                                    # too few
-    (("x", 0, 0, 0, 4, 8, 1, 0, None, None, None, 0), AssertionError),                         # neither tensor, address nor None
+    (("x", 0, 0, 0, 4, 8, 1, 0, None, None, None, 0), AssertionError),                         # neither tensor nor None
     ((None, None, None, 4.0, 8, 1, 0, None, None, None, 0), TypeError),                        # a float for a count
     ((None, None, None, 2 ** 70, 8, 1, 0, None, None, None, 0), OverflowError),
 ])
@@ -58,3 +58,59 @@ def test_shapes_and_levels_that_are_refused(shape, levels, error):
 def test_row_counts():
     K = [torch.zeros(1, 1, 5, 4), None, torch.zeros(1, 1, 0, 4)]
     assert b._row_counts(K) == (5, 0, 0) == b._row_counts(tuple(K)) == b._row_counts(dict(enumerate(K)))
+
+
+class _Legacy:
+    cuda_stream = 0                                           # (asking for the current stream would need a GPU)
+
+
+def _calls():
+    """Each call of the public functions with nothing to launch, and the names of its arguments that are memory."""
+    none, n = [None] * 3, dict(stream=_Legacy())
+    Q, q = torch.zeros(1, 2, 0, 64, dtype=torch.bfloat16), torch.zeros(0, 2, 64, dtype=torch.bfloat16)
+    g, lse, ws, X, W = torch.zeros(1, 0, 3), torch.zeros(1, 2, 0), torch.zeros(256, dtype=torch.uint8), torch.zeros(0, 8), torch.zeros(8, 3)
+    seqs, steps = _shape(T=0), _shape(B=0, T=1)
+    out = dict(O=torch.zeros(1, 2, 0, 64), LSE=lse)
+    return {
+        "router": (mka.mka_router, dict(R=X, W_r=W, b_r=None, gate=g, **n), ("b_r", "gate", "log2_gate", "route_idx")),
+        "fwd": (mka.mka_fwd, dict(shape=seqs, Q=Q, K=none, V=none, gate=g, ws=ws, **out, **n), ("Q", "gate", "O", "LSE", "ws")),
+        "fwd_paged": (mka.mka_fwd_paged, dict(shape=seqs, H_kv=2, Q=Q, pools_k=none, pools_v=none, tables=none, n=(0, 0, 0), gate=g, ws=ws, **out, **n),
+                      ("Q", "gate", "O", "LSE", "ws")),
+        "decode": (mka.mka_decode, dict(shape=steps, q=q, K=none, V=none, gate=g, ws=ws, **out, **n), ("q", "gate", "O", "LSE", "ws")),
+        "decode_paged": (mka.mka_decode_paged, dict(shape=steps, H_kv=2, q=q, pools_k=none, pools_v=none, tables=none, n=(0, 0, 0), gate=g, ws=ws, **out, **n),
+                         ("q", "gate", "O", "LSE", "ws")),
+        "bwd": (mka.mka_bwd, dict(shape=seqs, Q=Q, K=none, V=none, gate=g, O=Q, LSE=lse, dO=Q, ws=ws, **n),
+                ("Q", "gate", "O", "LSE", "dO", "R", "dQ", "dG", "dW_r", "db_r", "ws")),
+    }
+
+
+@pytest.mark.parametrize("name", ["router", "fwd", "fwd_paged", "decode", "decode_paged", "bwd"])
+def test_numbers_are_no_memory(name):
+    function, args, memory = _calls()[name]
+    function(**args)
+    for key in memory:
+        for wrong in (True, False, 0, 1, 2 ** 40):
+            with pytest.raises((AssertionError, AttributeError)):
+                function(**{**args, key: wrong})
+
+
+def test_every_pointer_of_a_native_call_refuses_numbers():
+    none = [None] * 3
+    lv, gr, pl = b._levels(none, none), H.grads(none, none, none), b._paged_levels(none, none, none, None, (0, 0, 0))
+    empty, step = _shape(T=0), _shape(B=0, T=1)
+    for call, address, args in [
+            (H.call_router, b._router, (None, None, None, 0, 8, 1, 0, None, None, None)),
+            (H.call_fwd, b._fwd, (empty, None, lv, None, None, None, None, 0, None, 0)),
+            (H.call_fwd_paged, b._fwd_paged, (empty, 1, None, pl, None, None, None, None, 0, None, 0)),
+            (H.call_decode, b._decode, (step, None, lv, None, None, None, None, 0)),
+            (H.call_decode_paged, b._decode_paged, (step, 1, None, pl, None, None, None, None, 0)),
+            (H.call_bwd, b._bwd, (empty, None, lv, None, None, None, None, None, 0, None, gr, None, None, None, None, 0))]:
+        for i, x in enumerate(args):
+            if x is not None:
+                continue
+            for wrong in (True, 0, 8):
+                with pytest.raises(AssertionError):
+                    call(address, *args[:i], wrong, *args[i + 1:], 0)
+        for wrong in (1.0, torch.zeros(1)):                    # nor is a tensor a stream
+            with pytest.raises(AssertionError):
+                call(address, *args, wrong)
