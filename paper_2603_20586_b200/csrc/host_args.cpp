@@ -210,12 +210,9 @@ PyObject* empty_f32(PyObject*, PyObject* const* a, Py_ssize_t n) {
 template <typename P> struct Arg;
 template <> struct Arg<int64_t> {
     int64_t v;
-    explicit Arg(PyObject* o) : v(0) {
-        if (!PyLong_Check(o)) {
-            PyErr_SetString(PyExc_TypeError, "an int is expected");
-            throw PyErrSet();
-        }
-        v = PyLong_AsLongLong(o);
+    explicit Arg(PyObject* o) : v(0) {                // an int or what answers __index__ as one (numpy's, a tensor's); no float
+        const Held whole(PyNumber_Index(o));
+        v = PyLong_AsLongLong(whole.o);
         if (v == -1 && PyErr_Occurred()) throw PyErrSet();
     }
 };
@@ -227,19 +224,36 @@ template <> struct Arg<size_t> {
     size_t v;
     explicit Arg(PyObject* o) : v(static_cast<size_t>(Arg<int64_t>(o).v)) {}
 };
-template <typename T> struct Arg<T*> {               // a tensor's memory, or None; no int, as True in an output's place would be address 1
+void* pointer(PyObject* o) {                         // an int, or None for null
+    if (o == Py_None) return nullptr;
+    if (!PyLong_Check(o)) throw Bad();
+    void* const v = PyLong_AsVoidPtr(o);
+    if (!v && PyErr_Occurred()) throw PyErrSet();
+    return v;
+}
+// A tensor's memory, or that of whatever else has a data_ptr(), as a storage has, or None; no int, as True in an output's place would be address 1.
+template <typename T> struct Arg<T*> {
     T* v;
     explicit Arg(PyObject* o) : v(nullptr) {
-        if (o != Py_None) v = static_cast<T*>(tensor(o).data_ptr());
+        if (o == Py_None) return;
+        if (THPVariable_Check(o)) {
+            v = static_cast<T*>(tensor(o).data_ptr());
+            return;
+        }
+        if (!PyObject_HasAttrString(o, "data_ptr")) throw Bad();
+        const Held at(PyObject_CallMethod(o, "data_ptr", nullptr));
+        v = static_cast<T*>(pointer(at.o));
     }
 };
-struct Address {                                     // of a function, or a stream's handle
+struct Address {                                     // of a function, or a stream's handle: an int, or what holds one as a c_void_p does
     void* v;
     explicit Address(PyObject* o) : v(nullptr) {
-        if (o == Py_None) return;
-        if (!PyLong_Check(o)) throw Bad();
-        v = PyLong_AsVoidPtr(o);
-        if (!v && PyErr_Occurred()) throw PyErrSet();
+        if (o == Py_None || PyLong_Check(o) || !PyObject_HasAttrString(o, "value")) {
+            v = pointer(o);
+            return;
+        }
+        const Held at(PyObject_GetAttrString(o, "value"));
+        v = pointer(at.o);
     }
 };
 template <typename T> struct Levels {                // three levels as `levels`, `grads` or `paged_levels` returned them

@@ -2,6 +2,7 @@
 (calls that end at the library's own checks or have nothing to do: no GPU is needed)."""
 import ctypes
 
+import numpy as np
 import pytest
 import torch
 
@@ -114,3 +115,22 @@ def test_every_pointer_of_a_native_call_refuses_numbers():
         for wrong in (1.0, torch.zeros(1)):                    # nor is a tensor a stream
             with pytest.raises(AssertionError):
                 call(address, *args, wrong)
+
+
+@pytest.mark.parametrize("whole", [np.int64, np.int32, torch.tensor, int])
+def test_counts_may_be_whole_numbers_of_any_kind(whole):
+    calls = _calls()
+    for name, key, value in (("router", "route", 1), ("fwd_paged", "H_kv", 2), ("decode_paged", "H_kv", 2)):
+        function, args, _ = calls[name]
+        function(**{**args, key: whole(value)})
+        with pytest.raises((TypeError, ctypes.ArgumentError)):
+            function(**{**args, key: float(value)})
+
+
+def test_memory_and_streams_of_other_kinds():
+    function, args, _ = _calls()["router"]
+    function(**{**args, "log2_gate": torch.zeros(4).untyped_storage()})
+    for handle in (ctypes.c_void_p(0), ctypes.c_void_p(), None):
+        stream = _Legacy()
+        stream.cuda_stream = handle
+        function(**{**args, "stream": stream})
