@@ -184,6 +184,7 @@ _paged_levels = _host_args.paged_levels    # (pools_k, pools_v, tables, rows or 
                                            # [pages, H_kv, page_rows, d], any strides with d contiguous; tables [B, pages] or [B, H_kv, pages]
 _empty_f32 = _host_args.empty_f32          # (t, keep, extra) -> fp32 tensor of t's first `keep` dimensions (and `extra`)
 _empty_like = _host_args.empty_like
+_host_args.shape_type(mka_shape)
 _row_counts = _host_args.row_counts        # (K) -> the rows of three levels, 0 for None
 
 

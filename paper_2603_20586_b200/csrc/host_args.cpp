@@ -266,10 +266,25 @@ template <typename T> struct Levels {                // three levels as `levels`
 template <> struct Arg<const mka_level*> : Levels<mka_level> { using Levels::Levels; };
 template <> struct Arg<const mka_level_grad*> : Levels<mka_level_grad> { using Levels::Levels; };
 template <> struct Arg<const mka_paged_level*> : Levels<mka_paged_level> { using Levels::Levels; };
+PyObject* shape_class = nullptr;                     // the binding's mka_shape: other buffers of its size are no shapes
+PyObject* shape_type(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    if (n != 1 || !PyType_Check(a[0])) {
+        PyErr_SetString(PyExc_TypeError, "a class is expected");
+        return nullptr;
+    }
+    Py_INCREF(a[0]);
+    Py_XDECREF(shape_class);
+    shape_class = a[0];
+    Py_RETURN_NONE;
+}
 template <> struct Arg<const mka_shape*> {
     mka_shape copy;
     const mka_shape* v;
     explicit Arg(PyObject* o) : v(&copy) {
+        if (!shape_class || !PyObject_TypeCheck(o, reinterpret_cast<PyTypeObject*>(shape_class))) {
+            PyErr_SetString(PyExc_TypeError, "an mka_shape is expected");
+            throw PyErrSet();
+        }
         Py_buffer view;
         if (PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) != 0) throw PyErrSet();
         const bool fits = view.len == static_cast<Py_ssize_t>(sizeof(mka_shape));
@@ -342,6 +357,7 @@ PyMethodDef methods[] = {
     method("paged_level", paged_level, "paged_level(pool_k, pool_v, table) -> one mka_paged_level over the table's width as bytes"),
     method("empties_like", empties_like, "empties_like(tensors) -> list of empty_like, None for None"),
     method("empty_f32", empty_f32, "empty_f32(t, keep, extra) -> fp32 tensor of t's first `keep` dimensions, then `extra` if not 0"),
+    method("shape_type", shape_type, "shape_type(cls): the class whose instances are shapes"),
     method("empty_like", empty_like, "empty_like(t)"),
     method("row_counts", row_counts, "row_counts(K) -> the rows of three levels, 0 for None"),
     method("call_router", call_router, "call_router(address, arguments of mka_router...) -> its status"),

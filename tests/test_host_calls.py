@@ -134,3 +134,23 @@ def test_memory_and_streams_of_other_kinds():
         stream = _Legacy()
         stream.cuda_stream = handle
         function(**{**args, "stream": stream})
+
+
+@pytest.mark.parametrize("name", ["fwd", "fwd_paged", "decode", "decode_paged", "bwd"])
+def test_only_a_shape_is_a_shape(name):
+    native = {"fwd": (H.call_fwd, b._fwd), "fwd_paged": (H.call_fwd_paged, b._fwd_paged), "decode": (H.call_decode, b._decode),
+              "decode_paged": (H.call_decode_paged, b._decode_paged), "bwd": (H.call_bwd, b._bwd)}[name]
+    none = [None] * 3
+    lv, gr, pl = b._levels(none, none), H.grads(none, none, none), b._paged_levels(none, none, none, None, (0, 0, 0))
+    rest = {"fwd": (None, lv, None, None, None, None, 0, None, 0, 0), "fwd_paged": (1, None, pl, None, None, None, None, 0, None, 0, 0),
+            "decode": (None, lv, None, None, None, None, 0, 0), "decode_paged": (1, None, pl, None, None, None, None, 0, 0),
+            "bwd": (None, lv, None, None, None, None, None, 0, None, gr, None, None, None, None, 0, 0)}[name]
+    shape = _calls()[name][1]["shape"]
+
+    class Own(mka.mka_shape):
+        pass
+
+    native[0](native[1], Own.from_buffer_copy(shape), *rest)
+    for wrong in (bytes(shape), bytearray(shape), np.frombuffer(bytes(shape), dtype=np.uint8), (ctypes.c_int32 * 12).from_buffer_copy(shape)):
+        with pytest.raises(TypeError):
+            native[0](native[1], wrong, *rest)
