@@ -19,11 +19,14 @@
 
 namespace {
 
-struct Bad {};                                       // what an assertion of the binding would have refused
+constexpr char kLevelsWanted[] = "levels: tensors [batch, head, row, column] with dense columns, K and V alike; tables and row counts int32";
+constexpr char kTensorWanted[] = "a tensor (or None where an argument may be left out) is expected";
+constexpr char kCountWanted[] = "wrong number of arguments";
+struct Bad { const char* what = kLevelsWanted; };    // what an assertion of the binding would have refused
 struct PyErrSet {};                                  // the Python error is set
 
 const at::Tensor& tensor(PyObject* o) {
-    if (!THPVariable_Check(o)) throw Bad();
+    if (!THPVariable_Check(o)) throw Bad{kTensorWanted};
     return THPVariable_Unpack(o);
 }
 
@@ -78,11 +81,11 @@ template <size_t N> PyObject* bytes(const int64_t (&w)[N]) { return PyBytes_From
 
 // Four dimensions, the last one dense, and V laid out as K.
 void check_layout(const at::Tensor& k, const at::Tensor& v) {
-    if (k.dim() != 4 || k.stride(3) != 1 || v.strides() != k.strides()) throw Bad();
+    if (k.dim() != 4 || k.stride(3) != 1 || v.strides() != k.strides()) throw Bad{};
 }
 void check_pair(const at::Tensor& k, const at::Tensor& v) {
     check_layout(k, v);
-    if (v.sizes() != k.sizes()) throw Bad();
+    if (v.sizes() != k.sizes()) throw Bad{};
 }
 
 template <typename F>
@@ -90,8 +93,8 @@ PyObject* guarded(F f) {
     HANDLE_TH_ERRORS
     try {
         return f();
-    } catch (const Bad&) {
-        PyErr_SetString(PyExc_AssertionError, "levels: tensors [batch, head, row, column] with dense columns, K and V alike; tables and row counts int32");
+    } catch (const Bad& bad) {
+        PyErr_SetString(PyExc_AssertionError, bad.what);
         return nullptr;
     } catch (const PyErrSet&) {
         return nullptr;
@@ -106,14 +109,14 @@ void put_level(int64_t* o, const at::Tensor& k, const at::Tensor& v) {
 }
 PyObject* levels(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
-        if (n != 2) throw Bad();
+        if (n != 2) throw Bad{kCountWanted};
         Seq K(a[0]), V(a[1]);
         int64_t w[18] = {};
         for (int l = 0; l < 3; ++l) {
             const at::Tensor* k = K.tensor_at(l);
             if (!k || k->size(2) == 0) continue;
             const at::Tensor* v = V.tensor_at(l);
-            if (!v) throw Bad();
+            if (!v) throw Bad{};
             check_pair(*k, *v);
             put_level(w + 6 * l, *k, *v);
         }
@@ -122,14 +125,14 @@ PyObject* levels(PyObject*, PyObject* const* a, Py_ssize_t n) {
 }
 PyObject* grads(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
-        if (n != 3) throw Bad();
+        if (n != 3) throw Bad{kCountWanted};
         Seq K(a[0]), dK(a[1]), dV(a[2]);
         int64_t w[18] = {};
         for (int l = 0; l < 3; ++l) {
             const at::Tensor* k = K.tensor_at(l);
             if (!k || k->size(2) == 0) continue;
             const at::Tensor *dk = dK.tensor_at(l), *dv = dV.tensor_at(l);
-            if (!dk || !dv) throw Bad();
+            if (!dk || !dv) throw Bad{};
             check_layout(*dk, *dv);
             put_level(w + 6 * l, *dk, *dv);
         }
@@ -139,7 +142,7 @@ PyObject* grads(PyObject*, PyObject* const* a, Py_ssize_t n) {
 
 PyObject* paged_levels(PyObject*, PyObject* const* a, Py_ssize_t n_args) {
     return guarded([&]() -> PyObject* {
-        if (n_args != 5) throw Bad();
+        if (n_args != 5) throw Bad{kCountWanted};
         Seq K(a[0]), V(a[1]), tabs(a[2]), rows(a[3]), n(a[4]);
         const bool counted = a[3] != Py_None;
         int64_t w[36] = {};
@@ -151,11 +154,11 @@ PyObject* paged_levels(PyObject*, PyObject* const* a, Py_ssize_t n_args) {
             const int64_t most = integer(n.at(l));
             if (most == 0) continue;
             const at::Tensor *v = V.tensor_at(l), *tab = tabs.tensor_at(l), *r = counted ? rows.tensor_at(l) : nullptr;
-            if (!v || !tab) throw Bad();
+            if (!v || !tab) throw Bad{};
             check_pair(*k, *v);
             // [B, pages]: one table per sequence; [B, H_kv, pages]: one per (sequence, KV head)
-            if (tab->scalar_type() != at::kInt || (tab->dim() != 2 && tab->dim() != 3) || tab->stride(tab->dim() - 1) != 1) throw Bad();
-            if (r && (r->scalar_type() != at::kInt || !r->is_contiguous())) throw Bad();
+            if (tab->scalar_type() != at::kInt || (tab->dim() != 2 && tab->dim() != 3) || tab->stride(tab->dim() - 1) != 1) throw Bad{};
+            if (r && (r->scalar_type() != at::kInt || !r->is_contiguous())) throw Bad{};
             o[0] = address(*k); o[1] = address(*v); o[2] = address(*tab); o[3] = r ? address(*r) : 0;
             o[4] = most; o[5] = tab->stride(0); o[6] = tab->dim() == 3 ? tab->stride(1) : 0; o[7] = k->size(2);
             for (int i = 0; i < 3; ++i) o[8 + i] = k->stride(i);
@@ -167,10 +170,10 @@ PyObject* paged_levels(PyObject*, PyObject* const* a, Py_ssize_t n_args) {
 
 PyObject* paged_level(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
-        if (n != 3) throw Bad();
+        if (n != 3) throw Bad{kCountWanted};
         const at::Tensor &k = tensor(a[0]), &v = tensor(a[1]), &tab = tensor(a[2]);
         check_layout(k, v);
-        if (tab.scalar_type() != at::kInt || tab.dim() != 2 || tab.stride(1) != 1) throw Bad();
+        if (tab.scalar_type() != at::kInt || tab.dim() != 2 || tab.stride(1) != 1) throw Bad{};
         const int64_t w[12] = {address(k), address(v), address(tab), 0, tab.size(1) * k.size(2), tab.stride(0), 0, k.size(2),
                                k.stride(0), k.stride(1), k.stride(2), k.size(0)};
         return bytes(w);
@@ -179,7 +182,7 @@ PyObject* paged_level(PyObject*, PyObject* const* a, Py_ssize_t n) {
 
 PyObject* empties_like(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
-        if (n != 1) throw Bad();
+        if (n != 1) throw Bad{kCountWanted};
         const Held in(PySequence_Fast(a[0], "a sequence of tensors is expected"));
         const Py_ssize_t size = PySequence_Fast_GET_SIZE(in.o);
         Held out(PyList_New(size));
@@ -196,10 +199,10 @@ PyObject* empties_like(PyObject*, PyObject* const* a, Py_ssize_t n) {
 
 PyObject* empty_f32(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
-        if (n != 3) throw Bad();
+        if (n != 3) throw Bad{kCountWanted};
         const at::Tensor& t = tensor(a[0]);
         const int64_t keep = integer(a[1]), extra = integer(a[2]);
-        if (keep < 0 || keep > t.dim()) throw Bad();
+        if (keep < 0 || keep > t.dim()) throw Bad{"as many dimensions as the tensor has, at most"};
         std::vector<int64_t> size(t.sizes().begin(), t.sizes().begin() + keep);
         if (extra) size.push_back(extra);
         return THPVariable_Wrap(at::empty(size, at::TensorOptions().device(t.device()).dtype(at::kFloat)));
@@ -226,7 +229,7 @@ template <> struct Arg<size_t> {
 };
 void* pointer(PyObject* o) {                         // an int, or None for null
     if (o == Py_None) return nullptr;
-    if (!PyLong_Check(o)) throw Bad();
+    if (!PyLong_Check(o)) throw Bad{"an address is expected: an int or None"};
     void* const v = PyLong_AsVoidPtr(o);
     if (!v && PyErr_Occurred()) throw PyErrSet();
     return v;
@@ -240,7 +243,7 @@ template <typename T> struct Arg<T*> {
             v = static_cast<T*>(tensor(o).data_ptr());
             return;
         }
-        if (!PyObject_HasAttrString(o, "data_ptr")) throw Bad();
+        if (!PyObject_HasAttrString(o, "data_ptr")) throw Bad{kTensorWanted};
         const Held at(PyObject_CallMethod(o, "data_ptr", nullptr));
         v = static_cast<T*>(pointer(at.o));
     }
@@ -259,7 +262,7 @@ struct Address {                                     // of a function, or a stre
 template <typename T> struct Levels {                // three levels as `levels`, `grads` or `paged_levels` returned them
     const T* v;
     explicit Levels(PyObject* o) : v(nullptr) {
-        if (!PyBytes_Check(o) || PyBytes_GET_SIZE(o) != static_cast<Py_ssize_t>(3 * sizeof(T))) throw Bad();
+        if (!PyBytes_Check(o) || PyBytes_GET_SIZE(o) != static_cast<Py_ssize_t>(3 * sizeof(T))) throw Bad{};
         v = reinterpret_cast<const T*>(PyBytes_AS_STRING(o));
     }
 };
@@ -303,7 +306,7 @@ template <> struct Arg<const mka_shape*> {
 template <typename R, typename... P, size_t... I>
 PyObject* invoke(R (*)(P...), PyObject* const* a, std::index_sequence<I...>) {
     const auto f = reinterpret_cast<R (*)(P...)>(Address(a[0]).v);
-    if (!f) throw Bad();
+    if (!f) throw Bad{"the address of a function is expected"};
     const std::tuple<std::conditional_t<I + 1 == sizeof...(P), Address, Arg<P>>...> args{a[1 + I]...};
     R status;
     Py_BEGIN_ALLOW_THREADS
@@ -314,7 +317,7 @@ PyObject* invoke(R (*)(P...), PyObject* const* a, std::index_sequence<I...>) {
 template <typename R, typename... P>
 PyObject* call(R (*declared)(P...), PyObject* const* a, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
-        if (n != static_cast<Py_ssize_t>(1 + sizeof...(P))) throw Bad();
+        if (n != static_cast<Py_ssize_t>(1 + sizeof...(P))) throw Bad{kCountWanted};
         return invoke(declared, a, std::index_sequence_for<P...>());
     });
 }
@@ -330,13 +333,13 @@ MKA_CALL(bwd)
 
 PyObject* empty_like(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
-        if (n != 1) throw Bad();
+        if (n != 1) throw Bad{kCountWanted};
         return THPVariable_Wrap(at::empty_like(tensor(a[0])));
     });
 }
 PyObject* row_counts(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
-        if (n != 1) throw Bad();
+        if (n != 1) throw Bad{kCountWanted};
         Seq K(a[0]);
         int64_t rows[3];
         for (int l = 0; l < 3; ++l) {

@@ -154,3 +154,18 @@ def test_only_a_shape_is_a_shape(name):
     for wrong in (bytes(shape), bytearray(shape), np.frombuffer(bytes(shape), dtype=np.uint8), (ctypes.c_int32 * 12).from_buffer_copy(shape)):
         with pytest.raises(TypeError):
             native[0](native[1], wrong, *rest)
+
+
+@pytest.mark.parametrize("args,message", [
+    ((1,), "number of arguments"),
+    ((None, "x", None, 0, 8, 1, 0, None, None, None, 0), "a tensor"),
+    ((None, None, None, 0, 8, 1, 0, None, True, None, 0), "a tensor"),
+    ((None, None, None, 0, 8, 1, 0, None, None, None, 1.0), "an address"),
+])
+def test_refusals_say_what_is_wrong(args, message):
+    with pytest.raises(AssertionError, match=message):
+        H.call_router(b._router, *args)
+    with pytest.raises(AssertionError, match="the address of a function"):
+        H.call_router(0, None, None, None, 0, 8, 1, 0, None, None, None, 0)
+    with pytest.raises(AssertionError, match="levels"):
+        H.call_decode(b._decode, _shape(T=1), None, b"", None, None, None, None, 0, 0)
