@@ -718,7 +718,7 @@ __global__ void __launch_bounds__(kTmaThreads, 2) decode_paged_tma_kernel(const 
                     for (int w = 0; w < 4; ++w)
 #pragma unroll
                         for (int j = 0; j < 2; ++j) v[j] = fmaf(at[(w * kState + nb * 4 + 2 * h + j) * 32], f[w], v[j]);
-                    *reinterpret_cast<float2*>(out + 2 + nb * 8 + 2 * t4) = make_float2(v[0], v[1]);
+                    out[2 + nb * 8 + 2 * t4] = v[0]; out[3 + nb * 8 + 2 * t4] = v[1];       // (4 bytes each: the workspace may lie at any multiple of 4)
                 }
             }
             break;

@@ -57,3 +57,32 @@ def test_matches_64_bits(mka, B, H, Hkv, d, n2):
         assert (LSE[b].double() - torch.logsumexp(x, 2).view(-1)).abs().max().item() <= 1e-5
         want = (torch.softmax(x, 2) @ v).view(H, d)
         assert (O[b].double() - want).abs().max().item() <= 2e-2 and (O[b].double() - want).abs().mean().item() <= 2e-3
+
+
+@pytest.mark.parametrize("paged,B,H,Hkv,d", [(True, 1, 8, 1, 128), (True, 3, 6, 2, 64), (True, 33, 4, 2, 64), (False, 2, 8, 2, 128), (False, 1, 28, 4, 64)])
+def test_workspace_at_any_multiple_of_four_bytes(mka, paged, B, H, Hkv, d):
+    """Partial results and the status word are written and read 4 bytes at a time: a slice of a caller's arena will do, and gives the same bits."""
+    g = torch.Generator(device="cuda").manual_seed(B + d)
+    mk = lambda *n: torch.randn(*n, device="cuda", dtype=torch.bfloat16, generator=g)
+    N, page = (160, 2096, 48), 16
+    q, gate = mk(B, H, d), torch.softmax(torch.randn(B, 3, device="cuda", generator=g), -1)
+    if paged:
+        shape = mka.make_shape(B, H, 1, d)
+        pools = [[mk(B * n // page, Hkv, page, d) for n in N] for _ in range(2)]
+        tabs = [torch.arange(B * n // page, device="cuda", dtype=torch.int32).view(B, n // page) for n in N]
+        nbytes = mka.mka_decode_paged_workspace_bytes(shape, Hkv, N)
+        run = lambda ws: mka.mka_decode_paged(shape, Hkv, q, *pools, tabs, N, gate, ws=ws)
+    else:
+        shape = mka.make_shape(B, H, 1, d, kv_heads=Hkv)
+        K, V = ([mk(B, Hkv, n, d) for n in N] for _ in range(2))
+        nbytes = mka.mka_workspace_bytes(shape, N, mka.MKA_WS_DECODE)
+        run = lambda ws: mka.mka_decode(shape, q, K, V, gate, ws=ws)
+    arena = torch.full((nbytes + 16,), 0xff, dtype=torch.uint8, device="cuda")
+    want = run(arena[:nbytes])
+    for off in (4, 8, 12):
+        arena.fill_(0xff)
+        ws = arena[off:off + nbytes]
+        O, LSE = run(ws)
+        assert mka.mka_device_status(ws) == 0
+        assert torch.equal(O, want[0]) and torch.equal(LSE, want[1])
+        assert bool((arena[:off] == 0xff).all()) and bool((arena[off + nbytes:] == 0xff).all())
