@@ -721,11 +721,14 @@ __global__ void __launch_bounds__(Cfg<DH>::kThreads, Cfg<DH>::kCtasPerSm) fwd_tc
                 float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
                 for (int c = 0; c < kTileN; c += 8) {
-                    mx4[0] = max3(mx4[0], s[c], s[c + 1]); mx4[1] = max3(mx4[1], s[c + 2], s[c + 3]);
-                    mx4[2] = max3(mx4[2], s[c + 4], s[c + 5]); mx4[3] = max3(mx4[3], s[c + 6], s[c + 7]);
+                    mx4[0] = max3_nan(mx4[0], s[c], s[c + 1]); mx4[1] = max3_nan(mx4[1], s[c + 2], s[c + 3]);
+                    mx4[2] = max3_nan(mx4[2], s[c + 4], s[c + 5]); mx4[3] = max3_nan(mx4[3], s[c + 6], s[c + 7]);
                 }
-                const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-                const float x_max = fmaf(mx, p.scale_log2, bias);            // -inf when the whole row is masked
+                const float mx = max3_nan(max3_nan(mx4[0], mx4[1], mx4[2]), mx4[3], mx4[3]);
+                const float x_row = fmaf(mx, p.scale_log2, bias);            // -inf when the whole row is masked
+                // A score of NaN is taken for +inf: from here on the row's weights are 0 or NaN in every column, whatever forms them, its sum is
+                // not above 0, and the row ends as O = 0 with LSE = -inf, as one with a score of +inf does.
+                const float x_max = x_row == x_row ? x_row : INFINITY;
                 const float m_new = fmaxf(m_run, x_max);
                 const bool grow = m_new > m_run + kRescaleThreshold;         // also true for the first finite max
                 const float m_use = grow ? m_new : m_run;

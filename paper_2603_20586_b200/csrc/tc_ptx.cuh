@@ -197,7 +197,8 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
 // 2^x for two arguments on the FMA pipe, as good as ex2 (largest relative error 1.7e-7, that of ex2.approx is 2^-22): x is clamped to -127 and split
 // into n = round(x) and f = x - n in [-1/2, 1/2] by adding and subtracting 1.5 * 2^23 (the sum's low mantissa bits are n); 2^f is a
 // polynomial of degree 5 with constant term exactly 1, fitted for the smallest maximum relative error (9.1e-8); n is added to the
-// exponent field.  x <= -127 gives exactly 0, as ex2 does for -inf; x < 128.
+// exponent field.  x <= -127 gives exactly 0, as ex2 does for -inf; x < 128.  NaN gives 0 too: a caller whose arguments may be NaN has to
+// see that by itself (fwd_tc_kernel's row maximum does).
 __device__ __forceinline__ void exp2_pair_poly(float x0, float x1, float& p0, float& p1) {
     const float kMagic = 12582912.f;
     const uint64_t x = pack2(fmaxf(x0, -127.f), fmaxf(x1, -127.f));
@@ -215,9 +216,10 @@ __device__ __forceinline__ void exp2_pair_poly(float x0, float x1, float& p0, fl
     p0 = __uint_as_float(__float_as_uint(r0) + (__float_as_uint(t0) << 23));
     p1 = __uint_as_float(__float_as_uint(r1) + (__float_as_uint(t1) << 23));
 }
-__device__ __forceinline__ float max3(float a, float b, float c) {
+// The largest of three; NaN if one of them is.
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
     float d;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
     return d;
 }
 // Value at shared-memory address `addr` (of this CTA's layout) in CTA `rank` of the cluster.
