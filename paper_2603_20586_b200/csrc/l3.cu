@@ -33,10 +33,10 @@ struct L3IndexParams {
     int H_kv, page_rows, d, bits;
 };
 
-constexpr __host__ __device__ int idx_pitch(int d) { return d + 4; }
-
 // Dynamic shared memory: projT [d][bits + 4] floats (16 consecutive bits of one column are four broadcast reads), then two
-// buffers s [kIdxPairs][d + 4] floats (the key sums; with that pitch the 16-byte reads of eight lanes fall on different banks).
+// buffers s [kIdxPairs][d] floats (the key sums; four columns of row r lie at place c ^ (r & 7) of it instead of c, so that the 16-byte reads of
+// eight lanes fall on different banks).  Rows padded to d + 4 floats did the same with 1.5 KB more, which at 256 bits and d = 128 took the SM's
+// shared memory past 196 KB, and with 228 set aside the L1 cache has half of the room for loads in flight: [30517 pages, 1 head, 64 rows, 128] 124 -> 158 us.
 // A batch = 64 (page, head) pairs.  The first LOADERS threads load: 16 of them cover one 256-byte row, a thread sums its eight
 // columns row by row, with up to 24 (512 loaders: 16) loads in flight across items and batches.  Four more warps project: lane = two pairs,
 // warp = 16 bits; four columns cost two 16-byte reads of s, 16 broadcast reads of projT and 128 fmaf.  The two sides work on different batches,
@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(LOADERS + kIdxThreads, LOADERS == 128 ? 2 : 1)
     chain_enter();
     extern __shared__ __align__(16) float sm[];
     const int ppitch = p.bits + 4;                             // floats between columns of projT (keeps the fill off one bank)
-    constexpr int pitch = idx_pitch(DH), kSumFloats = kIdxPairs * pitch;
+    constexpr int pitch = DH, kSumFloats = kIdxPairs * pitch;
     float* projT = sm;
     float* sums = sm + (size_t)DH * ppitch;
     const bool loads = threadIdx.x < LOADERS;
@@ -142,9 +142,10 @@ __global__ void __launch_bounds__(LOADERS + kIdxThreads, LOADERS == 128 ? 2 : 1)
                 row += 8;
                 if (row >= p.page_rows) {
                     if (item == 0 && n >= 2) wait(3 + (n & 1));            // the batch before last has been projected
-                    float* s = sums + (n & 1) * kSumFloats + (slot0 + item * kSlotStep) * pitch + piece * 8;
-                    *reinterpret_cast<ulonglong2*>(s) = make_ulonglong2(acc[0], acc[1]);
-                    *reinterpret_cast<ulonglong2*>(s + 4) = make_ulonglong2(acc[2], acc[3]);
+                    const int slot = slot0 + item * kSlotStep, swap = (slot & 7) * 4;
+                    float* s = sums + (n & 1) * kSumFloats + slot * pitch;
+                    *reinterpret_cast<ulonglong2*>(s + ((piece * 8) ^ swap)) = make_ulonglong2(acc[0], acc[1]);
+                    *reinterpret_cast<ulonglong2*>(s + ((piece * 8 + 4) ^ swap)) = make_ulonglong2(acc[2], acc[3]);
 #pragma unroll
                     for (int i = 0; i < 4; ++i) acc[i] = 0ull;
                     row = 0;
@@ -163,6 +164,7 @@ __global__ void __launch_bounds__(LOADERS + kIdxThreads, LOADERS == 128 ? 2 : 1)
             // ---- projections: one fmaf chain per (pair, bit) over the columns 0..d-1
             wait(1 + (n & 1));
             const float* sv = sums + (n & 1) * kSumFloats + lane * pitch;
+            const int swap = (lane & 7) * 4;                               // (of row lane + 32 too)
             for (int j0 = warp * kIdxBitsPerWarp; j0 < p.bits; j0 += (kIdxThreads / 32) * kIdxBitsPerWarp) {
                 // two chains per instruction (fma.rn.f32x2: each half is the same correctly rounded fma as fmaf)
                 unsigned long long a2[2][kIdxBitsPerWarp / 2];
@@ -177,7 +179,7 @@ __global__ void __launch_bounds__(LOADERS + kIdxThreads, LOADERS == 128 ? 2 : 1)
                 // 256 bits [20000, 2, 8, 128] 93.0 / 89.3 / 85.4 / 81.9.
 #pragma unroll 8
                 for (int i4 = 0; i4 < DH; i4 += 4) {
-                    const float4 xa4 = *reinterpret_cast<const float4*>(sv + i4), xb4 = *reinterpret_cast<const float4*>(sv + 32 * pitch + i4);
+                    const float4 xa4 = *reinterpret_cast<const float4*>(sv + (i4 ^ swap)), xb4 = *reinterpret_cast<const float4*>(sv + 32 * pitch + (i4 ^ swap));
                     const float xa[4] = {xa4.x, xa4.y, xa4.z, xa4.w}, xb[4] = {xb4.x, xb4.y, xb4.z, xb4.w};
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
@@ -611,7 +613,7 @@ cudaError_t launch_l3_index(const void* k, long long n_pages, int H_kv, int page
     // persistent CTAs: every CTA transposes the projection into shared memory once and then walks its batches
     // (the grid is shrunk so that all CTAs get the same number of batches)
     auto launch = [&](auto kern, int batch, int buffers, int threads, auto ctas_per_sm) {
-        const size_t smem = ((size_t)d * (bits + 4) + (size_t)buffers * batch * (buffers == 2 ? idx_pitch(d) : d + 1)) * sizeof(float);
+        const size_t smem = ((size_t)d * (bits + 4) + (size_t)buffers * batch * (buffers == 2 ? d : d + 1)) * sizeof(float);
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         const long long batches = (n_pages * H_kv + batch - 1) / batch, resident = 148LL * ctas_per_sm(smem);
