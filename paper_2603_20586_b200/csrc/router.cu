@@ -437,13 +437,11 @@ cudaError_t router_t(const T* R, const float* W_r, const float* b_r, long long r
         return launch_chained(router_any_kernel<T>, dim3((unsigned)((rows + rows_per_cta - 1) / rows_per_cta)), dim3(kWarps * 32), 0, st, 0,
                               R, W_r, b_r, rows, D, route, gate, log2_gate, idx);
     }
-    // Up to two rows per SM: one row to a CTA, for the shortest chain; to four per SM: two; above: four (777 rows of 1024: 2.56 us, 2.9 with two;
-    // 1000 rows of 4096: 4.5 against 4.7; 512 rows of 3584: two 3.84, four 5.0; 2000 rows of 2048: four 4.1, eight 4.6; 4700 of 4096: 10.8, 12.9).
-    // With many rows the warps have enough to do on their own, a row each: the sooner the shorter the rows (a CTA's time against the
-    // warps': 4800 rows of 768 4.10 us, 4.95, 9400 of 256 4.4, 3.7 and of 768 6.4, 6.0; 8192 of 1024 6.7, 7.5, 9400 of 1536 10.4, 10.1; 5000 of 4096 12.4, 20.7,
-    // 16384 of 1024 10.8, 9.0, 32768 of 2048 36, 28; loads ahead of the sums and W_r in shared memory were slower too, 35 and 44 us).
+    // With many rows the warps have enough to do on their own, a row each, the sooner the shorter the rows are (us, a CTA's columns against the warps':
+    // 9400 x 256 4.4, 3.7 and x 768 6.4, 6.0; 8192 x 1024 6.7, 7.5, 9400 x 1536 10.4, 10.1; 5000 x 4096 12.4, 20.7, 32768 x 2048 36, 28; loads ahead
+    // of the sums and W_r in shared memory were slower too, 35 and 44).
     const int warps_from = D >= 2048 ? 64 : (D >= 1024 ? 56 : (D >= 768 ? 40 : 32));   // rows per SM
-    if (rows >= warps_from * 148) {
+    if (rows >= warps_from * 148LL) {
         const long long rows_per_cta = kWarps * kRowsPerWarp;
         return launch_chained(router_rows_kernel<T>, dim3((unsigned)((rows + rows_per_cta - 1) / rows_per_cta)), dim3(kWarps * 32), 0, st, 0,
                               R, W_r, b_r, rows, D, route, gate, log2_gate, idx);
@@ -453,10 +451,34 @@ cudaError_t router_t(const T* R, const float* W_r, const float* b_r, long long r
         return launch_chained(kern, dim3((unsigned)((rows + per_cta - 1) / per_cta)), dim3(threads), 0, st, 0, R, W_r, b_r, rows, D, route, gate,
                               log2_gate, idx);
     };
-    if (rows >= 8 * 148) return go(router_kernel<T, 4, 8, 256>, 4, 8, 256);
-    if (rows >= 4 * 148) return go(router_kernel<T, 4, 4, 512>, 4, 4, 512);
-    if (rows >= 2 * 148) return go(router_kernel<T, 2, 4, 512>, 2, 4, 512);
-    return go(router_kernel<T, 1, 4, 512>, 1, 4, 512);
+    // Below that D is spread over a CTA.  Few rows: one row to a CTA, then two, for the shortest chain, and four once their CTAs are enough (at 1024
+    // to 2048 columns from five quarters of a row per SM on: 400 x 1536 bf16, two rows 2.72, four 2.36).  Then a launch lasts as long as its rounds of
+    // resident CTAs, so the form with fewer rounds is taken.  A CTA has a warp to 128 columns (four a thread, 16 at most) or to 256 (eight, 8 at most), and the
+    // registers let an SM hold 36 warps (fp32 32) of four rows by four columns, 32 of four by eight, 16 of eight by eight.  us, fp32 but where it says bf16:
+    //             4x4 / 4x8 / 8x8, chosen in brackets                   4x4 / 4x8 / 8x8
+    //   1500 x 1024 bf16   [2.86] / 3.05 / 3.24       2500 x 512        [2.81] / 3.70 / 3.39
+    //   1500 x 1536          4.38 / 3.90 / [3.66]     3000 x 1024         4.32 / 4.24 / [3.90]
+    //   2500 x 1536          5.96 / [4.09] / 5.79     2500 x 4096       [8.42] / 10.3 / 10.2
+    //   2000 x 1536 bf16     4.41 / 3.48 / [3.21]     2000 x 4096 bf16    6.39 / [4.93] / 4.93
+    //   5000 x 512 bf16      3.21 / 3.82 / 3.51 (warps [4.13])          8192 x 3584   29.0 / [24.2] / 27.9
+    // Over 16 widths from 128 to 8192, 36 row counts up to 32,768 and both types the pick takes 2.6 % more than the best form on average, and what was there before
+    // four columns a thread (one, two or eight rows by eight columns, warps from 32 rows per SM on) is faster by more than 4 % at 6 of 1152 sizes, by 7 % at most (2500 x 8192 bf16, 11.3 against 12.1).
+    const bool fp32 = sizeof(T) == 4, mid = D >= 1024 && D <= 2048;
+    const int warps4 = D >= 16 * 128 ? 16 : (D + 127) / 128, warps8 = D >= 8 * 256 ? 8 : (D + 255) / 256;
+    auto rounds = [&](int per_cta, int cta_warps, int sm_warps) {
+        const long long per_round = 148LL * per_cta * (sm_warps / cta_warps);
+        return (rows + per_round - 1) / per_round;
+    };
+    const long long n44 = rounds(4, warps4, fp32 ? 32 : 36), n48 = rounds(4, warps8, 32), n88 = rounds(8, warps8, 16);
+    if (rows < 2 * 148 && !(mid && rows > 148 * 5 / 4)) return go(router_kernel<T, 1, 4, 512>, 1, 4, 512);
+    if (rows < (D >= 512 && D < 1024 ? 3 : 4) * 148 && !mid) return go(router_kernel<T, 2, 4, 512>, 2, 4, 512);
+    // (short rows: four columns leave a CTA with two warps or less; long fp32 rows: three rounds of half the rows are shorter than two)
+    const bool halves = fp32 && D > 2048 && n44 == 3 && (n48 < n88 ? n48 : n88) == 2;
+    if ((n44 == 1 && (D > 256 || rows < 8 * 148)) || halves) return go(router_kernel<T, 4, 4, 512>, 4, 4, 512);
+    // (a tie: eight rows read W_r half as often, four put more loads of R in flight)
+    const bool tie8 = D <= 1024 || (n88 < 3 && (D < 2048 || (D == 2048 && n88 == 2) || (fp32 && (D <= 4096 || n88 == 1))));
+    if (D > 256 && (n88 < n48 || (n88 == n48 && tie8))) return go(router_kernel<T, 8, 8, 256>, 8, 8, 256);
+    return go(router_kernel<T, 4, 8, 256>, 4, 8, 256);
 }
 }  // namespace
 

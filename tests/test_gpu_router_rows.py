@@ -5,6 +5,15 @@ import torch
 pytestmark = pytest.mark.gpu
 
 
+# edges of the rounds of resident CTAs (bf16 / fp32): four rows by four columns end their first at 2368 of 1024 columns (both), 1776 / 1184 of 1536, 1184 of 2056, fp32
+# rows of 2568 their third at 3552; eight rows in place of four by eight columns around them; 186 rows at 1024 to 2048 columns; short rows; a row to the last CTA
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("rows,D", [(185, 1032), (186, 1032), (186, 2048), (1183, 256), (1184, 256), (2368, 1024), (2369, 1024), (4097, 1000), (1776, 1536), (1777, 1536),
+                                    (1185, 2056), (2368, 2568), (2369, 2568), (3553, 2568), (1191, 4104), (2001, 5128), (4735, 2040)])
+def test_router_rounds(dtype, rows, D):
+    test_router_splits(dtype, rows, D)
+
+
 # two rows a CTA end at 591, four of 512 threads at 1183, four of 256 threads at 4735, 5919, 8287 or 9471 by the width; widths below, at and past one pass (2048 columns)
 # and such that the last pass has threads and whole warps without a column
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
