@@ -576,27 +576,31 @@ __global__ void __launch_bounds__(kRetThreads) l3_retrieve_kernel(const L3Retrie
 
 // Sixteen loading warps in a CTA that has its SM to itself, instead of eight in two CTAs: half of the warp cycles of the eight went
 // into the adds' latencies with their loads not yet asked for again (DRAM 53 % busy), and the two CTAs' copies of the projection take
-// the room of loads in flight.  The four projecting warps then serve twice the rows, so the form is for pools that come from
-// memory and for few code bits to a row.  Time of the better of the two other forms over its, 300 MB of keys, pages of 16 / 32 / 64 rows:
-//   d = 64    32 bits 1.04 / 1.09 / 1.02    64 bits 1.12 / 1.20 / 1.07    128 bits 0.88 / 1.26 / 1.18    256 bits 0.86 / 1.00 / 1.42
-//   d = 128           1.09 / 1.10 / 1.09            1.22 / 1.41 / 1.52             1.19 / 1.54 / 1.53             0.92 / 1.23 / 1.79
-//   pages of 8 rows 0.8 .. 0.9;  pools of 40 MB 0.7 .. 1.2, of 60 MB 0.91 .. 1.22, of 90 MB and more 1.02 .. 1.44 (32 bits: 0.8 .. 1.03)
-// [32769 pages, 4 heads, 16 rows, 128], 64 bits: 119.5 us with eight loading warps, 106 with sixteen (109.5 against 117.6 on another day with longer turns of the projecting warps).
+// the room of loads in flight.  The four projecting warps then serve twice the rows, so the form is for few code bits to a row, and for pools
+// that give its CTAs a batch of 64 pairs.  Time of the better of the two other forms over its, 4 KV heads, pages of 16 / 24 / 32 / 64 rows, 300 MB of keys:
+//   d = 64    32 bits 1.09 / 1.12 / 1.05 / 0.99    64 bits 1.16 / 1.23 / 1.11 / 1.05    128 bits 0.93 / 1.16 / 1.25 / 1.18    256 bits 0.91 / 1.01 / 0.99 / 1.27
+//   d = 128           1.15 / 1.10 / 1.07 / 0.99            1.25 / 1.37 / 1.33 / 1.30             1.31 / 1.65 / 1.63 / 1.36             0.96 / 1.12 / 1.34 / 1.74
+// and over those pages by size, in the L2 cache and not: 64 and 128 bits, 20 to 60 MB 0.99 .. 2.09, 90 and 150 MB 0.96 .. 2.2, 5 MB 0.83 .. 1.5; 256 bits,
+// 40 to 150 MB 0.95 .. 1.8, 20 MB 0.93 .. 1.7; 32 bits, 20 to 60 MB 0.84 .. 1.5, 90 and 150 MB 0.84 .. 1.13 (d = 64), 1.00 .. 1.5 (d = 128).
+// Pages of 8 rows from 90 MB on 0.86 .. 1.14.  Over 560 sizes of 5 to 500 MB, no pick is slower than with the line at 80 MB, where it lay before the projecting
+// warps took longer turns, and those between the lines are up to twice as fast ([1831 pages, 4 heads, 32 rows, 128], 64 bits: 23.8 -> 12.5 us).
+// [32769 pages, 4 heads, 16 rows, 128], 64 bits: 117 us with eight loading warps, 104 with sixteen.
 bool many_loaders(const L3IndexParams& p) {
-    return p.page_rows >= 16 && p.bits <= (p.d == 128 ? 8 : 4) * p.page_rows &&
-           (double)p.n_pages * p.H_kv * p.page_rows * p.d * 2.0 >= (p.bits == 32 ? 200e6 : 80e6);
+    if (p.page_rows < 16 || p.bits > (p.d == 128 ? 11 : (p.page_rows >= 24 ? 8 : 4)) * p.page_rows) return false;
+    const double from = p.bits == 32 ? (p.d == 128 ? 80e6 : 200e6) : (p.bits == 256 ? 30e6 : 15e6);
+    return (double)p.n_pages * p.H_kv * p.page_rows * p.d * 2.0 >= from;
 }
 
-// Which form of the index kernel.  The one with projecting warps of its own wins where projections are a good part of the work and
+// Which of the two others.  The one with projecting warps of its own wins where projections are a good part of the work and
 // there are batches enough for all SMs; where a key row carries few code bits (its projecting half idles; at 32 bits two of those four
 // warps never have work, at 128 bits and d = 128 one CTA fits an SM) and for small pools the two-phase form does.  Time of the
-// first over that of the second, [5 .. 500 MB of keys], 4 KV heads:
-//   d = 64    32 bits, pages of 1 to 128 rows    1.04 .. 1.9            d = 128    32 bits    1.03 .. 1.9
-//             64 bits, 8 / 16 rows               0.75 / 0.96 (large)               64 bits, 8 / 16 rows     0.71 / 0.81 (large)
-//             64 bits, 24 / 32 / 64 rows         1.09 / 1.19 / 1.34                64 bits, 24 / 32 / 64    0.92 .. 1.10 / 0.97 .. 1.14 / 1.01 .. 1.25
-//             128 bits, 24 / 32 / 64 rows        0.88 / 0.98 .. 1.13 / 1.20        128 bits, 16 / 32 / 64   0.84 / 1.16 / 1.49
-//             256 bits, 16 / 64 rows             0.63 / 0.79                       256 bits, 16 / 64        0.57 / 0.97
-//   pools of at most 74 batches of 64 pairs, at any width (138 sizes): 0.95 .. 1.9
+// first over that of the second, 20 to 500 MB of keys, 4 KV heads (the lines matter below and beside those of many_loaders only):
+//   d = 64    32 bits, pages of 8 to 64 rows     1.04 .. 1.7            d = 128   32 bits    1.03 .. 1.6
+//             64 bits, 8 / 16 rows               0.74 .. 0.97                     64 bits, 8 / 16 rows     0.68 .. 0.96
+//             64 bits, 24 / 32 / 64 rows         0.93 .. 1.12 / 1.02 .. 1.23 / 1.15 .. 1.49                0.88 .. 0.92 / 0.93 .. 1.02 / 0.99 .. 1.21
+//             128 bits, 24 / 32 / 64 rows        0.82 .. 0.89 / 0.90 .. 0.99 / 1.03 .. 1.26                0.84 .. 1.04 / 0.97 .. 1.18 / 1.39 .. 1.54
+//             256 bits, 16 / 64 rows             0.45 .. 0.84 / 0.65 .. 1.08                               0.52 .. 0.85 / 0.88 .. 0.96
+//   pools of at most 74 batches of 64 pairs      0.97 .. 1.87                                              0.89 .. 1.58
 bool two_phases(const L3IndexParams& p) {
     if (p.bits == 32 || p.n_pages * p.H_kv <= 74 * kIdxPairs) return true;
     return (p.bits == 64 && p.page_rows >= 24) || (p.bits == 128 && p.page_rows >= 32);

@@ -29,8 +29,25 @@ def test_codes_of_a_large_pool_are_those_of_its_slices(mka, orc, pages, H_kv, ro
     if strided: pool = pool.permute(0, 2, 1, 3)
     proj = torch.randn(bits, d, generator=g, device="cuda")
     codes = mka.mka_l3_index(pool, proj)
-    parts = [mka.mka_l3_index(p, proj) for p in pool.split(max(1, int(30e6) // (H_kv * rows * d * 2)))]
+    parts = [mka.mka_l3_index(p, proj) for p in pool.split(max(1, int(10e6) // (H_kv * rows * d * 2)))]
     assert torch.equal(codes, torch.cat(parts))
+    for end in (slice(0, 3), slice(pages - 3, pages)):
+        want = orc.l3_index(pool[end].float().cpu().numpy(), proj.cpu().numpy())
+        assert np.array_equal(codes[end].cpu().numpy().view(np.uint32), want)
+
+
+# (pages, KV heads, rows of a page, d, bits): just past the lines from which that form is taken, 15 and 30 MB, with the widest codes for their pages
+MIDDLE = [(7325, 1, 16, 64, 64), (1221, 4, 24, 64, 128), (1954, 3, 20, 64, 64), (917, 4, 16, 128, 128), (1222, 4, 24, 128, 256), (1833, 4, 32, 64, 256)]
+
+
+@pytest.mark.parametrize("pages,H_kv,rows,d,bits", MIDDLE, ids=lambda v: str(v))
+def test_codes_of_a_middle_pool_are_those_of_its_slices(mka, orc, pages, H_kv, rows, d, bits):
+    assert (30e6 if bits == 256 else 15e6) <= pages * H_kv * rows * d * 2 <= 32e6
+    g = torch.Generator(device="cuda").manual_seed(pages + bits)
+    pool = torch.randn(pages, H_kv, rows, d, generator=g, device="cuda", dtype=torch.bfloat16)
+    proj = torch.randn(bits, d, generator=g, device="cuda")
+    codes = mka.mka_l3_index(pool, proj)
+    assert torch.equal(codes, torch.cat([mka.mka_l3_index(p, proj) for p in pool.split(max(1, int(10e6) // (H_kv * rows * d * 2)))]))
     for end in (slice(0, 3), slice(pages - 3, pages)):
         want = orc.l3_index(pool[end].float().cpu().numpy(), proj.cpu().numpy())
         assert np.array_equal(codes[end].cpu().numpy().view(np.uint32), want)
