@@ -33,10 +33,14 @@ struct L3IndexParams {
     int H_kv, page_rows, d, bits;
 };
 
+constexpr __host__ __device__ bool idx_swaps(int d, int loaders) { return d == 128 && loaders == 512; }
+constexpr __host__ __device__ int idx_pitch(int d, int loaders) { return idx_swaps(d, loaders) ? d : d + 4; }
+
 // Dynamic shared memory: projT [d][bits + 4] floats (16 consecutive bits of one column are four broadcast reads), then two
-// buffers s [kIdxPairs][d] floats (the key sums; four columns of row r lie at place c ^ (r & 7) of it instead of c, so that the 16-byte reads of
-// eight lanes fall on different banks).  Rows padded to d + 4 floats did the same with 1.5 KB more, which at 256 bits and d = 128 took the SM's
-// shared memory past 196 KB, and with 228 set aside the L1 cache has half of the room for loads in flight: [30517 pages, 1 head, 64 rows, 128] 124 -> 158 us.
+// buffers s [kIdxPairs][idx_pitch] floats (the key sums).  With rows of d + 4 floats the 16-byte reads of eight lanes fall on different
+// banks; with sixteen loading warps at d = 128 four columns of row r lie at place c ^ (r & 7) instead of c (idx_swaps): padded there too, 256 bits would take
+// the SM's shared memory past 196 KB, and with 228 set aside the L1 cache has half of the room for loads in flight ([7629 pages, 4 heads, 64 rows, 128]
+// 124 -> 158 us).  In the other forms the exchange costs more than it gives (1.00 to 1.05 of the time).
 // A batch = 64 (page, head) pairs.  The first LOADERS threads load: 16 of them cover one 256-byte row, a thread sums its eight
 // columns row by row, with up to 24 (512 loaders: 16) loads in flight across items and batches.  Four more warps project: lane = two pairs,
 // warp = 16 bits; four columns cost two 16-byte reads of s, 16 broadcast reads of projT and 128 fmaf.  The two sides work on different batches,
@@ -49,7 +53,8 @@ __global__ void __launch_bounds__(LOADERS + kIdxThreads, LOADERS == 128 ? 2 : 1)
     chain_enter();
     extern __shared__ __align__(16) float sm[];
     const int ppitch = p.bits + 4;                             // floats between columns of projT (keeps the fill off one bank)
-    constexpr int pitch = DH, kSumFloats = kIdxPairs * pitch;
+    constexpr int pitch = idx_pitch(DH, LOADERS), kSumFloats = kIdxPairs * pitch;
+    constexpr int kSwap = idx_swaps(DH, LOADERS) ? 7 : 0;                    // lowest bits of a row's number that exchange its columns
     float* projT = sm;
     float* sums = sm + (size_t)DH * ppitch;
     const bool loads = threadIdx.x < LOADERS;
@@ -142,7 +147,7 @@ __global__ void __launch_bounds__(LOADERS + kIdxThreads, LOADERS == 128 ? 2 : 1)
                 row += 8;
                 if (row >= p.page_rows) {
                     if (item == 0 && n >= 2) wait(3 + (n & 1));            // the batch before last has been projected
-                    const int slot = slot0 + item * kSlotStep, swap = (slot & 7) * 4;
+                    const int slot = slot0 + item * kSlotStep, swap = (slot & kSwap) * 4;
                     float* s = sums + (n & 1) * kSumFloats + slot * pitch;
                     *reinterpret_cast<ulonglong2*>(s + ((piece * 8) ^ swap)) = make_ulonglong2(acc[0], acc[1]);
                     *reinterpret_cast<ulonglong2*>(s + ((piece * 8 + 4) ^ swap)) = make_ulonglong2(acc[2], acc[3]);
@@ -164,7 +169,7 @@ __global__ void __launch_bounds__(LOADERS + kIdxThreads, LOADERS == 128 ? 2 : 1)
             // ---- projections: one fmaf chain per (pair, bit) over the columns 0..d-1
             wait(1 + (n & 1));
             const float* sv = sums + (n & 1) * kSumFloats + lane * pitch;
-            const int swap = (lane & 7) * 4;                               // (of row lane + 32 too)
+            const int swap = (lane & kSwap) * 4;                               // (of row lane + 32 too)
             for (int j0 = warp * kIdxBitsPerWarp; j0 < p.bits; j0 += (kIdxThreads / 32) * kIdxBitsPerWarp) {
                 // two chains per instruction (fma.rn.f32x2: each half is the same correctly rounded fma as fmaf)
                 unsigned long long a2[2][kIdxBitsPerWarp / 2];
@@ -587,7 +592,7 @@ __global__ void __launch_bounds__(kRetThreads) l3_retrieve_kernel(const L3Retrie
 // [32769 pages, 4 heads, 16 rows, 128], 64 bits: 117 us with eight loading warps, 104 with sixteen.
 bool many_loaders(const L3IndexParams& p) {
     if (p.page_rows < 16 || p.bits > (p.d == 128 ? 11 : (p.page_rows >= 24 ? 8 : 4)) * p.page_rows) return false;
-    const double from = p.bits == 32 ? (p.d == 128 ? 80e6 : 200e6) : (p.bits == 256 ? 30e6 : 15e6);
+    const double from = p.bits == 32 ? (p.d == 128 ? 80e6 : 200e6) : (p.d == 64 && p.page_rows < 24 ? 80e6 : (p.bits == 256 ? 30e6 : 15e6));
     return (double)p.n_pages * p.H_kv * p.page_rows * p.d * 2.0 >= from;
 }
 
@@ -617,7 +622,7 @@ cudaError_t launch_l3_index(const void* k, long long n_pages, int H_kv, int page
     // persistent CTAs: every CTA transposes the projection into shared memory once and then walks its batches
     // (the grid is shrunk so that all CTAs get the same number of batches)
     auto launch = [&](auto kern, int batch, int buffers, int threads, auto ctas_per_sm) {
-        const size_t smem = ((size_t)d * (bits + 4) + (size_t)buffers * batch * (buffers == 2 ? d : d + 1)) * sizeof(float);
+        const size_t smem = ((size_t)d * (bits + 4) + (size_t)buffers * batch * (buffers == 2 ? idx_pitch(d, threads - kIdxThreads) : d + 1)) * sizeof(float);
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         const long long batches = (n_pages * H_kv + batch - 1) / batch, resident = 148LL * ctas_per_sm(smem);

@@ -37,7 +37,7 @@ def test_codes_of_a_large_pool_are_those_of_its_slices(mka, orc, pages, H_kv, ro
 
 
 # (pages, KV heads, rows of a page, d, bits): just past the lines from which that form is taken, 15 and 30 MB, with the widest codes for their pages
-MIDDLE = [(7325, 1, 16, 64, 64), (1221, 4, 24, 64, 128), (1954, 3, 20, 64, 64), (917, 4, 16, 128, 128), (1222, 4, 24, 128, 256), (1833, 4, 32, 64, 256)]
+MIDDLE = [(1018, 1, 230, 64, 64), (1221, 4, 24, 64, 128), (1303, 3, 30, 64, 64), (917, 4, 16, 128, 128), (1222, 4, 24, 128, 256), (1833, 4, 32, 64, 256)]
 
 
 @pytest.mark.parametrize("pages,H_kv,rows,d,bits", MIDDLE, ids=lambda v: str(v))
