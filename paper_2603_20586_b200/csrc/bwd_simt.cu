@@ -390,7 +390,7 @@ cudaError_t launch_dkv(const BwdParams& p, int vec, cudaStream_t st) {
 template <typename T, int DH>
 cudaError_t launch_t(const BwdParams& p, cudaStream_t st) {
     const int vec = simt_vec_bits(p.L, p.Q, p.O, p.dO, sizeof(T) == 2 ? MKA_BF16 : MKA_F32);
-    const int groups = simt_query_groups(p, 50.0);
+    const int groups = simt_query_groups(p, 80.0);
     cudaError_t e;
     if constexpr (DH < 128) e = groups == 8 ? launch_dq<T, DH, 8>(p, vec, st) : (groups == 4 ? launch_dq<T, DH, 4>(p, vec, st) : launch_dq<T, DH, 1>(p, vec, st));
     else e = groups == 4 ? launch_dq<T, DH, 4>(p, vec, st) : launch_dq<T, DH, 1>(p, vec, st);

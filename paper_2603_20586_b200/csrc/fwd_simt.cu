@@ -217,7 +217,7 @@ cudaError_t launch_g(const FwdParams& p, cudaStream_t st) {
 
 template <typename T, int DH>
 cudaError_t launch_t(const FwdParams& p, cudaStream_t st) {
-    const int groups = simt_query_groups(p, DH <= 64 ? 28.0 : 40.0);
+    const int groups = simt_query_groups(p, 40.0);
     if constexpr (DH < 128) {                            // (eight groups' tiles of 128 columns do not fit shared memory)
         if (groups == 8) return p.mode == MKA_MODE_FULL ? launch_g<T, DH, MKA_MODE_FULL, 8>(p, st) : launch_g<T, DH, MKA_MODE_FAST, 8>(p, st);
     }

@@ -109,14 +109,14 @@ inline int simt_vec_bits(const LevelDev L[3], const void* a, const void* b, cons
 
 // Which shape.  Four groups shorten the walk of a CTA and leave fewer CTAs on an SM at a time: they are for launches whose blocks
 // do not fill the chip, and for long walks; one group has the better throughput.  `blocks`: CTAs of 16 rows;
-// `walk`: tiles that a row block visits, on average; `k`, tiles for a block more than one per SM: 28 in the forward (40 above
-// d = 64, where an SM holds one CTA of four groups), 50 for dQ and 120 (of the longest walk) for dK/dV, where four groups hold
-// out longer.  Over 200 shapes of d = 32 to 128 the rule costs 1 % on average against the better shape.  fp32, us, four groups /
-// one group (in brackets one group with scalar loads, the only shape there once was):
-//   forward, d = 64    8 heads x 200 rows, 104 blocks, 17 tiles   29.8 / 57.4 (84.1)      24 x 200, 312, 10    39.0 / 50.1 (63.6)
-//                      24 x 512, 768, 13                          121 / 116 (135)         8 x 3000, 1504, 53   735 / 726 (874)
-//                      128 x 64, 512, 14                          86.1 / 63.5 (82.2)      8 x 1024, 512, 2     22.6 / 14.4 (18.5)
-//   forward, d = 128   32 x 200, 416, 8                           43.1 / 51.2
+// `walk`: tiles that a row block visits, on average; `k`, tiles for a block more than one per SM: 40 in the forward,
+// 80 for dQ and 120 (of the longest walk) for dK/dV, where four groups hold out longer.  Over 167 shapes of d = 32 to 128, timed with a tile's loads all in
+// flight, the rule costs 1.6 % on average against the best shape in the forward at d = 32 and 64 (0.2 % above), 0.8 % (0.1) in the backward with dQ's,
+// 0.2 % with dK/dV's; the most where a second round is nearly empty (the last of these).  fp32, us, four groups / one group:
+//   forward, d = 64    [1, 8, 200], window 200, 300 slots, 104 blocks    29.1 / 63.4 (eight 31.9)    [3, 8, 200], 100 slots, 312    47.5 / 68.7
+//                      [3, 8, 512], 100 slots, 768                       140 / 155                   [1, 8, 3000], 100 slots, 1504  718 / 777
+//                      [1, 8, 1024], window 16, 32 slots, 512            108 / 132                   [8, 16, 64], 400 slots, 512    83.8 / 70.8
+//   forward, d = 128   [4, 8, 200], window 100, 100 slots, 416           87.5 / 103
 inline bool simt_four_groups(long long blocks, double walk, double k) { return blocks <= 148 || (double)(blocks - 148) <= k * walk; }
 template <typename P> inline double simt_query_walk(const P& p) {                     // forward and dQ: row blocks of queries
     double keys = 0.0;
@@ -129,11 +129,12 @@ template <typename P> inline double simt_query_walk(const P& p) {               
 template <typename P> inline int simt_query_groups(const P& p, double k) {
     const long long blocks = (long long)p.B * p.H * ((p.T + 15) / 16);
     const double walk = simt_query_walk(p);
-    // Half as many rows to a CTA where even twice the blocks find an SM each and every group still has a tile: an SM's shared-memory
+    // Half as many rows to a CTA where even twice the blocks find an SM each: an SM's shared-memory
     // reads, which bound a step of the walk, are the same, but a step covers eight tiles.  [1, 4, 256, 64] (window 64, 128 slots): both
     // forwards and the backward together 106 us in four groups, 94 in eight and with the longest key blocks of dK/dV first (clusters of
-    // two to four CTAs of four groups instead: 118).
-    if (p.d < 128 && blocks * 2 <= 148 && walk >= 8.0) return 8;
+    // two to four CTAs of four groups instead: 118).  Walks of 5.5 to 8 tiles, four / eight: forward 9.1 / 7.4 (d = 32, 53 to 103 rows), 12.0 / 9.3 (d = 64,
+    // 49 to 84), 15.1 / 11.6 (d = 96, 94); before a tile's loads were in flight together they were equal there.
+    if (p.d < 128 && blocks * 2 <= 148 && walk >= 5.0) return 8;
     return simt_four_groups(blocks, walk, k) ? 4 : 1;
 }
 // dK/dV: the levels' key blocks walk very different numbers of query tiles, and a launch lasts at least as long as its longest walk

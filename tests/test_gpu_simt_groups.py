@@ -1,4 +1,4 @@
-"""CUDA-core kernels with eight rows to a CTA (few blocks, walks of eight tiles or more): rows around a block's eight, tiles around a
+"""CUDA-core kernels with eight rows to a CTA (few blocks, walks of five tiles or more): rows around a block's eight, tiles around a
 group's share, against the oracle."""
 import numpy as np
 import pytest
@@ -23,6 +23,7 @@ CASES = [
     (2, 2, 145, 96, 100, 33),
     (1, 3, 97, 64, 1, 257),
     (1, 2, 8, 96, 8, 255),
+    (1, 2, 72, 32, 9, 46), (3, 1, 62, 96, 7, 28), (2, 2, 49, 64, 16, 91),        # walks of 5.5 to 7.6 tiles: groups without any
 ]
 
 
