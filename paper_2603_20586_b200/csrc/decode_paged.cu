@@ -710,6 +710,9 @@ __global__ void __launch_bounds__(kTmaThreads, 2) decode_paged_tma_kernel(const 
                     if (slot == 0) head[0] = (float)n_slots;
                     out[0] = mx; out[1] = zs;
                 }
+                // (One address for the stores: at d = 64 six registers more would leave no room beside two of these CTAs for the combine's, which start under
+                // their tail: 224 heads of 6500 rows 17.5 -> 19.1 us.)
+                float* const to = out + 2 + warp * (NB / 4) * 8 + 2 * t4;
 #pragma unroll
                 for (int i = 0; i < NB / 4; ++i) {
                     const int nb = warp * (NB / 4) + i;
@@ -718,7 +721,7 @@ __global__ void __launch_bounds__(kTmaThreads, 2) decode_paged_tma_kernel(const 
                     for (int w = 0; w < 4; ++w)
 #pragma unroll
                         for (int j = 0; j < 2; ++j) v[j] = fmaf(at[(w * kState + nb * 4 + 2 * h + j) * 32], f[w], v[j]);
-                    out[2 + nb * 8 + 2 * t4] = v[0]; out[3 + nb * 8 + 2 * t4] = v[1];       // (4 bytes each: the workspace may lie at any multiple of 4)
+                    to[i * 8] = v[0]; to[i * 8 + 1] = v[1];                                   // (4 bytes each: the workspace may lie at any multiple of 4)
                 }
             }
             break;
