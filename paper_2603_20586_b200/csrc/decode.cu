@@ -404,13 +404,17 @@ __global__ void __launch_bounds__(DH * GROUPS) decode_combine_kernel(const Decod
     if (p.LSE && tid == 0) p.LSE[bh] = Z > 0.f ? (M + log2f(Z)) * kLn2 : -INFINITY;
 }
 
-// Four groups where a thread would have many chunks and the CTAs leave SMs idle; at d = 64, where a group is two warps, for more than it
-// asks for at once.  Router and decode, us, one group / four: 4 x 28 heads on 4 at 6500 rows, d = 128 (19 partials) 25.1 / [23.3]; at 10,500 rows,
-// d = 64 [18.2] / 18.9; 28 heads on 4 at 10,500 rows, d = 128 (56 partials) 20.8 with a third round trip, [16.8].
+// Four groups where a thread would have many chunks and the CTAs leave SMs idle; at d = 64, where a group is two warps, for well more than it
+// asks for at once.  Whole decode of grouped heads, four groups over one, lists of 1500 / 6500 / 20,000 rows, by the partials of a list of equal lengths:
+//   d = 128   3 to 8 partials (160 to 288 heads)  0.98 .. 0.99 / 0.95 .. 0.99 / 0.97 .. 0.99      10  0.98 .. 1.05 / 0.94 .. 0.97 / 0.97 .. 0.99
+//             19 and 25  0.99 .. 1.00 / 0.94 .. 0.95 / 0.95 .. 0.97      38 and 75  0.96 .. 0.99 / 0.87 .. 0.88 / 0.87 .. 0.92      297  1.05 / 0.86 / 0.63 .. 0.65
+//   d = 64    up to 25  1.02 .. 1.08 / 1.01 .. 1.07 / 1.00 .. 1.04      38  1.06 .. 1.09 / 1.01 / 1.02      75  1.04 / 0.90 / 0.90      297  0.99 .. 1.04 / 0.79 .. 0.85 / 0.70
+// (28 heads on 4 at 6500 rows, d = 128: 14.2 us, 12.4; a list of 1500 rows fills fewer partials than its share of the CTAs).  Chunks cut on the host: 34 and 40 of them 0.99 .. 1.00, 86 and
+// 89 0.96 .. 1.00, 157 0.81 .. 0.91, 235 and more 0.55 .. 0.75.
 template <int DH>
 cudaError_t launch_combine(const DecodeParams& p, cudaStream_t st) {
     const dim3 grid((unsigned)((long long)p.B * p.H));
-    if ((p.counted ? p.expected > (DH == 128 ? 8 : 32) : p.total_chunks > 32) && grid.x <= 296) return launch_chained(decode_combine_kernel<DH, 4>, grid, dim3(DH * 4), 0, st, 0, p);
+    if ((p.counted ? p.expected > (DH == 128 ? 2 : 48) : p.total_chunks > 32) && grid.x <= 296) return launch_chained(decode_combine_kernel<DH, 4>, grid, dim3(DH * 4), 0, st, 0, p);
     return launch_chained(decode_combine_kernel<DH, 1>, grid, dim3(DH), 0, st, 0, p);
 }
 

@@ -16,7 +16,8 @@ def mka():
 @pytest.mark.parametrize("B,H,Hkv,d,n2", [
     (1, 8, 1, 128, 19100),        # 299 tiles, two to a share: 150 partials of one list
     (1, 5, 1, 64, 64 * 296 * 2),  # even shares
-    (2, 8, 2, 64, 5000), (3, 16, 1, 128, 130), (31, 4, 2, 128, 700), (32, 8, 2, 64, 333), (33, 8, 2, 64, 333), (40, 4, 4, 128, 65)])
+    (2, 8, 2, 64, 5000), (3, 16, 1, 128, 130), (31, 4, 2, 128, 700), (32, 8, 2, 64, 333), (33, 8, 2, 64, 333), (40, 4, 4, 128, 65),
+    (8, 16, 8, 128, 700), (2, 8, 4, 64, 900), (1, 8, 4, 64, 900)])     # few partials in four groups (d = 128), 38 in one and 75 in four (d = 64)
 def test_matches_64_bits(mka, B, H, Hkv, d, n2):
     """O is a bf16 rounding (2^-9 of |O| <= 4) and weights rounded to bf16 for the product away from the exact value; LSE only fp32 sums."""
     g = torch.Generator(device="cuda").manual_seed(B * 100 + d)
