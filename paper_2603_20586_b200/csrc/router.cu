@@ -120,8 +120,8 @@ __device__ __forceinline__ void sum_rows(float (&acc)[ROWS * 3], int lane, int& 
 // one load's latency: a warp that walks four rows by itself took 11 us for ONE row of D = 4096.  With thousands of rows
 // the order turns round (see router_rows_kernel).  A thread's columns of W_r lie 12 COLS bytes from its neighbour's, so a 16-byte read by a warp
 // touches 24 lines at eight columns and 12 at four, and all of W_r (48 KB at D = 4096) goes through each CTA's L1: with four columns and
-// twice the threads one row of 4096 takes 2.30 us instead of 2.56, 512 rows of 3584 3.84 instead of 4.78.  From 8 rows per SM on it is the
-// rows' own loads that count, and they shrink to 8 bytes: eight columns and 256 threads there (2000 rows of 2048: 4.1 us against 5.9).
+// twice the threads one row of 4096 takes 2.30 us instead of 2.56, 512 rows of 3584 3.84 instead of 4.78.  Past one round
+// of CTAs it is the rows' own loads that count, and with four columns they shrink to 8 bytes: eight and 256 threads there (2000 rows of 2048: 4.1 us against 5.9).
 template <typename T, int ROWS, int COLS, int THREADS>
 __global__ void __launch_bounds__(THREADS)
 router_kernel(const T* __restrict__ R, const float* __restrict__ W_r, const float* __restrict__ b_r,

@@ -194,10 +194,11 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
-// 2^x for two arguments on the FMA pipe, as good as ex2 (largest relative error 1.7e-7, that of ex2.approx is 2^-22): x is clamped to -127 and split
-// into n = round(x) and f = x - n in [-1/2, 1/2] by adding and subtracting 1.5 * 2^23 (the sum's low mantissa bits are n); 2^f is a
-// polynomial of degree 5 with constant term exactly 1, fitted for the smallest maximum relative error (9.1e-8); n is added to the
-// exponent field.  x <= -127 gives exactly 0, as ex2 does for -inf; x < 128.  NaN gives 0 too: a caller whose arguments may be NaN has to
+// 2^x for two arguments on the FMA pipe, for -126 <= x < 128 as good as ex2 (largest relative error 1.7e-7, that of ex2.approx is 2^-22): range reduction by rounding
+// and a minimax polynomial.  x is clamped to -127 and split into n = round(x) and f = x - n in [-1/2, 1/2] by adding and subtracting
+// 1.5 * 2^23 (the sum's low mantissa bits are n); 2^f is a polynomial of degree 5 with constant term exactly 1, fitted for the smallest maximum
+// relative error (9.1e-8); n is added to the exponent field.  From -126 down to -127 that field is 0 and the result a subnormal number below the true one
+// (ex2 gives 0 there); x <= -127 gives exactly 0, as ex2 does for -inf.  NaN gives 0 too: a caller whose arguments may be NaN has to
 // see that by itself (fwd_tc_kernel's row maximum does).
 __device__ __forceinline__ void exp2_pair_poly(float x0, float x1, float& p0, float& p1) {
     const float kMagic = 12582912.f;
