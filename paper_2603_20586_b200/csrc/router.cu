@@ -451,33 +451,35 @@ cudaError_t router_t(const T* R, const float* W_r, const float* b_r, long long r
         return launch_chained(kern, dim3((unsigned)((rows + per_cta - 1) / per_cta)), dim3(threads), 0, st, 0, R, W_r, b_r, rows, D, route, gate,
                               log2_gate, idx);
     };
-    // Below that D is spread over a CTA.  Few rows: one row to a CTA, then two, for the shortest chain, and four once their CTAs are enough (at 1024
-    // to 2048 columns from five quarters of a row per SM on: 400 x 1536 bf16, two rows 2.72, four 2.36).  Then a launch lasts as long as its rounds of
-    // resident CTAs, so the form with fewer rounds is taken.  A CTA has a warp to 128 columns (four a thread, 16 at most) or to 256 (eight, 8 at most), and the
-    // registers let an SM hold 36 warps (fp32 32) of four rows by four columns, 32 of four by eight, 16 of eight by eight.  us, fp32 but where it says bf16:
-    //             4x4 / 4x8 / 8x8, chosen in brackets                   4x4 / 4x8 / 8x8
-    //   1500 x 1024 bf16   [2.86] / 3.05 / 3.24       2500 x 512        [2.81] / 3.70 / 3.39
-    //   1500 x 1536          4.38 / 3.90 / [3.66]     3000 x 1024         4.32 / 4.24 / [3.90]
-    //   2500 x 1536          5.96 / [4.09] / 5.79     2500 x 4096       [8.42] / 10.3 / 10.2
-    //   2000 x 1536 bf16     4.41 / 3.48 / [3.21]     2000 x 4096 bf16    6.39 / [4.93] / 4.93
-    //   5000 x 512 bf16      3.21 / 3.82 / 3.51 (warps [4.13])          8192 x 3584   29.0 / [24.2] / 27.9
-    // Over 16 widths from 128 to 8192, 36 row counts up to 32,768 and both types the pick takes 2.6 % more than the best form on average, and what was there before
-    // four columns a thread (one, two or eight rows by eight columns, warps from 32 rows per SM on) is faster by more than 4 % at 6 of 1152 sizes, by 7 % at most (2500 x 8192 bf16, 11.3 against 12.1).
-    const bool fp32 = sizeof(T) == 4, mid = D >= 1024 && D <= 2048;
+    // Below that D is spread over a CTA.  Few rows: one row to a CTA, then two, for the shortest chain, and four where their CTAs are enough (at 768 to
+    // 2048 columns from two rows per SM on: 400 x 2048 with a forward behind it 17.0 us, four 16.6).  Then a launch lasts as long as its rounds of
+    // resident CTAs: four columns a thread while all rows fit one, eight past it.  A CTA has a warp to 128 columns (four a thread, 16 at most) or to 256
+    // (eight, 8 at most), and the registers let an SM hold 36 warps (fp32 32) of four rows by four columns, 32 of four by eight, 16 of eight by eight.
+    // Routers one after the other, us, four by four / four by eight / eight by eight:
+    //   1500 x 1024 bf16   [2.86] / 3.05 / 3.24     2000 x 1536 bf16   4.41 / [3.48] / 3.21     2500 x 512 fp32    [2.81] / 3.70 / 3.39
+    //   2000 x 1024 bf16   [2.77] / 3.16 / 3.30     2000 x 4096 bf16   6.39 / [4.93] / 4.93     2500 x 4096 fp32   [8.42] / 10.3 / 10.2
+    //   1500 x 1536 fp32     4.38 / 3.90 / [3.66]   3000 x 1024 fp32   4.32 / 4.24 / [3.90]     8192 x 3584 fp32   29.0 / [24.2] / 27.9
+    // In bf16 a tensor-core forward follows, whose CTAs start beside the router's last ones if those leave them registers: eight rows by eight columns do not,
+    // and behind them the pass is as long or longer (2626 x 1536: 40.9 us with four rows, 42.7 with eight, 2626 x 1024 35.2 and 35.7, 2000 x 1536 34.4 and 34.3).
+    // Against one, two or eight rows by eight columns and warps from 32 rows per SM on, which was there before four columns a thread: 0.89 of the time over 16 widths from 128 to
+    // 8192, 36 row counts and both types, routers one after the other; 12 of the 1152 sizes are slower by more than 4 %, by 9 % at most (2000 x 1536 bf16), none with
+    // a forward behind it (50 sizes, 0.93).
+    const bool fp32 = sizeof(T) == 4, mid = D >= 768 && D <= 2048;
     const int warps4 = D >= 16 * 128 ? 16 : (D + 127) / 128, warps8 = D >= 8 * 256 ? 8 : (D + 255) / 256;
     auto rounds = [&](int per_cta, int cta_warps, int sm_warps) {
         const long long per_round = 148LL * per_cta * (sm_warps / cta_warps);
         return (rows + per_round - 1) / per_round;
     };
     const long long n44 = rounds(4, warps4, fp32 ? 32 : 36), n48 = rounds(4, warps8, 32), n88 = rounds(8, warps8, 16);
-    if (rows < 2 * 148 && !(mid && rows > 148 * 5 / 4)) return go(router_kernel<T, 1, 4, 512>, 1, 4, 512);
-    if (rows < (D >= 512 && D < 1024 ? 3 : 4) * 148 && !mid) return go(router_kernel<T, 2, 4, 512>, 2, 4, 512);
-    // (short rows: four columns leave a CTA with two warps or less; long fp32 rows: three rounds of half the rows are shorter than two)
+    if (rows < 2 * 148) return go(router_kernel<T, 1, 4, 512>, 1, 4, 512);
+    if (rows < 4 * 148 && !mid) return go(router_kernel<T, 2, 4, 512>, 2, 4, 512);
+    // (short rows leave a CTA with two warps or less; long fp32 rows: three rounds of half the rows are shorter than two)
     const bool halves = fp32 && D > 2048 && n44 == 3 && (n48 < n88 ? n48 : n88) == 2;
     if ((n44 == 1 && (D > 256 || rows < 8 * 148)) || halves) return go(router_kernel<T, 4, 4, 512>, 4, 4, 512);
-    // (a tie: eight rows read W_r half as often, four put more loads of R in flight)
-    const bool tie8 = D <= 1024 || (n88 < 3 && (D < 2048 || (D == 2048 && n88 == 2) || (fp32 && (D <= 4096 || n88 == 1))));
-    if (D > 256 && (n88 < n48 || (n88 == n48 && tie8))) return go(router_kernel<T, 8, 8, 256>, 8, 8, 256);
+    if constexpr (sizeof(T) == 4) {                            // (a tie: eight rows read W_r half as often, four put more loads of R in flight)
+        const bool tie8 = D <= 1024 || (n88 < 3 && (D <= 4096 || n88 == 1));
+        if (D > 256 && (n88 < n48 || (n88 == n48 && tie8))) return go(router_kernel<T, 8, 8, 256>, 8, 8, 256);
+    }
     return go(router_kernel<T, 4, 8, 256>, 4, 8, 256);
 }
 }  // namespace
