@@ -33,14 +33,13 @@ struct L3IndexParams {
     int H_kv, page_rows, d, bits;
 };
 
-constexpr __host__ __device__ bool idx_swaps(int d, int loaders) { return d == 128 && loaders == 512; }
-constexpr __host__ __device__ int idx_pitch(int d, int loaders) { return idx_swaps(d, loaders) ? d : d + 4; }
+constexpr __host__ __device__ int idx_pitch(int d, bool swaps) { return swaps ? d : d + 4; }
 
 // Dynamic shared memory: projT [d][bits + 4] floats (16 consecutive bits of one column are four broadcast reads), then two
 // buffers s [kIdxPairs][idx_pitch] floats (the key sums).  With rows of d + 4 floats the 16-byte reads of eight lanes fall on different
-// banks; with sixteen loading warps at d = 128 four columns of row r lie at place c ^ (r & 7) instead of c (idx_swaps): padded there too, 256 bits would take
-// the SM's shared memory past 196 KB, and with 228 set aside the L1 cache has half of the room for loads in flight ([7629 pages, 4 heads, 64 rows, 128]
-// 124 -> 158 us).  In the other forms the exchange costs more than it gives (1.00 to 1.05 of the time).
+// banks; SWAPS (256 bits, d = 128, sixteen loading warps): four columns of row r lie at place c ^ (r & 7) instead of c.  Padded there too, the SM's shared memory would go
+// past 196 KB, and with 228 set aside the L1 cache has half of the room for loads in flight ([7629 pages, 4 heads, 64 rows, 128] 124 -> 158 us).
+// Elsewhere the exchange costs more than it gives (1.00 to 1.05 of the time).
 // A batch = 64 (page, head) pairs.  The first LOADERS threads load: 16 of them cover one 256-byte row, a thread sums its eight
 // columns row by row, with up to 24 (512 loaders: 16) loads in flight across items and batches.  Four more warps project: lane = two pairs,
 // warp = 16 bits; four columns cost two 16-byte reads of s, 16 broadcast reads of projT and 128 fmaf.  The two sides work on different batches,
@@ -48,13 +47,13 @@ constexpr __host__ __device__ int idx_pitch(int d, int loaders) { return idx_swa
 // lane, the shared-memory pipe was busy for 78 us and HBM idle half of the time: 147 us (3.6 TB/s) for [32769 pages, 4 heads, 16
 // rows, 128] at 64 bits, 123 us with four loading warps in each of two CTAs (registers moved to them from the projecting ones);
 // sixteen in one CTA: see many_loaders.
-template <int DH, int LOADERS>
+template <int DH, int LOADERS, bool SWAPS = false>
 __global__ void __launch_bounds__(LOADERS + kIdxThreads, LOADERS == 128 ? 2 : 1) l3_index_kernel(const L3IndexParams p) {
     chain_enter();
     extern __shared__ __align__(16) float sm[];
     const int ppitch = p.bits + 4;                             // floats between columns of projT (keeps the fill off one bank)
-    constexpr int pitch = idx_pitch(DH, LOADERS), kSumFloats = kIdxPairs * pitch;
-    constexpr int kSwap = idx_swaps(DH, LOADERS) ? 7 : 0;                    // lowest bits of a row's number that exchange its columns
+    constexpr int pitch = idx_pitch(DH, SWAPS), kSumFloats = kIdxPairs * pitch;
+    constexpr int kSwap = SWAPS ? 7 : 0;                                      // lowest bits of a row's number that exchange its columns
     float* projT = sm;
     float* sums = sm + (size_t)DH * ppitch;
     const bool loads = threadIdx.x < LOADERS;
@@ -621,20 +620,23 @@ cudaError_t launch_l3_index(const void* k, long long n_pages, int H_kv, int page
     p.n_pages = n_pages; p.sp = sp; p.sh = sh; p.sn = sn; p.H_kv = H_kv; p.page_rows = page_rows; p.d = d; p.bits = bits;
     // persistent CTAs: every CTA transposes the projection into shared memory once and then walks its batches
     // (the grid is shrunk so that all CTAs get the same number of batches)
-    auto launch = [&](auto kern, int batch, int buffers, int threads, auto ctas_per_sm) {
-        const size_t smem = ((size_t)d * (bits + 4) + (size_t)buffers * batch * (buffers == 2 ? idx_pitch(d, threads - kIdxThreads) : d + 1)) * sizeof(float);
+    auto launch = [&](auto kern, int batch, int buffers, int pitch, int threads, auto ctas_per_sm) {
+        const size_t smem = ((size_t)d * (bits + 4) + (size_t)buffers * batch * pitch) * sizeof(float);
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         const long long batches = (n_pages * H_kv + batch - 1) / batch, resident = 148LL * ctas_per_sm(smem);
         const long long per_cta = (batches + resident - 1) / resident, grid = (batches + per_cta - 1) / per_cta;
         return launch_chained(kern, dim3((unsigned)grid), dim3(threads), smem, st, 0, p);
     };
-    if (many_loaders(p))
-        return launch(d == 128 ? l3_index_kernel<128, 512> : l3_index_kernel<64, 512>, kIdxPairs, 2, 512 + kIdxThreads, [](size_t) { return 1; });
+    if (many_loaders(p)) {
+        const bool swaps = d == 128 && bits == 256;
+        return launch(swaps ? l3_index_kernel<128, 512, true> : (d == 128 ? l3_index_kernel<128, 512> : l3_index_kernel<64, 512>), kIdxPairs, 2,
+                      idx_pitch(d, swaps), 512 + kIdxThreads, [](size_t) { return 1; });
+    }
     if (two_phases(p))
-        return launch(d == 128 ? l3_index_phases_kernel<128> : l3_index_phases_kernel<64>, kPhasePairs, 1, kIdxThreads,
+        return launch(d == 128 ? l3_index_phases_kernel<128> : l3_index_phases_kernel<64>, kPhasePairs, 1, d + 1, kIdxThreads,
                       [](size_t smem) { return smem > 110 * 1024 ? 1 : (smem > 72 * 1024 ? 2 : (smem > 54 * 1024 ? 3 : 4)); });
-    return launch(d == 128 ? l3_index_kernel<128, 128> : l3_index_kernel<64, 128>, kIdxPairs, 2, 2 * kIdxThreads,
+    return launch(d == 128 ? l3_index_kernel<128, 128> : l3_index_kernel<64, 128>, kIdxPairs, 2, idx_pitch(d, false), 2 * kIdxThreads,
                   [](size_t smem) { return smem > 112 * 1024 ? 1 : 2; });
 }
 
