@@ -54,15 +54,15 @@ def load_peaks():
 # as it was when the counters were taken: when the file has changed since, the figure is reported as null ("stale").
 NCU_TRAFFIC = {
     # kernel@workload: (bytes in the capture, units of the capture, summary file under profiles/, source file, its digest)
-    "fwd_tc_kernel@c3": (375.179264e6 + 56.739328e6, 1 * 8, "fwd_tc_kernel_c3p.md", "fwd_tc.cu", "4c90380f91c4"),
-    "fwd_tc_kernel64@c2": (206.649344e6 + 27.328256e6, 8 * 16, "fwd_tc_kernel64_c2.md", "fwd_tc.cu", "4c90380f91c4"),   # the whole configuration
-    "decode_partial_kernel@c4": (1.476449e9 + 4.224768e6, 2 * 32, "decode_partial_kernel_c4p.md", "decode.cu", "502997e1c1d8"),
+    "fwd_tc_kernel@c3": (375.344384e6 + 56.876800e6, 1 * 8, "fwd_tc_kernel_c3p.md", "fwd_tc.cu", "7f2d78173779"),
+    "fwd_tc_kernel64@c2": (204.381184e6 + 25.607168e6, 8 * 16, "fwd_tc_kernel64_c2.md", "fwd_tc.cu", "7f2d78173779"),   # the whole configuration
+    "decode_partial_kernel@c4": (1.476440e9 + 4.305664e6, 2 * 32, "decode_partial_kernel_c4p.md", "decode.cu", "3c41c073302a"),
     "bwd_dq_tc_kernel@c5": (220.644864e6 + 26.942464e6, 1 * 16, "bwd_tc_kernels_c5p.md", "bwd_tc.cu", "1809b0267c2d"),
     "bwd_dkv_tc_kernel@c5": (221.846528e6 + 118.659072e6, 1 * 16, "bwd_tc_kernels_c5p.md", "bwd_tc.cu", "1809b0267c2d"),
     "l2_summary_pipe_kernel@s3": (100.699392e6 + 54.012160e6, 12288.0 / 32768.0, "l2_summary_seg_kernel_s3p.md", "summary_seg.cu", "f824f10a3d76"),   # 12288 of the 32768 tokens
     "fuse_kv_kernel@f3": (403.136512e6 + 83.408640e6, 1 * 8, "fuse_kv_kernel_f3p.md", "fuse_kv.cu", "b1ef4c991e47"),
-    "decode_paged_kernel@g4": (293.750528e6 + 3.454976e6, 1 * 4, "decode_paged_kernel_g4p.md", "decode_paged.cu", "0d8f44cbc542"),   # one of the four sequences (g4p)
-    "l3_index_kernel@r3": (134.585856e6 + 3.313920e6, 1, "l3_index_kernel_r3p.md", "l3.cu", "00671588e2bc"),            # one of the four sequences (r3p)
+    "decode_paged_kernel@g4": (293.749248e6 + 3.900416e6, 1 * 4, "decode_paged_kernel_g4p.md", "decode_paged.cu", "da97c9d38b63"),   # one of the four sequences (g4p)
+    "l3_index_kernel@r3": (134.604544e6 + 3.368192e6, 1, "l3_index_kernel_r3p.md", "l3.cu", "d9141162470e"),            # one of the four sequences (r3p)
 }
 
 

@@ -129,8 +129,8 @@ template <typename P> inline double simt_query_walk(const P& p) {               
 template <typename P> inline int simt_query_groups(const P& p, double k) {
     const long long blocks = (long long)p.B * p.H * ((p.T + 15) / 16);
     const double walk = simt_query_walk(p);
-    // Half as many rows to a CTA where even twice the blocks find an SM each: an SM's shared-memory
-    // reads, which bound a step of the walk, are the same, but a step covers eight tiles.  [1, 4, 256, 64] (window 64, 128 slots): both
+    // Half as many rows to a CTA where even twice the blocks find an SM each: a step of the walk takes as long (its sixteen warps wait at barriers and for
+    // shared-memory reads, which are busy 22 to 35 % of the time) but covers eight tiles.  [1, 4, 256, 64] (window 64, 128 slots): both
     // forwards and the backward together 106 us in four groups, 94 in eight and with the longest key blocks of dK/dV first (clusters of
     // two to four CTAs of four groups instead: 118).  Walks of 5.5 to 8 tiles, four / eight: forward 9.1 / 7.4 (d = 32, 53 to 103 rows), 12.0 / 9.3 (d = 64,
     // 49 to 84), 15.1 / 11.6 (d = 96, 94); before a tile's loads were in flight together they were equal there.
