@@ -23,7 +23,7 @@ CASES = [
     ("cluster", 1, 16, 16, 128, 64, 3072, 11), ("cluster", 1, 16, 16, 128, 64, 3072, -1),
     ("cluster", 1, 16, 16, 128, 128, 3072, 11), ("cluster", 1, 16, 16, 128, 128, 3072, -1),
     ("ranges", 2, 32, 32, 627, 64, 7815, 30), ("ranges", 1, 56, 14, 256, 128, 12800, 50),
-    ("ranges of one tile", 1, 56, 14, 256, 128, 12800, 0),
+    ("ranges of one tile", 1, 56, 14, 256, 128, 12800, 0), ("paged", 2, 32, 32, 640, 64, 7808, 30), ("paged", 1, 56, 14, 256, 128, 12800, 50),
 ]
 
 
